@@ -25,6 +25,7 @@
 #include "gemm_simt.cuh"
 #include "gemm_tc.cuh"
 #include "graph.cuh"
+#include "host_io.cuh"
 
 namespace pd {
 
@@ -174,7 +175,12 @@ struct pdadmm_ctx {
   bool r_valid = false;
   bool t_valid = false;             // every layer's t matches the stored u, p, q
   int *d_flag = nullptr;            // device counter (z_L solver non-convergence)
-  int *h_pinned = nullptr;          // pinned host words for small read-backs
+  // page-locked block (CTX_PINNED_BYTES): words 0..63 small read-backs, 64..127 the lanes' accept flags, from byte 1024 on
+  // the results that kernels write themselves (objective, residuals, counts of pdadmm_predict)
+  int *h_pinned = nullptr;
+  double *h_results = nullptr;
+  int *done = nullptr;              // device: finished blocks per layer of a read-out kernel, zero between launches
+  unsigned long long *counts = nullptr;   // device: the four counts of pdadmm_predict, zero between calls
   int64_t launches = 0;
   cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
   double last_step_ms = 0.0;
@@ -965,11 +971,8 @@ static int check_config(const pdadmm_config *cfg) {
 
 // Host -> device copies go through the context's stream, so that they are ordered with its kernels
 // (the stream does not synchronise with the default stream).
-static int upload_rows(cudaStream_t st, float *dst, int ld, const float *src, int width, int64_t rows) {
-  PD_CUDA(cudaMemcpy2DAsync(dst, (size_t)ld * 4, src, (size_t)width * 4, (size_t)width * 4, (size_t)rows,
-                            cudaMemcpyHostToDevice, st));
-  PD_CUDA(cudaStreamSynchronize(st));
-  return PDADMM_OK;
+static int upload_rows(pdadmm_ctx *c, cudaStream_t st, float *dst, int ld, const float *src, int width, int64_t rows) {
+  return copy_rows(c->device, st, const_cast<float *>(src), dst, (size_t)ld * 4, (size_t)width * 4, (size_t)rows, false);
 }
 
 // Temporary device buffers of the CSR construction, released when the builder returns.
@@ -1051,7 +1054,7 @@ static int alloc_trial_buffers(pdadmm_ctx *c, Scratch &s, size_t n) {
     PD_TRY(dev_alloc(c, &s.pn_plane, n));
     PD_TRY(dev_alloc(c, &s.d_plane, n));
   }
-  PD_CUDA(cudaMallocHost((void **)&s.h_flag, sizeof(int)));
+  s.h_flag = c->h_pinned + 64 + (&s == &c->scr ? 0 : (int)c->more_lanes.size());
   PD_CUDA(cudaEventCreateWithFlags(&s.ev_flag, cudaEventDisableTiming));
   return PDADMM_OK;
 }
@@ -1140,6 +1143,13 @@ static int feasible_start(pdadmm_ctx *c, int first) {
   return PDADMM_OK;
 }
 
+static int take_ctx_pinned(pdadmm_ctx *c) {
+  c->h_pinned = (int *)ctx_pinned_pool().take();
+  if (!c->h_pinned) return fail(PDADMM_ENOMEM, "page-locked host memory is exhausted");
+  c->h_results = (double *)((char *)c->h_pinned + 1024);
+  return PDADMM_OK;
+}
+
 static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *shard) {
   const int64_t Ntot = cfg->n_nodes;
   const bool sharded = shard != nullptr && shard->allreduce != nullptr;
@@ -1167,10 +1177,12 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, cfg->device));
   PD_CUDA(cudaStreamCreateWithFlags(&c->scr.st, cudaStreamNonBlocking));
   cudaStream_t st = c->scr.st;
-  PD_CUDA(cudaMallocHost((void **)&c->h_pinned, 64 * sizeof(int)));
+  PD_TRY(take_ctx_pinned(c));
   PD_CUDA(cudaEventCreate(&c->ev_begin));
   PD_CUDA(cudaEventCreate(&c->ev_end));
   PD_TRY(dev_alloc(c, &c->d_flag, 4));
+  PD_TRY(dev_alloc(c, &c->done, OBJ_MAX_LAYERS + 1));
+  PD_TRY(dev_alloc(c, &c->counts, 4));
 
   // graph: CSR pattern, values and sparse products all on the device
   PD_TRY(build_csr(c, cfg));
@@ -1231,7 +1243,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     if (l > 0) PD_TRY(dev_alloc(c, &ly.g_exp, 1));
     PD_TRY(dev_alloc(c, &ly.amax_p, 1));
     PD_TRY(dev_alloc(c, &ly.amax_r, 1));
-    PD_TRY(upload_rows(st, ly.W, ly.ld_in, cfg->init_W[l], ly.n_in, ly.n_out));
+    PD_TRY(upload_rows(c, st, ly.W, ly.ld_in, cfg->init_W[l], ly.n_in, ly.n_out));
     // Node slices of the W-gradient product (slices >= 256 nodes, at most 32).  The persistent grid works through
     // tiles x slices units in rounds of n_sms, so the count is chosen to fill its last round: the smallest number
     // of slices within 3 % (relative) of the best fill (fewer slices = fewer partial tiles to write and add up).
@@ -1332,7 +1344,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   Layer &l0 = c->layers[0];
   {
     float *xb = sharded ? x_full : l0.p;
-    PD_TRY(upload_rows(st, xb, l0.ld_in, cfg->features, c->d, Ntot));
+    PD_TRY(upload_rows(c, st, xb, l0.ld_in, cfg->features, c->d, Ntot));
     for (int k = 1; k < c->n_blocks; ++k)
       launch_spmm(st, c->row_ptr, c->col_idx, c->csr_val, (int)Ntot, xb + (size_t)(k - 1) * c->d, xb + (size_t)k * c->d,
                   c->d, l0.ld_in);
@@ -1359,7 +1371,7 @@ static void destroy(pdadmm_ctx *c) {
   for (auto &r : c->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
   for (auto e : c->ev_pool) cudaEventDestroy(e);
   for (void *p : c->allocs) cudaFree(p);
-  if (c->h_pinned) cudaFreeHost(c->h_pinned);
+  ctx_pinned_pool().give(c->h_pinned);
   if (c->ev_begin) cudaEventDestroy(c->ev_begin);
   if (c->ev_end) cudaEventDestroy(c->ev_end);
   if (c->iter_graph) cudaGraphExecDestroy(c->iter_graph);
@@ -1367,7 +1379,6 @@ static void destroy(pdadmm_ctx *c) {
   for (auto e : c->ev_lane) cudaEventDestroy(e);
   for (int i = 0; i <= (int)c->more_lanes.size(); ++i) {
     pd::Scratch &x = i == 0 ? c->scr : *c->more_lanes[i - 1];
-    if (x.h_flag) cudaFreeHost(x.h_flag);
     if (x.ev_flag) cudaEventDestroy(x.ev_flag);
   }
   for (auto &x : c->more_lanes) if (x->st) cudaStreamDestroy(x->st);
@@ -1543,11 +1554,41 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
   return PDADMM_OK;
 }
 
-static int read_slots(pdadmm_ctx *c, int n_slots, int stride, int n_out, double *host) {
-  double *dst = c->scr.slots + c->scr.n_slots - 8;            // tail of the slot buffer: results
-  reduce_slots_kernel<<<1, 256, 0, c->scr.st>>>(c->scr.slots, n_slots, stride, n_out, dst);
-  PD_CUDA(cudaMemcpyAsync(host, dst, n_out * sizeof(double), cudaMemcpyDeviceToHost, c->scr.st));
-  PD_CUDA(cudaStreamSynchronize(c->scr.st));
+// The objective's sums of every layer (parts: OBJ_ALL or OBJ_RESIDUALS) into h_results[4 l ..], and with OBJ_ALL the risk
+// into h_results[4 L]; returns when they are there.
+constexpr int OBJ_MAX_BLOCKS = 592;          // per layer: four per SM
+static int read_objective(pdadmm_ctx *c, int parts) {
+  cudaStream_t st = c->scr.st;
+  const int wide = c->code_bytes == 2;
+  for (int l0 = 0; l0 < c->L; l0 += OBJ_MAX_LAYERS) {
+    ObjLayers o;
+    const int n = std::min(OBJ_MAX_LAYERS, c->L - l0);
+    size_t n4_max = 0;
+    for (int i = 0; i < n; ++i) {
+      const Layer &ly = c->layers[l0 + i];
+      const bool hidden = l0 + i + 1 < c->L;
+      const Layer *nx = hidden ? &c->layers[l0 + i + 1] : nullptr;
+      o.l[i] = ObjLayer{ly.r, ly.z, hidden ? ly.q : nullptr, ly.u, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
+                        (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f};
+      n4_max = std::max(n4_max, o.l[i].n4);
+    }
+    // all layers side by side: about eight blocks per SM altogether, as many slots as the buffer holds
+    const size_t fit = std::min<size_t>(OBJ_MAX_BLOCKS, c->scr.n_slots / (4 * (size_t)n));
+    const int per_layer = (int)std::max<size_t>(1, std::min(fit, std::min<size_t>((n4_max + EW_THREADS - 1) / EW_THREADS,
+                                                                                  (size_t)ceil_div(c->n_sms * 8, n))));
+    const dim3 grid((unsigned)per_layer, (unsigned)n);
+    double *out = c->h_results + 4 * (size_t)l0;
+    if (parts == OBJ_ALL) objective_kernel<OBJ_ALL><<<grid, EW_THREADS, 0, st>>>(o, c->slope, wide, c->scr.slots, c->done, out);
+    else objective_kernel<OBJ_RESIDUALS><<<grid, EW_THREADS, 0, st>>>(o, c->slope, wide, c->scr.slots, c->done, out);
+  }
+  if (parts == OBJ_ALL) {
+    const Layer &ly = c->layers[c->L - 1];
+    const int grid = (int)std::min<int64_t>(512, ceil_div(c->N, EW_THREADS));
+    risk_kernel<<<grid, EW_THREADS, 0, st>>>(ly.z, c->labels, c->mask, (int)c->N, ly.n_out, ly.ld_out, c->scr.slots,
+                                             c->ls_risk ? 1 : 0, c->done + OBJ_MAX_LAYERS, c->h_results + 4 * (size_t)c->L);
+  }
+  PD_CUDA(cudaGetLastError());
+  PD_CUDA(cudaStreamSynchronize(st));
   return PDADMM_OK;
 }
 
@@ -1556,26 +1597,12 @@ extern "C" int pdadmm_objective(pdadmm_ctx *c, double out[6]) {
   PD_CUDA(cudaSetDevice(c->device));
   PD_TRY(ensure_residual(c));
   cudaStream_t st = c->scr.st;
-  double lin = 0, act = 0, dual = 0, pen = 0, R = 0;
+  PD_TRY(read_objective(c, OBJ_ALL));
+  double lin = 0, act = 0, dual = 0, pen = 0, R = c->h_results[4 * (size_t)c->L];
   for (int l = 0; l < c->L; ++l) {
-    Layer &ly = c->layers[l];
-    const size_t n = (size_t)c->N * ly.ld_out;
-    const int grid = std::min(ew_grid(n), 512);
-    const bool hidden = l + 1 < c->L;
-    objective_layer_kernel<<<grid, EW_THREADS, 0, st>>>(ly.r, ly.z, hidden ? ly.q : nullptr, ly.u,
-                                                       hidden ? c->layers[l + 1].p : nullptr, n, c->slope, c->scr.slots);
-    double h[4];
-    PD_TRY(read_slots(c, grid, 4, 4, h));
+    const double *h = c->h_results + 4 * (size_t)l;
     lin += h[0]; act += h[1]; dual += h[2]; pen += h[3];
   }
-  {
-    Layer &ly = c->layers[c->L - 1];
-    const int grid = (int)std::min<int64_t>(512, ceil_div(c->N, EW_THREADS));
-    risk_kernel<<<grid, EW_THREADS, 0, st>>>(ly.z, c->labels, c->mask, (int)c->N, ly.n_out, ly.ld_out, c->scr.slots,
-                                             c->ls_risk ? 1 : 0);
-    PD_TRY(read_slots(c, grid, 1, 1, &R));
-  }
-  PD_CUDA(cudaGetLastError());
   if (c->reduce != nullptr) {                 // every component is a sum over nodes
     double h[5] = {R, lin, act, dual, pen};
     PD_CUDA(cudaMemcpyAsync(c->scr.red, h, sizeof h, cudaMemcpyHostToDevice, st));
@@ -1605,7 +1632,8 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   const uint32_t *w_in = nullptr;            // max|activations| of the layer's input
   if (c->use_tc) {
     PD_TRY(amax_reset(c, st));               // one word per layer output, all from one pass through the pool
-    w_in = amax_of(c, st, in, (size_t)N * c->layers[0].ld_in / 4);
+    // max|X| is kept (X changes by pdadmm_set_tensor alone, which clears amax_p_valid)
+    w_in = c->amax_p_valid ? c->layers[0].amax_p : amax_of(c, st, in, (size_t)N * c->layers[0].ld_in / 4);
   }
   for (int l = 0; l < c->L; ++l) {
     Layer &ly = c->layers[l];
@@ -1622,23 +1650,30 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   }
   const Layer &last = c->layers[c->L - 1];
   int *d_pred = reinterpret_cast<int *>(bufs[c->L & 1]);              // the scratch matrix the logits are not in
-  unsigned long long *d_counts = reinterpret_cast<unsigned long long *>(c->scr.slots);
-  PD_CUDA(cudaMemsetAsync(d_counts, 0, 4 * sizeof(unsigned long long), st));
+  unsigned long long *h_counts = reinterpret_cast<unsigned long long *>(c->h_results);
   argmax_kernel<<<(int)std::min<int64_t>(1184, ceil_div(N, EW_THREADS)), EW_THREADS, 0, st>>>(
-      out, c->labels, c->mask, N, last.n_out, last.ld_out, d_pred, d_counts);
+      out, c->labels, c->mask, N, last.n_out, last.ld_out, d_pred, c->counts, c->done, c->d_flag + 1, h_counts);
   PD_CUDA(cudaGetLastError());
-  if (logits_out)
-    PD_CUDA(cudaMemcpy2DAsync(logits_out, (size_t)last.n_out * 4, out, (size_t)last.ld_out * 4, (size_t)last.n_out * 4,
-                              (size_t)N, cudaMemcpyDeviceToHost, st));
-  if (pred_out) PD_CUDA(cudaMemcpyAsync(pred_out, d_pred, (size_t)N * 4, cudaMemcpyDeviceToHost, st));
-  unsigned long long h_counts[4];
-  PD_CUDA(cudaMemcpyAsync(h_counts, d_counts, sizeof(h_counts), cudaMemcpyDeviceToHost, st));
-  PD_CUDA(cudaStreamSynchronize(st));
+  const size_t row = (size_t)last.n_out * 4, lg_bytes = logits_out ? (size_t)N * row : 0, pr_bytes = pred_out ? (size_t)N * 4 : 0;
+  char *stage = lg_bytes + pr_bytes <= STAGE_BYTES ? (char *)stage_pool().take() : nullptr;
+  if (stage != nullptr) {       // small: everything packed into one page-locked block, one wait for the whole call
+    if (logits_out) launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);
+    if (pred_out) launch_pack(st, d_pred, pr_bytes, pr_bytes, 1, stage + lg_bytes);
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) {
+      if (logits_out) memcpy(logits_out, stage, lg_bytes);
+      if (pred_out) memcpy(pred_out, stage + lg_bytes, pr_bytes);
+    }
+    stage_pool().give(stage);
+    PD_CUDA(e);
+  } else {
+    if (logits_out) PD_TRY(copy_rows(c->device, st, logits_out, out, (size_t)last.ld_out * 4, row, (size_t)N, true));
+    if (pred_out) PD_TRY(copy_rows(c->device, st, pred_out, d_pred, pr_bytes, pr_bytes, 1, true));
+    PD_CUDA(cudaStreamSynchronize(st));
+  }
   if (counts_out)
     for (int i = 0; i < 4; ++i) counts_out[i] = (int64_t)h_counts[i];
-  int h_err = 0;
-  PD_CUDA(cudaMemcpy(&h_err, c->d_flag + 1, 4, cudaMemcpyDeviceToHost));
-  if (h_err) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+  if (h_counts[4]) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
   return PDADMM_OK;
 }
 
@@ -1647,17 +1682,8 @@ extern "C" int pdadmm_residuals(pdadmm_ctx *c, double *per_layer_sq, int n) {
   if (n != c->L - 1 || (n > 0 && !per_layer_sq)) return fail(PDADMM_EINVAL, "n must be L-1 = %d", c->L - 1);
   PD_CUDA(cudaSetDevice(c->device));
   PD_TRY(ensure_residual(c));
-  for (int l = 0; l + 1 < c->L; ++l) {
-    Layer &ly = c->layers[l];
-    const size_t nn = (size_t)c->N * ly.ld_out;
-    const int grid = std::min(ew_grid(nn), 512);
-    objective_layer_kernel<<<grid, EW_THREADS, 0, c->scr.st>>>(ly.r, ly.z, ly.q, ly.u, c->layers[l + 1].p, nn,
-                                                              c->slope, c->scr.slots);
-    double h[4];
-    PD_TRY(read_slots(c, grid, 4, 4, h));
-    per_layer_sq[l] = h[3];
-  }
-  PD_CUDA(cudaGetLastError());
+  if (n > 0) PD_TRY(read_objective(c, OBJ_RESIDUALS));
+  for (int l = 0; l + 1 < c->L; ++l) per_layer_sq[l] = c->h_results[4 * (size_t)l + 3];
   if (c->reduce != nullptr && n > 0) {
     if ((size_t)n > 8 + (size_t)c->layers[0].ld_out) return fail(PDADMM_EINVAL, "too many layers for the reduction buffer");
     PD_CUDA(cudaMemcpyAsync(c->scr.red, per_layer_sq, (size_t)n * 8, cudaMemcpyHostToDevice, c->scr.st));
@@ -1714,10 +1740,7 @@ extern "C" int pdadmm_get_tensor(pdadmm_ctx *c, int kind, int layer, void *host_
   if (bytes != t.rows * t.width * t.elem)
     return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                 t.rows * t.width * t.elem, bytes);
-  PD_CUDA(cudaMemcpy2DAsync(host_dst, t.width * t.elem, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows,
-                            cudaMemcpyDeviceToHost, c->scr.st));
-  PD_CUDA(cudaStreamSynchronize(c->scr.st));
-  return PDADMM_OK;
+  return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
 }
 
 // pdADMM-G-Q: the kernels read p_l (l >= 2, paper numbering) as its codes, so the two must always agree: the codes
@@ -1754,9 +1777,7 @@ extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void 
   if (bytes != t.rows * t.width * t.elem)
     return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                 t.rows * t.width * t.elem, bytes);
-  PD_CUDA(cudaMemcpy2DAsync(t.ptr, t.ld * t.elem, host_src, t.width * t.elem, t.width * t.elem, t.rows,
-                            cudaMemcpyHostToDevice, c->scr.st));
-  PD_CUDA(cudaStreamSynchronize(c->scr.st));
+  PD_TRY(copy_rows(c->device, c->scr.st, const_cast<void *>(host_src), t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, false));
   if (kind == PDADMM_T_X || kind == PDADMM_T_P || kind == PDADMM_T_W || kind == PDADMM_T_B || kind == PDADMM_T_Z)
     c->r_valid = false;
   if (kind == PDADMM_T_W) c->w_planes_valid = false;
@@ -1862,8 +1883,8 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
     PD_TRY(dev_alloc(c, &dC, (size_t)M * ldc));
     const int n_slots = 8 * (int)(ceil_div(M, 128) * ceil_div(N, 128)) + 2048;
     PD_TRY(dev_alloc(c, &slots, (size_t)n_slots));
-    PD_TRY(upload_rows(st, dA, lda, A, a_cols, a_rows));
-    PD_TRY(upload_rows(st, dB, ldb, B, b_cols, b_rows));
+    PD_TRY(upload_rows(c, st, dA, lda, A, a_cols, a_rows));
+    PD_TRY(upload_rows(c, st, dB, ldb, B, b_cols, b_rows));
     if (c->use_tc) {
       PD_TRY(dev_alloc(c, &c->scr.amax_pool, (size_t)AMAX_POOL));
       // planes of B as [N][K]: B itself in mode 0, its transpose in mode 1
@@ -1917,7 +1938,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
     reduce_slots_kernel<<<1, 256, 0, st>>>(slots, np, 1, 1, res);
     double h = 0;
     PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
-    PD_CUDA(cudaMemcpy2DAsync(C, (size_t)N * 4, dC, (size_t)ldc * 4, (size_t)N * 4, (size_t)M, cudaMemcpyDeviceToHost, st));
+    PD_TRY(copy_rows(device, st, C, dC, (size_t)ldc * 4, (size_t)N * 4, (size_t)M, true));
     int err = 0;
     PD_CUDA(cudaMemcpyAsync(&err, c->d_flag + 1, 4, cudaMemcpyDeviceToHost, st));
     PD_CUDA(cudaStreamSynchronize(st));
