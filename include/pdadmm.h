@@ -318,8 +318,11 @@ int pdadmm_launches(pdadmm_ctx *ctx, int64_t *count);
  */
 int pdadmm_time_augmentation(pdadmm_ctx *ctx, int reps, double *ms_per_hop, double *bytes_per_hop);
 
-/* Release the context and all of its device memory.  Null is accepted. */
+/* Release the context and all of its device memory.  Null is accepted.  The library keeps a bounded amount of what it
+ * releases for the next context (at most 1/16 of the device's memory, and nothing while less than half of the device is
+ * free); it goes back to the driver when an allocation of the library fails, or by pdadmm_release_cached_memory. */
 int pdadmm_destroy(pdadmm_ctx *ctx);
+int pdadmm_release_cached_memory(int device);
 
 /* Text of the calling thread's last failure ("" if none).  The pointer stays valid until the next failing call. */
 const char *pdadmm_last_error(void);

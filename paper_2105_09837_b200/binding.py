@@ -31,7 +31,7 @@ EXPORTS = [
     "pdadmm_init", "pdadmm_init_sharded", "pdadmm_comm_bytes", "pdadmm_start_layers_from", "pdadmm_step", "pdadmm_last_step_ms", "pdadmm_objective", "pdadmm_residuals", "pdadmm_get_tensor",
     "pdadmm_set_tensor", "pdadmm_predict", "pdadmm_quantize", "pdadmm_spmm", "pdadmm_matmul", "pdadmm_matmul_tn_static", "pdadmm_selftest_bounded_wait",
     "pdadmm_profile", "pdadmm_profile_classes",
-    "pdadmm_profile_name", "pdadmm_profile_read", "pdadmm_launches", "pdadmm_time_augmentation", "pdadmm_destroy", "pdadmm_last_error",
+    "pdadmm_profile_name", "pdadmm_profile_read", "pdadmm_launches", "pdadmm_time_augmentation", "pdadmm_destroy", "pdadmm_release_cached_memory", "pdadmm_last_error",
 ]
 
 
@@ -282,6 +282,11 @@ def from_inputs(inp, device: int = 0, flags: int = 0, rho: Optional[float] = Non
                    inp.train_mask, w.widths, w.rho if rho is None else rho, w.nu if nu is None else nu,
                    w.quant_levels if quant_levels is None else quant_levels, inp.init_W, device, flags,
                    quant_neg_levels, quant_step, leaky_slope, shard, activation, table)
+
+
+def release_cached_memory(device: int = 0):
+    """``pdadmm_release_cached_memory``: device and page-locked memory kept from destroyed contexts goes back to the driver."""
+    _check(lib().pdadmm_release_cached_memory(int(device)))
 
 
 def quantize(x, scale: float, levels: int, device: int = 0, lo: float = 0.0):

@@ -3,7 +3,7 @@
 // The caller's arrays are dense and usually pageable, the device matrices have padded rows.  A pageable 2-D copy left to
 // the driver moves one row at a time through the driver's own staging (measured: 20 000 rows of 40 bytes 2.9 ms, 14 MB
 // of weights 2.1 ms).  Here the rows go through page-locked staging blocks in dense pieces: on the way out a kernel packs a
-// piece straight into the block over PCIe, on the way in the copy engine spreads it over the padded rows; large copies
+// piece straight into the block over PCIe, on the way in the copy engine (or, for short rows, a kernel) spreads it over the padded rows; large copies
 // are split among a few host threads, because one thread's memcpy (10 GB/s into fresh pages) is what bounds them.
 // Page-locked caller arrays skip the staging.
 #pragma once
@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "pools.cuh"
 
 namespace pd {
 
@@ -78,12 +79,34 @@ pack_rows_kernel(const T *__restrict__ src, size_t pitch, uint32_t width, uint32
     dst[i] = src[(size_t)row * pitch + (i - row * width)];
   }
 }
+// The other way.  The copy engine does wide rows as fast as the link (2 KB rows 30 GB/s) and short ones slowly (400-byte
+// rows 6 GB/s), so those are read over PCIe by a kernel.
+constexpr size_t UNPACK_BELOW = 2048;
+template <class T>
+__global__ void __launch_bounds__(256)
+unpack_rows_kernel(const T *__restrict__ src, size_t pitch, uint32_t width, uint32_t n, T *__restrict__ dst) {
+  for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+    const uint32_t row = i / width;
+    dst[(size_t)row * pitch + (i - row * width)] = src[i];
+  }
+}
 inline void launch_pack(cudaStream_t st, const void *src, size_t pitch_bytes, size_t width_bytes, size_t rows, void *dst) {
   const bool wide = pitch_bytes % 16 == 0 && width_bytes % 16 == 0 && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 16 == 0;
   const uint32_t n = (uint32_t)(rows * width_bytes / (wide ? 16 : 4));
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 148));
   if (wide) pack_rows_kernel<uint4><<<grid, 256, 0, st>>>((const uint4 *)src, pitch_bytes / 16, (uint32_t)(width_bytes / 16), n, (uint4 *)dst);
   else pack_rows_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t *)src, pitch_bytes / 4, (uint32_t)(width_bytes / 4), n, (uint32_t *)dst);
+}
+
+inline cudaError_t queue_unpack(cudaStream_t st, const void *src, void *dst, size_t pitch, size_t width, size_t rows) {
+  if (width >= UNPACK_BELOW || width % 4 || pitch % 4)
+    return cudaMemcpy2DAsync(dst, pitch, src, width, width, rows, cudaMemcpyHostToDevice, st);
+  const bool wide = pitch % 16 == 0 && width % 16 == 0 && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 16 == 0;
+  const uint32_t n = (uint32_t)(rows * width / (wide ? 16 : 4));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 296));
+  if (wide) unpack_rows_kernel<uint4><<<grid, 256, 0, st>>>((const uint4 *)src, pitch / 16, (uint32_t)(width / 16), n, (uint4 *)dst);
+  else unpack_rows_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t *)src, pitch / 4, (uint32_t)(width / 4), n, (uint32_t *)dst);
+  return cudaGetLastError();
 }
 
 // One direction of a copy, pieces piece0, piece0 + step, ... of `piece_rows` rows each.  Two staging blocks alternate, so
@@ -118,7 +141,7 @@ inline cudaError_t copy_pieces(const RowCopy &k, size_t piece0, size_t step, cha
       if (used[b]) e = cudaEventSynchronize(ev[b]);
       if (e != cudaSuccess) break;
       memcpy(stage[b], host_of(p), r * k.width);
-      e = cudaMemcpy2DAsync(dev_of(p), k.pitch, stage[b], k.width, k.width, r, cudaMemcpyHostToDevice, k.st);
+      e = queue_unpack(k.st, stage[b], dev_of(p), k.pitch, k.width, r);
       if (e == cudaSuccess) e = cudaEventRecord(ev[b], k.st);
       used[b] = true;
     }
@@ -154,7 +177,7 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
     cudaError_t e = cudaSuccess;
     if (!out) {
       memcpy(stage, host, rows * width);
-      e = cudaMemcpy2DAsync(dev, pitch, stage, width, width, rows, cudaMemcpyHostToDevice, st);
+      e = queue_unpack(st, stage, dev, pitch, width, rows);
     } else if (width % 4 == 0 && pitch % 4 == 0) {
       launch_pack(st, dev, pitch, width, rows, stage);
       e = cudaGetLastError();
@@ -179,7 +202,7 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
     for (int i = 0; i < 2 && err == cudaSuccess; ++i) {
       w.stage[i] = i < n_stage ? (char *)stage_pool().take() : w.stage[0];
       if (w.stage[i] == nullptr) err = cudaErrorMemoryAllocation;
-      else err = cudaEventCreateWithFlags(&w.ev[i], cudaEventDisableTiming);
+      else err = device_pool(device).take_event(false, &w.ev[i]);
     }
   if (err == cudaSuccess) {
     auto body = [&](int t) {
@@ -199,7 +222,7 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
   }
   for (auto &w : ws)
     for (int i = 0; i < 2; ++i) {
-      if (w.ev[i]) cudaEventDestroy(w.ev[i]);
+      device_pool(device).give_event(false, w.ev[i]);
       if (i < n_stage) stage_pool().give(w.stage[i]);
     }
   PD_CUDA(err);

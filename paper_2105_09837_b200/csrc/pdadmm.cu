@@ -26,6 +26,7 @@
 #include "gemm_tc.cuh"
 #include "graph.cuh"
 #include "host_io.cuh"
+#include "pools.cuh"
 
 namespace pd {
 
@@ -189,7 +190,7 @@ struct pdadmm_ctx {
   std::vector<cudaEvent_t> ev_pool;
   double prof_ms[pd::KC_COUNT] = {0}, prof_bytes[pd::KC_COUNT] = {0}, prof_flops[pd::KC_COUNT] = {0};
   int64_t prof_n[pd::KC_COUNT] = {0};
-  std::vector<void *> allocs;       // driver allocations: chunks and large arrays
+  std::vector<pd::DeviceBlock> allocs;   // from the device's pool: chunks and large arrays
   size_t bytes_handed_out = 0;      // device bytes handed out by dev_alloc so far
   char *arena_base = nullptr;       // current chunk
   size_t arena_cap = 0, arena_used = 0, arena_next = size_t(64) << 20;
@@ -213,9 +214,10 @@ namespace pd {
 
 // ---- allocation bookkeeping -------------------------------------------------------------------------
 // Device memory of a context.  Arrays of up to 64 MB are carved out of chunks (64 MB at first, doubling up to
-// 1 GB), 256-byte aligned: a context has some twenty arrays per layer, and one driver allocation each made
-// pdadmm_init spend most of its time in the allocator.  Larger arrays get an allocation of their own, so that
-// a chunk never wastes more than one small array at its end.  Everything is released by destroy().
+// 1 GB), 256-byte aligned: a context has some twenty arrays per layer, and one allocation each made
+// pdadmm_init spend most of its time in the allocator.  Larger arrays get a block of their own, so that
+// a chunk never wastes more than one small array at its end.  destroy() returns everything to the device's pool.
+// A chunk is cleared as a whole when it is taken (200 clears of small arrays cost the host 0.5 ms at c1's sizes).
 constexpr size_t ARENA_MAX_ARRAY = size_t(64) << 20, ARENA_MAX_CHUNK = size_t(1) << 30;   // first chunk: arena_next
 template <class T>
 static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
@@ -228,20 +230,17 @@ static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
   } else {
     const bool chunk = bytes <= ARENA_MAX_ARRAY;
     const size_t want = chunk ? std::max(bytes, c->arena_next) : bytes;
-    void *q = nullptr;
-    const cudaError_t e = cudaMalloc(&q, want);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed: %s", want, cudaGetErrorString(e));
-    }
-    c->allocs.push_back(q);
-    p = (char *)q;
+    DeviceBlock b;
+    const cudaError_t e = device_pool(c->device).take(want, &b);
+    if (e != cudaSuccess) return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed: %s", want, cudaGetErrorString(e));
+    c->allocs.push_back(b);
+    p = (char *)b.p;
     if (chunk) {
-      c->arena_base = p; c->arena_cap = want; c->arena_used = bytes;
+      c->arena_base = p; c->arena_cap = b.bytes; c->arena_used = bytes;
       c->arena_next = std::min(ARENA_MAX_CHUNK, 2 * want);
     }
+    if (chunk || zero) PD_CUDA(cudaMemsetAsync(p, 0, chunk ? b.bytes : bytes, c->scr.st));   // same stream as every kernel that uses it
   }
-  if (zero) PD_CUDA(cudaMemsetAsync(p, 0, bytes, c->scr.st));   // same stream as every kernel that uses it
   c->bytes_handed_out += bytes;
   *ptr = (T *)p;
   return PDADMM_OK;
@@ -975,21 +974,28 @@ static int upload_rows(pdadmm_ctx *c, cudaStream_t st, float *dst, int ld, const
   return copy_rows(c->device, st, const_cast<float *>(src), dst, (size_t)ld * 4, (size_t)width * 4, (size_t)rows, false);
 }
 
-// Temporary device buffers of the CSR construction, released when the builder returns.
+// Temporary device buffers of the CSR construction, carved out of one block that goes back when the builder returns.
 struct TempBuffers {
-  std::vector<void *> ptrs;
-  ~TempBuffers() { for (void *p : ptrs) cudaFree(p); }
+  int device;
+  std::vector<DeviceBlock> block;
+  size_t used = 0;
+  explicit TempBuffers(int dev) : device(dev) {}
+  ~TempBuffers() { if (!block.empty()) { cudaDeviceSynchronize(); device_pool(device).give(block); } }
+  static size_t room(size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) & ~size_t(255); }
+  int reserve(size_t bytes) {
+    DeviceBlock b;
+    const size_t want = (bytes + (size_t(2) << 20) - 1) & ~((size_t(2) << 20) - 1);
+    const cudaError_t e = device_pool(device).take(want, &b);
+    if (e != cudaSuccess) return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed: %s", want, cudaGetErrorString(e));
+    block.push_back(b);
+    return PDADMM_OK;
+  }
   template <class T>
   int get(T **out, size_t count) {
-    void *p = nullptr;
-    const size_t bytes = std::max<size_t>(count * sizeof(T), 16);
-    const cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
-    }
-    ptrs.push_back(p);
-    *out = (T *)p;
+    const size_t bytes = room(count * sizeof(T));
+    if (used + bytes > block[0].bytes) return fail(PDADMM_ENOMEM, "temporary buffers were reserved too small");
+    *out = (T *)((char *)block[0].p + used);
+    used += bytes;
     return PDADMM_OK;
   }
 };
@@ -1000,7 +1006,9 @@ static int build_csr(pdadmm_ctx *c, const pdadmm_config *cfg) {
   const size_t raw_cap = (size_t)(2 * E + N);
   if (raw_cap > (size_t)INT32_MAX) return fail(PDADMM_EINVAL, "more than 2^31-1 non-zeros");
   cudaStream_t st = c->scr.st;
-  TempBuffers tmp;
+  TempBuffers tmp(c->device);
+  const size_t n4 = TempBuffers::room((size_t)N * 4 + 4);
+  PD_TRY(tmp.reserve(2 * TempBuffers::room((size_t)E * 4) + 5 * n4 + 2 * TempBuffers::room(raw_cap * 4) + 1024));
   int *d_src, *d_dst, *deg, *cursor, *raw_ptr, *raw, *sorted, *len, *long_rows, *meta;
   unsigned long long *bad_edge;
   PD_TRY(tmp.get(&d_src, (size_t)E)); PD_TRY(tmp.get(&d_dst, (size_t)E));
@@ -1055,7 +1063,7 @@ static int alloc_trial_buffers(pdadmm_ctx *c, Scratch &s, size_t n) {
     PD_TRY(dev_alloc(c, &s.d_plane, n));
   }
   s.h_flag = c->h_pinned + 64 + (&s == &c->scr ? 0 : (int)c->more_lanes.size());
-  PD_CUDA(cudaEventCreateWithFlags(&s.ev_flag, cudaEventDisableTiming));
+  PD_CUDA(device_pool(c->device).take_event(false, &s.ev_flag));
   return PDADMM_OK;
 }
 
@@ -1175,11 +1183,12 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->int_operands = c->use_tc && c->levels >= 2 && c->levels <= 2048 && c->neg_levels == 0;
   PD_CUDA(cudaSetDevice(cfg->device));
   PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, cfg->device));
-  PD_CUDA(cudaStreamCreateWithFlags(&c->scr.st, cudaStreamNonBlocking));
+  DevicePool &pool = device_pool(c->device);
+  PD_CUDA(pool.take_stream(&c->scr.st));
   cudaStream_t st = c->scr.st;
   PD_TRY(take_ctx_pinned(c));
-  PD_CUDA(cudaEventCreate(&c->ev_begin));
-  PD_CUDA(cudaEventCreate(&c->ev_end));
+  PD_CUDA(pool.take_event(true, &c->ev_begin));
+  PD_CUDA(pool.take_event(true, &c->ev_end));
   PD_TRY(dev_alloc(c, &c->d_flag, 4));
   PD_TRY(dev_alloc(c, &c->done, OBJ_MAX_LAYERS + 1));
   PD_TRY(dev_alloc(c, &c->counts, 4));
@@ -1195,17 +1204,18 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   // X = [H, A~ H, A~^2 H, ...] for all nodes (a shard needs its neighbours' features, and theirs, ...); a shard then
   // keeps the rows of its own nodes
   float *x_full = nullptr;
-  void *x_full_alloc = nullptr;
+  struct BlockLater {
+    int device; std::vector<DeviceBlock> b;
+    ~BlockLater() { if (!b.empty()) { cudaDeviceSynchronize(); device_pool(device).give(b); } }
+  } x_full_block{c->device, {}};
   if (sharded) {
     const size_t bytes = (size_t)Ntot * c->ld0 * 4 + 256;
-    if (cudaMalloc(&x_full_alloc, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed", bytes);
-    }
-    x_full = (float *)x_full_alloc;
+    DeviceBlock b;
+    if (pool.take(bytes, &b) != cudaSuccess) return fail(PDADMM_ENOMEM, "cudaMalloc of %zu bytes failed", bytes);
+    x_full_block.b.push_back(b);
+    x_full = (float *)b.p;
     PD_CUDA(cudaMemsetAsync(x_full, 0, bytes, st));
   }
-  struct FreeLater { void *p; ~FreeLater() { if (p) cudaFree(p); } } free_x{x_full_alloc};
   c->N = N;                                  // from here on: the nodes this context owns
 
   // layers
@@ -1224,6 +1234,8 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     // quantised mode: p_l and its codes trade places with the trial buffers, so all share one size
     const size_t e_in = (size_t)N * ((c->levels && l > 0) ? max_in : ly.ld_in);
     PD_TRY(dev_alloc(c, &ly.p, e_in));
+    if (l == 0)      // the features go first: their copy overlaps the clearing of everything allocated after them
+      PD_TRY(upload_rows(c, st, sharded ? x_full : ly.p, ly.ld_in, cfg->features, c->d, Ntot));
     PD_TRY(dev_alloc(c, &ly.W, (size_t)ly.n_out * ly.ld_in));
     PD_TRY(dev_alloc(c, &ly.gradW, (size_t)ly.n_out * ly.ld_in));
     if (c->use_tc) {
@@ -1319,7 +1331,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   for (int i = 1; i < n_lanes; ++i) {
     c->more_lanes.emplace_back(new Scratch());
     Scratch &x = *c->more_lanes.back();
-    PD_CUDA(cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking));
+    PD_CUDA(pool.take_stream(&x.st));
     PD_TRY(dev_alloc(c, &x.s1, e_max));
     PD_TRY(dev_alloc(c, &x.s2, (size_t)N * max_out));
     PD_TRY(dev_alloc(c, &x.part, max_part));
@@ -1336,15 +1348,14 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     }
   }
   c->ev_p.resize(c->L);
-  for (auto &e : c->ev_p) PD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  for (auto &e : c->ev_p) PD_CUDA(pool.take_event(false, &e));
   c->ev_lane.resize(n_lanes);
-  for (auto &e : c->ev_lane) PD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  for (auto &e : c->ev_lane) PD_CUDA(pool.take_event(false, &e));
 
   // X = [H, A~ H, A~^2 H, ...] in the column blocks of p_1
   Layer &l0 = c->layers[0];
   {
     float *xb = sharded ? x_full : l0.p;
-    PD_TRY(upload_rows(c, st, xb, l0.ld_in, cfg->features, c->d, Ntot));
     for (int k = 1; k < c->n_blocks; ++k)
       launch_spmm(st, c->row_ptr, c->col_idx, c->csr_val, (int)Ntot, xb + (size_t)(k - 1) * c->d, xb + (size_t)k * c->d,
                   c->d, l0.ld_in);
@@ -1370,19 +1381,19 @@ static void destroy(pdadmm_ctx *c) {
   cudaDeviceSynchronize();
   for (auto &r : c->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
   for (auto e : c->ev_pool) cudaEventDestroy(e);
-  for (void *p : c->allocs) cudaFree(p);
-  ctx_pinned_pool().give(c->h_pinned);
-  if (c->ev_begin) cudaEventDestroy(c->ev_begin);
-  if (c->ev_end) cudaEventDestroy(c->ev_end);
   if (c->iter_graph) cudaGraphExecDestroy(c->iter_graph);
-  for (auto e : c->ev_p) cudaEventDestroy(e);
-  for (auto e : c->ev_lane) cudaEventDestroy(e);
+  DevicePool &pool = device_pool(c->device);
+  pool.give(c->allocs);
+  ctx_pinned_pool().give(c->h_pinned);
+  pool.give_event(true, c->ev_begin);
+  pool.give_event(true, c->ev_end);
+  for (auto e : c->ev_p) pool.give_event(false, e);
+  for (auto e : c->ev_lane) pool.give_event(false, e);
   for (int i = 0; i <= (int)c->more_lanes.size(); ++i) {
     pd::Scratch &x = i == 0 ? c->scr : *c->more_lanes[i - 1];
-    if (x.ev_flag) cudaEventDestroy(x.ev_flag);
+    pool.give_event(false, x.ev_flag);
+    pool.give_stream(x.st);
   }
-  for (auto &x : c->more_lanes) if (x->st) cudaStreamDestroy(x->st);
-  if (c->scr.st) cudaStreamDestroy(c->scr.st);
   delete c;
 }
 
@@ -1419,7 +1430,7 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
     cudaGetLastError();
     return fail(PDADMM_ECUDA, "no CUDA device is available");
   }
-  if (cfg->device < 0 || cfg->device >= n_dev) return fail(PDADMM_EINVAL, "device %d does not exist", cfg->device);
+  if (cfg->device < 0 || cfg->device >= n_dev || cfg->device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "device %d does not exist", cfg->device);
   pdadmm_ctx *c = new (std::nothrow) pdadmm_ctx();
   if (!c) return fail(PDADMM_ENOMEM, "out of host memory");
   int rc;
@@ -1443,6 +1454,20 @@ extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
   // the linear residual of the restarted layers is zero by construction; everything derived from the other tensors
   // (the residual of the kept layers, t, planes, largest magnitudes) is rebuilt by the next call that needs it
   c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false;
+  return PDADMM_OK;
+}
+
+extern "C" int pdadmm_release_cached_memory(int device) {
+  int n_dev = 0;
+  if (cudaGetDeviceCount(&n_dev) != cudaSuccess || n_dev == 0) {
+    cudaGetLastError();
+    return fail(PDADMM_ECUDA, "no CUDA device is available");
+  }
+  if (device < 0 || device >= n_dev || device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "device %d does not exist", device);
+  PD_CUDA(cudaSetDevice(device));
+  device_pool(device).trim();
+  stage_pool().trim();
+  ctx_pinned_pool().trim();
   return PDADMM_OK;
 }
 
@@ -1856,7 +1881,7 @@ extern "C" int pdadmm_spmm(int device, int64_t n_rows, const int32_t *row_ptr, c
 
 extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const float *A, const float *B, float *C,
                              double *sumsq, uint32_t flags) {
-  if (mode < 0 || mode > 2 || M < 1 || N < 1 || K < 1 || !A || !B || !C) return fail(PDADMM_EINVAL, "bad argument");
+  if (mode < 0 || mode > 2 || M < 1 || N < 1 || K < 1 || !A || !B || !C || device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "bad argument");
   PD_CUDA(cudaSetDevice(device));
   pdadmm_ctx *c = new (std::nothrow) pdadmm_ctx();
   if (!c) return fail(PDADMM_ENOMEM, "out of host memory");
@@ -1864,7 +1889,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
   c->use_tc = (flags & PDADMM_FLAG_SIMT_GEMM) == 0;
   auto body = [&]() -> int {
     PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device));
-    PD_CUDA(cudaStreamCreateWithFlags(&c->scr.st, cudaStreamNonBlocking));
+    PD_CUDA(device_pool(device).take_stream(&c->scr.st));
     cudaStream_t st = c->scr.st;
     PD_TRY(dev_alloc(c, &c->d_flag, 4));
     if (c->use_tc) {
