@@ -842,7 +842,7 @@ static void zqu_step(pdadmm_ctx *c, int l) {
     if (c->table_size > 0) {
       Launch k(c, KC_ZQU, s.st, (c->levels ? 37.0 : 40.0) * N * ly.n_out, 0);
       const Layer &nx = c->layers[l + 1];
-      zqu_table_kernel<<<grid, EW_THREADS, 2 * c->table_size * sizeof(float), s.st>>>(
+      zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), s.st>>>(
           ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu, c->slope, c->table_lo, c->table_step,
           c->table_size, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t, s.slots, ly.amax_r,
           c->levels ? nx.codes : nullptr, c->code_bytes == 2);

@@ -1,0 +1,48 @@
+"""The z-update from a lookup table: the chosen candidate against a search over all of them, where the descent can go wrong
+(tables of 2 and 3 candidates and of the largest size, minimisers at and beyond the ends of the table, values of q for
+which the objective is not convex and all candidates have to be tried)."""
+
+import numpy as np
+import pytest
+
+from paper_2105_09837_b200 import binding as B
+from paper_2105_09837_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("act,T,lo,hi,q_scale", [(1, 2, -1.0, 1.0, 0.5), (1, 3, -6.0, 6.0, 1.0), (1, 513, -0.25, 0.25, 1.0),
+                                                 (1, 513, -6.0, 6.0, 4.0), (1, 4096, -6.0, 6.0, 1.2), (2, 513, -6.0, 6.0, 1.0),
+                                                 (2, 257, -4.0, 4.0, 60.0), (1, 129, -300.0, 300.0, 1.0)])
+def test_the_table_candidate_is_the_best_of_all(act, T, lo, hi, q_scale):
+    inp = synth.make_inputs(synth.small("c2", 777, feat_dim=9, hidden=37, n_layers=3, quant_levels=0))
+    ctx = B.from_inputs(inp, activation=act, table=(T, lo, hi))
+    rng = np.random.default_rng(T)
+    z0, q0 = {}, {}
+    for l in (1, 2):
+        z0[l] = rng.standard_normal((777, 37)).astype(np.float32) * np.float32(0.4 * (hi - lo))
+        q0[l] = rng.standard_normal((777, 37)).astype(np.float32) * np.float32(q_scale)
+        ctx.set_tensor(B.T_Z, l, z0[l])
+        ctx.set_tensor(B.T_Q, l, q0[l])
+    ctx.step(1)
+    step = np.float32(np.float32(hi) - np.float32(lo)) / np.float32(T - 1)
+    pts = np.float32(lo) + np.arange(T, dtype=np.float32) * step          # one rounded multiply, one rounded add
+    f = np.tanh(pts.astype(np.float64)) if act == 1 else 1.0 / (1.0 + np.exp(-pts.astype(np.float64)))
+    for l in (1, 2):
+        W, b, p = (ctx.get_tensor(k, l).astype(np.float64) for k in (B.T_W, B.T_B, B.T_P))
+        z = ctx.get_tensor(B.T_Z, l)
+        a = p @ W.T + b
+        at = np.searchsorted(pts, z.ravel()).reshape(z.shape)
+        assert np.array_equal(pts[np.minimum(at, T - 1)], z), "z left the table"
+
+        def value(zc, fc):
+            return (zc - a) ** 2 + (q0[l] - fc) ** 2 + (zc - z0[l]) ** 2
+        got = value(z.astype(np.float64), f[at])
+        best = np.full(z.shape, np.inf)
+        for i in range(T):
+            best = np.minimum(best, value(np.float64(pts[i]), f[i]))
+        # a (a product of 27 or 37 terms, kept as r + z in single precision) and the values themselves carry at most
+        # 1e-6 of |a| + |z| + |q|: the difference of two values within 2 |d| times that, d the distances that enter them
+        size = np.abs(a) + np.abs(z0[l]) + np.abs(q0[l]) + abs(lo) + abs(hi)
+        assert np.all(got - best <= 1e-5 * best + 4e-6 * size * (np.sqrt(best) + step))
+    ctx.destroy()
