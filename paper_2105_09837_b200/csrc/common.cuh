@@ -54,21 +54,24 @@ __host__ __device__ __forceinline__ int tc_scale_exp(uint32_t amax_bits) {
   const int e = 14 - (E - 127);
   return e < -100 ? -100 : (e > 100 ? 100 : e);
 }
-// An fp16 copy of a matrix written before its largest magnitude is known takes its exponent from the maximum of the
-// previous iteration, two binary orders lower (room for a fourfold growth); TC_NO_PREDICTION if that maximum is no
-// normal number.  The copy is usable if the true maximum, scaled, lies in [2^4, 2^15): no overflow and at least 11
-// significant bits above the fp16 subnormals for the largest entries (it is used as a hi plane alone).
+// Planes of a matrix that are written before its largest magnitude is known take their exponent from a bound, or from
+// the maximum of the previous iteration, four binary orders lower (room for a sixteenfold growth); TC_NO_PREDICTION if that
+// maximum is no normal number.  They are usable if the true maximum, scaled, lies in [2^6, 2^15): no overflow, and the
+// pair still carries its 22 bits over 20 binary orders of magnitude below the maximum (all zero is fine whatever the
+// exponent).  Eight orders of the 29 that the exact exponent gives are spent at worst; what they cover enters a product
+// at 2^-20 of its largest terms with 11 bits instead of 22, i.e. far below the 2^-22 of the largest terms' own rounding.
 constexpr int TC_NO_PREDICTION = -1000;
 __host__ __device__ __forceinline__ int tc_predict_exp(uint32_t amax_bits) {
   const int E = (int)((amax_bits >> 23) & 0xFFu);
   if (E == 0 || E == 255) return TC_NO_PREDICTION;
-  return tc_scale_exp(amax_bits) - 2;
+  return tc_scale_exp(amax_bits) - 4;
 }
-__host__ __device__ __forceinline__ bool tc_prediction_usable(uint32_t amax_bits, int predicted) {
+__host__ __device__ __forceinline__ bool tc_planes_usable(uint32_t amax_bits, int e) {
+  if (amax_bits == 0u) return true;
   const int E = (int)((amax_bits >> 23) & 0xFFu);
-  if (E == 0 || E == 255 || predicted < -100 || predicted > 100) return false;
-  const int e = 14 - (E - 127);          // unclamped exponent of the exact scaling
-  return predicted <= e && predicted >= e - 10;
+  if (E == 0 || E == 255 || e < -100 || e > 100) return false;
+  const int top = E - 127 + e;          // max|x| 2^e lies in [2^top, 2^(top + 1))
+  return top >= 6 && top <= 14;
 }
 // ---- largest magnitude of an array, as a bit pattern ---------------------------------------------
 // The tensor-core products scale each operand by a power of two chosen from max|x|.  The maximum is kept as the

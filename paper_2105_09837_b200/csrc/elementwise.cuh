@@ -10,6 +10,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "planes.cuh"
 
 namespace pd {
 
@@ -90,37 +91,53 @@ __device__ __forceinline__ float4 levels_of4(const void *__restrict__ codes, int
                      __fadd_rn(lo, __fmul_rn(c3, s)));
 }
 
-// ---- y -= x * (*inv) ----------------------------------------------------------------------------
-// p-update  p+ = p - g/tau  (Eq. "update p") and the matching update of the linear residual,
-// r <- r - (W g)/tau, and r <- r - (grad_W p+)/theta after the W-update (Eq. "update W").
+// Planes of a matrix that a kernel writes beside the fp32 values, for a later tensor-core product: the exponent was chosen
+// before the kernel started (a bound or a prediction, see tc_planes_usable).  hi == nullptr: none are wanted.
+struct PlaneOut { __half *hi, *lo; const int *exp; };
+__device__ __forceinline__ void store_planes4(const PlaneOut &o, size_t i, float4 v, float scale) {
+  uint2 h, l;
+  tc_split4(v, scale, h, l);
+  reinterpret_cast<uint2 *>(o.hi)[i] = h;
+  reinterpret_cast<uint2 *>(o.lo)[i] = l;
+}
+
+// ---- p-step of pdADMM-G ----------------------------------------------------------------------------
+// p+ = p - g/tau  (Eq. "update p") and the matching update of the linear residual, r <- r - (W g)/tau, in one launch (the
+// elements of p first, then those of r), with the planes of both for the W-gradient and G p+.  16 bytes per element and
+// matrix: read 8, write 4 and the planes 4.  (Separate passes that split r and p again cost 8 bytes more each, and the
+// products that took them fp32 ran at 0.6 of their speed.)
 __global__ void __launch_bounds__(EW_THREADS)
-axpy_neg_kernel(float *__restrict__ y, const float *__restrict__ x, const float *__restrict__ inv, size_t n4,
-                uint32_t *__restrict__ amax /* receives max|y| (see commit_amax); may be null */) {
+pstep_kernel(float *__restrict__ p, const float *__restrict__ g, size_t n4p, float *__restrict__ r, const float *__restrict__ wg,
+             size_t n4r, const float *__restrict__ inv, PlaneOut pp, PlaneOut rp,
+             uint32_t *__restrict__ amax_p /* receives max|p| (see commit_amax); may be null */, uint32_t *__restrict__ amax_r) {
   const float a = *inv;
-  uint32_t m = 0u;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  // four groups per pass: eight loads in flight per thread
-  for (; i + 3 * stride < n4; i += 4 * stride) {
-    float4 v[4], w[4];
+  const size_t stride = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  auto pass = [&](float *__restrict__ y, const float *__restrict__ x, size_t n4, const PlaneOut &o, uint32_t *amax) {
+    const float scale = o.hi != nullptr ? tc_scale_of(*o.exp) : 1.f;
+    uint32_t m = 0u;
+    // four groups per pass: eight loads in flight per thread
+    for (size_t i = first; i < n4; i += 4 * stride) {
+      float4 v[4], w[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) { v[k] = ld4(y, i + k * stride); w[k] = ld4(x, i + k * stride); }
+      for (int k = 0; k < 4; ++k) {
+        const size_t q = i + k * stride;
+        if (q < n4) { v[k] = ld4(y, q); w[k] = ld4(x, q); }
+      }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
-      v[k].z = fmaf(-a, w[k].z, v[k].z); v[k].w = fmaf(-a, w[k].w, v[k].w);
-      st4(y, i + k * stride, v[k]);
-      m = max(m, abs_bits(v[k]));
+      for (int k = 0; k < 4; ++k) {
+        const size_t q = i + k * stride;
+        if (q >= n4) continue;
+        v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
+        v[k].z = fmaf(-a, w[k].z, v[k].z); v[k].w = fmaf(-a, w[k].w, v[k].w);
+        st4(y, q, v[k]);
+        if (o.hi != nullptr) store_planes4(o, q, v[k], scale);
+        m = max(m, abs_bits(v[k]));
+      }
     }
-  }
-  for (; i < n4; i += stride) {
-    float4 v = ld4(y, i);
-    const float4 w = ld4(x, i);
-    v.x = fmaf(-a, w.x, v.x); v.y = fmaf(-a, w.y, v.y); v.z = fmaf(-a, w.z, v.z); v.w = fmaf(-a, w.w, v.w);
-    st4(y, i, v);
-    m = max(m, abs_bits(v));
-  }
-  if (amax != nullptr) commit_amax(m, amax);
+    if (amax != nullptr) commit_amax(m, amax);
+  };
+  pass(p, g, n4p, pp, amax_p);
+  pass(r, wg, n4r, rp, amax_r);
 }
 
 // ---- quantised trial step ------------------------------------------------------------------------
@@ -198,7 +215,6 @@ quantize_kernel(const float *x, size_t n, float scale, float lo, int levels, flo
 
 // ---- operand planes of a quantised p from its codes ------------------------------------------------------------
 // p = code * s with code < 2048: the fp16 plane of the integer codes is the whole operand (the products multiply by s).
-// Same orientation [N][ld] ...
 __global__ void __launch_bounds__(EW_THREADS)
 codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, size_t n4, __half *__restrict__ plane) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
@@ -214,31 +230,6 @@ codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, size_t n4,
     reinterpret_cast<uint2 *>(plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
   }
 }
-// ... and transposed [cols][ldT] (node index contiguous), for the product that contracts over the nodes.  One block of
-// 32 x 8 threads per tile of 32 nodes x 32 columns, through shared memory.
-__global__ void __launch_bounds__(256)
-transpose_codes_kernel(const void *__restrict__ codes, int wide_codes, int rows, int cols, int ld,
-                       __half *__restrict__ planeT, int ldT) {
-  __shared__ __half sh[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = r0 + threadIdx.y + 8 * i, c = c0 + threadIdx.x;
-    float v = 0.f;
-    if (r < rows && c < cols) {
-      const size_t o = (size_t)r * ld + c;
-      v = wide_codes ? (float)reinterpret_cast<const uint16_t *>(codes)[o] : (float)reinterpret_cast<const uint8_t *>(codes)[o];
-    }
-    sh[threadIdx.y + 8 * i][threadIdx.x] = __float2half_rn(v);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int c = c0 + threadIdx.y + 8 * i, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) planeT[(size_t)c * ldT + r] = sh[threadIdx.x][threadIdx.y + 8 * i];
-  }
-}
-
 // ---- finalisers of the step parameters (one block of FIN_THREADS threads) ---------------------------------
 // Fixed-order sum of n slots by one block of FIN_THREADS threads: thread t adds slots t, t + FIN_THREADS, ..., then a
 // fixed tree.  Result in thread 0.
@@ -263,10 +254,16 @@ __device__ __forceinline__ double block_sum_slots(const double *__restrict__ slo
 }
 // ||g||^2 and ||W g||^2 from their slots, then
 // tau = rho + nu ||W g||^2 / ||g||^2 : the smallest tau with phi(p - g/tau) <= U_l(p - g/tau; tau).
+// Thread 0 also settles the exponents of planes that later kernels write (null words are skipped).  With w_wg, the
+// p-step of pdADMM-G follows: |p+| <= max|p| + max|g|/tau and |r+| <= max|r| + max|W g|/tau are bounds.  Without, r after the
+// trial is predicted from r before it.  g of the next iteration is predicted from this one's.
+struct TauPlanes { uint32_t *amax_p; const uint32_t *amax_r, *w_g, *w_wg; int *p_exp, *r_exp, *g_exp; };
+__device__ __forceinline__ int tc_bound_exp(uint32_t a, uint32_t b, float factor) {       // of a + b * factor, a little up
+  return tc_scale_exp(__float_as_uint((__uint_as_float(a) + __uint_as_float(b) * factor) * 1.0001f));
+}
 __global__ void __launch_bounds__(FIN_THREADS)
 finalize_tau_kernel(LayerScalars *sc, double rho, double nu, const double *slots_g, int n_g, const double *slots_wg, int n_wg,
-                    int *nonfinite, uint32_t *clear_word /* max|p| of the layer restarts with the coming p-step */,
-                    const uint32_t *amax_g = nullptr, int *next_g_exp = nullptr /* scaling of the next iteration's fp16 copy of g */) {
+                    int *nonfinite, TauPlanes t) {
   __shared__ double sh[FIN_THREADS];
   const double gg = block_sum_slots(slots_g, n_g, sh);
   const double wg = block_sum_slots(slots_wg, n_wg, sh);
@@ -275,12 +272,15 @@ finalize_tau_kernel(LayerScalars *sc, double rho, double nu, const double *slots
     sc->sum_wg2 = wg;
     if (!(isfinite(gg) && isfinite(wg))) *nonfinite = 1;      // a NaN or Inf anywhere in the state reaches these sums
     const double tau = gg > 0.0 ? rho + nu * wg / gg : rho;
+    const float inv_tau = (float)(1.0 / tau);
     sc->tau = tau;
-    sc->inv_tau = (float)(1.0 / tau);
+    sc->inv_tau = inv_tau;
     sc->accepted = 0;
     sc->trials = 0;
-    if (clear_word != nullptr) *clear_word = 0u;
-    if (next_g_exp != nullptr) *next_g_exp = tc_predict_exp(*amax_g);
+    if (t.p_exp != nullptr) *t.p_exp = tc_bound_exp(*t.amax_p, *t.w_g, inv_tau);
+    if (t.r_exp != nullptr) *t.r_exp = t.w_wg != nullptr ? tc_bound_exp(*t.amax_r, *t.w_wg, inv_tau) : tc_predict_exp(*t.amax_r);
+    if (t.g_exp != nullptr) *t.g_exp = tc_predict_exp(*t.w_g);
+    if (t.amax_p != nullptr) *t.amax_p = 0u;                  // max|p| of the layer restarts with the coming p-step
   }
 }
 // Stop condition of the quantised step in its quadratic form: nu||W d||^2 + rho||d||^2 <= tau||d||^2 (1 + slack).
@@ -305,9 +305,12 @@ finalize_trial_kernel(LayerScalars *sc, double rho, double nu, double slack, con
 }
 // ||grad_W||^2 and ||grad_W p+||^2 from their slots, then
 // theta = nu ||grad_W p+||^2 / ||grad_W||^2 : the smallest theta with phi(W+) <= V_l(W+; theta).
+// Exponents of planes as in finalize_tau_kernel: W+ is bounded by max|W| + max|G|/theta; the coming z-step's r and the next
+// iteration's G are predicted from this iteration's.
+struct ThetaPlanes { uint32_t *amax_r, *amax_W; const uint32_t *w_G; int *W_exp, *r_exp, *G_exp; };
 __global__ void __launch_bounds__(FIN_THREADS)
 finalize_theta_kernel(LayerScalars *sc, double nu, const double *slots_G, int n_G, const double *slots_Gp, int n_Gp,
-                      int *nonfinite, uint32_t *clear_word /* max|r| of the layer restarts with the coming z-step */) {
+                      int *nonfinite, ThetaPlanes t) {
   __shared__ double sh[FIN_THREADS];
   const double GG = block_sum_slots(slots_G, n_G, sh);
   const double Gp = block_sum_slots(slots_Gp, n_Gp, sh);
@@ -316,148 +319,41 @@ finalize_theta_kernel(LayerScalars *sc, double nu, const double *slots_G, int n_
     sc->sum_Gp2 = Gp;
     if (!(isfinite(GG) && isfinite(Gp))) *nonfinite = 1;
     const double theta = GG > 0.0 ? nu * Gp / GG : 0.0;
+    const float inv_theta = theta > 0.0 ? (float)(1.0 / theta) : 0.0f;
     sc->theta = theta;
-    sc->inv_theta = theta > 0.0 ? (float)(1.0 / theta) : 0.0f;
-    if (clear_word != nullptr) *clear_word = 0u;
+    sc->inv_theta = inv_theta;
+    if (t.W_exp != nullptr) *t.W_exp = tc_bound_exp(*t.amax_W, *t.w_G, inv_theta);
+    if (t.r_exp != nullptr) *t.r_exp = tc_predict_exp(*t.amax_r);
+    if (t.G_exp != nullptr) *t.G_exp = tc_predict_exp(*t.w_G);
+    if (t.amax_r != nullptr) *t.amax_r = 0u;                  // max|r| restarts with the coming z-step, max|W| with the W-step
+    if (t.amax_W != nullptr) *t.amax_W = 0u;
   }
 }
 
-// ---- fp16 operand planes of a weight-sized matrix --------------------------------------------------
-// x [rows][ld] fp32 -> hi, lo [rows][ldh] (same orientation) and, if asked for, hiT, loT [cols][ldhT] (transposed),
-// so that every tensor-core product finds its small operand contiguous along the contraction index.
-// xs = x 2^e with e from max|x| (`amax`, see tc_scale_exp); hi = xs rounded to 11 significant bits,
-// lo = (xs - hi) 2^11; e is stored in *exp_out for the products that use the planes.
-// One block of 32 x 8 threads per 32 x 32 tile.
-__global__ void __launch_bounds__(256)
-make_planes_kernel(const float *__restrict__ x, int rows, int cols, int ld, const uint32_t *__restrict__ amax,
-                   int *__restrict__ exp_out, __half *__restrict__ hi, __half *__restrict__ lo, int ldh,
-                   __half *__restrict__ hiT, __half *__restrict__ loT, int ldhT) {
-  __shared__ __half sh_hi[32][33], sh_lo[32][33];
-  const int e = tc_scale_exp(*amax);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) *exp_out = e;
-  const float scale = __uint_as_float((uint32_t)(e + 127) << 23);
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = r0 + threadIdx.y + 8 * i, c = c0 + threadIdx.x;
-    __half h = __float2half_rn(0.f), l = h;
-    if (r < rows && c < cols) {
-      const float xs = x[(size_t)r * ld + c] * scale;
-      const float hf = __uint_as_float((__float_as_uint(xs) + 0x1000u) & 0xFFFFE000u);
-      h = __float2half_rn(hf);
-      l = __float2half_rn((xs - hf) * 2048.0f);
-      if (hi != nullptr) { hi[(size_t)r * ldh + c] = h; lo[(size_t)r * ldh + c] = l; }
-    }
-    sh_hi[threadIdx.y + 8 * i][threadIdx.x] = h;
-    sh_lo[threadIdx.y + 8 * i][threadIdx.x] = l;
-  }
-  if (hiT == nullptr) return;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int c = c0 + threadIdx.y + 8 * i, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) {
-      hiT[(size_t)c * ldhT + r] = sh_hi[threadIdx.x][threadIdx.y + 8 * i];
-      loT[(size_t)c * ldhT + r] = sh_lo[threadIdx.x][threadIdx.y + 8 * i];
-    }
-  }
-}
-
-// ---- fp16 planes of a node-major matrix, same orientation -------------------------------------------
-// x [rows][ld] fp32 -> hi, lo [rows][ld] halves (the padding columns, zero in x, come out as zero): the streamed
-// operand of a product whose output is several column tiles wide, split once here instead of once per column tile
-// inside the product.  Scaling and split as in make_planes_kernel; the exponent goes to *exp_out.  A thread converts
-// eight consecutive values (two 16-byte loads, one 16-byte store per plane).
-// `predicted` (may be null): the hi plane was already written by the kernel that produced x, scaled by 2^(*predicted),
-// an exponent chosen before max|x| was known (from the previous iteration's maximum, see tc_predict_exp).  If that
-// scaling turned out usable -- no overflow, at least 11 bits left: max|x| 2^e in [2^4, 2^15) -- nothing is left to do
-// but to publish the exponent; otherwise the plane is written again here with the exponent from the true maximum.
-// Only for hi-plane-only operands (lo == nullptr): 11 bits are all such a product wants.
+// ---- planes of a stored matrix -----------------------------------------------------------------------
+// x [rows][ld] fp32 -> hi, lo [rows][ld] halves (the padding columns, zero in x, come out as zero), scaled by the exponent of
+// max|x|, which goes to *exp_out: for operands whose planes no kernel wrote (the start, after pdadmm_set_tensor, the
+// prediction's activations).  A thread converts eight consecutive values.
 __global__ void __launch_bounds__(256)
 rows_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__restrict__ amax, int *__restrict__ exp_out,
-                   __half *__restrict__ hi, __half *__restrict__ lo, const int *__restrict__ predicted = nullptr) {
-  if (predicted != nullptr && lo == nullptr && tc_prediction_usable(*amax, *predicted)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *exp_out = *predicted;
-    return;
-  }
+                   __half *__restrict__ hi, __half *__restrict__ lo /* may be null */) {
   const int e = tc_scale_exp(*amax);
   if (blockIdx.x == 0 && threadIdx.x == 0) *exp_out = e;
-  const float scale = __uint_as_float((uint32_t)(e + 127) << 23);
+  const float scale = tc_pow2(e);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 a = reinterpret_cast<const float4 *>(x)[2 * i], b = reinterpret_cast<const float4 *>(x)[2 * i + 1];
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    float h[8], l[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float xs = v[k] * scale;
-      h[k] = __uint_as_float((__float_as_uint(xs) + 0x1000u) & 0xFFFFE000u);
-      l[k] = (xs - h[k]) * 2048.0f;
-    }
-    auto pack = [](float p, float q) {
-      const __half2 t = __floats2half2_rn(p, q);
-      return *reinterpret_cast<const uint32_t *>(&t);
-    };
-    reinterpret_cast<uint4 *>(hi)[i] = make_uint4(pack(h[0], h[1]), pack(h[2], h[3]), pack(h[4], h[5]), pack(h[6], h[7]));
-    if (lo != nullptr)        // a product that only wants its squared norm uses the hi plane alone
-      reinterpret_cast<uint4 *>(lo)[i] = make_uint4(pack(l[0], l[1]), pack(l[2], l[3]), pack(l[4], l[5]), pack(l[6], l[7]));
-  }
-}
-
-// ---- fp16 planes of a node-major matrix, transposed -------------------------------------------------
-// x [rows = nodes][ld] fp32 -> hiT, loT [cols][ldT] with the node index contiguous: operands of the product that
-// contracts over the nodes (the W-gradient r^T p+), for layers where splitting them once here is cheaper than
-// splitting them once per output tile inside that product.  Scaling and split as in make_planes_kernel; the
-// exponent goes to *exp_out.
-// A warp handles 32 nodes x 32 columns: lane (q, g) loads the 4 x 8 block of nodes 4q..4q+3, columns 8g..8g+7
-// (eight 16-byte loads, 128 contiguous bytes per row and warp), transposes it in registers and stores, per column,
-// the four nodes as 8 bytes of each plane (64 contiguous bytes per column and warp): whole sectors both ways, no
-// shared memory.  Tiles are numbered with the node index fastest.
-__global__ void __launch_bounds__(256)
-transpose_planes_kernel(const float *__restrict__ x, int rows, int cols, int ld, const uint32_t *__restrict__ amax,
-                        int *__restrict__ exp_out, __half *__restrict__ hiT, __half *__restrict__ loT, int ldT) {
-  const int e = tc_scale_exp(*amax);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *exp_out = e;
-  const float scale = __uint_as_float((uint32_t)(e + 127) << 23);
-  const int lane = threadIdx.x & 31, q = lane & 7, g = lane >> 3;
-  const long long row_tiles = (rows + 31) / 32, n_tiles = row_tiles * ((cols + 31) / 32);
-  for (long long wt = blockIdx.x * 8ll + (threadIdx.x >> 5); wt < n_tiles; wt += gridDim.x * 8ll) {
-    const int node0 = (int)(wt % row_tiles) * 32 + 4 * q, col = (int)(wt / row_tiles) * 32 + 8 * g;
-    if (node0 >= rows || col >= cols) continue;
-    float v[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0;
-      if (node0 + i < rows) {                  // ld is a multiple of 4: a group of 4 columns is inside the row or not
-        t0 = *reinterpret_cast<const float4 *>(x + (size_t)(node0 + i) * ld + col);
-        if (col + 4 < ld) t1 = *reinterpret_cast<const float4 *>(x + (size_t)(node0 + i) * ld + col + 4);
-      }
-      v[i][0] = t0.x; v[i][1] = t0.y; v[i][2] = t0.z; v[i][3] = t0.w;
-      v[i][4] = t1.x; v[i][5] = t1.y; v[i][6] = t1.z; v[i][7] = t1.w;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (col + j >= cols) break;
-      float h[4], l[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float xs = v[i][j] * scale;
-        h[i] = __uint_as_float((__float_as_uint(xs) + 0x1000u) & 0xFFFFE000u);
-        l[i] = (xs - h[i]) * 2048.0f;
-      }
-      const __half2 h0 = __floats2half2_rn(h[0], h[1]), h1 = __floats2half2_rn(h[2], h[3]);
-      const __half2 l0 = __floats2half2_rn(l[0], l[1]), l1 = __floats2half2_rn(l[2], l[3]);
-      const size_t o = (size_t)(col + j) * ldT + node0;
-      *reinterpret_cast<uint2 *>(hiT + o) = make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
-      *reinterpret_cast<uint2 *>(loT + o) = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
-    }
+    uint4 h, l;
+    tc_split8(reinterpret_cast<const float4 *>(x)[2 * i], reinterpret_cast<const float4 *>(x)[2 * i + 1], scale, h, l);
+    reinterpret_cast<uint4 *>(hi)[i] = h;
+    if (lo != nullptr) reinterpret_cast<uint4 *>(lo)[i] = l;
   }
 }
 
 // ---- reduction of the split partial tiles of grad_W, scaling by nu, ||grad_W||^2 ------------------
 __global__ void __launch_bounds__(EW_THREADS)
 reduce_gradW_kernel(const float *__restrict__ part, int n_split, size_t n4, float nu, float *__restrict__ G,
-                    uint32_t *__restrict__ amax, double *__restrict__ slots) {
+                    uint32_t *__restrict__ amax, double *__restrict__ slots, PlaneOut planes) {
   __shared__ double red[EW_THREADS / 32];
+  const float scale = planes.hi != nullptr ? tc_scale_of(*planes.exp) : 1.f;
   double ss = 0.0;
   uint32_t m = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
@@ -469,9 +365,10 @@ reduce_gradW_kernel(const float *__restrict__ part, int n_split, size_t n4, floa
     a.x *= nu; a.y *= nu; a.z *= nu; a.w *= nu;
     ss += (double)a.x * a.x + (double)a.y * a.y + (double)a.z * a.z + (double)a.w * a.w;
     st4(G, i, a);
+    if (planes.hi != nullptr) store_planes4(planes, i, a, scale);
     m = max(m, abs_bits(a));
   }
-  if (amax != nullptr) commit_amax(m, amax);        // for the fp16 planes of the tensor-core product G p+
+  if (amax != nullptr) commit_amax(m, amax);        // the product G p+ checks the planes' scaling with it
   const double tot = block_sum<EW_THREADS>(ss, red);
   if (threadIdx.x == 0) slots[blockIdx.x] = tot;
 }
@@ -588,8 +485,10 @@ zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, 
            const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
            float rho, float nu, float slope, float q_scale, float q_lo, float q_top, float *__restrict__ t_next,
            double *__restrict__ slots, uint32_t *__restrict__ amax_r /* max|r| (see commit_amax); may be null */,
-           const void *__restrict__ codes_next = nullptr /* pdADMM-G-Q: codes of p_next, read instead of it */, int wide_codes = 0) {
+           PlaneOut rp /* planes of r for the coming p-gradient */,
+           const void *__restrict__ codes_next /* pdADMM-G-Q: codes of p_next, read instead of it */, int wide_codes) {
   __shared__ double red[EW_THREADS / 32];
+  const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
   const float inv_rn = 1.0f / (rho + nu), inv_neg = 1.0f / (2.0f + slope * slope);
   double ss = 0.0;
   uint32_t mr = 0u;
@@ -617,6 +516,7 @@ zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, 
     PD_ZQU(x) PD_ZQU(y) PD_ZQU(z) PD_ZQU(w)
 #undef PD_ZQU
     st4(z, i, zn); st4(q, i, qn); st4(u, i, un); st4(r, i, rn); st4(t_next, i, tn);
+    if (rp.hi != nullptr) store_planes4(rp, i, rn, scale);
     mr = max(mr, abs_bits(rn));
   }
   if (amax_r != nullptr) commit_amax(mr, amax_r);
@@ -690,13 +590,14 @@ __global__ void __launch_bounds__(EW_THREADS)
 zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, float *__restrict__ u,
                  const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
                  float rho, float nu, float act, float t_lo, float t_step, int T, float q_scale, float q_lo, float q_top,
-                 float *__restrict__ t_next, double *__restrict__ slots, uint32_t *__restrict__ amax_r,
-                 const void *__restrict__ codes_next = nullptr, int wide_codes = 0) {
+                 float *__restrict__ t_next, double *__restrict__ slots, uint32_t *__restrict__ amax_r, PlaneOut rp,
+                 const void *__restrict__ codes_next, int wide_codes) {
   extern __shared__ float table_sh[];              // f(z_i)
   __shared__ double red[EW_THREADS / 32];
   for (int i = threadIdx.x; i < T; i += blockDim.x) table_sh[i] = act_eval(__fadd_rn(t_lo, __fmul_rn((float)i, t_step)), act);
   __syncthreads();
   const float inv_rn = 1.0f / (rho + nu);
+  const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
   double ss = 0.0;
   uint32_t mr = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
@@ -722,6 +623,7 @@ zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict
     st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(q, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
     st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
     const float4 r4 = make_float4(rn[0], rn[1], rn[2], rn[3]);
+    if (rp.hi != nullptr) store_planes4(rp, i, r4, scale);
     st4(r, i, r4); st4(t_next, i, make_float4(tn[0], tn[1], tn[2], tn[3]));
     mr = max(mr, abs_bits(r4));
   }
@@ -1000,20 +902,22 @@ argmax_kernel(const float *__restrict__ z, const int *__restrict__ labels, const
   if (threadIdx.x == 0) *counter = 0;
 }
 
-// W+ = W - grad_W * inv_theta  (Eq. "update W")
+// W+ = W - grad_W * inv_theta  (Eq. "update W"), with the planes of W+
 __global__ void __launch_bounds__(EW_THREADS)
 wstep_kernel(float *__restrict__ W, const float *__restrict__ G, const LayerScalars *__restrict__ sc, size_t n4,
-             uint32_t *__restrict__ amax) {
+             uint32_t *__restrict__ amax, PlaneOut planes) {
   const float a = sc->inv_theta;
+  const float scale = planes.hi != nullptr ? tc_scale_of(*planes.exp) : 1.f;
   uint32_t m = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float4 v = ld4(W, i);
     const float4 g = ld4(G, i);
     v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
     st4(W, i, v);
+    if (planes.hi != nullptr) store_planes4(planes, i, v, scale);
     m = max(m, abs_bits(v));
   }
-  if (amax != nullptr) commit_amax(m, amax);        // max|W+| for the fp16 planes of the tensor-core products
+  if (amax != nullptr) commit_amax(m, amax);        // the next W-step bounds W by it
 }
 
 }  // namespace pd

@@ -9,6 +9,8 @@
 //                                                     K = nodes, split over grid.z into partial tiles)
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "common.cuh"
 
 namespace pd {
@@ -20,7 +22,7 @@ constexpr int SG_BM = 128, SG_BN = 128, SG_BK = 8, SG_THREADS = 256;
 // read soon (the tensor-core kernel issues it when it starts a tile).
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// kDirect: the output is the accumulator itself (the tensor-core kernel then stores the tile by TMA);
+// kDirect: the output is the accumulator itself;
 // kSumsq: the epilogue accumulates the sum of squares of the output.
 // `amax` (epilogues that feed a later tensor-core product): word that receives max|C| as a bit pattern; may be null.
 struct EpiStore {             // C = acc
@@ -31,9 +33,9 @@ struct EpiStore {             // C = acc
   __device__ __forceinline__ float4 operator()(int, int, float4 a, double &) const { return a; }
 };
 struct EpiStoreSumsq {        // C = acc, accumulates sum(acc^2)
-  static constexpr bool kDirect = true, kSumsq = true;
+  static constexpr bool kDirect = true, kSumsq = true, kAmax = true;
   static constexpr int kInputs = 0;
-  float *C; int ldc;
+  float *C; int ldc; uint32_t *amax = nullptr;
   __device__ __forceinline__ void prefetch(int, int) const {}
   __device__ __forceinline__ float4 operator()(int, int, float4 a, double &ss) const {
     ss += (double)a.x * a.x + (double)a.y * a.y + (double)a.z * a.z + (double)a.w * a.w;
@@ -52,7 +54,7 @@ struct EpiNormOnly {          // nothing is stored: only sum(acc^2) is wanted (|
   }
 };
 struct EpiLinearResidual {    // C = acc + b[col] - Z[row][col]     (r = W p + b - z)
-  static constexpr bool kDirect = false, kSumsq = false;
+  static constexpr bool kDirect = false, kSumsq = false, kAmax = true;
   static constexpr int kInputs = 1;        // float4 loads per output group: load() fetches, apply() combines
   float *C; int ldc; const float *bias; const float *Z; uint32_t *amax;
   __device__ __forceinline__ void prefetch(int row, int col) const { prefetch_l2(Z + (size_t)row * ldc + col); }
@@ -70,9 +72,10 @@ struct EpiLinearResidual {    // C = acc + b[col] - Z[row][col]     (r = W p + b
   }
 };
 struct EpiAddSumsq {          // C = acc + R, accumulates sum(acc^2)     (the quantised step: r + W d beside ||W d||^2)
-  static constexpr bool kDirect = false, kSumsq = true, kSumsqOfAcc = true;
+  static constexpr bool kDirect = false, kSumsq = true, kSumsqOfAcc = true, kAmax = true, kPlanes = true;
   static constexpr int kInputs = 1;
   float *C; int ldc; const float *R; uint32_t *amax;
+  __half *H = nullptr, *L = nullptr; const int *h_exp = nullptr;      // planes of the result (tensor-core kernel only)
   __device__ __forceinline__ void prefetch(int row, int col) const { prefetch_l2(R + (size_t)row * ldc + col); }
   __device__ __forceinline__ void load(int row, int col, float4 *in) const {
     in[0] = *reinterpret_cast<const float4 *>(R + (size_t)row * ldc + col);
@@ -88,7 +91,7 @@ struct EpiAddSumsq {          // C = acc + R, accumulates sum(acc^2)     (the qu
   }
 };
 struct EpiBiasAct {           // C = acc + b[col], then f (selected by `slope`, see act_eval) if relu != 0   (z = W p + b, p' = f(z))
-  static constexpr bool kDirect = false, kSumsq = false;
+  static constexpr bool kDirect = false, kSumsq = false, kAmax = true;
   static constexpr int kInputs = 0;
   float *C; int ldc; const float *bias; int relu; float slope; uint32_t *amax;
   __device__ __forceinline__ float f(float x) const { return act_eval(x, slope); }
@@ -104,9 +107,10 @@ struct EpiBiasAct {           // C = acc + b[col], then f (selected by `slope`, 
 };
 struct EpiGradT {             // C = nu*acc + T, accumulates sum(C^2); T = u_{l-1} + rho (p_l - q_{l-1}) is kept
                               // up to date by the kernel that updates q and u (p-gradient of Eq. "update p")
-  static constexpr bool kDirect = false, kSumsq = true;
+  static constexpr bool kDirect = false, kSumsq = true, kAmax = true, kPlanes = true;
   static constexpr int kInputs = 1;
   float *C; int ldc; const float *T; float nu; uint32_t *amax;
+  __half *H = nullptr, *L = nullptr; const int *h_exp = nullptr;      // planes of the result (tensor-core kernel only)
   __device__ __forceinline__ void load(int row, int col, float4 *in) const {
     in[0] = *reinterpret_cast<const float4 *>(T + (size_t)row * ldc + col);
   }
@@ -122,13 +126,6 @@ struct EpiGradT {             // C = nu*acc + T, accumulates sum(C^2); T = u_{l-
     return g;
   }
 };
-struct EpiGradTCopy : EpiGradT {   // the same, and (tensor-core kernel only) the result once more as an fp16 plane H [rows][ldc],
-                                   // scaled by 2^(*h_exp) and rounded to 11 bits like the hi plane of an operand
-                                   // (rows_planes_kernel says what it is for)
-  static constexpr bool kHalfCopy = true;
-  __half *H; const int *h_exp;
-};
-
 // ---- NT kernel -----------------------------------------------------------------------------------
 // Thread (tx, ty) of a 16x16 block owns rows {ty*4+i, 64+ty*4+i} and columns {tx*4+j, 64+tx*4+j}.
 // Rows are padded to a multiple of 4 columns and every group of 4 columns starts at a multiple of 4,

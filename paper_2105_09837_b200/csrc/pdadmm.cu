@@ -53,19 +53,32 @@ static const char *kclass_names[KC_COUNT] = {
     "gemm_resid", "gemm_gradp", "gemm_wg", "gemm_gradw", "gradw_reduce", "gemm_gp", "axpy",
     "quant_trial", "resid_colsum", "zqu", "zlast", "wstep", "finalize", "absmax", "make_planes"};
 
-// fp16 hi/lo planes of a weight-sized matrix [rows][cols] for the tensor-core products, in the orientation(s)
-// in which it is contracted, and the exponent of the power-of-two scaling they were made with.
+// fp16 hi/lo planes of a matrix, in its own orientation and with its leading dimension, and the device word with the
+// exponent of the power-of-two scaling they were made with.
 struct Planes {
-  __half *hi = nullptr, *lo = nullptr;     // [rows][ldh], ldh = cols rounded up to 8
-  __half *hiT = nullptr, *loT = nullptr;   // [cols][ldhT], ldhT = rows rounded up to 8 (only where needed)
-  int ldh = 0, ldhT = 0;
-  int *exp = nullptr;                      // device word
+  __half *hi = nullptr, *lo = nullptr;
+  int *exp = nullptr;
 };
-// one operand of a tensor-core product as two fp16 planes [n][ld], contiguous along the contraction index
-struct PlaneRef { const __half *hi, *lo; int ld; const int *exp; };
-// an operand that is `mul` times small integers (a quantised p = code * s, or the difference of two): one fp16 plane
-// of the integers [n][ld], no lo plane
-struct IntPlane { const __half *plane; int ld; float mul; };
+// One operand of a tensor-core product: its planes [rows][ld] (hi null: to be split first, from x), and, where the exponent was
+// chosen before the largest magnitude was known, the word `check` with that magnitude, by which the product decides whether
+// the planes are good or have to be made again from x.  int_mul > 0: hi holds small integers that are to be multiplied by
+// int_mul (a quantised p = code * s, or the difference of two), there is no lo plane.
+struct Operand {
+  const float *x; int ld;
+  const uint32_t *amax;             // for splitting x first (null: computed)
+  const __half *hi = nullptr, *lo = nullptr;
+  const int *exp = nullptr;
+  const uint32_t *check = nullptr;
+  float int_mul = 0.f;
+};
+static Operand int_operand(const __half *plane, int ld, float mul) {
+  Operand o{nullptr, ld, nullptr};
+  o.hi = plane; o.lo = plane; o.int_mul = mul;
+  return o;
+}
+static Operand plane_operand(const float *x, int ld, const Planes &p, const uint32_t *check = nullptr) {
+  return Operand{x, ld, check, p.hi, p.lo, p.exp, check};
+}
 
 // Rows of every node-major matrix start on a 128-byte boundary (leading dimensions are multiples of 32 floats):
 // tile copies and the coalesced stores of the epilogues then move whole 32-byte sectors.
@@ -84,13 +97,12 @@ struct Layer {
   float *q = nullptr, *u = nullptr;          // [N][ld_out], hidden layers only
   float *t = nullptr;       // [N][ld_in], l >= 2: u_{l-1} + rho (p_l - q_{l-1}), the product-free part of grad_p phi
   float *gradW = nullptr;   // [n_out][ld_in]
-  Planes Wp;                // fp16 planes of W: [n_out][ldh_in], and of W^T: [n_in][ldh_out] (tensor-core path)
-  Planes Gp;                // fp16 planes of grad_W: [n_out][ldh_in]
-  __half *xT_hi = nullptr, *xT_lo = nullptr;   // layer 1 only: transposed planes of p_1 = X, which never changes
-  int *xT_exp = nullptr;
-  __half *x_hi = nullptr, *x_lo = nullptr;     // layer 1 only: planes of X in its own orientation [N][ld_in]
-  int *x_exp = nullptr;
-  int *g_exp = nullptr;     // l >= 2: exponent predicted for the scaling of the next fp16 copy of g_l (tc_predict_exp)
+  // Tensor-core path: planes of W, of grad_W and of r (written by the z-step for the next p-gradient; hidden layers only, and
+  // none if the device has no room: the products then split r first), of p_1 = X, which never changes; the exponent words
+  // belong to finalize_tau_kernel / finalize_theta_kernel, which settle them before the planes are written
+  Planes Wp, Gp, rp, xp;
+  int *g_exp = nullptr;     // l >= 2: exponent of the next planes of g_l
+  uint32_t *amax_W = nullptr;      // max|W|, bit pattern
   float *shift = nullptr;   // [ld_out] column means removed by the b-update
   uint8_t *codes = nullptr; // [N][ld_in] codes of 1 byte (up to 256 levels) or 2 bytes, quantised mode, l >= 2
   __half *p_plane = nullptr; // [N][ld_in] the codes as fp16 integers: operand plane of p_l = code * scale (see int_operands)
@@ -120,17 +132,12 @@ struct Scratch {
   int *tail_count = nullptr;
   uint32_t *amax_pool = nullptr;   // words for the largest magnitudes of product operands, handed out in stream order
   int amax_next = 0;
-  // transposed fp16 planes ([width][ldT], node index contiguous) of r_l and p_l for the product over the nodes
-  __half *rT_hi = nullptr, *rT_lo = nullptr, *pT_hi = nullptr, *pT_lo = nullptr;
-  int *rT_exp = nullptr, *pT_exp = nullptr;
-  // planes [N][ld] of the streamed operand of a product over several column tiles (split once per product)
-  __half *a_hi = nullptr, *a_lo = nullptr;
-  size_t a_cap = 0;                // elements each of the two holds
+  // planes [N][ld] of node-sized operands, as wide as the widest matrix of the context.  pl0: of g, from the p-gradient to
+  // W g; then of r after the p-step (or the accepted trial), up to the W-gradient.  pl1: of p after the p-step, up to G p+;
+  // before that and outside iterations, of any operand that has to be split first.
+  Planes pl0, pl1;
   int *a_exp = nullptr;
-  // quantised mode: fp16 copy [N][ld] of g, written by the epilogue of the p-gradient's product with a predicted
-  // scaling, for the norm-only product W g that follows (rows_planes_kernel)
-  __half *g_hi = nullptr;
-  int *g_hi_exp = nullptr;
+  size_t pl_cap = 0;               // elements each plane holds
   int *h_flag = nullptr;           // pinned word that receives the accept flag of the lane's quantised trial
   cudaEvent_t ev_flag = nullptr;   // recorded after the copy of that flag
 };
@@ -205,9 +212,8 @@ struct pdadmm_ctx {
   int n_sms = 148;
   bool w_planes_valid = false;
   bool amax_p_valid = false;        // every layer's amax_p covers the stored p
-  bool xT_valid = false;            // the transposed planes of X match the stored X
-  int ldT = 0;                      // leading dimension of transposed planes: N rounded up to 8
-  std::map<std::tuple<const void *, uint64_t, uint64_t, uint64_t, uint32_t, uint32_t>, CUtensorMap> tmaps;
+  bool x_planes_valid = false;      // the planes of X match the stored X
+  std::map<std::tuple<const void *, uint64_t, uint64_t, uint64_t>, CUtensorMap> tmaps;
 };
 
 namespace pd {
@@ -315,30 +321,22 @@ static EncodeTiledFn encode_tiled_fn() {
   }();
   return fn;
 }
-// Operand tiles of the tensor-core products; elements outside the matrix read as zero.
-//   TM_RAW_K:  fp32 [outer][inner], tile = box of 32 floats x 128 rows, 128-byte swizzle (the contraction index is the
-//              inner one; a 64-deep K block is two such boxes)
-//   TM_RAW_MN: fp32 [outer][inner], tile = 128 floats x 64 rows, no swizzle (the contraction index is the outer one;
-//              only the converter warps read it)
-//   TM_PLANE:  fp16 [outer][inner], tile = 64 halves x 128 rows, 128-byte swizzle (what the MMA reads)
-enum TmapKind { TM_RAW_K = 0, TM_RAW_MN = 1, TM_PLANE = 2 };
-static int get_tmap(pdadmm_ctx *c, const void *base, uint64_t inner, uint64_t outer, uint64_t ld, TmapKind kind,
-                    CUtensorMap *out) {
-  auto key = std::make_tuple(base, inner, outer, ld, (uint32_t)kind, 0u);
+// Operand tiles of the tensor-core products: 64 x 64 halves of a plane [outer][inner], 128-byte swizzle; elements outside the
+// matrix read as zero.
+static int get_tmap(pdadmm_ctx *c, const void *base, uint64_t inner, uint64_t outer, uint64_t ld, CUtensorMap *out) {
+  auto key = std::make_tuple(base, inner, outer, ld);
   auto it = c->tmaps.find(key);
   if (it != c->tmaps.end()) { *out = it->second; return PDADMM_OK; }
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return fail(PDADMM_ECUDA, "cuTensorMapEncodeTiled is not available in this driver");
-  const uint64_t esize = kind == TM_PLANE ? 2 : 4;
   cuuint64_t dims[2] = {inner, outer};
-  cuuint64_t strides[1] = {ld * esize};
-  cuuint32_t box[2] = {kind == TM_RAW_K ? 32u : (kind == TM_RAW_MN ? 128u : 64u), kind == TM_RAW_MN ? 64u : 128u};
+  cuuint64_t strides[1] = {ld * 2};
+  cuuint32_t box[2] = {64u, 64u};
   cuuint32_t estr[2] = {1, 1};
   CUtensorMap m;
-  const CUresult r = fn(&m, kind == TM_PLANE ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                        const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        kind == TM_RAW_MN ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  const CUresult r = fn(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(PDADMM_ECUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
   if (c->tmaps.size() > 4096) c->tmaps.clear();
   c->tmaps[key] = m;
@@ -346,15 +344,22 @@ static int get_tmap(pdadmm_ctx *c, const void *base, uint64_t inner, uint64_t ou
   return PDADMM_OK;
 }
 
-template <int MODE, class Epi, int ZERO = 0>
-static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap &ma, const CUtensorMap &mal, const CUtensorMap &mb,
-                     const CUtensorMap &mbl, const TcParams &prm, const Epi &epi, double *partials, int n_tiles) {
-  auto kern = gemm_tc_kernel<MODE, Epi, ZERO>;
-  const dim3 grid((unsigned)std::min(n_tiles, c->n_sms));
+// Whether a product of M x N outputs in n_split slices runs on pairs of SMs: they halve the traffic of B, but a pair's tile has
+// 256 rows.  So: where at least three quarters of the pairs get a tile, and padding M to 256 rows instead of 128 adds at most
+// a tenth.  (20 000 x 500 x 500: 43.2 us in pairs, 45.5 us without; x 2000 x 2000: 399 against 457 us; 2000 x 100 x 100, 8
+// pairs: 12.5 against 10.7 us.)
+static bool use_pairs(const pdadmm_ctx *c, int M, int N, int n_split) {
+  const int64_t m1 = ceil_div(M, TC_BM), m2 = 2 * ceil_div(M, 2 * TC_BM);
+  return m2 * 10 <= m1 * 11 && (m2 / 2) * ceil_div(N, TC_BN) * n_split * 8 >= 3 * (int64_t)c->n_sms;
+}
+template <int LAYOUT, class Epi, int ZERO, bool PAIR>
+static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap (&maps)[4], const TcParams &prm, const Epi &epi,
+                          double *partials, int n_units) {
+  auto kern = gemm_tc_kernel<LAYOUT, Epi, ZERO, PAIR>;
   // the attribute belongs to (kernel, device): one flag per device ordinal for this instantiation
-  static bool configured[64] = {false};
+  static bool configured[MAX_DEVICES] = {false};
   const int dev = c->device;
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
+  if (dev < 0 || dev >= MAX_DEVICES || !configured[dev]) {
     // The kernel's warpgroups re-divide the registers the block is launched with; their shares were added up
     // against TC_REGS_LAUNCH per thread.  A build that launches with fewer would make an increase wait for ever:
     // refuse to launch it.
@@ -364,10 +369,59 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap &ma, cons
       return fail(PDADMM_ECUDA, "tensor-core product kernel was built with %d registers per thread, %d expected",
                   attr.numRegs, TC_REGS_LAUNCH);
     PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
-    if (dev >= 0 && dev < 64) configured[dev] = true;
+    if (dev >= 0 && dev < MAX_DEVICES) configured[dev] = true;
   }
-  kern<<<grid, TC_THREADS, TC_SMEM_BYTES, st>>>(ma, mal, mb, mbl, prm, epi, partials);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(PAIR ? 2 * std::min(n_units, c->n_sms / 2) : std::min(n_units, c->n_sms)));
+  cfg.blockDim = dim3(TC_THREADS);
+  cfg.dynamicSmemBytes = TC_SMEM_BYTES;
+  cfg.stream = st;
+  cudaLaunchAttribute cluster;
+  cluster.id = cudaLaunchAttributeClusterDimension;
+  cluster.val.clusterDim.x = 2; cluster.val.clusterDim.y = 1; cluster.val.clusterDim.z = 1;
+  cfg.attrs = &cluster;
+  cfg.numAttrs = PAIR ? 1 : 0;
+  PD_CUDA(cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], prm, epi, partials));
   return PDADMM_OK;
+}
+// op(A) is M x K, op(B) is N x K; A_MN: A is stored [K][M], B_MN: B is stored [K][N].  The tail of the persistent grid is
+// balanced here (prm.tail_*), *n_partials receives the number of slots.
+template <int LAYOUT, class Epi, int ZERO = 0>
+static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Operand &A, const Operand &B, TcParams prm, const Epi &epi,
+                     double *partials, int *n_partials) {
+  constexpr bool A_MN = (LAYOUT & TC_A_MN) != 0, B_MN = (LAYOUT & TC_B_MN) != 0;
+  const uint64_t M = (uint64_t)prm.M, N = (uint64_t)prm.N, K = (uint64_t)prm.K;
+  CUtensorMap maps[4];
+  PD_TRY(get_tmap(c, A.hi, A_MN ? M : K, A_MN ? K : M, (uint64_t)A.ld, &maps[0]));
+  if (A.lo && A.lo != A.hi) PD_TRY(get_tmap(c, A.lo, A_MN ? M : K, A_MN ? K : M, (uint64_t)A.ld, &maps[1]));
+  else maps[1] = maps[0];
+  PD_TRY(get_tmap(c, B.hi, B_MN ? N : K, B_MN ? K : N, (uint64_t)B.ld, &maps[2]));
+  if (B.lo && B.lo != B.hi) PD_TRY(get_tmap(c, B.lo, B_MN ? N : K, B_MN ? K : N, (uint64_t)B.ld, &maps[3]));
+  else maps[3] = maps[2];
+  prm.error = c->d_flag + 1;
+  prm.a = TcOperand{A.exp, A.check, A.x, A.ld};
+  prm.b = TcOperand{B.exp, B.check, B.x, B.ld};
+  const bool pair = use_pairs(c, prm.M, prm.N, prm.n_split);
+  const int n_tiles = (int)(ceil_div(prm.M, pair ? 2 * TC_BM : TC_BM) * ceil_div(prm.N, TC_BN)) * prm.n_split;
+  const int slots = pair ? c->n_sms / 2 : c->n_sms;          // tiles under way at a time
+  if (n_partials) *n_partials = (pair ? 8 : 4) * n_tiles;    // one slot per tile and row quarter
+  // The persistent grid works through the tiles in rounds; a last round that fills only part of the
+  // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit.
+  int n_units = n_tiles;
+  const int tail = n_tiles % slots, n_kb = (int)ceil_div(prm.K, TC_BK);
+  if (prm.n_split == 1 && tail > 0 && c->cur->tail_ws != nullptr) {
+    // at least 8 K blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks,
+    // and with two lanes the other layer's kernels fill the SMs that a short last round leaves idle (workload c2,
+    // 8 K blocks per tile: 281 iterations/s with 4 slices of 2 blocks, 289 without)
+    const int split = std::min(std::min(slots / tail, n_kb / 8), 8);
+    if (split > 1) {
+      prm.tail_begin = n_tiles - tail; prm.tail_split = split;
+      prm.tail_ws = c->cur->tail_ws; prm.tail_count = c->cur->tail_count;
+      n_units = prm.tail_begin + tail * split;
+    }
+  }
+  if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, maps, prm, epi, partials, n_units);
+  return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, maps, prm, epi, partials, n_units);
 }
 
 // ---- largest magnitudes of product operands ------------------------------------------------------------------
@@ -394,205 +448,112 @@ static uint32_t *amax_of(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t 
   return w;
 }
 
-// fp16 planes of x [rows][ld] (cols valid columns) from the largest magnitude in *amax
-static void make_planes(pdadmm_ctx *c, cudaStream_t st, const float *x, int rows, int cols, int ld, const uint32_t *amax,
-                        Planes &pl) {
-  Launch l(c, KC_PLANES, st, (4.0 + 4.0 + (pl.hiT ? 4.0 : 0.0)) * rows * cols, 0);
-  const dim3 grid((unsigned)ceil_div(cols, 32), (unsigned)ceil_div(rows, 32));
-  make_planes_kernel<<<grid, dim3(32, 8), 0, st>>>(x, rows, cols, ld, amax, pl.exp, pl.hi, pl.lo, pl.ldh, pl.hiT, pl.loT,
-                                                   pl.ldhT);
+// planes of x [rows][ld] from the largest magnitude in *amax (lo_too: both planes)
+static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t rows, int cols, int ld, const uint32_t *amax,
+                       const Planes &pl, bool lo_too = true) {
+  const size_t n8 = rows * ld / 8;
+  Launch l(c, KC_PLANES, st, (lo_too ? 8.0 : 6.0) * rows * cols, 0);
+  rows_planes_kernel<<<ew_grid(n8), 256, 0, st>>>(x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
 }
-// the same for a matrix whose largest magnitude is not known yet
-static int split_planes(pdadmm_ctx *c, cudaStream_t st, const float *x, int rows, int cols, int ld, Planes &pl) {
+static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
+  PD_TRY(dev_alloc(c, &pl->hi, n, zero));
+  PD_TRY(dev_alloc(c, &pl->lo, n, zero));
+  return dev_alloc(c, &pl->exp, 1);
+}
+// planes of W_l and its largest magnitude, after W was set
+static int refresh_W_planes(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
   if (!c->use_tc) return PDADMM_OK;
-  PD_TRY(amax_reserve(c, st, 1));
-  const uint32_t *w = amax_of(c, st, x, (size_t)rows * ld / 4);
-  make_planes(c, st, x, rows, cols, ld, w, pl);
-  return PDADMM_OK;
-}
-static int alloc_planes(pdadmm_ctx *c, int rows, int cols, bool transposed_too, bool natural, Planes *pl) {
-  pl->ldh = round_up(cols, 8); pl->ldhT = round_up(rows, 8);
-  if (natural) {
-    PD_TRY(dev_alloc(c, &pl->hi, (size_t)rows * pl->ldh));
-    PD_TRY(dev_alloc(c, &pl->lo, (size_t)rows * pl->ldh));
+  PD_CUDA(cudaMemsetAsync(ly.amax_W, 0, sizeof(uint32_t), st));
+  const size_t n4 = (size_t)ly.n_out * ly.ld_in / 4;
+  {
+    Launch l(c, KC_AMAX, st, 16.0 * (double)n4, 0);
+    absmax_kernel<<<ew_grid(n4), EW_THREADS, 0, st>>>(ly.W, n4, ly.amax_W);
   }
-  if (transposed_too) {
-    PD_TRY(dev_alloc(c, &pl->hiT, (size_t)cols * pl->ldhT));
-    PD_TRY(dev_alloc(c, &pl->loT, (size_t)cols * pl->ldhT));
-  }
-  PD_TRY(dev_alloc(c, &pl->exp, 1));
+  split_rows(c, st, ly.W, (size_t)ly.n_out, ly.n_in, ly.ld_in, ly.amax_W, ly.Wp);
   return PDADMM_OK;
 }
 
 // ---- dense products --------------------------------------------------------------------------------------
 // C[M][N] = A[M][K] * op(B), fused epilogue; per-block sums of squares go to `partials` (or nullptr).
-// B is given by its fp32 matrix (CUDA-core path; B_NMAJOR tells its orientation) and by its two fp16 planes
-// [N][K] (tensor-core path).  `amax_a`: the largest magnitude of A if the caller has it, else it is computed here.
-// The streamed operand A is split into its planes tile by tile inside the product, or once beforehand
-// (rows_planes_kernel into the lane's scratch, or planes the caller keeps: `Ap`).  Inside, every column tile of the
-// output converts the same rows of A again and the converters' tensor-memory stores slow the MMAs down (measured:
-// 2640 cycles per 64-deep K block against 1610 with both operands as planes); beforehand costs one pass of
-// 8 bytes per element at HBM speed.  Measured per product (split pass included): 4 column tiles 69 against 58 us,
-// 8 tiles 1.18 against 1.21 ms, 16 tiles 2.42 against 2.29 ms -- beforehand wins from 16 column tiles on, and
-// always where the planes are kept (X).  The norm-only product needs the hi plane alone (6 bytes per element) and
-// wins from 8 column tiles on (workload c4: 9.42 -> 9.74 iterations/s).
-constexpr int PLANES_FROM_COL_TILES = 16;
-template <bool B_NMAJOR, class Epi>
-static int gemm_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, const float *A, int lda,
-                      const float *B, int ldb, const PlaneRef &Bp, const Epi &epi, double *partials,
-                      int *n_partials, double extra_bytes, const uint32_t *amax_a = nullptr,
-                      const PlaneRef *Ap = nullptr, const IntPlane *Ai = nullptr) {
+// B_MN = false: B is [N][K]; true: B is [K][N].  An operand A without planes is split into the lane's pl1 first
+// (8 bytes per element; splitting inside the product, once per column tile, ran the MMAs at 0.6 of their speed).
+template <bool B_MN, class Epi>
+static int gemm_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, Operand A, const Operand &B, const Epi &epi,
+                      double *partials, int *n_partials, double extra_bytes) {
   const double bytes = 4.0 * ((double)M * K + (double)N * K + (double)M * N) + extra_bytes;
   if (!c->use_tc) {
     dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM));
     if (n_partials) *n_partials = (int)(grid.x * grid.y);
     Launch l(c, cls, st, bytes, 2.0 * M * N * K);
-    gemm_nt_kernel<B_NMAJOR, Epi><<<grid, SG_THREADS, 0, st>>>(M, N, K, A, lda, B, ldb, epi, partials);
+    gemm_nt_kernel<B_MN, Epi><<<grid, SG_THREADS, 0, st>>>(M, N, K, A.x, A.ld, B.x, B.ld, epi, partials);
     return PDADMM_OK;
   }
-  const int n_tiles = (int)(ceil_div(N, TC_BN) * ceil_div(M, TC_BM));
-  if (n_partials) *n_partials = 4 * n_tiles;        // one slot per tile and row quarter
-  const bool a_int = Ai != nullptr && Ai->plane != nullptr;
-  if (amax_a == nullptr && !a_int) {
-    PD_TRY(amax_reserve(c, st, 1));
-    amax_a = amax_of(c, st, A, (size_t)M * lda / 4);
-  }
-  PlaneRef a_planes{nullptr, nullptr, 0, nullptr};
-  if (a_int) {
-    a_planes = PlaneRef{Ai->plane, Ai->plane, Ai->ld, nullptr};
-  } else if (Ap != nullptr && Ap->hi != nullptr) {
-    a_planes = *Ap;
-  } else if (c->cur->a_hi != nullptr && lda % 8 == 0 && (size_t)M * lda <= c->cur->a_cap &&
-             (ceil_div(N, TC_BN) >= PLANES_FROM_COL_TILES || (epi_coarse<Epi>::value && ceil_div(N, TC_BN) >= PLANES_FROM_COL_TILES / 2))) {
+  if (A.hi == nullptr) {
     Scratch &sc = *c->cur;
-    const size_t n8 = (size_t)M * lda / 8;
-    constexpr bool coarse = epi_coarse<Epi>::value;
-    Launch l(c, KC_PLANES, st, (coarse ? 6.0 : 8.0) * M * K, 0);
-    rows_planes_kernel<<<ew_grid(n8), 256, 0, st>>>(A, n8, amax_a, sc.a_exp, sc.a_hi, coarse ? nullptr : sc.a_lo);
-    a_planes = PlaneRef{sc.a_hi, sc.a_lo, lda, sc.a_exp};
-  }
-  const bool pp = a_planes.hi != nullptr;
-  CUtensorMap ma, mal, mb, mbl;
-  if (pp) {
-    PD_TRY(get_tmap(c, a_planes.hi, (uint64_t)K, (uint64_t)M, (uint64_t)a_planes.ld, TM_PLANE, &ma));
-    PD_TRY(get_tmap(c, a_planes.lo, (uint64_t)K, (uint64_t)M, (uint64_t)a_planes.ld, TM_PLANE, &mal));
-  } else {
-    PD_TRY(get_tmap(c, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, TM_RAW_K, &ma));
-    mal = ma;
-  }
-  PD_TRY(get_tmap(c, Bp.hi, (uint64_t)K, (uint64_t)N, (uint64_t)Bp.ld, TM_PLANE, &mb));
-  PD_TRY(get_tmap(c, Bp.lo, (uint64_t)K, (uint64_t)N, (uint64_t)Bp.ld, TM_PLANE, &mbl));
-  TcParams prm{M, N, K, round_up(K, TC_BK), 1, 0, c->d_flag + 1, pp ? nullptr : amax_a, nullptr, pp ? a_planes.exp : nullptr, Bp.exp};
-  // The persistent grid works through the tiles in rounds of n_sms; a last round that fills only part of the
-  // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit.
-  int n_units = n_tiles;
-  const int tail = n_tiles % c->n_sms, n_kb = (int)ceil_div(K, TC_BK);
-  if (tail > 0 && c->cur->tail_ws != nullptr) {
-    // at least 8 K blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks,
-    // and with two lanes the other layer's kernels fill the SMs that a short last round leaves idle (workload c2,
-    // 8 K blocks per tile: 281 iterations/s with 4 slices of 2 blocks, 289 without)
-    const int split = std::min(std::min(c->n_sms / tail, n_kb / 8), 8);
-    if (split > 1) {
-      prm.tail_begin = n_tiles - tail; prm.tail_split = split;
-      prm.tail_ws = c->cur->tail_ws; prm.tail_count = c->cur->tail_count;
-      n_units = prm.tail_begin + tail * split;
+    if ((size_t)M * A.ld > sc.pl_cap || A.ld % 8) return fail(PDADMM_EINVAL, "operand does not fit the lane's planes");
+    if (A.amax == nullptr) {
+      PD_TRY(amax_reserve(c, st, 1));
+      A.amax = amax_of(c, st, A.x, (size_t)M * A.ld / 4);
     }
+    const Planes pl{sc.pl1.hi, sc.pl1.lo, sc.a_exp};
+    split_rows(c, st, A.x, (size_t)M, K, A.ld, A.amax, pl, !epi_coarse<Epi>::value);
+    A.hi = pl.hi; A.lo = pl.lo; A.exp = pl.exp; A.check = nullptr;
   }
+  TcParams prm = {};
+  prm.M = M; prm.N = N; prm.K = K; prm.k_chunk = round_up(K, TC_BK); prm.n_split = 1; prm.mul = 1.f;
+  constexpr int LAYOUT = B_MN ? TC_B_MN : TC_NT;
   Launch l(c, cls, st, bytes, 2.0 * M * N * K);
-  if constexpr (std::is_same<Epi, EpiStoreSumsq>::value || std::is_same<Epi, EpiAddSumsq>::value) {
-    if (a_int) {
-      prm.mul = Ai->mul;
-      return launch_tc<TC_PLANES, Epi, 1>(c, st, ma, ma, mb, mbl, prm, epi, partials, n_units);
+  if (A.int_mul > 0.f) {
+    if constexpr (std::is_same<Epi, EpiStoreSumsq>::value || std::is_same<Epi, EpiAddSumsq>::value) {
+      prm.mul = A.int_mul;
+      return launch_tc<LAYOUT, Epi, 1>(c, st, A, B, prm, epi, partials, n_partials);
+    } else {
+      return fail(PDADMM_EINVAL, "no integer-operand form of this product is built");
     }
-  } else {
-    if (a_int) return fail(PDADMM_EINVAL, "no integer-operand form of this product is built");
   }
-  if (pp) return launch_tc<TC_PLANES, Epi>(c, st, ma, mal, mb, mbl, prm, epi, partials, n_units);
-  return launch_tc<TC_RAW_K, Epi>(c, st, ma, ma, mb, mbl, prm, epi, partials, n_units);
+  return launch_tc<LAYOUT, Epi>(c, st, A, B, prm, epi, partials, n_partials);
 }
 
-// transposed fp16 planes [cols][ldT] of a node-major matrix x [rows][ld] whose largest magnitude is in *amax
-static void transpose_planes(pdadmm_ctx *c, cudaStream_t st, const float *x, int rows, int cols, int ld,
-                             const uint32_t *amax, __half *hiT, __half *loT, int ldT, int *exp_out) {
-  Launch l(c, KC_PLANES, st, 8.0 * rows * cols, 0);
-  const int64_t warp_tiles = ceil_div(rows, 32) * ceil_div(cols, 32);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(warp_tiles, 8), 148 * 16));
-  transpose_planes_kernel<<<grid, 256, 0, st>>>(x, rows, cols, ld, amax, exp_out, hiT, loT, ldT);
-}
-
-// C parts [n_split][M][ldc] = A^T B over node slices, both operands given by their transposed planes:
-// A^T = [M][K nodes], B^T = [N][K nodes]
-// b_mul > 0: B^T is one plane of integers (Bt.hi; the transposed codes of a quantised p) times b_mul
-static int gemm_over_nodes_tc(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, const PlaneRef &At,
-                              const PlaneRef &Bt, float *part, int ldc, int k_chunk, int n_split, float b_mul = 0.f) {
-  const int n_tiles = (int)(ceil_div(N, TC_BN) * ceil_div(M, TC_BM)) * n_split;
-  CUtensorMap ma, mal, mb, mbl;
-  PD_TRY(get_tmap(c, At.hi, (uint64_t)K, (uint64_t)M, (uint64_t)At.ld, TM_PLANE, &ma));
-  PD_TRY(get_tmap(c, At.lo, (uint64_t)K, (uint64_t)M, (uint64_t)At.ld, TM_PLANE, &mal));
-  PD_TRY(get_tmap(c, Bt.hi, (uint64_t)K, (uint64_t)N, (uint64_t)Bt.ld, TM_PLANE, &mb));
-  if (b_mul > 0.f) mbl = mb;
-  else PD_TRY(get_tmap(c, Bt.lo, (uint64_t)K, (uint64_t)N, (uint64_t)Bt.ld, TM_PLANE, &mbl));
-  TcParams prm{M, N, K, k_chunk, n_split, (size_t)M * ldc, c->d_flag + 1, nullptr, nullptr, At.exp, b_mul > 0.f ? nullptr : Bt.exp};
+// C parts [n_split][M][ldc] = A^T B over node slices, A = [K nodes][M], B = [K nodes][N], both as planes
+static int gemm_over_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, const Operand &A, const Operand &B,
+                           float *part, int ldc, int k_chunk, int n_split) {
+  TcParams prm = {};
+  prm.M = M; prm.N = N; prm.K = K; prm.k_chunk = k_chunk; prm.n_split = n_split; prm.c_split_stride = (size_t)M * ldc; prm.mul = 1.f;
   EpiStore epi{part, ldc};
   Launch k(c, cls, st, 4.0 * ((double)K * N + (double)K * M), 2.0 * K * N * M);
-  if (b_mul > 0.f) {
-    prm.mul = b_mul;
-    return launch_tc<TC_PLANES, EpiStore, 2>(c, st, ma, mal, mb, mb, prm, epi, nullptr, n_tiles);
+  if (B.int_mul > 0.f) {
+    prm.mul = B.int_mul;
+    return launch_tc<TC_A_MN | TC_B_MN, EpiStore, 2>(c, st, A, B, prm, epi, nullptr, nullptr);
   }
-  return launch_tc<TC_PLANES, EpiStore>(c, st, ma, mal, mb, mbl, prm, epi, nullptr, n_tiles);
+  return launch_tc<TC_A_MN | TC_B_MN, EpiStore>(c, st, A, B, prm, epi, nullptr, nullptr);
 }
-
-// The same from the fp32 operands themselves, A = [K][lda] (M valid columns), B = [K][ldb] (N valid columns), which
-// the product transposes and splits tile by tile; wa, wb: their largest magnitudes.
-static int gemm_over_nodes_raw(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, const float *A, int lda,
-                               const float *B, int ldb, float *part, int ldc, int k_chunk, int n_split,
-                               const uint32_t *wa, const uint32_t *wb) {
-  const int n_tiles = (int)(ceil_div(N, TC_BN) * ceil_div(M, TC_BM)) * n_split;
-  CUtensorMap ma, mb;
-  PD_TRY(get_tmap(c, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, TM_RAW_MN, &ma));
-  PD_TRY(get_tmap(c, B, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, TM_RAW_MN, &mb));
-  TcParams prm{M, N, K, k_chunk, n_split, (size_t)M * ldc, c->d_flag + 1, wa, wb, nullptr, nullptr};
-  EpiStore epi{part, ldc};
-  Launch k(c, cls, st, 4.0 * ((double)K * N + (double)K * M), 2.0 * K * N * M);
-  return launch_tc<TC_RAW_MN, EpiStore>(c, st, ma, ma, mb, mb, prm, epi, nullptr, n_tiles);
-}
-
-// Which form the product over the nodes takes for an M x N output.  Splitting the operands inside the product
-// costs every output tile its own conversion of the operand tiles (the converter warps then set the pace, about
-// twice the time of the MMAs); splitting them beforehand costs one bandwidth-bound pass per operand.  Measured on
-// the B200: 16 output tiles (500 x 500) 88 us inside against 53 + 2 x 21 us beforehand; 64 tiles and more are
-// faster beforehand (workloads c4, c5: +2 % and +6 % per iteration), and so is layer 1, whose second operand X
-// never changes and keeps its planes.
-static bool planes_beforehand(int M, int N, bool second_operand_cached) {
-  const int64_t tiles = ceil_div(M, TC_BM) * ceil_div(N, TC_BN);
-  return tiles >= 16 || (second_operand_cached && tiles >= 8);
-}
-
-}  // namespace pd
-
-namespace pd {
 
 // ---- pieces of one iteration -------------------------------------------------------------------------------
 
-// planes of W_l as the operand of a product with rows n_out contracted over n_in (P W^T, g W^T) ...
-static PlaneRef planes_W(const Layer &ly) { return PlaneRef{ly.Wp.hi, ly.Wp.lo, ly.Wp.ldh, ly.Wp.exp}; }
-// ... and of W_l^T, rows n_in contracted over n_out (r W)
-static PlaneRef planes_WT(const Layer &ly) { return PlaneRef{ly.Wp.hiT, ly.Wp.loT, ly.Wp.ldhT, ly.Wp.exp}; }
-static PlaneRef planes_G(const Layer &ly) { return PlaneRef{ly.Gp.hi, ly.Gp.lo, ly.Gp.ldh, ly.Gp.exp}; }
-
-// planes of p_1 = X, which never changes, in its own orientation (null planes if the layer does not keep them)
-static PlaneRef planes_X(const Layer &ly) { return PlaneRef{ly.x_hi, ly.x_lo, ly.ld_in, ly.x_exp}; }
+static Operand operand_W(const Layer &ly) { return plane_operand(ly.W, ly.ld_in, ly.Wp); }
+// p_1 = X, which never changes (its planes are kept on the tensor-core path)
+static Operand operand_X(const Layer &ly) { return plane_operand(ly.p, ly.ld_in, ly.xp); }
+// r_l as the z-step left it; the last layer has no planes from there (its exponent word says so), its few columns are split by
+// the product itself
+static Operand operand_r(const Layer &ly) {
+  Operand o = plane_operand(ly.r, ly.ld_out, ly.rp, ly.amax_r);
+  o.amax = ly.amax_r;
+  return o;
+}
 
 // r_l = P_l W_l^T + b_l - z_l from scratch (only when the cached residual is not valid).
 static int refresh_residual(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
   PD_CUDA(cudaMemsetAsync(ly.amax_r, 0, sizeof(uint32_t), st));
   EpiLinearResidual epi{ly.r, ly.ld_out, ly.b, ly.z, ly.amax_r};
-  const PlaneRef xp = planes_X(ly);
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)c->N, ly.n_out, ly.n_in, ly.p, ly.ld_in, ly.W, ly.ld_in,
-                           planes_W(ly), epi, nullptr, nullptr, 4.0 * c->N * ly.n_out, ly.amax_p, &xp));
+  Operand P{ly.p, ly.ld_in, ly.amax_p};
+  if (c->use_tc && ly.xp.hi != nullptr) P = operand_X(ly);
+  PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)c->N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr,
+                           4.0 * c->N * ly.n_out));
   if (!c->use_tc) {       // the CUDA-core product does not track the maximum of what it stores
     Launch l(c, KC_AMAX, st, 4.0 * c->N * ly.ld_out, 0);
     absmax_kernel<<<ew_grid((size_t)c->N * ly.ld_out / 4), EW_THREADS, 0, st>>>(ly.r, (size_t)c->N * ly.ld_out / 4, ly.amax_r);
+  } else if (ly.rp.hi != nullptr && &ly != &c->layers.back()) {
+    split_rows(c, st, ly.r, (size_t)c->N, ly.n_out, ly.ld_out, ly.amax_r, ly.rp);
   }
   return PDADMM_OK;
 }
@@ -600,75 +561,60 @@ static int refresh_residual(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
 // g = nu r W + u_{l-1} + rho (p - q_{l-1}) -> s1, ||g||^2 ; W g -> s2, ||W g||^2 ; tau.
 static int p_gradient_and_tau(pdadmm_ctx *c, int l /*0-based, >= 1*/) {
   Layer &ly = c->layers[l];
-  Layer &prev = c->layers[l - 1];
   Scratch &s = *c->cur;
   const int N = (int)c->N;
   int np = 0;
-  (void)prev;
-  uint32_t *w_g = nullptr;                 // max|g|, kept by the epilogue that writes g
-  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 1)); w_g = amax_take(c); }
-  // Quantised update, wide layers: the norm-only product W g takes g as one fp16 plane.  The epilogue that writes g
-  // writes that plane too, scaled by an exponent predicted from the previous iteration's max|g| (the true one is known
-  // only when the product has finished); rows_planes_kernel then confirms the prediction or, if max|g| moved by more
-  // than the plane can take, splits g again (6 bytes per element, the cost of every iteration before this).
-  const bool copy_g = c->levels && c->use_tc && s.g_hi != nullptr && (size_t)N * ly.ld_in <= s.a_cap &&
-                      ceil_div(ly.n_out, TC_BN) >= PLANES_FROM_COL_TILES / 2;
-  if (copy_g) {
-    EpiGradTCopy epi{{s.s1, ly.ld_in, ly.t, c->nu, w_g}, s.g_hi, ly.g_exp};
-    PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, ly.r, ly.ld_out, ly.W, ly.ld_in, planes_WT(ly),
-                            epi, s.slots, &np, 6.0 * N * ly.n_in, ly.amax_r));
-  } else {
-    EpiGradT epi{s.s1, ly.ld_in, ly.t, c->nu, w_g};
-    PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, ly.r, ly.ld_out, ly.W, ly.ld_in, planes_WT(ly),
-                            epi, s.slots, &np, 4.0 * N * ly.n_in, ly.amax_r));
+  const bool norm_only = c->levels && c->use_tc;     // the quantised update only needs ||W g||^2 (for the first tau); its
+                                                     // residual update uses W d
+  uint32_t *w_g = nullptr, *w_wg = nullptr;          // max|g|, max|W g|, kept by the epilogues that write them
+  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 2)); w_g = amax_take(c); w_wg = amax_take(c); }
+  // The epilogue that writes g writes its planes too (the hi plane alone for the norm-only product), scaled by an exponent
+  // predicted from the previous iteration's max|g|: the true one is known only when the product has finished.
+  EpiGradT epi{s.s1, ly.ld_in, ly.t, c->nu, w_g};
+  Operand G{s.s1, ly.ld_in, w_g};
+  if (c->use_tc) {
+    epi.H = s.pl0.hi; epi.L = norm_only ? nullptr : s.pl0.lo; epi.h_exp = ly.g_exp;
+    G = plane_operand(s.s1, ly.ld_in, Planes{s.pl0.hi, norm_only ? s.pl0.hi : s.pl0.lo, ly.g_exp}, w_g);
   }
+  PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, operand_r(ly), operand_W(ly), epi, s.slots, &np,
+                          (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in));
   int np2 = 0;
   double *slots_b = s.slots + s.n_slots / 2;          // second half of the slot buffer
-  if (c->levels && c->use_tc) {
-    // the quantised update only needs ||W g||^2 (for the first tau); its residual update uses W d
+  if (norm_only) {
     EpiNormOnly epi2{s.s2, ly.ld_out};
-    PlaneRef gp{nullptr, nullptr, 0, nullptr};
-    if (copy_g) {
-      const size_t n8 = (size_t)N * ly.ld_in / 8;
-      Launch k(c, KC_PLANES, s.st, 0.0, 0);          // normally only publishes the exponent
-      rows_planes_kernel<<<ew_grid(n8), 256, 0, s.st>>>(s.s1, n8, w_g, s.g_hi_exp, s.g_hi, nullptr, ly.g_exp);
-      gp = PlaneRef{s.g_hi, s.g_hi, ly.ld_in, s.g_hi_exp};
-    }
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, s.s1, ly.ld_in, ly.W, ly.ld_in, planes_W(ly),
-                             epi2, slots_b, &np2, 0, w_g, &gp));
+    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, G, operand_W(ly), epi2, slots_b, &np2, 0));
   } else {
-    EpiStoreSumsq epi2{s.s2, ly.ld_out};
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, s.s1, ly.ld_in, ly.W, ly.ld_in, planes_W(ly),
-                             epi2, slots_b, &np2, 0, w_g));
+    EpiStoreSumsq epi2{s.s2, ly.ld_out, w_wg};
+    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, G, operand_W(ly), epi2, slots_b, &np2, 0));
+  }
+  TauPlanes t{};
+  if (c->use_tc) {
+    t = TauPlanes{ly.amax_p, ly.amax_r, w_g, norm_only ? nullptr : w_wg, norm_only ? nullptr : s.pl1.exp, s.pl0.exp, ly.g_exp};
   }
   if (c->reduce != nullptr) {
     // ||g||^2 and ||W g||^2 are sums over nodes: this shard's totals, added over the shards, then tau
     PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, np, slots_b, np2));
-    finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.red, 1, s.red + 1, 1, c->d_flag + 2,
-                                             ly.amax_p, w_g, copy_g ? ly.g_exp : nullptr);
+    finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.red, 1, s.red + 1, 1, c->d_flag + 2, t);
     return PDADMM_OK;
   }
-  {
-    Launch k(c, KC_SMALL, s.st, 8.0 * (np + np2), 0);
-    finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.slots, np, slots_b, np2, c->d_flag + 2,
-                                             ly.amax_p, w_g, copy_g ? ly.g_exp : nullptr);
-  }
+  Launch k(c, KC_SMALL, s.st, 8.0 * (np + np2), 0);
+  finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.slots, np, slots_b, np2, c->d_flag + 2, t);
   return PDADMM_OK;
 }
 
-// pdADMM-G: p <- p - g/tau, r <- r - (W g)/tau.
+static PlaneOut plane_out(pdadmm_ctx *c, const Planes &p) {
+  return c->use_tc ? PlaneOut{p.hi, p.lo, p.exp} : PlaneOut{nullptr, nullptr, nullptr};
+}
+
+// pdADMM-G: p <- p - g/tau, r <- r - (W g)/tau, and the planes of both.
 static void p_step_plain(pdadmm_ctx *c, int l) {
   Layer &ly = c->layers[l];
   Scratch &s = *c->cur;
   const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
-  {
-    Launch k(c, KC_AXPY, s.st, 12.0 * c->N * ly.n_in, 0);
-    axpy_neg_kernel<<<ew_grid(n4p), EW_THREADS, 0, s.st>>>(ly.p, s.s1, &ly.sc->inv_tau, n4p, ly.amax_p);
-  }
-  {
-    Launch k(c, KC_AXPY, s.st, 12.0 * c->N * ly.n_out, 0);
-    axpy_neg_kernel<<<ew_grid(n4r), EW_THREADS, 0, s.st>>>(ly.r, s.s2, &ly.sc->inv_tau, n4r, ly.amax_r);
-  }
+  Launch k(c, KC_AXPY, s.st, (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out), 0);
+  pstep_kernel<<<ew_grid(std::max(n4p, n4r)), EW_THREADS, 0, s.st>>>(
+      ly.p, s.s1, n4p, ly.r, s.s2, n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0), c->use_tc ? ly.amax_p : nullptr,
+      c->use_tc ? ly.amax_r : nullptr);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
@@ -699,9 +645,11 @@ static int q_trial(pdadmm_ctx *c, int l) {
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
   // max|r| takes the trial's values too, which keeps it an upper bound whether or not the trial is taken
   EpiAddSumsq epi{s.s2, ly.ld_out, ly.r, c->use_tc ? ly.amax_r : nullptr};
-  const IntPlane di{c->int_operands ? s.d_plane : nullptr, ly.ld_in, ly.scale};      // d = (new code - old code) s
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, s.d, ly.ld_in, ly.W, ly.ld_in, planes_W(ly), epi,
-                           slots_b, &np, 4.0 * N * ly.n_out, w_d, nullptr, &di));
+  if (c->use_tc) { epi.H = s.pl0.hi; epi.L = s.pl0.lo; epi.h_exp = s.pl0.exp; }      // planes of the trial's r for the W-gradient
+  const Operand D = c->int_operands ? int_operand(s.d_plane, ly.ld_in, ly.scale)      // d = (new code - old code) s
+                                    : Operand{s.d, ly.ld_in, w_d};
+  PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, D, operand_W(ly), epi, slots_b, &np,
+                           (c->use_tc ? 8.0 : 4.0) * N * ly.n_out));
   if (c->reduce != nullptr) {
     PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, grid, slots_b, np));
     finalize_trial_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.red, 1, s.red + 1, 1);
@@ -740,72 +688,63 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
   Layer &ly = c->layers[l];
   Scratch &s = *c->cur;
   const int N = (int)c->N;
+  // p+ (layer 1: X, which never changes; pdADMM-G: planes from the p-step; pdADMM-G-Q: p+ = code * s)
+  Operand P{ly.p, ly.ld_in, ly.amax_p};
+  if (c->use_tc) P = l == 0 ? operand_X(ly) : (c->int_operands ? int_operand(ly.p_plane, ly.ld_in, ly.scale)
+                                                               : plane_operand(ly.p, ly.ld_in, s.pl1));
   if (!c->use_tc) {
     dim3 grid((unsigned)ceil_div(ly.n_in, SG_BN), (unsigned)ceil_div(ly.n_out, SG_BM), (unsigned)ly.n_split);
     Launch k(c, KC_GEMM_GRADW, s.st, 4.0 * ((double)N * ly.n_in + (double)N * ly.n_out), 2.0 * N * ly.n_in * ly.n_out);
     gemm_tn_kernel<<<grid, SG_THREADS, 0, s.st>>>(ly.n_out, ly.n_in, N, ly.k_chunk, ly.r, ly.ld_out, ly.p, ly.ld_in,
                                                  s.part, ly.ld_in);
   } else {
-    // both operands are node-major, i.e. contiguous along their output index (r is [nodes][n_out], p+ is
-    // [nodes][n_in]): transposed and split into planes beforehand, or tile by tile inside the product
-    if (planes_beforehand(ly.n_out, ly.n_in, l == 0)) {
-      transpose_planes(c, s.st, ly.r, N, ly.n_out, ly.ld_out, ly.amax_r, s.rT_hi, s.rT_lo, c->ldT, s.rT_exp);
-      PlaneRef Bt{s.pT_hi, s.pT_lo, c->ldT, s.pT_exp};
-      float b_mul = 0.f;
-      if (l == 0) {        // p_1 = X never changes: its planes are kept (made before the first iteration)
-        Bt = PlaneRef{ly.xT_hi, ly.xT_lo, c->ldT, ly.xT_exp};
-      } else if (c->int_operands) {
-        // p+ = code * s: the transposed codes are the whole operand (1 byte read, 2 written per element instead of 4 + 4)
-        Launch k(c, KC_PLANES, s.st, 3.0 * N * ly.n_in, 0);
-        const dim3 grid((unsigned)ceil_div(ly.n_in, 32), (unsigned)ceil_div(N, 32));
-        transpose_codes_kernel<<<grid, dim3(32, 8), 0, s.st>>>(ly.codes, c->code_bytes == 2, N, ly.n_in, ly.ld_in, s.pT_hi, c->ldT);
-        b_mul = ly.scale;
-      } else {
-        transpose_planes(c, s.st, ly.p, N, ly.n_in, ly.ld_in, ly.amax_p, s.pT_hi, s.pT_lo, c->ldT, s.pT_exp);
-      }
-      PD_TRY(gemm_over_nodes_tc(c, KC_GEMM_GRADW, s.st, ly.n_out, ly.n_in, N,
-                                PlaneRef{s.rT_hi, s.rT_lo, c->ldT, s.rT_exp}, Bt, s.part, ly.ld_in, ly.k_chunk, ly.n_split, b_mul));
-    } else {
-      PD_TRY(gemm_over_nodes_raw(c, KC_GEMM_GRADW, s.st, ly.n_out, ly.n_in, N, ly.r, ly.ld_out, ly.p, ly.ld_in, s.part,
-                                 ly.ld_in, ly.k_chunk, ly.n_split, ly.amax_r, ly.amax_p));
+    // both operands are node-major; the product contracts over the rows of their planes as they are
+    Operand R = l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, c->levels ? ly.amax_r : nullptr);
+    if (R.hi == nullptr) {                       // no room was left for the planes of r
+      const Planes pl{s.pl0.hi, s.pl0.lo, s.a_exp};
+      split_rows(c, s.st, ly.r, (size_t)N, ly.n_out, ly.ld_out, ly.amax_r, pl);
+      R = plane_operand(ly.r, ly.ld_out, pl);
     }
+    if (l > 0 && c->levels && !c->int_operands)  // p+ on a level set without integer planes
+      split_rows(c, s.st, ly.p, (size_t)N, ly.n_in, ly.ld_in, ly.amax_p, s.pl1);
+    PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, s.st, ly.n_out, ly.n_in, N, R, P, s.part, ly.ld_in, ly.k_chunk, ly.n_split));
   }
   const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
   const int gw = ew_grid(n4w);
+  uint32_t *w_G = nullptr;                       // max|G|
+  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 2)); w_G = amax_take(c); }
   {
-    Launch k(c, KC_GRADW_REDUCE, s.st, 4.0 * (ly.n_split + 1.0) * ly.n_out * ly.n_in, 0);
-    uint32_t *w = nullptr;
-    if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 1)); w = amax_take(c); }
-    reduce_gradW_kernel<<<gw, EW_THREADS, 0, s.st>>>(s.part, ly.n_split, n4w, c->nu, ly.gradW, w, s.slots);
-    if (c->reduce != nullptr) {
-      // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
-      PD_TRY(shard_sum(c, s.st, ly.gradW, n4w * 4, 0));
-      if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 1)); w = amax_take(c); }
-      sumsq_amax_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.gradW, n4w, w, s.slots);
-    }
-    if (c->use_tc) make_planes(c, s.st, ly.gradW, ly.n_out, ly.n_in, ly.ld_in, w, ly.Gp);
+    Launch k(c, KC_GRADW_REDUCE, s.st, (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in, 0);
+    // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
+    reduce_gradW_kernel<<<gw, EW_THREADS, 0, s.st>>>(s.part, ly.n_split, n4w, c->nu, ly.gradW, w_G, s.slots,
+                                                     c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp));
+  }
+  if (c->reduce != nullptr) {
+    // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
+    PD_TRY(shard_sum(c, s.st, ly.gradW, n4w * 4, 0));
+    if (c->use_tc) w_G = amax_take(c);
+    sumsq_amax_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.gradW, n4w, w_G, s.slots);
+    if (c->use_tc) split_rows(c, s.st, ly.gradW, (size_t)ly.n_out, ly.n_in, ly.ld_in, w_G, ly.Gp);
   }
   int np = 0;
   double *slots_b = s.slots + s.n_slots / 2;
   EpiStoreSumsq epi{s.s1, ly.ld_out};
-  const PlaneRef xp = planes_X(ly);
-  const IntPlane pi{(c->int_operands && l > 0) ? ly.p_plane : nullptr, ly.ld_in, ly.scale};          // p+ = code * s
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_GP, s.st, N, ly.n_out, ly.n_in, ly.p, ly.ld_in, ly.gradW, ly.ld_in, planes_G(ly),
-                           epi, slots_b, &np, 0, ly.amax_p, &xp, &pi));
+  PD_TRY(gemm_nodes<false>(c, KC_GEMM_GP, s.st, N, ly.n_out, ly.n_in, P, plane_operand(ly.gradW, ly.ld_in, ly.Gp, w_G), epi,
+                           slots_b, &np, 0));
+  ThetaPlanes tp{};
+  if (c->use_tc)       // no planes of r from the z-step of the last layer: its exponent stays TC_NO_PREDICTION
+    tp = ThetaPlanes{ly.amax_r, ly.amax_W, w_G, ly.Wp.exp, l + 1 < c->L ? ly.rp.exp : nullptr, ly.Gp.exp};
   if (c->reduce != nullptr) {
     // ||G p+||^2 is a sum over nodes (||G||^2 is the same on every shard already)
     PD_TRY(shard_sum_slots(c, s.st, s.red, slots_b, np, nullptr, 0));
-    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, s.red, 1, c->d_flag + 2, ly.amax_r);
+    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, s.red, 1, c->d_flag + 2, tp);
   } else {
     Launch k(c, KC_SMALL, s.st, 8.0 * (gw + np), 0);
-    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, slots_b, np, c->d_flag + 2, ly.amax_r);
+    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, slots_b, np, c->d_flag + 2, tp);
   }
   {
-    Launch k(c, KC_WSTEP, s.st, 20.0 * ly.n_out * ly.n_in, 0);
-    uint32_t *w = nullptr;
-    if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 1)); w = amax_take(c); }
-    wstep_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.W, ly.gradW, ly.sc, n4w, w);
-    if (c->use_tc) make_planes(c, s.st, ly.W, ly.n_out, ly.n_in, ly.ld_in, w, ly.Wp);
+    Launch k(c, KC_WSTEP, s.st, (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in, 0);
+    wstep_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.W, ly.gradW, ly.sc, n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp));
   }
   const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 16));
   const int rows_per_block = (int)ceil_div(N, n_blocks);
@@ -840,18 +779,19 @@ static void zqu_step(pdadmm_ctx *c, int l) {
     const size_t n4 = (size_t)N * ly.ld_out / 4;
     const int grid = ew_grid(n4);
     if (c->table_size > 0) {
-      Launch k(c, KC_ZQU, s.st, (c->levels ? 37.0 : 40.0) * N * ly.n_out, 0);
+      Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);
       const Layer &nx = c->layers[l + 1];
       zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), s.st>>>(
           ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu, c->slope, c->table_lo, c->table_step,
           c->table_size, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t, s.slots, ly.amax_r,
-          c->levels ? nx.codes : nullptr, c->code_bytes == 2);
+          plane_out(c, ly.rp), c->levels ? nx.codes : nullptr, c->code_bytes == 2);
     } else {
-      Launch k(c, KC_ZQU, s.st, (c->levels ? 37.0 : 40.0) * N * ly.n_out, 0);      // p_{l+1} as one-byte codes
+      Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);      // p_{l+1} as one-byte codes
       const Layer &nx = c->layers[l + 1];
       zqu_kernel<<<grid, EW_THREADS, 0, s.st>>>(ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu,
                                                c->slope, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t,
-                                               s.slots, ly.amax_r, c->levels ? nx.codes : nullptr, c->code_bytes == 2);
+                                               s.slots, ly.amax_r, plane_out(c, ly.rp), c->levels ? nx.codes : nullptr,
+                                               c->code_bytes == 2);
     }
   } else {
     Launch k(c, KC_ZLAST, s.st, 16.0 * N * ly.n_out, 0);
@@ -874,38 +814,39 @@ static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
   }
   if (c->use_tc)
     for (int i = 0; i < S; ++i) { c->cur = &lane(c, i); PD_TRY(amax_reset(c, c->cur->st)); }
-  // p-update of layers 2..L from the iterates of the previous iteration.  The quantised update reads an accept
-  // flag on the host after every trial: the host queues layer l's gradient and first trial on its lane, and only
-  // then waits for the flag of the layer that it queued on that lane before (layer l - S), so that the GPU always
-  // has the other lane's work while a flag travels.
+  // p-update (layers 2..L, from the iterates of the previous iteration) and W-, b-update with the new p, layer by layer: the
+  // lane's planes of r and p go from the one to the other.  The quantised p-update reads an accept flag on the host after
+  // every trial: the host queues layer l's gradient and first trial on its lane, and only then waits for the flag of the
+  // layer that it queued on another lane before, so that the GPU always has other lanes' work while a flag travels.
   std::vector<int> waiting(S, -1);                   // layer whose first trial is in flight on each lane
-  for (int l = 1; l < c->L; ++l) {
+  auto take_trial = [&](int i) -> int {              // on lane i, which is current
+    const int w = waiting[i];
+    if (w < 0) return PDADMM_OK;
+    waiting[i] = -1;
+    PD_TRY(q_finish(c, w, hit_cap));
+    if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[w], c->cur->st));
+    return w_and_b_step(c, w);
+  };
+  for (int l = 0; l < c->L; ++l) {
     c->cur = &lane_of(l);
-    if (c->levels) {
-      int &w = waiting[l % S];
-      if (w >= 0) {
-        PD_TRY(q_finish(c, w, hit_cap));
-        if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[w], c->cur->st));
-      }
+    if (c->levels && l > 0) {
+      PD_TRY(take_trial(l % S));
       PD_TRY(p_gradient_and_tau(c, l));
       PD_TRY(q_trial(c, l));
-      w = l;
-    } else {
+      waiting[l % S] = l;
+      continue;
+    }
+    if (l > 0) {
       PD_TRY(p_gradient_and_tau(c, l));
       p_step_plain(c, l);
       if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[l], c->cur->st));
     }
+    PD_TRY(w_and_b_step(c, l));
   }
   for (int i = 0; i < S && c->levels; ++i) {
-    if (waiting[i] < 0) continue;
-    c->cur = &lane(c, i);
-    PD_TRY(q_finish(c, waiting[i], hit_cap));
-    if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[waiting[i]], c->cur->st));
-  }
-  // W- and b-update of every layer with the new p
-  for (int l = 0; l < c->L; ++l) {
-    c->cur = &lane_of(l);
-    PD_TRY(w_and_b_step(c, l));
+    const int next = (c->L + i) % S;                 // the lane whose trial was queued first
+    c->cur = &lane(c, next);
+    PD_TRY(take_trial(next));
   }
   // z-, q-, u-update (q_l and u_l need p_{l+1} of this iteration, which another lane may have written)
   for (int l = 0; l < c->L; ++l) {
@@ -1067,34 +1008,6 @@ static int alloc_trial_buffers(pdadmm_ctx *c, Scratch &s, size_t n) {
   return PDADMM_OK;
 }
 
-// transposed planes of r_l (up to max_out columns) and of p_l, l >= 2 (up to max_in columns) of one lane
-// planes of the streamed operand of a product, once per lane: as wide as the widest matrix the lane's s1 holds
-static int alloc_row_planes(pdadmm_ctx *c, Scratch &s, size_t n) {
-  PD_TRY(dev_alloc(c, &s.a_hi, n, false));
-  PD_TRY(dev_alloc(c, &s.a_lo, n, false));
-  PD_TRY(dev_alloc(c, &s.a_exp, 1));
-  s.a_cap = n;
-  if (c->levels) {
-    PD_TRY(dev_alloc(c, &s.g_hi, n, false));
-    PD_TRY(dev_alloc(c, &s.g_hi_exp, 1));
-  }
-  return PDADMM_OK;
-}
-
-static int alloc_transposed(pdadmm_ctx *c, Scratch &s, int max_out, int max_in) {
-  if (max_out > 0) {
-    PD_TRY(dev_alloc(c, &s.rT_hi, (size_t)max_out * c->ldT));
-    PD_TRY(dev_alloc(c, &s.rT_lo, (size_t)max_out * c->ldT));
-  }
-  PD_TRY(dev_alloc(c, &s.rT_exp, 1));
-  if (max_in > 0) {
-    PD_TRY(dev_alloc(c, &s.pT_hi, (size_t)max_in * c->ldT));
-    PD_TRY(dev_alloc(c, &s.pT_lo, (size_t)max_in * c->ldT));
-  }
-  PD_TRY(dev_alloc(c, &s.pT_exp, 1));
-  return PDADMM_OK;
-}
-
 // Start of Algorithm 1 for layers first..L-1 (0-based) from the current p_first: b = 0, z_l = W_l p_l, q_l = f(z_l),
 // p_{l+1} = q_l (projected in -Q mode, with the level spacing from max(q_l)), u = 0, r = 0.
 static int feasible_start(pdadmm_ctx *c, int first) {
@@ -1104,16 +1017,15 @@ static int feasible_start(pdadmm_ctx *c, int first) {
   for (int l = first; l < c->L; ++l) {
     Layer &ly = c->layers[l];
     EpiStore epi{ly.z, ly.ld_out};
-    PD_TRY(split_planes(c, st, ly.W, ly.n_out, ly.n_in, ly.ld_in, ly.Wp));
+    PD_TRY(refresh_W_planes(c, ly, st));
     PD_CUDA(cudaMemsetAsync(ly.amax_p, 0, sizeof(uint32_t), st));
     absmax_kernel<<<ew_grid((size_t)N * ly.ld_in / 4), EW_THREADS, 0, st>>>(ly.p, (size_t)N * ly.ld_in / 4, ly.amax_p);
-    if (l == 0 && ly.x_hi != nullptr) {
-      const size_t n8 = (size_t)N * ly.ld_in / 8;
-      rows_planes_kernel<<<ew_grid(n8), 256, 0, st>>>(ly.p, n8, ly.amax_p, ly.x_exp, ly.x_hi, ly.x_lo);
+    Operand P{ly.p, ly.ld_in, ly.amax_p};
+    if (l == 0 && c->use_tc) {
+      split_rows(c, st, ly.p, (size_t)N, ly.n_in, ly.ld_in, ly.amax_p, ly.xp);
+      P = operand_X(ly);
     }
-    const PlaneRef xp = planes_X(ly);
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)N, ly.n_out, ly.n_in, ly.p, ly.ld_in, ly.W, ly.ld_in, planes_W(ly),
-                             epi, nullptr, nullptr, 0, ly.amax_p, &xp));
+    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr, 0));
     PD_CUDA(cudaMemsetAsync(ly.b, 0, (size_t)ly.ld_out * 4, st));
     PD_CUDA(cudaMemsetAsync(ly.shift, 0, (size_t)ly.ld_out * 4, st));
     PD_CUDA(cudaMemsetAsync(ly.r, 0, (size_t)N * ly.ld_out * 4, st));
@@ -1239,8 +1151,10 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &ly.W, (size_t)ly.n_out * ly.ld_in));
     PD_TRY(dev_alloc(c, &ly.gradW, (size_t)ly.n_out * ly.ld_in));
     if (c->use_tc) {
-      PD_TRY(alloc_planes(c, ly.n_out, ly.n_in, l > 0, true, &ly.Wp));     // W^T only where a p-gradient is taken
-      PD_TRY(alloc_planes(c, ly.n_out, ly.n_in, false, true, &ly.Gp));
+      PD_TRY(alloc_planes(c, (size_t)ly.n_out * ly.ld_in, &ly.Wp));
+      PD_TRY(alloc_planes(c, (size_t)ly.n_out * ly.ld_in, &ly.Gp));
+      PD_TRY(dev_alloc(c, &ly.amax_W, 1));
+      if (l == 0) PD_TRY(alloc_planes(c, (size_t)N * ly.ld_in, &ly.xp));
     }
     PD_TRY(dev_alloc(c, &ly.b, (size_t)ly.ld_out));
     PD_TRY(dev_alloc(c, &ly.shift, (size_t)ly.ld_out));
@@ -1259,7 +1173,8 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     // Node slices of the W-gradient product (slices >= 256 nodes, at most 32).  The persistent grid works through
     // tiles x slices units in rounds of n_sms, so the count is chosen to fill its last round: the smallest number
     // of slices within 3 % (relative) of the best fill (fewer slices = fewer partial tiles to write and add up).
-    const int64_t tiles = ceil_div(ly.n_in, SG_BN) * ceil_div(ly.n_out, SG_BM);   // same tile for both kernels
+    const int64_t tiles = ceil_div(ly.n_in, SG_BN) * ceil_div(ly.n_out, SG_BM);   // same tile for both kernels; a pair of
+                                                                                    // SMs works on two of them
     const int max_split = (int)std::max<int64_t>(1, std::min<int64_t>(32, ceil_div(N, 256)));
     auto slices_for = [&](int want) { return (int)ceil_div(N, round_up((int)ceil_div(N, want), TC_BK)); };
     auto fill = [&](int want) {
@@ -1276,7 +1191,6 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   }
   // scratch
   Scratch &s = c->scr;
-  int tr_out = 0, tr_in = 0;
   const size_t bytes_before_scratch = c->bytes_handed_out;
   const size_t e_max = (size_t)N * std::max(max_in, max_out);
   PD_TRY(dev_alloc(c, &s.s1, e_max));
@@ -1291,32 +1205,10 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &s.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
     PD_TRY(dev_alloc(c, &s.tail_count, (size_t)c->n_sms * 8));
     PD_TRY(dev_alloc(c, &s.amax_pool, (size_t)AMAX_POOL));
-    c->ldT = round_up((int)N, 8);
-    // widest r_l and p_l (l >= 2) among the layers whose product over the nodes takes its operands as planes
-    for (int l = 0; l < c->L; ++l) {
-      const Layer &ly = c->layers[l];
-      if (!planes_beforehand(ly.n_out, ly.n_in, l == 0)) continue;
-      tr_out = std::max(tr_out, ly.n_out);
-      if (l > 0) tr_in = std::max(tr_in, ly.n_in);
-    }
-    PD_TRY(alloc_transposed(c, s, tr_out, tr_in));
-    // planes of streamed operands: needed if some layer's products are at least PLANES_FROM_COL_TILES column tiles wide
-    bool want_row_planes = false;
-    for (int l = 0; l < c->L; ++l)
-      want_row_planes |= std::max(ceil_div(c->layers[l].n_out, TC_BN), l > 0 ? ceil_div(c->layers[l].n_in, TC_BN) : 0) >= PLANES_FROM_COL_TILES;
-    want_row_planes |= c->levels > 0;       // the norm-only product of the quantised update always takes a hi plane
-    if (want_row_planes) PD_TRY(alloc_row_planes(c, s, e_max));
-    Layer &l0 = c->layers[0];
-    if (ceil_div(l0.n_out, TC_BN) >= 2) {      // X is split once for ever: worth it from two column tiles on
-      PD_TRY(dev_alloc(c, &l0.x_hi, (size_t)N * l0.ld_in, false));
-      PD_TRY(dev_alloc(c, &l0.x_lo, (size_t)N * l0.ld_in, false));
-      PD_TRY(dev_alloc(c, &l0.x_exp, 1));
-    }
-    if (planes_beforehand(l0.n_out, l0.n_in, true)) {
-      PD_TRY(dev_alloc(c, &l0.xT_hi, (size_t)l0.n_in * c->ldT));
-      PD_TRY(dev_alloc(c, &l0.xT_lo, (size_t)l0.n_in * c->ldT));
-    }
-    PD_TRY(dev_alloc(c, &l0.xT_exp, 1));
+    s.pl_cap = e_max;
+    PD_TRY(alloc_planes(c, s.pl_cap, &s.pl0));
+    PD_TRY(alloc_planes(c, s.pl_cap, &s.pl1));
+    PD_TRY(dev_alloc(c, &s.a_exp, 1));
   }
 
   // further lanes for the concurrency across layers: own stream, product outputs, partial tiles, slots.
@@ -1343,8 +1235,27 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
       PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
       PD_TRY(dev_alloc(c, &x.tail_count, (size_t)c->n_sms * 8));
       PD_TRY(dev_alloc(c, &x.amax_pool, (size_t)AMAX_POOL));
-      PD_TRY(alloc_transposed(c, x, tr_out, tr_in));
-      if (s.a_hi != nullptr) PD_TRY(alloc_row_planes(c, x, e_max));
+      x.pl_cap = s.pl_cap;
+      PD_TRY(alloc_planes(c, x.pl_cap, &x.pl0));
+      PD_TRY(alloc_planes(c, x.pl_cap, &x.pl1));
+      PD_TRY(dev_alloc(c, &x.a_exp, 1));
+    }
+  }
+  // Planes of r from one iteration to the next, hidden layers: worth their memory (the p-gradient's product would have to split
+  // r first otherwise, 8 bytes per element), but nothing depends on them.  All or none, and at most 7/8 of what is free.
+  if (c->use_tc) {
+    size_t need = 0, free_bytes = 0, total = 0;
+    for (int l = 0; l + 1 < c->L; ++l) need += (size_t)N * c->layers[l].ld_out * 4;
+    PD_CUDA(cudaMemGetInfo(&free_bytes, &total));
+    const bool room = need <= free_bytes / 8 * 7 || need <= c->arena_cap - c->arena_used;
+    for (int l = 0; l < c->L; ++l) {
+      Layer &ly = c->layers[l];
+      if (l + 1 < c->L && room) {
+        PD_TRY(alloc_planes(c, (size_t)N * ly.ld_out, &ly.rp));
+      } else if (l + 1 == c->L) {        // the product splits the last layer's few columns itself: planes of no use, refused
+        PD_TRY(alloc_planes(c, (size_t)N * ly.ld_out, &ly.rp));
+        PD_CUDA(cudaMemsetAsync(ly.rp.exp, 0x80, sizeof(int), st));       // no exponent: TC_NO_PREDICTION
+      }
     }
   }
   c->ev_p.resize(c->L);
@@ -1369,7 +1280,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->r_valid = true;                        // z = W p + b exactly by construction, r = 0 (allocated as zero)
   c->w_planes_valid = true;
   c->amax_p_valid = true;
-  c->xT_valid = false;            // the transposed planes of X are made by the first step
+  c->x_planes_valid = true;
   c->launches = 0;
   c->comm_bytes = 0;
   return PDADMM_OK;
@@ -1476,9 +1387,10 @@ extern "C" int pdadmm_destroy(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
-static int ensure_residual(pdadmm_ctx *c) {
+// What products read beside the stored tensors: planes of W, largest magnitudes of p, planes of X.
+static int ensure_operands(pdadmm_ctx *c) {
   if (!c->w_planes_valid) {
-    for (auto &ly : c->layers) PD_TRY(split_planes(c, c->scr.st, ly.W, ly.n_out, ly.n_in, ly.ld_in, ly.Wp));
+    for (auto &ly : c->layers) PD_TRY(refresh_W_planes(c, ly, c->scr.st));
     c->w_planes_valid = true;
   }
   if (!c->amax_p_valid) {
@@ -1490,17 +1402,16 @@ static int ensure_residual(pdadmm_ctx *c) {
     }
     c->amax_p_valid = true;
   }
-  if (!c->xT_valid && c->use_tc) {          // both kinds of planes of X follow the stored X
+  if (!c->x_planes_valid && c->use_tc) {          // the planes of X follow the stored X
     Layer &l0 = c->layers[0];
-    if (planes_beforehand(l0.n_out, l0.n_in, true))
-      transpose_planes(c, c->scr.st, l0.p, (int)c->N, l0.n_in, l0.ld_in, l0.amax_p, l0.xT_hi, l0.xT_lo, c->ldT, l0.xT_exp);
-    if (l0.x_hi != nullptr) {
-      const size_t n8 = (size_t)c->N * l0.ld_in / 8;
-      Launch k(c, KC_PLANES, c->scr.st, 8.0 * c->N * l0.n_in, 0);
-      rows_planes_kernel<<<ew_grid(n8), 256, 0, c->scr.st>>>(l0.p, n8, l0.amax_p, l0.x_exp, l0.x_hi, l0.x_lo);
-    }
-    c->xT_valid = true;
+    split_rows(c, c->scr.st, l0.p, (size_t)c->N, l0.n_in, l0.ld_in, l0.amax_p, l0.xp);
+    c->x_planes_valid = true;
   }
+  return PDADMM_OK;
+}
+
+static int ensure_residual(pdadmm_ctx *c) {
+  PD_TRY(ensure_operands(c));
   if (!c->t_valid) {
     for (int l = 1; l < c->L; ++l) {
       Layer &ly = c->layers[l];
@@ -1645,10 +1556,7 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   if (!c) return fail(PDADMM_EINVAL, "context is null");
   PD_CUDA(cudaSetDevice(c->device));
   cudaStream_t st = c->scr.st;
-  if (!c->w_planes_valid) {
-    for (auto &ly : c->layers) PD_TRY(split_planes(c, st, ly.W, ly.n_out, ly.n_in, ly.ld_in, ly.Wp));
-    c->w_planes_valid = true;
-  }
+  PD_TRY(ensure_operands(c));
   // forward pass with the constraints enforced: activations alternate between the two scratch matrices
   const int N = (int)c->N;
   const float *in = c->layers[0].p;
@@ -1657,8 +1565,7 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   const uint32_t *w_in = nullptr;            // max|activations| of the layer's input
   if (c->use_tc) {
     PD_TRY(amax_reset(c, st));               // one word per layer output, all from one pass through the pool
-    // max|X| is kept (X changes by pdadmm_set_tensor alone, which clears amax_p_valid)
-    w_in = c->amax_p_valid ? c->layers[0].amax_p : amax_of(c, st, in, (size_t)N * c->layers[0].ld_in / 4);
+    w_in = c->layers[0].amax_p;
   }
   for (int l = 0; l < c->L; ++l) {
     Layer &ly = c->layers[l];
@@ -1666,10 +1573,9 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
     uint32_t *w_out = nullptr;
     if (c->use_tc) w_out = amax_take(c);
     EpiBiasAct epi{out, ly.ld_out, ly.b, l + 1 < c->L ? 1 : 0, c->slope, w_out};
-    // the first layer's input is X: its planes are kept by the context while they match the stored X
-    const PlaneRef xp = (l == 0 && c->xT_valid) ? planes_X(ly) : PlaneRef{nullptr, nullptr, 0, nullptr};
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, N, ly.n_out, ly.n_in, in, ly.ld_in, ly.W, ly.ld_in, planes_W(ly),
-                             epi, nullptr, nullptr, 0, w_in, &xp));
+    Operand P{in, ly.ld_in, w_in};
+    if (l == 0 && c->use_tc) P = operand_X(ly);
+    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr, 0));
     w_in = w_out;
     in = out;
   }
@@ -1807,7 +1713,7 @@ extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void 
     c->r_valid = false;
   if (kind == PDADMM_T_W) c->w_planes_valid = false;
   if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->amax_p_valid = false;
-  if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->xT_valid = false;
+  if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->x_planes_valid = false;
   if (kind == PDADMM_T_P || kind == PDADMM_T_Q || kind == PDADMM_T_U) c->t_valid = false;
   if (kind == PDADMM_T_P && c->levels && layer >= 2) PD_TRY(project_p_on_its_levels(c, layer));
   return PDADMM_OK;
@@ -1899,33 +1805,35 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
     // operand shapes as stored: rows x cols
     const int a_rows = mode == 2 ? K : M, a_cols = mode == 2 ? M : K;
     const int b_rows = mode == 0 ? N : K, b_cols = mode == 0 ? K : N;
-    const int lda = round_up(a_cols, mode == 2 ? 4 : 8), ldb = round_up(b_cols, 4), ldc = round_up(N, 4);
+    const int lda = round_up(a_cols, 8), ldb = round_up(b_cols, 8), ldc = round_up(N, 4);
     float *dA, *dB, *dC, *part = nullptr;
     double *slots;
-    Planes Bp;
+    Planes Ap, Bp;
     PD_TRY(dev_alloc(c, &dA, (size_t)a_rows * lda));
     PD_TRY(dev_alloc(c, &dB, (size_t)b_rows * ldb));
     PD_TRY(dev_alloc(c, &dC, (size_t)M * ldc));
-    const int n_slots = 8 * (int)(ceil_div(M, 128) * ceil_div(N, 128)) + 2048;
+    const int n_slots = 16 * (int)(ceil_div(M, 128) * ceil_div(N, 128)) + 2048;
     PD_TRY(dev_alloc(c, &slots, (size_t)n_slots));
     PD_TRY(upload_rows(c, st, dA, lda, A, a_cols, a_rows));
     PD_TRY(upload_rows(c, st, dB, ldb, B, b_cols, b_rows));
-    if (c->use_tc) {
+    Operand oA{dA, lda, nullptr}, oB{dB, ldb, nullptr};
+    if (c->use_tc) {        // planes of both operands as they are stored
       PD_TRY(dev_alloc(c, &c->scr.amax_pool, (size_t)AMAX_POOL));
-      // planes of B as [N][K]: B itself in mode 0, its transpose in mode 1
-      if (mode != 2) PD_TRY(alloc_planes(c, b_rows, b_cols, mode == 1, mode == 0, &Bp));
-      if (mode != 2) PD_TRY(split_planes(c, st, dB, b_rows, b_cols, ldb, Bp));
-      if (mode != 2) PD_TRY(alloc_row_planes(c, c->scr, (size_t)a_rows * lda));     // used from four column tiles on
+      PD_TRY(alloc_planes(c, (size_t)a_rows * lda, &Ap));
+      PD_TRY(alloc_planes(c, (size_t)b_rows * ldb, &Bp));
+      PD_TRY(amax_reserve(c, st, 2));
+      split_rows(c, st, dA, (size_t)a_rows, a_cols, lda, amax_of(c, st, dA, (size_t)a_rows * lda / 4), Ap);
+      split_rows(c, st, dB, (size_t)b_rows, b_cols, ldb, amax_of(c, st, dB, (size_t)b_rows * ldb / 4), Bp);
+      oA = plane_operand(dA, lda, Ap);
+      oB = plane_operand(dB, ldb, Bp);
     }
     int np = 0;
     if (mode == 0) {
       EpiStoreSumsq epi{dC, ldc};
-      PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, st, M, N, K, dA, lda, dB, ldb, PlaneRef{Bp.hi, Bp.lo, Bp.ldh, Bp.exp}, epi,
-                               slots, &np, 0));
+      PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, st, M, N, K, oA, oB, epi, slots, &np, 0));
     } else if (mode == 1) {
       EpiStoreSumsq epi{dC, ldc};
-      PD_TRY(gemm_nodes<true>(c, KC_GEMM_WG, st, M, N, K, dA, lda, dB, ldb, PlaneRef{Bp.hiT, Bp.loT, Bp.ldhT, Bp.exp}, epi,
-                              slots, &np, 0));
+      PD_TRY(gemm_nodes<true>(c, KC_GEMM_WG, st, M, N, K, oA, oB, epi, slots, &np, 0));
     } else {
       const int split = (int)std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(K, 64)));
       const int k_chunk = round_up((int)ceil_div(K, split), TC_BK);
@@ -1935,29 +1843,11 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
         dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM), (unsigned)n_split);
         gemm_tn_kernel<<<grid, SG_THREADS, 0, st>>>(M, N, K, k_chunk, dA, lda, dB, ldb, part, ldc);
       } else {
-        if (!planes_beforehand(M, N, false)) {
-          PD_TRY(amax_reserve(c, st, 2));
-          const uint32_t *wa = amax_of(c, st, dA, (size_t)K * lda / 4), *wb = amax_of(c, st, dB, (size_t)K * ldb / 4);
-          PD_TRY(gemm_over_nodes_raw(c, KC_GEMM_GRADW, st, M, N, K, dA, lda, dB, ldb, part, ldc, k_chunk, n_split, wa, wb));
-        } else {
-        // transposed planes of both operands, then the contraction over their rows
-        const int ldT = round_up(K, 8);
-        __half *ah, *al, *bh, *bl;
-        int *ea, *eb;
-        PD_TRY(dev_alloc(c, &ah, (size_t)M * ldT)); PD_TRY(dev_alloc(c, &al, (size_t)M * ldT));
-        PD_TRY(dev_alloc(c, &bh, (size_t)N * ldT)); PD_TRY(dev_alloc(c, &bl, (size_t)N * ldT));
-        PD_TRY(dev_alloc(c, &ea, 1)); PD_TRY(dev_alloc(c, &eb, 1));
-        PD_TRY(amax_reserve(c, st, 2));
-        const uint32_t *wa = amax_of(c, st, dA, (size_t)K * lda / 4), *wb = amax_of(c, st, dB, (size_t)K * ldb / 4);
-        transpose_planes(c, st, dA, K, M, lda, wa, ah, al, ldT, ea);
-        transpose_planes(c, st, dB, K, N, ldb, wb, bh, bl, ldT, eb);
-        PD_TRY(gemm_over_nodes_tc(c, KC_GEMM_GRADW, st, M, N, K, PlaneRef{ah, al, ldT, ea}, PlaneRef{bh, bl, ldT, eb}, part,
-                                  ldc, k_chunk, n_split));
-        }
+        PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, M, N, K, oA, oB, part, ldc, k_chunk, n_split));
       }
       const size_t n4 = (size_t)M * ldc / 4;
       np = ew_grid(n4);
-      reduce_gradW_kernel<<<np, EW_THREADS, 0, st>>>(part, n_split, n4, 1.0f, dC, nullptr, slots);
+      reduce_gradW_kernel<<<np, EW_THREADS, 0, st>>>(part, n_split, n4, 1.0f, dC, nullptr, slots, PlaneOut{nullptr, nullptr, nullptr});
     }
     double *res = slots + n_slots - 1;
     reduce_slots_kernel<<<1, 256, 0, st>>>(slots, np, 1, 1, res);

@@ -23,6 +23,35 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// ---- pairs of blocks (clusters of two) ---------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// the address of the same shared-memory location in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+// An arrival on a barrier of either block.  It orders what the tensor cores and tcgen05.ld did (with the tcgen05 fences
+// around it); ordinary shared-memory writes that the other block's thread has to see need fence_cluster() before it, and
+// after the wait (release and acquire at cluster scope in every arrival and wait cost 1.6 times the product).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
+__device__ __forceinline__ int ld_cluster_int(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_sync() {          // all threads of both blocks
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -58,12 +87,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
   }
 }
 
-// ---- TMA: 2-D tile load global -> shared, completion on an mbarrier -------------------
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-      : "memory");
+// ---- TMA: 2-D tile load global -> this block's shared memory, completion on an mbarrier (a cluster address; CG = 2: it may
+// be the other block's of the pair) -------------------
+template <int CG>
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
+  if constexpr (CG == 1)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y) : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -72,50 +107,65 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map) {
 // generic-proxy writes to shared memory -> visible to the async proxy (TMA, tensor cores)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// True in one lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ---- tensor memory -------------------------------------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t n_cols) {     // one full warp
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(n_cols) : "memory");
+// One full warp; CG = 2: the same warp of both blocks of the pair.
+template <int CG>
+__device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t n_cols) {
+  if constexpr (CG == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(n_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(n_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
 }
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {       // one full warp
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
+template <int CG>
+__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {
+  if constexpr (CG == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
+  else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // D[tmem] (+)= A[smem desc] * B[smem desc], fp16 inputs (K = 16 per instruction), fp32 accumulate; one thread issues.
+// COLL: what happens to the collector buffer that holds A: A_ONCE = nothing is kept, A_KEEP = A stays in it, A_AGAIN = A is
+// the one the previous MMA kept, so shared memory is not read for it (two consecutive MMAs share their A operand).
+enum : int { A_ONCE = 0, A_KEEP = 1, A_AGAIN = 2 };
+template <int CG, int COLL>
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
-      : "memory");
+#define PD_MMA(variant)                                                                                        \
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma." variant " [%0], %1, %2, %3, p;\n\t}"  \
+               ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory")
+  if constexpr (CG == 1) {
+    if constexpr (COLL == A_KEEP) PD_MMA("cta_group::1.kind::f16.collector::a::fill");
+    else if constexpr (COLL == A_AGAIN) PD_MMA("cta_group::1.kind::f16.collector::a::lastuse");
+    else PD_MMA("cta_group::1.kind::f16");
+  } else {
+    if constexpr (COLL == A_KEEP) PD_MMA("cta_group::2.kind::f16.collector::a::fill");
+    else if constexpr (COLL == A_AGAIN) PD_MMA("cta_group::2.kind::f16.collector::a::lastuse");
+    else PD_MMA("cta_group::2.kind::f16");
+  }
+#undef PD_MMA
 }
-// The same with A read from tensor memory: row i of the 128 x 16 A tile in lane i, two fp16 per 32-bit column
-// (8 columns from a_tmem on).
-__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
-      : "memory");
-}
-// The mbarrier receives one arrival once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// 32 lanes x 16 consecutive 32-bit columns: thread i of the warp receives lane (base + i), columns c..c+15.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr) : "memory");
+// The mbarrier receives one arrival once every MMA issued so far by this thread has completed; CG = 2: the barrier at this
+// place in both blocks of the pair does (`both`), or this block's alone.
+template <int CG>
+__device__ __forceinline__ void mma_commit(uint64_t *bar, bool both = true) {
+  if constexpr (CG == 1) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+  } else if (both) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+  } else {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+  }
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base + i), columns c..c+31.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
@@ -129,57 +179,67 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
       : "r"(taddr) : "memory");
 }
-// 32 lanes x 16 consecutive 32-bit columns: thread i of the warp writes lane (base + i), columns c..c+15.
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-      : "memory");
+// Waits for the warp's tensor-memory loads; the registers of the last one pass through the instruction, so that nothing
+// that uses them can be scheduled before it.
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]),
+                 "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]),
+                 "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]),
+                 "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+               :: "memory");
 }
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// two single-precision operations in one instruction, each rounded to nearest
+__device__ __forceinline__ uint64_t pack_f2(uint32_t lo, uint32_t hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f2(uint64_t v, float &lo, float &hi) {
+  uint32_t a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+  lo = __uint_as_float(a); hi = __uint_as_float(b);
+}
+__device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul_f2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 
 // ---- register budget of a warpgroup (four consecutive warps, all of which must execute the instruction) -----------
 template <int N> __device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // ---- descriptors -------------------------------------------------------------------------------------------
-// Shared-memory matrix descriptor (the tile base must be aligned to the swizzle period).
-// K-major operand  (rows = output index, k_row_bytes = 64 or 128 bytes of K per row): swizzle of the row width
-//                   with 16-byte atoms, 8-row groups 8 rows apart (sbo); lbo is not used by the hardware here.
-// MN-major operand (rows = K index, 32 floats of the output index per row): for 32-bit types the only
-//                   layout is the 128-byte swizzle with 32-byte atoms; 4-row groups 512 bytes apart (sbo),
-//                   the next 32 output indices lbo bytes further.
+// Shared-memory matrix descriptor of an fp16 operand tile in the 128-byte swizzle (tile base aligned to 1024 bytes).
+// K-major   (rows = output index, 64 values of the contraction index per 128-byte row): groups of 8 rows are 1024 bytes
+//            apart (sbo); lbo is not used.
+// MN-major  (rows = contraction index, 64 values of the output index per 128-byte row): groups of 8 rows are 1024 bytes
+//            apart (sbo), the next 64 output indices lbo bytes further.
 // The descriptor is built from two words so that a loop only has to add to the low one: the start address
 // field counts 16-byte units and shared-memory addresses stay below 2^18, so (address >> 4) needs no mask.
-__device__ __forceinline__ uint32_t smem_desc_hi(bool mn_major, uint32_t k_row_bytes) {
-  const uint32_t sbo = mn_major ? 512u : 8u * k_row_bytes;
-  const uint32_t layout = mn_major ? 1u /* 128B swizzle, 32B atoms */ : (k_row_bytes == 128u ? 2u /* 128B */ : 4u /* 64B */);
-  return ((sbo >> 4) & 0x3FFFu) | (1u << 14) /* descriptor version */ | (layout << 29);
+__device__ __forceinline__ uint32_t smem_desc_hi() {
+  return (1024u >> 4) | (1u << 14) /* descriptor version */ | (2u << 29) /* 128-byte swizzle */;
 }
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, bool mn_major, uint32_t lbo_mn) {
   const uint32_t lbo = mn_major ? lbo_mn : 16u;
   return (saddr >> 4) | (((lbo >> 4) & 0x3FFFu) << 16);
 }
 __device__ __forceinline__ uint64_t smem_desc(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
-// Instruction descriptor: fp16 x fp16 -> fp32, M x N tile, both operands K-major.
-__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
-  return (1u << 4) /* D: f32 */ | (0u << 7) /* A: f16 */ | (0u << 10) /* B: f16 */ | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
-
-// Barrier `id` (1..15) among `count` threads (a multiple of 32) of the block; returns the OR of `flag` over them.
-__device__ __forceinline__ bool named_barrier_or(uint32_t id, uint32_t count, bool flag) {
-  uint32_t out;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.b32 q, %3, 0;\n\t"
-      "bar.red.or.pred p, %1, %2, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(out) : "r"(id), "r"(count), "r"((uint32_t)flag) : "memory");
-  return out != 0;
+// Instruction descriptor: fp16 x fp16 -> fp32, M x N tile; a_mn, b_mn: the operand is MN-major in shared memory.
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn, bool b_mn) {
+  return (1u << 4) /* D: f32 */ | (0u << 7) /* A: f16 */ | (0u << 10) /* B: f16 */ | ((a_mn ? 1u : 0u) << 15) |
+         ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 }  // namespace ptx
