@@ -9,6 +9,8 @@
 
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "planes.cuh"
 
@@ -348,6 +350,23 @@ rows_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__res
   }
 }
 
+// Planes whose exponent was chosen before the largest magnitude was known, in front of a product of a large matrix: normally
+// nothing to do; if the scaling turned out unusable they are made again, with the exponent of *amax (which is what the product
+// assumes then; *exp stays as it is).  (Inside the product, per output tile, it would take 5 to 10 times the product: a
+// few such iterations at the start of a context of 20 000 x 500 cost more than all these launches.)
+__global__ void __launch_bounds__(256)
+check_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__restrict__ amax, const int *__restrict__ exp,
+                    __half *__restrict__ hi, __half *__restrict__ lo /* may be null */) {
+  if (tc_planes_usable(*amax, *exp)) return;
+  const float scale = tc_pow2(tc_scale_exp(*amax));
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
+    uint4 h, l;
+    tc_split8(reinterpret_cast<const float4 *>(x)[2 * i], reinterpret_cast<const float4 *>(x)[2 * i + 1], scale, h, l);
+    reinterpret_cast<uint4 *>(hi)[i] = h;
+    if (lo != nullptr) reinterpret_cast<uint4 *>(lo)[i] = l;
+  }
+}
+
 // ---- reduction of the split partial tiles of grad_W, scaling by nu, ||grad_W||^2 ------------------
 __global__ void __launch_bounds__(EW_THREADS)
 reduce_gradW_kernel(const float *__restrict__ part, int n_split, size_t n4, float nu, float *__restrict__ G,
@@ -358,6 +377,7 @@ reduce_gradW_kernel(const float *__restrict__ part, int n_split, size_t n4, floa
   uint32_t m = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
     for (int s = 0; s < n_split; ++s) {
       const float4 v = ld4(part + (size_t)s * n4 * 4, i);
       a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
@@ -633,82 +653,124 @@ zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict
 }
 
 // ---- z-update of the last layer -------------------------------------------------------------------
-// One thread per node.  a = (r - shift) + z.  Labelled node: z+ = argmin CE(z; y) + (nu/2)||z - a||^2
+// a = (r - shift) + z.  Labelled node: z+ = argmin CE(z; y) + (nu/2)||z - a||^2
 // (Eq. "update zl"), the unique root of softmax(z) - e_y + nu (z - a) = 0, by damped Newton with the
 // Hessian diag(s) + nu I - s s^T inverted through the rank-one update formula; double precision
 // inside, since nu is small and the Hessian is close to singular along (1,..,1).  Unlabelled: z+ = a.
+// The search starts from the stored z, the root for the previous a, where the gradient is nu (a_old - a) alone.
+//
+// G lanes share a node, two classes each, everything in registers, sums by shuffles; the loop is common to the warp and has
+// one evaluation per turn: a group whose trial point is accepted takes the gradient there from the exponentials it just
+// computed and sets out on the next step, another one halves its step.  (One thread per node with the C-long arrays in
+// local memory, two sets of exponentials per step and a start from a: 170 000 x 40 1150 us, 20 000 x 10 31 us.)
 constexpr int ZL_MAX_C = 64;
+template <int G>
 __global__ void __launch_bounds__(128)
 zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restrict__ shift,
              const int *__restrict__ labels, const uint8_t *__restrict__ mask, int n_rows, int C, int ld,
              double nu, int *__restrict__ not_converged, uint32_t *__restrict__ amax_r /* max|r|, may be null */,
-             int least_squares /* R = 1/2 ||z - e_y||^2: z+ = (e_y + nu a)/(1 + nu) */) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_rows) return;
-  float *rj = r + (size_t)j * ld, *zj = z + (size_t)j * ld;
-  double a[ZL_MAX_C], x[ZL_MAX_C], s[ZL_MAX_C], st[ZL_MAX_C];
-  for (int c = 0; c < C; ++c) { a[c] = (double)((rj[c] - shift[c]) + zj[c]); x[c] = a[c]; }
-  if (mask[j] && least_squares) {
-    const int y = labels[j];
-    for (int c = 0; c < C; ++c) x[c] = ((c == y ? 1.0 : 0.0) + nu * a[c]) / (1.0 + nu);
-  } else if (mask[j]) {
-    const int y = labels[j];
-    auto fval = [&](const double *v) {
-      double m = v[0];
-      for (int c = 1; c < C; ++c) m = fmax(m, v[c]);
-      double se = 0.0, sq = 0.0;
-      for (int c = 0; c < C; ++c) { se += exp(v[c] - m); sq += (v[c] - a[c]) * (v[c] - a[c]); }
-      return m + log(se) - v[y] + 0.5 * nu * sq;
-    };
-    double fx = fval(x);
-    bool done = false;
-    for (int it = 0; it < 100 && !done; ++it) {
-      double m = x[0];
-      for (int c = 1; c < C; ++c) m = fmax(m, x[c]);
-      double se = 0.0;
-      for (int c = 0; c < C; ++c) { s[c] = exp(x[c] - m); se += s[c]; }
-      double gmax = 0.0, s_mg = 0.0, s_ms = 0.0;
-      for (int c = 0; c < C; ++c) {
-        s[c] /= se;
-        const double g = s[c] - (c == y ? 1.0 : 0.0) + nu * (x[c] - a[c]);
-        gmax = fmax(gmax, fabs(g));
-        const double mi = 1.0 / (s[c] + nu);
-        st[c] = g;                       // gradient for now
-        s_mg += s[c] * mi * g;
-        s_ms += s[c] * mi * s[c];
+             int least_squares /* R = 1/2 ||z - e_y||^2: z+ = (e_y + nu a)/(1 + nu) */, PlaneOut rp) {
+  const int j = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) / G), lane = threadIdx.x % G;
+  const bool row = j < n_rows;
+  const size_t at = (size_t)(row ? j : n_rows - 1) * ld + 2 * lane;          // ld is a multiple of 32 and C <= 2 G
+  const int c0 = 2 * lane;
+  const bool in[2] = {c0 < C, c0 + 1 < C};
+  auto sum = [&](double v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, G);
+    return v;
+  };
+  auto top = [&](double v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o, G));
+    return v;
+  };
+  double a[2] = {0.0, 0.0}, x[2] = {0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (in[i]) { x[i] = (double)z[at + i]; a[i] = (double)((r[at + i] - shift[c0 + i]) + z[at + i]); }
+  const bool labelled = row && mask[j];
+  const int y = labelled ? labels[j] : -1;
+  const double e[2] = {c0 == y ? 1.0 : 0.0, c0 + 1 == y ? 1.0 : 0.0};
+  if (least_squares) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) x[i] = labelled ? (e[i] + nu * a[i]) / (1.0 + nu) : a[i];
+  } else {
+    if (!labelled) { x[0] = a[0]; x[1] = a[1]; }
+    bool done = !labelled, resolvable = false;
+    double d[2] = {0.0, 0.0}, t = 0.0, fx = 0.0, slope = 0.0;
+    int steps = 0;
+    while (__any_sync(0xffffffffu, !done)) {
+      const double v[2] = {x[0] + t * d[0], x[1] + t * d[1]};
+      const double m = top(fmax(in[0] ? v[0] : -1e300, in[1] ? v[1] : -1e300));
+      const double ex[2] = {in[0] ? exp(v[0] - m) : 0.0, in[1] ? exp(v[1] - m) : 0.0};
+      const double se = sum(ex[0] + ex[1]);
+      const double rest = sum(0.5 * nu * ((v[0] - a[0]) * (v[0] - a[0]) + (v[1] - a[1]) * (v[1] - a[1])) - (e[0] * v[0] + e[1] * v[1]));
+      const double f = m + log(se) + rest;
+      const bool accept = !resolvable || f <= fx + 1e-4 * t * slope || t < 1e-12;
+      // gradient, Newton step and slope at v; used if v is accepted
+      double g[2], mi[2], s[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        s[i] = ex[i] / se;
+        g[i] = in[i] ? s[i] - e[i] + nu * (v[i] - a[i]) : 0.0;
+        mi[i] = 1.0 / (s[i] + nu);
       }
-      if (gmax <= 1e-10) { done = true; break; }
+      const double gmax = top(fmax(fabs(g[0]), fabs(g[1])));
+      const double s_mg = sum(s[0] * mi[0] * g[0] + s[1] * mi[1] * g[1]), s_ms = sum(s[0] * mi[0] * s[0] + s[1] * mi[1] * s[1]);
       const double k = s_mg / (1.0 - s_ms);
-      double slope = 0.0;
-      for (int c = 0; c < C; ++c) {
-        const double mi = 1.0 / (s[c] + nu);
-        const double g = st[c];
-        const double d = -(mi * g + mi * s[c] * k);
-        slope += g * d;
-        st[c] = d;                       // Newton step
+      const double nd[2] = {-(mi[0] * g[0] + mi[0] * s[0] * k), -(mi[1] * g[1] + mi[1] * s[1] * k)};
+      const double ns = sum(g[0] * nd[0] + g[1] * nd[1]);
+      if (!done) {
+        if (accept) {
+          x[0] = v[0]; x[1] = v[1]; fx = f;
+          d[0] = nd[0]; d[1] = nd[1]; slope = ns; t = 1.0;
+          resolvable = -slope > 1e-9 * (1.0 + fabs(fx));
+          if (gmax <= 1e-10) done = true;
+          else if (++steps >= 100) {
+            done = true;
+            if (lane == 0) atomicAdd(not_converged, 1);
+          }
+        } else {
+          t *= 0.5;
+        }
       }
-      const bool resolvable = -slope > 1e-9 * (1.0 + fabs(fx));
-      double t = 1.0, ft;
-      for (;;) {
-        for (int c = 0; c < C; ++c) s[c] = x[c] + t * st[c];
-        ft = fval(s);
-        if (!resolvable || ft <= fx + 1e-4 * t * slope || t < 1e-12) break;
-        t *= 0.5;
-      }
-      for (int c = 0; c < C; ++c) x[c] = s[c];
-      fx = ft;
     }
-    if (!done) atomicAdd(not_converged, 1);
   }
   uint32_t mr = 0u;
-  for (int c = 0; c < C; ++c) {
-    const float zn = (float)x[c];
-    zj[c] = zn;
-    const float rn = (float)(a[c] - (double)zn);
-    rj[c] = rn;
-    mr = max(mr, abs_bits(rn));
+  if (row) {
+    float rn[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (!in[i]) continue;
+      const float zn = (float)x[i];
+      z[at + i] = zn;
+      rn[i] = (float)(a[i] - (double)zn);
+      r[at + i] = rn[i];
+      mr = max(mr, abs_bits(rn[i]));
+    }
+    if (rp.hi != nullptr && in[0]) {
+      const float scale = tc_scale_of(*rp.exp);
+      float h0, l0, h1, l1;
+      tc_split(rn[0], scale, h0, l0);
+      tc_split(rn[1], scale, h1, l1);
+      *reinterpret_cast<uint32_t *>(rp.hi + at) = tc_pack(h0, h1);
+      *reinterpret_cast<uint32_t *>(rp.lo + at) = tc_pack(l0, l1);
+    }
   }
   if (amax_r != nullptr) commit_amax(mr, amax_r);
+}
+inline void launch_zlast(cudaStream_t st, float *r, float *z, const float *shift, const int *labels, const uint8_t *mask, int n_rows,
+                         int C, int ld, double nu, int *not_converged, uint32_t *amax_r, int least_squares, const PlaneOut &rp) {
+  auto go = [&](auto G) {
+    constexpr int g = decltype(G)::value;
+    zlast_kernel<g><<<(int)ceil_div((int64_t)n_rows * g, 128), 128, 0, st>>>(r, z, shift, labels, mask, n_rows, C, ld, nu, not_converged,
+                                                                            amax_r, least_squares, rp);
+  };
+  if (C <= 8) go(std::integral_constant<int, 4>{});
+  else if (C <= 16) go(std::integral_constant<int, 8>{});
+  else if (C <= 32) go(std::integral_constant<int, 16>{});
+  else go(std::integral_constant<int, 32>{});
 }
 
 // t = u + rho (p - q) from the stored iterates (after the start or after the caller has set a tensor); the same

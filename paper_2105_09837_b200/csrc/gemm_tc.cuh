@@ -16,7 +16,8 @@
 // transposed, and the kernels that write a matrix write its planes beside it.  Such a kernel does not know the
 // largest magnitude of what it writes and takes the exponent from a bound or a prediction (TcOperand::exp); the product
 // compares it with the largest magnitude that was then seen, and if the scaling turns out unusable two spare warps build
-// that operand's planes from the fp32 matrix instead of loading them (rare, slower, same result).
+// that operand's planes from the fp32 matrix instead of loading them (rare, slower, same result; large matrices get a
+// kernel that does it beforehand, see check_planes_kernel).
 //
 // One thread issues tcgen05.mma; completion is tracked with mbarriers; two sets of four accumulate warps take the output
 // tiles of a block in turn: a set reads each K block's main term from tensor memory, adds it to a register accumulator and
@@ -93,7 +94,8 @@ template <class Epi> struct epi_planes<Epi, std::enable_if_t<Epi::kPlanes>> { st
 struct TcOperand {
   const int *exp = nullptr;        // exponent the planes were made with; null: 0 (integer planes)
   const uint32_t *amax = nullptr;  // bit pattern of max|x| as seen by now; null: the planes are known to be good
-  const float *x = nullptr;        // the fp32 matrix (read only if the planes are refused), leading dimension ld
+  const float *x = nullptr;        // the fp32 matrix (read only if the planes are refused), leading dimension ld; null: refused
+                                   // planes were made again beforehand, with the exponent of amax (check_planes_kernel)
   int ld = 0;
 };
 
@@ -177,10 +179,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // scaling exponents of the two operands (written by earlier kernels of the stream), and whether the planes made with
   // them are usable; the same for every block
   int exp_a = prm.a.exp ? *prm.a.exp : 0, exp_b = prm.b.exp ? *prm.b.exp : 0;
-  const bool split_a = prm.a.amax != nullptr && !tc_planes_usable(*prm.a.amax, exp_a);
-  const bool split_b = prm.b.amax != nullptr && !tc_planes_usable(*prm.b.amax, exp_b);
-  if (split_a) exp_a = tc_scale_exp(*prm.a.amax);
-  if (split_b) exp_b = tc_scale_exp(*prm.b.amax);
+  bool split_a = prm.a.amax != nullptr && !tc_planes_usable(*prm.a.amax, exp_a);
+  bool split_b = prm.b.amax != nullptr && !tc_planes_usable(*prm.b.amax, exp_b);
+  if (split_a) { exp_a = tc_scale_exp(*prm.a.amax); split_a = prm.a.x != nullptr; }
+  if (split_b) { exp_b = tc_scale_exp(*prm.b.amax); split_b = prm.b.x != nullptr; }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -378,6 +380,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // K-major: 64 or 128 rows of 8 chunks, inner = contraction; MN-major: 64 rows of 8 or 16 chunks, inner = output index
         const int rows = mn ? n_k - k0 : n_outer - o0, chunks = mn ? 8 * boxes : 8, inner0 = mn ? o0 : k0;
         const float *src = o.x + (size_t)(mn ? k0 : o0) * o.ld + inner0;
+#pragma unroll 4
         for (int i = t; i < 512 * boxes; i += 32 * TC_SPLIT_WARPS) {
           const int r = i / chunks, c = i % chunks;
           float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;

@@ -97,7 +97,7 @@ struct Layer {
   float *q = nullptr, *u = nullptr;          // [N][ld_out], hidden layers only
   float *t = nullptr;       // [N][ld_in], l >= 2: u_{l-1} + rho (p_l - q_{l-1}), the product-free part of grad_p phi
   float *gradW = nullptr;   // [n_out][ld_in]
-  // Tensor-core path: planes of W, of grad_W and of r (written by the z-step for the next p-gradient; hidden layers only, and
+  // Tensor-core path: planes of W, of grad_W and of r (written by the z-step for the next p-gradient;
   // none if the device has no room: the products then split r first), of p_1 = X, which never changes; the exponent words
   // belong to finalize_tau_kernel / finalize_theta_kernel, which settle them before the planes are written
   Planes Wp, Gp, rp, xp;
@@ -455,6 +455,17 @@ static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t ro
   Launch l(c, KC_PLANES, st, (lo_too ? 8.0 : 6.0) * rows * cols, 0);
   rows_planes_kernel<<<ew_grid(n8), 256, 0, st>>>(x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
 }
+// Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel).
+// From 2^20 elements on: below, the launch costs more than it saves.
+constexpr size_t CHECK_PLANES_FROM = size_t(1) << 20;
+static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, Operand &o) {
+  const size_t n = rows * o.ld;
+  if (!c->use_tc || o.hi == nullptr || o.check == nullptr || o.x == nullptr || n < CHECK_PLANES_FROM) return;
+  Launch l(c, KC_PLANES, st, 0, 0);
+  check_planes_kernel<<<ew_grid(n / 8), 256, 0, st>>>(o.x, n / 8, o.check, o.exp, const_cast<__half *>(o.hi),
+                                                     o.lo == o.hi ? nullptr : const_cast<__half *>(o.lo));
+  o.x = nullptr;
+}
 static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
   PD_TRY(dev_alloc(c, &pl->hi, n, zero));
   PD_TRY(dev_alloc(c, &pl->lo, n, zero));
@@ -530,11 +541,10 @@ static int gemm_over_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N
 
 // ---- pieces of one iteration -------------------------------------------------------------------------------
 
-static Operand operand_W(const Layer &ly) { return plane_operand(ly.W, ly.ld_in, ly.Wp); }
+static Operand operand_W(const Layer &ly) { return plane_operand(ly.W, ly.ld_in, ly.Wp, ly.amax_W); }
 // p_1 = X, which never changes (its planes are kept on the tensor-core path)
 static Operand operand_X(const Layer &ly) { return plane_operand(ly.p, ly.ld_in, ly.xp); }
-// r_l as the z-step left it; the last layer has no planes from there (its exponent word says so), its few columns are split by
-// the product itself
+// r_l as the z-step left it
 static Operand operand_r(const Layer &ly) {
   Operand o = plane_operand(ly.r, ly.ld_out, ly.rp, ly.amax_r);
   o.amax = ly.amax_r;
@@ -552,7 +562,7 @@ static int refresh_residual(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
   if (!c->use_tc) {       // the CUDA-core product does not track the maximum of what it stores
     Launch l(c, KC_AMAX, st, 4.0 * c->N * ly.ld_out, 0);
     absmax_kernel<<<ew_grid((size_t)c->N * ly.ld_out / 4), EW_THREADS, 0, st>>>(ly.r, (size_t)c->N * ly.ld_out / 4, ly.amax_r);
-  } else if (ly.rp.hi != nullptr && &ly != &c->layers.back()) {
+  } else if (ly.rp.hi != nullptr) {
     split_rows(c, st, ly.r, (size_t)c->N, ly.n_out, ly.ld_out, ly.amax_r, ly.rp);
   }
   return PDADMM_OK;
@@ -576,8 +586,11 @@ static int p_gradient_and_tau(pdadmm_ctx *c, int l /*0-based, >= 1*/) {
     epi.H = s.pl0.hi; epi.L = norm_only ? nullptr : s.pl0.lo; epi.h_exp = ly.g_exp;
     G = plane_operand(s.s1, ly.ld_in, Planes{s.pl0.hi, norm_only ? s.pl0.hi : s.pl0.lo, ly.g_exp}, w_g);
   }
-  PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, operand_r(ly), operand_W(ly), epi, s.slots, &np,
+  Operand R = operand_r(ly);
+  check_planes(c, s.st, (size_t)N, R);
+  PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, R, operand_W(ly), epi, s.slots, &np,
                           (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in));
+  check_planes(c, s.st, (size_t)N, G);
   int np2 = 0;
   double *slots_b = s.slots + s.n_slots / 2;          // second half of the slot buffer
   if (norm_only) {
@@ -691,7 +704,7 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
   // p+ (layer 1: X, which never changes; pdADMM-G: planes from the p-step; pdADMM-G-Q: p+ = code * s)
   Operand P{ly.p, ly.ld_in, ly.amax_p};
   if (c->use_tc) P = l == 0 ? operand_X(ly) : (c->int_operands ? int_operand(ly.p_plane, ly.ld_in, ly.scale)
-                                                               : plane_operand(ly.p, ly.ld_in, s.pl1));
+                                                               : plane_operand(ly.p, ly.ld_in, s.pl1, ly.amax_p));
   if (!c->use_tc) {
     dim3 grid((unsigned)ceil_div(ly.n_in, SG_BN), (unsigned)ceil_div(ly.n_out, SG_BM), (unsigned)ly.n_split);
     Launch k(c, KC_GEMM_GRADW, s.st, 4.0 * ((double)N * ly.n_in + (double)N * ly.n_out), 2.0 * N * ly.n_in * ly.n_out);
@@ -699,7 +712,8 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
                                                  s.part, ly.ld_in);
   } else {
     // both operands are node-major; the product contracts over the rows of their planes as they are
-    Operand R = l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, c->levels ? ly.amax_r : nullptr);
+    Operand R = l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, ly.amax_r);
+    if (l == 0 || c->levels) check_planes(c, s.st, (size_t)N, R);      // (the p-step's planes are scaled by a bound)
     if (R.hi == nullptr) {                       // no room was left for the planes of r
       const Planes pl{s.pl0.hi, s.pl0.lo, s.a_exp};
       split_rows(c, s.st, ly.r, (size_t)N, ly.n_out, ly.ld_out, ly.amax_r, pl);
@@ -729,11 +743,11 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
   int np = 0;
   double *slots_b = s.slots + s.n_slots / 2;
   EpiStoreSumsq epi{s.s1, ly.ld_out};
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_GP, s.st, N, ly.n_out, ly.n_in, P, plane_operand(ly.gradW, ly.ld_in, ly.Gp, w_G), epi,
-                           slots_b, &np, 0));
+  Operand G = plane_operand(ly.gradW, ly.ld_in, ly.Gp, w_G);
+  check_planes(c, s.st, (size_t)ly.n_out, G);
+  PD_TRY(gemm_nodes<false>(c, KC_GEMM_GP, s.st, N, ly.n_out, ly.n_in, P, G, epi, slots_b, &np, 0));
   ThetaPlanes tp{};
-  if (c->use_tc)       // no planes of r from the z-step of the last layer: its exponent stays TC_NO_PREDICTION
-    tp = ThetaPlanes{ly.amax_r, ly.amax_W, w_G, ly.Wp.exp, l + 1 < c->L ? ly.rp.exp : nullptr, ly.Gp.exp};
+  if (c->use_tc) tp = ThetaPlanes{ly.amax_r, ly.amax_W, w_G, ly.Wp.exp, ly.rp.exp, ly.Gp.exp};
   if (c->reduce != nullptr) {
     // ||G p+||^2 is a sum over nodes (||G||^2 is the same on every shard already)
     PD_TRY(shard_sum_slots(c, s.st, s.red, slots_b, np, nullptr, 0));
@@ -794,9 +808,9 @@ static void zqu_step(pdadmm_ctx *c, int l) {
                                                c->code_bytes == 2);
     }
   } else {
-    Launch k(c, KC_ZLAST, s.st, 16.0 * N * ly.n_out, 0);
-    zlast_kernel<<<(int)ceil_div(N, 128), 128, 0, s.st>>>(ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out,
-                                                          ly.ld_out, (double)c->nu, c->d_flag, ly.amax_r, c->ls_risk ? 1 : 0);
+    Launch k(c, KC_ZLAST, s.st, (c->use_tc ? 20.0 : 16.0) * N * ly.n_out, 0);
+    launch_zlast(s.st, ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out, ly.ld_out, (double)c->nu, c->d_flag, ly.amax_r,
+                 c->ls_risk ? 1 : 0, plane_out(c, ly.rp));
   }
 }
 
@@ -1241,22 +1255,14 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
       PD_TRY(dev_alloc(c, &x.a_exp, 1));
     }
   }
-  // Planes of r from one iteration to the next, hidden layers: worth their memory (the p-gradient's product would have to split
+  // Planes of r from one iteration to the next: worth their memory (the p-gradient's product would have to split
   // r first otherwise, 8 bytes per element), but nothing depends on them.  All or none, and at most 7/8 of what is free.
   if (c->use_tc) {
     size_t need = 0, free_bytes = 0, total = 0;
-    for (int l = 0; l + 1 < c->L; ++l) need += (size_t)N * c->layers[l].ld_out * 4;
+    for (int l = 0; l < c->L; ++l) need += (size_t)N * c->layers[l].ld_out * 4;
     PD_CUDA(cudaMemGetInfo(&free_bytes, &total));
-    const bool room = need <= free_bytes / 8 * 7 || need <= c->arena_cap - c->arena_used;
-    for (int l = 0; l < c->L; ++l) {
-      Layer &ly = c->layers[l];
-      if (l + 1 < c->L && room) {
-        PD_TRY(alloc_planes(c, (size_t)N * ly.ld_out, &ly.rp));
-      } else if (l + 1 == c->L) {        // the product splits the last layer's few columns itself: planes of no use, refused
-        PD_TRY(alloc_planes(c, (size_t)N * ly.ld_out, &ly.rp));
-        PD_CUDA(cudaMemsetAsync(ly.rp.exp, 0x80, sizeof(int), st));       // no exponent: TC_NO_PREDICTION
-      }
-    }
+    if (need <= free_bytes / 8 * 7 || need <= c->arena_cap - c->arena_used)
+      for (int l = 0; l < c->L; ++l) PD_TRY(alloc_planes(c, (size_t)N * c->layers[l].ld_out, &c->layers[l].rp));
   }
   c->ev_p.resize(c->L);
   for (auto &e : c->ev_p) PD_CUDA(pool.take_event(false, &e));
