@@ -35,7 +35,6 @@ struct LayerScalars {
   double sum_wd2;     // ||W (p+ - p)||^2    (quantised trial)
   double sum_G2;      // ||grad_W||^2
   double sum_Gp2;     // ||grad_W p+||^2
-  double res2;        // ||p_{l+1} - q_l||^2
   double tau;         // tau_l
   double theta;       // theta_l (0 if grad_W = 0)
   float inv_tau;      // 1/tau
@@ -108,7 +107,7 @@ __device__ __forceinline__ void store_planes4(const PlaneOut &o, size_t i, float
 // elements of p first, then those of r), with the planes of both for the W-gradient and G p+.  16 bytes per element and
 // matrix: read 8, write 4 and the planes 4.  (Separate passes that split r and p again cost 8 bytes more each, and the
 // products that took them fp32 ran at 0.6 of their speed.)
-__global__ void __launch_bounds__(EW_THREADS)
+__global__ void __launch_bounds__(EW_THREADS, 5)
 pstep_kernel(float *__restrict__ p, const float *__restrict__ g, size_t n4p, float *__restrict__ r, const float *__restrict__ wg,
              size_t n4r, const float *__restrict__ inv, PlaneOut pp, PlaneOut rp,
              uint32_t *__restrict__ amax_p /* receives max|p| (see commit_amax); may be null */, uint32_t *__restrict__ amax_r) {
@@ -117,16 +116,16 @@ pstep_kernel(float *__restrict__ p, const float *__restrict__ g, size_t n4p, flo
   auto pass = [&](float *__restrict__ y, const float *__restrict__ x, size_t n4, const PlaneOut &o, uint32_t *amax) {
     const float scale = o.hi != nullptr ? tc_scale_of(*o.exp) : 1.f;
     uint32_t m = 0u;
-    // four groups per pass: eight loads in flight per thread
-    for (size_t i = first; i < n4; i += 4 * stride) {
-      float4 v[4], w[4];
+    // two groups per pass: four loads in flight per thread (four groups take more registers than two blocks have beside a product)
+    for (size_t i = first; i < n4; i += 2 * stride) {
+      float4 v[2], w[2];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < 2; ++k) {
         const size_t q = i + k * stride;
         if (q < n4) { v[k] = ld4(y, q); w[k] = ld4(x, q); }
       }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < 2; ++k) {
         const size_t q = i + k * stride;
         if (q >= n4) continue;
         v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
@@ -235,7 +234,8 @@ codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, size_t n4,
 // ---- finalisers of the step parameters (one block of FIN_THREADS threads) ---------------------------------
 // Fixed-order sum of n slots by one block of FIN_THREADS threads: thread t adds slots t, t + FIN_THREADS, ..., then a
 // fixed tree.  Result in thread 0.
-constexpr int FIN_THREADS = 1024;
+// 256 threads fit beside a product; there are a few thousand slots at most.
+constexpr int FIN_THREADS = 256;
 __device__ __forceinline__ double block_sum_slots(const double *__restrict__ slots, int n, double *sh /* FIN_THREADS */) {
   // four independent partial sums per thread keep four loads in flight; the order of the additions is fixed
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
@@ -437,13 +437,14 @@ resid_colsum_kernel(float *__restrict__ r, const float *__restrict__ gp, const L
 
 // out[c] = sum over the blocks' slots of column c (the first half of finalize_bias_kernel, for a context that owns only
 // part of the nodes: the totals are then added over the shards before the mean is taken).  Same thread layout.
-constexpr int BIAS_GROUPS = 32;          // slot groups per block of the two kernels below (blockDim = (32, BIAS_GROUPS))
+constexpr int BIAS_GROUPS = 8;          // slot groups per block of the two kernels below (blockDim = (32, BIAS_GROUPS))
 __global__ void __launch_bounds__(32 * BIAS_GROUPS)
 colsum_total_kernel(const double *__restrict__ slots, int n_slots, int ld, double *__restrict__ out) {
   __shared__ double sh[BIAS_GROUPS][33];
   const int c = blockIdx.x * 32 + threadIdx.x;
   double s = 0.0;
   if (c < ld)
+#pragma unroll 8
     for (int i = threadIdx.y; i < n_slots; i += BIAS_GROUPS) s += slots[(size_t)i * ld + c];
   sh[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
@@ -472,8 +473,7 @@ sumsq_amax_kernel(const float *__restrict__ G, size_t n4, uint32_t *__restrict__
 
 // b+ = b - mean_j r[j][:]  (Eq. "update b" with the step 1/(nu N), i.e. the exact minimiser);
 // shift[c] = that mean, which the z-update subtracts from r.  blockDim = (32 columns, BIAS_GROUPS slot groups): group g
-// adds the slots g, g + BIAS_GROUPS, ... of its column, the group sums are then added in group order (32 groups keep
-// 32 rows of slots in flight per block; the kernel has only ld / 32 blocks).
+// adds the slots g, g + BIAS_GROUPS, ... of its column, the group sums are then added in group order.
 __global__ void __launch_bounds__(32 * BIAS_GROUPS)
 finalize_bias_kernel(const double *__restrict__ slots, int n_slots, int ld, int width, double inv_n,
                      float *__restrict__ b, float *__restrict__ shift) {
@@ -481,6 +481,7 @@ finalize_bias_kernel(const double *__restrict__ slots, int n_slots, int ld, int 
   const int c = blockIdx.x * 32 + threadIdx.x;
   double s = 0.0;
   if (c < ld)
+#pragma unroll 8
     for (int i = threadIdx.y; i < n_slots; i += BIAS_GROUPS) s += slots[(size_t)i * ld + c];
   sh[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
@@ -500,17 +501,16 @@ finalize_bias_kernel(const double *__restrict__ slots, int n_slots, int ld, int 
 // the level set of p_{l+1}, the variant at the end of Sec. "Quantization Extension"), residual p_{l+1} - q+,
 // u+ by Eq. "update u", the linear residual of the next iteration r = a - z+, and t_{l+1} = u+ + rho (p_{l+1} - q+),
 // the part of the next p-gradient that does not involve a product.
-__global__ void __launch_bounds__(EW_THREADS)
+// At most 48 registers: two blocks fit on an SM beside a product.
+__global__ void __launch_bounds__(EW_THREADS, 5)
 zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, float *__restrict__ u,
            const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
            float rho, float nu, float slope, float q_scale, float q_lo, float q_top, float *__restrict__ t_next,
-           double *__restrict__ slots, uint32_t *__restrict__ amax_r /* max|r| (see commit_amax); may be null */,
+           uint32_t *__restrict__ amax_r /* max|r| (see commit_amax); may be null */,
            PlaneOut rp /* planes of r for the coming p-gradient */,
            const void *__restrict__ codes_next /* pdADMM-G-Q: codes of p_next, read instead of it */, int wide_codes) {
-  __shared__ double red[EW_THREADS / 32];
   const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
   const float inv_rn = 1.0f / (rho + nu), inv_neg = 1.0f / (2.0f + slope * slope);
-  double ss = 0.0;
   uint32_t mr = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     const float4 sh = ld4(shift, i % ld4cols);
@@ -531,7 +531,6 @@ zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, 
       const float res = pv.f - qq;                                                  \
       zn.f = zz; qn.f = qq; un.f = fmaf(rho, res, uv.f); rn.f = a - zz;             \
       tn.f = fmaf(rho, res, un.f);                                                  \
-      ss += (double)res * res;                                                      \
     }
     PD_ZQU(x) PD_ZQU(y) PD_ZQU(z) PD_ZQU(w)
 #undef PD_ZQU
@@ -540,8 +539,6 @@ zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, 
     mr = max(mr, abs_bits(rn));
   }
   if (amax_r != nullptr) commit_amax(mr, amax_r);
-  const double tot = block_sum<EW_THREADS>(ss, red);
-  if (threadIdx.x == 0) slots[blockIdx.x] = tot;
 }
 
 // ---- the same for a smooth activation: z-update by lookup table ---------------------------------------------
@@ -610,15 +607,13 @@ __global__ void __launch_bounds__(EW_THREADS)
 zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, float *__restrict__ u,
                  const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
                  float rho, float nu, float act, float t_lo, float t_step, int T, float q_scale, float q_lo, float q_top,
-                 float *__restrict__ t_next, double *__restrict__ slots, uint32_t *__restrict__ amax_r, PlaneOut rp,
+                 float *__restrict__ t_next, uint32_t *__restrict__ amax_r, PlaneOut rp,
                  const void *__restrict__ codes_next, int wide_codes) {
   extern __shared__ float table_sh[];              // f(z_i)
-  __shared__ double red[EW_THREADS / 32];
   for (int i = threadIdx.x; i < T; i += blockDim.x) table_sh[i] = act_eval(__fadd_rn(t_lo, __fmul_rn((float)i, t_step)), act);
   __syncthreads();
   const float inv_rn = 1.0f / (rho + nu);
   const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
-  double ss = 0.0;
   uint32_t mr = 0u;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     const float4 sh = ld4(shift, i % ld4cols);
@@ -638,7 +633,6 @@ zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict
       const float res = pn[e] - qq;
       zn[e] = zb[e]; qn[e] = qq; un[e] = fmaf(rho, res, uo[e]); rn[e] = a[e] - zb[e];
       tn[e] = fmaf(rho, res, un[e]);
-      ss += (double)res * res;
     }
     st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(q, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
     st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
@@ -648,8 +642,6 @@ zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict
     mr = max(mr, abs_bits(r4));
   }
   if (amax_r != nullptr) commit_amax(mr, amax_r);
-  const double tot = block_sum<EW_THREADS>(ss, red);
-  if (threadIdx.x == 0) slots[blockIdx.x] = tot;
 }
 
 // ---- z-update of the last layer -------------------------------------------------------------------

@@ -19,11 +19,12 @@
 // that operand's planes from the fp32 matrix instead of loading them (rare, slower, same result; large matrices get a
 // kernel that does it beforehand, see check_planes_kernel).
 //
-// One thread issues tcgen05.mma; completion is tracked with mbarriers; two sets of four accumulate warps take the output
-// tiles of a block in turn: a set reads each K block's main term from tensor memory, adds it to a register accumulator and
-// finally applies the scaling and the fused epilogue -- while it is in that epilogue the other set already accumulates
-// the next tile, so the tensor pipe never waits for a store phase.
+// One thread issues tcgen05.mma; completion is tracked with mbarriers; eight accumulate warps read each K block's main term
+// from tensor memory, add it to register accumulators and finally apply the scaling and the fused epilogue.  While
+// they are in that epilogue the MMAs run up to three K blocks ahead into the next tile.
 //
+// A block takes 61 % of an SM's registers and leaves 17 KB of its shared memory: bandwidth-bound kernels of other layers run
+// beside it (they are launched with a higher priority), which hides about half of their time behind the products.
 // Tile: 128 x 128 outputs per block, 64-deep K blocks.  What bounds the product is the traffic between L2 and the SMs
 // (10.6 TB/s measured, whatever the number of planes): a block on its own loads A and B planes of 64 KB per K block for
 // three times 2 MFLOP.  So two neighbouring SMs work as a pair on 256 x 128 outputs (tcgen05 cta_group::2): each loads the
@@ -51,24 +52,24 @@ constexpr int TC_BOX_BYTES = 64 * TC_BK * 2;                   // 8 KB: what one
 constexpr int TC_STAGE_SPACE = 12 * TC_PLANE_BYTES;            // 192 KB: 3 to 8 stages, by the number of planes
 constexpr int TC_MAX_STAGES = 8;
 // Three warpgroups (register budgets are set per warpgroup): 0 = TMA warp, MMA warp and two warps that split operands when
-// a scaling was unusable; 1, 2 = the two accumulate sets, four warps each (a warp owns one 32-lane quarter of tensor memory,
-// i.e. a quarter of the tile's rows, and all 128 columns: 128 accumulators per thread, and 64 registers for the read-out
-// that is under way).  Registers: the block is launched with 384 x 168 = 64512; warpgroup 0 keeps 72 per thread, the
-// accumulate sets take 216: 128 (72 + 2 x 216) = 64512, so every increase is satisfiable.
+// a scaling was unusable; 1, 2 = the accumulate warps: a warp can only reach its own 32-lane quarter of tensor memory, so
+// warp w owns the rows of quarter w mod 4 and columns 64 (w / 4) .. +63 of the tile, 64 accumulators per thread.
+// Registers: the block is launched with 384 x 104 = 39936; warpgroup 0 keeps 56 per thread, the
+// accumulate warps take 128: 128 (56 + 2 x 128) = 39936, so every increase is satisfiable.
 constexpr int TC_SPLIT0 = 2, TC_SPLIT_WARPS = 2;               // first splitting warp
 constexpr int TC_ACC0 = 4;                                     // first accumulate warp
 constexpr int TC_THREADS = 384;
-constexpr int TC_ACC_WARPS = 4;                                // warps of one accumulate set
-constexpr int TC_REGS_LAUNCH = 168, TC_REGS_CTRL = 72, TC_REGS_ACC = 216;
+constexpr int TC_ACC_WARPS = 8;
+constexpr int TC_REGS_LAUNCH = 104, TC_REGS_CTRL = 56, TC_REGS_ACC = 128;
 static_assert(TC_THREADS * TC_REGS_LAUNCH <= 65536, "register file");
 static_assert(128 * (TC_REGS_CTRL + 2 * TC_REGS_ACC) <= TC_THREADS * TC_REGS_LAUNCH,
               "the warpgroups' register shares exceed what the block is launched with: an increase would wait for ever");
 constexpr int TC_ACC_BUFS = 3;                                 // main-term accumulator tiles in tensor memory
 constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 1 correction tile
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
-constexpr int TC_TR_BYTES = 8 * 32 * 32 * 4;                   // epilogue transpose: 8 warps x 32 rows x 32 columns
+constexpr int TC_TR_BYTES = 8 * 32 * 16 * 4;                   // epilogue transpose: 8 warps x 32 rows x 16 columns
 constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
-static_assert(8 * (2 * TC_MAX_STAGES + 3 * TC_ACC_BUFS + 2) + 12 <= 256, "barriers");
+static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 2) + 12 <= 256, "barriers");
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -111,8 +112,10 @@ struct TcParams {
   // A slice leaves its accumulators in tail_ws; the warp that finds itself last (tail_count) adds the slices
   // in slice order and runs the epilogue.  tail_split <= 1 switches this off.
   int tail_begin, tail_split;
-  float *tail_ws;         // [tiles from tail_begin][tail_split][4 or 8 row quarters][128][32] floats
-  int *tail_count;        // [tiles from tail_begin][4 or 8 row quarters], zero before and after every launch
+  // Sums of squares: one slot per accumulate warp of the grid for the whole tiles of its block, then one per tail tile and
+  // warp of its block (pair), all in a fixed order whichever block finishes a tail tile.
+  float *tail_ws;         // [tiles from tail_begin][tail_split][8 or 16 warps][64][32] floats
+  int *tail_count;        // [tiles from tail_begin][8 or 16 warps], zero before and after every launch
   float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
 };
 
@@ -140,7 +143,7 @@ struct TcParams {
 // plane to load and no MMA for it (two MMAs per product instead of three), and prm.mul = s restores the values.
 enum : int { TC_NT = 0, TC_A_MN = 1, TC_B_MN = 2 };
 template <int LAYOUT, class Epi, int ZERO, bool PAIR>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __maxnreg__(TC_REGS_LAUNCH)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_alo,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_blo,
                const __grid_constant__ TcParams prm, Epi epi, double *__restrict__ partials) {
@@ -151,7 +154,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   constexpr bool A_LO = !(ZERO & 1) && !COARSE, B_LO = !(ZERO & 2) && !COARSE;
   constexpr int FLUSH = COARSE ? (1 << 30) : TC_FLUSH;        // K blocks per read-out of the main accumulator
   constexpr int A_PLANES = A_LO ? 2 : 1, B_PLANES = B_LO ? 2 : 1;
-  constexpr int CG = PAIR ? 2 : 1, QUARTERS = PAIR ? 8 : 4, TILE_M = PAIR ? 2 * TC_BM : TC_BM;
+  constexpr int CG = PAIR ? 2 : 1, WARPS = CG * TC_ACC_WARPS, TILE_M = PAIR ? 2 * TC_BM : TC_BM;
   constexpr int B_PLANE_BYTES = PAIR ? TC_BOX_BYTES : TC_PLANE_BYTES, BN = PAIR ? TC_BN / 2 : TC_BN;    // B held by this block
   constexpr int STAGE_BYTES = A_PLANES * TC_PLANE_BYTES + B_PLANES * B_PLANE_BYTES;
   constexpr int STAGES = TC_STAGE_SPACE / STAGE_BYTES < TC_MAX_STAGES ? TC_STAGE_SPACE / STAGE_BYTES : TC_MAX_STAGES;
@@ -161,7 +164,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   uint8_t *tr_base = smem + TC_STAGE_SPACE;
   uint64_t *bars = reinterpret_cast<uint64_t *>(tr_base + TC_TR_BYTES);
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
-  uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + 2 * TC_ACC_BUFS;     // acc_full: [set][buffer]
+  uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
   uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain_bar + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
@@ -191,7 +194,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
     for (int b = 0; b < TC_ACC_BUFS; ++b) {
       ptx::mbar_init(&acc_full[b], 1);
-      ptx::mbar_init(&acc_full[TC_ACC_BUFS + b], 1);
       ptx::mbar_init(&acc_empty[b], CG * TC_ACC_WARPS);
     }
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
@@ -352,10 +354,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 }
               }
               ptx::mma_commit<CG>(&empty_bar[s]);          // stage can be refilled once these MMAs have read it
-              // the group's partial product is complete.  Each accumulate set has its own barriers: a set
-              // is idle during the other set's tiles, and a waiter that lags by more than one phase of a barrier
-              // would take an earlier completion of the same parity for its own.
-              if (last) ptx::mma_commit<CG>(&acc_full[(ti & 1) * TC_ACC_BUFS + b]);
+              if (last) ptx::mma_commit<CG>(&acc_full[b]);      // the group's partial product is complete
             }
             if (last) {
               ++used;
@@ -418,40 +417,38 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else {
     ptx::setmaxnreg_inc<TC_REGS_ACC>();
-    // -------------------------------------------------------------- accumulate, then epilogue (2 sets x 128 threads)
-    // The block's output tiles go to the two sets in turn.  Warp w of a set owns tensor-memory lanes 32 (w mod 4) ..
-    // +31 = output rows m0 + that range, and all 128 columns of the tile.  Both sets count every K block, so that the
-    // accumulator buffers stay in step.
-    const int aw = warp - TC_ACC0, set = aw >> 2, quarter = warp & 3;
-    const int lane_base = quarter * 32;
-    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 8;    // 32 rows x 8 float4 per warp
+    // -------------------------------------------------------------- accumulate, then epilogue (8 warps)
+    const int aw = warp - TC_ACC0, quarter = warp & 3, col_base = 64 * (aw >> 2);
+    const int lane_base = quarter * 32, piece = (int)rank * TC_ACC_WARPS + aw;
+    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 4;    // 32 rows x 4 float4 per warp
     // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
     // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
     const int n_pad = epi.ldc;
     bool ok = true;
-    int b = 0, ti = 0;
-    uint32_t phases = 0u;                              // bit b: parity of this set's next completion of acc_full[set][b]
-    for (int tile = unit0; tile < n_tiles && ok; tile += unit_step, ++ti) {
+    int b = 0;
+    double ss = 0.0;                                   // this thread's part of its warp's slot
+    uint32_t ph = 0;                                   // phase of acc_full[b]
+    for (int tile = unit0; tile < n_tiles && ok; tile += unit_step) {
       int m0, n0, k_begin, n_kb, z;
       tile_coords(tile, m0, n0, k_begin, n_kb, z);
+      n0 += col_base;                               // of this warp
       const int n_grp = COARSE ? (n_kb > 0 ? 1 : 0) : n_kb;   // read-outs of the main accumulator for this tile
-      if ((ti & 1) != set) { b = (b + n_grp) % TC_ACC_BUFS; continue; }    // the other set's tile
       if (m0 + lane_base + lane < prm.M) {          // this thread's row of the epilogue inputs, on its way to L2
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
+        for (int h = 0; h < 2; ++h) {
           const int col = n0 + h * 32;
           if (col < n_pad) epi.prefetch(m0 + lane_base + lane, col);
         }
       }
-      uint64_t acc[64];                             // columns 2 j, 2 j + 1 in acc[j]
+      uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
 #pragma unroll
-      for (int j = 0; j < 64; ++j) acc[j] = 0ull;
-      // acc += tile (or tile * 2^-11): the load of the next 32 columns is under way while the last ones are added, and
-      // the tile is given back (one arrival per warp on `done` of block 0, whose MMA thread waits) as soon as its last columns are in registers
-      auto add_tile = [&](uint32_t col_base, auto plain, uint64_t *done) {
-        const uint32_t src = tmem_base + ((uint32_t)lane_base << 16) + col_base;
-        uint32_t v0[32], v1[32];
-        auto add = [&](const uint32_t (&v)[32], int h) {
+      for (int j = 0; j < 32; ++j) acc[j] = 0ull;
+      // acc += tile (or tile * 2^-11).  The tile is given back (one arrival per warp on `done` of block 0, whose MMA thread
+      // waits) as soon as its last columns are in registers.
+      auto add_tile = [&](uint32_t col, auto plain, uint64_t *done) {
+        const uint32_t src = tmem_base + ((uint32_t)lane_base << 16) + col + (uint32_t)col_base;
+        uint32_t v[32];
+        auto add = [&](int h) {
           const uint64_t w = ptx::pack_f2(0x3A000000u, 0x3A000000u);       // 2^-11 twice
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -459,29 +456,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             acc[16 * h + j] = decltype(plain)::value ? ptx::add_f2(acc[16 * h + j], x) : ptx::fma_f2(w, x, acc[16 * h + j]);
           }
         };
-        ptx::tmem_ld32(src, v0);
-        ptx::tmem_ld_wait(v0);
-        ptx::tmem_ld32(src + 32u, v1);
-        add(v0, 0);
-        ptx::tmem_ld_wait(v1);
-        ptx::tmem_ld32(src + 64u, v0);
-        add(v1, 1);
-        ptx::tmem_ld_wait(v0);
-        ptx::tmem_ld32(src + 96u, v1);
-        add(v0, 2);
-        ptx::tmem_ld_wait(v1);
+        ptx::tmem_ld32(src, v);
+        ptx::tmem_ld_wait(v);
+        add(0);
+        ptx::tmem_ld32(src + 32u, v);
+        ptx::tmem_ld_wait(v);
         ptx::tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(done, 0));
-        add(v1, 3);
+        add(1);
       };
       for (int g = 0; g < n_grp && ok; ++g) {
-        ok = ptx::mbar_wait(&acc_full[set * TC_ACC_BUFS + b], (phases >> b) & 1u, abort_flag);
+        ok = ptx::mbar_wait(&acc_full[b], ph, abort_flag);
         if (!ok) break;
-        phases ^= 1u << b;
         ptx::tc_fence_after_sync();
         add_tile((uint32_t)(b * TC_BN), std::true_type{}, &acc_empty[b]);
-        if (++b == TC_ACC_BUFS) b = 0;
+        if (++b == TC_ACC_BUFS) { b = 0; ph ^= 1u; }
       }
       if (!ok) break;
       if (n_kb > 0) {
@@ -492,11 +482,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t u1 = __float_as_uint(tc_pow2(-e1)), u2 = __float_as_uint(tc_pow2(-e2));
         const uint64_t w1 = ptx::pack_f2(u1, u1), w2 = ptx::pack_f2(u2, u2);
 #pragma unroll
-        for (int j = 0; j < 64; ++j) acc[j] = ptx::mul_f2(ptx::mul_f2(acc[j], w1), w2);
+        for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(ptx::mul_f2(acc[j], w1), w2);
         if constexpr (ZERO != 0) {
           const uint64_t mul = ptx::pack_f2(__float_as_uint(prm.mul), __float_as_uint(prm.mul));
 #pragma unroll
-          for (int j = 0; j < 64; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
+          for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
         }
       }
       auto acc_at = [&](int j) {                      // columns 4 j .. 4 j + 3
@@ -510,45 +500,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // contraction slice of a tail tile: park the accumulators; the last warp to arrive sums the slices
         const int u = tile - tail_begin, t_idx = u / prm.tail_split;
         out_tile = tail_begin + t_idx;
-        float4 *mine = reinterpret_cast<float4 *>(prm.tail_ws) + ((size_t)u * QUARTERS + rank * 4 + quarter) * 1024;
+        float4 *mine = reinterpret_cast<float4 *>(prm.tail_ws) + ((size_t)u * WARPS + piece) * 512;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) mine[j * 32 + lane] = acc_at(j);
+        for (int j = 0; j < 16; ++j) mine[j * 32 + lane] = acc_at(j);
         __threadfence();
         __syncwarp();
         int prev = 0;
-        if (lane == 0) prev = atomicAdd(prm.tail_count + t_idx * QUARTERS + rank * 4 + quarter, 1);
+        if (lane == 0) prev = atomicAdd(prm.tail_count + t_idx * WARPS + piece, 1);
         prev = __shfl_sync(0xffffffffu, prev, 0);
         if (prev != prm.tail_split - 1) continue;
         __threadfence();
-        if (lane == 0) prm.tail_count[t_idx * QUARTERS + rank * 4 + quarter] = 0;
+        if (lane == 0) prm.tail_count[t_idx * WARPS + piece] = 0;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) acc[j] = 0ull;
+        for (int j = 0; j < 32; ++j) acc[j] = 0ull;
         for (int sl = 0; sl < prm.tail_split; ++sl) {
-          const float4 *part = reinterpret_cast<const float4 *>(prm.tail_ws) + ((size_t)(t_idx * prm.tail_split + sl) * QUARTERS + rank * 4 + quarter) * 1024;
+          const float4 *part = reinterpret_cast<const float4 *>(prm.tail_ws) + ((size_t)(t_idx * prm.tail_split + sl) * WARPS + piece) * 512;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
+          for (int j = 0; j < 16; ++j) {
             const float4 v = __ldcg(part + j * 32 + lane);
             acc[2 * j] = ptx::add_f2(acc[2 * j], ptx::pack_f2(__float_as_uint(v.x), __float_as_uint(v.y)));
             acc[2 * j + 1] = ptx::add_f2(acc[2 * j + 1], ptx::pack_f2(__float_as_uint(v.z), __float_as_uint(v.w)));
           }
         }
       }
-      // Epilogue.  Thread i of the warp holds row (lane_base + i), 128 columns.  The warp's piece goes through shared
-      // memory 32 columns at a time: thread i writes its 8 float4 groups with the group index XOR-ed by (i mod 8)
+      // Epilogue.  Thread i of the warp holds row (lane_base + i), 64 columns.  The warp's piece goes through shared
+      // memory 16 columns at a time: thread i writes its 4 float4 groups with the group index XOR-ed by (i / 2 mod 4)
       // (conflict-free 128-bit stores), then the warp reads the piece back transposed, so that the output is written,
-      // and the inputs of the epilogue are read, in a coalesced pattern: the warp walks over its rows four at a
-      // time, lanes 8g..8g+7 take row 4 step + g, 4 consecutive columns per lane.  The loads of four or eight steps
+      // and the inputs of the epilogue are read, in a coalesced pattern: the warp walks over its rows eight at a
+      // time, lanes 4g..4g+3 take row 8 step + g, 4 consecutive columns per lane.  The loads of the four steps
       // are issued together (rows past the end are clamped, their results dropped).
-      double ss = 0.0;
+      double ss_tile = 0.0;
       if constexpr (!epi_stores<Epi>::value) {
         // only the squared norm: straight from the registers (rows and columns outside the matrix hold exact zeros)
         uint64_t s2[2] = {0ull, 0ull};
 #pragma unroll
-        for (int j = 0; j < 64; ++j) s2[j & 1] = ptx::fma_f2(acc[j], acc[j], s2[j & 1]);
+        for (int j = 0; j < 32; ++j) s2[j & 1] = ptx::fma_f2(acc[j], acc[j], s2[j & 1]);
         float s4[4];
         ptx::unpack_f2(s2[0], s4[0], s4[1]);
         ptx::unpack_f2(s2[1], s4[2], s4[3]);
-        ss = ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]);
+        ss_tile = ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]);
       } else {
         float *C = epi.C + (size_t)z * prm.c_split_stride;
         float ssf = 0.f;
@@ -564,7 +554,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           __syncwarp();
           auto stash = [&](auto H) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) tr[lane * 8 + (j ^ (lane & 7))] = acc_at(decltype(H)::value * 8 + j);
+            for (int j = 0; j < 4; ++j) tr[lane * 4 + (j ^ ((lane >> 1) & 3))] = acc_at(decltype(H)::value * 4 + j);
           };
           switch (h) {
             case 0: stash(std::integral_constant<int, 0>{}); break;
@@ -573,22 +563,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             default: stash(std::integral_constant<int, 3>{}); break;
           }
           __syncwarp();
-          const int col = n0 + h * 32 + 4 * (lane & 7);
+          const int col = n0 + h * 16 + 4 * (lane & 3);
           if (col < n_pad) {
-            constexpr int BATCH = Epi::kInputs <= 1 ? 8 : 4;       // row steps whose loads are in flight together
-#pragma unroll
-            for (int s0 = 0; s0 < 8; s0 += BATCH) {
+            constexpr int BATCH = 4;                               // row steps whose loads are in flight together
+            {
               float4 in[BATCH][Epi::kInputs > 0 ? Epi::kInputs : 1];
 #pragma unroll
               for (int i = 0; i < BATCH; ++i) {
-                const int r = 4 * (s0 + i) + (lane >> 3);
+                const int r = 8 * i + (lane >> 2);
                 if constexpr (!Epi::kDirect) epi.load(min(m0 + lane_base + r, prm.M - 1), col, in[i]);
               }
 #pragma unroll
               for (int i = 0; i < BATCH; ++i) {
-                const int r = 4 * (s0 + i) + (lane >> 3);
+                const int r = 8 * i + (lane >> 2);
                 const int row = m0 + lane_base + r;
-                float4 o = tr[r * 8 + ((lane & 7) ^ (r & 7))];
+                float4 o = tr[r * 4 + ((lane & 3) ^ ((r >> 1) & 3))];
                 if constexpr (epi_sumsq_acc<Epi>::value) {
                   if (row < prm.M) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
                 }
@@ -610,15 +599,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
           }
         }
-        ss = (double)ssf;
+        ss_tile = (double)ssf;
         if constexpr (epi_amax<Epi>::value) {
           if (epi.amax != nullptr) commit_amax(mx, epi.amax);      // the output is an operand of a later product
         }
       }
-      if (partials != nullptr) {          // one slot per tile and row quarter; a single block adds the slots in index order
-        ss = warp_sum(ss);
-        if (lane == 0) partials[(size_t)out_tile * QUARTERS + rank * 4 + quarter] = ss;
+      if (tile < tail_begin) {
+        ss += ss_tile;
+      } else if (partials != nullptr) {
+        ss_tile = warp_sum(ss_tile);
+        if (lane == 0) partials[(size_t)gridDim.x * TC_ACC_WARPS + (size_t)(out_tile - tail_begin) * WARPS + piece] = ss_tile;
       }
+    }
+    if (partials != nullptr) {
+      ss = warp_sum(ss);
+      if (lane == 0) partials[(size_t)blockIdx.x * TC_ACC_WARPS + aw] = ss;
     }
   }
   ptx::tc_fence_before_sync();

@@ -252,6 +252,24 @@ static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
   return PDADMM_OK;
 }
 
+// Launches a kernel of an iteration with a priority above the products': its blocks go to the SMs as soon as one has room,
+// beside the products of other lanes, instead of behind them.  (The work distributor serves equal priorities in the order of
+// arrival, and a product's blocks fill the queue.)
+template <class... P, class... A>
+static void launch_first(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args) {
+  static const int top = [] { int lo = 0, hi = 0; cudaDeviceGetStreamPriorityRange(&lo, &hi); return hi; }();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute a[2];
+  a[0].id = cudaLaunchAttributePriority;
+  a[0].val.priority = top;
+  // the products' division of the SM's memory between L1 and shared memory: blocks with another one wait until the SM is empty
+  a[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  a[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  cfg.attrs = a; cfg.numAttrs = 2;
+  cudaLaunchKernelEx(&cfg, kern, P(args)...);            // errors surface at the call's end (cudaGetLastError)
+}
+
 static inline int ew_grid(size_t n_items) {
   return (int)std::max<size_t>(1, std::min<size_t>(ceil_div((int64_t)n_items, EW_THREADS), 148 * 8));
 }
@@ -404,7 +422,6 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Operand &A, const Ope
   const bool pair = use_pairs(c, prm.M, prm.N, prm.n_split);
   const int n_tiles = (int)(ceil_div(prm.M, pair ? 2 * TC_BM : TC_BM) * ceil_div(prm.N, TC_BN)) * prm.n_split;
   const int slots = pair ? c->n_sms / 2 : c->n_sms;          // tiles under way at a time
-  if (n_partials) *n_partials = (pair ? 8 : 4) * n_tiles;    // one slot per tile and row quarter
   // The persistent grid works through the tiles in rounds; a last round that fills only part of the
   // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit.
   int n_units = n_tiles;
@@ -419,6 +436,10 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Operand &A, const Ope
       prm.tail_ws = c->cur->tail_ws; prm.tail_count = c->cur->tail_count;
       n_units = prm.tail_begin + tail * split;
     }
+  }
+  if (n_partials) {
+    const int blocks = pair ? 2 * std::min(n_units, slots) : std::min(n_units, slots);
+    *n_partials = TC_ACC_WARPS * (blocks + (prm.tail_split > 1 ? (pair ? 2 : 1) * (n_tiles - prm.tail_begin) : 0));
   }
   if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, maps, prm, epi, partials, n_units);
   return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, maps, prm, epi, partials, n_units);
@@ -453,7 +474,7 @@ static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t ro
                        const Planes &pl, bool lo_too = true) {
   const size_t n8 = rows * ld / 8;
   Launch l(c, KC_PLANES, st, (lo_too ? 8.0 : 6.0) * rows * cols, 0);
-  rows_planes_kernel<<<ew_grid(n8), 256, 0, st>>>(x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
+  launch_first(st, rows_planes_kernel, dim3(ew_grid(n8)), 256, 0, x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
 }
 // Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel).
 // From 2^20 elements on: below, the launch costs more than it saves.
@@ -462,7 +483,7 @@ static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, Operand &o
   const size_t n = rows * o.ld;
   if (!c->use_tc || o.hi == nullptr || o.check == nullptr || o.x == nullptr || n < CHECK_PLANES_FROM) return;
   Launch l(c, KC_PLANES, st, 0, 0);
-  check_planes_kernel<<<ew_grid(n / 8), 256, 0, st>>>(o.x, n / 8, o.check, o.exp, const_cast<__half *>(o.hi),
+  launch_first(st, check_planes_kernel, dim3(ew_grid(n / 8)), 256, 0, o.x, n / 8, o.check, o.exp, const_cast<__half *>(o.hi),
                                                      o.lo == o.hi ? nullptr : const_cast<__half *>(o.lo));
   o.x = nullptr;
 }
@@ -607,11 +628,11 @@ static int p_gradient_and_tau(pdadmm_ctx *c, int l /*0-based, >= 1*/) {
   if (c->reduce != nullptr) {
     // ||g||^2 and ||W g||^2 are sums over nodes: this shard's totals, added over the shards, then tau
     PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, np, slots_b, np2));
-    finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.red, 1, s.red + 1, 1, c->d_flag + 2, t);
+    launch_first(s.st, finalize_tau_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, s.red, 1, s.red + 1, 1, c->d_flag + 2, t);
     return PDADMM_OK;
   }
   Launch k(c, KC_SMALL, s.st, 8.0 * (np + np2), 0);
-  finalize_tau_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, s.slots, np, slots_b, np2, c->d_flag + 2, t);
+  launch_first(s.st, finalize_tau_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, s.slots, np, slots_b, np2, c->d_flag + 2, t);
   return PDADMM_OK;
 }
 
@@ -625,7 +646,7 @@ static void p_step_plain(pdadmm_ctx *c, int l) {
   Scratch &s = *c->cur;
   const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
   Launch k(c, KC_AXPY, s.st, (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out), 0);
-  pstep_kernel<<<ew_grid(std::max(n4p, n4r)), EW_THREADS, 0, s.st>>>(
+  launch_first(s.st, pstep_kernel, dim3(ew_grid(std::max(n4p, n4r))), EW_THREADS, 0, 
       ly.p, s.s1, n4p, ly.r, s.s2, n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0), c->use_tc ? ly.amax_p : nullptr,
       c->use_tc ? ly.amax_r : nullptr);
 }
@@ -647,7 +668,7 @@ static int q_trial(pdadmm_ctx *c, int l) {
     // reads g and the codes of p; writes p+, the new codes and d -- as fp32, or, with integer operands, as the two
     // fp16 planes of integers: 14 bytes per element with one-byte codes either way
     Launch k(c, KC_QUANT, s.st, 14.0 * N * ly.n_in, 0);
-    quant_trial_kernel<<<grid, EW_THREADS, 0, s.st>>>(s.s1, ly.sc, ly.scale, ly.lo, c->levels, s.p_new,
+    launch_first(s.st, quant_trial_kernel, dim3(grid), EW_THREADS, 0, s.s1, ly.sc, ly.scale, ly.lo, c->levels, s.p_new,
                                                      c->int_operands ? nullptr : s.d,
                                                      s.codes_new, c->code_bytes == 2, n4p, s.slots,
                                                      c->use_tc ? ly.amax_p : nullptr, w_d,
@@ -665,10 +686,10 @@ static int q_trial(pdadmm_ctx *c, int l) {
                            (c->use_tc ? 8.0 : 4.0) * N * ly.n_out));
   if (c->reduce != nullptr) {
     PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, grid, slots_b, np));
-    finalize_trial_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.red, 1, s.red + 1, 1);
+    launch_first(s.st, finalize_trial_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.red, 1, s.red + 1, 1);
   } else {
     Launch k(c, KC_SMALL, s.st, 8.0 * (grid + np), 0);
-    finalize_trial_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.slots, grid, slots_b, np);
+    launch_first(s.st, finalize_trial_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.slots, grid, slots_b, np);
   }
   PD_CUDA(cudaMemcpyAsync(s.h_flag, &ly.sc->accepted, sizeof(int), cudaMemcpyDeviceToHost, s.st));
   PD_CUDA(cudaEventRecord(s.ev_flag, s.st));
@@ -730,14 +751,14 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
   {
     Launch k(c, KC_GRADW_REDUCE, s.st, (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in, 0);
     // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
-    reduce_gradW_kernel<<<gw, EW_THREADS, 0, s.st>>>(s.part, ly.n_split, n4w, c->nu, ly.gradW, w_G, s.slots,
+    launch_first(s.st, reduce_gradW_kernel, dim3(gw), EW_THREADS, 0, s.part, ly.n_split, n4w, c->nu, ly.gradW, w_G, s.slots,
                                                      c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp));
   }
   if (c->reduce != nullptr) {
     // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
     PD_TRY(shard_sum(c, s.st, ly.gradW, n4w * 4, 0));
     if (c->use_tc) w_G = amax_take(c);
-    sumsq_amax_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.gradW, n4w, w_G, s.slots);
+    launch_first(s.st, sumsq_amax_kernel, dim3(gw), EW_THREADS, 0, ly.gradW, n4w, w_G, s.slots);
     if (c->use_tc) split_rows(c, s.st, ly.gradW, (size_t)ly.n_out, ly.n_in, ly.ld_in, w_G, ly.Gp);
   }
   int np = 0;
@@ -751,14 +772,14 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
   if (c->reduce != nullptr) {
     // ||G p+||^2 is a sum over nodes (||G||^2 is the same on every shard already)
     PD_TRY(shard_sum_slots(c, s.st, s.red, slots_b, np, nullptr, 0));
-    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, s.red, 1, c->d_flag + 2, tp);
+    launch_first(s.st, finalize_theta_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->nu, s.slots, gw, s.red, 1, c->d_flag + 2, tp);
   } else {
     Launch k(c, KC_SMALL, s.st, 8.0 * (gw + np), 0);
-    finalize_theta_kernel<<<1, FIN_THREADS, 0, s.st>>>(ly.sc, (double)c->nu, s.slots, gw, slots_b, np, c->d_flag + 2, tp);
+    launch_first(s.st, finalize_theta_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->nu, s.slots, gw, slots_b, np, c->d_flag + 2, tp);
   }
   {
     Launch k(c, KC_WSTEP, s.st, (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in, 0);
-    wstep_kernel<<<gw, EW_THREADS, 0, s.st>>>(ly.W, ly.gradW, ly.sc, n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp));
+    launch_first(s.st, wstep_kernel, dim3(gw), EW_THREADS, 0, ly.W, ly.gradW, ly.sc, n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp));
   }
   const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 16));
   const int rows_per_block = (int)ceil_div(N, n_blocks);
@@ -768,17 +789,17 @@ static int w_and_b_step(pdadmm_ctx *c, int l) {
     const int n_sub = std::min(EW_THREADS / cols_per_pass, COLSUM_MAX_SUB);
     const size_t sh = n_sub > 1 ? (size_t)n_sub * ly.ld_out * sizeof(double) : 0;
     Launch k(c, KC_COLSUM, s.st, 12.0 * N * ly.n_out, 0);
-    resid_colsum_kernel<<<used_blocks, EW_THREADS, sh, s.st>>>(ly.r, s.s1, ly.sc, N, ly.ld_out, rows_per_block, s.slots);
+    launch_first(s.st, resid_colsum_kernel, dim3(used_blocks), EW_THREADS, sh, ly.r, s.s1, ly.sc, N, ly.ld_out, rows_per_block, s.slots);
   }
   if (c->reduce != nullptr) {
     // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
-    colsum_total_kernel<<<(int)ceil_div(ly.ld_out, 32), dim3(32, BIAS_GROUPS), 0, s.st>>>(s.slots, used_blocks, ly.ld_out, s.red);
+    launch_first(s.st, colsum_total_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.slots, used_blocks, ly.ld_out, s.red);
     PD_TRY(shard_sum(c, s.st, s.red, (size_t)ly.ld_out, 1));
-    finalize_bias_kernel<<<(int)ceil_div(ly.ld_out, 32), dim3(32, BIAS_GROUPS), 0, s.st>>>(s.red, 1, ly.ld_out, ly.n_out,
+    launch_first(s.st, finalize_bias_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.red, 1, ly.ld_out, ly.n_out,
                                                                                 1.0 / (double)c->N_total, ly.b, ly.shift);
   } else {
     Launch k(c, KC_SMALL, s.st, 8.0 * used_blocks * ly.ld_out, 0);
-    finalize_bias_kernel<<<(int)ceil_div(ly.ld_out, 32), dim3(32, BIAS_GROUPS), 0, s.st>>>(s.slots, used_blocks, ly.ld_out, ly.n_out,
+    launch_first(s.st, finalize_bias_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.slots, used_blocks, ly.ld_out, ly.n_out,
                                                                                 1.0 / (double)N, ly.b, ly.shift);
   }
   return PDADMM_OK;
@@ -795,16 +816,16 @@ static void zqu_step(pdadmm_ctx *c, int l) {
     if (c->table_size > 0) {
       Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);
       const Layer &nx = c->layers[l + 1];
-      zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), s.st>>>(
+      launch_first(s.st, zqu_table_kernel, dim3(grid), EW_THREADS, c->table_size * sizeof(float), 
           ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu, c->slope, c->table_lo, c->table_step,
-          c->table_size, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t, s.slots, ly.amax_r,
+          c->table_size, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t, ly.amax_r,
           plane_out(c, ly.rp), c->levels ? nx.codes : nullptr, c->code_bytes == 2);
     } else {
       Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);      // p_{l+1} as one-byte codes
       const Layer &nx = c->layers[l + 1];
-      zqu_kernel<<<grid, EW_THREADS, 0, s.st>>>(ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu,
+      launch_first(s.st, zqu_kernel, dim3(grid), EW_THREADS, 0, ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu,
                                                c->slope, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t,
-                                               s.slots, ly.amax_r, plane_out(c, ly.rp), c->levels ? nx.codes : nullptr,
+                                               ly.amax_r, plane_out(c, ly.rp), c->levels ? nx.codes : nullptr,
                                                c->code_bytes == 2);
     }
   } else {
