@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "planes.cuh"
+#include "scalars.cuh"
 
 namespace pd {
 
@@ -27,21 +28,23 @@ absmax_kernel(const float *__restrict__ x, size_t n4, uint32_t *__restrict__ wor
   commit_amax(m, word);
 }
 
-// Scalars of one layer that live on the device (so that an iteration needs no host round trip).
-struct LayerScalars {
-  double sum_g2;      // ||g||^2
-  double sum_wg2;     // ||W g||^2
-  double sum_d2;      // ||p+ - p||^2        (quantised trial)
-  double sum_wd2;     // ||W (p+ - p)||^2    (quantised trial)
-  double sum_G2;      // ||grad_W||^2
-  double sum_Gp2;     // ||grad_W p+||^2
-  double tau;         // tau_l
-  double theta;       // theta_l (0 if grad_W = 0)
-  float inv_tau;      // 1/tau
-  float inv_theta;    // 1/theta, 0 if grad_W = 0
-  int accepted;       // quantised trial: 1 if the stop condition held
-  int trials;         // trials so far in this iteration
-};
+// Kernels of an iteration work on several layers at a time: blocks (x, y) = part x of layer y of the group.  What a layer's
+// blocks do, and the order of its sums, depends on the layer alone.
+constexpr int MAX_GROUP = 16;
+template <class T> struct Group { T l[MAX_GROUP]; };
+// The last block of a layer to arrive (`done`: zero before and after the kernel) has every slot that the others wrote.
+__device__ __forceinline__ bool last_block(int *done, int n_blocks, int *sh) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *sh = atomicAdd(done, 1) == n_blocks - 1;
+    if (*sh) *done = 0;
+  }
+  __syncthreads();
+  if (!*sh) return false;
+  __threadfence();
+  return true;
+}
 
 __device__ __forceinline__ float4 ld4(const float *p, size_t i) { return reinterpret_cast<const float4 *>(p)[i]; }
 __device__ __forceinline__ float4 ld4f(const float *p, size_t i) { return reinterpret_cast<const float4 *>(p)[i]; }
@@ -107,57 +110,82 @@ __device__ __forceinline__ void store_planes4(const PlaneOut &o, size_t i, float
 // elements of p first, then those of r), with the planes of both for the W-gradient and G p+.  16 bytes per element and
 // matrix: read 8, write 4 and the planes 4.  (Separate passes that split r and p again cost 8 bytes more each, and the
 // products that took them fp32 ran at 0.6 of their speed.)
+struct PStep {
+  float *p; const float *g; uint32_t n4p;
+  float *r; const float *wg; uint32_t n4r;
+  const float *inv_tau;
+  PlaneOut pp, rp;
+  uint32_t *amax_p, *amax_r;          // receive max|p|, max|r| (see commit_amax); may be null
+  int n_blocks;
+};
 __global__ void __launch_bounds__(EW_THREADS, 5)
-pstep_kernel(float *__restrict__ p, const float *__restrict__ g, size_t n4p, float *__restrict__ r, const float *__restrict__ wg,
-             size_t n4r, const float *__restrict__ inv, PlaneOut pp, PlaneOut rp,
-             uint32_t *__restrict__ amax_p /* receives max|p| (see commit_amax); may be null */, uint32_t *__restrict__ amax_r) {
-  const float a = *inv;
-  const size_t stride = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  auto pass = [&](float *__restrict__ y, const float *__restrict__ x, size_t n4, const PlaneOut &o, uint32_t *amax) {
+pstep_kernel(const __grid_constant__ Group<PStep> group) {
+  const PStep &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.n_blocks) return;
+  const float a = *y.inv_tau;
+  const uint32_t stride = y.n_blocks * EW_THREADS, first = blockIdx.x * EW_THREADS + threadIdx.x;
+  auto pass = [&](float *__restrict__ out, const float *__restrict__ x, uint32_t n4, const PlaneOut &o, uint32_t *amax) {
     const float scale = o.hi != nullptr ? tc_scale_of(*o.exp) : 1.f;
     uint32_t m = 0u;
-    // two groups per pass: four loads in flight per thread (four groups take more registers than two blocks have beside a product)
-    for (size_t i = first; i < n4; i += 2 * stride) {
+    // two groups per pass: four loads in flight per thread (four groups take more registers than two blocks have beside a
+    // product)
+    for (uint32_t i = first; i < n4; i += 2 * stride) {
       float4 v[2], w[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const size_t q = i + k * stride;
-        if (q < n4) { v[k] = ld4(y, q); w[k] = ld4(x, q); }
+        const uint32_t q = i + k * stride;
+        if (q < n4) { v[k] = ld4(out, q); w[k] = ld4(x, q); }
       }
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const size_t q = i + k * stride;
+        const uint32_t q = i + k * stride;
         if (q >= n4) continue;
         v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
         v[k].z = fmaf(-a, w[k].z, v[k].z); v[k].w = fmaf(-a, w[k].w, v[k].w);
-        st4(y, q, v[k]);
+        st4(out, q, v[k]);
         if (o.hi != nullptr) store_planes4(o, q, v[k], scale);
         m = max(m, abs_bits(v[k]));
       }
     }
     if (amax != nullptr) commit_amax(m, amax);
   };
-  pass(p, g, n4p, pp, amax_p);
-  pass(r, wg, n4r, rp, amax_r);
+  pass(y.p, y.g, y.n4p, y.pp, y.amax_p);
+  pass(y.r, y.wg, y.n4r, y.rp, y.amax_r);
 }
 
 // ---- quantised trial step ------------------------------------------------------------------------
 // x = p - g/tau; p_new = nearest level; d = p_new - p; codes; per-block sum of d^2.
 // p lies on the level set, p = lo + code * scale bit for bit (quantize_one), so it is read as its 1- or 2-byte codes
 // instead of as 4-byte values.
+struct QuantTrial {
+  const float *g; LayerScalars *sc; float scale, lo;
+  float *p_new, *d /* may be null */;
+  const void *codes_old; void *codes;      // of p; of p_new
+  __half *pn_plane;                        // the new codes, counted from the level zero, as fp16 integers: operand plane of
+                                           // p_new = (code - neg_levels) * scale; may be null
+  __half *d_plane;                         // new code - old code as fp16 integers (operand plane of d)
+  uint32_t n4;
+  uint32_t *amax_p /* max|p_new|, may be null */, *amax_d /* max|d| */;
+  double *slots; int *done; int n_blocks;
+};
 __global__ void __launch_bounds__(EW_THREADS)
-quant_trial_kernel(const float *__restrict__ g, const LayerScalars *__restrict__ sc,
-                   float scale, float lo, int levels, float *__restrict__ p_new, float *__restrict__ d /* may be null */,
-                   void *__restrict__ codes, int wide_codes, size_t n4, double *__restrict__ slots,
-                   uint32_t *__restrict__ amax_p /* max|p_new|, may be null */, uint32_t *__restrict__ amax_d /* max|d| */,
-                   const void *__restrict__ codes_old /* codes of p */,
-                   __half *__restrict__ pn_plane /* the new codes as fp16 integers (operand plane of p_new = code * scale) */,
-                   __half *__restrict__ d_plane /* new code - old code as fp16 integers (operand plane of d) */) {
+quant_trial_kernel(const __grid_constant__ Group<QuantTrial> group, int levels, int wide_codes, int neg_levels) {
   __shared__ double red[EW_THREADS / 32];
-  const float inv_tau = sc->inv_tau, top = (float)(levels - 1);
+  __shared__ int is_last;
+  const QuantTrial &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.n_blocks) return;
+  const float *__restrict__ g = y.g;
+  const void *__restrict__ codes_old = y.codes_old;
+  void *__restrict__ codes = y.codes;
+  float *__restrict__ p_new = y.p_new, *__restrict__ d = y.d;
+  __half *__restrict__ pn_plane = y.pn_plane, *__restrict__ d_plane = y.d_plane;
+  const float scale = y.scale, lo = y.lo;
+  const uint32_t n4 = y.n4;
+  uint32_t *amax_p = y.amax_p, *amax_d = y.amax_d;
+  const float inv_tau = y.sc->inv_tau, top = (float)(levels - 1);
   double ss = 0.0;
   uint32_t mp = 0u, md = 0u;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < n4; i += y.n_blocks * EW_THREADS) {
     const float4 gv = ld4(g, i);
     int o0, o1, o2, o3;
     if (wide_codes) {
@@ -177,7 +205,7 @@ quant_trial_kernel(const float *__restrict__ g, const LayerScalars *__restrict__
     nv.w = quantize_one(fmaf(-inv_tau, gv.w, pv.w), scale, lo, top, c3);
     dv.x = nv.x - pv.x; dv.y = nv.y - pv.y; dv.z = nv.z - pv.z; dv.w = nv.w - pv.w;
     ss += (double)dv.x * dv.x + (double)dv.y * dv.y + (double)dv.z * dv.z + (double)dv.w * dv.w;
-    st4(p_new, i, nv);
+    if (p_new != nullptr) st4(p_new, i, nv);      // with integer planes p+ exists as its codes alone
     if (d != nullptr) st4(d, i, dv);     // with the integer planes below the product W d reads d_plane instead
     mp = max(mp, abs_bits(nv)); md = max(md, abs_bits(dv));
     if (wide_codes)      // more than 256 levels: 16-bit codes
@@ -185,8 +213,9 @@ quant_trial_kernel(const float *__restrict__ g, const LayerScalars *__restrict__
     else
       reinterpret_cast<uchar4 *>(codes)[i] = make_uchar4((unsigned char)c0, (unsigned char)c1, (unsigned char)c2, (unsigned char)c3);
     if (pn_plane != nullptr) {
-      // integers below 2048 are exact in fp16: the planes hold the codes themselves and their change
-      const __half2 a = __floats2half2_rn((float)c0, (float)c1), b = __floats2half2_rn((float)c2, (float)c3);
+      // integers up to 2048 are exact in fp16: the planes hold the codes (counted from the level zero) and their change
+      const __half2 a = __floats2half2_rn((float)((int)c0 - neg_levels), (float)((int)c1 - neg_levels));
+      const __half2 b = __floats2half2_rn((float)((int)c2 - neg_levels), (float)((int)c3 - neg_levels));
       const __half2 e = __floats2half2_rn((float)((int)c0 - o0), (float)((int)c1 - o1));
       const __half2 f = __floats2half2_rn((float)((int)c2 - o2), (float)((int)c3 - o3));
       reinterpret_cast<uint2 *>(pn_plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
@@ -195,7 +224,12 @@ quant_trial_kernel(const float *__restrict__ g, const LayerScalars *__restrict__
   }
   if (amax_p != nullptr) { commit_amax(mp, amax_p); commit_amax(md, amax_d); }
   const double tot = block_sum<EW_THREADS>(ss, red);
-  if (threadIdx.x == 0) slots[blockIdx.x] = tot;
+  if (threadIdx.x == 0) y.slots[blockIdx.x] = tot;
+  if (!last_block(y.done, y.n_blocks, &is_last)) return;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < y.n_blocks; i += EW_THREADS) v += __ldcg(y.slots + i);
+  v = block_sum<EW_THREADS>(v, red);
+  if (threadIdx.x == 0) y.sc->sum_d2 = v;
 }
 
 // Plain projection of an array (initial forward pass, pdadmm_quantize, pdadmm_set_tensor).
@@ -215,9 +249,10 @@ quantize_kernel(const float *x, size_t n, float scale, float lo, int levels, flo
 }
 
 // ---- operand planes of a quantised p from its codes ------------------------------------------------------------
-// p = code * s with code < 2048: the fp16 plane of the integer codes is the whole operand (the products multiply by s).
+// p = (code - neg_levels) s with at most 2048 levels: the fp16 plane of the integers is the whole operand (the products
+// multiply by s).
 __global__ void __launch_bounds__(EW_THREADS)
-codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, size_t n4, __half *__restrict__ plane) {
+codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, int neg_levels, size_t n4, __half *__restrict__ plane) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float c0, c1, c2, c3;
     if (wide_codes) {
@@ -227,110 +262,32 @@ codes_to_plane_kernel(const void *__restrict__ codes, int wide_codes, size_t n4,
       const uchar4 o = reinterpret_cast<const uchar4 *>(codes)[i];
       c0 = o.x; c1 = o.y; c2 = o.z; c3 = o.w;
     }
-    const __half2 a = __floats2half2_rn(c0, c1), b = __floats2half2_rn(c2, c3);
+    const float j = (float)neg_levels;
+    const __half2 a = __floats2half2_rn(c0 - j, c1 - j), b = __floats2half2_rn(c2 - j, c3 - j);
     reinterpret_cast<uint2 *>(plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
   }
 }
-// ---- finalisers of the step parameters (one block of FIN_THREADS threads) ---------------------------------
-// Fixed-order sum of n slots by one block of FIN_THREADS threads: thread t adds slots t, t + FIN_THREADS, ..., then a
-// fixed tree.  Result in thread 0.
-// 256 threads fit beside a product; there are a few thousand slots at most.
+// p itself from its codes, for whoever wants the values (pdadmm_get_tensor, a residual from scratch).
+__global__ void __launch_bounds__(EW_THREADS)
+codes_to_levels_kernel(const void *__restrict__ codes, int wide_codes, size_t n4, float s, float lo, float *__restrict__ p) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
+    st4(p, i, levels_of4(codes, wide_codes, i, s, lo));
+}
+
+// ---- sums that no product completed ---------------------------------------------------------------------------
+// The CUDA-core products leave one slot per block: fixed-order sum by one block (thread t adds slots t, t + FIN_THREADS, ...),
+// then the step.
 constexpr int FIN_THREADS = 256;
-__device__ __forceinline__ double block_sum_slots(const double *__restrict__ slots, int n, double *sh /* FIN_THREADS */) {
-  // four independent partial sums per thread keep four loads in flight; the order of the additions is fixed
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  int i = threadIdx.x;
-  for (; i + 3 * FIN_THREADS < n; i += 4 * FIN_THREADS) {
-    s0 += slots[i]; s1 += slots[i + FIN_THREADS]; s2 += slots[i + 2 * FIN_THREADS]; s3 += slots[i + 3 * FIN_THREADS];
-  }
-  for (; i < n; i += FIN_THREADS) s0 += slots[i];
-  const double s = (s0 + s1) + (s2 + s3);
-  __syncthreads();
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = FIN_THREADS / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  return sh[0];
-}
-// ||g||^2 and ||W g||^2 from their slots, then
-// tau = rho + nu ||W g||^2 / ||g||^2 : the smallest tau with phi(p - g/tau) <= U_l(p - g/tau; tau).
-// Thread 0 also settles the exponents of planes that later kernels write (null words are skipped).  With w_wg, the
-// p-step of pdADMM-G follows: |p+| <= max|p| + max|g|/tau and |r+| <= max|r| + max|W g|/tau are bounds.  Without, r after the
-// trial is predicted from r before it.  g of the next iteration is predicted from this one's.
-struct TauPlanes { uint32_t *amax_p; const uint32_t *amax_r, *w_g, *w_wg; int *p_exp, *r_exp, *g_exp; };
-__device__ __forceinline__ int tc_bound_exp(uint32_t a, uint32_t b, float factor) {       // of a + b * factor, a little up
-  return tc_scale_exp(__float_as_uint((__uint_as_float(a) + __uint_as_float(b) * factor) * 1.0001f));
-}
 __global__ void __launch_bounds__(FIN_THREADS)
-finalize_tau_kernel(LayerScalars *sc, double rho, double nu, const double *slots_g, int n_g, const double *slots_wg, int n_wg,
-                    int *nonfinite, TauPlanes t) {
-  __shared__ double sh[FIN_THREADS];
-  const double gg = block_sum_slots(slots_g, n_g, sh);
-  const double wg = block_sum_slots(slots_wg, n_wg, sh);
-  if (threadIdx.x == 0) {
-    sc->sum_g2 = gg;
-    sc->sum_wg2 = wg;
-    if (!(isfinite(gg) && isfinite(wg))) *nonfinite = 1;      // a NaN or Inf anywhere in the state reaches these sums
-    const double tau = gg > 0.0 ? rho + nu * wg / gg : rho;
-    const float inv_tau = (float)(1.0 / tau);
-    sc->tau = tau;
-    sc->inv_tau = inv_tau;
-    sc->accepted = 0;
-    sc->trials = 0;
-    if (t.p_exp != nullptr) *t.p_exp = tc_bound_exp(*t.amax_p, *t.w_g, inv_tau);
-    if (t.r_exp != nullptr) *t.r_exp = t.w_wg != nullptr ? tc_bound_exp(*t.amax_r, *t.w_wg, inv_tau) : tc_predict_exp(*t.amax_r);
-    if (t.g_exp != nullptr) *t.g_exp = tc_predict_exp(*t.w_g);
-    if (t.amax_p != nullptr) *t.amax_p = 0u;                  // max|p| of the layer restarts with the coming p-step
-  }
+finish_sum_kernel(const double *__restrict__ slots, int n, Step step) {
+  __shared__ double red[FIN_THREADS / 32];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += FIN_THREADS) v += slots[i];
+  v = block_sum<FIN_THREADS>(v, red);
+  if (threadIdx.x == 0) finish_step(step, v);
 }
-// Stop condition of the quantised step in its quadratic form: nu||W d||^2 + rho||d||^2 <= tau||d||^2 (1 + slack).
-// Not accepted: tau is doubled for the next trial.
-__global__ void __launch_bounds__(FIN_THREADS)
-finalize_trial_kernel(LayerScalars *sc, double rho, double nu, double slack, const double *slots_d, int n_d,
-                      const double *slots_wd, int n_wd) {
-  __shared__ double sh[FIN_THREADS];
-  const double dd = block_sum_slots(slots_d, n_d, sh);
-  const double wd = block_sum_slots(slots_wd, n_wd, sh);
-  if (threadIdx.x == 0) {
-    sc->sum_d2 = dd;
-    sc->sum_wd2 = wd;
-    const bool ok = nu * wd + rho * dd <= sc->tau * dd * (1.0 + slack);
-    sc->trials += 1;
-    sc->accepted = ok ? 1 : 0;
-    if (!ok) {
-      sc->tau *= 2.0;
-      sc->inv_tau = (float)(1.0 / sc->tau);
-    }
-  }
-}
-// ||grad_W||^2 and ||grad_W p+||^2 from their slots, then
-// theta = nu ||grad_W p+||^2 / ||grad_W||^2 : the smallest theta with phi(W+) <= V_l(W+; theta).
-// Exponents of planes as in finalize_tau_kernel: W+ is bounded by max|W| + max|G|/theta; the coming z-step's r and the next
-// iteration's G are predicted from this iteration's.
-struct ThetaPlanes { uint32_t *amax_r, *amax_W; const uint32_t *w_G; int *W_exp, *r_exp, *G_exp; };
-__global__ void __launch_bounds__(FIN_THREADS)
-finalize_theta_kernel(LayerScalars *sc, double nu, const double *slots_G, int n_G, const double *slots_Gp, int n_Gp,
-                      int *nonfinite, ThetaPlanes t) {
-  __shared__ double sh[FIN_THREADS];
-  const double GG = block_sum_slots(slots_G, n_G, sh);
-  const double Gp = block_sum_slots(slots_Gp, n_Gp, sh);
-  if (threadIdx.x == 0) {
-    sc->sum_G2 = GG;
-    sc->sum_Gp2 = Gp;
-    if (!(isfinite(GG) && isfinite(Gp))) *nonfinite = 1;
-    const double theta = GG > 0.0 ? nu * Gp / GG : 0.0;
-    const float inv_theta = theta > 0.0 ? (float)(1.0 / theta) : 0.0f;
-    sc->theta = theta;
-    sc->inv_theta = inv_theta;
-    if (t.W_exp != nullptr) *t.W_exp = tc_bound_exp(*t.amax_W, *t.w_G, inv_theta);
-    if (t.r_exp != nullptr) *t.r_exp = tc_predict_exp(*t.amax_r);
-    if (t.G_exp != nullptr) *t.G_exp = tc_predict_exp(*t.w_G);
-    if (t.amax_r != nullptr) *t.amax_r = 0u;                  // max|r| restarts with the coming z-step, max|W| with the W-step
-    if (t.amax_W != nullptr) *t.amax_W = 0u;
-  }
-}
+// A context that owns part of the nodes: the step after its sums were added over the shards.
+__global__ void run_step_kernel(Step step) { run_step(step); }
 
 // ---- planes of a stored matrix -----------------------------------------------------------------------
 // x [rows][ld] fp32 -> hi, lo [rows][ld] halves (the padding columns, zero in x, come out as zero), scaled by the exponent of
@@ -354,69 +311,112 @@ rows_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__res
 // nothing to do; if the scaling turned out unusable they are made again, with the exponent of *amax (which is what the product
 // assumes then; *exp stays as it is).  (Inside the product, per output tile, it would take 5 to 10 times the product: a
 // few such iterations at the start of a context of 20 000 x 500 cost more than all these launches.)
+struct PlaneCheck { const float *x; uint32_t n8; const uint32_t *amax; const int *exp; __half *hi, *lo /* may be null */; };
 __global__ void __launch_bounds__(256)
-check_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__restrict__ amax, const int *__restrict__ exp,
-                    __half *__restrict__ hi, __half *__restrict__ lo /* may be null */) {
-  if (tc_planes_usable(*amax, *exp)) return;
-  const float scale = tc_pow2(tc_scale_exp(*amax));
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
+check_planes_kernel(const __grid_constant__ Group<PlaneCheck> group) {
+  const PlaneCheck &y = group.l[blockIdx.y];
+  if (tc_planes_usable(*y.amax, *y.exp)) return;
+  const float scale = tc_pow2(tc_scale_exp(*y.amax));
+  for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < y.n8; i += gridDim.x * 256u) {
     uint4 h, l;
-    tc_split8(reinterpret_cast<const float4 *>(x)[2 * i], reinterpret_cast<const float4 *>(x)[2 * i + 1], scale, h, l);
-    reinterpret_cast<uint4 *>(hi)[i] = h;
-    if (lo != nullptr) reinterpret_cast<uint4 *>(lo)[i] = l;
+    tc_split8(reinterpret_cast<const float4 *>(y.x)[2 * (size_t)i], reinterpret_cast<const float4 *>(y.x)[2 * (size_t)i + 1], scale, h, l);
+    reinterpret_cast<uint4 *>(y.hi)[i] = h;
+    if (y.lo != nullptr) reinterpret_cast<uint4 *>(y.lo)[i] = l;
   }
 }
 
 // ---- reduction of the split partial tiles of grad_W, scaling by nu, ||grad_W||^2 ------------------
+struct GradWSum {
+  const float *part; int n_split; uint32_t n4;
+  float *G;
+  uint32_t *amax /* max|G|, may be null */; PlaneOut planes;
+  double *slots; int *done; double *sum /* ||G||^2 */; int n_blocks;
+};
 __global__ void __launch_bounds__(EW_THREADS)
-reduce_gradW_kernel(const float *__restrict__ part, int n_split, size_t n4, float nu, float *__restrict__ G,
-                    uint32_t *__restrict__ amax, double *__restrict__ slots, PlaneOut planes) {
+reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
   __shared__ double red[EW_THREADS / 32];
-  const float scale = planes.hi != nullptr ? tc_scale_of(*planes.exp) : 1.f;
+  __shared__ int is_last;
+  const GradWSum &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.n_blocks) return;
+  const float scale = y.planes.hi != nullptr ? tc_scale_of(*y.planes.exp) : 1.f;
+  const float *__restrict__ part = y.part;
+  const int n_split = y.n_split;
   double ss = 0.0;
   uint32_t m = 0u;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4; i += y.n_blocks * EW_THREADS) {
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
     for (int s = 0; s < n_split; ++s) {
-      const float4 v = ld4(part + (size_t)s * n4 * 4, i);
+      const float4 v = ld4(part + (size_t)s * y.n4 * 4, i);
       a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
     }
     a.x *= nu; a.y *= nu; a.z *= nu; a.w *= nu;
     ss += (double)a.x * a.x + (double)a.y * a.y + (double)a.z * a.z + (double)a.w * a.w;
-    st4(G, i, a);
-    if (planes.hi != nullptr) store_planes4(planes, i, a, scale);
+    st4(y.G, i, a);
+    if (y.planes.hi != nullptr) store_planes4(y.planes, i, a, scale);
     m = max(m, abs_bits(a));
   }
-  if (amax != nullptr) commit_amax(m, amax);        // the product G p+ checks the planes' scaling with it
+  if (y.amax != nullptr) commit_amax(m, y.amax);        // the product G p+ checks the planes' scaling with it
   const double tot = block_sum<EW_THREADS>(ss, red);
-  if (threadIdx.x == 0) slots[blockIdx.x] = tot;
+  if (threadIdx.x == 0) y.slots[blockIdx.x] = tot;
+  if (!last_block(y.done, y.n_blocks, &is_last)) return;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < y.n_blocks; i += EW_THREADS) v += __ldcg(y.slots + i);
+  v = block_sum<EW_THREADS>(v, red);
+  if (threadIdx.x == 0) *y.sum = v;
 }
 
-// ---- column sums of r - gp * inv_theta  (for the b-update) ----------------------------------------
-// Block b handles rows [b*rows_per_block, ...).  A thread owns one group of 4 columns (float4) and one row
+// ---- what follows theta: W+ and r - (G p+)/theta with its column sums (for the b-update) ----------------------------------
+// W+ = W - G/theta  (Eq. "update W"), with the planes of W+: the first n_blocks_w blocks of a layer.
+// The other blocks: block b handles rows [b*rows_per_block, ...).  A thread owns one group of 4 columns (float4) and one row
 // subgroup: with ld/4 <= 128 column groups the block's 256 threads cover several rows per pass.  The row
 // subgroups' sums are combined in subgroup order, then written to slots[b][ld].
 constexpr int COLSUM_MAX_SUB = 8;
+struct ThetaStep {
+  float *W; const float *G; uint32_t n4w;
+  uint32_t *amax_W /* may be null */; PlaneOut Wp;
+  float *r; const float *gp; int n_rows, ld, rows_per_block;
+  double *slots;
+  const LayerScalars *sc;
+  int n_blocks_w, n_blocks_r;
+};
 __global__ void __launch_bounds__(EW_THREADS)
-resid_colsum_kernel(float *__restrict__ r, const float *__restrict__ gp, const LayerScalars *__restrict__ sc,
-                    int n_rows, int ld, int rows_per_block, double *__restrict__ slots) {
+theta_step_kernel(const __grid_constant__ Group<ThetaStep> group) {
   extern __shared__ double colsum_sh[];                       // [n_sub][ld] when n_sub > 1
-  const float a = sc->inv_theta;
-  const int ld4 = ld >> 2;
-  const int cols_per_pass = min(ld4, EW_THREADS);
+  const ThetaStep &y = group.l[blockIdx.y];
+  const float a = y.sc->inv_theta;
+  if ((int)blockIdx.x < y.n_blocks_w) {
+    const float scale = y.Wp.hi != nullptr ? tc_scale_of(*y.Wp.exp) : 1.f;
+    uint32_t m = 0u;
+    for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4w; i += y.n_blocks_w * EW_THREADS) {
+      float4 v = ld4(y.W, i);
+      const float4 g = ld4(y.G, i);
+      v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
+      st4(y.W, i, v);
+      if (y.Wp.hi != nullptr) store_planes4(y.Wp, i, v, scale);
+      m = max(m, abs_bits(v));
+    }
+    if (y.amax_W != nullptr) commit_amax(m, y.amax_W);        // the next W-step bounds W by it
+    return;
+  }
+  const int block = (int)blockIdx.x - y.n_blocks_w;
+  if (block >= y.n_blocks_r) return;
+  const int ld = y.ld, n_groups = ld >> 2;
+  float *__restrict__ r = y.r;
+  const float *__restrict__ gp = y.gp;
+  const int cols_per_pass = min(n_groups, EW_THREADS);
   const int n_sub = min(EW_THREADS / cols_per_pass, COLSUM_MAX_SUB);
   const int sub = threadIdx.x / cols_per_pass, c0 = threadIdx.x % cols_per_pass;
-  const int r0 = blockIdx.x * rows_per_block, r1 = min(n_rows, r0 + rows_per_block);
-  double *out = slots + (size_t)blockIdx.x * ld;
+  const int r0 = block * y.rows_per_block, r1 = min(y.n_rows, r0 + y.rows_per_block);
+  double *out = y.slots + (size_t)block * ld;
   if (sub < n_sub) {
-    for (int cg = c0; cg < ld4; cg += cols_per_pass) {
+    for (int cg = c0; cg < n_groups; cg += cols_per_pass) {
       double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
 #pragma unroll 4
       for (int j = r0 + sub; j < r1; j += n_sub) {
-        const size_t o = (size_t)j * ld4 + cg;
-        float4 v = ld4f(r, o);
-        const float4 g = ld4f(gp, o);
+        const size_t o = (size_t)j * n_groups + cg;
+        float4 v = ld4(r, o);
+        const float4 g = ld4(gp, o);
         v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
         st4(r, o, v);
         s0 += (double)v.x; s1 += (double)v.y; s2 += (double)v.z; s3 += (double)v.w;
@@ -427,7 +427,7 @@ resid_colsum_kernel(float *__restrict__ r, const float *__restrict__ gp, const L
   }
   if (n_sub > 1) {
     __syncthreads();
-    for (int c = threadIdx.x; c < ld; c += blockDim.x) {
+    for (int c = threadIdx.x; c < ld; c += EW_THREADS) {
       double s = 0.0;
       for (int k = 0; k < n_sub; ++k) s += colsum_sh[(size_t)k * ld + c];
       out[c] = s;
@@ -474,23 +474,25 @@ sumsq_amax_kernel(const float *__restrict__ G, size_t n4, uint32_t *__restrict__
 // b+ = b - mean_j r[j][:]  (Eq. "update b" with the step 1/(nu N), i.e. the exact minimiser);
 // shift[c] = that mean, which the z-update subtracts from r.  blockDim = (32 columns, BIAS_GROUPS slot groups): group g
 // adds the slots g, g + BIAS_GROUPS, ... of its column, the group sums are then added in group order.
+struct BiasStep { const double *slots; int n_slots, ld, width; float *b, *shift; };
 __global__ void __launch_bounds__(32 * BIAS_GROUPS)
-finalize_bias_kernel(const double *__restrict__ slots, int n_slots, int ld, int width, double inv_n,
-                     float *__restrict__ b, float *__restrict__ shift) {
+finalize_bias_kernel(const __grid_constant__ Group<BiasStep> group, double inv_n) {
   __shared__ double sh[BIAS_GROUPS][33];
+  const BiasStep &y = group.l[blockIdx.y];
   const int c = blockIdx.x * 32 + threadIdx.x;
+  if (blockIdx.x * 32 >= (unsigned)y.ld) return;
   double s = 0.0;
-  if (c < ld)
+  if (c < y.ld)
 #pragma unroll 8
-    for (int i = threadIdx.y; i < n_slots; i += BIAS_GROUPS) s += slots[(size_t)i * ld + c];
+    for (int i = threadIdx.y; i < y.n_slots; i += BIAS_GROUPS) s += y.slots[(size_t)i * y.ld + c];
   sh[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.y == 0 && c < ld) {
+  if (threadIdx.y == 0 && c < y.ld) {
     double t = 0.0;
     for (int k = 0; k < BIAS_GROUPS; ++k) t += sh[k][threadIdx.x];
-    const float m = c < width ? (float)(t * inv_n) : 0.0f;
-    shift[c] = m;
-    if (c < width) b[c] -= m;
+    const float m = c < y.width ? (float)(t * inv_n) : 0.0f;
+    y.shift[c] = m;
+    if (c < y.width) y.b[c] -= m;
   }
 }
 
@@ -502,20 +504,35 @@ finalize_bias_kernel(const double *__restrict__ slots, int n_slots, int ld, int 
 // u+ by Eq. "update u", the linear residual of the next iteration r = a - z+, and t_{l+1} = u+ + rho (p_{l+1} - q+),
 // the part of the next p-gradient that does not involve a product.
 // At most 48 registers: two blocks fit on an SM beside a product.
+struct Zqu {
+  float *r, *z, *q, *u; const float *p_next, *shift; float *t_next;
+  const void *codes_next;                 // pdADMM-G-Q: codes of p_next, read instead of it
+  float q_scale, q_lo; uint32_t ld4cols, n4;
+  uint32_t *amax_r;                       // max|r| (see commit_amax); may be null
+  PlaneOut rp;                            // planes of r for the coming p-gradient
+  int n_blocks;
+};
+struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T; };
 __global__ void __launch_bounds__(EW_THREADS, 5)
-zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, float *__restrict__ u,
-           const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
-           float rho, float nu, float slope, float q_scale, float q_lo, float q_top, float *__restrict__ t_next,
-           uint32_t *__restrict__ amax_r /* max|r| (see commit_amax); may be null */,
-           PlaneOut rp /* planes of r for the coming p-gradient */,
-           const void *__restrict__ codes_next /* pdADMM-G-Q: codes of p_next, read instead of it */, int wide_codes) {
-  const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
+zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
+  const Zqu &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.n_blocks) return;
+  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
+  const float *__restrict__ p_next = y.p_next;
+  const void *__restrict__ codes_next = y.codes_next;
+  const float rho = prm.rho, nu = prm.nu, slope = prm.slope, q_top = prm.q_top, q_scale = y.q_scale, q_lo = y.q_lo;
+  const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
   const float inv_rn = 1.0f / (rho + nu), inv_neg = 1.0f / (2.0f + slope * slope);
   uint32_t mr = 0u;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 sh = ld4(shift, i % ld4cols);
+  // the column group of element i is carried along (a division per element costs more than the arithmetic of the update)
+  const uint32_t stride = y.n_blocks * EW_THREADS, stride_col = stride % y.ld4cols;
+  uint32_t col = (blockIdx.x * EW_THREADS + threadIdx.x) % y.ld4cols;
+  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4; i += stride) {
+    const float4 sh = ld4(y.shift, col);
+    col += stride_col;
+    if (col >= y.ld4cols) col -= y.ld4cols;
     const float4 rv = ld4(r, i), zv = ld4(z, i), qv = ld4(q, i), uv = ld4(u, i);
-    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
+    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
     float4 zn, qn, un, rn, tn;
 #define PD_ZQU(f)                                                                   \
     {                                                                               \
@@ -535,10 +552,10 @@ zqu_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, 
     PD_ZQU(x) PD_ZQU(y) PD_ZQU(z) PD_ZQU(w)
 #undef PD_ZQU
     st4(z, i, zn); st4(q, i, qn); st4(u, i, un); st4(r, i, rn); st4(t_next, i, tn);
-    if (rp.hi != nullptr) store_planes4(rp, i, rn, scale);
+    if (y.rp.hi != nullptr) store_planes4(y.rp, i, rn, scale);
     mr = max(mr, abs_bits(rn));
   }
-  if (amax_r != nullptr) commit_amax(mr, amax_r);
+  if (y.amax_r != nullptr) commit_amax(mr, y.amax_r);
 }
 
 // ---- the same for a smooth activation: z-update by lookup table ---------------------------------------------
@@ -604,21 +621,29 @@ __device__ __forceinline__ void table_best(const float *__restrict__ f_sh, int T
   }
 }
 __global__ void __launch_bounds__(EW_THREADS)
-zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict__ q, float *__restrict__ u,
-                 const float *__restrict__ p_next, const float *__restrict__ shift, int ld4cols, size_t n4,
-                 float rho, float nu, float act, float t_lo, float t_step, int T, float q_scale, float q_lo, float q_top,
-                 float *__restrict__ t_next, uint32_t *__restrict__ amax_r, PlaneOut rp,
-                 const void *__restrict__ codes_next, int wide_codes) {
+zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
+  const Zqu &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.n_blocks) return;
+  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
+  const float *__restrict__ p_next = y.p_next;
+  const void *__restrict__ codes_next = y.codes_next;
+  const float rho = prm.rho, nu = prm.nu, act = prm.slope, q_top = prm.q_top, q_scale = y.q_scale, q_lo = y.q_lo;
+  const float t_lo = prm.t_lo, t_step = prm.t_step;
+  const int T = prm.T;
   extern __shared__ float table_sh[];              // f(z_i)
   for (int i = threadIdx.x; i < T; i += blockDim.x) table_sh[i] = act_eval(__fadd_rn(t_lo, __fmul_rn((float)i, t_step)), act);
   __syncthreads();
   const float inv_rn = 1.0f / (rho + nu);
-  const float scale = rp.hi != nullptr ? tc_scale_of(*rp.exp) : 1.f;
+  const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
   uint32_t mr = 0u;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 sh = ld4(shift, i % ld4cols);
+  const uint32_t stride = y.n_blocks * EW_THREADS, stride_col = stride % y.ld4cols;
+  uint32_t col = (blockIdx.x * EW_THREADS + threadIdx.x) % y.ld4cols;
+  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4; i += stride) {
+    const float4 sh = ld4(y.shift, col);
+    col += stride_col;
+    if (col >= y.ld4cols) col -= y.ld4cols;
     const float4 rv = ld4(r, i), zv = ld4(z, i), qv = ld4(q, i), uv = ld4(u, i);
-    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
+    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
     const float a[4] = {(rv.x - sh.x) + zv.x, (rv.y - sh.y) + zv.y, (rv.z - sh.z) + zv.z, (rv.w - sh.w) + zv.w};
     const float zo[4] = {zv.x, zv.y, zv.z, zv.w}, qo[4] = {qv.x, qv.y, qv.z, qv.w};
     float zb[4], fb[4];
@@ -637,11 +662,11 @@ zqu_table_kernel(float *__restrict__ r, float *__restrict__ z, float *__restrict
     st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(q, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
     st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
     const float4 r4 = make_float4(rn[0], rn[1], rn[2], rn[3]);
-    if (rp.hi != nullptr) store_planes4(rp, i, r4, scale);
+    if (y.rp.hi != nullptr) store_planes4(y.rp, i, r4, scale);
     st4(r, i, r4); st4(t_next, i, make_float4(tn[0], tn[1], tn[2], tn[3]));
     mr = max(mr, abs_bits(r4));
   }
-  if (amax_r != nullptr) commit_amax(mr, amax_r);
+  if (y.amax_r != nullptr) commit_amax(mr, y.amax_r);
 }
 
 // ---- z-update of the last layer -------------------------------------------------------------------
@@ -954,24 +979,6 @@ argmax_kernel(const float *__restrict__ z, const int *__restrict__ labels, const
   }
   if (threadIdx.x == 4) out[4] = (unsigned long long)(unsigned)*error;
   if (threadIdx.x == 0) *counter = 0;
-}
-
-// W+ = W - grad_W * inv_theta  (Eq. "update W"), with the planes of W+
-__global__ void __launch_bounds__(EW_THREADS)
-wstep_kernel(float *__restrict__ W, const float *__restrict__ G, const LayerScalars *__restrict__ sc, size_t n4,
-             uint32_t *__restrict__ amax, PlaneOut planes) {
-  const float a = sc->inv_theta;
-  const float scale = planes.hi != nullptr ? tc_scale_of(*planes.exp) : 1.f;
-  uint32_t m = 0u;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    float4 v = ld4(W, i);
-    const float4 g = ld4(G, i);
-    v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
-    st4(W, i, v);
-    if (planes.hi != nullptr) store_planes4(planes, i, v, scale);
-    m = max(m, abs_bits(v));
-  }
-  if (amax != nullptr) commit_amax(m, amax);        // the next W-step bounds W by it
 }
 
 }  // namespace pd

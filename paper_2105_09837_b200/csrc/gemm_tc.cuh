@@ -39,6 +39,7 @@
 
 #include "common.cuh"
 #include "planes.cuh"
+#include "scalars.cuh"
 #include "gemm_simt.cuh"   // epilogue functors
 #include "tc_ptx.cuh"
 
@@ -69,7 +70,7 @@ constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
 constexpr int TC_TR_BYTES = 8 * 32 * 16 * 4;                   // epilogue transpose: 8 warps x 32 rows x 16 columns
 constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
-static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 2) + 12 <= 256, "barriers");
+static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3) + 12 <= 256, "barriers");
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -100,26 +101,42 @@ struct TcOperand {
   int ld = 0;
 };
 
-struct TcParams {
+// One launch works on the same product of several layers, whose output tiles form one sequence of work units: a small
+// problem's layers fill the GPU together, and a large one has one partly filled last round instead of one per layer.
+constexpr int TC_MAX_GROUP = 16;
+template <class Epi>
+struct TcLayer {
+  CUtensorMap a, alo, b, blo;      // planes of the operands
   int M, N, K;            // output rows, output columns, contraction length
   int k_chunk;            // contraction slice (multiple of TC_BK); K rounded up if not split
   int n_split;            // number of contraction slices; slice z writes its own partial output
+  int unit_end;           // work units of this layer and of those before it
   size_t c_split_stride;  // elements between the partial outputs of consecutive slices
-  int *error;             // set to 1 if a bounded wait expired
-  TcOperand a, b;
-  // Tail balancing (n_split == 1 only): output tiles from tail_begin on are cut into tail_split contraction
+  TcOperand oa, ob;
+  float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
+  Epi epi;
+  // Sums of squares (Epi::kSumsq and slots != null): one slot per 128-row tile, column tile and accumulate warp, written by
+  // whichever block has the tile; the block that completes the layer (`done`, zero before and after) adds them in index order
+  // and passes the sum to `step`.  Neither depends on how the tiles were shared out.
+  double *slots;
+  int *done;
+  Step step;
+  // Tail balancing (one layer, n_split == 1): output tiles from tail_begin on are cut into tail_split contraction
   // slices, one work unit each, so that the last, partly filled round of the persistent grid is shorter.
   // A slice leaves its accumulators in tail_ws; the warp that finds itself last (tail_count) adds the slices
   // in slice order and runs the epilogue.  tail_split <= 1 switches this off.
   int tail_begin, tail_split;
-  // Sums of squares: one slot per accumulate warp of the grid for the whole tiles of its block, then one per tail tile and
-  // warp of its block (pair), all in a fixed order whichever block finishes a tail tile.
   float *tail_ws;         // [tiles from tail_begin][tail_split][8 or 16 warps][64][32] floats
   int *tail_count;        // [tiles from tail_begin][8 or 16 warps], zero before and after every launch
-  float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
+};
+template <class Epi>
+struct TcGroup {
+  int n;
+  int *error;             // set to 1 if a bounded wait expired
+  TcLayer<Epi> l[TC_MAX_GROUP];
 };
 
-// LAYOUT bit 0: A is MN-major, bit 1: B is MN-major.  Tensor maps: planes of A (map_a = hi, map_alo = lo) and of B.
+// LAYOUT bit 0: A is MN-major, bit 1: B is MN-major.  Tensor maps: planes of A (a = hi, alo = lo) and of B.
 //   K-major:  matrix [output index][contraction index];  MN-major: matrix [contraction index][output index];
 //   boxes of 64 x 64 either way: 64 output indices (rows) x 64 values, or 64 rows x 64 output indices
 // PAIR: clusters of two blocks, each pair one tile of 256 x 128 outputs: block `rank` of the pair holds rows 128 rank .. +127
@@ -140,13 +157,11 @@ struct TcParams {
 // ZERO: bit 0 = the lo plane of A is identically zero, bit 1 = the lo plane of B is.  An operand of
 // pdADMM-G-Q that lies on a level set {c s} (the quantised p, or the difference of two of them) is the spacing s times
 // a small integer, and integers up to 2048 are exact in one fp16 plane: its plane holds the integers, there is no lo
-// plane to load and no MMA for it (two MMAs per product instead of three), and prm.mul = s restores the values.
+// plane to load and no MMA for it (two MMAs per product instead of three), and mul = s restores the values.
 enum : int { TC_NT = 0, TC_A_MN = 1, TC_B_MN = 2 };
 template <int LAYOUT, class Epi, int ZERO, bool PAIR>
 __global__ void __maxnreg__(TC_REGS_LAUNCH)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_alo,
-               const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_blo,
-               const __grid_constant__ TcParams prm, Epi epi, double *__restrict__ partials) {
+gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   constexpr bool A_MN = (LAYOUT & TC_A_MN) != 0, B_MN = (LAYOUT & TC_B_MN) != 0, COARSE = epi_coarse<Epi>::value || ZERO == 3;
   // which lo planes are loaded and used (a product that only wants its squared norm uses neither, and lets the main
   // term accumulate in tensor memory over the whole contraction: the truncation of that accumulation, 1e-5 relative,
@@ -165,31 +180,46 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   uint64_t *bars = reinterpret_cast<uint64_t *>(tr_base + TC_TR_BYTES);
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
   uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
-  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain_bar + 1);
+  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(team_bar + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_rank() : 0u;
-  const int unit0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, unit_step = PAIR ? gridDim.x >> 1 : gridDim.x;
-  const int tiles_n = (prm.N + TC_BN - 1) / TC_BN, tiles_m = (prm.M + TILE_M - 1) / TILE_M;
-  const int n_out_tiles = tiles_n * tiles_m * prm.n_split;
-  const bool tail_on = prm.tail_split > 1;
-  const int tail_begin = tail_on ? prm.tail_begin : n_out_tiles;
-  const int n_tiles = tail_begin + (n_out_tiles - tail_begin) * (tail_on ? prm.tail_split : 1);   // work units
+  const int unit0 = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x), unit_step = (int)(PAIR ? gridDim.x >> 1 : gridDim.x);
+  const int n_units = grp.l[grp.n - 1].unit_end;
 
-  // scaling exponents of the two operands (written by earlier kernels of the stream), and whether the planes made with
+  // scaling exponents of every layer's operands (written by earlier kernels of the stream), and whether the planes made with
   // them are usable; the same for every block
-  int exp_a = prm.a.exp ? *prm.a.exp : 0, exp_b = prm.b.exp ? *prm.b.exp : 0;
-  bool split_a = prm.a.amax != nullptr && !tc_planes_usable(*prm.a.amax, exp_a);
-  bool split_b = prm.b.amax != nullptr && !tc_planes_usable(*prm.b.amax, exp_b);
-  if (split_a) { exp_a = tc_scale_exp(*prm.a.amax); split_a = prm.a.x != nullptr; }
-  if (split_b) { exp_b = tc_scale_exp(*prm.b.amax); split_b = prm.b.x != nullptr; }
-
+  __shared__ int lay_exp[TC_MAX_GROUP][2];
+  __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
+  bool my_split = false;
+  // (only of layers this block works on: the step of a finished layer may already have changed the words of the others)
+  if (threadIdx.x < (unsigned)grp.n) {
+    int split = 0;
+    const int g = (int)threadIdx.x, begin = g > 0 ? grp.l[g - 1].unit_end : 0;
+    const int ahead = (unit0 - begin) % unit_step, first = begin + (ahead < 0 ? ahead + unit_step : ahead);
+    const bool has_unit = first < grp.l[g].unit_end;
+    auto look = [&](const TcOperand &o, int bit) {
+      int e = o.exp ? *o.exp : 0;
+      if (o.amax != nullptr && !tc_planes_usable(*o.amax, e)) {
+        e = tc_scale_exp(*o.amax);
+        if (o.x != nullptr) split |= bit;
+      }
+      return e;
+    };
+    if (has_unit) {
+      lay_exp[g][0] = look(grp.l[g].oa, 1);
+      lay_exp[g][1] = look(grp.l[g].ob, 2);
+      lay_split[g] = split;
+      my_split = split != 0;
+    }
+  }
+  const bool any_split = __syncthreads_or(my_split);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      ptx::mbar_init(&full_bar[s], 1 + ((split_a || split_b) ? CG * TC_SPLIT_WARPS : 0));
+      ptx::mbar_init(&full_bar[s], 1 + (any_split ? CG * TC_SPLIT_WARPS : 0));
       ptx::mbar_init(&empty_bar[s], 1);
     }
     for (int b = 0; b < TC_ACC_BUFS; ++b) {
@@ -198,15 +228,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
+    ptx::mbar_init(team_bar, TC_ACC_WARPS);
     *abort_flag = 0;
     // One thread reads the error word for the whole block, so that all warps take the same path: every block still
     // allocates and releases its tensor memory and passes both block-wide barriers.
-    *skip_flag = *reinterpret_cast<volatile int *>(prm.error) != 0;
+    *skip_flag = *reinterpret_cast<volatile int *>(grp.error) != 0;
     ptx::fence_barrier_init();
-    ptx::prefetch_tmap(&map_a);
-    ptx::prefetch_tmap(&map_b);
-    if (A_LO) ptx::prefetch_tmap(&map_alo);
-    if (B_LO) ptx::prefetch_tmap(&map_blo);
+    ptx::prefetch_tmap(&grp.l[0].a);
+    ptx::prefetch_tmap(&grp.l[0].b);
   }
   if (warp == 1) ptx::tmem_alloc<CG>(tmem_slot, TC_TMEM_COLS);
   ptx::tc_fence_before_sync();
@@ -215,25 +244,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
-  // work unit -> (row tile origin, column tile origin, first and number of K blocks); a unit is an output tile or,
-  // in the tail, one contraction slice of an output tile
-  auto tile_coords = [&](int unit, int &m0, int &n0, int &k_begin, int &n_kb, int &z) {
-    int tile = unit, slice = 0;
-    if (unit >= tail_begin) {
-      tile = tail_begin + (unit - tail_begin) / prm.tail_split;
-      slice = (unit - tail_begin) % prm.tail_split;
+  // Work unit -> its layer, row and column tile origin, first and number of K blocks, contraction slice; a unit is an output
+  // tile or, in the tail, one contraction slice of an output tile.  Units are visited in ascending order.
+  struct Tile { int g = 0, m0, n0, k_begin, n_kb, z, out, slice; };
+  auto locate = [&](int unit, Tile &t) {
+    while (unit >= grp.l[t.g].unit_end) ++t.g;
+    const TcLayer<Epi> &y = grp.l[t.g];
+    if (t.g > 0) unit -= grp.l[t.g - 1].unit_end;
+    const int tiles_n = (y.N + TC_BN - 1) / TC_BN, tiles_m = (y.M + TILE_M - 1) / TILE_M;
+    t.out = unit; t.slice = -1;
+    if (y.tail_split > 1 && unit >= y.tail_begin) {
+      t.out = y.tail_begin + (unit - y.tail_begin) / y.tail_split;
+      t.slice = (unit - y.tail_begin) % y.tail_split;
     }
-    z = tile / (tiles_m * tiles_n);
-    const int rem = tile - z * tiles_m * tiles_n;
-    m0 = (rem / tiles_n) * TILE_M + (int)rank * TC_BM;       // of this block
-    n0 = (rem % tiles_n) * TC_BN;
-    k_begin = z * prm.k_chunk;
-    const int k_end = min(prm.K, k_begin + prm.k_chunk);
-    n_kb = (max(k_end - k_begin, 0) + TC_BK - 1) / TC_BK;
-    if (unit >= tail_begin) {
-      const int kb0 = slice * n_kb / prm.tail_split, kb1 = (slice + 1) * n_kb / prm.tail_split;
-      k_begin += kb0 * TC_BK;
-      n_kb = kb1 - kb0;
+    t.z = t.out / (tiles_m * tiles_n);
+    const int rem = t.out - t.z * tiles_m * tiles_n;
+    t.m0 = (rem / tiles_n) * TILE_M + (int)rank * TC_BM;       // of this block
+    t.n0 = (rem % tiles_n) * TC_BN;
+    t.k_begin = t.z * y.k_chunk;
+    const int k_end = min(y.K, t.k_begin + y.k_chunk);
+    t.n_kb = (max(k_end - t.k_begin, 0) + TC_BK - 1) / TC_BK;
+    if (t.slice >= 0) {
+      const int kb0 = t.slice * t.n_kb / y.tail_split, kb1 = (t.slice + 1) * t.n_kb / y.tail_split;
+      t.k_begin += kb0 * TC_BK;
+      t.n_kb = kb1 - kb0;
     }
   };
 
@@ -247,7 +281,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (warp == 0) {
       // -------------------------------------------------------------- TMA producer (one lane)
       if (lane == 0) {
-        const uint32_t tx = CG * (uint32_t)((split_a ? 0 : A_PLANES * TC_PLANE_BYTES) + (split_b ? 0 : B_PLANES * B_PLANE_BYTES));
         int s = 0, it = 0;
         uint32_t ph = 1;                                // phase of the stage's previous use
         bool ok = true;
@@ -257,22 +290,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           for (int i = 0; i < boxes; ++i)
             ptx::tma_load_2d<CG>(dst + i * TC_BOX_BYTES, map, mn ? o0 + 64 * i : k0, mn ? k0 : o0 + 64 * i, bar);
         };
-        for (int tile = unit0; tile < n_tiles && ok; tile += unit_step) {
-          int m0, n0, k_begin, n_kb, z;
-          tile_coords(tile, m0, n0, k_begin, n_kb, z);
-          for (int kb = 0; kb < n_kb; ++kb, ++it) {
+        Tile t;
+        for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+          locate(unit, t);
+          const TcLayer<Epi> &y = grp.l[t.g];
+          const bool split_a = any_split && (lay_split[t.g] & 1), split_b = any_split && (lay_split[t.g] & 2);
+          const uint32_t tx = CG * (uint32_t)((split_a ? 0 : A_PLANES * TC_PLANE_BYTES) + (split_b ? 0 : B_PLANES * B_PLANE_BYTES));
+          for (int kb = 0; kb < t.n_kb; ++kb, ++it) {
             if (it >= STAGES && !ptx::mbar_wait(&empty_bar[s], ph, abort_flag)) { ok = false; break; }
             uint8_t *st = smem + s * STAGE_BYTES;
-            const int k0 = k_begin + kb * TC_BK;
-            const int nb = n0 + (int)rank * BN;            // columns of B that this block loads
+            const int k0 = t.k_begin + kb * TC_BK;
+            const int nb = t.n0 + (int)rank * BN;          // columns of B that this block loads
             if (rank == 0) ptx::mbar_expect_tx(&full_bar[s], tx);       // the bytes of both blocks
             if (!split_a) {
-              load(st, &map_a, A_MN, m0, k0, 2);
-              if (A_LO) load(st + TC_PLANE_BYTES, &map_alo, A_MN, m0, k0, 2);
+              load(st, &y.a, A_MN, t.m0, k0, 2);
+              if (A_LO) load(st + TC_PLANE_BYTES, &y.alo, A_MN, t.m0, k0, 2);
             }
             if (!split_b) {
-              load(st + B_OFF, &map_b, B_MN, nb, k0, BN / 64);
-              if (B_LO) load(st + B_OFF + B_PLANE_BYTES, &map_blo, B_MN, nb, k0, BN / 64);
+              load(st + B_OFF, &y.b, B_MN, nb, k0, BN / 64);
+              if (B_LO) load(st + B_OFF + B_PLANE_BYTES, &y.blo, B_MN, nb, k0, BN / 64);
             }
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
@@ -304,16 +340,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // running state: stage s with phase bit sp, accumulator buffer b with phase bit bp (of its *previous* use)
         int s = 0, b = 0, ti = 0, used = 0;
         uint32_t sp = 0, bp = 1;
-        for (int tile = unit0; tile < n_tiles && ok; tile += unit_step, ++ti) {
-          int m0, n0, k_begin, n_kb, z;
-          tile_coords(tile, m0, n0, k_begin, n_kb, z);
+        Tile t;
+        for (int unit = unit0; unit < n_units && ok; unit += unit_step, ++ti) {
+          locate(unit, t);
+          const int n_kb = t.n_kb;
           for (int kb = 0; kb < n_kb; ++kb) {
             const bool first = kb % FLUSH == 0, last = kb % FLUSH == FLUSH - 1 || kb == n_kb - 1;
             bool good = ptx::mbar_wait(&full_bar[s], sp, abort_flag);
             if (first && used >= TC_ACC_BUFS) good = good && ptx::mbar_wait(&acc_empty[b], bp, abort_flag);
             ok = __all_sync(0xffffffffu, good);
             if (!ok) break;
-            if (PAIR && (split_a || split_b)) ptx::fence_cluster();
+            if (PAIR && any_split) ptx::fence_cluster();
             ptx::tc_fence_after_sync();
             const uint32_t la = lo_a0 + (uint32_t)s * (STAGE_BYTES >> 4), lb = lo_b0 + (uint32_t)s * (STAGE_BYTES >> 4);
             const uint32_t d = tmem_base + (uint32_t)(b * TC_BN);
@@ -369,12 +406,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           ptx::mbar_wait(drain_bar, 0, abort_flag, 200000000ll, false);
         }
       }
-    } else if (split_a || split_b) {
+    } else if (any_split) {
       // -------------------------------------------------------------- planes of a refused operand (two warps)
       // Eight consecutive values at a time, rows in order, so that a warp reads whole rows; written where TMA would have
       // put them (16-byte chunk c of a 128-byte row r at position c ^ (r mod 8)).
       const int t = threadIdx.x - 32 * TC_SPLIT0;
-      const float scale_a = tc_pow2(exp_a), scale_b = tc_pow2(exp_b);
       auto split_tile = [&](const TcOperand &o, bool mn, bool lo_too, float scale, uint8_t *dst, int boxes, int o0, int k0, int n_outer, int n_k) {
         // K-major: 64 or 128 rows of 8 chunks, inner = contraction; MN-major: 64 rows of 8 or 16 chunks, inner = output index
         const int rows = mn ? n_k - k0 : n_outer - o0, chunks = mn ? 8 * boxes : 8, inner0 = mn ? o0 : k0;
@@ -397,16 +433,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       int s = 0, it = 0;
       uint32_t ph = 1;
       bool ok = true;
-      for (int tile = unit0; tile < n_tiles && ok; tile += unit_step) {
-        int m0, n0, k_begin, n_kb, z;
-        tile_coords(tile, m0, n0, k_begin, n_kb, z);
-        for (int kb = 0; kb < n_kb; ++kb, ++it) {
+      Tile u;
+      for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+        locate(unit, u);
+        const TcLayer<Epi> &y = grp.l[u.g];
+        const int split = lay_split[u.g];
+        const float scale_a = tc_pow2(lay_exp[u.g][0]), scale_b = tc_pow2(lay_exp[u.g][1]);
+        for (int kb = 0; kb < u.n_kb; ++kb, ++it) {
           ok = it < STAGES || ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           uint8_t *st = smem + s * STAGE_BYTES;
-          const int k0 = k_begin + kb * TC_BK;
-          if (split_a) split_tile(prm.a, A_MN, A_LO, scale_a, st, 2, m0, k0, prm.M, prm.K);
-          if (split_b) split_tile(prm.b, B_MN, B_LO, scale_b, st + B_OFF, BN / 64, n0 + (int)rank * BN, k0, prm.N, prm.K);
+          const int k0 = u.k_begin + kb * TC_BK;
+          if (split & 1) split_tile(y.oa, A_MN, A_LO, scale_a, st, 2, u.m0, k0, y.M, y.K);
+          if (split & 2) split_tile(y.ob, B_MN, B_LO, scale_b, st + B_OFF, BN / 64, u.n0 + (int)rank * BN, k0, y.N, y.K);
           ptx::fence_proxy_async_smem();
           if (PAIR) ptx::fence_cluster();
           __syncwarp();
@@ -421,19 +460,68 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int aw = warp - TC_ACC0, quarter = warp & 3, col_base = 64 * (aw >> 2);
     const int lane_base = quarter * 32, piece = (int)rank * TC_ACC_WARPS + aw;
     float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 4;    // 32 rows x 4 float4 per warp
-    // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
-    // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
-    const int n_pad = epi.ldc;
     bool ok = true;
     int b = 0;
-    double ss = 0.0;                                   // this thread's part of its warp's slot
     uint32_t ph = 0;                                   // phase of acc_full[b]
-    for (int tile = unit0; tile < n_tiles && ok; tile += unit_step) {
-      int m0, n0, k_begin, n_kb, z;
-      tile_coords(tile, m0, n0, k_begin, n_kb, z);
-      n0 += col_base;                               // of this warp
+    Tile t;
+    int visited = 0;                                   // units of layer t.g that this block has finished
+    // all accumulate warps of the block; bounded like every other wait
+    uint32_t team_ph = 0;
+    auto team_sync = [&]() {
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(team_bar);
+      const bool there = ptx::mbar_wait(team_bar, team_ph, abort_flag);
+      team_ph ^= 1u;
+      return __all_sync(0xffffffffu, there) != 0;
+    };
+    // The block has no further unit of layer g: if every unit of the layer is finished with this, add the slots.
+    auto leave = [&](int g) {
+      const TcLayer<Epi> &y = grp.l[g];
+      if (!Epi::kSumsq || y.slots == nullptr || visited == 0) return true;
+      constexpr int n_threads = 32 * TC_ACC_WARPS;
+      const int tid = aw * 32 + lane;
+      volatile int *last = reinterpret_cast<int *>(tr_base);              // the first warp's staging buffer
+      volatile double *part = reinterpret_cast<double *>(tr_base) + 8;
+      __threadfence();
+      if (!team_sync()) return false;
+      if (tid == 0) {
+        const int units = (y.unit_end - (g > 0 ? grp.l[g - 1].unit_end : 0)) * CG;
+        const int before = atomicAdd(y.done, visited);
+        *last = before + visited == units;
+      }
+      if (!team_sync()) return false;
+      if (*last != 0) {
+        __threadfence();
+        const int n = (y.M + TC_BM - 1) / TC_BM * ((y.N + TC_BN - 1) / TC_BN) * TC_ACC_WARPS;
+        double v = 0.0;
+#pragma unroll 4
+        for (int i = tid; i < n; i += n_threads) v += __ldcg(y.slots + i);
+        v = warp_sum(v);
+        if (lane == 0) part[aw] = v;
+        if (!team_sync()) return false;
+        if (tid == 0) {
+          double sum = 0.0;
+          for (int i = 0; i < TC_ACC_WARPS; ++i) sum += part[i];
+          *y.done = 0;
+          finish_step(y.step, sum);
+        }
+      }
+      visited = 0;
+      return team_sync();                              // the staging buffer is free again
+    };
+    for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+      const int g_before = t.g;
+      locate(unit, t);
+      if (t.g != g_before && !leave(g_before)) { ok = false; break; }
+      ++visited;
+      const TcLayer<Epi> &y = grp.l[t.g];
+      const Epi &epi = y.epi;
+      const int m0 = t.m0, n0 = t.n0 + col_base, n_kb = t.n_kb;       // n0: of this warp
+      // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
+      // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
+      const int n_pad = epi.ldc;
       const int n_grp = COARSE ? (n_kb > 0 ? 1 : 0) : n_kb;   // read-outs of the main accumulator for this tile
-      if (m0 + lane_base + lane < prm.M) {          // this thread's row of the epilogue inputs, on its way to L2
+      if (m0 + lane_base + lane < y.M) {          // this thread's row of the epilogue inputs, on its way to L2
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int col = n0 + h * 32;
@@ -478,13 +566,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // correction terms: complete once the last block's commit has arrived (it covers every earlier MMA)
         if constexpr (!COARSE) add_tile(TC_COL_CORR, std::false_type{}, corr_empty);
         // undo the operand scalings (two exact factors, so that neither leaves the range on its own)
-        const int e1 = (exp_a + exp_b) / 2, e2 = exp_a + exp_b - e1;
+        const int e = lay_exp[t.g][0] + lay_exp[t.g][1], e1 = e / 2, e2 = e - e1;
         const uint32_t u1 = __float_as_uint(tc_pow2(-e1)), u2 = __float_as_uint(tc_pow2(-e2));
         const uint64_t w1 = ptx::pack_f2(u1, u1), w2 = ptx::pack_f2(u2, u2);
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(ptx::mul_f2(acc[j], w1), w2);
         if constexpr (ZERO != 0) {
-          const uint64_t mul = ptx::pack_f2(__float_as_uint(prm.mul), __float_as_uint(prm.mul));
+          const uint64_t mul = ptx::pack_f2(__float_as_uint(y.mul), __float_as_uint(y.mul));
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
         }
@@ -495,26 +583,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ptx::unpack_f2(acc[2 * j + 1], v.z, v.w);
         return v;
       };
-      int out_tile = tile;
-      if (tile >= tail_begin) {
+      if (t.slice >= 0) {
         // contraction slice of a tail tile: park the accumulators; the last warp to arrive sums the slices
-        const int u = tile - tail_begin, t_idx = u / prm.tail_split;
-        out_tile = tail_begin + t_idx;
-        float4 *mine = reinterpret_cast<float4 *>(prm.tail_ws) + ((size_t)u * WARPS + piece) * 512;
+        const int t_idx = t.out - y.tail_begin, u = t_idx * y.tail_split + t.slice;
+        float4 *mine = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)u * WARPS + piece) * 512;
 #pragma unroll
         for (int j = 0; j < 16; ++j) mine[j * 32 + lane] = acc_at(j);
         __threadfence();
         __syncwarp();
         int prev = 0;
-        if (lane == 0) prev = atomicAdd(prm.tail_count + t_idx * WARPS + piece, 1);
+        if (lane == 0) prev = atomicAdd(y.tail_count + t_idx * WARPS + piece, 1);
         prev = __shfl_sync(0xffffffffu, prev, 0);
-        if (prev != prm.tail_split - 1) continue;
+        if (prev != y.tail_split - 1) continue;
         __threadfence();
-        if (lane == 0) prm.tail_count[t_idx * WARPS + piece] = 0;
+        if (lane == 0) y.tail_count[t_idx * WARPS + piece] = 0;
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = 0ull;
-        for (int sl = 0; sl < prm.tail_split; ++sl) {
-          const float4 *part = reinterpret_cast<const float4 *>(prm.tail_ws) + ((size_t)(t_idx * prm.tail_split + sl) * WARPS + piece) * 512;
+        for (int sl = 0; sl < y.tail_split; ++sl) {
+          const float4 *part = reinterpret_cast<const float4 *>(y.tail_ws) + ((size_t)(t_idx * y.tail_split + sl) * WARPS + piece) * 512;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const float4 v = __ldcg(part + j * 32 + lane);
@@ -540,7 +626,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ptx::unpack_f2(s2[1], s4[2], s4[3]);
         ss_tile = ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]);
       } else {
-        float *C = epi.C + (size_t)z * prm.c_split_stride;
+        float *C = epi.C + (size_t)t.z * y.c_split_stride;
         float ssf = 0.f;
         uint32_t mx = 0u;                  // largest magnitude stored by this thread
         float h_scale = 0.f;               // scaling of the planes of the result, if they are wanted
@@ -571,7 +657,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
               for (int i = 0; i < BATCH; ++i) {
                 const int r = 8 * i + (lane >> 2);
-                if constexpr (!Epi::kDirect) epi.load(min(m0 + lane_base + r, prm.M - 1), col, in[i]);
+                if constexpr (!Epi::kDirect) epi.load(min(m0 + lane_base + r, y.M - 1), col, in[i]);
               }
 #pragma unroll
               for (int i = 0; i < BATCH; ++i) {
@@ -579,10 +665,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const int row = m0 + lane_base + r;
                 float4 o = tr[r * 4 + ((lane & 3) ^ ((r >> 1) & 3))];
                 if constexpr (epi_sumsq_acc<Epi>::value) {
-                  if (row < prm.M) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
+                  if (row < y.M) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
                 }
                 if constexpr (!Epi::kDirect) o = epi.apply(col, o, in[i]);
-                if (row < prm.M) {
+                if (row < y.M) {
                   if (Epi::kSumsq && !epi_sumsq_acc<Epi>::value) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
                   *reinterpret_cast<float4 *>(C + (size_t)row * epi.ldc + col) = o;
                   if constexpr (epi_planes<Epi>::value) {
@@ -604,17 +690,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (epi.amax != nullptr) commit_amax(mx, epi.amax);      // the output is an operand of a later product
         }
       }
-      if (tile < tail_begin) {
-        ss += ss_tile;
-      } else if (partials != nullptr) {
+      if (Epi::kSumsq && y.slots != nullptr && m0 < y.M) {
         ss_tile = warp_sum(ss_tile);
-        if (lane == 0) partials[(size_t)gridDim.x * TC_ACC_WARPS + (size_t)(out_tile - tail_begin) * WARPS + piece] = ss_tile;
+        const int tiles_n = (y.N + TC_BN - 1) / TC_BN;
+        if (lane == 0) y.slots[((size_t)(m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw] = ss_tile;
       }
     }
-    if (partials != nullptr) {
-      ss = warp_sum(ss);
-      if (lane == 0) partials[(size_t)blockIdx.x * TC_ACC_WARPS + aw] = ss;
-    }
+    if (ok) leave(t.g);
   }
   ptx::tc_fence_before_sync();
   // neither block of a pair leaves while the other may still arrive on its barriers or read its shared memory
@@ -624,7 +706,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc<CG>(tmem_base, TC_TMEM_COLS);
   }
-  if (threadIdx.x == 0 && *abort_flag) atomicExch(prm.error, 1);
+  if (threadIdx.x == 0 && *abort_flag) atomicExch(grp.error, 1);
 }
 
 }  // namespace pd

@@ -13,6 +13,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -113,11 +114,15 @@ struct Layer {
   // that write them: amax_p covers every p_l written since the last tau of the layer, amax_r every r_l written
   // since its last theta -- upper bounds of the current maxima, which is all the power-of-two scaling needs.
   uint32_t *amax_p = nullptr, *amax_r = nullptr;
+  // largest magnitudes of an iteration's g, W g, G and d: zero before the kernel that writes the matrix
+  uint32_t *w_g = nullptr, *w_wg = nullptr, *w_G = nullptr, *w_d = nullptr;
+  int *done = nullptr;             // counters of finished blocks (products; trial; gradient sum), zero between kernels
   int n_split = 1, k_chunk = 0;
 };
 
 struct Scratch {
-  cudaStream_t st = nullptr;
+  cudaStream_t st = nullptr;       // where its layers' kernels are queued
+  cudaStream_t own = nullptr;      // the stream it owns (grouped: st is the main stream)
   float *s1 = nullptr;      // g, later G p+
   float *s2 = nullptr;      // W g, later W d
   float *p_new = nullptr;   // quantised trial
@@ -178,6 +183,12 @@ struct pdadmm_ctx {
   // tensor-bound ones.  `cur` is the lane that the host code is queueing on.
   std::vector<std::unique_ptr<pd::Scratch>> more_lanes;
   pd::Scratch *cur = &scr;
+  // A problem small enough for scratch per layer is worked on in batches instead: every kernel is launched once for up to
+  // MAX_GROUP layers, on the main stream.
+  bool grouped = false;
+  bool tail_split = true;           // large problems: products cut the tiles of a partly filled last round (launch_tc)
+  int n_active = 1;                 // scratches in use: layer l works with number l mod n_active
+  bool p_stale = false;             // p_l, l >= 2, exists as codes alone (integer operands): the fp32 values are older
   std::vector<cudaEvent_t> ev_p;    // [L]: p_l of this iteration is complete
   std::vector<cudaEvent_t> ev_lane; // [n_lanes]: fork / join
   bool r_valid = false;
@@ -202,7 +213,7 @@ struct pdadmm_ctx {
   char *arena_base = nullptr;       // current chunk
   size_t arena_cap = 0, arena_used = 0, arena_next = size_t(64) << 20;
   bool use_tc = true;               // dense products on the tensor cores
-  // pdADMM-G-Q with at most 2048 levels starting at zero: p_l = code * s_l exactly, and the codes are exact in fp16, so
+  // pdADMM-G-Q with at most 2048 levels: p_l = (code - levels below zero) * s_l, integers that are exact in fp16, so
   // the products whose operand is p_l (or d = p+ - p) take one plane of integers instead of a hi and a lo plane of
   // the values: two MMAs per product instead of three, a quarter of the operand bytes, no split pass
   bool int_operands = false;
@@ -282,13 +293,6 @@ static int shard_sum(pdadmm_ctx *c, cudaStream_t st, void *buf, size_t count, in
   if (rc != 0) return fail(PDADMM_ECUDA, "the reduction callback returned %d", rc);
   return PDADMM_OK;
 }
-// fixed-order totals of up to two slot arrays into red[0], red[1], then their sum over the shards
-static int shard_sum_slots(pdadmm_ctx *c, cudaStream_t st, double *red, const double *a, int na, const double *b, int nb) {
-  reduce_slots_kernel<<<1, 256, 0, st>>>(a, na, 1, 1, red);
-  if (b != nullptr) reduce_slots_kernel<<<1, 256, 0, st>>>(b, nb, 1, 1, red + 1);
-  return shard_sum(c, st, red, b != nullptr ? 2 : 1, 1);
-}
-
 // ---- profiling hooks ----------------------------------------------------------------------------------
 static cudaEvent_t take_event(pdadmm_ctx *c) {
   cudaEvent_t e;
@@ -362,17 +366,21 @@ static int get_tmap(pdadmm_ctx *c, const void *base, uint64_t inner, uint64_t ou
   return PDADMM_OK;
 }
 
-// Whether a product of M x N outputs in n_split slices runs on pairs of SMs: they halve the traffic of B, but a pair's tile has
-// 256 rows.  So: where at least three quarters of the pairs get a tile, and padding M to 256 rows instead of 128 adds at most
-// a tenth.  (20 000 x 500 x 500: 43.2 us in pairs, 45.5 us without; x 2000 x 2000: 399 against 457 us; 2000 x 100 x 100, 8
-// pairs: 12.5 against 10.7 us.)
-static bool use_pairs(const pdadmm_ctx *c, int M, int N, int n_split) {
-  const int64_t m1 = ceil_div(M, TC_BM), m2 = 2 * ceil_div(M, 2 * TC_BM);
-  return m2 * 10 <= m1 * 11 && (m2 / 2) * ceil_div(N, TC_BN) * n_split * 8 >= 3 * (int64_t)c->n_sms;
-}
+// One layer's part of a product launch.
+template <class Epi>
+struct Prod {
+  int M, N, K;
+  Operand A, B;
+  Epi epi;
+  Scratch *s;                      // of the layer: room for planes that have to be made first
+  double *slots = nullptr;         // one per tile and warp (null: no sum is wanted)
+  int *done = nullptr;
+  Step step{};
+  int n_split = 1, k_chunk = 0;    // contraction slices, and their length
+  size_t stride = 0;               // floats between the partial outputs of two slices
+};
 template <int LAYOUT, class Epi, int ZERO, bool PAIR>
-static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap (&maps)[4], const TcParams &prm, const Epi &epi,
-                          double *partials, int n_units) {
+static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &grp) {
   auto kern = gemm_tc_kernel<LAYOUT, Epi, ZERO, PAIR>;
   // the attribute belongs to (kernel, device): one flag per device ordinal for this instantiation
   static bool configured[MAX_DEVICES] = {false};
@@ -389,6 +397,7 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap (&ma
     PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
     if (dev >= 0 && dev < MAX_DEVICES) configured[dev] = true;
   }
+  const int n_units = grp.l[grp.n - 1].unit_end;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(PAIR ? 2 * std::min(n_units, c->n_sms / 2) : std::min(n_units, c->n_sms)));
   cfg.blockDim = dim3(TC_THREADS);
@@ -399,50 +408,71 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const CUtensorMap (&ma
   cluster.val.clusterDim.x = 2; cluster.val.clusterDim.y = 1; cluster.val.clusterDim.z = 1;
   cfg.attrs = &cluster;
   cfg.numAttrs = PAIR ? 1 : 0;
-  PD_CUDA(cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], prm, epi, partials));
+  PD_CUDA(cudaLaunchKernelEx(&cfg, kern, grp));
   return PDADMM_OK;
 }
-// op(A) is M x K, op(B) is N x K; A_MN: A is stored [K][M], B_MN: B is stored [K][N].  The tail of the persistent grid is
-// balanced here (prm.tail_*), *n_partials receives the number of slots.
+// Whether products run on pairs of SMs: pairs halve the traffic of B, but a pair's tile has
+// 256 rows.  So: where at least three quarters of the pairs get a tile, and padding M to 256 rows instead of 128 adds at most
+// a tenth.  (20 000 x 500 x 500: 43.2 us in pairs, 45.5 us without; x 2000 x 2000: 399 against 457 us; 2000 x 100 x 100, 8
+// pairs: 12.5 against 10.7 us.)
+template <class Epi>
+static bool use_pairs(const pdadmm_ctx *c, const Prod<Epi> *v, int n) {
+  int64_t single = 0, paired = 0;
+  for (int i = 0; i < n; ++i) {
+    const int64_t cols = ceil_div(v[i].N, TC_BN) * v[i].n_split;
+    single += ceil_div(v[i].M, TC_BM) * cols;
+    paired += 2 * ceil_div(v[i].M, 2 * TC_BM) * cols;
+  }
+  return paired * 10 <= single * 11 && (paired / 2) * 8 >= 3 * (int64_t)c->n_sms;
+}
+// op(A) is M x K, op(B) is N x K; A_MN: A is stored [K][M], B_MN: B is stored [K][N].  At most TC_MAX_GROUP products.
 template <int LAYOUT, class Epi, int ZERO = 0>
-static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Operand &A, const Operand &B, TcParams prm, const Epi &epi,
-                     double *partials, int *n_partials) {
+static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) {
   constexpr bool A_MN = (LAYOUT & TC_A_MN) != 0, B_MN = (LAYOUT & TC_B_MN) != 0;
-  const uint64_t M = (uint64_t)prm.M, N = (uint64_t)prm.N, K = (uint64_t)prm.K;
-  CUtensorMap maps[4];
-  PD_TRY(get_tmap(c, A.hi, A_MN ? M : K, A_MN ? K : M, (uint64_t)A.ld, &maps[0]));
-  if (A.lo && A.lo != A.hi) PD_TRY(get_tmap(c, A.lo, A_MN ? M : K, A_MN ? K : M, (uint64_t)A.ld, &maps[1]));
-  else maps[1] = maps[0];
-  PD_TRY(get_tmap(c, B.hi, B_MN ? N : K, B_MN ? K : N, (uint64_t)B.ld, &maps[2]));
-  if (B.lo && B.lo != B.hi) PD_TRY(get_tmap(c, B.lo, B_MN ? N : K, B_MN ? K : N, (uint64_t)B.ld, &maps[3]));
-  else maps[3] = maps[2];
-  prm.error = c->d_flag + 1;
-  prm.a = TcOperand{A.exp, A.check, A.x, A.ld};
-  prm.b = TcOperand{B.exp, B.check, B.x, B.ld};
-  const bool pair = use_pairs(c, prm.M, prm.N, prm.n_split);
-  const int n_tiles = (int)(ceil_div(prm.M, pair ? 2 * TC_BM : TC_BM) * ceil_div(prm.N, TC_BN)) * prm.n_split;
-  const int slots = pair ? c->n_sms / 2 : c->n_sms;          // tiles under way at a time
-  // The persistent grid works through the tiles in rounds; a last round that fills only part of the
-  // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit.
-  int n_units = n_tiles;
-  const int tail = n_tiles % slots, n_kb = (int)ceil_div(prm.K, TC_BK);
-  if (prm.n_split == 1 && tail > 0 && c->cur->tail_ws != nullptr) {
-    // at least 8 K blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks,
-    // and with two lanes the other layer's kernels fill the SMs that a short last round leaves idle (workload c2,
-    // 8 K blocks per tile: 281 iterations/s with 4 slices of 2 blocks, 289 without)
-    const int split = std::min(std::min(slots / tail, n_kb / 8), 8);
-    if (split > 1) {
-      prm.tail_begin = n_tiles - tail; prm.tail_split = split;
-      prm.tail_ws = c->cur->tail_ws; prm.tail_count = c->cur->tail_count;
-      n_units = prm.tail_begin + tail * split;
+  static_assert(sizeof(TcGroup<Epi>) <= 32000, "kernel parameters");
+  TcGroup<Epi> grp;
+  grp.n = n;
+  grp.error = c->d_flag + 1;
+  const bool pair = use_pairs(c, v, n);
+  int units = 0;
+  for (int i = 0; i < n; ++i) {
+    const Prod<Epi> &p = v[i];
+    TcLayer<Epi> &y = grp.l[i];
+    const uint64_t M = (uint64_t)p.M, N = (uint64_t)p.N, K = (uint64_t)p.K;
+    PD_TRY(get_tmap(c, p.A.hi, A_MN ? M : K, A_MN ? K : M, (uint64_t)p.A.ld, &y.a));
+    if (p.A.lo && p.A.lo != p.A.hi) PD_TRY(get_tmap(c, p.A.lo, A_MN ? M : K, A_MN ? K : M, (uint64_t)p.A.ld, &y.alo));
+    else y.alo = y.a;
+    PD_TRY(get_tmap(c, p.B.hi, B_MN ? N : K, B_MN ? K : N, (uint64_t)p.B.ld, &y.b));
+    if (p.B.lo && p.B.lo != p.B.hi) PD_TRY(get_tmap(c, p.B.lo, B_MN ? N : K, B_MN ? K : N, (uint64_t)p.B.ld, &y.blo));
+    else y.blo = y.b;
+    y.M = p.M; y.N = p.N; y.K = p.K;
+    y.k_chunk = p.n_split > 1 ? p.k_chunk : round_up(p.K, TC_BK);
+    y.n_split = p.n_split;
+    y.c_split_stride = p.stride;
+    y.oa = TcOperand{p.A.exp, p.A.check, p.A.x, p.A.ld};
+    y.ob = TcOperand{p.B.exp, p.B.check, p.B.x, p.B.ld};
+    y.mul = p.A.int_mul > 0.f ? p.A.int_mul : (p.B.int_mul > 0.f ? p.B.int_mul : 1.f);
+    y.epi = p.epi;
+    y.slots = p.slots; y.done = p.done; y.step = p.step;
+    y.tail_begin = 0; y.tail_split = 0; y.tail_ws = nullptr; y.tail_count = nullptr;
+    const int n_tiles = (int)(ceil_div(p.M, pair ? 2 * TC_BM : TC_BM) * ceil_div(p.N, TC_BN)) * p.n_split;
+    units += n_tiles;
+    // The persistent grid works through the tiles in rounds; a last round that fills only part of the
+    // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit (at least 8 K
+    // blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks).
+    const int slots = pair ? c->n_sms / 2 : c->n_sms, tail = n_tiles % slots;
+    if (c->tail_split && n == 1 && p.n_split == 1 && tail > 0 && p.s != nullptr && p.s->tail_ws != nullptr) {
+      const int split = std::min(std::min(slots / tail, (int)ceil_div(p.K, TC_BK) / 8), 8);
+      if (split > 1) {
+        y.tail_begin = n_tiles - tail; y.tail_split = split;
+        y.tail_ws = p.s->tail_ws; y.tail_count = p.s->tail_count;
+        units = y.tail_begin + tail * split;
+      }
     }
+    y.unit_end = units;
   }
-  if (n_partials) {
-    const int blocks = pair ? 2 * std::min(n_units, slots) : std::min(n_units, slots);
-    *n_partials = TC_ACC_WARPS * (blocks + (prm.tail_split > 1 ? (pair ? 2 : 1) * (n_tiles - prm.tail_begin) : 0));
-  }
-  if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, maps, prm, epi, partials, n_units);
-  return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, maps, prm, epi, partials, n_units);
+  if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, grp);
+  return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, grp);
 }
 
 // ---- largest magnitudes of product operands ------------------------------------------------------------------
@@ -479,13 +509,21 @@ static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t ro
 // Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel).
 // From 2^20 elements on: below, the launch costs more than it saves.
 constexpr size_t CHECK_PLANES_FROM = size_t(1) << 20;
-static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, Operand &o) {
-  const size_t n = rows * o.ld;
-  if (!c->use_tc || o.hi == nullptr || o.check == nullptr || o.x == nullptr || n < CHECK_PLANES_FROM) return;
+static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, const std::vector<Operand *> &ops) {
+  Group<PlaneCheck> g;
+  int n = 0;
+  uint32_t n8_max = 0;
+  for (Operand *o : ops) {
+    const size_t e = rows * o->ld;
+    if (!c->use_tc || o->hi == nullptr || o->check == nullptr || o->x == nullptr || e < CHECK_PLANES_FROM) continue;
+    g.l[n++] = PlaneCheck{o->x, (uint32_t)(e / 8), o->check, o->exp, const_cast<__half *>(o->hi),
+                          o->lo == o->hi ? nullptr : const_cast<__half *>(o->lo)};
+    n8_max = std::max(n8_max, (uint32_t)(e / 8));
+    o->x = nullptr;
+  }
+  if (n == 0) return;
   Launch l(c, KC_PLANES, st, 0, 0);
-  launch_first(st, check_planes_kernel, dim3(ew_grid(n / 8)), 256, 0, o.x, n / 8, o.check, o.exp, const_cast<__half *>(o.hi),
-                                                     o.lo == o.hi ? nullptr : const_cast<__half *>(o.lo));
-  o.x = nullptr;
+  launch_first(st, check_planes_kernel, dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, g);
 }
 static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
   PD_TRY(dev_alloc(c, &pl->hi, n, zero));
@@ -506,58 +544,85 @@ static int refresh_W_planes(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
 }
 
 // ---- dense products --------------------------------------------------------------------------------------
-// C[M][N] = A[M][K] * op(B), fused epilogue; per-block sums of squares go to `partials` (or nullptr).
-// B_MN = false: B is [N][K]; true: B is [K][N].  An operand A without planes is split into the lane's pl1 first
-// (8 bytes per element; splitting inside the product, once per column tile, ran the MMAs at 0.6 of their speed).
+// C[M][N] = A[M][K] * op(B) for several layers, fused epilogue.  B_MN = false: B is [N][K]; true: B is [K][N].  An operand A without
+// planes is split into its layer's pl1 first (8 bytes per element; splitting inside the product, once per column tile, ran
+// the MMAs at 0.6 of their speed).  bytes: what the epilogues move beside the operands and the output.
 template <bool B_MN, class Epi>
-static int gemm_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, Operand A, const Operand &B, const Epi &epi,
-                      double *partials, int *n_partials, double extra_bytes) {
-  const double bytes = 4.0 * ((double)M * K + (double)N * K + (double)M * N) + extra_bytes;
+static int gemm_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, std::vector<Prod<Epi>> v, double extra_bytes) {
+  if (v.empty()) return PDADMM_OK;
+  double bytes = extra_bytes, flops = 0;
+  for (const Prod<Epi> &p : v) {
+    bytes += 4.0 * ((double)p.M * p.K + (double)p.N * p.K + (double)p.M * p.N);
+    flops += 2.0 * p.M * p.N * p.K;
+  }
   if (!c->use_tc) {
-    dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM));
-    if (n_partials) *n_partials = (int)(grid.x * grid.y);
-    Launch l(c, cls, st, bytes, 2.0 * M * N * K);
-    gemm_nt_kernel<B_MN, Epi><<<grid, SG_THREADS, 0, st>>>(M, N, K, A.x, A.ld, B.x, B.ld, epi, partials);
+    for (const Prod<Epi> &p : v) {
+      dim3 grid((unsigned)ceil_div(p.N, SG_BN), (unsigned)ceil_div(p.M, SG_BM));
+      {
+        Launch l(c, cls, st, bytes / v.size(), 2.0 * p.M * p.N * p.K);
+        gemm_nt_kernel<B_MN, Epi><<<grid, SG_THREADS, 0, st>>>(p.M, p.N, p.K, p.A.x, p.A.ld, p.B.x, p.B.ld, p.epi, p.slots);
+      }
+      if (p.slots == nullptr) continue;
+      Launch l(c, KC_SMALL, st, 8.0 * grid.x * grid.y, 0);
+      launch_first(st, finish_sum_kernel, dim3(1), FIN_THREADS, 0, p.slots, (int)(grid.x * grid.y), p.step);
+    }
     return PDADMM_OK;
   }
-  if (A.hi == nullptr) {
-    Scratch &sc = *c->cur;
-    if ((size_t)M * A.ld > sc.pl_cap || A.ld % 8) return fail(PDADMM_EINVAL, "operand does not fit the lane's planes");
-    if (A.amax == nullptr) {
+  for (Prod<Epi> &p : v) {
+    if (p.A.hi != nullptr) continue;
+    Scratch &sc = *p.s;
+    if ((size_t)p.M * p.A.ld > sc.pl_cap || p.A.ld % 8) return fail(PDADMM_EINVAL, "operand does not fit the lane's planes");
+    if (p.A.amax == nullptr) {
       PD_TRY(amax_reserve(c, st, 1));
-      A.amax = amax_of(c, st, A.x, (size_t)M * A.ld / 4);
+      p.A.amax = amax_of(c, st, p.A.x, (size_t)p.M * p.A.ld / 4);
     }
     const Planes pl{sc.pl1.hi, sc.pl1.lo, sc.a_exp};
-    split_rows(c, st, A.x, (size_t)M, K, A.ld, A.amax, pl, !epi_coarse<Epi>::value);
-    A.hi = pl.hi; A.lo = pl.lo; A.exp = pl.exp; A.check = nullptr;
+    split_rows(c, st, p.A.x, (size_t)p.M, p.K, p.A.ld, p.A.amax, pl, !epi_coarse<Epi>::value);
+    p.A.hi = pl.hi; p.A.lo = pl.lo; p.A.exp = pl.exp; p.A.check = nullptr;
   }
-  TcParams prm = {};
-  prm.M = M; prm.N = N; prm.K = K; prm.k_chunk = round_up(K, TC_BK); prm.n_split = 1; prm.mul = 1.f;
   constexpr int LAYOUT = B_MN ? TC_B_MN : TC_NT;
-  Launch l(c, cls, st, bytes, 2.0 * M * N * K);
-  if (A.int_mul > 0.f) {
-    if constexpr (std::is_same<Epi, EpiStoreSumsq>::value || std::is_same<Epi, EpiAddSumsq>::value) {
-      prm.mul = A.int_mul;
-      return launch_tc<LAYOUT, Epi, 1>(c, st, A, B, prm, epi, partials, n_partials);
+  constexpr bool INT_FORM = std::is_same<Epi, EpiStoreSumsq>::value || std::is_same<Epi, EpiAddSumsq>::value;
+  // operands of integers and others take different kernels
+  const auto mid = std::stable_partition(v.begin(), v.end(), [](const Prod<Epi> &p) { return p.A.int_mul <= 0.f; });
+  const int n = (int)(mid - v.begin()), n_int = (int)(v.end() - mid);
+  if (n > 0) {
+    Launch l(c, cls, st, bytes * n / (n + n_int), flops * n / (n + n_int));
+    PD_TRY((launch_tc<LAYOUT, Epi>(c, st, v.data(), n)));
+  }
+  if (n_int > 0) {
+    if constexpr (INT_FORM) {
+      Launch l(c, cls, st, bytes * n_int / (n + n_int), flops * n_int / (n + n_int));
+      PD_TRY((launch_tc<LAYOUT, Epi, 1>(c, st, v.data() + n, n_int)));
     } else {
       return fail(PDADMM_EINVAL, "no integer-operand form of this product is built");
     }
   }
-  return launch_tc<LAYOUT, Epi>(c, st, A, B, prm, epi, partials, n_partials);
+  return PDADMM_OK;
 }
 
-// C parts [n_split][M][ldc] = A^T B over node slices, A = [K nodes][M], B = [K nodes][N], both as planes
-static int gemm_over_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, int M, int N, int K, const Operand &A, const Operand &B,
-                           float *part, int ldc, int k_chunk, int n_split) {
-  TcParams prm = {};
-  prm.M = M; prm.N = N; prm.K = K; prm.k_chunk = k_chunk; prm.n_split = n_split; prm.c_split_stride = (size_t)M * ldc; prm.mul = 1.f;
-  EpiStore epi{part, ldc};
-  Launch k(c, cls, st, 4.0 * ((double)K * N + (double)K * M), 2.0 * K * N * M);
-  if (B.int_mul > 0.f) {
-    prm.mul = B.int_mul;
-    return launch_tc<TC_A_MN | TC_B_MN, EpiStore, 2>(c, st, A, B, prm, epi, nullptr, nullptr);
+// C parts [n_split][M][ldc] = A^T B over node slices, A = [K nodes][M], B = [K nodes][N], both as planes, for several layers
+static int gemm_over_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, std::vector<Prod<EpiStore>> v) {
+  const auto mid = std::stable_partition(v.begin(), v.end(), [](const Prod<EpiStore> &p) { return p.B.int_mul <= 0.f; });
+  const int n = (int)(mid - v.begin()), n_int = (int)(v.end() - mid);
+  auto count = [&](int i0, int i1, double &bytes, double &flops) {
+    bytes = flops = 0;
+    for (int i = i0; i < i1; ++i) {
+      bytes += 4.0 * ((double)v[i].K * v[i].N + (double)v[i].K * v[i].M);
+      flops += 2.0 * v[i].K * v[i].N * v[i].M;
+    }
+  };
+  double bytes, flops;
+  if (n > 0) {
+    count(0, n, bytes, flops);
+    Launch k(c, cls, st, bytes, flops);
+    PD_TRY((launch_tc<TC_A_MN | TC_B_MN, EpiStore>(c, st, v.data(), n)));
   }
-  return launch_tc<TC_A_MN | TC_B_MN, EpiStore>(c, st, A, B, prm, epi, nullptr, nullptr);
+  if (n_int > 0) {
+    count(n, n + n_int, bytes, flops);
+    Launch k(c, cls, st, bytes, flops);
+    PD_TRY((launch_tc<TC_A_MN | TC_B_MN, EpiStore, 2>(c, st, v.data() + n, n_int)));
+  }
+  return PDADMM_OK;
 }
 
 // ---- pieces of one iteration -------------------------------------------------------------------------------
@@ -572,14 +637,37 @@ static Operand operand_r(const Layer &ly) {
   return o;
 }
 
+// The layers of a batch are consecutive, at most MAX_GROUP, and share a stream; layer l uses scratch l mod the number of them.
+typedef std::vector<int> Batch;
+static Scratch &lane(pdadmm_ctx *c, int i) { return i == 0 ? c->scr : *c->more_lanes[i - 1]; }
+static Scratch &scratch_of(pdadmm_ctx *c, int l) { return lane(c, l % c->n_active); }
+static PlaneOut plane_out(pdadmm_ctx *c, const Planes &p) {
+  return c->use_tc ? PlaneOut{p.hi, p.lo, p.exp} : PlaneOut{nullptr, nullptr, nullptr};
+}
+static Step make_step(pdadmm_ctx *c, Layer &ly, int kind) {
+  Step t;
+  t.kind = kind;
+  t.sc = ly.sc; t.rho = c->rho; t.nu = c->nu; t.nonfinite = c->d_flag + 2;
+  t.apply = kind != STEP_G2 && c->reduce == nullptr;     // a sharded context adds the sums over the shards first
+  if (c->use_tc) { t.amax_p = ly.amax_p; t.amax_r = ly.amax_r; t.amax_W = ly.amax_W; }
+  return t;
+}
+// The sums at `sums` are those of this shard: add them over the shards, then the step.
+static int shard_step(pdadmm_ctx *c, cudaStream_t st, double *sums, size_t n, const Step &t) {
+  if (c->reduce == nullptr) return PDADMM_OK;
+  PD_TRY(shard_sum(c, st, sums, n, 1));
+  run_step_kernel<<<1, 1, 0, st>>>(t);
+  return PDADMM_OK;
+}
+
 // r_l = P_l W_l^T + b_l - z_l from scratch (only when the cached residual is not valid).
 static int refresh_residual(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
   PD_CUDA(cudaMemsetAsync(ly.amax_r, 0, sizeof(uint32_t), st));
   EpiLinearResidual epi{ly.r, ly.ld_out, ly.b, ly.z, ly.amax_r};
   Operand P{ly.p, ly.ld_in, ly.amax_p};
   if (c->use_tc && ly.xp.hi != nullptr) P = operand_X(ly);
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)c->N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr,
-                           4.0 * c->N * ly.n_out));
+  PD_TRY((gemm_nodes<false, EpiLinearResidual>(c, KC_GEMM_RESID, st, {{(int)c->N, ly.n_out, ly.n_in, P, operand_W(ly), epi, &c->scr}},
+                                               4.0 * c->N * ly.n_out)));
   if (!c->use_tc) {       // the CUDA-core product does not track the maximum of what it stores
     Launch l(c, KC_AMAX, st, 4.0 * c->N * ly.ld_out, 0);
     absmax_kernel<<<ew_grid((size_t)c->N * ly.ld_out / 4), EW_THREADS, 0, st>>>(ly.r, (size_t)c->N * ly.ld_out / 4, ly.amax_r);
@@ -589,310 +677,435 @@ static int refresh_residual(pdadmm_ctx *c, Layer &ly, cudaStream_t st) {
   return PDADMM_OK;
 }
 
-// g = nu r W + u_{l-1} + rho (p - q_{l-1}) -> s1, ||g||^2 ; W g -> s2, ||W g||^2 ; tau.
-static int p_gradient_and_tau(pdadmm_ctx *c, int l /*0-based, >= 1*/) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
+// Layers 2..L (0-based l >= 1): g = nu r W + u_{l-1} + rho (p - q_{l-1}) -> s1, ||g||^2 ; W g -> s2, ||W g||^2 ; tau.
+static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const int N = (int)c->N;
-  int np = 0;
   const bool norm_only = c->levels && c->use_tc;     // the quantised update only needs ||W g||^2 (for the first tau); its
                                                      // residual update uses W d
-  uint32_t *w_g = nullptr, *w_wg = nullptr;          // max|g|, max|W g|, kept by the epilogues that write them
-  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 2)); w_g = amax_take(c); w_wg = amax_take(c); }
-  // The epilogue that writes g writes its planes too (the hi plane alone for the norm-only product), scaled by an exponent
-  // predicted from the previous iteration's max|g|: the true one is known only when the product has finished.
-  EpiGradT epi{s.s1, ly.ld_in, ly.t, c->nu, w_g};
-  Operand G{s.s1, ly.ld_in, w_g};
-  if (c->use_tc) {
-    epi.H = s.pl0.hi; epi.L = norm_only ? nullptr : s.pl0.lo; epi.h_exp = ly.g_exp;
-    G = plane_operand(s.s1, ly.ld_in, Planes{s.pl0.hi, norm_only ? s.pl0.hi : s.pl0.lo, ly.g_exp}, w_g);
+  std::vector<Operand> R, G;
+  std::vector<Prod<EpiGradT>> grad;
+  double bytes = 0;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    Scratch &s = scratch_of(c, l);
+    R.push_back(operand_r(ly));
+    // The epilogue that writes g writes its planes too (the hi plane alone for the norm-only product), scaled by an exponent
+    // predicted from the previous iteration's max|g|: the true one is known only when the product has finished.
+    EpiGradT epi{s.s1, ly.ld_in, ly.t, c->nu, c->use_tc ? ly.w_g : nullptr};
+    if (c->use_tc) {
+      epi.H = s.pl0.hi; epi.L = norm_only ? nullptr : s.pl0.lo; epi.h_exp = ly.g_exp;
+      G.push_back(plane_operand(s.s1, ly.ld_in, Planes{s.pl0.hi, norm_only ? s.pl0.hi : s.pl0.lo, ly.g_exp}, ly.w_g));
+    } else {
+      G.push_back(Operand{s.s1, ly.ld_in, nullptr});
+    }
+    Prod<EpiGradT> p{N, ly.n_in, ly.n_out, R.back(), operand_W(ly), epi, &s, s.slots, ly.done};
+    p.step = make_step(c, ly, STEP_G2);
+    grad.push_back(p);
+    bytes += (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in;
   }
-  Operand R = operand_r(ly);
-  check_planes(c, s.st, (size_t)N, R);
-  PD_TRY(gemm_nodes<true>(c, KC_GEMM_GRADP, s.st, N, ly.n_in, ly.n_out, R, operand_W(ly), epi, s.slots, &np,
-                          (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in));
-  check_planes(c, s.st, (size_t)N, G);
-  int np2 = 0;
-  double *slots_b = s.slots + s.n_slots / 2;          // second half of the slot buffer
-  if (norm_only) {
-    EpiNormOnly epi2{s.s2, ly.ld_out};
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, G, operand_W(ly), epi2, slots_b, &np2, 0));
-  } else {
-    EpiStoreSumsq epi2{s.s2, ly.ld_out, w_wg};
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, G, operand_W(ly), epi2, slots_b, &np2, 0));
-  }
-  TauPlanes t{};
-  if (c->use_tc) {
-    t = TauPlanes{ly.amax_p, ly.amax_r, w_g, norm_only ? nullptr : w_wg, norm_only ? nullptr : s.pl1.exp, s.pl0.exp, ly.g_exp};
-  }
-  if (c->reduce != nullptr) {
-    // ||g||^2 and ||W g||^2 are sums over nodes: this shard's totals, added over the shards, then tau
-    PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, np, slots_b, np2));
-    launch_first(s.st, finalize_tau_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, s.red, 1, s.red + 1, 1, c->d_flag + 2, t);
+  auto check = [&](std::vector<Operand> &ops) {
+    std::vector<Operand *> v;
+    for (Operand &o : ops) v.push_back(&o);
+    check_planes(c, st, (size_t)N, v);
+  };
+  check(R);
+  for (size_t i = 0; i < batch.size(); ++i) grad[i].A = R[i];
+  PD_TRY((gemm_nodes<true, EpiGradT>(c, KC_GEMM_GRADP, st, grad, bytes)));
+  check(G);
+  auto wg = [&](auto make_epi) -> int {
+    std::vector<Prod<decltype(make_epi(0))>> v;
+    for (size_t i = 0; i < batch.size(); ++i) {
+      Layer &ly = c->layers[batch[i]];
+      Scratch &s = scratch_of(c, batch[i]);
+      Prod<decltype(make_epi(0))> p{N, ly.n_out, ly.n_in, G[i], operand_W(ly), make_epi(batch[i]), &s, s.slots + s.n_slots / 2, ly.done};
+      Step t = make_step(c, ly, STEP_TAU);
+      if (c->use_tc) {
+        t.w_in = ly.w_g; t.w_out = norm_only ? nullptr : ly.w_wg;
+        t.exp_p = norm_only ? nullptr : s.pl1.exp; t.exp_r = s.pl0.exp; t.exp_g = ly.g_exp;
+      }
+      p.step = t;
+      v.push_back(p);
+    }
+    PD_TRY((gemm_nodes<false>(c, KC_GEMM_WG, st, v, 0)));
+    // ||g||^2 and ||W g||^2 are sums over nodes
+    for (size_t i = 0; i < batch.size(); ++i) PD_TRY(shard_step(c, st, &c->layers[batch[i]].sc->sum_g2, 2, v[i].step));
     return PDADMM_OK;
-  }
-  Launch k(c, KC_SMALL, s.st, 8.0 * (np + np2), 0);
-  launch_first(s.st, finalize_tau_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, s.slots, np, slots_b, np2, c->d_flag + 2, t);
-  return PDADMM_OK;
-}
-
-static PlaneOut plane_out(pdadmm_ctx *c, const Planes &p) {
-  return c->use_tc ? PlaneOut{p.hi, p.lo, p.exp} : PlaneOut{nullptr, nullptr, nullptr};
+  };
+  if (norm_only) return wg([&](int l) { return EpiNormOnly{scratch_of(c, l).s2, c->layers[l].ld_out}; });
+  return wg([&](int l) { return EpiStoreSumsq{scratch_of(c, l).s2, c->layers[l].ld_out, c->use_tc ? c->layers[l].w_wg : nullptr}; });
 }
 
 // pdADMM-G: p <- p - g/tau, r <- r - (W g)/tau, and the planes of both.
-static void p_step_plain(pdadmm_ctx *c, int l) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
-  const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
-  Launch k(c, KC_AXPY, s.st, (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out), 0);
-  launch_first(s.st, pstep_kernel, dim3(ew_grid(std::max(n4p, n4r))), EW_THREADS, 0, 
-      ly.p, s.s1, n4p, ly.r, s.s2, n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0), c->use_tc ? ly.amax_p : nullptr,
-      c->use_tc ? ly.amax_r : nullptr);
+static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
+  Group<PStep> g;
+  int n = 0, blocks = 0;
+  double bytes = 0;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    Scratch &s = scratch_of(c, l);
+    const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
+    const int nb = ew_grid(std::max(n4p, n4r));
+    g.l[n++] = PStep{ly.p, s.s1, (uint32_t)n4p, ly.r, s.s2, (uint32_t)n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0),
+                     c->use_tc ? ly.amax_p : nullptr, c->use_tc ? ly.amax_r : nullptr, nb};
+    blocks = std::max(blocks, nb);
+    bytes += (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out);
+  }
+  Launch k(c, KC_AXPY, st, bytes, 0);
+  launch_first(st, pstep_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
-// with a copy of the accept flag to the host, which decides whether another trial is needed (the only host round
-// trips of an iteration).  The two halves below let the caller queue another layer's work on the other lane before
-// it waits for the flag.
-// One trial: trial p, d = trial p - p and its codes, W d with its squared norm, the accept test, the flag's copy.
-static int q_trial(pdadmm_ctx *c, int l) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
+// with the accept flags on the host, which decides whether another trial is needed (the only host round
+// trips of an iteration).
+// One trial of some layers: trial p, d = trial p - p and its codes, W d with its squared norm, the accept test, the flag.
+static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const int N = (int)c->N;
-  const size_t n4p = (size_t)N * ly.ld_in / 4;
-  const int grid = ew_grid(n4p);
-  uint32_t *w_d = nullptr;               // max|d| of this trial
-  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 1)); w_d = amax_take(c); }
   {
-    // reads g and the codes of p; writes p+, the new codes and d -- as fp32, or, with integer operands, as the two
-    // fp16 planes of integers: 14 bytes per element with one-byte codes either way
-    Launch k(c, KC_QUANT, s.st, 14.0 * N * ly.n_in, 0);
-    launch_first(s.st, quant_trial_kernel, dim3(grid), EW_THREADS, 0, s.s1, ly.sc, ly.scale, ly.lo, c->levels, s.p_new,
-                                                     c->int_operands ? nullptr : s.d,
-                                                     s.codes_new, c->code_bytes == 2, n4p, s.slots,
-                                                     c->use_tc ? ly.amax_p : nullptr, w_d,
-                                                     ly.codes, s.pn_plane, s.d_plane);
+    Group<QuantTrial> g;
+    int n = 0, blocks = 0;
+    double bytes = 0;
+    for (int l : batch) {
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      const size_t n4 = (size_t)N * ly.ld_in / 4;
+      const int nb = ew_grid(n4);
+      // with integer operands p+ and d exist as codes and planes of integers alone
+      g.l[n++] = QuantTrial{s.s1, ly.sc, ly.scale, ly.lo, c->int_operands ? nullptr : s.p_new, c->int_operands ? nullptr : s.d, ly.codes,
+                            s.codes_new, s.pn_plane, s.d_plane, (uint32_t)n4, c->use_tc && !c->int_operands ? ly.amax_p : nullptr,
+                            ly.w_d, s.slots, ly.done + 1, nb};
+      blocks = std::max(blocks, nb);
+      bytes += (c->int_operands ? 8.0 + 2.0 * c->code_bytes : 12.0 + 2.0 * c->code_bytes) * N * ly.n_in;
+    }
+    Launch k(c, KC_QUANT, st, bytes, 0);
+    launch_first(st, quant_trial_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->levels, c->code_bytes == 2,
+                 c->neg_levels);
   }
-  int np = 0;
-  double *slots_b = s.slots + s.n_slots / 2;
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
   // max|r| takes the trial's values too, which keeps it an upper bound whether or not the trial is taken
-  EpiAddSumsq epi{s.s2, ly.ld_out, ly.r, c->use_tc ? ly.amax_r : nullptr};
-  if (c->use_tc) { epi.H = s.pl0.hi; epi.L = s.pl0.lo; epi.h_exp = s.pl0.exp; }      // planes of the trial's r for the W-gradient
-  const Operand D = c->int_operands ? int_operand(s.d_plane, ly.ld_in, ly.scale)      // d = (new code - old code) s
-                                    : Operand{s.d, ly.ld_in, w_d};
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, s.st, N, ly.n_out, ly.n_in, D, operand_W(ly), epi, slots_b, &np,
-                           (c->use_tc ? 8.0 : 4.0) * N * ly.n_out));
-  if (c->reduce != nullptr) {
-    PD_TRY(shard_sum_slots(c, s.st, s.red, s.slots, grid, slots_b, np));
-    launch_first(s.st, finalize_trial_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.red, 1, s.red + 1, 1);
-  } else {
-    Launch k(c, KC_SMALL, s.st, 8.0 * (grid + np), 0);
-    launch_first(s.st, finalize_trial_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->rho, (double)c->nu, 1e-6, s.slots, grid, slots_b, np);
+  std::vector<Prod<EpiAddSumsq>> v;
+  double bytes = 0;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    Scratch &s = scratch_of(c, l);
+    EpiAddSumsq epi{s.s2, ly.ld_out, ly.r, c->use_tc ? ly.amax_r : nullptr};
+    if (c->use_tc) { epi.H = s.pl0.hi; epi.L = s.pl0.lo; epi.h_exp = s.pl0.exp; }      // planes of the trial's r for the W-gradient
+    const Operand D = c->int_operands ? int_operand(s.d_plane, ly.ld_in, ly.scale)      // d = (new code - old code) s
+                                      : Operand{s.d, ly.ld_in, c->use_tc ? ly.w_d : nullptr};
+    Prod<EpiAddSumsq> p{N, ly.n_out, ly.n_in, D, operand_W(ly), epi, &s, s.slots + s.n_slots / 2, ly.done};
+    p.step = make_step(c, ly, STEP_TRIAL);
+    p.step.w_in = c->use_tc && !c->int_operands ? ly.w_d : nullptr;
+    p.step.host_flag = s.h_flag;
+    *s.h_flag = 0;
+    v.push_back(p);
+    bytes += (c->use_tc ? 8.0 : 4.0) * N * ly.n_out;
   }
-  PD_CUDA(cudaMemcpyAsync(s.h_flag, &ly.sc->accepted, sizeof(int), cudaMemcpyDeviceToHost, s.st));
-  PD_CUDA(cudaEventRecord(s.ev_flag, s.st));
+  PD_TRY((gemm_nodes<false>(c, KC_GEMM_WG, st, v, bytes)));
+  for (size_t i = 0; i < batch.size(); ++i) PD_TRY(shard_step(c, st, &c->layers[batch[i]].sc->sum_d2, 2, v[i].step));
+  PD_CUDA(cudaEventRecord(scratch_of(c, batch[0]).ev_flag, st));
   return PDADMM_OK;
 }
-// After the first trial of layer l was queued on the current lane: wait for its flag, run further trials while it
-// says no, then take the trial: p, codes <- trial, r <- r + W d.
-static int q_finish(pdadmm_ctx *c, int l, bool *hit_cap) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
+// After the first trial of a batch was queued: wait for the flags, run further trials of the layers that say no, then take the
+// trials: p, codes <- trial, r <- r + W d.
+static int q_finish(pdadmm_ctx *c, cudaStream_t st, const Batch &batch, bool *hit_cap) {
   const int max_trials = 30;
+  Batch open = batch;
   for (int trial = 0;; ++trial) {
-    PD_CUDA(cudaEventSynchronize(s.ev_flag));
-    if (*s.h_flag || trial + 1 >= max_trials) {
-      if (!*s.h_flag) *hit_cap = true;
-      break;
-    }
-    PD_TRY(q_trial(c, l));
+    PD_CUDA(cudaEventSynchronize(scratch_of(c, open[0]).ev_flag));
+    Batch refused;
+    for (int l : open)
+      if (!*scratch_of(c, l).h_flag) refused.push_back(l);
+    if (refused.empty()) break;
+    if (trial + 1 >= max_trials) { *hit_cap = true; break; }
+    PD_TRY(q_trial(c, st, refused));
+    open = refused;
   }
-  std::swap(ly.p, s.p_new);
-  std::swap(ly.codes, s.codes_new);
-  std::swap(ly.p_plane, s.pn_plane);
-  std::swap(ly.r, s.s2);                // r <- r + W d, written by the trial's product
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    Scratch &s = scratch_of(c, l);
+    if (!c->int_operands) std::swap(ly.p, s.p_new);
+    std::swap(ly.codes, s.codes_new);
+    std::swap(ly.p_plane, s.pn_plane);
+    std::swap(ly.r, s.s2);                // r <- r + W d, written by the trial's product
+  }
+  if (c->int_operands) c->p_stale = true;
   return PDADMM_OK;
 }
 
 // G = nu r^T p+ (contraction over nodes), theta, W <- W - G/theta, r <- r - (G p+)/theta,
 // b <- b - mean_j r, shift = mean_j r.
-static int w_and_b_step(pdadmm_ctx *c, int l) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
+static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const int N = (int)c->N;
   // p+ (layer 1: X, which never changes; pdADMM-G: planes from the p-step; pdADMM-G-Q: p+ = code * s)
-  Operand P{ly.p, ly.ld_in, ly.amax_p};
-  if (c->use_tc) P = l == 0 ? operand_X(ly) : (c->int_operands ? int_operand(ly.p_plane, ly.ld_in, ly.scale)
-                                                               : plane_operand(ly.p, ly.ld_in, s.pl1, ly.amax_p));
+  std::vector<Operand> P, R;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    Scratch &s = scratch_of(c, l);
+    if (!c->use_tc) {
+      P.push_back(Operand{ly.p, ly.ld_in, nullptr});
+      R.push_back(Operand{ly.r, ly.ld_out, nullptr});
+      continue;
+    }
+    P.push_back(l == 0 ? operand_X(ly) : c->int_operands ? int_operand(ly.p_plane, ly.ld_in, ly.scale)
+                                                          : plane_operand(ly.p, ly.ld_in, s.pl1, ly.amax_p));
+    R.push_back(l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, ly.amax_r));
+  }
   if (!c->use_tc) {
-    dim3 grid((unsigned)ceil_div(ly.n_in, SG_BN), (unsigned)ceil_div(ly.n_out, SG_BM), (unsigned)ly.n_split);
-    Launch k(c, KC_GEMM_GRADW, s.st, 4.0 * ((double)N * ly.n_in + (double)N * ly.n_out), 2.0 * N * ly.n_in * ly.n_out);
-    gemm_tn_kernel<<<grid, SG_THREADS, 0, s.st>>>(ly.n_out, ly.n_in, N, ly.k_chunk, ly.r, ly.ld_out, ly.p, ly.ld_in,
-                                                 s.part, ly.ld_in);
+    for (int l : batch) {
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      dim3 grid((unsigned)ceil_div(ly.n_in, SG_BN), (unsigned)ceil_div(ly.n_out, SG_BM), (unsigned)ly.n_split);
+      Launch k(c, KC_GEMM_GRADW, st, 4.0 * ((double)N * ly.n_in + (double)N * ly.n_out), 2.0 * N * ly.n_in * ly.n_out);
+      gemm_tn_kernel<<<grid, SG_THREADS, 0, st>>>(ly.n_out, ly.n_in, N, ly.k_chunk, ly.r, ly.ld_out, ly.p, ly.ld_in, s.part, ly.ld_in);
+    }
   } else {
     // both operands are node-major; the product contracts over the rows of their planes as they are
-    Operand R = l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, ly.amax_r);
-    if (l == 0 || c->levels) check_planes(c, s.st, (size_t)N, R);      // (the p-step's planes are scaled by a bound)
-    if (R.hi == nullptr) {                       // no room was left for the planes of r
-      const Planes pl{s.pl0.hi, s.pl0.lo, s.a_exp};
-      split_rows(c, s.st, ly.r, (size_t)N, ly.n_out, ly.ld_out, ly.amax_r, pl);
-      R = plane_operand(ly.r, ly.ld_out, pl);
+    std::vector<Operand *> to_check;
+    std::vector<Prod<EpiStore>> v;
+    for (size_t i = 0; i < batch.size(); ++i) {
+      const int l = batch[i];
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      if (l == 0 || c->levels) to_check.push_back(&R[i]);       // (the p-step's planes are scaled by a bound)
+      if (R[i].hi == nullptr) {                                 // no room was left for the planes of r
+        const Planes pl{s.pl0.hi, s.pl0.lo, s.a_exp};
+        split_rows(c, st, ly.r, (size_t)N, ly.n_out, ly.ld_out, ly.amax_r, pl);
+        R[i] = plane_operand(ly.r, ly.ld_out, pl);
+      }
+      if (l > 0 && c->levels && !c->int_operands)               // p+ on a level set without integer planes
+        split_rows(c, st, ly.p, (size_t)N, ly.n_in, ly.ld_in, ly.amax_p, s.pl1);
     }
-    if (l > 0 && c->levels && !c->int_operands)  // p+ on a level set without integer planes
-      split_rows(c, s.st, ly.p, (size_t)N, ly.n_in, ly.ld_in, ly.amax_p, s.pl1);
-    PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, s.st, ly.n_out, ly.n_in, N, R, P, s.part, ly.ld_in, ly.k_chunk, ly.n_split));
+    check_planes(c, st, (size_t)N, to_check);
+    for (size_t i = 0; i < batch.size(); ++i) {
+      Layer &ly = c->layers[batch[i]];
+      Scratch &s = scratch_of(c, batch[i]);
+      Prod<EpiStore> p{ly.n_out, ly.n_in, N, R[i], P[i], EpiStore{s.part, ly.ld_in}, &s};
+      p.n_split = ly.n_split; p.k_chunk = ly.k_chunk; p.stride = (size_t)ly.n_out * ly.ld_in;
+      v.push_back(p);
+    }
+    PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, v));
   }
-  const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
-  const int gw = ew_grid(n4w);
-  uint32_t *w_G = nullptr;                       // max|G|
-  if (c->use_tc) { PD_TRY(amax_reserve(c, s.st, 2)); w_G = amax_take(c); }
   {
-    Launch k(c, KC_GRADW_REDUCE, s.st, (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in, 0);
-    // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
-    launch_first(s.st, reduce_gradW_kernel, dim3(gw), EW_THREADS, 0, s.part, ly.n_split, n4w, c->nu, ly.gradW, w_G, s.slots,
-                                                     c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp));
+    Group<GradWSum> g;
+    int n = 0, blocks = 0;
+    double bytes = 0;
+    for (int l : batch) {
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      const size_t n4 = (size_t)ly.n_out * ly.ld_in / 4;
+      const int nb = ew_grid(n4);
+      // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
+      g.l[n++] = GradWSum{s.part, ly.n_split, (uint32_t)n4, ly.gradW, c->use_tc ? ly.w_G : nullptr,
+                          c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp), s.slots, ly.done + 2,
+                          &ly.sc->sum_G2, nb};
+      blocks = std::max(blocks, nb);
+      bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
+    }
+    Launch k(c, KC_GRADW_REDUCE, st, bytes, 0);
+    launch_first(st, reduce_gradW_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->nu);
   }
   if (c->reduce != nullptr) {
     // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
-    PD_TRY(shard_sum(c, s.st, ly.gradW, n4w * 4, 0));
-    if (c->use_tc) w_G = amax_take(c);
-    launch_first(s.st, sumsq_amax_kernel, dim3(gw), EW_THREADS, 0, ly.gradW, n4w, w_G, s.slots);
-    if (c->use_tc) split_rows(c, s.st, ly.gradW, (size_t)ly.n_out, ly.n_in, ly.ld_in, w_G, ly.Gp);
+    for (int l : batch) {
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      const size_t n4 = (size_t)ly.n_out * ly.ld_in / 4;
+      PD_TRY(shard_sum(c, st, ly.gradW, n4 * 4, 0));
+      if (c->use_tc) PD_CUDA(cudaMemsetAsync(ly.w_G, 0, sizeof(uint32_t), st));
+      sumsq_amax_kernel<<<ew_grid(n4), EW_THREADS, 0, st>>>(ly.gradW, n4, c->use_tc ? ly.w_G : nullptr, s.slots);
+      reduce_slots_kernel<<<1, 256, 0, st>>>(s.slots, ew_grid(n4), 1, 1, &ly.sc->sum_G2);
+      if (c->use_tc) split_rows(c, st, ly.gradW, (size_t)ly.n_out, ly.n_in, ly.ld_in, ly.w_G, ly.Gp);
+    }
   }
-  int np = 0;
-  double *slots_b = s.slots + s.n_slots / 2;
-  EpiStoreSumsq epi{s.s1, ly.ld_out};
-  Operand G = plane_operand(ly.gradW, ly.ld_in, ly.Gp, w_G);
-  check_planes(c, s.st, (size_t)ly.n_out, G);
-  PD_TRY(gemm_nodes<false>(c, KC_GEMM_GP, s.st, N, ly.n_out, ly.n_in, P, G, epi, slots_b, &np, 0));
-  ThetaPlanes tp{};
-  if (c->use_tc) tp = ThetaPlanes{ly.amax_r, ly.amax_W, w_G, ly.Wp.exp, ly.rp.exp, ly.Gp.exp};
-  if (c->reduce != nullptr) {
+  std::vector<Operand> G;
+  std::vector<Operand *> to_check;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    G.push_back(c->use_tc ? plane_operand(ly.gradW, ly.ld_in, ly.Gp, ly.w_G) : Operand{ly.gradW, ly.ld_in, nullptr});
+  }
+  for (size_t i = 0; i < batch.size(); ++i) {
+    const Layer &ly = c->layers[batch[i]];
+    if ((size_t)ly.n_out * ly.ld_in < CHECK_PLANES_FROM) continue;
+    check_planes(c, st, (size_t)ly.n_out, {&G[i]});
+  }
+  {
+    std::vector<Prod<EpiStoreSumsq>> v;
+    for (size_t i = 0; i < batch.size(); ++i) {
+      const int l = batch[i];
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done};
+      p.step = make_step(c, ly, STEP_THETA);
+      if (c->use_tc) { p.step.w_in = ly.w_G; p.step.exp_W = ly.Wp.exp; p.step.exp_r = ly.rp.exp; p.step.exp_g = ly.Gp.exp; }
+      v.push_back(p);
+    }
+    PD_TRY((gemm_nodes<false>(c, KC_GEMM_GP, st, v, 0)));
     // ||G p+||^2 is a sum over nodes (||G||^2 is the same on every shard already)
-    PD_TRY(shard_sum_slots(c, s.st, s.red, slots_b, np, nullptr, 0));
-    launch_first(s.st, finalize_theta_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->nu, s.slots, gw, s.red, 1, c->d_flag + 2, tp);
-  } else {
-    Launch k(c, KC_SMALL, s.st, 8.0 * (gw + np), 0);
-    launch_first(s.st, finalize_theta_kernel, dim3(1), FIN_THREADS, 0, ly.sc, (double)c->nu, s.slots, gw, slots_b, np, c->d_flag + 2, tp);
+    for (size_t i = 0; i < batch.size(); ++i) PD_TRY(shard_step(c, st, &c->layers[batch[i]].sc->sum_Gp2, 1, v[i].step));
   }
   {
-    Launch k(c, KC_WSTEP, s.st, (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in, 0);
-    launch_first(s.st, wstep_kernel, dim3(gw), EW_THREADS, 0, ly.W, ly.gradW, ly.sc, n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp));
-  }
-  const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 16));
-  const int rows_per_block = (int)ceil_div(N, n_blocks);
-  const int used_blocks = (int)ceil_div(N, rows_per_block);
-  {
-    const int ld4 = ly.ld_out / 4, cols_per_pass = std::min(ld4, EW_THREADS);
-    const int n_sub = std::min(EW_THREADS / cols_per_pass, COLSUM_MAX_SUB);
-    const size_t sh = n_sub > 1 ? (size_t)n_sub * ly.ld_out * sizeof(double) : 0;
-    Launch k(c, KC_COLSUM, s.st, 12.0 * N * ly.n_out, 0);
-    launch_first(s.st, resid_colsum_kernel, dim3(used_blocks), EW_THREADS, sh, ly.r, s.s1, ly.sc, N, ly.ld_out, rows_per_block, s.slots);
-  }
-  if (c->reduce != nullptr) {
-    // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
-    launch_first(s.st, colsum_total_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.slots, used_blocks, ly.ld_out, s.red);
-    PD_TRY(shard_sum(c, s.st, s.red, (size_t)ly.ld_out, 1));
-    launch_first(s.st, finalize_bias_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.red, 1, ly.ld_out, ly.n_out,
-                                                                                1.0 / (double)c->N_total, ly.b, ly.shift);
-  } else {
-    Launch k(c, KC_SMALL, s.st, 8.0 * used_blocks * ly.ld_out, 0);
-    launch_first(s.st, finalize_bias_kernel, dim3((int)ceil_div(ly.ld_out, 32)), dim3(32, BIAS_GROUPS), 0, s.slots, used_blocks, ly.ld_out, ly.n_out,
-                                                                                1.0 / (double)N, ly.b, ly.shift);
+    Group<ThetaStep> g;
+    Group<BiasStep> gb;
+    int n = 0, blocks = 0, ld_max = 0;
+    size_t sh = 0;
+    double bytes = 0, bias_bytes = 0;
+    for (int l : batch) {
+      Layer &ly = c->layers[l];
+      Scratch &s = scratch_of(c, l);
+      const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
+      const int nbw = (int)std::min<int64_t>(ceil_div((int64_t)n4w, EW_THREADS), 2 * c->n_sms);
+      // rows in as many blocks as keep the SMs busy, at least 16 of them each
+      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 3, ceil_div(N, 16));
+      const int rows_per_block = (int)ceil_div(N, n_blocks), nbr = (int)ceil_div(N, rows_per_block);
+      const int ld4 = ly.ld_out / 4, n_sub = std::min(EW_THREADS / std::min(ld4, EW_THREADS), COLSUM_MAX_SUB);
+      if (n_sub > 1) sh = std::max(sh, (size_t)n_sub * ly.ld_out * sizeof(double));
+      g.l[n] = ThetaStep{ly.W, ly.gradW, (uint32_t)n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp), ly.r, s.s1, N, ly.ld_out,
+                         rows_per_block, s.slots, ly.sc, nbw, nbr};
+      gb.l[n] = BiasStep{s.slots, nbr, ly.ld_out, ly.n_out, ly.b, ly.shift};
+      ++n;
+      blocks = std::max(blocks, nbw + nbr);
+      ld_max = std::max(ld_max, ly.ld_out);
+      bytes += 12.0 * N * ly.n_out + (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in;
+      bias_bytes += 8.0 * nbr * ly.ld_out;
+    }
+    {
+      Launch k(c, KC_COLSUM, st, bytes, 0);
+      launch_first(st, theta_step_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, g);
+    }
+    if (c->reduce != nullptr) {
+      // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
+      for (int i = 0; i < n; ++i) {
+        Scratch &s = scratch_of(c, batch[i]);
+        BiasStep &b = gb.l[i];
+        colsum_total_kernel<<<(int)ceil_div(b.ld, 32), dim3(32, BIAS_GROUPS), 0, st>>>(b.slots, b.n_slots, b.ld, s.red);
+        PD_TRY(shard_sum(c, st, s.red, (size_t)b.ld, 1));
+        b.slots = s.red; b.n_slots = 1;
+      }
+    }
+    Launch k(c, KC_SMALL, st, bias_bytes, 0);
+    launch_first(st, finalize_bias_kernel, dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, gb,
+                 1.0 / (double)c->N_total);
   }
   return PDADMM_OK;
 }
 
-// z (and q, u for hidden layers) of layer l; needs p_{l+1} of this iteration.
-static void zqu_step(pdadmm_ctx *c, int l) {
-  Layer &ly = c->layers[l];
-  Scratch &s = *c->cur;
-  const int N = (int)c->N;
-  if (l + 1 < c->L) {
-    const size_t n4 = (size_t)N * ly.ld_out / 4;
-    const int grid = ew_grid(n4);
-    if (c->table_size > 0) {
-      Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);
-      const Layer &nx = c->layers[l + 1];
-      launch_first(s.st, zqu_table_kernel, dim3(grid), EW_THREADS, c->table_size * sizeof(float), 
-          ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu, c->slope, c->table_lo, c->table_step,
-          c->table_size, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t, ly.amax_r,
-          plane_out(c, ly.rp), c->levels ? nx.codes : nullptr, c->code_bytes == 2);
-    } else {
-      Launch k(c, KC_ZQU, s.st, ((c->levels ? 37.0 : 40.0) + (ly.rp.hi ? 4.0 : 0.0)) * N * ly.n_out, 0);      // p_{l+1} as one-byte codes
-      const Layer &nx = c->layers[l + 1];
-      launch_first(s.st, zqu_kernel, dim3(grid), EW_THREADS, 0, ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, ly.ld_out / 4, n4, c->rho, c->nu,
-                                               c->slope, nx.scale, nx.lo, c->quant_q ? (float)(c->levels - 1) : -1.0f, nx.t,
-                                               ly.amax_r, plane_out(c, ly.rp), c->levels ? nx.codes : nullptr,
-                                               c->code_bytes == 2);
-    }
-  } else {
-    Launch k(c, KC_ZLAST, s.st, (c->use_tc ? 20.0 : 16.0) * N * ly.n_out, 0);
-    launch_zlast(s.st, ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out, ly.ld_out, (double)c->nu, c->d_flag, ly.amax_r,
-                 c->ls_risk ? 1 : 0, plane_out(c, ly.rp));
+// z, q and u of hidden layers; needs p_{l+1} of this iteration.
+static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
+  Group<Zqu> g;
+  int n = 0, blocks = 0;
+  double bytes = 0;
+  for (int l : batch) {
+    Layer &ly = c->layers[l];
+    const Layer &nx = c->layers[l + 1];
+    const size_t n4 = (size_t)c->N * ly.ld_out / 4;
+    const int nb = ew_grid(n4);
+    g.l[n++] = Zqu{ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, nx.t, c->levels ? nx.codes : nullptr, nx.scale, nx.lo, (uint32_t)ly.ld_out / 4,
+                   (uint32_t)n4, c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), nb};
+    blocks = std::max(blocks, nb);
+    bytes += ((c->levels ? 36.0 + c->code_bytes : 40.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
   }
+  Launch k(c, KC_ZQU, st, bytes, 0);
+  const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
+                      c->table_step, c->table_size};
+  const dim3 grid((unsigned)blocks, (unsigned)n);
+  if (c->table_size > 0) launch_first(st, zqu_table_kernel, grid, EW_THREADS, c->table_size * sizeof(float), g, prm);
+  else launch_first(st, zqu_kernel, grid, EW_THREADS, 0, g, prm);
+}
+static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
+  Layer &ly = c->layers[c->L - 1];
+  const int N = (int)c->N;
+  Launch k(c, KC_ZLAST, st, (c->use_tc ? 20.0 : 16.0) * N * ly.n_out, 0);
+  launch_zlast(st, ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out, ly.ld_out, (double)c->nu, c->d_flag,
+               c->use_tc ? ly.amax_r : nullptr, c->ls_risk ? 1 : 0, plane_out(c, ly.rp));
 }
 
-static Scratch &lane(pdadmm_ctx *c, int i) { return i == 0 ? c->scr : *c->more_lanes[i - 1]; }
-
 static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
-  // per-kernel timing wants one kernel at a time: a single lane then
-  const int S = c->profiling ? 1 : 1 + (int)c->more_lanes.size();
-  auto lane_of = [&](int l) -> Scratch & { return lane(c, l % S); };
-  struct Restore { pdadmm_ctx *c; ~Restore() { c->cur = &c->scr; } } restore{c};
+  const int S_all = 1 + (int)c->more_lanes.size();
+  // Grouped: batches of up to S layers, one launch per kernel and batch, all on the main stream.  Otherwise one layer at a time,
+  // layer l on lane l mod S; per-kernel timing wants one kernel at a time, a single lane then.
+  const bool grouped = c->grouped;
+  const int S = grouped || !c->profiling ? S_all : 1;
+  c->n_active = S;
+  const cudaStream_t main = c->scr.st;
+  auto stream_of = [&](int l) { return grouped ? main : lane(c, l % S).st; };
+  const bool many = !grouped && S > 1;
   // the other lanes start after everything queued on the main stream so far
-  if (S > 1) {
-    PD_CUDA(cudaEventRecord(c->ev_lane[0], c->scr.st));
+  if (many) {
+    PD_CUDA(cudaEventRecord(c->ev_lane[0], main));
     for (int i = 1; i < S; ++i) PD_CUDA(cudaStreamWaitEvent(lane(c, i).st, c->ev_lane[0], 0));
   }
-  if (c->use_tc)
-    for (int i = 0; i < S; ++i) { c->cur = &lane(c, i); PD_TRY(amax_reset(c, c->cur->st)); }
-  // p-update (layers 2..L, from the iterates of the previous iteration) and W-, b-update with the new p, layer by layer: the
-  // lane's planes of r and p go from the one to the other.  The quantised p-update reads an accept flag on the host after
-  // every trial: the host queues layer l's gradient and first trial on its lane, and only then waits for the flag of the
-  // layer that it queued on another lane before, so that the GPU always has other lanes' work while a flag travels.
-  std::vector<int> waiting(S, -1);                   // layer whose first trial is in flight on each lane
-  auto take_trial = [&](int i) -> int {              // on lane i, which is current
-    const int w = waiting[i];
-    if (w < 0) return PDADMM_OK;
-    waiting[i] = -1;
-    PD_TRY(q_finish(c, w, hit_cap));
-    if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[w], c->cur->st));
-    return w_and_b_step(c, w);
+  // p-update (layers 2..L, from the iterates of the previous iteration) and W-, b-update with the new p, batch by batch: the
+  // scratch planes of r and p go from the one to the other.  The quantised p-update reads accept flags on the host after
+  // every trial: the host queues a batch's gradient and first trial, and only then waits for the flags of the
+  // batch that it queued on another lane before, so that the GPU always has other lanes' work while a flag travels.
+  const int per_batch = grouped ? std::min(S, MAX_GROUP) : 1;
+  std::vector<Batch> waiting(many ? S : 1);          // batch whose first trial is in flight on each lane
+  auto finish = [&](int i) -> int {
+    Batch b;
+    b.swap(waiting[i]);
+    if (b.empty()) return PDADMM_OK;
+    Batch p;                                         // (layer 1 has no p-update)
+    for (int l : b) if (l > 0) p.push_back(l);
+    const cudaStream_t st = stream_of(b[0]);
+    if (!p.empty()) PD_TRY(q_finish(c, st, p, hit_cap));
+    if (many) for (int l : p) PD_CUDA(cudaEventRecord(c->ev_p[l], st));
+    return w_and_b_step(c, st, b);
   };
-  for (int l = 0; l < c->L; ++l) {
-    c->cur = &lane_of(l);
-    if (c->levels && l > 0) {
-      PD_TRY(take_trial(l % S));
-      PD_TRY(p_gradient_and_tau(c, l));
-      PD_TRY(q_trial(c, l));
-      waiting[l % S] = l;
-      continue;
+  for (int l0 = 0; l0 < c->L; l0 += per_batch) {
+    Batch b, p;
+    for (int l = l0; l < std::min(c->L, l0 + per_batch); ++l) {
+      b.push_back(l);
+      if (l > 0) p.push_back(l);
     }
-    if (l > 0) {
-      PD_TRY(p_gradient_and_tau(c, l));
-      p_step_plain(c, l);
-      if (S > 1) PD_CUDA(cudaEventRecord(c->ev_p[l], c->cur->st));
+    const cudaStream_t st = stream_of(l0);
+    const int slot = many ? l0 % S : 0;
+    if (c->levels) PD_TRY(finish(slot));
+    if (!p.empty()) {
+      PD_TRY(p_gradient_and_tau(c, st, p));
+      if (c->levels) {
+        PD_TRY(q_trial(c, st, p));
+        waiting[slot] = b;
+        continue;
+      }
+      p_step_plain(c, st, p);
+      if (many) for (int l : p) PD_CUDA(cudaEventRecord(c->ev_p[l], st));
     }
-    PD_TRY(w_and_b_step(c, l));
+    PD_TRY(w_and_b_step(c, st, b));
   }
-  for (int i = 0; i < S && c->levels; ++i) {
-    const int next = (c->L + i) % S;                 // the lane whose trial was queued first
-    c->cur = &lane(c, next);
-    PD_TRY(take_trial(next));
-  }
+  const int n_batches = (int)ceil_div(c->L, per_batch);
+  for (size_t i = 0; i < waiting.size(); ++i) PD_TRY(finish((int)((n_batches + i) % waiting.size())));    // the oldest first
   // z-, q-, u-update (q_l and u_l need p_{l+1} of this iteration, which another lane may have written)
+  if (grouped) {
+    // the last layer's Newton steps run beside the hidden layers' update
+    const bool beside = S > 1 && !c->profiling && c->L > 1;
+    const cudaStream_t other = beside ? c->more_lanes[0]->own : main;
+    if (beside) {
+      PD_CUDA(cudaEventRecord(c->ev_lane[0], main));
+      PD_CUDA(cudaStreamWaitEvent(other, c->ev_lane[0], 0));
+    }
+    zlast_step(c, other);
+    // up to three hidden layers one launch each: nothing to gain from a common one
+    const int per = c->L - 1 > 3 ? MAX_GROUP : 1;
+    for (int l0 = 0; l0 + 1 < c->L; l0 += per) {
+      Batch b;
+      for (int l = l0; l < std::min(c->L - 1, l0 + per); ++l) b.push_back(l);
+      zqu_step(c, main, b);
+    }
+    if (beside) {
+      PD_CUDA(cudaEventRecord(c->ev_lane[1], other));
+      PD_CUDA(cudaStreamWaitEvent(main, c->ev_lane[1], 0));
+    }
+    return PDADMM_OK;
+  }
   for (int l = 0; l < c->L; ++l) {
-    c->cur = &lane_of(l);
-    if (S > 1 && l + 1 < c->L) PD_CUDA(cudaStreamWaitEvent(c->cur->st, c->ev_p[l + 1], 0));
-    zqu_step(c, l);
+    const cudaStream_t st = stream_of(l);
+    if (l + 1 == c->L) { zlast_step(c, st); break; }
+    if (many) PD_CUDA(cudaStreamWaitEvent(st, c->ev_p[l + 1], 0));
+    zqu_step(c, st, {l});
   }
   // join: the main stream continues after every lane
-  for (int i = 1; i < S; ++i) {
+  for (int i = 1; many && i < S; ++i) {
     PD_CUDA(cudaEventRecord(c->ev_lane[i], lane(c, i).st));
-    PD_CUDA(cudaStreamWaitEvent(c->scr.st, c->ev_lane[i], 0));
+    PD_CUDA(cudaStreamWaitEvent(main, c->ev_lane[i], 0));
   }
   return PDADMM_OK;
 }
@@ -1031,8 +1244,10 @@ static int build_csr(pdadmm_ctx *c, const pdadmm_config *cfg) {
 // buffers of a lane's quantised trials: trial p, d, codes (they trade places with a layer's p and codes when a
 // trial is taken, so all have one size), the pinned word and the event of the accept flag
 static int alloc_trial_buffers(pdadmm_ctx *c, Scratch &s, size_t n) {
-  PD_TRY(dev_alloc(c, &s.p_new, n));
-  if (!c->int_operands) PD_TRY(dev_alloc(c, &s.d, n));       // with integer operands d exists as d_plane only
+  if (!c->int_operands) {                                    // with integer operands p+ and d exist as codes and planes only
+    PD_TRY(dev_alloc(c, &s.p_new, n));
+    PD_TRY(dev_alloc(c, &s.d, n));
+  }
   PD_TRY(dev_alloc(c, &s.codes_new, n * c->code_bytes));
   if (c->int_operands) {
     PD_TRY(dev_alloc(c, &s.pn_plane, n));
@@ -1060,7 +1275,7 @@ static int feasible_start(pdadmm_ctx *c, int first) {
       split_rows(c, st, ly.p, (size_t)N, ly.n_in, ly.ld_in, ly.amax_p, ly.xp);
       P = operand_X(ly);
     }
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, (int)N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr, 0));
+    PD_TRY((gemm_nodes<false, EpiStore>(c, KC_GEMM_RESID, st, {{(int)N, ly.n_out, ly.n_in, P, operand_W(ly), epi, &c->scr}}, 0)));
     PD_CUDA(cudaMemsetAsync(ly.b, 0, (size_t)ly.ld_out * 4, st));
     PD_CUDA(cudaMemsetAsync(ly.shift, 0, (size_t)ly.ld_out * 4, st));
     PD_CUDA(cudaMemsetAsync(ly.r, 0, (size_t)N * ly.ld_out * 4, st));
@@ -1088,7 +1303,7 @@ static int feasible_start(pdadmm_ctx *c, int first) {
       nx.lo = -(float)c->neg_levels * nx.scale;
       quantize_kernel<<<ew_grid(n4 * 4), EW_THREADS, 0, st>>>(ly.q, n4 * 4, nx.scale, nx.lo, c->levels, nx.p, nx.codes,
                                                               c->code_bytes == 2);
-      if (c->int_operands) codes_to_plane_kernel<<<ew_grid(n4), EW_THREADS, 0, st>>>(nx.codes, c->code_bytes == 2, n4, nx.p_plane);
+      if (c->int_operands) codes_to_plane_kernel<<<ew_grid(n4), EW_THREADS, 0, st>>>(nx.codes, c->code_bytes == 2, c->neg_levels, n4, nx.p_plane);
       if (c->quant_q)      // start inside the level set: q_l = p_{l+1}
         PD_CUDA(cudaMemcpyAsync(ly.q, nx.p, n4 * 16, cudaMemcpyDeviceToDevice, st));
     } else {
@@ -1127,11 +1342,12 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->ls_risk = (cfg->flags & PDADMM_FLAG_LEAST_SQUARES) != 0;
   c->rho = cfg->rho; c->nu = cfg->nu; c->flags = cfg->flags;
   c->use_tc = (cfg->flags & PDADMM_FLAG_SIMT_GEMM) == 0;
-  c->int_operands = c->use_tc && c->levels >= 2 && c->levels <= 2048 && c->neg_levels == 0;
+  c->int_operands = c->use_tc && c->levels >= 2 && c->levels <= 2048;
   PD_CUDA(cudaSetDevice(cfg->device));
   PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, cfg->device));
   DevicePool &pool = device_pool(c->device);
-  PD_CUDA(pool.take_stream(&c->scr.st));
+  PD_CUDA(pool.take_stream(&c->scr.own));
+  c->scr.st = c->scr.own;
   cudaStream_t st = c->scr.st;
   PD_TRY(take_ctx_pinned(c));
   PD_CUDA(pool.take_event(true, &c->ev_begin));
@@ -1180,7 +1396,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     const size_t e_out = (size_t)N * ly.ld_out;
     // quantised mode: p_l and its codes trade places with the trial buffers, so all share one size
     const size_t e_in = (size_t)N * ((c->levels && l > 0) ? max_in : ly.ld_in);
-    PD_TRY(dev_alloc(c, &ly.p, e_in));
+    PD_TRY(dev_alloc(c, &ly.p, c->int_operands ? (size_t)N * ly.ld_in : e_in));
     if (l == 0)      // the features go first: their copy overlaps the clearing of everything allocated after them
       PD_TRY(upload_rows(c, st, sharded ? x_full : ly.p, ly.ld_in, cfg->features, c->d, Ntot));
     PD_TRY(dev_alloc(c, &ly.W, (size_t)ly.n_out * ly.ld_in));
@@ -1201,15 +1417,25 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     if (c->int_operands && l > 0) PD_TRY(dev_alloc(c, &ly.p_plane, e_in));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.t, (size_t)N * ly.ld_in));
     PD_TRY(dev_alloc(c, &ly.sc, 1));
+    PD_TRY(dev_alloc(c, &ly.w_g, 4));
+    ly.w_wg = ly.w_g + 1; ly.w_G = ly.w_g + 2; ly.w_d = ly.w_g + 3;
+    PD_TRY(dev_alloc(c, &ly.done, 4));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.g_exp, 1));
     PD_TRY(dev_alloc(c, &ly.amax_p, 1));
     PD_TRY(dev_alloc(c, &ly.amax_r, 1));
     PD_TRY(upload_rows(c, st, ly.W, ly.ld_in, cfg->init_W[l], ly.n_in, ly.n_out));
-    // Node slices of the W-gradient product (slices >= 256 nodes, at most 32).  The persistent grid works through
-    // tiles x slices units in rounds of n_sms, so the count is chosen to fill its last round: the smallest number
-    // of slices within 3 % (relative) of the best fill (fewer slices = fewer partial tiles to write and add up).
-    const int64_t tiles = ceil_div(ly.n_in, SG_BN) * ceil_div(ly.n_out, SG_BM);   // same tile for both kernels; a pair of
-                                                                                    // SMs works on two of them
+  }
+  // Scratch per layer, for working on the layers in batches, if it fits 4 GB for three layers at least; estimated from the two
+  // fp32 matrices and the two pairs of planes, which are most of it.
+  const size_t e_max = (size_t)N * std::max(max_in, max_out);
+  const bool small = c->L > 1 && 3 * 16 * e_max <= (size_t(4) << 30);
+  // Node slices of the W-gradient product (slices >= 256 nodes, at most 32).  The persistent grid works through
+  // tiles x slices units in rounds of n_sms, so the count is chosen to fill its last round: the smallest number
+  // of slices within 3 % (relative) of the best fill (fewer slices = fewer partial tiles to write and add up).  Layers that are
+  // worked on together have one common count.
+  auto choose_slices = [&](int l0, int l1) {
+    int64_t tiles = 0;
+    for (int l = l0; l < l1; ++l) tiles += ceil_div(c->layers[l].n_in, SG_BN) * ceil_div(c->layers[l].n_out, SG_BM);
     const int max_split = (int)std::max<int64_t>(1, std::min<int64_t>(32, ceil_div(N, 256)));
     auto slices_for = [&](int want) { return (int)ceil_div(N, round_up((int)ceil_div(N, want), TC_BK)); };
     auto fill = [&](int want) {
@@ -1220,14 +1446,17 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     for (int w = 1; w <= max_split; ++w) best = std::max(best, fill(w));
     int split = 1;
     while (split < max_split && fill(split) < 0.97 * best) ++split;
-    ly.k_chunk = round_up((int)ceil_div(N, split), TC_BK);      // multiple of both kernels' K blocks
-    ly.n_split = (int)ceil_div(N, ly.k_chunk);
-    max_part = std::max(max_part, (size_t)ly.n_split * ly.n_out * ly.ld_in);
-  }
+    for (int l = l0; l < l1; ++l) {
+      Layer &ly = c->layers[l];
+      ly.k_chunk = round_up((int)ceil_div(N, split), TC_BK);      // multiple of both kernels' K blocks
+      ly.n_split = (int)ceil_div(N, ly.k_chunk);
+      max_part = std::max(max_part, (size_t)ly.n_split * ly.n_out * ly.ld_in);
+    }
+  };
+  for (int l = 0; l < c->L; l += small ? MAX_GROUP : 1) choose_slices(l, std::min(c->L, l + (small ? MAX_GROUP : 1)));
   // scratch
   Scratch &s = c->scr;
   const size_t bytes_before_scratch = c->bytes_handed_out;
-  const size_t e_max = (size_t)N * std::max(max_in, max_out);
   PD_TRY(dev_alloc(c, &s.s1, e_max));
   PD_TRY(dev_alloc(c, &s.s2, (size_t)N * max_out));
   if (c->levels) PD_TRY(alloc_trial_buffers(c, s, (size_t)N * max_in));
@@ -1246,19 +1475,20 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &s.a_exp, 1));
   }
 
-  // further lanes for the concurrency across layers: own stream, product outputs, partial tiles, slots.
-  // Small problems are bound by the latency of their chain of launches, which only more concurrent chains shorten
-  // (workload c1, 10 layers: 2 lanes 0.40 ms per iteration); large ones gain little beyond two (c2: 2 lanes 273,
-  // 4 lanes 278 iterations/s) and their scratch is gigabytes per lane.  So: as many lanes as 4 GB of scratch pay for,
-  // at least PDADMM_N_LANES, at most one per layer (c3, 0.4 GB per lane: 6 lanes 280, 10 lanes 301 iterations/s;
-  // c4, 5.5 GB per lane: 2 lanes 9.95, 4 lanes 9.99).
+  // Further scratch: small problems are bound by the latency of their chain of launches, so their layers are worked on in
+  // batches, every kernel launched once per batch; as much scratch as 4 GB pay for, at most one per layer.  Large ones keep two
+  // lanes with a stream each (their scratch is gigabytes per lane, and more lanes gained nothing).
   const size_t lane_bytes = std::max<size_t>(c->bytes_handed_out - bytes_before_scratch, 1);
-  const int affordable = (int)std::min<size_t>(64, (size_t(4) << 30) / lane_bytes);
-  const int n_lanes = (cfg->flags & PDADMM_FLAG_ONE_LANE) ? 1 : std::min(c->L, std::max(PDADMM_N_LANES, affordable));
+  const int affordable = (int)std::max<size_t>(2, (size_t(4) << 30) / lane_bytes);
+  const bool one_lane = (cfg->flags & PDADMM_FLAG_ONE_LANE) != 0;
+  c->tail_split = !small;
+  c->grouped = small && !one_lane;
+  const int n_lanes = one_lane ? 1 : std::min(c->L, small ? std::min(affordable, MAX_GROUP) : PDADMM_N_LANES);
   for (int i = 1; i < n_lanes; ++i) {
     c->more_lanes.emplace_back(new Scratch());
     Scratch &x = *c->more_lanes.back();
-    PD_CUDA(pool.take_stream(&x.st));
+    PD_CUDA(pool.take_stream(&x.own));
+    x.st = c->grouped ? c->scr.st : x.own;
     PD_TRY(dev_alloc(c, &x.s1, e_max));
     PD_TRY(dev_alloc(c, &x.s2, (size_t)N * max_out));
     PD_TRY(dev_alloc(c, &x.part, max_part));
@@ -1269,7 +1499,6 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     if (c->use_tc) {
       PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
       PD_TRY(dev_alloc(c, &x.tail_count, (size_t)c->n_sms * 8));
-      PD_TRY(dev_alloc(c, &x.amax_pool, (size_t)AMAX_POOL));
       x.pl_cap = s.pl_cap;
       PD_TRY(alloc_planes(c, x.pl_cap, &x.pl0));
       PD_TRY(alloc_planes(c, x.pl_cap, &x.pl1));
@@ -1287,7 +1516,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   }
   c->ev_p.resize(c->L);
   for (auto &e : c->ev_p) PD_CUDA(pool.take_event(false, &e));
-  c->ev_lane.resize(n_lanes);
+  c->ev_lane.resize(std::max(n_lanes, 2));
   for (auto &e : c->ev_lane) PD_CUDA(pool.take_event(false, &e));
 
   // X = [H, A~ H, A~^2 H, ...] in the column blocks of p_1
@@ -1330,7 +1559,7 @@ static void destroy(pdadmm_ctx *c) {
   for (int i = 0; i <= (int)c->more_lanes.size(); ++i) {
     pd::Scratch &x = i == 0 ? c->scr : *c->more_lanes[i - 1];
     pool.give_event(false, x.ev_flag);
-    pool.give_stream(x.st);
+    pool.give_stream(x.own);
   }
   delete c;
 }
@@ -1382,10 +1611,13 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
   return PDADMM_OK;
 }
 
+static int refresh_p(pdadmm_ctx *c);
+
 extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
   if (!c) return fail(PDADMM_EINVAL, "context is null");
   if (first_layer < 1 || first_layer > c->L) return fail(PDADMM_EINVAL, "first_layer must be in [1, %d]", c->L);
   PD_CUDA(cudaSetDevice(c->device));
+  PD_TRY(refresh_p(c));
   PD_TRY(feasible_start(c, first_layer - 1));
   PD_CUDA(cudaStreamSynchronize(c->scr.st));
   PD_CUDA(cudaGetLastError());
@@ -1414,8 +1646,22 @@ extern "C" int pdadmm_destroy(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
+// p_l, l >= 2, from its codes where the fp32 values are older (integer operands)
+static int refresh_p(pdadmm_ctx *c) {
+  if (!c->p_stale) return PDADMM_OK;
+  for (int l = 1; l < c->L; ++l) {
+    Layer &ly = c->layers[l];
+    const size_t n4 = (size_t)c->N * ly.ld_in / 4;
+    codes_to_levels_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.codes, c->code_bytes == 2, n4, ly.scale, ly.lo, ly.p);
+  }
+  PD_CUDA(cudaGetLastError());
+  c->p_stale = false;
+  return PDADMM_OK;
+}
+
 // What products read beside the stored tensors: planes of W, largest magnitudes of p, planes of X.
 static int ensure_operands(pdadmm_ctx *c) {
+  if (!c->amax_p_valid || !c->t_valid || !c->r_valid) PD_TRY(refresh_p(c));
   if (!c->w_planes_valid) {
     for (auto &ly : c->layers) PD_TRY(refresh_W_planes(c, ly, c->scr.st));
     c->w_planes_valid = true;
@@ -1602,7 +1848,7 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
     EpiBiasAct epi{out, ly.ld_out, ly.b, l + 1 < c->L ? 1 : 0, c->slope, w_out};
     Operand P{in, ly.ld_in, w_in};
     if (l == 0 && c->use_tc) P = operand_X(ly);
-    PD_TRY(gemm_nodes<false>(c, KC_GEMM_RESID, st, N, ly.n_out, ly.n_in, P, operand_W(ly), epi, nullptr, nullptr, 0));
+    PD_TRY((gemm_nodes<false, EpiBiasAct>(c, KC_GEMM_RESID, st, {{N, ly.n_out, ly.n_in, P, operand_W(ly), epi, &c->scr}}, 0)));
     w_in = w_out;
     in = out;
   }
@@ -1698,6 +1944,7 @@ extern "C" int pdadmm_get_tensor(pdadmm_ctx *c, int kind, int layer, void *host_
   if (bytes != t.rows * t.width * t.elem)
     return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                 t.rows * t.width * t.elem, bytes);
+  if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
   return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
 }
 
@@ -1707,7 +1954,7 @@ static int project_p_on_its_levels(pdadmm_ctx *c, int layer) {
   Layer &y = c->layers[layer - 1];
   const size_t n = (size_t)c->N * y.ld_in;
   quantize_kernel<<<ew_grid(n), EW_THREADS, 0, c->scr.st>>>(y.p, n, y.scale, y.lo, c->levels, y.p, y.codes, c->code_bytes == 2);
-  if (c->int_operands) codes_to_plane_kernel<<<ew_grid(n / 4), EW_THREADS, 0, c->scr.st>>>(y.codes, c->code_bytes == 2, n / 4, y.p_plane);
+  if (c->int_operands) codes_to_plane_kernel<<<ew_grid(n / 4), EW_THREADS, 0, c->scr.st>>>(y.codes, c->code_bytes == 2, c->neg_levels, n / 4, y.p_plane);
   PD_CUDA(cudaGetLastError());
   PD_CUDA(cudaStreamSynchronize(c->scr.st));
   c->r_valid = false;
@@ -1724,12 +1971,14 @@ extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void 
     float v;
     memcpy(&v, host_src, 4);
     if (!(v > 0.f)) return fail(PDADMM_EINVAL, "QSCALE must be positive");
+    PD_TRY(refresh_p(c));
     c->layers[layer - 1].scale = v;
     c->layers[layer - 1].lo = -(float)c->neg_levels * v;
     if (c->levels) PD_TRY(project_p_on_its_levels(c, layer));       // p_l moves to the new level set
     return PDADMM_OK;
   }
   TensorRef t;
+  if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
   PD_TRY(locate(c, kind, layer, &t));
   if (!t.settable) return fail(PDADMM_EINVAL, "tensor kind %d is read-only", kind);
   if (bytes != t.rows * t.width * t.elem)
@@ -1822,7 +2071,8 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
   c->use_tc = (flags & PDADMM_FLAG_SIMT_GEMM) == 0;
   auto body = [&]() -> int {
     PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device));
-    PD_CUDA(device_pool(device).take_stream(&c->scr.st));
+    PD_CUDA(device_pool(device).take_stream(&c->scr.own));
+    c->scr.st = c->scr.own;
     cudaStream_t st = c->scr.st;
     PD_TRY(dev_alloc(c, &c->d_flag, 4));
     if (c->use_tc) {
@@ -1854,13 +2104,16 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       oA = plane_operand(dA, lda, Ap);
       oB = plane_operand(dB, ldb, Bp);
     }
-    int np = 0;
+    double *res = slots + n_slots - 1;
+    int *done;
+    PD_TRY(dev_alloc(c, &done, 1));
+    Step step;
+    step.kind = STEP_SUM; step.sum = res;
+    EpiStoreSumsq epi{dC, ldc};
     if (mode == 0) {
-      EpiStoreSumsq epi{dC, ldc};
-      PD_TRY(gemm_nodes<false>(c, KC_GEMM_WG, st, M, N, K, oA, oB, epi, slots, &np, 0));
+      PD_TRY((gemm_nodes<false, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
     } else if (mode == 1) {
-      EpiStoreSumsq epi{dC, ldc};
-      PD_TRY(gemm_nodes<true>(c, KC_GEMM_WG, st, M, N, K, oA, oB, epi, slots, &np, 0));
+      PD_TRY((gemm_nodes<true, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
     } else {
       const int split = (int)std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(K, 64)));
       const int k_chunk = round_up((int)ceil_div(K, split), TC_BK);
@@ -1870,14 +2123,15 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
         dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM), (unsigned)n_split);
         gemm_tn_kernel<<<grid, SG_THREADS, 0, st>>>(M, N, K, k_chunk, dA, lda, dB, ldb, part, ldc);
       } else {
-        PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, M, N, K, oA, oB, part, ldc, k_chunk, n_split));
+        Prod<EpiStore> p{M, N, K, oA, oB, EpiStore{part, ldc}, &c->scr};
+        p.n_split = n_split; p.k_chunk = k_chunk; p.stride = (size_t)M * ldc;
+        PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, {p}));
       }
       const size_t n4 = (size_t)M * ldc / 4;
-      np = ew_grid(n4);
-      reduce_gradW_kernel<<<np, EW_THREADS, 0, st>>>(part, n_split, n4, 1.0f, dC, nullptr, slots, PlaneOut{nullptr, nullptr, nullptr});
+      Group<GradWSum> g;
+      g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
+      launch_first(st, reduce_gradW_kernel, dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, g, 1.0f);
     }
-    double *res = slots + n_slots - 1;
-    reduce_slots_kernel<<<1, 256, 0, st>>>(slots, np, 1, 1, res);
     double h = 0;
     PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
     PD_TRY(copy_rows(device, st, C, dC, (size_t)ldc * 4, (size_t)N * 4, (size_t)M, true));
