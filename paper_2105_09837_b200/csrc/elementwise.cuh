@@ -118,7 +118,7 @@ struct PStep {
   uint32_t *amax_p, *amax_r;          // receive max|p|, max|r| (see commit_amax); may be null
   int n_blocks;
 };
-__global__ void __launch_bounds__(EW_THREADS, 5)
+__global__ void __launch_bounds__(EW_THREADS)
 pstep_kernel(const __grid_constant__ Group<PStep> group) {
   const PStep &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.n_blocks) return;
@@ -127,17 +127,16 @@ pstep_kernel(const __grid_constant__ Group<PStep> group) {
   auto pass = [&](float *__restrict__ out, const float *__restrict__ x, uint32_t n4, const PlaneOut &o, uint32_t *amax) {
     const float scale = o.hi != nullptr ? tc_scale_of(*o.exp) : 1.f;
     uint32_t m = 0u;
-    // two groups per pass: four loads in flight per thread (four groups take more registers than two blocks have beside a
-    // product)
-    for (uint32_t i = first; i < n4; i += 2 * stride) {
-      float4 v[2], w[2];
+    // four groups per pass: eight loads in flight per thread
+    for (uint32_t i = first; i < n4; i += 4 * stride) {
+      float4 v[4], w[4];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < 4; ++k) {
         const uint32_t q = i + k * stride;
         if (q < n4) { v[k] = ld4(out, q); w[k] = ld4(x, q); }
       }
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < 4; ++k) {
         const uint32_t q = i + k * stride;
         if (q >= n4) continue;
         v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
@@ -503,7 +502,6 @@ finalize_bias_kernel(const __grid_constant__ Group<BiasStep> group, double inv_n
 // the level set of p_{l+1}, the variant at the end of Sec. "Quantization Extension"), residual p_{l+1} - q+,
 // u+ by Eq. "update u", the linear residual of the next iteration r = a - z+, and t_{l+1} = u+ + rho (p_{l+1} - q+),
 // the part of the next p-gradient that does not involve a product.
-// At most 48 registers: two blocks fit on an SM beside a product.
 struct Zqu {
   float *r, *z, *q, *u; const float *p_next, *shift; float *t_next;
   const void *codes_next;                 // pdADMM-G-Q: codes of p_next, read instead of it
@@ -513,7 +511,7 @@ struct Zqu {
   int n_blocks;
 };
 struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T; };
-__global__ void __launch_bounds__(EW_THREADS, 5)
+__global__ void __launch_bounds__(EW_THREADS)
 zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
   const Zqu &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.n_blocks) return;

@@ -19,12 +19,12 @@
 // that operand's planes from the fp32 matrix instead of loading them (rare, slower, same result; large matrices get a
 // kernel that does it beforehand, see check_planes_kernel).
 //
-// One thread issues tcgen05.mma; completion is tracked with mbarriers; eight accumulate warps read each K block's main term
-// from tensor memory, add it to register accumulators and finally apply the scaling and the fused epilogue.  While
-// they are in that epilogue the MMAs run up to three K blocks ahead into the next tile.
+// One thread issues tcgen05.mma; completion is tracked with mbarriers.  Eight accumulate warps read each K block's main term
+// from tensor memory and add it to register accumulators; a finished tile goes through shared memory to eight epilogue
+// warps, which apply the fused operations and store it while the next tile is accumulated.  (With one set of warps for
+// both, the loads and stores of the epilogue had 16 KB in flight per SM and the tensor pipe waited for them: 9 layers of
+// 20 000 x 500 x 500, r W with its epilogue 533 us.)
 //
-// A block takes 61 % of an SM's registers and leaves 17 KB of its shared memory: bandwidth-bound kernels of other layers run
-// beside it (they are launched with a higher priority), which hides about half of their time behind the products.
 // Tile: 128 x 128 outputs per block, 64-deep K blocks.  What bounds the product is the traffic between L2 and the SMs
 // (10.6 TB/s measured, whatever the number of planes): a block on its own loads A and B planes of 64 KB per K block for
 // three times 2 MFLOP.  So two neighbouring SMs work as a pair on 256 x 128 outputs (tcgen05 cta_group::2): each loads the
@@ -50,27 +50,28 @@ constexpr int TC_KSTEPS = TC_BK / 16;                          // MMAs (K = 16) 
 constexpr int TC_FLUSH = 1;                                    // K blocks per read-out of the main accumulator
 constexpr int TC_PLANE_BYTES = 128 * TC_BK * 2;                // 16 KB: one 128 x 64 fp16 operand plane
 constexpr int TC_BOX_BYTES = 64 * TC_BK * 2;                   // 8 KB: what one TMA load brings, 64 x 64
-constexpr int TC_STAGE_SPACE = 12 * TC_PLANE_BYTES;            // 192 KB: 3 to 8 stages, by the number of planes
+constexpr int TC_STAGE_SPACE = 10 * TC_PLANE_BYTES;            // 160 KB: 2 to 6 stages, by the number of planes
 constexpr int TC_MAX_STAGES = 8;
-// Three warpgroups (register budgets are set per warpgroup): 0 = TMA warp, MMA warp and two warps that split operands when
+// Five warpgroups (register budgets are set per warpgroup): 0 = TMA warp, MMA warp and two warps that split operands when
 // a scaling was unusable; 1, 2 = the accumulate warps: a warp can only reach its own 32-lane quarter of tensor memory, so
-// warp w owns the rows of quarter w mod 4 and columns 64 (w / 4) .. +63 of the tile, 64 accumulators per thread.
-// Registers: the block is launched with 384 x 104 = 39936; warpgroup 0 keeps 56 per thread, the
-// accumulate warps take 128: 128 (56 + 2 x 128) = 39936, so every increase is satisfiable.
+// warp w owns the rows of quarter w mod 4 and columns 64 (w / 4) .. +63 of the tile, 64 accumulators per thread; 3, 4 = the
+// epilogue warps, each with an accumulate warp to serve.
+// Registers: the block is launched with 640 x 96 = 61440; warpgroup 0 keeps 56 per thread, the accumulate warps take 120, the
+// epilogue warps 88: 128 (56 + 2 x 120 + 2 x 88) = 60416, so every increase is satisfiable.
 constexpr int TC_SPLIT0 = 2, TC_SPLIT_WARPS = 2;               // first splitting warp
-constexpr int TC_ACC0 = 4;                                     // first accumulate warp
-constexpr int TC_THREADS = 384;
+constexpr int TC_ACC0 = 4, TC_EPI0 = 12;                       // first accumulate warp, first epilogue warp
+constexpr int TC_THREADS = 640;
 constexpr int TC_ACC_WARPS = 8;
-constexpr int TC_REGS_LAUNCH = 104, TC_REGS_CTRL = 56, TC_REGS_ACC = 128;
+constexpr int TC_REGS_LAUNCH = 96, TC_REGS_CTRL = 56, TC_REGS_ACC = 120, TC_REGS_EPI = 88;
 static_assert(TC_THREADS * TC_REGS_LAUNCH <= 65536, "register file");
-static_assert(128 * (TC_REGS_CTRL + 2 * TC_REGS_ACC) <= TC_THREADS * TC_REGS_LAUNCH,
+static_assert(128 * (TC_REGS_CTRL + 2 * TC_REGS_ACC + 2 * TC_REGS_EPI) <= TC_THREADS * TC_REGS_LAUNCH,
               "the warpgroups' register shares exceed what the block is launched with: an increase would wait for ever");
 constexpr int TC_ACC_BUFS = 3;                                 // main-term accumulator tiles in tensor memory
 constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 1 correction tile
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
-constexpr int TC_TR_BYTES = 8 * 32 * 16 * 4;                   // epilogue transpose: 8 warps x 32 rows x 16 columns
-constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
-static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3) + 12 <= 256, "barriers");
+constexpr int TC_TR_BYTES = 8 * 32 * 64 * 4;                   // finished tile: 8 warps x 32 rows x 64 columns
+constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 512 /* barriers */;
+static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -181,7 +182,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
   uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
   uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(team_bar + 1);
+  uint64_t *done_full = team_bar + 1, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
 
@@ -193,6 +195,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   // scaling exponents of every layer's operands (written by earlier kernels of the stream), and whether the planes made with
   // them are usable; the same for every block
   __shared__ int lay_exp[TC_MAX_GROUP][2];
+  __shared__ double team_scratch[1 + TC_ACC_WARPS];
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
   bool my_split = false;
   // (only of layers this block works on: the step of a finished layer may already have changed the words of the others)
@@ -229,6 +232,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
     ptx::mbar_init(team_bar, TC_ACC_WARPS);
+    for (int w = 0; w < TC_ACC_WARPS; ++w) {
+      ptx::mbar_init(&done_full[w], 1);
+      ptx::mbar_init(&done_empty[w], 1);
+    }
     *abort_flag = 0;
     // One thread reads the error word for the whole block, so that all warps take the same path: every block still
     // allocates and releases its tensor memory and passes both block-wide barriers.
@@ -455,17 +462,19 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       }
     }
   } else {
-    ptx::setmaxnreg_inc<TC_REGS_ACC>();
-    // -------------------------------------------------------------- accumulate, then epilogue (8 warps)
-    const int aw = warp - TC_ACC0, quarter = warp & 3, col_base = 64 * (aw >> 2);
+    // Accumulate warp aw and epilogue warp aw: rows of quarter aw mod 4, columns col_base .. +63 of every tile of the block.
+    constexpr bool STORES = epi_stores<Epi>::value;
+    const bool accumulates = warp < TC_EPI0;
+    const int aw = warp - (accumulates ? TC_ACC0 : TC_EPI0), quarter = warp & 3, col_base = 64 * (aw >> 2);
     const int lane_base = quarter * 32, piece = (int)rank * TC_ACC_WARPS + aw;
-    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 4;    // 32 rows x 4 float4 per warp
+    // the warp pair's part of the finished tile: row i at 16 i, its 16 float4 groups with the group index XOR-ed by (i mod 8), so
+    // that both sides (a lane per row; 16 lanes per row) are free of bank conflicts
+    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 16;
     bool ok = true;
-    int b = 0;
-    uint32_t ph = 0;                                   // phase of acc_full[b]
     Tile t;
     int visited = 0;                                   // units of layer t.g that this block has finished
-    // all accumulate warps of the block; bounded like every other wait
+    // The eight warps that know the sums of squares (the epilogue warps; the accumulate warps if nothing is stored), bounded
+    // like every other wait.
     uint32_t team_ph = 0;
     auto team_sync = [&]() {
       __syncwarp();
@@ -480,8 +489,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       if (!Epi::kSumsq || y.slots == nullptr || visited == 0) return true;
       constexpr int n_threads = 32 * TC_ACC_WARPS;
       const int tid = aw * 32 + lane;
-      volatile int *last = reinterpret_cast<int *>(tr_base);              // the first warp's staging buffer
-      volatile double *part = reinterpret_cast<double *>(tr_base) + 8;
+      volatile int *last = reinterpret_cast<volatile int *>(team_scratch);
+      volatile double *part = team_scratch + 1;
       __threadfence();
       if (!team_sync()) return false;
       if (tid == 0) {
@@ -507,168 +516,182 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
         }
       }
       visited = 0;
-      return team_sync();                              // the staging buffer is free again
+      return team_sync();                              // the scratch is free again
     };
-    for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
-      const int g_before = t.g;
-      locate(unit, t);
-      if (t.g != g_before && !leave(g_before)) { ok = false; break; }
-      ++visited;
-      const TcLayer<Epi> &y = grp.l[t.g];
-      const Epi &epi = y.epi;
-      const int m0 = t.m0, n0 = t.n0 + col_base, n_kb = t.n_kb;       // n0: of this warp
-      // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
-      // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
-      const int n_pad = epi.ldc;
-      const int n_grp = COARSE ? (n_kb > 0 ? 1 : 0) : n_kb;   // read-outs of the main accumulator for this tile
-      if (m0 + lane_base + lane < y.M) {          // this thread's row of the epilogue inputs, on its way to L2
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int col = n0 + h * 32;
-          if (col < n_pad) epi.prefetch(m0 + lane_base + lane, col);
+    auto put_sum = [&](const TcLayer<Epi> &y, double v) {
+      v = warp_sum(v);
+      const int tiles_n = (y.N + TC_BN - 1) / TC_BN;
+      if (lane == 0) y.slots[((size_t)(t.m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw] = v;
+    };
+    if (accumulates) {
+      ptx::setmaxnreg_inc<TC_REGS_ACC>();
+      // ------------------------------------------------------------ accumulate
+      int b = 0;
+      uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; tiles handed over so far
+      for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+        const int g_before = t.g;
+        locate(unit, t);
+        if (!STORES) {
+          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
+          ++visited;
         }
-      }
-      uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
-#pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0ull;
-      // acc += tile (or tile * 2^-11).  The tile is given back (one arrival per warp on `done` of block 0, whose MMA thread
-      // waits) as soon as its last columns are in registers.
-      auto add_tile = [&](uint32_t col, auto plain, uint64_t *done) {
-        const uint32_t src = tmem_base + ((uint32_t)lane_base << 16) + col + (uint32_t)col_base;
-        uint32_t v[32];
-        auto add = [&](int h) {
-          const uint64_t w = ptx::pack_f2(0x3A000000u, 0x3A000000u);       // 2^-11 twice
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const uint64_t x = ptx::pack_f2(v[2 * j], v[2 * j + 1]);
-            acc[16 * h + j] = decltype(plain)::value ? ptx::add_f2(acc[16 * h + j], x) : ptx::fma_f2(w, x, acc[16 * h + j]);
-          }
-        };
-        ptx::tmem_ld32(src, v);
-        ptx::tmem_ld_wait(v);
-        add(0);
-        ptx::tmem_ld32(src + 32u, v);
-        ptx::tmem_ld_wait(v);
-        ptx::tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(done, 0));
-        add(1);
-      };
-      for (int g = 0; g < n_grp && ok; ++g) {
-        ok = ptx::mbar_wait(&acc_full[b], ph, abort_flag);
-        if (!ok) break;
-        ptx::tc_fence_after_sync();
-        add_tile((uint32_t)(b * TC_BN), std::true_type{}, &acc_empty[b]);
-        if (++b == TC_ACC_BUFS) { b = 0; ph ^= 1u; }
-      }
-      if (!ok) break;
-      if (n_kb > 0) {
-        // correction terms: complete once the last block's commit has arrived (it covers every earlier MMA)
-        if constexpr (!COARSE) add_tile(TC_COL_CORR, std::false_type{}, corr_empty);
-        // undo the operand scalings (two exact factors, so that neither leaves the range on its own)
-        const int e = lay_exp[t.g][0] + lay_exp[t.g][1], e1 = e / 2, e2 = e - e1;
-        const uint32_t u1 = __float_as_uint(tc_pow2(-e1)), u2 = __float_as_uint(tc_pow2(-e2));
-        const uint64_t w1 = ptx::pack_f2(u1, u1), w2 = ptx::pack_f2(u2, u2);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(ptx::mul_f2(acc[j], w1), w2);
-        if constexpr (ZERO != 0) {
-          const uint64_t mul = ptx::pack_f2(__float_as_uint(y.mul), __float_as_uint(y.mul));
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
-        }
-      }
-      auto acc_at = [&](int j) {                      // columns 4 j .. 4 j + 3
-        float4 v;
-        ptx::unpack_f2(acc[2 * j], v.x, v.y);
-        ptx::unpack_f2(acc[2 * j + 1], v.z, v.w);
-        return v;
-      };
-      if (t.slice >= 0) {
-        // contraction slice of a tail tile: park the accumulators; the last warp to arrive sums the slices
-        const int t_idx = t.out - y.tail_begin, u = t_idx * y.tail_split + t.slice;
-        float4 *mine = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)u * WARPS + piece) * 512;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) mine[j * 32 + lane] = acc_at(j);
-        __threadfence();
-        __syncwarp();
-        int prev = 0;
-        if (lane == 0) prev = atomicAdd(y.tail_count + t_idx * WARPS + piece, 1);
-        prev = __shfl_sync(0xffffffffu, prev, 0);
-        if (prev != y.tail_split - 1) continue;
-        __threadfence();
-        if (lane == 0) y.tail_count[t_idx * WARPS + piece] = 0;
+        const TcLayer<Epi> &y = grp.l[t.g];
+        const int n_grp = COARSE ? (t.n_kb > 0 ? 1 : 0) : t.n_kb;   // read-outs of the main accumulator for this tile
+        uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = 0ull;
-        for (int sl = 0; sl < y.tail_split; ++sl) {
-          const float4 *part = reinterpret_cast<const float4 *>(y.tail_ws) + ((size_t)(t_idx * y.tail_split + sl) * WARPS + piece) * 512;
+        // acc += tile (or tile * 2^-11).  The tile is given back (one arrival per warp on `done` of block 0, whose MMA thread
+        // waits) as soon as its last columns are in registers.
+        auto add_tile = [&](uint32_t col, auto plain, uint64_t *done) {
+          const uint32_t src = tmem_base + ((uint32_t)lane_base << 16) + col + (uint32_t)col_base;
+          uint32_t v[32];
+          auto add = [&](int h) {
+            const uint64_t w = ptx::pack_f2(0x3A000000u, 0x3A000000u);       // 2^-11 twice
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const uint64_t x = ptx::pack_f2(v[2 * j], v[2 * j + 1]);
+              acc[16 * h + j] = decltype(plain)::value ? ptx::add_f2(acc[16 * h + j], x) : ptx::fma_f2(w, x, acc[16 * h + j]);
+            }
+          };
+          ptx::tmem_ld32(src, v);
+          ptx::tmem_ld_wait(v);
+          add(0);
+          ptx::tmem_ld32(src + 32u, v);
+          ptx::tmem_ld_wait(v);
+          ptx::tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(done, 0));
+          add(1);
+        };
+        for (int g = 0; g < n_grp && ok; ++g) {
+          ok = ptx::mbar_wait(&acc_full[b], ph, abort_flag);
+          if (!ok) break;
+          ptx::tc_fence_after_sync();
+          add_tile((uint32_t)(b * TC_BN), std::true_type{}, &acc_empty[b]);
+          if (++b == TC_ACC_BUFS) { b = 0; ph ^= 1u; }
+        }
+        if (!ok) break;
+        if (t.n_kb > 0) {
+          // correction terms: complete once the last block's commit has arrived (it covers every earlier MMA)
+          if constexpr (!COARSE) add_tile(TC_COL_CORR, std::false_type{}, corr_empty);
+          // undo the operand scalings (two exact factors, so that neither leaves the range on its own)
+          const int e = lay_exp[t.g][0] + lay_exp[t.g][1], e1 = e / 2, e2 = e - e1;
+          const uint32_t u1 = __float_as_uint(tc_pow2(-e1)), u2 = __float_as_uint(tc_pow2(-e2));
+          const uint64_t w1 = ptx::pack_f2(u1, u1), w2 = ptx::pack_f2(u2, u2);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(ptx::mul_f2(acc[j], w1), w2);
+          if constexpr (ZERO != 0) {
+            const uint64_t mul = ptx::pack_f2(__float_as_uint(y.mul), __float_as_uint(y.mul));
+#pragma unroll
+            for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
+          }
+        }
+        if constexpr (!STORES) {
+          // only the squared norm: straight from the registers (rows and columns outside the matrix hold exact zeros)
+          uint64_t s2[2] = {0ull, 0ull};
+#pragma unroll
+          for (int j = 0; j < 32; ++j) s2[j & 1] = ptx::fma_f2(acc[j], acc[j], s2[j & 1]);
+          float s4[4];
+          ptx::unpack_f2(s2[0], s4[0], s4[1]);
+          ptx::unpack_f2(s2[1], s4[2], s4[3]);
+          if (y.slots != nullptr && t.m0 < y.M) put_sum(y, ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]));
+        } else {
+          // hand the piece over; the epilogue warp has finished with the previous one
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&done_empty[aw], (handed & 1u) ^ 1u, abort_flag));
+          if (!ok) break;
+          ++handed;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const float4 v = __ldcg(part + j * 32 + lane);
-            acc[2 * j] = ptx::add_f2(acc[2 * j], ptx::pack_f2(__float_as_uint(v.x), __float_as_uint(v.y)));
-            acc[2 * j + 1] = ptx::add_f2(acc[2 * j + 1], ptx::pack_f2(__float_as_uint(v.z), __float_as_uint(v.w)));
+            float4 v;
+            ptx::unpack_f2(acc[2 * j], v.x, v.y);
+            ptx::unpack_f2(acc[2 * j + 1], v.z, v.w);
+            tr[lane * 16 + (j ^ (lane & 7))] = v;
           }
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&done_full[aw]);
         }
       }
-      // Epilogue.  Thread i of the warp holds row (lane_base + i), 64 columns.  The warp's piece goes through shared
-      // memory 16 columns at a time: thread i writes its 4 float4 groups with the group index XOR-ed by (i / 2 mod 4)
-      // (conflict-free 128-bit stores), then the warp reads the piece back transposed, so that the output is written,
-      // and the inputs of the epilogue are read, in a coalesced pattern: the warp walks over its rows eight at a
-      // time, lanes 4g..4g+3 take row 8 step + g, 4 consecutive columns per lane.  The loads of the four steps
-      // are issued together (rows past the end are clamped, their results dropped).
-      double ss_tile = 0.0;
-      if constexpr (!epi_stores<Epi>::value) {
-        // only the squared norm: straight from the registers (rows and columns outside the matrix hold exact zeros)
-        uint64_t s2[2] = {0ull, 0ull};
+      if (!STORES && ok) leave(t.g);
+    } else {
+      ptx::setmaxnreg_dec<TC_REGS_EPI>();
+      // ------------------------------------------------------------ epilogue
+      // The warp walks over its 32 rows two at a time: lanes 16 h .. +15 take row 2 step + h, 4 consecutive columns per lane, so
+      // that every access is two runs of 256 bytes.  The loads of eight steps are issued together (rows past the end are
+      // clamped, their results dropped).
+      if constexpr (STORES) {
+        uint32_t taken = 0;
+        for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+          const int g_before = t.g;
+          locate(unit, t);
+          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
+          ++visited;
+          const TcLayer<Epi> &y = grp.l[t.g];
+          const Epi &epi = y.epi;
+          const int row0 = t.m0 + lane_base + (lane >> 4), col = t.n0 + col_base + 4 * (lane & 15);
+          // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
+          // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
+          const bool col_in = col < epi.ldc;
+          if (t.m0 + lane_base + lane < y.M) {          // this lane's row of the epilogue inputs, on its way to L2
 #pragma unroll
-        for (int j = 0; j < 32; ++j) s2[j & 1] = ptx::fma_f2(acc[j], acc[j], s2[j & 1]);
-        float s4[4];
-        ptx::unpack_f2(s2[0], s4[0], s4[1]);
-        ptx::unpack_f2(s2[1], s4[2], s4[3]);
-        ss_tile = ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]);
-      } else {
-        float *C = epi.C + (size_t)t.z * y.c_split_stride;
-        float ssf = 0.f;
-        uint32_t mx = 0u;                  // largest magnitude stored by this thread
-        float h_scale = 0.f;               // scaling of the planes of the result, if they are wanted
-        if constexpr (epi_planes<Epi>::value) {
-          if (epi.H != nullptr) h_scale = tc_scale_of(*epi.h_exp);
-        }
-        // only the copy out of the registers exists four times: one pass of this code is all that a small product runs, and it
-        // has to be fetched (the whole body four times over cost such products 2 us)
-#pragma unroll 1
-        for (int h = 0; h < 4; ++h) {
-          __syncwarp();
-          auto stash = [&](auto H) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) tr[lane * 4 + (j ^ ((lane >> 1) & 3))] = acc_at(decltype(H)::value * 4 + j);
-          };
-          switch (h) {
-            case 0: stash(std::integral_constant<int, 0>{}); break;
-            case 1: stash(std::integral_constant<int, 1>{}); break;
-            case 2: stash(std::integral_constant<int, 2>{}); break;
-            default: stash(std::integral_constant<int, 3>{}); break;
+            for (int h = 0; h < 2; ++h) {
+              const int c = t.n0 + col_base + h * 32;
+              if (c < epi.ldc) epi.prefetch(t.m0 + lane_base + lane, c);
+            }
           }
-          __syncwarp();
-          const int col = n0 + h * 16 + 4 * (lane & 3);
-          if (col < n_pad) {
-            constexpr int BATCH = 4;                               // row steps whose loads are in flight together
-            {
-              float4 in[BATCH][Epi::kInputs > 0 ? Epi::kInputs : 1];
-#pragma unroll
-              for (int i = 0; i < BATCH; ++i) {
-                const int r = 8 * i + (lane >> 2);
-                if constexpr (!Epi::kDirect) epi.load(min(m0 + lane_base + r, y.M - 1), col, in[i]);
-              }
-#pragma unroll
-              for (int i = 0; i < BATCH; ++i) {
-                const int r = 8 * i + (lane >> 2);
-                const int row = m0 + lane_base + r;
-                float4 o = tr[r * 4 + ((lane & 3) ^ ((r >> 1) & 3))];
-                if constexpr (epi_sumsq_acc<Epi>::value) {
-                  if (row < y.M) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&done_full[aw], taken & 1u, abort_flag));
+          if (!ok) break;
+          ++taken;
+          bool whole = true;
+          if (t.slice >= 0) {
+            // contraction slice of a tail tile: park the piece; the last warp to arrive sums the slices
+            const int t_idx = t.out - y.tail_begin, u = t_idx * y.tail_split + t.slice;
+            float4 *mine = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)u * WARPS + piece) * 512;
+#pragma unroll 4
+            for (int j = 0; j < 16; ++j) mine[j * 32 + lane] = tr[j * 32 + lane];
+            __threadfence();
+            __syncwarp();
+            int prev = 0;
+            if (lane == 0) prev = atomicAdd(y.tail_count + t_idx * WARPS + piece, 1);
+            prev = __shfl_sync(0xffffffffu, prev, 0);
+            whole = prev == y.tail_split - 1;
+            if (whole) {
+              __threadfence();
+              if (lane == 0) y.tail_count[t_idx * WARPS + piece] = 0;
+              const float4 *part = reinterpret_cast<const float4 *>(y.tail_ws) + ((size_t)t_idx * y.tail_split * WARPS + piece) * 512;
+#pragma unroll 4
+              for (int j = 0; j < 16; ++j) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int sl = 0; sl < y.tail_split; ++sl) {
+                  const float4 v = __ldcg(part + (size_t)sl * WARPS * 512 + j * 32 + lane);
+                  a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
                 }
-                if constexpr (!Epi::kDirect) o = epi.apply(col, o, in[i]);
-                if (row < y.M) {
+                tr[j * 32 + lane] = a;
+              }
+              __syncwarp();
+            }
+          }
+          if (whole) {
+            float *C = epi.C + (size_t)t.z * y.c_split_stride;
+            float ssf = 0.f;
+            uint32_t mx = 0u;                  // largest magnitude stored by this thread
+            float h_scale = 0.f;               // scaling of the planes of the result, if they are wanted
+            if constexpr (epi_planes<Epi>::value) {
+              if (epi.H != nullptr) h_scale = tc_scale_of(*epi.h_exp);
+            }
+            if (col_in) {
+#pragma unroll 1
+              for (int s0 = 0; s0 < 16; s0 += 8) {
+                float4 in[8][Epi::kInputs > 0 ? Epi::kInputs : 1];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  if constexpr (!Epi::kDirect) epi.load(min(row0 + 2 * (s0 + i), y.M - 1), col, in[i]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  const int r = 2 * (s0 + i) + (lane >> 4), row = row0 + 2 * (s0 + i);
+                  float4 o = tr[r * 16 + ((lane & 15) ^ (r & 7))];
+                  if (row >= y.M) continue;
+                  if constexpr (epi_sumsq_acc<Epi>::value) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
+                  if constexpr (!Epi::kDirect) o = epi.apply(col, o, in[i]);
                   if (Epi::kSumsq && !epi_sumsq_acc<Epi>::value) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
                   *reinterpret_cast<float4 *>(C + (size_t)row * epi.ldc + col) = o;
                   if constexpr (epi_planes<Epi>::value) {
@@ -683,20 +706,20 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
                 }
               }
             }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&done_empty[aw]);            // the piece has been read
+            if constexpr (epi_amax<Epi>::value) {
+              if (epi.amax != nullptr) commit_amax(mx, epi.amax);      // the output is an operand of a later product
+            }
+            if (Epi::kSumsq && y.slots != nullptr && t.m0 < y.M) put_sum(y, (double)ssf);
+          } else {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&done_empty[aw]);
           }
         }
-        ss_tile = (double)ssf;
-        if constexpr (epi_amax<Epi>::value) {
-          if (epi.amax != nullptr) commit_amax(mx, epi.amax);      // the output is an operand of a later product
-        }
-      }
-      if (Epi::kSumsq && y.slots != nullptr && m0 < y.M) {
-        ss_tile = warp_sum(ss_tile);
-        const int tiles_n = (y.N + TC_BN - 1) / TC_BN;
-        if (lane == 0) y.slots[((size_t)(m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw] = ss_tile;
+        if (ok) leave(t.g);
       }
     }
-    if (ok) leave(t.g);
   }
   ptx::tc_fence_before_sync();
   // neither block of a pair leaves while the other may still arrive on its barriers or read its shared memory

@@ -263,24 +263,6 @@ static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
   return PDADMM_OK;
 }
 
-// Launches a kernel of an iteration with a priority above the products': its blocks go to the SMs as soon as one has room,
-// beside the products of other lanes, instead of behind them.  (The work distributor serves equal priorities in the order of
-// arrival, and a product's blocks fill the queue.)
-template <class... P, class... A>
-static void launch_first(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args) {
-  static const int top = [] { int lo = 0, hi = 0; cudaDeviceGetStreamPriorityRange(&lo, &hi); return hi; }();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute a[2];
-  a[0].id = cudaLaunchAttributePriority;
-  a[0].val.priority = top;
-  // the products' division of the SM's memory between L1 and shared memory: blocks with another one wait until the SM is empty
-  a[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  a[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
-  cfg.attrs = a; cfg.numAttrs = 2;
-  cudaLaunchKernelEx(&cfg, kern, P(args)...);            // errors surface at the call's end (cudaGetLastError)
-}
-
 static inline int ew_grid(size_t n_items) {
   return (int)std::max<size_t>(1, std::min<size_t>(ceil_div((int64_t)n_items, EW_THREADS), 148 * 8));
 }
@@ -504,7 +486,7 @@ static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t ro
                        const Planes &pl, bool lo_too = true) {
   const size_t n8 = rows * ld / 8;
   Launch l(c, KC_PLANES, st, (lo_too ? 8.0 : 6.0) * rows * cols, 0);
-  launch_first(st, rows_planes_kernel, dim3(ew_grid(n8)), 256, 0, x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
+  rows_planes_kernel<<<dim3(ew_grid(n8)), 256, 0, st>>>(x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
 }
 // Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel).
 // From 2^20 elements on: below, the launch costs more than it saves.
@@ -523,7 +505,7 @@ static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, const std:
   }
   if (n == 0) return;
   Launch l(c, KC_PLANES, st, 0, 0);
-  launch_first(st, check_planes_kernel, dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, g);
+  check_planes_kernel<<<dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, st>>>(g);
 }
 static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
   PD_TRY(dev_alloc(c, &pl->hi, n, zero));
@@ -564,7 +546,7 @@ static int gemm_nodes(pdadmm_ctx *c, int cls, cudaStream_t st, std::vector<Prod<
       }
       if (p.slots == nullptr) continue;
       Launch l(c, KC_SMALL, st, 8.0 * grid.x * grid.y, 0);
-      launch_first(st, finish_sum_kernel, dim3(1), FIN_THREADS, 0, p.slots, (int)(grid.x * grid.y), p.step);
+      finish_sum_kernel<<<1, FIN_THREADS, 0, st>>>(p.slots, (int)(grid.x * grid.y), p.step);
     }
     return PDADMM_OK;
   }
@@ -751,7 +733,7 @@ static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     bytes += (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out);
   }
   Launch k(c, KC_AXPY, st, bytes, 0);
-  launch_first(st, pstep_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g);
+  pstep_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
@@ -777,7 +759,7 @@ static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       bytes += (c->int_operands ? 8.0 + 2.0 * c->code_bytes : 12.0 + 2.0 * c->code_bytes) * N * ly.n_in;
     }
     Launch k(c, KC_QUANT, st, bytes, 0);
-    launch_first(st, quant_trial_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->levels, c->code_bytes == 2,
+    quant_trial_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->levels, c->code_bytes == 2,
                  c->neg_levels);
   }
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
@@ -901,7 +883,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
     }
     Launch k(c, KC_GRADW_REDUCE, st, bytes, 0);
-    launch_first(st, reduce_gradW_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->nu);
+    reduce_gradW_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->nu);
   }
   if (c->reduce != nullptr) {
     // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
@@ -954,7 +936,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
       const int nbw = (int)std::min<int64_t>(ceil_div((int64_t)n4w, EW_THREADS), 2 * c->n_sms);
       // rows in as many blocks as keep the SMs busy, at least 16 of them each
-      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 3, ceil_div(N, 16));
+      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 16));
       const int rows_per_block = (int)ceil_div(N, n_blocks), nbr = (int)ceil_div(N, rows_per_block);
       const int ld4 = ly.ld_out / 4, n_sub = std::min(EW_THREADS / std::min(ld4, EW_THREADS), COLSUM_MAX_SUB);
       if (n_sub > 1) sh = std::max(sh, (size_t)n_sub * ly.ld_out * sizeof(double));
@@ -969,7 +951,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     }
     {
       Launch k(c, KC_COLSUM, st, bytes, 0);
-      launch_first(st, theta_step_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, g);
+      theta_step_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, st>>>(g);
     }
     if (c->reduce != nullptr) {
       // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
@@ -982,7 +964,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       }
     }
     Launch k(c, KC_SMALL, st, bias_bytes, 0);
-    launch_first(st, finalize_bias_kernel, dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, gb,
+    finalize_bias_kernel<<<dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, st>>>(gb,
                  1.0 / (double)c->N_total);
   }
   return PDADMM_OK;
@@ -1007,8 +989,8 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
                       c->table_step, c->table_size};
   const dim3 grid((unsigned)blocks, (unsigned)n);
-  if (c->table_size > 0) launch_first(st, zqu_table_kernel, grid, EW_THREADS, c->table_size * sizeof(float), g, prm);
-  else launch_first(st, zqu_kernel, grid, EW_THREADS, 0, g, prm);
+  if (c->table_size > 0) zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), st>>>(g, prm);
+  else zqu_kernel<<<grid, EW_THREADS, 0, st>>>(g, prm);
 }
 static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
   Layer &ly = c->layers[c->L - 1];
@@ -2130,7 +2112,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       const size_t n4 = (size_t)M * ldc / 4;
       Group<GradWSum> g;
       g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
-      launch_first(st, reduce_gradW_kernel, dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, g, 1.0f);
+      reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
     }
     double h = 0;
     PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
