@@ -71,7 +71,7 @@ constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
 constexpr int TC_TR_BYTES = 8 * 32 * 64 * 4;                   // finished tile: 8 warps x 32 rows x 64 columns
 constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 512 /* barriers */;
-static_assert(8 * (2 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
+static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 2 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -105,6 +105,12 @@ struct TcOperand {
 // One launch works on the same product of several layers, whose output tiles form one sequence of work units: a small
 // problem's layers fill the GPU together, and a large one has one partly filled last round instead of one per layer.
 constexpr int TC_MAX_GROUP = 16;
+constexpr int TC_SUM_CHUNK = 1024;
+inline size_t tc_sum_slots(int64_t M, int64_t N) {
+  const size_t n = (size_t)(ceil_div(M, TC_BM) * ceil_div(N, TC_BN)) * TC_ACC_WARPS;
+  return n + n / TC_SUM_CHUNK + 1;
+}
+inline size_t tc_sum_counters(int64_t M, int64_t N) { return 2 + tc_sum_slots(M, N) / TC_SUM_CHUNK + 1; }
 template <class Epi>
 struct TcLayer {
   CUtensorMap a, alo, b, blo;      // planes of the operands
@@ -117,10 +123,10 @@ struct TcLayer {
   float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
   Epi epi;
   // Sums of squares (Epi::kSumsq and slots != null): one slot per 128-row tile, column tile and accumulate warp, written by
-  // whichever block has the tile; the block that completes the layer (`done`, zero before and after) adds them in index order
-  // and passes the sum to `step`.  Neither depends on how the tiles were shared out.
-  double *slots;
-  int *done;
+  // whichever block has the tile; the warp that completes the layer adds them in index order and passes the sum to `step`.
+  // Neither depends on how the tiles were shared out.
+  double *slots;          // tc_sum_slots() of them
+  int *done;              // tc_sum_counters() of them, zero before and after
   Step step;
   // Tail balancing (one layer, n_split == 1): output tiles from tail_begin on are cut into tail_split contraction
   // slices, one work unit each, so that the last, partly filled round of the persistent grid is shorter.
@@ -181,8 +187,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint64_t *bars = reinterpret_cast<uint64_t *>(tr_base + TC_TR_BYTES);
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
   uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
-  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1;
-  uint64_t *done_full = team_bar + 1, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
+  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *split_bar = drain_bar + 1;
+  uint64_t *done_full = split_bar + STAGES, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
@@ -192,38 +198,11 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   const int unit0 = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x), unit_step = (int)(PAIR ? gridDim.x >> 1 : gridDim.x);
   const int n_units = grp.l[grp.n - 1].unit_end;
 
-  // scaling exponents of every layer's operands (written by earlier kernels of the stream), and whether the planes made with
-  // them are usable; the same for every block
-  __shared__ int lay_exp[TC_MAX_GROUP][2];
-  __shared__ double team_scratch[1 + TC_ACC_WARPS];
-  __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
-  bool my_split = false;
-  // (only of layers this block works on: the step of a finished layer may already have changed the words of the others)
-  if (threadIdx.x < (unsigned)grp.n) {
-    int split = 0;
-    const int g = (int)threadIdx.x, begin = g > 0 ? grp.l[g - 1].unit_end : 0;
-    const int ahead = (unit0 - begin) % unit_step, first = begin + (ahead < 0 ? ahead + unit_step : ahead);
-    const bool has_unit = first < grp.l[g].unit_end;
-    auto look = [&](const TcOperand &o, int bit) {
-      int e = o.exp ? *o.exp : 0;
-      if (o.amax != nullptr && !tc_planes_usable(*o.amax, e)) {
-        e = tc_scale_exp(*o.amax);
-        if (o.x != nullptr) split |= bit;
-      }
-      return e;
-    };
-    if (has_unit) {
-      lay_exp[g][0] = look(grp.l[g].oa, 1);
-      lay_exp[g][1] = look(grp.l[g].ob, 2);
-      lay_split[g] = split;
-      my_split = split != 0;
-    }
-  }
-  const bool any_split = __syncthreads_or(my_split);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      ptx::mbar_init(&full_bar[s], 1 + (any_split ? CG * TC_SPLIT_WARPS : 0));
+      ptx::mbar_init(&full_bar[s], 1);
       ptx::mbar_init(&empty_bar[s], 1);
+      ptx::mbar_init(&split_bar[s], CG * TC_SPLIT_WARPS);
     }
     for (int b = 0; b < TC_ACC_BUFS; ++b) {
       ptx::mbar_init(&acc_full[b], 1);
@@ -231,25 +210,51 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     }
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
-    ptx::mbar_init(team_bar, TC_ACC_WARPS);
     for (int w = 0; w < TC_ACC_WARPS; ++w) {
       ptx::mbar_init(&done_full[w], 1);
       ptx::mbar_init(&done_empty[w], 1);
     }
     *abort_flag = 0;
+    ptx::fence_barrier_init();
+  }
+  if (warp == 1) ptx::tmem_alloc<CG>(tmem_slot, TC_TMEM_COLS);
+  // Scaling exponents of every layer's operands (written by earlier kernels of the stream), and whether the planes made with
+  // them are usable; only of layers this block works on: the step of a finished layer may already have changed the words of
+  // the others.
+  __shared__ int lay_exp[TC_MAX_GROUP][2];
+  __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
+  ptx::grid_wait();                                   // everything above runs while the previous kernel finishes
+  if (warp == 2 && lane < grp.n) {
+    const TcLayer<Epi> &y = grp.l[lane];
+    const int begin = lane > 0 ? grp.l[lane - 1].unit_end : 0;
+    const int ahead = (unit0 - begin) % unit_step, first = begin + (ahead < 0 ? ahead + unit_step : ahead);
+    lay_split[lane] = 0;
+    if (first < y.unit_end) {
+      const int ea = y.oa.exp ? *y.oa.exp : 0, eb = y.ob.exp ? *y.ob.exp : 0;
+      const uint32_t ma = y.oa.amax ? *y.oa.amax : 0u, mb = y.ob.amax ? *y.ob.amax : 0u;
+      const bool good_a = y.oa.amax == nullptr || tc_planes_usable(ma, ea), good_b = y.ob.amax == nullptr || tc_planes_usable(mb, eb);
+      lay_exp[lane][0] = good_a ? ea : tc_scale_exp(ma);
+      lay_exp[lane][1] = good_b ? eb : tc_scale_exp(mb);
+      lay_split[lane] = (!good_a && y.oa.x != nullptr ? 1 : 0) | (!good_b && y.ob.x != nullptr ? 2 : 0);
+    }
+  }
+  if (warp == 3 && lane == 0) {
     // One thread reads the error word for the whole block, so that all warps take the same path: every block still
     // allocates and releases its tensor memory and passes both block-wide barriers.
     *skip_flag = *reinterpret_cast<volatile int *>(grp.error) != 0;
-    ptx::fence_barrier_init();
-    ptx::prefetch_tmap(&grp.l[0].a);
-    ptx::prefetch_tmap(&grp.l[0].b);
+    int g = 0;
+    while (g + 1 < grp.n && unit0 >= grp.l[g].unit_end) ++g;
+    ptx::prefetch_tmap(&grp.l[g].a);
+    ptx::prefetch_tmap(&grp.l[g].b);
+    if (A_LO) ptx::prefetch_tmap(&grp.l[g].alo);
+    if (B_LO) ptx::prefetch_tmap(&grp.l[g].blo);
   }
-  if (warp == 1) ptx::tmem_alloc<CG>(tmem_slot, TC_TMEM_COLS);
   ptx::tc_fence_before_sync();
   if constexpr (PAIR) ptx::cluster_sync();          // the barriers of both blocks are in place
   else __syncthreads();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  ptx::grid_release();
 
   // Work unit -> its layer, row and column tile origin, first and number of K blocks, contraction slice; a unit is an output
   // tile or, in the tail, one contraction slice of an output tile.  Units are visited in ascending order.
@@ -290,7 +295,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       if (lane == 0) {
         int s = 0, it = 0;
         uint32_t ph = 1;                                // phase of the stage's previous use
-        bool ok = true;
+        bool ok = true, any_split = false;
+        for (int g = 0; g < grp.n; ++g) any_split |= lay_split[g] != 0;
         // `boxes` boxes of 64 output indices from o0 on
         auto load = [&](uint8_t *dst, const CUtensorMap *map, bool mn, int o0, int k0, int boxes) {
           const uint32_t bar = PAIR ? ptx::cluster_addr(&full_bar[s], 0) : ptx::smem_u32(&full_bar[s]);
@@ -301,14 +307,14 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
         for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
           locate(unit, t);
           const TcLayer<Epi> &y = grp.l[t.g];
-          const bool split_a = any_split && (lay_split[t.g] & 1), split_b = any_split && (lay_split[t.g] & 2);
+          const bool split_a = lay_split[t.g] & 1, split_b = lay_split[t.g] & 2;
           const uint32_t tx = CG * (uint32_t)((split_a ? 0 : A_PLANES * TC_PLANE_BYTES) + (split_b ? 0 : B_PLANES * B_PLANE_BYTES));
           for (int kb = 0; kb < t.n_kb; ++kb, ++it) {
             if (it >= STAGES && !ptx::mbar_wait(&empty_bar[s], ph, abort_flag)) { ok = false; break; }
             uint8_t *st = smem + s * STAGE_BYTES;
             const int k0 = t.k_begin + kb * TC_BK;
             const int nb = t.n0 + (int)rank * BN;          // columns of B that this block loads
-            if (rank == 0) ptx::mbar_expect_tx(&full_bar[s], tx);       // the bytes of both blocks
+            if (rank == 0 && !any_split) ptx::mbar_expect_tx(&full_bar[s], tx);       // the bytes of both blocks
             if (!split_a) {
               load(st, &y.a, A_MN, t.m0, k0, 2);
               if (A_LO) load(st + TC_PLANE_BYTES, &y.alo, A_MN, t.m0, k0, 2);
@@ -317,6 +323,12 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
               load(st + B_OFF, &y.b, B_MN, nb, k0, BN / 64);
               if (B_LO) load(st + B_OFF + B_PLANE_BYTES, &y.blo, B_MN, nb, k0, BN / 64);
             }
+            if (rank == 0 && any_split) {
+              // what the splitting warps of both blocks have written comes before this arrival
+              if (!ptx::mbar_wait(&split_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+              if (PAIR) ptx::fence_cluster();
+              ptx::mbar_expect_tx(&full_bar[s], tx);
+            }
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
         }
@@ -324,7 +336,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           // copies in flight must land before shared memory is released (block 1 of a pair is held by the cluster barrier at
           // the end).  A barrier that the splitting warps or the other block feed as well may never complete: its copies
           // are waited for until the limit of the wait.
-          for (int j = max(it - STAGES, 0); j < it; ++j)
+          for (int j = max(it - STAGES, 0); j < it; ++j)      // (a stage that never got its arrival runs into the limit)
             ptx::mbar_wait(&full_bar[j % STAGES], (j / STAGES) & 1, abort_flag, 200000000ll, false);
         }
       }
@@ -344,6 +356,9 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
         constexpr uint32_t step_a = (A_MN ? 2048u : 32u) >> 4, step_b = (B_MN ? 2048u : 32u) >> 4;
         constexpr uint32_t plane_a = TC_PLANE_BYTES >> 4, plane_b = B_PLANE_BYTES >> 4;
         bool ok = true;
+        int splits = 0;
+        for (int g = 0; g < grp.n; ++g) splits |= lay_split[g];
+        const bool any_split = __any_sync(0xffffffffu, splits != 0);
         // running state: stage s with phase bit sp, accumulator buffer b with phase bit bp (of its *previous* use)
         int s = 0, b = 0, ti = 0, used = 0;
         uint32_t sp = 0, bp = 1;
@@ -413,10 +428,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           ptx::mbar_wait(drain_bar, 0, abort_flag, 200000000ll, false);
         }
       }
-    } else if (any_split) {
+    } else {
       // -------------------------------------------------------------- planes of a refused operand (two warps)
-      // Eight consecutive values at a time, rows in order, so that a warp reads whole rows; written where TMA would have
-      // put them (16-byte chunk c of a 128-byte row r at position c ^ (r mod 8)).
+      // Once a layer of this block needs them, they and the producer go through every stage together: a waiter that lags by
+      // more than one phase of a barrier would take an earlier completion of the same parity for its own.
       const int t = threadIdx.x - 32 * TC_SPLIT0;
       auto split_tile = [&](const TcOperand &o, bool mn, bool lo_too, float scale, uint8_t *dst, int boxes, int o0, int k0, int n_outer, int n_k) {
         // K-major: 64 or 128 rows of 8 chunks, inner = contraction; MN-major: 64 rows of 8 or 16 chunks, inner = output index
@@ -439,7 +454,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       };
       int s = 0, it = 0;
       uint32_t ph = 1;
-      bool ok = true;
+      bool ok = false;
+      for (int g = 0; g < grp.n; ++g) ok |= lay_split[g] != 0;
       Tile u;
       for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
         locate(unit, u);
@@ -453,10 +469,12 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           const int k0 = u.k_begin + kb * TC_BK;
           if (split & 1) split_tile(y.oa, A_MN, A_LO, scale_a, st, 2, u.m0, k0, y.M, y.K);
           if (split & 2) split_tile(y.ob, B_MN, B_LO, scale_b, st + B_OFF, BN / 64, u.n0 + (int)rank * BN, k0, y.N, y.K);
-          ptx::fence_proxy_async_smem();
-          if (PAIR) ptx::fence_cluster();
+          if (split != 0) {
+            ptx::fence_proxy_async_smem();
+            if (PAIR) ptx::fence_cluster();
+          }
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(&full_bar[s], 0));
+          if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(&split_bar[s], 0));      // (every stage: the phases stay in step)
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
@@ -472,56 +490,37 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 16;
     bool ok = true;
     Tile t;
-    int visited = 0;                                   // units of layer t.g that this block has finished
-    // The eight warps that know the sums of squares (the epilogue warps; the accumulate warps if nothing is stored), bounded
-    // like every other wait.
-    uint32_t team_ph = 0;
-    auto team_sync = [&]() {
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(team_bar);
-      const bool there = ptx::mbar_wait(team_bar, team_ph, abort_flag);
-      team_ph ^= 1u;
-      return __all_sync(0xffffffffu, there) != 0;
-    };
-    // The block has no further unit of layer g: if every unit of the layer is finished with this, add the slots.
-    auto leave = [&](int g) {
-      const TcLayer<Epi> &y = grp.l[g];
-      if (!Epi::kSumsq || y.slots == nullptr || visited == 0) return true;
-      constexpr int n_threads = 32 * TC_ACC_WARPS;
-      const int tid = aw * 32 + lane;
-      volatile int *last = reinterpret_cast<volatile int *>(team_scratch);
-      volatile double *part = team_scratch + 1;
-      __threadfence();
-      if (!team_sync()) return false;
-      if (tid == 0) {
-        const int units = (y.unit_end - (g > 0 ? grp.l[g - 1].unit_end : 0)) * CG;
-        const int before = atomicAdd(y.done, visited);
-        *last = before + visited == units;
-      }
-      if (!team_sync()) return false;
-      if (*last != 0) {
-        __threadfence();
-        const int n = (y.M + TC_BM - 1) / TC_BM * ((y.N + TC_BN - 1) / TC_BN) * TC_ACC_WARPS;
-        double v = 0.0;
-#pragma unroll 4
-        for (int i = tid; i < n; i += n_threads) v += __ldcg(y.slots + i);
-        v = warp_sum(v);
-        if (lane == 0) part[aw] = v;
-        if (!team_sync()) return false;
-        if (tid == 0) {
-          double sum = 0.0;
-          for (int i = 0; i < TC_ACC_WARPS; ++i) sum += part[i];
-          *y.done = 0;
-          finish_step(y.step, sum);
-        }
-      }
-      visited = 0;
-      return team_sync();                              // the scratch is free again
-    };
+    // A warp leaves its part of the tile's sum of squares in its slot.  Counters find the last one to arrive: it adds the
+    // slots, 1024 at a time in two levels, always in index order.  The arrival releases the slot and acquires the others'.
     auto put_sum = [&](const TcLayer<Epi> &y, double v) {
       v = warp_sum(v);
-      const int tiles_n = (y.N + TC_BN - 1) / TC_BN;
-      if (lane == 0) y.slots[((size_t)(t.m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw] = v;
+      const int tiles_n = (y.N + TC_BN - 1) / TC_BN, n = (y.M + TC_BM - 1) / TC_BM * tiles_n * TC_ACC_WARPS;
+      const int slot = ((t.m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw;
+      const int chunk = slot / TC_SUM_CHUNK, n_chunks = (n + TC_SUM_CHUNK - 1) / TC_SUM_CHUNK;
+      int last = 0;
+      if (lane == 0) {
+        y.slots[slot] = v;
+        last = ptx::arrive_count(y.done + 1 + chunk) == min(TC_SUM_CHUNK, n - chunk * TC_SUM_CHUNK) - 1;
+      }
+      if (!__shfl_sync(0xffffffffu, last, 0)) return;
+      auto add_up = [&](const double *from, int count) {
+        double sum = 0.0;
+#pragma unroll 8
+        for (int i = lane; i < count; i += 32) sum += __ldcg(from + i);
+        return warp_sum(sum);
+      };
+      double sum = add_up(y.slots + (size_t)chunk * TC_SUM_CHUNK, min(TC_SUM_CHUNK, n - chunk * TC_SUM_CHUNK));
+      if (lane == 0) {
+        y.done[1 + chunk] = 0;
+        if (n_chunks > 1) y.slots[n + chunk] = sum;
+        last = n_chunks == 1 || ptx::arrive_count(y.done) == n_chunks - 1;
+      }
+      if (!__shfl_sync(0xffffffffu, last, 0)) return;
+      if (n_chunks > 1) sum = add_up(y.slots + n, n_chunks);
+      if (lane == 0) {
+        *y.done = 0;
+        finish_step(y.step, sum);
+      }
     };
     if (accumulates) {
       ptx::setmaxnreg_inc<TC_REGS_ACC>();
@@ -529,12 +528,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       int b = 0;
       uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; tiles handed over so far
       for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
-        const int g_before = t.g;
         locate(unit, t);
-        if (!STORES) {
-          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
-          ++visited;
-        }
         const TcLayer<Epi> &y = grp.l[t.g];
         const int n_grp = COARSE ? (t.n_kb > 0 ? 1 : 0) : t.n_kb;   // read-outs of the main accumulator for this tile
         uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
@@ -611,7 +605,6 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           if (lane == 0) ptx::mbar_arrive(&done_full[aw]);
         }
       }
-      if (!STORES && ok) leave(t.g);
     } else {
       ptx::setmaxnreg_dec<TC_REGS_EPI>();
       // ------------------------------------------------------------ epilogue
@@ -621,12 +614,9 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       if constexpr (STORES) {
         uint32_t taken = 0;
         for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
-          const int g_before = t.g;
           locate(unit, t);
-          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
-          ++visited;
           const TcLayer<Epi> &y = grp.l[t.g];
-          const Epi &epi = y.epi;
+          const Epi epi = y.epi;
           const int row0 = t.m0 + lane_base + (lane >> 4), col = t.n0 + col_base + 4 * (lane & 15);
           // columns up to the leading dimension are written: those from N on come out as exact zeros (zero-filled
           // operand rows, zero padding of the epilogue inputs), which keeps the padding of every matrix zero
@@ -638,6 +628,18 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
               if (c < epi.ldc) epi.prefetch(t.m0 + lane_base + lane, c);
             }
           }
+          // the inputs of the first eight steps are on their way before the tile is complete
+          float4 in[8][Epi::kInputs > 0 ? Epi::kInputs : 1];
+          auto load_inputs = [&](int s0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if constexpr (!Epi::kDirect) epi.load(min(row0 + 2 * (s0 + i), y.M - 1), col, in[i]);
+          };
+          float h_scale = 0.f;               // scaling of the planes of the result, if they are wanted
+          if constexpr (epi_planes<Epi>::value) {
+            if (epi.H != nullptr) h_scale = tc_scale_of(*epi.h_exp);
+          }
+          if (col_in) load_inputs(0);
           ok = __all_sync(0xffffffffu, ptx::mbar_wait(&done_full[aw], taken & 1u, abort_flag));
           if (!ok) break;
           ++taken;
@@ -674,17 +676,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             float *C = epi.C + (size_t)t.z * y.c_split_stride;
             float ssf = 0.f;
             uint32_t mx = 0u;                  // largest magnitude stored by this thread
-            float h_scale = 0.f;               // scaling of the planes of the result, if they are wanted
-            if constexpr (epi_planes<Epi>::value) {
-              if (epi.H != nullptr) h_scale = tc_scale_of(*epi.h_exp);
-            }
             if (col_in) {
 #pragma unroll 1
               for (int s0 = 0; s0 < 16; s0 += 8) {
-                float4 in[8][Epi::kInputs > 0 ? Epi::kInputs : 1];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                  if constexpr (!Epi::kDirect) epi.load(min(row0 + 2 * (s0 + i), y.M - 1), col, in[i]);
+                if (s0 > 0) load_inputs(s0);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                   const int r = 2 * (s0 + i) + (lane >> 4), row = row0 + 2 * (s0 + i);
@@ -717,7 +712,6 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             if (lane == 0) ptx::mbar_arrive(&done_empty[aw]);
           }
         }
-        if (ok) leave(t.g);
       }
     }
   }

@@ -116,7 +116,7 @@ struct Layer {
   uint32_t *amax_p = nullptr, *amax_r = nullptr;
   // largest magnitudes of an iteration's g, W g, G and d: zero before the kernel that writes the matrix
   uint32_t *w_g = nullptr, *w_wg = nullptr, *w_G = nullptr, *w_d = nullptr;
-  int *done = nullptr;             // counters of finished blocks (products; trial; gradient sum), zero between kernels
+  int *done = nullptr;             // counters of finished blocks (trial, gradient sum, then products), zero between kernels
   int n_split = 1, k_chunk = 0;
 };
 
@@ -263,6 +263,19 @@ static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
   return PDADMM_OK;
 }
 
+// Launches a kernel of an iteration so that it may start while the one before it in the stream finishes: the kernel calls
+// grid_wait() before it touches memory.  (An iteration of a small problem is a chain of a dozen kernels of 5 us.)
+template <class... P, class... A>
+static void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute a;
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &a; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, P(args)...);            // errors surface at the call's end (cudaGetLastError)
+}
+
 static inline int ew_grid(size_t n_items) {
   return (int)std::max<size_t>(1, std::min<size_t>(ceil_div((int64_t)n_items, EW_THREADS), 148 * 8));
 }
@@ -385,11 +398,13 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &gr
   cfg.blockDim = dim3(TC_THREADS);
   cfg.dynamicSmemBytes = TC_SMEM_BYTES;
   cfg.stream = st;
-  cudaLaunchAttribute cluster;
-  cluster.id = cudaLaunchAttributeClusterDimension;
-  cluster.val.clusterDim.x = 2; cluster.val.clusterDim.y = 1; cluster.val.clusterDim.z = 1;
-  cfg.attrs = &cluster;
-  cfg.numAttrs = PAIR ? 1 : 0;
+  cudaLaunchAttribute a[2];
+  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see launch_next
+  a[0].val.programmaticStreamSerializationAllowed = 1;
+  a[1].id = cudaLaunchAttributeClusterDimension;
+  a[1].val.clusterDim.x = 2; a[1].val.clusterDim.y = 1; a[1].val.clusterDim.z = 1;
+  cfg.attrs = a;
+  cfg.numAttrs = PAIR ? 2 : 1;
   PD_CUDA(cudaLaunchKernelEx(&cfg, kern, grp));
   return PDADMM_OK;
 }
@@ -505,7 +520,7 @@ static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, const std:
   }
   if (n == 0) return;
   Launch l(c, KC_PLANES, st, 0, 0);
-  check_planes_kernel<<<dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, st>>>(g);
+  launch_next(st, check_planes_kernel, dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, g);
 }
 static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
   PD_TRY(dev_alloc(c, &pl->hi, n, zero));
@@ -680,7 +695,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
     } else {
       G.push_back(Operand{s.s1, ly.ld_in, nullptr});
     }
-    Prod<EpiGradT> p{N, ly.n_in, ly.n_out, R.back(), operand_W(ly), epi, &s, s.slots, ly.done};
+    Prod<EpiGradT> p{N, ly.n_in, ly.n_out, R.back(), operand_W(ly), epi, &s, s.slots, ly.done + 2};
     p.step = make_step(c, ly, STEP_G2);
     grad.push_back(p);
     bytes += (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in;
@@ -699,7 +714,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
     for (size_t i = 0; i < batch.size(); ++i) {
       Layer &ly = c->layers[batch[i]];
       Scratch &s = scratch_of(c, batch[i]);
-      Prod<decltype(make_epi(0))> p{N, ly.n_out, ly.n_in, G[i], operand_W(ly), make_epi(batch[i]), &s, s.slots + s.n_slots / 2, ly.done};
+      Prod<decltype(make_epi(0))> p{N, ly.n_out, ly.n_in, G[i], operand_W(ly), make_epi(batch[i]), &s, s.slots + s.n_slots / 2, ly.done + 2};
       Step t = make_step(c, ly, STEP_TAU);
       if (c->use_tc) {
         t.w_in = ly.w_g; t.w_out = norm_only ? nullptr : ly.w_wg;
@@ -733,7 +748,7 @@ static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     bytes += (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out);
   }
   Launch k(c, KC_AXPY, st, bytes, 0);
-  pstep_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g);
+  launch_next(st, pstep_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
@@ -754,12 +769,12 @@ static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       // with integer operands p+ and d exist as codes and planes of integers alone
       g.l[n++] = QuantTrial{s.s1, ly.sc, ly.scale, ly.lo, c->int_operands ? nullptr : s.p_new, c->int_operands ? nullptr : s.d, ly.codes,
                             s.codes_new, s.pn_plane, s.d_plane, (uint32_t)n4, c->use_tc && !c->int_operands ? ly.amax_p : nullptr,
-                            ly.w_d, s.slots, ly.done + 1, nb};
+                            ly.w_d, s.slots, ly.done, nb};
       blocks = std::max(blocks, nb);
       bytes += (c->int_operands ? 8.0 + 2.0 * c->code_bytes : 12.0 + 2.0 * c->code_bytes) * N * ly.n_in;
     }
     Launch k(c, KC_QUANT, st, bytes, 0);
-    quant_trial_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->levels, c->code_bytes == 2,
+    launch_next(st, quant_trial_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->levels, c->code_bytes == 2,
                  c->neg_levels);
   }
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
@@ -773,7 +788,7 @@ static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     if (c->use_tc) { epi.H = s.pl0.hi; epi.L = s.pl0.lo; epi.h_exp = s.pl0.exp; }      // planes of the trial's r for the W-gradient
     const Operand D = c->int_operands ? int_operand(s.d_plane, ly.ld_in, ly.scale)      // d = (new code - old code) s
                                       : Operand{s.d, ly.ld_in, c->use_tc ? ly.w_d : nullptr};
-    Prod<EpiAddSumsq> p{N, ly.n_out, ly.n_in, D, operand_W(ly), epi, &s, s.slots + s.n_slots / 2, ly.done};
+    Prod<EpiAddSumsq> p{N, ly.n_out, ly.n_in, D, operand_W(ly), epi, &s, s.slots + s.n_slots / 2, ly.done + 2};
     p.step = make_step(c, ly, STEP_TRIAL);
     p.step.w_in = c->use_tc && !c->int_operands ? ly.w_d : nullptr;
     p.step.host_flag = s.h_flag;
@@ -877,13 +892,13 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       const int nb = ew_grid(n4);
       // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
       g.l[n++] = GradWSum{s.part, ly.n_split, (uint32_t)n4, ly.gradW, c->use_tc ? ly.w_G : nullptr,
-                          c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp), s.slots, ly.done + 2,
+                          c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp), s.slots, ly.done + 1,
                           &ly.sc->sum_G2, nb};
       blocks = std::max(blocks, nb);
       bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
     }
     Launch k(c, KC_GRADW_REDUCE, st, bytes, 0);
-    reduce_gradW_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->nu);
+    launch_next(st, reduce_gradW_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->nu);
   }
   if (c->reduce != nullptr) {
     // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
@@ -915,7 +930,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       const int l = batch[i];
       Layer &ly = c->layers[l];
       Scratch &s = scratch_of(c, l);
-      Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done};
+      Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done + 2};
       p.step = make_step(c, ly, STEP_THETA);
       if (c->use_tc) { p.step.w_in = ly.w_G; p.step.exp_W = ly.Wp.exp; p.step.exp_r = ly.rp.exp; p.step.exp_g = ly.Gp.exp; }
       v.push_back(p);
@@ -951,7 +966,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     }
     {
       Launch k(c, KC_COLSUM, st, bytes, 0);
-      theta_step_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, st>>>(g);
+      launch_next(st, theta_step_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, g);
     }
     if (c->reduce != nullptr) {
       // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
@@ -964,7 +979,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       }
     }
     Launch k(c, KC_SMALL, st, bias_bytes, 0);
-    finalize_bias_kernel<<<dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, st>>>(gb,
+    launch_next(st, finalize_bias_kernel, dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, gb,
                  1.0 / (double)c->N_total);
   }
   return PDADMM_OK;
@@ -989,8 +1004,8 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
                       c->table_step, c->table_size};
   const dim3 grid((unsigned)blocks, (unsigned)n);
-  if (c->table_size > 0) zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), st>>>(g, prm);
-  else zqu_kernel<<<grid, EW_THREADS, 0, st>>>(g, prm);
+  if (c->table_size > 0) launch_next(st, zqu_table_kernel, grid, EW_THREADS, c->table_size * sizeof(float), g, prm);
+  else launch_next(st, zqu_kernel, grid, EW_THREADS, 0, g, prm);
 }
 static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
   Layer &ly = c->layers[c->L - 1];
@@ -1401,7 +1416,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &ly.sc, 1));
     PD_TRY(dev_alloc(c, &ly.w_g, 4));
     ly.w_wg = ly.w_g + 1; ly.w_G = ly.w_g + 2; ly.w_d = ly.w_g + 3;
-    PD_TRY(dev_alloc(c, &ly.done, 4));
+    PD_TRY(dev_alloc(c, &ly.done, 2 + tc_sum_counters(N, std::max(ly.n_in, ly.n_out))));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.g_exp, 1));
     PD_TRY(dev_alloc(c, &ly.amax_p, 1));
     PD_TRY(dev_alloc(c, &ly.amax_r, 1));
@@ -2088,7 +2103,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
     }
     double *res = slots + n_slots - 1;
     int *done;
-    PD_TRY(dev_alloc(c, &done, 1));
+    PD_TRY(dev_alloc(c, &done, tc_sum_counters(M, N)));
     Step step;
     step.kind = STEP_SUM; step.sum = res;
     EpiStoreSumsq epi{dC, ldc};
@@ -2112,7 +2127,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       const size_t n4 = (size_t)M * ldc / 4;
       Group<GradWSum> g;
       g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
-      reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
+      launch_next(st, reduce_gradW_kernel, dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, g, 1.0f);
     }
     double h = 0;
     PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
