@@ -71,7 +71,7 @@ constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
 constexpr int TC_TR_BYTES = 8 * 32 * 64 * 4;                   // finished tile: 8 warps x 32 rows x 64 columns
 constexpr int TC_SMEM_BYTES = TC_STAGE_SPACE + TC_TR_BYTES + 1024 /* alignment slack */ + 512 /* barriers */;
-static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 2 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
+static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -105,12 +105,6 @@ struct TcOperand {
 // One launch works on the same product of several layers, whose output tiles form one sequence of work units: a small
 // problem's layers fill the GPU together, and a large one has one partly filled last round instead of one per layer.
 constexpr int TC_MAX_GROUP = 16;
-constexpr int TC_SUM_CHUNK = 1024;
-inline size_t tc_sum_slots(int64_t M, int64_t N) {
-  const size_t n = (size_t)(ceil_div(M, TC_BM) * ceil_div(N, TC_BN)) * TC_ACC_WARPS;
-  return n + n / TC_SUM_CHUNK + 1;
-}
-inline size_t tc_sum_counters(int64_t M, int64_t N) { return 2 + tc_sum_slots(M, N) / TC_SUM_CHUNK + 1; }
 template <class Epi>
 struct TcLayer {
   CUtensorMap a, alo, b, blo;      // planes of the operands
@@ -123,10 +117,11 @@ struct TcLayer {
   float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
   Epi epi;
   // Sums of squares (Epi::kSumsq and slots != null): one slot per 128-row tile, column tile and accumulate warp, written by
-  // whichever block has the tile; the warp that completes the layer adds them in index order and passes the sum to `step`.
-  // Neither depends on how the tiles were shared out.
-  double *slots;          // tc_sum_slots() of them
-  int *done;              // tc_sum_counters() of them, zero before and after
+  // whichever block has the tile; the block that completes the layer (`done`, zero before and after) adds them in index order
+  // and passes the sum to `step`.  Neither depends on how the tiles were shared out.  (One arrival per block and layer: an
+  // arrival per tile and warp held up the epilogue by 3 us a tile.)
+  double *slots;
+  int *done;
   Step step;
   // Tail balancing (one layer, n_split == 1): output tiles from tail_begin on are cut into tail_split contraction
   // slices, one work unit each, so that the last, partly filled round of the persistent grid is shorter.
@@ -187,7 +182,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint64_t *bars = reinterpret_cast<uint64_t *>(tr_base + TC_TR_BYTES);
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
   uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
-  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *split_bar = drain_bar + 1;
+  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1, *split_bar = team_bar + 1;
   uint64_t *done_full = split_bar + STAGES, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
@@ -210,6 +205,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     }
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
+    ptx::mbar_init(team_bar, TC_ACC_WARPS);
     for (int w = 0; w < TC_ACC_WARPS; ++w) {
       ptx::mbar_init(&done_full[w], 1);
       ptx::mbar_init(&done_empty[w], 1);
@@ -222,6 +218,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   // them are usable; only of layers this block works on: the step of a finished layer may already have changed the words of
   // the others.
   __shared__ int lay_exp[TC_MAX_GROUP][2];
+  __shared__ double team_scratch[1 + TC_ACC_WARPS];
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
   ptx::grid_wait();                                   // everything above runs while the previous kernel finishes
   if (warp == 2 && lane < grp.n) {
@@ -490,37 +487,56 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 32 * 16;
     bool ok = true;
     Tile t;
-    // A warp leaves its part of the tile's sum of squares in its slot.  Counters find the last one to arrive: it adds the
-    // slots, 1024 at a time in two levels, always in index order.  The arrival releases the slot and acquires the others'.
+    int visited = 0;                                   // units of layer t.g that this block has finished
+    // The eight warps that know the sums of squares (the epilogue warps; the accumulate warps if nothing is stored), bounded
+    // like every other wait.
+    uint32_t team_ph = 0;
+    auto team_sync = [&]() {
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(team_bar);
+      const bool there = ptx::mbar_wait(team_bar, team_ph, abort_flag);
+      team_ph ^= 1u;
+      return __all_sync(0xffffffffu, there) != 0;
+    };
+    // The block has no further unit of layer g: if every unit of the layer is finished with this, add the slots.
+    auto leave = [&](int g) {
+      const TcLayer<Epi> &y = grp.l[g];
+      if (!Epi::kSumsq || y.slots == nullptr || visited == 0) return true;
+      constexpr int n_threads = 32 * TC_ACC_WARPS;
+      const int tid = aw * 32 + lane;
+      volatile int *last = reinterpret_cast<volatile int *>(team_scratch);
+      volatile double *part = team_scratch + 1;
+      __threadfence();
+      if (!team_sync()) return false;
+      if (tid == 0) {
+        const int units = (y.unit_end - (g > 0 ? grp.l[g - 1].unit_end : 0)) * CG;
+        const int before = atomicAdd(y.done, visited);
+        *last = before + visited == units;
+      }
+      if (!team_sync()) return false;
+      if (*last != 0) {
+        __threadfence();
+        const int n = (y.M + TC_BM - 1) / TC_BM * ((y.N + TC_BN - 1) / TC_BN) * TC_ACC_WARPS;
+        double v = 0.0;
+#pragma unroll 4
+        for (int i = tid; i < n; i += n_threads) v += __ldcg(y.slots + i);
+        v = warp_sum(v);
+        if (lane == 0) part[aw] = v;
+        if (!team_sync()) return false;
+        if (tid == 0) {
+          double sum = 0.0;
+          for (int i = 0; i < TC_ACC_WARPS; ++i) sum += part[i];
+          *y.done = 0;
+          finish_step(y.step, sum);
+        }
+      }
+      visited = 0;
+      return team_sync();                              // the scratch is free again
+    };
     auto put_sum = [&](const TcLayer<Epi> &y, double v) {
       v = warp_sum(v);
-      const int tiles_n = (y.N + TC_BN - 1) / TC_BN, n = (y.M + TC_BM - 1) / TC_BM * tiles_n * TC_ACC_WARPS;
-      const int slot = ((t.m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw;
-      const int chunk = slot / TC_SUM_CHUNK, n_chunks = (n + TC_SUM_CHUNK - 1) / TC_SUM_CHUNK;
-      int last = 0;
-      if (lane == 0) {
-        y.slots[slot] = v;
-        last = ptx::arrive_count(y.done + 1 + chunk) == min(TC_SUM_CHUNK, n - chunk * TC_SUM_CHUNK) - 1;
-      }
-      if (!__shfl_sync(0xffffffffu, last, 0)) return;
-      auto add_up = [&](const double *from, int count) {
-        double sum = 0.0;
-#pragma unroll 8
-        for (int i = lane; i < count; i += 32) sum += __ldcg(from + i);
-        return warp_sum(sum);
-      };
-      double sum = add_up(y.slots + (size_t)chunk * TC_SUM_CHUNK, min(TC_SUM_CHUNK, n - chunk * TC_SUM_CHUNK));
-      if (lane == 0) {
-        y.done[1 + chunk] = 0;
-        if (n_chunks > 1) y.slots[n + chunk] = sum;
-        last = n_chunks == 1 || ptx::arrive_count(y.done) == n_chunks - 1;
-      }
-      if (!__shfl_sync(0xffffffffu, last, 0)) return;
-      if (n_chunks > 1) sum = add_up(y.slots + n, n_chunks);
-      if (lane == 0) {
-        *y.done = 0;
-        finish_step(y.step, sum);
-      }
+      const int tiles_n = (y.N + TC_BN - 1) / TC_BN;
+      if (lane == 0) y.slots[((size_t)(t.m0 / TC_BM) * tiles_n + t.n0 / TC_BN) * TC_ACC_WARPS + aw] = v;
     };
     if (accumulates) {
       ptx::setmaxnreg_inc<TC_REGS_ACC>();
@@ -528,7 +544,12 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       int b = 0;
       uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; tiles handed over so far
       for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+        const int g_before = t.g;
         locate(unit, t);
+        if (!STORES) {
+          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
+          ++visited;
+        }
         const TcLayer<Epi> &y = grp.l[t.g];
         const int n_grp = COARSE ? (t.n_kb > 0 ? 1 : 0) : t.n_kb;   // read-outs of the main accumulator for this tile
         uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
@@ -605,6 +626,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           if (lane == 0) ptx::mbar_arrive(&done_full[aw]);
         }
       }
+      if (!STORES && ok) leave(t.g);
     } else {
       ptx::setmaxnreg_dec<TC_REGS_EPI>();
       // ------------------------------------------------------------ epilogue
@@ -614,7 +636,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       if constexpr (STORES) {
         uint32_t taken = 0;
         for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+          const int g_before = t.g;
           locate(unit, t);
+          if (t.g != g_before && !leave(g_before)) { ok = false; break; }
+          ++visited;
           const TcLayer<Epi> &y = grp.l[t.g];
           const Epi epi = y.epi;
           const int row0 = t.m0 + lane_base + (lane >> 4), col = t.n0 + col_base + 4 * (lane & 15);
@@ -712,6 +737,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             if (lane == 0) ptx::mbar_arrive(&done_empty[aw]);
           }
         }
+        if (ok) leave(t.g);
       }
     }
   }

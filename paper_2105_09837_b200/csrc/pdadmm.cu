@@ -1416,7 +1416,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &ly.sc, 1));
     PD_TRY(dev_alloc(c, &ly.w_g, 4));
     ly.w_wg = ly.w_g + 1; ly.w_G = ly.w_g + 2; ly.w_d = ly.w_g + 3;
-    PD_TRY(dev_alloc(c, &ly.done, 2 + tc_sum_counters(N, std::max(ly.n_in, ly.n_out))));
+    PD_TRY(dev_alloc(c, &ly.done, 4));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.g_exp, 1));
     PD_TRY(dev_alloc(c, &ly.amax_p, 1));
     PD_TRY(dev_alloc(c, &ly.amax_r, 1));
@@ -2103,7 +2103,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
     }
     double *res = slots + n_slots - 1;
     int *done;
-    PD_TRY(dev_alloc(c, &done, tc_sum_counters(M, N)));
+    PD_TRY(dev_alloc(c, &done, 1));
     Step step;
     step.kind = STEP_SUM; step.sum = res;
     EpiStoreSumsq epi{dC, ldc};
