@@ -121,8 +121,6 @@ struct PStep {
 };
 __global__ void __launch_bounds__(EW_THREADS)
 pstep_kernel(const __grid_constant__ Group<PStep> group) {
-  ptx::grid_wait();
-  ptx::grid_release();
   const PStep &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.n_blocks) return;
   const float a = *y.inv_tau;
@@ -172,8 +170,6 @@ struct QuantTrial {
 };
 __global__ void __launch_bounds__(EW_THREADS)
 quant_trial_kernel(const __grid_constant__ Group<QuantTrial> group, int levels, int wide_codes, int neg_levels) {
-  ptx::grid_wait();
-  ptx::grid_release();
   __shared__ double red[EW_THREADS / 32];
   __shared__ int is_last;
   const QuantTrial &y = group.l[blockIdx.y];
@@ -318,8 +314,6 @@ rows_planes_kernel(const float *__restrict__ x, size_t n8, const uint32_t *__res
 struct PlaneCheck { const float *x; uint32_t n8; const uint32_t *amax; const int *exp; __half *hi, *lo /* may be null */; };
 __global__ void __launch_bounds__(256)
 check_planes_kernel(const __grid_constant__ Group<PlaneCheck> group) {
-  ptx::grid_wait();
-  ptx::grid_release();
   const PlaneCheck &y = group.l[blockIdx.y];
   if (tc_planes_usable(*y.amax, *y.exp)) return;
   const float scale = tc_pow2(tc_scale_exp(*y.amax));
@@ -340,8 +334,6 @@ struct GradWSum {
 };
 __global__ void __launch_bounds__(EW_THREADS)
 reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
-  ptx::grid_wait();
-  ptx::grid_release();
   __shared__ double red[EW_THREADS / 32];
   __shared__ int is_last;
   const GradWSum &y = group.l[blockIdx.y];
@@ -390,8 +382,6 @@ struct ThetaStep {
 };
 __global__ void __launch_bounds__(EW_THREADS)
 theta_step_kernel(const __grid_constant__ Group<ThetaStep> group) {
-  ptx::grid_wait();
-  ptx::grid_release();
   extern __shared__ double colsum_sh[];                       // [n_sub][ld] when n_sub > 1
   const ThetaStep &y = group.l[blockIdx.y];
   const float a = y.sc->inv_theta;
@@ -487,8 +477,6 @@ sumsq_amax_kernel(const float *__restrict__ G, size_t n4, uint32_t *__restrict__
 struct BiasStep { const double *slots; int n_slots, ld, width; float *b, *shift; };
 __global__ void __launch_bounds__(32 * BIAS_GROUPS)
 finalize_bias_kernel(const __grid_constant__ Group<BiasStep> group, double inv_n) {
-  ptx::grid_wait();
-  ptx::grid_release();
   __shared__ double sh[BIAS_GROUPS][33];
   const BiasStep &y = group.l[blockIdx.y];
   const int c = blockIdx.x * 32 + threadIdx.x;
@@ -526,8 +514,6 @@ struct Zqu {
 struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T; };
 __global__ void __launch_bounds__(EW_THREADS)
 zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
-  ptx::grid_wait();
-  ptx::grid_release();
   const Zqu &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.n_blocks) return;
   float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
@@ -635,8 +621,6 @@ __device__ __forceinline__ void table_best(const float *__restrict__ f_sh, int T
 }
 __global__ void __launch_bounds__(EW_THREADS)
 zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
-  ptx::grid_wait();
-  ptx::grid_release();
   const Zqu &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.n_blocks) return;
   float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;

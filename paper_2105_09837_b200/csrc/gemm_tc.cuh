@@ -220,7 +220,6 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   __shared__ int lay_exp[TC_MAX_GROUP][2];
   __shared__ double team_scratch[1 + TC_ACC_WARPS];
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
-  ptx::grid_wait();                                   // everything above runs while the previous kernel finishes
   if (warp == 2 && lane < grp.n) {
     const TcLayer<Epi> &y = grp.l[lane];
     const int begin = lane > 0 ? grp.l[lane - 1].unit_end : 0;
@@ -251,7 +250,6 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   else __syncthreads();
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  ptx::grid_release();
 
   // Work unit -> its layer, row and column tile origin, first and number of K blocks, contraction slice; a unit is an output
   // tile or, in the tail, one contraction slice of an output tile.  Units are visited in ascending order.

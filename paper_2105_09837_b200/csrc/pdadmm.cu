@@ -263,19 +263,6 @@ static int dev_alloc(pdadmm_ctx *c, T **ptr, size_t count, bool zero = true) {
   return PDADMM_OK;
 }
 
-// Launches a kernel of an iteration so that it may start while the one before it in the stream finishes: the kernel calls
-// grid_wait() before it touches memory.  (An iteration of a small problem is a chain of a dozen kernels of 5 us.)
-template <class... P, class... A>
-static void launch_next(cudaStream_t st, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute a;
-  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  a.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &a; cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kern, P(args)...);            // errors surface at the call's end (cudaGetLastError)
-}
-
 static inline int ew_grid(size_t n_items) {
   return (int)std::max<size_t>(1, std::min<size_t>(ceil_div((int64_t)n_items, EW_THREADS), 148 * 8));
 }
@@ -398,13 +385,11 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &gr
   cfg.blockDim = dim3(TC_THREADS);
   cfg.dynamicSmemBytes = TC_SMEM_BYTES;
   cfg.stream = st;
-  cudaLaunchAttribute a[2];
-  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see launch_next
-  a[0].val.programmaticStreamSerializationAllowed = 1;
-  a[1].id = cudaLaunchAttributeClusterDimension;
-  a[1].val.clusterDim.x = 2; a[1].val.clusterDim.y = 1; a[1].val.clusterDim.z = 1;
-  cfg.attrs = a;
-  cfg.numAttrs = PAIR ? 2 : 1;
+  cudaLaunchAttribute a;
+  a.id = cudaLaunchAttributeClusterDimension;
+  a.val.clusterDim.x = 2; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
+  cfg.attrs = &a;
+  cfg.numAttrs = PAIR ? 1 : 0;
   PD_CUDA(cudaLaunchKernelEx(&cfg, kern, grp));
   return PDADMM_OK;
 }
@@ -456,9 +441,10 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
     units += n_tiles;
     // The persistent grid works through the tiles in rounds; a last round that fills only part of the
     // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit (at least 8 K
-    // blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks).
+    // blocks per slice: parking and merging the slices of a tile costs about as much as four K blocks).  A product that only
+    // wants its squared norm keeps whole tiles: it stores nothing that could be merged.
     const int slots = pair ? c->n_sms / 2 : c->n_sms, tail = n_tiles % slots;
-    if (c->tail_split && n == 1 && p.n_split == 1 && tail > 0 && p.s != nullptr && p.s->tail_ws != nullptr) {
+    if (epi_stores<Epi>::value && c->tail_split && n == 1 && p.n_split == 1 && tail > 0 && p.s != nullptr && p.s->tail_ws != nullptr) {
       const int split = std::min(std::min(slots / tail, (int)ceil_div(p.K, TC_BK) / 8), 8);
       if (split > 1) {
         y.tail_begin = n_tiles - tail; y.tail_split = split;
@@ -520,7 +506,7 @@ static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, const std:
   }
   if (n == 0) return;
   Launch l(c, KC_PLANES, st, 0, 0);
-  launch_next(st, check_planes_kernel, dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, g);
+  check_planes_kernel<<<dim3((unsigned)std::max(1, ew_grid(n8_max) / n), (unsigned)n), 256, 0, st>>>(g);
 }
 static int alloc_planes(pdadmm_ctx *c, size_t n, Planes *pl, bool zero = true) {
   PD_TRY(dev_alloc(c, &pl->hi, n, zero));
@@ -748,7 +734,7 @@ static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     bytes += (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out);
   }
   Launch k(c, KC_AXPY, st, bytes, 0);
-  launch_next(st, pstep_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g);
+  pstep_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
@@ -774,8 +760,7 @@ static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       bytes += (c->int_operands ? 8.0 + 2.0 * c->code_bytes : 12.0 + 2.0 * c->code_bytes) * N * ly.n_in;
     }
     Launch k(c, KC_QUANT, st, bytes, 0);
-    launch_next(st, quant_trial_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->levels, c->code_bytes == 2,
-                 c->neg_levels);
+    quant_trial_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->levels, c->code_bytes == 2, c->neg_levels);
   }
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
   // max|r| takes the trial's values too, which keeps it an upper bound whether or not the trial is taken
@@ -898,7 +883,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
     }
     Launch k(c, KC_GRADW_REDUCE, st, bytes, 0);
-    launch_next(st, reduce_gradW_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, g, c->nu);
+    reduce_gradW_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->nu);
   }
   if (c->reduce != nullptr) {
     // nabla_W phi is a sum over nodes: add the shards' parts, then take the norm and the largest magnitude of the total
@@ -966,7 +951,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     }
     {
       Launch k(c, KC_COLSUM, st, bytes, 0);
-      launch_next(st, theta_step_kernel, dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, g);
+      theta_step_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, st>>>(g);
     }
     if (c->reduce != nullptr) {
       // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
@@ -979,8 +964,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       }
     }
     Launch k(c, KC_SMALL, st, bias_bytes, 0);
-    launch_next(st, finalize_bias_kernel, dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, gb,
-                 1.0 / (double)c->N_total);
+    finalize_bias_kernel<<<dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, st>>>(gb, 1.0 / (double)c->N_total);
   }
   return PDADMM_OK;
 }
@@ -1004,8 +988,8 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
                       c->table_step, c->table_size};
   const dim3 grid((unsigned)blocks, (unsigned)n);
-  if (c->table_size > 0) launch_next(st, zqu_table_kernel, grid, EW_THREADS, c->table_size * sizeof(float), g, prm);
-  else launch_next(st, zqu_kernel, grid, EW_THREADS, 0, g, prm);
+  if (c->table_size > 0) zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), st>>>(g, prm);
+  else zqu_kernel<<<grid, EW_THREADS, 0, st>>>(g, prm);
 }
 static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
   Layer &ly = c->layers[c->L - 1];
@@ -2127,7 +2111,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       const size_t n4 = (size_t)M * ldc / 4;
       Group<GradWSum> g;
       g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
-      launch_next(st, reduce_gradW_kernel, dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, g, 1.0f);
+      reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
     }
     double h = 0;
     PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));

@@ -242,12 +242,5 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn, bool b
          ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// ---- order between kernels ------------------------------------------------------------------------
-// Launched with programmatic stream serialisation, a kernel starts while the one before it in the stream still runs: it may
-// touch memory that the other works on only after grid_wait(), and lets its own successor start with grid_release() (both do
-// nothing in an ordinary launch).
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 }  // namespace ptx
 }  // namespace pd
