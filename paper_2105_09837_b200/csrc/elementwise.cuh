@@ -14,7 +14,6 @@
 #include "common.cuh"
 #include "planes.cuh"
 #include "scalars.cuh"
-#include "tc_ptx.cuh"
 
 namespace pd {
 

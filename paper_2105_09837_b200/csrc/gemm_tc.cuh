@@ -166,10 +166,10 @@ __global__ void __maxnreg__(TC_REGS_LAUNCH)
 gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   constexpr bool A_MN = (LAYOUT & TC_A_MN) != 0, B_MN = (LAYOUT & TC_B_MN) != 0, COARSE = epi_coarse<Epi>::value || ZERO == 3;
   // which lo planes are loaded and used (a product that only wants its squared norm uses neither, and lets the main
-  // term accumulate in tensor memory over the whole contraction: the truncation of that accumulation, 1e-5 relative,
-  // does not matter to a norm that only starts a search)
+  // term accumulate in tensor memory over 8 K blocks: the truncation of that accumulation, 2e-6 relative, does not matter to a
+  // norm that only starts a search; over the whole contraction it was 1e-5 at 1000 values)
   constexpr bool A_LO = !(ZERO & 1) && !COARSE, B_LO = !(ZERO & 2) && !COARSE;
-  constexpr int FLUSH = COARSE ? (1 << 30) : TC_FLUSH;        // K blocks per read-out of the main accumulator
+  constexpr int FLUSH = COARSE ? 8 : TC_FLUSH;        // K blocks per read-out of the main accumulator
   constexpr int A_PLANES = A_LO ? 2 : 1, B_PLANES = B_LO ? 2 : 1;
   constexpr int CG = PAIR ? 2 : 1, WARPS = CG * TC_ACC_WARPS, TILE_M = PAIR ? 2 * TC_BM : TC_BM;
   constexpr int B_PLANE_BYTES = PAIR ? TC_BOX_BYTES : TC_PLANE_BYTES, BN = PAIR ? TC_BN / 2 : TC_BN;    // B held by this block
@@ -549,7 +549,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           ++visited;
         }
         const TcLayer<Epi> &y = grp.l[t.g];
-        const int n_grp = COARSE ? (t.n_kb > 0 ? 1 : 0) : t.n_kb;   // read-outs of the main accumulator for this tile
+        const int n_grp = (t.n_kb + FLUSH - 1) / FLUSH;   // read-outs of the main accumulator for this tile
         uint64_t acc[32];                             // columns 2 j, 2 j + 1 in acc[j]
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = 0ull;
