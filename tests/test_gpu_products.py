@@ -1,0 +1,74 @@
+"""The product kernel inside whole iterations where its variants meet their edges: single blocks and pairs of SMs, ragged
+tiles, operands whose planes were refused (made again inside the product, or by a kernel beforehand), more layers than one
+launch takes; and the last layer's update at the edges of its lanes-per-node rule, host copies at the edges of their pieces."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2105_09837_b200 import binding as B
+from paper_2105_09837_b200 import synth
+import parity_util as U
+from test_gpu_parity import _compare_iteration
+
+pytestmark = pytest.mark.gpu
+
+
+# nodes x width: single blocks below three quarters of the pairs (56 tiles of 256 x 128 over the layers of a launch), pairs from
+# there on; refused planes are made again beforehand from 2^20 elements on, by the product's own warps below.
+@pytest.mark.parametrize("n_nodes,hidden,n_layers", [(131, 68, 4),          # single blocks, split in the product
+                                                     (14336 + 3, 64, 6),    # pairs, split in the product
+                                                     (4200, 260, 3),        # single blocks, planes made again beforehand
+                                                     (8200, 132, 6)])       # pairs, planes made again beforehand
+def test_refused_planes_in_every_form_of_the_product(n_nodes, hidden, n_layers):
+    """u is scaled so that the gradients jump by 300 up and down between teacher-forced iterations: the exponents predicted
+    for their planes do not fit.  Every variable is held to the rounding bounds of its own computation."""
+    inp = synth.make_inputs(synth.small("c2", n_nodes, feat_dim=20, hidden=hidden, n_layers=n_layers, quant_levels=0))
+    prm, s, _ = U.oracle_problem(inp)
+    ctx = B.from_inputs(inp)
+    for k, factor in enumerate([1.0, 1.0, 300.0, 1 / 300.0]):
+        prev = U.round_state(dataclasses.replace(s, u=[x * factor for x in s.u]))
+        U.load_state(ctx, prev, False)
+        s = _compare_iteration(ctx, prev, prm, f"N={n_nodes}/h={hidden}/k={k}", single_bounds=True)
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("n_layers", [17, 18, 19])                          # 15, 16 and 17 hidden layers: one launch or two
+@pytest.mark.parametrize("levels", [0, 16])
+def test_grouped_launches_do_not_change_a_bit(n_layers, levels):
+    inp = synth.make_inputs(synth.small("c2", 700, feat_dim=30, hidden=72, n_layers=n_layers, quant_levels=levels))
+    ref = None
+    for flags in (B.FLAG_ONE_LANE | B.FLAG_NO_GRAPH, 0):
+        ctx = B.from_inputs(inp, flags=flags)
+        ctx.step(2)
+        st = U.read_state(ctx)
+        ctx.destroy()
+        if ref is None:
+            ref = st
+        else:
+            for k in st:
+                assert all(np.array_equal(a, b) for a, b in zip(st[k], ref[k])), k
+
+
+@pytest.mark.parametrize("n_classes", [2, 4, 5, 8, 9, 16, 17, 32, 33, 64])
+def test_last_layer_update_at_the_edges_of_its_lanes_per_node(n_classes):
+    inp = synth.make_inputs(synth.small("c2", 517, feat_dim=11, hidden=24, n_layers=3, n_classes=n_classes, quant_levels=0))
+    prm, s, _ = U.oracle_problem(inp)
+    ctx = B.from_inputs(inp)
+    for k in range(2):
+        prev = U.round_state(s)
+        U.load_state(ctx, prev, False)
+        s = _compare_iteration(ctx, prev, prm, f"C={n_classes}/k={k}")
+    ctx.destroy()
+
+
+# rows of 1 to 333 values, matrices of a piece (512 KB) and a little less and more
+@pytest.mark.parametrize("n_nodes,hidden", [(1, 1), (2047, 64), (2048, 64), (2049, 64), (4000, 333), (131073, 1)])
+def test_host_copies_at_the_edges_of_a_piece(n_nodes, hidden):
+    inp = synth.make_inputs(synth.small("c2", n_nodes, feat_dim=3, hidden=hidden, n_layers=3, n_hops=1, quant_levels=0))
+    ctx = B.from_inputs(inp)
+    x = np.random.default_rng(0).standard_normal((n_nodes, hidden)).astype(np.float32)
+    ctx.set_tensor(B.T_Z, 1, x)
+    assert np.array_equal(ctx.get_tensor(B.T_Z, 1), x)
+    ctx.destroy()
