@@ -45,12 +45,14 @@
 
 namespace pd {
 
+// Operands that are MN-major (output index contiguous) where the others are K-major.
+enum : int { TC_NT = 0, TC_A_MN = 1, TC_B_MN = 2 };
 constexpr int TC_BM = 128, TC_BN = 128, TC_BK = 64;
 constexpr int TC_KSTEPS = TC_BK / 16;                          // MMAs (K = 16) per pair of planes and K block
 constexpr int TC_FLUSH = 1;                                    // K blocks per read-out of the main accumulator
 constexpr int TC_PLANE_BYTES = 128 * TC_BK * 2;                // 16 KB: one 128 x 64 fp16 operand plane
 constexpr int TC_BOX_BYTES = 64 * TC_BK * 2;                   // 8 KB: what one TMA load brings, 64 x 64
-constexpr int TC_SPACE = 14 * TC_PLANE_BYTES;                  // 224 KB: stages and slots of finished tiles
+constexpr int TC_SPACE = 14 * TC_PLANE_BYTES;                  // 224 KB: stages and finished tile
 constexpr int TC_MAX_STAGES = 8;
 // Five warpgroups (register budgets are set per warpgroup): 0 = TMA warp, MMA warp and two warps that split operands when
 // a scaling was unusable; 1, 2 = the accumulate warps: a warp can only reach its own 32-lane quarter of tensor memory, so
@@ -69,15 +71,14 @@ static_assert(128 * (TC_REGS_CTRL + 2 * TC_REGS_ACC + 2 * TC_REGS_EPI) <= TC_THR
 constexpr int TC_ACC_BUFS = 3;                                 // main-term accumulator tiles in tensor memory
 constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 1 correction tile
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
-constexpr int TC_SLOT_BYTES = 8 * 16 * 64 * 4;                 // half a finished tile: 8 warps x 16 rows x 64 columns
-constexpr int TC_SMEM_BYTES = TC_SPACE + 1024 /* alignment slack */ + 768 /* barriers */;
-static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 4 * TC_ACC_WARPS) + 12 <= 768, "barriers");
-// Slots for halves of finished tiles: two, or one where the space of the other makes room for one more stage; none if nothing
-// is stored.
-__host__ __device__ constexpr int tc_slots(int stage_bytes, bool stores) {
-  const int two = (TC_SPACE - 2 * TC_SLOT_BYTES) / stage_bytes, one = (TC_SPACE - TC_SLOT_BYTES) / stage_bytes;
-  return !stores ? 0 : (one > two && two < TC_MAX_STAGES) ? 1 : 2;
-}
+constexpr int TC_TILE_BYTES = 8 * 32 * 64 * 4;                 // finished tile: 8 warps x 32 rows x 64 columns
+constexpr int TC_SMEM_BYTES = TC_SPACE + 1024 /* alignment slack */ + 512 /* barriers */;
+static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
+// How many parts a finished tile is handed over in (none if nothing is stored).  In one part it takes 64 KB; in two, one after
+// the other through 32 KB, it leaves room for one more stage if a stage holds four planes.  Two parts for the contraction
+// over the nodes, which is long and stores little: 100 000 x 500 x 500, 8 layers: 395 us against 444.  For the other products, whose
+// contraction is a layer's width, the second part holds up the accumulate warps: x W^T 468 us against 453.
+__host__ __device__ constexpr int tc_parts(int layout, bool stores) { return !stores ? 0 : layout == (TC_A_MN | TC_B_MN) ? 2 : 1; }
 
 // Epilogues store their result unless they say otherwise (kStore = false).
 template <class Epi, class = void> struct epi_stores { static constexpr bool value = true; };
@@ -166,7 +167,6 @@ struct TcGroup {
 // pdADMM-G-Q that lies on a level set {c s} (the quantised p, or the difference of two of them) is the spacing s times
 // a small integer, and integers up to 2048 are exact in one fp16 plane: its plane holds the integers, there is no lo
 // plane to load and no MMA for it (two MMAs per product instead of three), and mul = s restores the values.
-enum : int { TC_NT = 0, TC_A_MN = 1, TC_B_MN = 2 };
 template <int LAYOUT, class Epi, int ZERO, bool PAIR>
 __global__ void __maxnreg__(TC_REGS_LAUNCH)
 gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
@@ -181,7 +181,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   constexpr int B_PLANE_BYTES = PAIR ? TC_BOX_BYTES : TC_PLANE_BYTES, BN = PAIR ? TC_BN / 2 : TC_BN;    // B held by this block
   constexpr int STAGE_BYTES = A_PLANES * TC_PLANE_BYTES + B_PLANES * B_PLANE_BYTES;
   constexpr bool STORES = epi_stores<Epi>::value;
-  constexpr int SLOTS = tc_slots(STAGE_BYTES, STORES), STAGE_SPACE = TC_SPACE - SLOTS * TC_SLOT_BYTES;
+  constexpr int PARTS = tc_parts(LAYOUT, STORES), STAGE_SPACE = TC_SPACE - (PARTS > 0 ? TC_TILE_BYTES / PARTS : 0);
   constexpr int STAGES = STAGE_SPACE / STAGE_BYTES < TC_MAX_STAGES ? STAGE_SPACE / STAGE_BYTES : TC_MAX_STAGES;
   constexpr int B_OFF = A_PLANES * TC_PLANE_BYTES;            // stage: A_hi, A_lo, B_hi, B_lo (those that exist)
   extern __shared__ uint8_t smem_raw[];
@@ -191,8 +191,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
   uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
   uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1, *split_bar = team_bar + 1;
-  uint64_t *done_full = split_bar + STAGES, *done_empty = done_full + 2 * TC_ACC_WARPS;     // per accumulate warp and slot
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + 2 * TC_ACC_WARPS);
+  uint64_t *done_full = split_bar + STAGES, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
 
@@ -214,7 +214,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
     ptx::mbar_init(team_bar, TC_ACC_WARPS);
-    for (int w = 0; w < 2 * TC_ACC_WARPS; ++w) {
+    for (int w = 0; w < TC_ACC_WARPS; ++w) {
       ptx::mbar_init(&done_full[w], 1);
       ptx::mbar_init(&done_empty[w], 1);
     }
@@ -487,13 +487,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     const bool accumulates = warp < TC_EPI0;
     const int aw = warp - (accumulates ? TC_ACC0 : TC_EPI0), quarter = warp & 3, col_base = 64 * (aw >> 2);
     const int lane_base = quarter * 32, piece = (int)rank * TC_ACC_WARPS + aw;
-    // The warp pair's piece of a finished tile goes over in two halves of 16 rows, each through a slot: row i at 16 i, its 16
-    // float4 groups with the group index XOR-ed by (i mod 8), so that both sides (a lane per row; 16 lanes per row) are free of
-    // bank conflicts.
-    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * 256;
-    constexpr int SLOT_F4 = TC_SLOT_BYTES / 16;
-    auto slot_of = [](int half) { return SLOTS == 2 ? half : 0; };
-    auto use_of = [](uint32_t tile, int half) { return SLOTS == 2 ? tile : 2 * tile + (uint32_t)half; };   // earlier uses of its slot
+    // The warp pair's piece of the finished tile (or one half of its rows after the other): row i at 16 i, its 16 float4 groups
+    // with the group index XOR-ed by (i mod 8), so that both sides (a lane per row; 16 lanes per row) are free of bank conflicts.
+    constexpr int PART_ROWS = PARTS == 2 ? 16 : 32, PART_F4 = PART_ROWS * 16;
+    float4 *tr = reinterpret_cast<float4 *>(tr_base) + (size_t)aw * PART_F4;
     bool ok = true;
     Tile t;
     int visited = 0;                                   // units of layer t.g that this block has finished
@@ -551,7 +548,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       ptx::setmaxnreg_inc<TC_REGS_ACC>();
       // ------------------------------------------------------------ accumulate
       int b = 0;
-      uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; tiles handed over so far
+      uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; parts handed over so far
       for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
         const int g_before = t.g;
         locate(unit, t);
@@ -620,26 +617,25 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           ptx::unpack_f2(s2[1], s4[2], s4[3]);
           if (y.slots != nullptr && t.m0 < y.M) put_sum(y, ((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3]));
         } else {
-          // hand the piece over, each half as soon as the epilogue warp has taken what its slot held before
+          // hand the piece over; the epilogue warp has finished with the previous one
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int sl = slot_of(h);
-            ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(&done_empty[2 * aw + sl], (use_of(handed, h) & 1u) ^ 1u, abort_flag));
+          for (int h = 0; h < PARTS; ++h) {
+            ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(&done_empty[aw], (handed & 1u) ^ 1u, abort_flag));
             if (!ok) break;
-            if ((lane >> 4) == h) {
+            ++handed;
+            if (PARTS == 1 || (lane >> 4) == h) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
                 float4 v;
                 ptx::unpack_f2(acc[2 * j], v.x, v.y);
                 ptx::unpack_f2(acc[2 * j + 1], v.z, v.w);
-                tr[sl * SLOT_F4 + (lane & 15) * 16 + (j ^ (lane & 7))] = v;
+                tr[(lane & (PART_ROWS - 1)) * 16 + (j ^ (lane & 7))] = v;
               }
             }
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&done_full[2 * aw + sl]);
+            if (lane == 0) ptx::mbar_arrive(&done_full[aw]);
           }
           if (!ok) break;
-          ++handed;
         }
       }
       if (!STORES && ok) leave(t.g);
@@ -684,20 +680,19 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           float *C = epi.C + (size_t)t.z * y.c_split_stride;
           float ssf = 0.f;
           uint32_t mx = 0u;                  // largest magnitude stored by this thread
-          auto wait_half = [&](int h) {
-            return __all_sync(0xffffffffu, ptx::mbar_wait(&done_full[2 * aw + slot_of(h)], use_of(taken, h) & 1u, abort_flag)) != 0;
-          };
-          auto release_half = [&](int h) {
+          auto wait_part = [&]() { return __all_sync(0xffffffffu, ptx::mbar_wait(&done_full[aw], taken++ & 1u, abort_flag)) != 0; };
+          auto release_part = [&]() {
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&done_empty[2 * aw + slot_of(h)]);
+            if (lane == 0) ptx::mbar_arrive(&done_empty[aw]);
           };
-          // eight steps on the values v, whose inputs have been loaded
-          auto finish_half = [&](int h, const float4 (&v)[8]) {
+          auto at = [&](int i) { const int r = 2 * i + (lane >> 4); return r * 16 + ((lane & 15) ^ (r & 7)); };     // step i of a part
+          // eight steps, value i from get(i), whose inputs have been loaded
+          auto finish_half = [&](int h, auto get) {
             if (!col_in) return;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const int row = row0 + 16 * h + 2 * i;
-              float4 o = v[i];
+              float4 o = get(i);
               if (row >= y.M) continue;
               if constexpr (epi_sumsq_acc<Epi>::value) ssf = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, ssf))));
               if constexpr (!Epi::kDirect) o = epi.apply(col, o, in[i]);
@@ -714,34 +709,18 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
               if constexpr (epi_amax<Epi>::value) mx = max(mx, abs_bits(o));
             }
           };
-          auto at = [&](int i) { const int r = 2 * i + (lane >> 4); return r * 16 + ((lane & 15) ^ (r & 7)); };     // step i of a half
-          bool whole = true;
-          if (t.slice < 0) {
-#pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-              if (h > 0 && col_in) load_inputs(8);
-              ok = wait_half(h);
-              if (!ok) break;
-              const float4 *src = tr + slot_of(h) * SLOT_F4;
-              float4 v[8];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) v[i] = src[at(i)];
-              release_half(h);
-              finish_half(h, v);
-            }
-            if (!ok) break;
-          } else {
+          const int t_idx = t.out - y.tail_begin;
+          bool whole = t.slice < 0;
+          if (!whole) {
             // contraction slice of a tail tile: park the piece; the last warp to arrive sums the slices
-            const int t_idx = t.out - y.tail_begin, u = t_idx * y.tail_split + t.slice;
-            float4 *mine = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)u * WARPS + piece) * 512;
+            float4 *mine = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)(t_idx * y.tail_split + t.slice) * WARPS + piece) * 512;
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-              ok = wait_half(h);
+            for (int h = 0; h < PARTS && ok; ++h) {
+              ok = wait_part();
               if (!ok) break;
-              const float4 *src = tr + slot_of(h) * SLOT_F4;
 #pragma unroll 4
-              for (int j = 0; j < 8; ++j) mine[h * 256 + j * 32 + lane] = src[j * 32 + lane];
-              release_half(h);
+              for (int j = 0; j < PART_F4 / 32; ++j) mine[h * PART_F4 + j * 32 + lane] = tr[j * 32 + lane];
+              release_part();
             }
             if (!ok) break;
             __threadfence();
@@ -753,25 +732,31 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             if (whole) {
               __threadfence();
               if (lane == 0) y.tail_count[t_idx * WARPS + piece] = 0;
-              const float4 *part = reinterpret_cast<const float4 *>(y.tail_ws) + ((size_t)t_idx * y.tail_split * WARPS + piece) * 512;
-#pragma unroll 1
-              for (int h = 0; h < 2; ++h) {
-                if (h > 0 && col_in) load_inputs(8);
-                float4 v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int sl = 0; sl < y.tail_split; ++sl)
-#pragma unroll
-                  for (int i = 0; i < 8; ++i) {
-                    const float4 x = __ldcg(part + (size_t)sl * WARPS * 512 + h * 256 + at(i));
-                    v[i].x += x.x; v[i].y += x.y; v[i].z += x.z; v[i].w += x.w;
-                  }
-                finish_half(h, v);
-              }
             }
           }
-          ++taken;
           if (whole) {
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+              if (h > 0 && col_in) load_inputs(8);
+              if (t.slice >= 0) {
+                const float4 *part = reinterpret_cast<const float4 *>(y.tail_ws) + ((size_t)t_idx * y.tail_split * WARPS + piece) * 512 + h * 256;
+                finish_half(h, [&](int i) {
+                  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                  for (int sl = 0; sl < y.tail_split; ++sl) {
+                    const float4 v = __ldcg(part + (size_t)sl * WARPS * 512 + at(i));
+                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                  }
+                  return a;
+                });
+                continue;
+              }
+              if (h == 0 || PARTS == 2) ok = wait_part();
+              if (!ok) break;
+              const float4 *src = tr + (PARTS == 2 ? 0 : h * 256);
+              finish_half(h, [&](int i) { return src[at(i)]; });
+              if (h == 1 || PARTS == 2) release_part();
+            }
+            if (!ok) break;
             if constexpr (epi_amax<Epi>::value) {
               if (epi.amax != nullptr) commit_amax(mx, epi.amax);      // the output is an operand of a later product
             }
