@@ -118,7 +118,6 @@ struct TcLayer {
   int M, N, K;            // output rows, output columns, contraction length
   int k_chunk;            // contraction slice (multiple of TC_BK); K rounded up if not split
   int n_split;            // number of contraction slices; slice z writes its own partial output
-  int unit_end;           // work units of this layer and of those before it
   size_t c_split_stride;  // elements between the partial outputs of consecutive slices
   TcOperand oa, ob;
   float mul;              // factor applied to the result after the power-of-two scalings (integer operands, see ZERO)
@@ -141,6 +140,8 @@ struct TcLayer {
 template <class Epi>
 struct TcGroup {
   int n;
+  int unit_end[TC_MAX_GROUP];      // work units of a layer and of those before it (side by side: walking through the layers'
+                                   // descriptions cost a miss in the constant cache each, half of a small launch's start)
   int *error;             // set to 1 if a bounded wait expired
   TcLayer<Epi> l[TC_MAX_GROUP];
 };
@@ -152,9 +153,11 @@ struct TcGroup {
 // of A, of the accumulators and of the output, and columns 64 rank .. +63 of B.  Block 0 issues the MMAs of both; its
 // barriers collect what both blocks loaded and read out.
 //
-// Persistent: the grid has at most one block per SM and block (pair) i works on output tiles i, i + their number, ...
-// (column tile fastest, so that neighbouring blocks share the streamed operand in L2).  All roles keep running
-// counters over K blocks, so the producer prefetches the next tile while the current one is in its epilogue.
+// Persistent: the grid has at most one block per SM and the blocks (pairs) take the output tiles in rounds, upwards in even
+// rounds and downwards in odd ones (column tile fastest, so that neighbouring blocks share the streamed operand in L2): the
+// first layer's contraction is often several times as long, and the blocks that began with it get nothing of a partly filled
+// second round.  All roles keep running counters over K blocks, so the producer prefetches the next tile while the current one
+// is in its epilogue.
 //
 // The tensor cores add into their fp32 accumulator with truncation, which costs about 2^-24 of the
 // accumulator per MMA and always in the same direction.  To keep fp32-class accuracy the main term
@@ -199,7 +202,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_rank() : 0u;
   const int unit0 = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x), unit_step = (int)(PAIR ? gridDim.x >> 1 : gridDim.x);
-  const int n_units = grp.l[grp.n - 1].unit_end;
+  const int n_units = grp.unit_end[grp.n - 1];
+  auto unit_of = [&](int round) { return round & 1 ? (round + 1) * unit_step - 1 - unit0 : round * unit_step + unit0; };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -230,10 +234,11 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
   if (warp == 2 && lane < grp.n) {
     const TcLayer<Epi> &y = grp.l[lane];
-    const int begin = lane > 0 ? grp.l[lane - 1].unit_end : 0;
-    const int ahead = (unit0 - begin) % unit_step, first = begin + (ahead < 0 ? ahead + unit_step : ahead);
+    const int begin = lane > 0 ? grp.unit_end[lane - 1] : 0, end = grp.unit_end[lane];
+    bool has_unit = false;
+    for (int k = begin / unit_step; k * unit_step < end && !has_unit; ++k) has_unit = unit_of(k) >= begin && unit_of(k) < end;
     lay_split[lane] = 0;
-    if (first < y.unit_end) {
+    if (has_unit) {
       const int ea = y.oa.exp ? *y.oa.exp : 0, eb = y.ob.exp ? *y.ob.exp : 0;
       const uint32_t ma = y.oa.amax ? *y.oa.amax : 0u, mb = y.ob.amax ? *y.ob.amax : 0u;
       const bool good_a = y.oa.amax == nullptr || tc_planes_usable(ma, ea), good_b = y.ob.amax == nullptr || tc_planes_usable(mb, eb);
@@ -247,7 +252,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     // allocates and releases its tensor memory and passes both block-wide barriers.
     *skip_flag = *reinterpret_cast<volatile int *>(grp.error) != 0;
     int g = 0;
-    while (g + 1 < grp.n && unit0 >= grp.l[g].unit_end) ++g;
+    while (g + 1 < grp.n && unit0 >= grp.unit_end[g]) ++g;
     ptx::prefetch_tmap(&grp.l[g].a);
     ptx::prefetch_tmap(&grp.l[g].b);
     if (A_LO) ptx::prefetch_tmap(&grp.l[g].alo);
@@ -263,9 +268,9 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   // tile or, in the tail, one contraction slice of an output tile.  Units are visited in ascending order.
   struct Tile { int g = 0, m0, n0, k_begin, n_kb, z, out, slice; };
   auto locate = [&](int unit, Tile &t) {
-    while (unit >= grp.l[t.g].unit_end) ++t.g;
+    while (unit >= grp.unit_end[t.g]) ++t.g;
     const TcLayer<Epi> &y = grp.l[t.g];
-    if (t.g > 0) unit -= grp.l[t.g - 1].unit_end;
+    if (t.g > 0) unit -= grp.unit_end[t.g - 1];
     const int tiles_n = (y.N + TC_BN - 1) / TC_BN, tiles_m = (y.M + TILE_M - 1) / TILE_M;
     t.out = unit; t.slice = -1;
     if (y.tail_split > 1 && unit >= y.tail_begin) {
@@ -307,7 +312,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             ptx::tma_load_2d<CG>(dst + i * TC_BOX_BYTES, map, mn ? o0 + 64 * i : k0, mn ? k0 : o0 + 64 * i, bar);
         };
         Tile t;
-        for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+        for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
           locate(unit, t);
           const TcLayer<Epi> &y = grp.l[t.g];
           const bool split_a = lay_split[t.g] & 1, split_b = lay_split[t.g] & 2;
@@ -366,7 +371,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
         int s = 0, b = 0, ti = 0, used = 0;
         uint32_t sp = 0, bp = 1;
         Tile t;
-        for (int unit = unit0; unit < n_units && ok; unit += unit_step, ++ti) {
+        for (int unit = unit0; unit < n_units && ok; unit = unit_of(++ti)) {
           locate(unit, t);
           const int n_kb = t.n_kb;
           for (int kb = 0; kb < n_kb; ++kb) {
@@ -460,7 +465,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       bool ok = false;
       for (int g = 0; g < grp.n; ++g) ok |= lay_split[g] != 0;
       Tile u;
-      for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+      for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
         locate(unit, u);
         const TcLayer<Epi> &y = grp.l[u.g];
         const int split = lay_split[u.g];
@@ -515,7 +520,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       __threadfence();
       if (!team_sync()) return false;
       if (tid == 0) {
-        const int units = (y.unit_end - (g > 0 ? grp.l[g - 1].unit_end : 0)) * CG;
+        const int units = (grp.unit_end[g] - (g > 0 ? grp.unit_end[g - 1] : 0)) * CG;
         const int before = atomicAdd(y.done, visited);
         *last = before + visited == units;
       }
@@ -549,7 +554,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       // ------------------------------------------------------------ accumulate
       int b = 0;
       uint32_t ph = 0, handed = 0;                     // phase of acc_full[b]; parts handed over so far
-      for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+      for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
         const int g_before = t.g;
         locate(unit, t);
         if (!STORES) {
@@ -647,7 +652,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       // clamped, their results dropped).
       if constexpr (STORES) {
         uint32_t taken = 0;
-        for (int unit = unit0; unit < n_units && ok; unit += unit_step) {
+        for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
           const int g_before = t.g;
           locate(unit, t);
           if (t.g != g_before && !leave(g_before)) { ok = false; break; }

@@ -379,7 +379,7 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &gr
     PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
     if (dev >= 0 && dev < MAX_DEVICES) configured[dev] = true;
   }
-  const int n_units = grp.l[grp.n - 1].unit_end;
+  const int n_units = grp.unit_end[grp.n - 1];
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(PAIR ? 2 * std::min(n_units, c->n_sms / 2) : std::min(n_units, c->n_sms)));
   cfg.blockDim = dim3(TC_THREADS);
@@ -452,7 +452,7 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
         units = y.tail_begin + tail * split;
       }
     }
-    y.unit_end = units;
+    grp.unit_end[i] = units;
   }
   if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, grp);
   return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, grp);
