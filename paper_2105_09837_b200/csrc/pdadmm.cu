@@ -727,7 +727,9 @@ static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     Layer &ly = c->layers[l];
     Scratch &s = scratch_of(c, l);
     const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
-    const int nb = ew_grid(std::max(n4p, n4r));
+    // a thread has eight loads in flight if it gets four groups (2000 x 100: 9 layers 18.8 us with a group per thread, 14.7 so;
+    // 10 007 x 333: 80.9 and 71.5)
+    const int nb = ew_grid((size_t)ceil_div((int64_t)std::max(n4p, n4r), 4));
     g.l[n++] = PStep{ly.p, s.s1, (uint32_t)n4p, ly.r, s.s2, (uint32_t)n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0),
                      c->use_tc ? ly.amax_p : nullptr, c->use_tc ? ly.amax_r : nullptr, nb};
     blocks = std::max(blocks, nb);
@@ -935,8 +937,9 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       Scratch &s = scratch_of(c, l);
       const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
       const int nbw = (int)std::min<int64_t>(ceil_div((int64_t)n4w, EW_THREADS), 2 * c->n_sms);
-      // rows in as many blocks as keep the SMs busy, at least 16 of them each
-      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 16));
+      // rows in as many blocks as keep the SMs busy, at least 32 of them each (16: an iteration of 2000 x 100 1 % longer, the
+      // bias kernel reads twice as many sums)
+      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 32));
       const int rows_per_block = (int)ceil_div(N, n_blocks), nbr = (int)ceil_div(N, rows_per_block);
       const int ld4 = ly.ld_out / 4, n_sub = std::min(EW_THREADS / std::min(ld4, EW_THREADS), COLSUM_MAX_SUB);
       if (n_sub > 1) sh = std::max(sh, (size_t)n_sub * ly.ld_out * sizeof(double));
