@@ -39,20 +39,19 @@ enum KClass {
   KC_GEMM_GRADW,      // partial tiles of r^T p+ over node slices
   KC_GRADW_REDUCE,    // sum of the partial tiles, nu, ||G||^2
   KC_GEMM_GP,         // G p+, squared norm
-  KC_AXPY,            // p -= g/tau ; r -= (Wg)/tau ; r += W d
+  KC_AXPY,            // p -= g/tau, r -= (Wg)/tau
   KC_QUANT,           // quantised trial step
-  KC_COLSUM,          // r -= (G p+)/theta with column sums
+  KC_COLSUM,          // W -= G/theta; r -= (G p+)/theta with column sums
   KC_ZQU,             // fused z, q, u update of a hidden layer
   KC_ZLAST,           // z update of the last layer
-  KC_WSTEP,           // W -= G/theta
-  KC_SMALL,           // single-block finalisers
+  KC_SMALL,           // bias from the column sums; sums of the CUDA-core products
   KC_AMAX,            // largest magnitude of a product's node-sized operand (for its power-of-two scaling)
-  KC_PLANES,          // fp16 planes of a weight-sized operand
+  KC_PLANES,          // fp16 planes made or made again by a kernel of their own
   KC_COUNT
 };
 static const char *kclass_names[KC_COUNT] = {
     "gemm_resid", "gemm_gradp", "gemm_wg", "gemm_gradw", "gradw_reduce", "gemm_gp", "axpy",
-    "quant_trial", "resid_colsum", "zqu", "zlast", "wstep", "finalize", "absmax", "make_planes"};
+    "quant_trial", "resid_colsum", "zqu", "zlast", "finalize", "absmax", "make_planes"};
 
 // fp16 hi/lo planes of a matrix, in its own orientation and with its leading dimension, and the device word with the
 // exponent of the power-of-two scaling they were made with.
@@ -728,7 +727,7 @@ static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     Scratch &s = scratch_of(c, l);
     const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
     // a thread has eight loads in flight if it gets four groups (2000 x 100: 9 layers 18.8 us with a group per thread, 14.7 so;
-    // 10 007 x 333: 80.9 and 71.5)
+    // 7013 x 333, 6 layers: 80.9 and 71.5)
     const int nb = ew_grid((size_t)ceil_div((int64_t)std::max(n4p, n4r), 4));
     g.l[n++] = PStep{ly.p, s.s1, (uint32_t)n4p, ly.r, s.s2, (uint32_t)n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0),
                      c->use_tc ? ly.amax_p : nullptr, c->use_tc ? ly.amax_r : nullptr, nb};
