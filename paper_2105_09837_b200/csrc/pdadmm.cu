@@ -1493,8 +1493,9 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   if (c->use_tc) {
     size_t need = 0, free_bytes = 0, total = 0;
     for (int l = 0; l < c->L; ++l) need += (size_t)N * c->layers[l].ld_out * 4;
-    PD_CUDA(cudaMemGetInfo(&free_bytes, &total));
-    if (need <= free_bytes / 8 * 7 || need <= c->arena_cap - c->arena_used)
+    const bool fits = need <= c->arena_cap - c->arena_used;            // (no question to the driver then, see DevicePool)
+    if (!fits) PD_CUDA(cudaMemGetInfo(&free_bytes, &total));
+    if (fits || need <= free_bytes / 8 * 7)
       for (int l = 0; l < c->L; ++l) PD_TRY(alloc_planes(c, (size_t)N * c->layers[l].ld_out, &c->layers[l].rp));
   }
   c->ev_p.resize(c->L);

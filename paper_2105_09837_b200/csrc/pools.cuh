@@ -6,7 +6,9 @@
 // after another: the greedy schedule grows one into the next, a sweep over settings rebuilds the same problem.  So what
 // destroy returns is kept for the next context of the process, within bounds:
 //   - device memory: at most 1/16 of the device, the oldest block goes first, and nothing while less than half of the
-//     device is free (somebody else may need it); all of it goes back to the driver when an allocation of this library
+//     device is free (somebody else may need it; asked at most twice a second: the question goes to the driver's resource
+//     manager, 0.1 ms, and 5 ms and more while other processes of the machine keep it busy); all of it goes back to the
+//     driver when an allocation of this library
 //     fails, and in pdadmm_release_cached_memory();
 //   - at most 64 streams and 256 events of each kind per device.
 // Everything is returned only after the context's device work has finished.  One lock per device; any thread.
@@ -14,6 +16,7 @@
 
 #include <cuda_runtime.h>
 
+#include <chrono>
 #include <mutex>
 #include <vector>
 
@@ -53,11 +56,18 @@ class DevicePool {
   // No device work may use the blocks any more.
   void give(const std::vector<DeviceBlock> &blocks) {
     if (blocks.empty()) return;
-    size_t free_bytes = 0, total = 0;
-    const bool keep = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= total / 2;
     std::vector<DeviceBlock> out;
     {
       std::lock_guard<std::mutex> g(m_);
+      const auto now = std::chrono::steady_clock::now();
+      if (asked_ == std::chrono::steady_clock::time_point{} || now - asked_ > std::chrono::milliseconds(500)) {
+        size_t free_bytes = 0, total = 0;
+        roomy_ = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= total / 2;
+        total_ = total;
+        asked_ = now;
+      }
+      const bool keep = roomy_;
+      const size_t total = total_;
       for (const DeviceBlock &b : blocks) {
         if (!keep || b.bytes > total / 16) { out.push_back(b); continue; }
         free_.push_back(b);
@@ -115,7 +125,9 @@ class DevicePool {
  private:
   std::mutex m_;
   std::vector<DeviceBlock> free_;          // oldest first
-  size_t held_ = 0;
+  size_t held_ = 0, total_ = 0;
+  bool roomy_ = false;
+  std::chrono::steady_clock::time_point asked_{};
   std::vector<cudaStream_t> streams_;
   std::vector<cudaEvent_t> events_[2];
 };
