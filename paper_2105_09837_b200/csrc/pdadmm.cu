@@ -1640,6 +1640,7 @@ static int refresh_p(pdadmm_ctx *c) {
   }
   PD_CUDA(cudaGetLastError());
   c->p_stale = false;
+  c->amax_p_valid = false;          // no kernel of an iteration keeps max|p| of values that it does not write
   return PDADMM_OK;
 }
 
@@ -1650,7 +1651,8 @@ static int ensure_operands(pdadmm_ctx *c) {
     for (auto &ly : c->layers) PD_TRY(refresh_W_planes(c, ly, c->scr.st));
     c->w_planes_valid = true;
   }
-  if (!c->amax_p_valid) {
+  // with integer operands max|p_l|, l >= 2, is read for a residual from scratch alone: not paid for after every look at p
+  if (!c->amax_p_valid && (!c->int_operands || !c->r_valid || !c->x_planes_valid)) {
     for (auto &ly : c->layers) {
       const size_t n4 = (size_t)c->N * ly.ld_in / 4;
       PD_CUDA(cudaMemsetAsync(ly.amax_p, 0, sizeof(uint32_t), c->scr.st));
