@@ -37,7 +37,7 @@ typedef enum {
   PDADMM_EINVAL = -1,    /* bad argument (null pointer, size, range, unsorted or out-of-range index) */
   PDADMM_ENOMEM = -2,    /* host or device allocation failed                                         */
   PDADMM_ECUDA = -3,     /* a CUDA call failed, or no usable device                                  */
-  PDADMM_ETIMEOUT = -4,  /* a bounded device-side wait expired                                       */
+  PDADMM_ETIMEOUT = -4,  /* a bounded device-side wait expired; the tensors hold an unfinished iteration */
   PDADMM_ENUMERIC = -5,  /* a non-finite value was detected in the state                             */
   PDADMM_ENOTCONV = -6   /* the tau search of the quantised p-update hit its trial cap               */
 } pdadmm_status;
@@ -293,6 +293,13 @@ int pdadmm_matmul_tn_static(int device, int M, int N, int K, const float *dA, in
  * a product launched afterwards runs normally.
  */
 int pdadmm_selftest_bounded_wait(int device, long long limit_cycles, long long *waited_cycles);
+/*
+ * pdadmm_selftest_expired_wait -- the host's side of the same path: leaves the context's words as blocks that gave up in the
+ * middle of their products leave them and returns what pdadmm_step then returns, PDADMM_ETIMEOUT.  No kernel is launched.
+ * The context stays usable: the tensors hold what an unfinished iteration left (here: what they held), everything derived
+ * from them is formed again by the next call.
+ */
+int pdadmm_selftest_expired_wait(pdadmm_ctx *ctx);
 
 /*
  * Per-kernel timing.  pdadmm_profile(ctx, 1) makes every later kernel launch of pdadmm_step be

@@ -29,7 +29,7 @@ OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT, ENUMERIC, ENOTCONV = 0, -1, -2, -3, -4, -5,
 
 EXPORTS = [
     "pdadmm_init", "pdadmm_init_sharded", "pdadmm_comm_bytes", "pdadmm_start_layers_from", "pdadmm_step", "pdadmm_last_step_ms", "pdadmm_objective", "pdadmm_residuals", "pdadmm_get_tensor",
-    "pdadmm_set_tensor", "pdadmm_predict", "pdadmm_quantize", "pdadmm_spmm", "pdadmm_matmul", "pdadmm_matmul_tn_static", "pdadmm_selftest_bounded_wait",
+    "pdadmm_set_tensor", "pdadmm_predict", "pdadmm_quantize", "pdadmm_spmm", "pdadmm_matmul", "pdadmm_matmul_tn_static", "pdadmm_selftest_bounded_wait", "pdadmm_selftest_expired_wait",
     "pdadmm_profile", "pdadmm_profile_classes",
     "pdadmm_profile_name", "pdadmm_profile_read", "pdadmm_launches", "pdadmm_time_augmentation", "pdadmm_destroy", "pdadmm_release_cached_memory", "pdadmm_last_error",
 ]
@@ -91,6 +91,7 @@ def lib() -> C.CDLL:
                                     C.POINTER(C.c_double), C.c_uint32]
         L.pdadmm_matmul_tn_static.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_int,
                                               C.c_void_p, C.c_void_p]
+        L.pdadmm_selftest_expired_wait.argtypes = [C.c_void_p]
         L.pdadmm_selftest_bounded_wait.argtypes = [C.c_int, C.c_longlong, C.POINTER(C.c_longlong)]
         L.pdadmm_profile.argtypes = [C.c_void_p, C.c_int]
         L.pdadmm_profile_name.argtypes = [C.c_int]

@@ -115,7 +115,7 @@ struct Layer {
   uint32_t *amax_p = nullptr, *amax_r = nullptr;
   // largest magnitudes of an iteration's g, W g, G and d: zero before the kernel that writes the matrix
   uint32_t *w_g = nullptr, *w_wg = nullptr, *w_G = nullptr, *w_d = nullptr;
-  int *done = nullptr;             // counters of finished blocks (trial, gradient sum, then products), zero between kernels
+  int *done = nullptr;             // [4] counters of finished blocks (trial, gradient sum, then products), zero between kernels
   int n_split = 1, k_chunk = 0;
 };
 
@@ -192,7 +192,11 @@ struct pdadmm_ctx {
   std::vector<cudaEvent_t> ev_lane; // [n_lanes]: fork / join
   bool r_valid = false;
   bool t_valid = false;             // every layer's t matches the stored u, p, q
-  int *d_flag = nullptr;            // device counter (z_L solver non-convergence)
+  // Words that are zero between calls, one block so that one clear covers them: d_flag[0..3] (z_L solver non-convergence, expired
+  // wait, non-finite sum, unused), the layers' `done` and w_* words, the tail counts of the lanes that cut tails.
+  int *control = nullptr;
+  size_t control_words = 0;
+  int *d_flag = nullptr;
   // page-locked block (CTX_PINNED_BYTES): words 0..63 small read-backs, 64..127 the lanes' accept flags, from byte 1024 on
   // the results that kernels write themselves (objective, residuals, counts of pdadmm_predict)
   int *h_pinned = nullptr;
@@ -1335,7 +1339,9 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   PD_TRY(take_ctx_pinned(c));
   PD_CUDA(pool.take_event(true, &c->ev_begin));
   PD_CUDA(pool.take_event(true, &c->ev_end));
-  PD_TRY(dev_alloc(c, &c->d_flag, 4));
+  c->control_words = 4 + 8 * (size_t)c->L + (size_t)PDADMM_N_LANES * c->n_sms * 8;
+  PD_TRY(dev_alloc(c, &c->control, c->control_words));
+  c->d_flag = c->control;
   PD_TRY(dev_alloc(c, &c->done, OBJ_MAX_LAYERS + 1));
   PD_TRY(dev_alloc(c, &c->counts, 4));
 
@@ -1400,9 +1406,9 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     if (c->int_operands && l > 0) PD_TRY(dev_alloc(c, &ly.p_plane, e_in));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.t, (size_t)N * ly.ld_in));
     PD_TRY(dev_alloc(c, &ly.sc, 1));
-    PD_TRY(dev_alloc(c, &ly.w_g, 4));
+    ly.done = c->control + 4 + 8 * l;
+    ly.w_g = reinterpret_cast<uint32_t *>(ly.done + 4);
     ly.w_wg = ly.w_g + 1; ly.w_G = ly.w_g + 2; ly.w_d = ly.w_g + 3;
-    PD_TRY(dev_alloc(c, &ly.done, 4));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.g_exp, 1));
     PD_TRY(dev_alloc(c, &ly.amax_p, 1));
     PD_TRY(dev_alloc(c, &ly.amax_r, 1));
@@ -1449,8 +1455,10 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   PD_TRY(dev_alloc(c, &s.slots, s.n_slots));
   PD_TRY(dev_alloc(c, &s.red, (size_t)max_out + 8));
   if (c->use_tc) {
-    PD_TRY(dev_alloc(c, &s.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
-    PD_TRY(dev_alloc(c, &s.tail_count, (size_t)c->n_sms * 8));
+    if (!small) {                       // (small problems cut no tails)
+      PD_TRY(dev_alloc(c, &s.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+      s.tail_count = c->control + 4 + 8 * (size_t)c->L;
+    }
     PD_TRY(dev_alloc(c, &s.amax_pool, (size_t)AMAX_POOL));
     s.pl_cap = e_max;
     PD_TRY(alloc_planes(c, s.pl_cap, &s.pl0));
@@ -1480,8 +1488,10 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &x.slots, x.n_slots));
     PD_TRY(dev_alloc(c, &x.red, (size_t)max_out + 8));
     if (c->use_tc) {
-      PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
-      PD_TRY(dev_alloc(c, &x.tail_count, (size_t)c->n_sms * 8));
+      if (!small) {
+        PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+        x.tail_count = s.tail_count + (size_t)i * c->n_sms * 8;
+      }
       x.pl_cap = s.pl_cap;
       PD_TRY(alloc_planes(c, x.pl_cap, &x.pl0));
       PD_TRY(alloc_planes(c, x.pl_cap, &x.pl1));
@@ -1687,12 +1697,16 @@ static int ensure_residual(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
+static int finish_steps(pdadmm_ctx *c, bool hit_cap);
+
 extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
   if (!c) return fail(PDADMM_EINVAL, "context is null");
   if (n_iters < 0) return fail(PDADMM_EINVAL, "n_iters is negative");
   PD_CUDA(cudaSetDevice(c->device));
   PD_CUDA(cudaEventRecord(c->ev_begin, c->scr.st));
-  PD_CUDA(cudaMemsetAsync(c->d_flag, 0, 3 * sizeof(int), c->scr.st));
+  // The counters are zero already, unless a bounded wait expired in a product: its blocks then gave up between one arrival and
+  // the last, and a count that starts from the leftover would take incomplete sums for complete ones.
+  PD_CUDA(cudaMemsetAsync(c->control, 0, c->control_words * sizeof(int), c->scr.st));
   PD_TRY(ensure_residual(c));
   bool hit_cap = false;
   // pdADMM-G has no host decision inside an iteration, so after a first eager iteration the sequence of launches
@@ -1731,6 +1745,11 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
       PD_TRY(iterate_once(c, &hit_cap));
     }
   }
+  return finish_steps(c, hit_cap);
+}
+
+// What the iterations left in the error words.
+static int finish_steps(pdadmm_ctx *c, bool hit_cap) {
   PD_CUDA(cudaMemcpyAsync(c->h_pinned + 8, c->d_flag, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->scr.st));
   PD_CUDA(cudaEventRecord(c->ev_end, c->scr.st));
   PD_CUDA(cudaStreamSynchronize(c->scr.st));
@@ -1741,7 +1760,11 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
     c->last_step_ms = ms;
   }
   if (c->profiling) PD_TRY(prof_collect(c));
-  if (c->h_pinned[9] != 0) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+  if (c->h_pinned[9] != 0) {
+    // nothing derived from the tensors was finished either
+    c->r_valid = c->t_valid = c->w_planes_valid = c->amax_p_valid = false;
+    return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+  }
   if (c->h_pinned[10] != 0) return fail(PDADMM_ENUMERIC, "a non-finite value reached the gradient norms: the state holds NaN or Inf");
   if (c->h_pinned[8] != 0)
     return fail(PDADMM_ENOTCONV, "the last-layer z solver did not converge on %d nodes", c->h_pinned[8]);
@@ -1863,7 +1886,10 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   }
   if (counts_out)
     for (int i = 0; i < 4; ++i) counts_out[i] = (int64_t)h_counts[i];
-  if (h_counts[4]) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+  if (h_counts[4]) {
+    PD_CUDA(cudaMemsetAsync(c->control, 0, c->control_words * sizeof(int), st));
+    return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+  }
   return PDADMM_OK;
 }
 
@@ -2177,6 +2203,21 @@ extern "C" int pdadmm_selftest_bounded_wait(int device, long long limit_cycles, 
   const int rc = body();
   cudaFree(d_err);
   return rc;
+}
+
+// The words of a context as blocks that gave up in the middle of their products leave them (the error word set, counters between
+// one arrival and the last, largest magnitudes of no number), then what pdadmm_step does after its last iteration.
+extern "C" int pdadmm_selftest_expired_wait(pdadmm_ctx *c) {
+  if (!c) return fail(PDADMM_EINVAL, "context is null");
+  PD_CUDA(cudaSetDevice(c->device));
+  std::vector<int> words(c->control_words, 1);
+  words[0] = words[2] = 0;
+  for (int l = 0; l < c->L; ++l)
+    for (int i = 4; i < 8; ++i) words[4 + 8 * (size_t)l + i] = 0x7fc00000;
+  PD_CUDA(cudaEventRecord(c->ev_begin, c->scr.st));
+  PD_CUDA(cudaMemcpyAsync(c->control, words.data(), words.size() * sizeof(int), cudaMemcpyHostToDevice, c->scr.st));
+  PD_CUDA(cudaStreamSynchronize(c->scr.st));
+  return finish_steps(c, false);
 }
 
 // ---- timing ----------------------------------------------------------------------------------------------------
