@@ -9,6 +9,8 @@
 
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -547,7 +549,7 @@ struct Zqu {
   PlaneOut rp;                            // planes of r for the coming p-gradient
   int n_blocks;
 };
-struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T; };
+struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T, table_even; };
 __global__ void __launch_bounds__(EW_THREADS)
 zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
   const Zqu &y = group.l[blockIdx.y];
@@ -609,18 +611,24 @@ zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ Zqu
 // c h^2 j (j - 1) / 2 - (10 j + 11) eps g - 4 (j + 1) sqrt(g) d, which is positive for every j >= 2 if it is for j = 2:
 // c h^2 > 31 eps g + 12 sqrt(g) d.  Elements that fail the test (and NaN) try all candidates as before, so the result is the same
 // bit for bit.  10 000 x 256, 513 candidates: 474 us with all candidates tried, 35 us so.
+// All this for candidates that lie where they should: z_i = fl(lo + fl(i h)) is up to 3 eps max|z| off, and the room left in the
+// constants of the test (8 %) covers 0.25 % of h at every candidate.  A table whose spacing is below 1200 eps max|z| (one far from zero: lo = 1000, 1010
+// wide, 4096 candidates; never one that reaches from -x to x) is searched as a whole (table_is_even, on the host).
+inline bool table_is_even(float lo, float hi, float step) {
+  return (double)step >= 1200.0 * 5.9604644775390625e-8 * std::max(std::fabs((double)lo), std::fabs((double)hi));
+}
 __device__ __forceinline__ float table_h(float z, float f, float a, float q, float zk) {
   const float d0 = z - a, d1 = q - f, d2 = z - zk;
   return fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
 }
-__device__ __forceinline__ void table_best(const float *__restrict__ f_sh, int T, float lo, float step, float act, float a, float q,
-                                           float zk, float &z_best, float &f_best) {
+__device__ __forceinline__ void table_best(const float *__restrict__ f_sh, int T, float lo, float step, bool even, float act, float a,
+                                           float q, float zk, float &z_best, float &f_best) {
   auto z_at = [&](int i) { return __fadd_rn(lo, __fmul_rn((float)i, step)); };
   auto h_at = [&](int i) { return table_h(z_at(i), f_sh[i], a, q, zk); };
   const bool th = act == ACT_TANH;
   const float c = 4.0f - 2.0f * (th ? 0.77f : 0.0963f) * (fabsf(q) + 1.0f);
   const float m = 0.5f * (a + zk), inv_step = 1.0f / step, top = (float)(T - 1);
-  if (c > 0.1f && fabsf(m) < 1e30f) {
+  if (even && c > 0.1f && fabsf(m) < 1e30f) {
     float x = fminf(fmaxf((m - lo) * inv_step, 0.0f), top);
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
@@ -666,6 +674,7 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
   const float rho = prm.rho, nu = prm.nu, act = prm.slope, q_top = prm.q_top, q_scale = y.q_scale, q_lo = y.q_lo;
   const float t_lo = prm.t_lo, t_step = prm.t_step;
   const int T = prm.T;
+  const bool even = prm.table_even != 0;
   extern __shared__ float table_sh[];              // f(z_i)
   for (int i = threadIdx.x; i < T; i += blockDim.x) table_sh[i] = act_eval(__fadd_rn(t_lo, __fmul_rn((float)i, t_step)), act);
   __syncthreads();
@@ -685,7 +694,7 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
     const float zo[4] = {zv.x, zv.y, zv.z, zv.w}, qo[4] = {qv.x, qv.y, qv.z, qv.w};
     float zb[4], fb[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) table_best(table_sh, T, t_lo, t_step, act, a[e], qo[e], zo[e], zb[e], fb[e]);
+    for (int e = 0; e < 4; ++e) table_best(table_sh, T, t_lo, t_step, even, act, a[e], qo[e], zo[e], zb[e], fb[e]);
     const float pn[4] = {pv.x, pv.y, pv.z, pv.w}, uo[4] = {uv.x, uv.y, uv.z, uv.w};
     float zn[4], qn[4], un[4], rn[4], tn[4];
 #pragma unroll

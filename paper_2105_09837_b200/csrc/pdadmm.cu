@@ -165,6 +165,7 @@ struct pdadmm_ctx {
   float slope = 0.f;               // f_l (see act_eval): [0, 1) = (leaky) ReLU with that slope for x <= 0, 2 = tanh, 3 = sigmoid
   float table_lo = 0.f, table_step = 0.f;   // lookup table of the z-update of a smooth activation: z_i = lo + i step
   int table_size = 0;
+  bool table_even = false;         // see table_is_even
   bool ls_risk = false;            // R = least squares instead of cross-entropy
   float rho = 0, nu = 0;
   uint32_t flags = 0;
@@ -992,7 +993,7 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   }
   Launch k(c, KC_ZQU, st, bytes, 0);
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
-                      c->table_step, c->table_size};
+                      c->table_step, c->table_size, c->table_even ? 1 : 0};
   const dim3 grid((unsigned)blocks, (unsigned)n);
   if (c->table_size > 0) zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), st>>>(g, prm);
   else zqu_kernel<<<grid, EW_THREADS, 0, st>>>(g, prm);
@@ -1325,6 +1326,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     c->table_size = cfg->table_size;
     c->table_lo = cfg->table_lo;
     c->table_step = (cfg->table_hi - cfg->table_lo) / (float)(cfg->table_size - 1);      // single precision, like the candidates
+    c->table_even = table_is_even(cfg->table_lo, cfg->table_hi, c->table_step);
   }
   c->ls_risk = (cfg->flags & PDADMM_FLAG_LEAST_SQUARES) != 0;
   c->rho = cfg->rho; c->nu = cfg->nu; c->flags = cfg->flags;

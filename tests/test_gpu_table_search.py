@@ -46,3 +46,42 @@ def test_the_table_candidate_is_the_best_of_all(act, T, lo, hi, q_scale):
         size = np.abs(a) + np.abs(z0[l]) + np.abs(q0[l]) + abs(lo) + abs(hi)
         assert np.all(got - best <= 1e-5 * best + 4e-6 * size * (np.sqrt(best) + step))
     ctx.destroy()
+
+
+@pytest.mark.parametrize("act", [1, 2])
+@pytest.mark.parametrize("lo,r,T", [(1e6, 0.3, 78), (7.3e6, 0.1, 66), (3e6, 0.7, 58), (1e6, 4.0, 50), (600.0, 1000.0, 50)])
+def test_a_table_finer_than_the_numbers_it_holds(act, lo, r, T):
+    """Spacings of r units in the last place of the candidates: neighbouring candidates coincide or lie unevenly, and only a search
+    over all of them finds the first smallest one.  With p = 0 every operand is known bit for bit: b = 0 at the start, so
+    r = -z, its column mean (a sum that double precision holds exactly) goes to b, a = (r - mean) + z, and f is 1 at such z.
+    (The spacing of the last table is resolved: it takes the short search.)"""
+    f = np.float32
+    n, width = 777, 64
+    lo = f(lo)
+    hi = f(lo + r * np.spacing(lo) * (T - 1))
+    inp = synth.make_inputs(synth.small("c2", n, feat_dim=9, hidden=width, n_layers=2, quant_levels=0))
+    inp.features = np.zeros_like(inp.features)
+    rng = np.random.default_rng(T)
+    col = rng.uniform(lo - 0.3 * (hi - lo), hi + 0.3 * (hi - lo), width).astype(f)
+    z0 = (col + np.spacing(lo) * rng.integers(-5, 6, (n, width))).astype(f)
+    q0 = (1 + rng.standard_normal((n, width)) * rng.choice([0, 1e-2, 0.3], (n, width))).astype(f)
+    ctx = B.from_inputs(inp, activation=act, table=(T, float(lo), float(hi)))
+    ctx.set_tensor(B.T_Z, 1, z0)
+    ctx.set_tensor(B.T_Q, 1, q0)
+    ctx.step(1)
+    z = ctx.get_tensor(B.T_Z, 1)
+    ctx.destroy()
+    step = f(hi - lo) / f(T - 1)
+    pts = lo + np.arange(T, dtype=f) * step
+    fv = (np.tanh(pts.astype(np.float64)) if act == 1 else 1 / (1 + np.exp(-pts.astype(np.float64)))).astype(f)
+    mean = (-z0).astype(np.float64).sum(0) * (1.0 / n)
+    a = ((-z0) - mean.astype(f)) + z0
+
+    def fma(x, y, c):
+        return (x.astype(np.float64) * y + c).astype(f)      # the product is exact in double precision
+    best, want = np.full(z.shape, np.inf, f), np.zeros(z.shape, f)
+    for i in range(T):
+        d0, d1, d2 = pts[i] - a, q0 - fv[i], pts[i] - z0
+        h = fma(d0, d0, fma(d1, d1, d2 * d2))
+        want, best = np.where(h < best, pts[i], want), np.minimum(h, best)
+    assert np.array_equal(z, want)
