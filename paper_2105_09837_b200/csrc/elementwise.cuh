@@ -720,7 +720,8 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
 // (Eq. "update zl"), the unique root of softmax(z) - e_y + nu (z - a) = 0, by damped Newton with the
 // Hessian diag(s) + nu I - s s^T inverted through the rank-one update formula; double precision
 // inside, since nu is small and the Hessian is close to singular along (1,..,1).  Unlabelled: z+ = a.
-// The search starts from the stored z, the root for the previous a, where the gradient is nu (a_old - a) alone.
+// The search starts from the stored z, the root for the previous a, where the gradient is nu (a_old - a) alone; where that does
+// not converge (an a that moved by 1e4 at nu = 1e-6) it starts again from a.
 //
 // G lanes share a node, two classes each, everything in registers, sums by shuffles; the loop is common to the warp and has
 // one evaluation per turn: a group whose trial point is accepted takes the gradient there from the exponentials it just
@@ -763,6 +764,7 @@ zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restri
     bool done = !labelled, resolvable = false;
     double d[2] = {0.0, 0.0}, t = 0.0, fx = 0.0, slope = 0.0;
     int steps = 0;
+    bool from_a = false;
     while (__any_sync(0xffffffffu, !done)) {
       const double v[2] = {x[0] + t * d[0], x[1] + t * d[1]};
       const double m = top(fmax(in[0] ? v[0] : -1e300, in[1] ? v[1] : -1e300));
@@ -790,7 +792,11 @@ zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restri
           d[0] = nd[0]; d[1] = nd[1]; slope = ns; t = 1.0;
           resolvable = -slope > 1e-9 * (1.0 + fabs(fx));
           if (gmax <= 1e-10) done = true;
-          else if (++steps >= 100) {
+          else if (++steps >= 100 && !from_a) {
+            from_a = true;
+            x[0] = a[0]; x[1] = a[1];
+            steps = 0; t = 0.0; resolvable = false;
+          } else if (steps >= 100) {
             done = true;
             if (lane == 0) atomicAdd(not_converged, 1);
           }
