@@ -303,7 +303,7 @@ struct Launch {                    // brackets one kernel launch
 };
 static int prof_collect(pdadmm_ctx *c) {
   if (c->prof.empty()) return PDADMM_OK;
-  PD_CUDA(cudaDeviceSynchronize());
+  PD_CUDA(cudaStreamSynchronize(c->scr.st));          // every lane has joined it
   for (auto &r : c->prof) {
     float ms = 0.f;
     cudaEventElapsedTime(&ms, r.e0, r.e1);
@@ -1151,13 +1151,16 @@ static int upload_rows(pdadmm_ctx *c, cudaStream_t st, float *dst, int ld, const
   return copy_rows(c->device, st, const_cast<float *>(src), dst, (size_t)ld * 4, (size_t)width * 4, (size_t)rows, false);
 }
 
-// Temporary device buffers of the CSR construction, carved out of one block that goes back when the builder returns.
+// Temporary device buffers of the CSR construction, carved out of one block that goes back when the builder returns.  The stream
+// is waited for, not the device: that would wait for other threads' contexts too, and it is an error while one of them
+// captures its iteration.
 struct TempBuffers {
   int device;
+  cudaStream_t st;
   std::vector<DeviceBlock> block;
   size_t used = 0;
-  explicit TempBuffers(int dev) : device(dev) {}
-  ~TempBuffers() { if (!block.empty()) { cudaDeviceSynchronize(); device_pool(device).give(block); } }
+  TempBuffers(int dev, cudaStream_t s) : device(dev), st(s) {}
+  ~TempBuffers() { if (!block.empty()) { cudaStreamSynchronize(st); device_pool(device).give(block); } }
   static size_t room(size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) & ~size_t(255); }
   int reserve(size_t bytes) {
     DeviceBlock b;
@@ -1183,7 +1186,7 @@ static int build_csr(pdadmm_ctx *c, const pdadmm_config *cfg) {
   const size_t raw_cap = (size_t)(2 * E + N);
   if (raw_cap > (size_t)INT32_MAX) return fail(PDADMM_EINVAL, "more than 2^31-1 non-zeros");
   cudaStream_t st = c->scr.st;
-  TempBuffers tmp(c->device);
+  TempBuffers tmp(c->device, st);
   const size_t n4 = TempBuffers::room((size_t)N * 4 + 4);
   PD_TRY(tmp.reserve(2 * TempBuffers::room((size_t)E * 4) + 5 * n4 + 2 * TempBuffers::room(raw_cap * 4) + 1024));
   int *d_src, *d_dst, *deg, *cursor, *raw_ptr, *raw, *sorted, *len, *long_rows, *meta;
@@ -1359,9 +1362,9 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   // keeps the rows of its own nodes
   float *x_full = nullptr;
   struct BlockLater {
-    int device; std::vector<DeviceBlock> b;
-    ~BlockLater() { if (!b.empty()) { cudaDeviceSynchronize(); device_pool(device).give(b); } }
-  } x_full_block{c->device, {}};
+    int device; cudaStream_t st; std::vector<DeviceBlock> b;
+    ~BlockLater() { if (!b.empty()) { cudaStreamSynchronize(st); device_pool(device).give(b); } }
+  } x_full_block{c->device, st, {}};
   if (sharded) {
     const size_t bytes = (size_t)Ntot * c->ld0 * 4 + 256;
     DeviceBlock b;
@@ -1541,7 +1544,10 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
 static void destroy(pdadmm_ctx *c) {
   if (!c) return;
   cudaSetDevice(c->device);
-  cudaDeviceSynchronize();
+  for (int i = 0; i <= (int)c->more_lanes.size(); ++i) {            // everything of this context runs on streams of its own
+    const cudaStream_t st = i == 0 ? c->scr.own : c->more_lanes[i - 1]->own;
+    if (st != nullptr) cudaStreamSynchronize(st);
+  }
   for (auto &r : c->prof) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
   for (auto e : c->ev_pool) cudaEventDestroy(e);
   if (c->iter_graph) cudaGraphExecDestroy(c->iter_graph);
