@@ -242,8 +242,9 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       const int ea = y.oa.exp ? *y.oa.exp : 0, eb = y.ob.exp ? *y.ob.exp : 0;
       const uint32_t ma = y.oa.amax ? *y.oa.amax : 0u, mb = y.ob.amax ? *y.ob.amax : 0u;
       const bool good_a = y.oa.amax == nullptr || tc_planes_usable(ma, ea), good_b = y.ob.amax == nullptr || tc_planes_usable(mb, eb);
-      lay_exp[lane][0] = good_a ? ea : tc_scale_exp(ma);
-      lay_exp[lane][1] = good_b ? eb : tc_scale_exp(mb);
+      // (a matrix of zeros is good whatever its exponent, that of no prediction included: any factor will do then)
+      lay_exp[lane][0] = !good_a ? tc_scale_exp(ma) : ea < -100 || ea > 100 ? 0 : ea;
+      lay_exp[lane][1] = !good_b ? tc_scale_exp(mb) : eb < -100 || eb > 100 ? 0 : eb;
       lay_split[lane] = (!good_a && y.oa.x != nullptr ? 1 : 0) | (!good_b && y.ob.x != nullptr ? 2 : 0);
     }
   }
@@ -517,10 +518,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       const int tid = aw * 32 + lane;
       volatile int *last = reinterpret_cast<volatile int *>(team_scratch);
       volatile double *part = team_scratch + 1;
-      __threadfence();
       if (!team_sync()) return false;
       if (tid == 0) {
         const int units = (grp.unit_end[g] - (g > 0 ? grp.unit_end[g - 1] : 0)) * CG;
+        __threadfence();                 // the team's sums and maxima, which its arrivals put before this, come before the count
         const int before = atomicAdd(y.done, visited);
         *last = before + visited == units;
       }
@@ -728,10 +729,12 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
               release_part();
             }
             if (!ok) break;
-            __threadfence();
             __syncwarp();
             int prev = 0;
-            if (lane == 0) prev = atomicAdd(y.tail_count + t_idx * WARPS + piece, 1);
+            if (lane == 0) {
+              __threadfence();             // of the whole warp's parked values
+              prev = atomicAdd(y.tail_count + t_idx * WARPS + piece, 1);
+            }
             prev = __shfl_sync(0xffffffffu, prev, 0);
             whole = prev == y.tail_split - 1;
             if (whole) {
