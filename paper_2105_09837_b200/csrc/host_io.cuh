@@ -90,12 +90,13 @@ unpack_rows_kernel(const T *__restrict__ src, size_t pitch, uint32_t width, uint
     dst[(size_t)row * pitch + (i - row * width)] = src[i];
   }
 }
-inline void launch_pack(cudaStream_t st, const void *src, size_t pitch_bytes, size_t width_bytes, size_t rows, void *dst) {
+inline cudaError_t launch_pack(cudaStream_t st, const void *src, size_t pitch_bytes, size_t width_bytes, size_t rows, void *dst) {
   const bool wide = pitch_bytes % 16 == 0 && width_bytes % 16 == 0 && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 16 == 0;
   const uint32_t n = (uint32_t)(rows * width_bytes / (wide ? 16 : 4));
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 148));
   if (wide) pack_rows_kernel<uint4><<<grid, 256, 0, st>>>((const uint4 *)src, pitch_bytes / 16, (uint32_t)(width_bytes / 16), n, (uint4 *)dst);
   else pack_rows_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t *)src, pitch_bytes / 4, (uint32_t)(width_bytes / 4), n, (uint32_t *)dst);
+  return cudaGetLastError();           // (kept per host thread: nobody else could ask for it later)
 }
 
 inline cudaError_t queue_unpack(cudaStream_t st, const void *src, void *dst, size_t pitch, size_t width, size_t rows) {
@@ -132,7 +133,7 @@ inline cudaError_t copy_pieces(const RowCopy &k, size_t piece0, size_t step, cha
   for (size_t p = piece0; p < n_pieces && e == cudaSuccess; p += step, b ^= 1) {
     const size_t r = rows_of(p);
     if (k.out) {
-      if (k.width % 4 == 0 && k.pitch % 4 == 0) launch_pack(k.st, dev_of(p), k.pitch, k.width, r, stage[b]);
+      if (k.width % 4 == 0 && k.pitch % 4 == 0) e = launch_pack(k.st, dev_of(p), k.pitch, k.width, r, stage[b]);
       else e = cudaMemcpy2DAsync(stage[b], k.width, dev_of(p), k.pitch, k.width, r, cudaMemcpyDeviceToHost, k.st);
       if (e == cudaSuccess) e = cudaEventRecord(ev[b], k.st);
       if (e == cudaSuccess && before != SIZE_MAX) land(before, b ^ 1);
@@ -179,8 +180,7 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
       memcpy(stage, host, rows * width);
       e = queue_unpack(st, stage, dev, pitch, width, rows);
     } else if (width % 4 == 0 && pitch % 4 == 0) {
-      launch_pack(st, dev, pitch, width, rows, stage);
-      e = cudaGetLastError();
+      e = launch_pack(st, dev, pitch, width, rows, stage);
     } else {
       e = cudaMemcpy2DAsync(stage, width, dev, pitch, width, rows, cudaMemcpyDeviceToHost, st);
     }

@@ -1878,9 +1878,11 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
   const size_t row = (size_t)last.n_out * 4, lg_bytes = logits_out ? (size_t)N * row : 0, pr_bytes = pred_out ? (size_t)N * 4 : 0;
   char *stage = lg_bytes + pr_bytes <= STAGE_BYTES ? (char *)stage_pool().take() : nullptr;
   if (stage != nullptr) {       // small: everything packed into one page-locked block, one wait for the whole call
-    if (logits_out) launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);
-    if (pred_out) launch_pack(st, d_pred, pr_bytes, pr_bytes, 1, stage + lg_bytes);
-    const cudaError_t e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaSuccess;
+    if (logits_out) e = launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);
+    if (pred_out && e == cudaSuccess) e = launch_pack(st, d_pred, pr_bytes, pr_bytes, 1, stage + lg_bytes);
+    const cudaError_t w = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = w;
     if (e == cudaSuccess) {
       if (logits_out) memcpy(logits_out, stage, lg_bytes);
       if (pred_out) memcpy(pred_out, stage + lg_bytes, pr_bytes);

@@ -1,0 +1,29 @@
+// The host side of the library's copies and pools against a CUDA runtime that is a fake (host_paths_fake.cpp).  Built and run by
+// test_host_paths.py, one scenario per process.
+#include "../paper_2105_09837_b200/csrc/host_io.cuh"
+
+#include "host_paths_fake.h"
+
+
+using namespace pd;
+static int check(bool ok, const char *what) { printf("%s: %s\n", what, ok ? "yes" : "NO"); return ok ? 0 : 1; }
+
+int main(int argc, char **argv) {
+  main_thread = true;
+  const std::string what = argc > 1 ? argv[1] : "";
+  constexpr size_t rows = 20000, width = 400, pitch = 512;           // 8 MB: four threads
+  std::vector<char> host(rows * width), dev(rows * pitch);
+  if (what == "copies") {
+    return check(copy_rows(0, nullptr, host.data(), dev.data(), pitch, width, rows, true) == PDADMM_OK && launches > 1, "a copy in pieces succeeds");
+  }
+  if (what == "launch fails in workers") {
+    launches_fail_in_workers = true;
+    return check(copy_rows(0, nullptr, host.data(), dev.data(), pitch, width, rows, true) == PDADMM_ECUDA, "the failed launch is reported");
+  }
+  if (what == "launch fails") {
+    launches_fail = true;
+    return check(copy_rows(0, nullptr, host.data(), dev.data(), pitch, width, 100, true) == PDADMM_ECUDA, "one piece: reported") +
+           check(launch_pack(nullptr, dev.data(), pitch, width, 100, host.data()) != cudaSuccess, "the launch says so itself");
+  }
+  return 2;
+}
