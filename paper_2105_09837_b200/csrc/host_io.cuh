@@ -63,10 +63,11 @@ class PinnedPool {
 inline PinnedPool &stage_pool() { static PinnedPool &p = *new PinnedPool(STAGE_BYTES, PINNED_KEEP); return p; }
 inline PinnedPool &ctx_pinned_pool() { static PinnedPool &p = *new PinnedPool(CTX_PINNED_BYTES, CTX_PINNED_KEEP); return p; }
 
-inline bool is_pinned(const void *p) {
+// Memory that the driver copies by itself: page-locked or managed, or device memory, which the host must not touch.
+inline bool is_direct(const void *p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
-  return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeManaged;
+  return a.type != cudaMemoryTypeUnregistered;
 }
 
 // rows of `width` words at a pitch of `pitch` words -> dense; T = uint4 where both allow it, so that a warp writes whole
@@ -166,9 +167,9 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
     PD_TRY(copy_rows(device, st, host, dev, unit, unit, whole, out));
     return copy_rows(device, st, (char *)host + whole * unit, (char *)dev + whole * unit, unit, total % unit, 1, out);
   }
-  if (width > STAGE_BYTES || is_pinned(host)) {
-    if (out) PD_CUDA(cudaMemcpy2DAsync(host, width, dev, pitch, width, rows, cudaMemcpyDeviceToHost, st));
-    else PD_CUDA(cudaMemcpy2DAsync(dev, pitch, host, width, width, rows, cudaMemcpyHostToDevice, st));
+  if (width > STAGE_BYTES || is_direct(host)) {
+    if (out) PD_CUDA(cudaMemcpy2DAsync(host, width, dev, pitch, width, rows, cudaMemcpyDefault, st));
+    else PD_CUDA(cudaMemcpy2DAsync(dev, pitch, host, width, width, rows, cudaMemcpyDefault, st));
     PD_CUDA(cudaStreamSynchronize(st));
     return PDADMM_OK;
   }

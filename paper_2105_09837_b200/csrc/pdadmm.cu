@@ -1876,7 +1876,8 @@ extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_ou
       out, c->labels, c->mask, N, last.n_out, last.ld_out, d_pred, c->counts, c->done, c->d_flag + 1, h_counts);
   PD_CUDA(cudaGetLastError());
   const size_t row = (size_t)last.n_out * 4, lg_bytes = logits_out ? (size_t)N * row : 0, pr_bytes = pred_out ? (size_t)N * 4 : 0;
-  char *stage = lg_bytes + pr_bytes <= STAGE_BYTES ? (char *)stage_pool().take() : nullptr;
+  const bool staged = lg_bytes + pr_bytes <= STAGE_BYTES && !(logits_out && is_direct(logits_out)) && !(pred_out && is_direct(pred_out));
+  char *stage = staged ? (char *)stage_pool().take() : nullptr;
   if (stage != nullptr) {       // small: everything packed into one page-locked block, one wait for the whole call
     cudaError_t e = cudaSuccess;
     if (logits_out) e = launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);

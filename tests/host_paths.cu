@@ -4,6 +4,7 @@
 
 #include "host_paths_fake.h"
 
+#include <sys/mman.h>
 
 using namespace pd;
 static int check(bool ok, const char *what) { printf("%s: %s\n", what, ok ? "yes" : "NO"); return ok ? 0 : 1; }
@@ -24,6 +25,14 @@ int main(int argc, char **argv) {
     launches_fail = true;
     return check(copy_rows(0, nullptr, host.data(), dev.data(), pitch, width, 100, true) == PDADMM_ECUDA, "one piece: reported") +
            check(launch_pack(nullptr, dev.data(), pitch, width, 100, host.data()) != cudaSuccess, "the launch says so itself");
+  }
+  if (what == "device pointer") {                                    // neither readable nor writable for the host
+    on_device = mmap(nullptr, rows * width, PROT_NONE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+    int bad = 0;
+    for (const bool out : {true, false})
+      for (const size_t n : {size_t(1), size_t(100), rows})
+        bad += check(copy_rows(0, nullptr, on_device, dev.data(), pitch, width, n, out) == PDADMM_OK, "copied");
+    return bad + check(direct_copies >= 6 && launches == 0, "by the driver");
   }
   return 2;
 }
