@@ -5,6 +5,8 @@
 #include <stdarg.h>
 #include <stdint.h>
 #include <stdio.h>
+#include <exception>
+#include <new>
 #include <string>
 
 #include "../../include/pdadmm.h"
@@ -23,8 +25,23 @@ inline int fail(int code, const char *fmt, ...) {
   va_start(ap, fmt);
   vsnprintf(buf, sizeof buf, fmt, ap);
   va_end(ap);
-  err_text() = buf;
+  try {
+    err_text() = buf;
+  } catch (...) {                       // no memory for the text either
+    err_text().clear();
+  }
   return code;
+}
+// The body of an entry point: no C++ exception leaves the C ABI.
+template <class F>
+inline int guarded(F &&body) {
+  try {
+    return body();
+  } catch (const std::bad_alloc &) {
+    return fail(PDADMM_ENOMEM, "out of host memory");
+  } catch (const std::exception &e) {
+    return fail(PDADMM_ECUDA, "unexpected exception: %s", e.what());
+  }
 }
 
 #define PD_CUDA(expr)                                                                             \

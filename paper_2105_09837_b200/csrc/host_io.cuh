@@ -13,7 +13,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
-#include <system_error>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -31,7 +31,7 @@ constexpr size_t CTX_PINNED_BYTES = size_t(64) << 10;  // the read-back words of
 constexpr size_t PINNED_KEEP = 8, CTX_PINNED_KEEP = 16;
 class PinnedPool {
  public:
-  PinnedPool(size_t bytes, size_t keep) : bytes_(bytes), keep_(keep) {}
+  PinnedPool(size_t bytes, size_t keep) : bytes_(bytes), keep_(keep) { free_.reserve(keep); }     // (give never allocates)
   void *take() {
     {
       std::lock_guard<std::mutex> g(m_);
@@ -50,9 +50,16 @@ class PinnedPool {
     cudaFreeHost(p);
   }
   void trim() {
-    std::vector<void *> f;
-    { std::lock_guard<std::mutex> g(m_); f.swap(free_); }
-    for (void *p : f) cudaFreeHost(p);
+    for (;;) {
+      void *p = nullptr;
+      {
+        std::lock_guard<std::mutex> g(m_);
+        if (free_.empty()) return;
+        p = free_.back();
+        free_.pop_back();
+      }
+      cudaFreeHost(p);
+    }
   }
  private:
   const size_t bytes_, keep_;
@@ -196,35 +203,37 @@ inline int copy_rows(int device, cudaStream_t st, void *host, void *dev, size_t 
   const size_t n_pieces = (size_t)ceil_div((int64_t)rows, (int64_t)k.piece_rows);
   const int T = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(4, n_pieces), rows * width / (size_t(2) << 20)));
   struct Worker { char *stage[2] = {nullptr, nullptr}; cudaEvent_t ev[2] = {nullptr, nullptr}; cudaError_t e = cudaSuccess; };
-  std::vector<Worker> ws(T);
+  Worker ws[4];
+  DevicePool &events = device_pool(device);        // (made before anything is taken: the first call allocates)
   cudaError_t err = cudaSuccess;
   const int n_stage = n_pieces > (size_t)T ? 2 : 1;
-  for (auto &w : ws)
+  for (int t = 0; t < T; ++t)
     for (int i = 0; i < 2 && err == cudaSuccess; ++i) {
+      Worker &w = ws[t];
       w.stage[i] = i < n_stage ? (char *)stage_pool().take() : w.stage[0];
       if (w.stage[i] == nullptr) err = cudaErrorMemoryAllocation;
-      else err = device_pool(device).take_event(false, &w.ev[i]);
+      else err = events.take_event(false, &w.ev[i]);
     }
   if (err == cudaSuccess) {
     auto body = [&](int t) {
       cudaSetDevice(device);
       ws[t].e = copy_pieces(k, (size_t)t, (size_t)T, ws[t].stage, ws[t].ev);
     };
-    std::vector<std::thread> threads;
+    std::thread threads[4];
     int started = 1;
     try {
-      for (; started < T; ++started) threads.emplace_back(body, started);
-    } catch (const std::system_error &) {     // no thread to be had: this one does their pieces
+      for (; started < T; ++started) threads[started] = std::thread(body, started);
+    } catch (const std::exception &) {        // no thread, or no memory for one, to be had: this one does their pieces
     }
     body(0);
     for (int t = started; t < T; ++t) body(t);
-    for (auto &t : threads) t.join();
-    for (auto &w : ws) if (err == cudaSuccess) err = w.e;
+    for (int t = 1; t < started; ++t) threads[t].join();
+    for (int t = 0; t < T; ++t) if (err == cudaSuccess) err = ws[t].e;
   }
-  for (auto &w : ws)
+  for (int t = 0; t < T; ++t)
     for (int i = 0; i < 2; ++i) {
-      device_pool(device).give_event(false, w.ev[i]);
-      if (i < n_stage) stage_pool().give(w.stage[i]);
+      events.give_event(false, ws[t].ev[i]);
+      if (i < n_stage) stage_pool().give(ws[t].stage[i]);
     }
   PD_CUDA(err);
   PD_CUDA(cudaGetLastError());

@@ -1602,12 +1602,7 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
   if (cfg->device < 0 || cfg->device >= n_dev || cfg->device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "device %d does not exist", cfg->device);
   pdadmm_ctx *c = new (std::nothrow) pdadmm_ctx();
   if (!c) return fail(PDADMM_ENOMEM, "out of host memory");
-  int rc;
-  try {
-    rc = build(c, cfg, shard);
-  } catch (const std::bad_alloc &) {
-    rc = fail(PDADMM_ENOMEM, "out of host memory");
-  }
+  const int rc = guarded([&] { return build(c, cfg, shard); });
   if (rc != PDADMM_OK) { destroy(c); return rc; }
   *out = c;
   return PDADMM_OK;
@@ -1616,17 +1611,19 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
 static int refresh_p(pdadmm_ctx *c);
 
 extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
-  if (first_layer < 1 || first_layer > c->L) return fail(PDADMM_EINVAL, "first_layer must be in [1, %d]", c->L);
-  PD_CUDA(cudaSetDevice(c->device));
-  PD_TRY(refresh_p(c));
-  PD_TRY(feasible_start(c, first_layer - 1));
-  PD_CUDA(cudaStreamSynchronize(c->scr.st));
-  PD_CUDA(cudaGetLastError());
-  // the linear residual of the restarted layers is zero by construction; everything derived from the other tensors
-  // (the residual of the kept layers, t, planes, largest magnitudes) is rebuilt by the next call that needs it
-  c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false;
-  return PDADMM_OK;
+  return guarded([&]() -> int {
+    if (!c) return fail(PDADMM_EINVAL, "context is null");
+    if (first_layer < 1 || first_layer > c->L) return fail(PDADMM_EINVAL, "first_layer must be in [1, %d]", c->L);
+    PD_CUDA(cudaSetDevice(c->device));
+    PD_TRY(refresh_p(c));
+    PD_TRY(feasible_start(c, first_layer - 1));
+    PD_CUDA(cudaStreamSynchronize(c->scr.st));
+    PD_CUDA(cudaGetLastError());
+    // the linear residual of the restarted layers is zero by construction; everything derived from the other tensors
+    // (the residual of the kept layers, t, planes, largest magnitudes) is rebuilt by the next call that needs it
+    c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false;
+    return PDADMM_OK;
+  });
 }
 
 extern "C" int pdadmm_release_cached_memory(int device) {
@@ -1707,8 +1704,7 @@ static int ensure_residual(pdadmm_ctx *c) {
 
 static int finish_steps(pdadmm_ctx *c, bool hit_cap);
 
-extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
+static int run_steps(pdadmm_ctx *c, int n_iters) {
   if (n_iters < 0) return fail(PDADMM_EINVAL, "n_iters is negative");
   PD_CUDA(cudaSetDevice(c->device));
   PD_CUDA(cudaEventRecord(c->ev_begin, c->scr.st));
@@ -1731,7 +1727,7 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
     const int64_t before = c->launches;
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(c->scr.st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      const int rc = iterate_once(c, &hit_cap);
+      const int rc = guarded([&] { return iterate_once(c, &hit_cap); });      // the capture has to be ended whatever happens
       const cudaError_t e = cudaStreamEndCapture(c->scr.st, &g);
       if (rc != PDADMM_OK || e != cudaSuccess || cudaGraphInstantiate(&c->iter_graph, g, 0) != cudaSuccess) {
         c->iter_graph = nullptr;
@@ -1754,6 +1750,15 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
     }
   }
   return finish_steps(c, hit_cap);
+}
+
+extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
+  if (!c) return fail(PDADMM_EINVAL, "context is null");
+  const int rc = guarded([&] { return run_steps(c, n_iters); });
+  // an iteration that was abandoned half way may have work on lanes that the main stream has not joined
+  if (rc == PDADMM_ENOMEM || rc == PDADMM_ECUDA)
+    for (auto &x : c->more_lanes) cudaStreamSynchronize(x->own);
+  return rc;
 }
 
 // What the iterations left in the error words.
@@ -1819,106 +1824,112 @@ static int read_objective(pdadmm_ctx *c, int parts) {
 }
 
 extern "C" int pdadmm_objective(pdadmm_ctx *c, double out[6]) {
-  if (!c || !out) return fail(PDADMM_EINVAL, "null argument");
-  PD_CUDA(cudaSetDevice(c->device));
-  PD_TRY(ensure_residual(c));
-  cudaStream_t st = c->scr.st;
-  PD_TRY(read_objective(c, OBJ_ALL));
-  double lin = 0, act = 0, dual = 0, pen = 0, R = c->h_results[4 * (size_t)c->L];
-  for (int l = 0; l < c->L; ++l) {
-    const double *h = c->h_results + 4 * (size_t)l;
-    lin += h[0]; act += h[1]; dual += h[2]; pen += h[3];
-  }
-  if (c->reduce != nullptr) {                 // every component is a sum over nodes
-    double h[5] = {R, lin, act, dual, pen};
-    PD_CUDA(cudaMemcpyAsync(c->scr.red, h, sizeof h, cudaMemcpyHostToDevice, st));
-    PD_TRY(shard_sum(c, st, c->scr.red, 5, 1));
-    PD_CUDA(cudaMemcpyAsync(h, c->scr.red, sizeof h, cudaMemcpyDeviceToHost, st));
-    PD_CUDA(cudaStreamSynchronize(st));
-    R = h[0]; lin = h[1]; act = h[2]; dual = h[3]; pen = h[4];
-  }
-  out[0] = R; out[1] = 0.5 * c->nu * lin; out[2] = 0.5 * c->nu * act; out[3] = dual; out[4] = 0.5 * c->rho * pen;
-  out[5] = out[0] + out[1] + out[2] + out[3] + out[4];
-  return PDADMM_OK;
+  return guarded([&]() -> int {
+    if (!c || !out) return fail(PDADMM_EINVAL, "null argument");
+    PD_CUDA(cudaSetDevice(c->device));
+    PD_TRY(ensure_residual(c));
+    cudaStream_t st = c->scr.st;
+    PD_TRY(read_objective(c, OBJ_ALL));
+    double lin = 0, act = 0, dual = 0, pen = 0, R = c->h_results[4 * (size_t)c->L];
+    for (int l = 0; l < c->L; ++l) {
+      const double *h = c->h_results + 4 * (size_t)l;
+      lin += h[0]; act += h[1]; dual += h[2]; pen += h[3];
+    }
+    if (c->reduce != nullptr) {                 // every component is a sum over nodes
+      double h[5] = {R, lin, act, dual, pen};
+      PD_CUDA(cudaMemcpyAsync(c->scr.red, h, sizeof h, cudaMemcpyHostToDevice, st));
+      PD_TRY(shard_sum(c, st, c->scr.red, 5, 1));
+      PD_CUDA(cudaMemcpyAsync(h, c->scr.red, sizeof h, cudaMemcpyDeviceToHost, st));
+      PD_CUDA(cudaStreamSynchronize(st));
+      R = h[0]; lin = h[1]; act = h[2]; dual = h[3]; pen = h[4];
+    }
+    out[0] = R; out[1] = 0.5 * c->nu * lin; out[2] = 0.5 * c->nu * act; out[3] = dual; out[4] = 0.5 * c->rho * pen;
+    out[5] = out[0] + out[1] + out[2] + out[3] + out[4];
+    return PDADMM_OK;
+  });
 }
 
 extern "C" int pdadmm_predict(pdadmm_ctx *c, float *logits_out, int32_t *pred_out, int64_t counts_out[4]) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
-  PD_CUDA(cudaSetDevice(c->device));
-  cudaStream_t st = c->scr.st;
-  PD_TRY(ensure_operands(c));
-  // forward pass with the constraints enforced: activations alternate between the two scratch matrices
-  const int N = (int)c->N;
-  const float *in = c->layers[0].p;
-  float *bufs[2] = {c->scr.s1, c->scr.s2};
-  float *out = nullptr;
-  const uint32_t *w_in = nullptr;            // max|activations| of the layer's input
-  if (c->use_tc) {
-    PD_TRY(amax_reset(c, st));               // one word per layer output, all from one pass through the pool
-    w_in = c->layers[0].amax_p;
-  }
-  for (int l = 0; l < c->L; ++l) {
-    Layer &ly = c->layers[l];
-    out = bufs[l & 1];
-    uint32_t *w_out = nullptr;
-    if (c->use_tc) w_out = amax_take(c);
-    EpiBiasAct epi{out, ly.ld_out, ly.b, l + 1 < c->L ? 1 : 0, c->slope, w_out};
-    Operand P{in, ly.ld_in, w_in};
-    if (l == 0 && c->use_tc) P = operand_X(ly);
-    PD_TRY((gemm_nodes<false, EpiBiasAct>(c, KC_GEMM_RESID, st, {{N, ly.n_out, ly.n_in, P, operand_W(ly), epi, &c->scr}}, 0)));
-    w_in = w_out;
-    in = out;
-  }
-  const Layer &last = c->layers[c->L - 1];
-  int *d_pred = reinterpret_cast<int *>(bufs[c->L & 1]);              // the scratch matrix the logits are not in
-  unsigned long long *h_counts = reinterpret_cast<unsigned long long *>(c->h_results);
-  argmax_kernel<<<(int)std::min<int64_t>(1184, ceil_div(N, EW_THREADS)), EW_THREADS, 0, st>>>(
-      out, c->labels, c->mask, N, last.n_out, last.ld_out, d_pred, c->counts, c->done, c->d_flag + 1, h_counts);
-  PD_CUDA(cudaGetLastError());
-  const size_t row = (size_t)last.n_out * 4, lg_bytes = logits_out ? (size_t)N * row : 0, pr_bytes = pred_out ? (size_t)N * 4 : 0;
-  const bool staged = lg_bytes + pr_bytes <= STAGE_BYTES && !(logits_out && is_direct(logits_out)) && !(pred_out && is_direct(pred_out));
-  char *stage = staged ? (char *)stage_pool().take() : nullptr;
-  if (stage != nullptr) {       // small: everything packed into one page-locked block, one wait for the whole call
-    cudaError_t e = cudaSuccess;
-    if (logits_out) e = launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);
-    if (pred_out && e == cudaSuccess) e = launch_pack(st, d_pred, pr_bytes, pr_bytes, 1, stage + lg_bytes);
-    const cudaError_t w = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) e = w;
-    if (e == cudaSuccess) {
-      if (logits_out) memcpy(logits_out, stage, lg_bytes);
-      if (pred_out) memcpy(pred_out, stage + lg_bytes, pr_bytes);
+  return guarded([&]() -> int {
+    if (!c) return fail(PDADMM_EINVAL, "context is null");
+    PD_CUDA(cudaSetDevice(c->device));
+    cudaStream_t st = c->scr.st;
+    PD_TRY(ensure_operands(c));
+    // forward pass with the constraints enforced: activations alternate between the two scratch matrices
+    const int N = (int)c->N;
+    const float *in = c->layers[0].p;
+    float *bufs[2] = {c->scr.s1, c->scr.s2};
+    float *out = nullptr;
+    const uint32_t *w_in = nullptr;            // max|activations| of the layer's input
+    if (c->use_tc) {
+      PD_TRY(amax_reset(c, st));               // one word per layer output, all from one pass through the pool
+      w_in = c->layers[0].amax_p;
     }
-    stage_pool().give(stage);
-    PD_CUDA(e);
-  } else {
-    if (logits_out) PD_TRY(copy_rows(c->device, st, logits_out, out, (size_t)last.ld_out * 4, row, (size_t)N, true));
-    if (pred_out) PD_TRY(copy_rows(c->device, st, pred_out, d_pred, pr_bytes, pr_bytes, 1, true));
-    PD_CUDA(cudaStreamSynchronize(st));
-  }
-  if (counts_out)
-    for (int i = 0; i < 4; ++i) counts_out[i] = (int64_t)h_counts[i];
-  if (h_counts[4]) {
-    PD_CUDA(cudaMemsetAsync(c->control, 0, c->control_words * sizeof(int), st));
-    return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
-  }
-  return PDADMM_OK;
+    for (int l = 0; l < c->L; ++l) {
+      Layer &ly = c->layers[l];
+      out = bufs[l & 1];
+      uint32_t *w_out = nullptr;
+      if (c->use_tc) w_out = amax_take(c);
+      EpiBiasAct epi{out, ly.ld_out, ly.b, l + 1 < c->L ? 1 : 0, c->slope, w_out};
+      Operand P{in, ly.ld_in, w_in};
+      if (l == 0 && c->use_tc) P = operand_X(ly);
+      PD_TRY((gemm_nodes<false, EpiBiasAct>(c, KC_GEMM_RESID, st, {{N, ly.n_out, ly.n_in, P, operand_W(ly), epi, &c->scr}}, 0)));
+      w_in = w_out;
+      in = out;
+    }
+    const Layer &last = c->layers[c->L - 1];
+    int *d_pred = reinterpret_cast<int *>(bufs[c->L & 1]);              // the scratch matrix the logits are not in
+    unsigned long long *h_counts = reinterpret_cast<unsigned long long *>(c->h_results);
+    argmax_kernel<<<(int)std::min<int64_t>(1184, ceil_div(N, EW_THREADS)), EW_THREADS, 0, st>>>(
+        out, c->labels, c->mask, N, last.n_out, last.ld_out, d_pred, c->counts, c->done, c->d_flag + 1, h_counts);
+    PD_CUDA(cudaGetLastError());
+    const size_t row = (size_t)last.n_out * 4, lg_bytes = logits_out ? (size_t)N * row : 0, pr_bytes = pred_out ? (size_t)N * 4 : 0;
+    const bool staged = lg_bytes + pr_bytes <= STAGE_BYTES && !(logits_out && is_direct(logits_out)) && !(pred_out && is_direct(pred_out));
+    char *stage = staged ? (char *)stage_pool().take() : nullptr;
+    if (stage != nullptr) {       // small: everything packed into one page-locked block, one wait for the whole call
+      cudaError_t e = cudaSuccess;
+      if (logits_out) e = launch_pack(st, out, (size_t)last.ld_out * 4, row, (size_t)N, stage);
+      if (pred_out && e == cudaSuccess) e = launch_pack(st, d_pred, pr_bytes, pr_bytes, 1, stage + lg_bytes);
+      const cudaError_t w = cudaStreamSynchronize(st);
+      if (e == cudaSuccess) e = w;
+      if (e == cudaSuccess) {
+        if (logits_out) memcpy(logits_out, stage, lg_bytes);
+        if (pred_out) memcpy(pred_out, stage + lg_bytes, pr_bytes);
+      }
+      stage_pool().give(stage);
+      PD_CUDA(e);
+    } else {
+      if (logits_out) PD_TRY(copy_rows(c->device, st, logits_out, out, (size_t)last.ld_out * 4, row, (size_t)N, true));
+      if (pred_out) PD_TRY(copy_rows(c->device, st, pred_out, d_pred, pr_bytes, pr_bytes, 1, true));
+      PD_CUDA(cudaStreamSynchronize(st));
+    }
+    if (counts_out)
+      for (int i = 0; i < 4; ++i) counts_out[i] = (int64_t)h_counts[i];
+    if (h_counts[4]) {
+      PD_CUDA(cudaMemsetAsync(c->control, 0, c->control_words * sizeof(int), st));
+      return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+    }
+    return PDADMM_OK;
+  });
 }
 
 extern "C" int pdadmm_residuals(pdadmm_ctx *c, double *per_layer_sq, int n) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
-  if (n != c->L - 1 || (n > 0 && !per_layer_sq)) return fail(PDADMM_EINVAL, "n must be L-1 = %d", c->L - 1);
-  PD_CUDA(cudaSetDevice(c->device));
-  PD_TRY(ensure_residual(c));
-  if (n > 0) PD_TRY(read_objective(c, OBJ_RESIDUALS));
-  for (int l = 0; l + 1 < c->L; ++l) per_layer_sq[l] = c->h_results[4 * (size_t)l + 3];
-  if (c->reduce != nullptr && n > 0) {
-    if ((size_t)n > 8 + (size_t)c->layers[0].ld_out) return fail(PDADMM_EINVAL, "too many layers for the reduction buffer");
-    PD_CUDA(cudaMemcpyAsync(c->scr.red, per_layer_sq, (size_t)n * 8, cudaMemcpyHostToDevice, c->scr.st));
-    PD_TRY(shard_sum(c, c->scr.st, c->scr.red, (size_t)n, 1));
-    PD_CUDA(cudaMemcpyAsync(per_layer_sq, c->scr.red, (size_t)n * 8, cudaMemcpyDeviceToHost, c->scr.st));
-    PD_CUDA(cudaStreamSynchronize(c->scr.st));
-  }
-  return PDADMM_OK;
+  return guarded([&]() -> int {
+    if (!c) return fail(PDADMM_EINVAL, "context is null");
+    if (n != c->L - 1 || (n > 0 && !per_layer_sq)) return fail(PDADMM_EINVAL, "n must be L-1 = %d", c->L - 1);
+    PD_CUDA(cudaSetDevice(c->device));
+    PD_TRY(ensure_residual(c));
+    if (n > 0) PD_TRY(read_objective(c, OBJ_RESIDUALS));
+    for (int l = 0; l + 1 < c->L; ++l) per_layer_sq[l] = c->h_results[4 * (size_t)l + 3];
+    if (c->reduce != nullptr && n > 0) {
+      if ((size_t)n > 8 + (size_t)c->layers[0].ld_out) return fail(PDADMM_EINVAL, "too many layers for the reduction buffer");
+      PD_CUDA(cudaMemcpyAsync(c->scr.red, per_layer_sq, (size_t)n * 8, cudaMemcpyHostToDevice, c->scr.st));
+      PD_TRY(shard_sum(c, c->scr.st, c->scr.red, (size_t)n, 1));
+      PD_CUDA(cudaMemcpyAsync(per_layer_sq, c->scr.red, (size_t)n * 8, cudaMemcpyDeviceToHost, c->scr.st));
+      PD_CUDA(cudaStreamSynchronize(c->scr.st));
+    }
+    return PDADMM_OK;
+  });
 }
 
 // ---- tensors in and out -------------------------------------------------------------------------------------
@@ -1955,20 +1966,22 @@ static int locate(pdadmm_ctx *c, int kind, int layer, TensorRef *t) {
 }
 
 extern "C" int pdadmm_get_tensor(pdadmm_ctx *c, int kind, int layer, void *host_dst, size_t bytes) {
-  if (!c || !host_dst) return fail(PDADMM_EINVAL, "null argument");
-  PD_CUDA(cudaSetDevice(c->device));
-  if (kind == PDADMM_T_QSCALE) {
-    if (layer < 2 || layer > c->L || bytes != 4) return fail(PDADMM_EINVAL, "QSCALE: layer in [2, L], 4 bytes");
-    memcpy(host_dst, &c->layers[layer - 1].scale, 4);
-    return PDADMM_OK;
-  }
-  TensorRef t;
-  PD_TRY(locate(c, kind, layer, &t));
-  if (bytes != t.rows * t.width * t.elem)
-    return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
-                t.rows * t.width * t.elem, bytes);
-  if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
-  return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
+  return guarded([&]() -> int {
+    if (!c || !host_dst) return fail(PDADMM_EINVAL, "null argument");
+    PD_CUDA(cudaSetDevice(c->device));
+    if (kind == PDADMM_T_QSCALE) {
+      if (layer < 2 || layer > c->L || bytes != 4) return fail(PDADMM_EINVAL, "QSCALE: layer in [2, L], 4 bytes");
+      memcpy(host_dst, &c->layers[layer - 1].scale, 4);
+      return PDADMM_OK;
+    }
+    TensorRef t;
+    PD_TRY(locate(c, kind, layer, &t));
+    if (bytes != t.rows * t.width * t.elem)
+      return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
+                  t.rows * t.width * t.elem, bytes);
+    if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
+    return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
+  });
 }
 
 // pdADMM-G-Q: the kernels read p_l (l >= 2, paper numbering) as its codes, so the two must always agree: the codes
@@ -1987,35 +2000,37 @@ static int project_p_on_its_levels(pdadmm_ctx *c, int layer) {
 }
 
 extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void *host_src, size_t bytes) {
-  if (!c || !host_src) return fail(PDADMM_EINVAL, "null argument");
-  PD_CUDA(cudaSetDevice(c->device));
-  if (kind == PDADMM_T_QSCALE) {
-    if (layer < 2 || layer > c->L || bytes != 4) return fail(PDADMM_EINVAL, "QSCALE: layer in [2, L], 4 bytes");
-    float v;
-    memcpy(&v, host_src, 4);
-    if (!(v > 0.f)) return fail(PDADMM_EINVAL, "QSCALE must be positive");
-    PD_TRY(refresh_p(c));
-    c->layers[layer - 1].scale = v;
-    c->layers[layer - 1].lo = -(float)c->neg_levels * v;
-    if (c->levels) PD_TRY(project_p_on_its_levels(c, layer));       // p_l moves to the new level set
+  return guarded([&]() -> int {
+    if (!c || !host_src) return fail(PDADMM_EINVAL, "null argument");
+    PD_CUDA(cudaSetDevice(c->device));
+    if (kind == PDADMM_T_QSCALE) {
+      if (layer < 2 || layer > c->L || bytes != 4) return fail(PDADMM_EINVAL, "QSCALE: layer in [2, L], 4 bytes");
+      float v;
+      memcpy(&v, host_src, 4);
+      if (!(v > 0.f)) return fail(PDADMM_EINVAL, "QSCALE must be positive");
+      PD_TRY(refresh_p(c));
+      c->layers[layer - 1].scale = v;
+      c->layers[layer - 1].lo = -(float)c->neg_levels * v;
+      if (c->levels) PD_TRY(project_p_on_its_levels(c, layer));       // p_l moves to the new level set
+      return PDADMM_OK;
+    }
+    TensorRef t;
+    if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
+    PD_TRY(locate(c, kind, layer, &t));
+    if (!t.settable) return fail(PDADMM_EINVAL, "tensor kind %d is read-only", kind);
+    if (bytes != t.rows * t.width * t.elem)
+      return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
+                  t.rows * t.width * t.elem, bytes);
+    PD_TRY(copy_rows(c->device, c->scr.st, const_cast<void *>(host_src), t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, false));
+    if (kind == PDADMM_T_X || kind == PDADMM_T_P || kind == PDADMM_T_W || kind == PDADMM_T_B || kind == PDADMM_T_Z)
+      c->r_valid = false;
+    if (kind == PDADMM_T_W) c->w_planes_valid = false;
+    if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->amax_p_valid = false;
+    if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->x_planes_valid = false;
+    if (kind == PDADMM_T_P || kind == PDADMM_T_Q || kind == PDADMM_T_U) c->t_valid = false;
+    if (kind == PDADMM_T_P && c->levels && layer >= 2) PD_TRY(project_p_on_its_levels(c, layer));
     return PDADMM_OK;
-  }
-  TensorRef t;
-  if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
-  PD_TRY(locate(c, kind, layer, &t));
-  if (!t.settable) return fail(PDADMM_EINVAL, "tensor kind %d is read-only", kind);
-  if (bytes != t.rows * t.width * t.elem)
-    return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
-                t.rows * t.width * t.elem, bytes);
-  PD_TRY(copy_rows(c->device, c->scr.st, const_cast<void *>(host_src), t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, false));
-  if (kind == PDADMM_T_X || kind == PDADMM_T_P || kind == PDADMM_T_W || kind == PDADMM_T_B || kind == PDADMM_T_Z)
-    c->r_valid = false;
-  if (kind == PDADMM_T_W) c->w_planes_valid = false;
-  if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->amax_p_valid = false;
-  if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->x_planes_valid = false;
-  if (kind == PDADMM_T_P || kind == PDADMM_T_Q || kind == PDADMM_T_U) c->t_valid = false;
-  if (kind == PDADMM_T_P && c->levels && layer >= 2) PD_TRY(project_p_on_its_levels(c, layer));
-  return PDADMM_OK;
+  });
 }
 
 // ---- stand-alone entry points for single kernels ------------------------------------------------------------------
@@ -2086,89 +2101,91 @@ extern "C" int pdadmm_spmm(int device, int64_t n_rows, const int32_t *row_ptr, c
 
 extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const float *A, const float *B, float *C,
                              double *sumsq, uint32_t flags) {
-  if (mode < 0 || mode > 2 || M < 1 || N < 1 || K < 1 || !A || !B || !C || device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "bad argument");
-  PD_CUDA(cudaSetDevice(device));
-  pdadmm_ctx *c = new (std::nothrow) pdadmm_ctx();
-  if (!c) return fail(PDADMM_ENOMEM, "out of host memory");
-  c->device = device;
-  c->use_tc = (flags & PDADMM_FLAG_SIMT_GEMM) == 0;
-  auto body = [&]() -> int {
-    PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device));
-    PD_CUDA(device_pool(device).take_stream(&c->scr.own));
-    c->scr.st = c->scr.own;
-    cudaStream_t st = c->scr.st;
-    PD_TRY(dev_alloc(c, &c->d_flag, 4));
-    if (c->use_tc) {
-      PD_TRY(dev_alloc(c, &c->scr.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
-      PD_TRY(dev_alloc(c, &c->scr.tail_count, (size_t)c->n_sms * 8));
-    }
-    // operand shapes as stored: rows x cols
-    const int a_rows = mode == 2 ? K : M, a_cols = mode == 2 ? M : K;
-    const int b_rows = mode == 0 ? N : K, b_cols = mode == 0 ? K : N;
-    const int lda = round_up(a_cols, 8), ldb = round_up(b_cols, 8), ldc = round_up(N, 4);
-    float *dA, *dB, *dC, *part = nullptr;
-    double *slots;
-    Planes Ap, Bp;
-    PD_TRY(dev_alloc(c, &dA, (size_t)a_rows * lda));
-    PD_TRY(dev_alloc(c, &dB, (size_t)b_rows * ldb));
-    PD_TRY(dev_alloc(c, &dC, (size_t)M * ldc));
-    const int n_slots = 16 * (int)(ceil_div(M, 128) * ceil_div(N, 128)) + 2048;
-    PD_TRY(dev_alloc(c, &slots, (size_t)n_slots));
-    PD_TRY(upload_rows(c, st, dA, lda, A, a_cols, a_rows));
-    PD_TRY(upload_rows(c, st, dB, ldb, B, b_cols, b_rows));
-    Operand oA{dA, lda, nullptr}, oB{dB, ldb, nullptr};
-    if (c->use_tc) {        // planes of both operands as they are stored
-      PD_TRY(dev_alloc(c, &c->scr.amax_pool, (size_t)AMAX_POOL));
-      PD_TRY(alloc_planes(c, (size_t)a_rows * lda, &Ap));
-      PD_TRY(alloc_planes(c, (size_t)b_rows * ldb, &Bp));
-      PD_TRY(amax_reserve(c, st, 2));
-      split_rows(c, st, dA, (size_t)a_rows, a_cols, lda, amax_of(c, st, dA, (size_t)a_rows * lda / 4), Ap);
-      split_rows(c, st, dB, (size_t)b_rows, b_cols, ldb, amax_of(c, st, dB, (size_t)b_rows * ldb / 4), Bp);
-      oA = plane_operand(dA, lda, Ap);
-      oB = plane_operand(dB, ldb, Bp);
-    }
-    double *res = slots + n_slots - 1;
-    int *done;
-    PD_TRY(dev_alloc(c, &done, 1));
-    Step step;
-    step.kind = STEP_SUM; step.sum = res;
-    EpiStoreSumsq epi{dC, ldc};
-    if (mode == 0) {
-      PD_TRY((gemm_nodes<false, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
-    } else if (mode == 1) {
-      PD_TRY((gemm_nodes<true, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
-    } else {
-      const int split = (int)std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(K, 64)));
-      const int k_chunk = round_up((int)ceil_div(K, split), TC_BK);
-      const int n_split = (int)ceil_div(K, k_chunk);
-      PD_TRY(dev_alloc(c, &part, (size_t)n_split * M * ldc));
-      if (!c->use_tc) {
-        dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM), (unsigned)n_split);
-        gemm_tn_kernel<<<grid, SG_THREADS, 0, st>>>(M, N, K, k_chunk, dA, lda, dB, ldb, part, ldc);
-      } else {
-        Prod<EpiStore> p{M, N, K, oA, oB, EpiStore{part, ldc}, &c->scr};
-        p.n_split = n_split; p.k_chunk = k_chunk; p.stride = (size_t)M * ldc;
-        PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, {p}));
+  return guarded([&]() -> int {
+    if (mode < 0 || mode > 2 || M < 1 || N < 1 || K < 1 || !A || !B || !C || device >= MAX_DEVICES) return fail(PDADMM_EINVAL, "bad argument");
+    PD_CUDA(cudaSetDevice(device));
+    pdadmm_ctx *c = new (std::nothrow) pdadmm_ctx();
+    if (!c) return fail(PDADMM_ENOMEM, "out of host memory");
+    c->device = device;
+    c->use_tc = (flags & PDADMM_FLAG_SIMT_GEMM) == 0;
+    auto body = [&]() -> int {
+      PD_CUDA(cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device));
+      PD_CUDA(device_pool(device).take_stream(&c->scr.own));
+      c->scr.st = c->scr.own;
+      cudaStream_t st = c->scr.st;
+      PD_TRY(dev_alloc(c, &c->d_flag, 4));
+      if (c->use_tc) {
+        PD_TRY(dev_alloc(c, &c->scr.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+        PD_TRY(dev_alloc(c, &c->scr.tail_count, (size_t)c->n_sms * 8));
       }
-      const size_t n4 = (size_t)M * ldc / 4;
-      Group<GradWSum> g;
-      g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
-      reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
-    }
-    double h = 0;
-    PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
-    PD_TRY(copy_rows(device, st, C, dC, (size_t)ldc * 4, (size_t)N * 4, (size_t)M, true));
-    int err = 0;
-    PD_CUDA(cudaMemcpyAsync(&err, c->d_flag + 1, 4, cudaMemcpyDeviceToHost, st));
-    PD_CUDA(cudaStreamSynchronize(st));
-    PD_CUDA(cudaGetLastError());
-    if (sumsq) *sumsq = h;
-    if (err) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
-    return PDADMM_OK;
-  };
-  const int rc = body();
-  destroy(c);
-  return rc;
+      // operand shapes as stored: rows x cols
+      const int a_rows = mode == 2 ? K : M, a_cols = mode == 2 ? M : K;
+      const int b_rows = mode == 0 ? N : K, b_cols = mode == 0 ? K : N;
+      const int lda = round_up(a_cols, 8), ldb = round_up(b_cols, 8), ldc = round_up(N, 4);
+      float *dA, *dB, *dC, *part = nullptr;
+      double *slots;
+      Planes Ap, Bp;
+      PD_TRY(dev_alloc(c, &dA, (size_t)a_rows * lda));
+      PD_TRY(dev_alloc(c, &dB, (size_t)b_rows * ldb));
+      PD_TRY(dev_alloc(c, &dC, (size_t)M * ldc));
+      const int n_slots = 16 * (int)(ceil_div(M, 128) * ceil_div(N, 128)) + 2048;
+      PD_TRY(dev_alloc(c, &slots, (size_t)n_slots));
+      PD_TRY(upload_rows(c, st, dA, lda, A, a_cols, a_rows));
+      PD_TRY(upload_rows(c, st, dB, ldb, B, b_cols, b_rows));
+      Operand oA{dA, lda, nullptr}, oB{dB, ldb, nullptr};
+      if (c->use_tc) {        // planes of both operands as they are stored
+        PD_TRY(dev_alloc(c, &c->scr.amax_pool, (size_t)AMAX_POOL));
+        PD_TRY(alloc_planes(c, (size_t)a_rows * lda, &Ap));
+        PD_TRY(alloc_planes(c, (size_t)b_rows * ldb, &Bp));
+        PD_TRY(amax_reserve(c, st, 2));
+        split_rows(c, st, dA, (size_t)a_rows, a_cols, lda, amax_of(c, st, dA, (size_t)a_rows * lda / 4), Ap);
+        split_rows(c, st, dB, (size_t)b_rows, b_cols, ldb, amax_of(c, st, dB, (size_t)b_rows * ldb / 4), Bp);
+        oA = plane_operand(dA, lda, Ap);
+        oB = plane_operand(dB, ldb, Bp);
+      }
+      double *res = slots + n_slots - 1;
+      int *done;
+      PD_TRY(dev_alloc(c, &done, 1));
+      Step step;
+      step.kind = STEP_SUM; step.sum = res;
+      EpiStoreSumsq epi{dC, ldc};
+      if (mode == 0) {
+        PD_TRY((gemm_nodes<false, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
+      } else if (mode == 1) {
+        PD_TRY((gemm_nodes<true, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
+      } else {
+        const int split = (int)std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(K, 64)));
+        const int k_chunk = round_up((int)ceil_div(K, split), TC_BK);
+        const int n_split = (int)ceil_div(K, k_chunk);
+        PD_TRY(dev_alloc(c, &part, (size_t)n_split * M * ldc));
+        if (!c->use_tc) {
+          dim3 grid((unsigned)ceil_div(N, SG_BN), (unsigned)ceil_div(M, SG_BM), (unsigned)n_split);
+          gemm_tn_kernel<<<grid, SG_THREADS, 0, st>>>(M, N, K, k_chunk, dA, lda, dB, ldb, part, ldc);
+        } else {
+          Prod<EpiStore> p{M, N, K, oA, oB, EpiStore{part, ldc}, &c->scr};
+          p.n_split = n_split; p.k_chunk = k_chunk; p.stride = (size_t)M * ldc;
+          PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, {p}));
+        }
+        const size_t n4 = (size_t)M * ldc / 4;
+        Group<GradWSum> g;
+        g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
+        reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
+      }
+      double h = 0;
+      PD_CUDA(cudaMemcpyAsync(&h, res, 8, cudaMemcpyDeviceToHost, st));
+      PD_TRY(copy_rows(device, st, C, dC, (size_t)ldc * 4, (size_t)N * 4, (size_t)M, true));
+      int err = 0;
+      PD_CUDA(cudaMemcpyAsync(&err, c->d_flag + 1, 4, cudaMemcpyDeviceToHost, st));
+      PD_CUDA(cudaStreamSynchronize(st));
+      PD_CUDA(cudaGetLastError());
+      if (sumsq) *sumsq = h;
+      if (err) return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
+      return PDADMM_OK;
+    };
+    const int rc = body();
+    destroy(c);
+    return rc;
+  });
 }
 
 // ---- self-test of the bounded waits ------------------------------------------------------------------------------
@@ -2219,37 +2236,43 @@ extern "C" int pdadmm_selftest_bounded_wait(int device, long long limit_cycles, 
 // The words of a context as blocks that gave up in the middle of their products leave them (the error word set, counters between
 // one arrival and the last, largest magnitudes of no number), then what pdadmm_step does after its last iteration.
 extern "C" int pdadmm_selftest_expired_wait(pdadmm_ctx *c) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
-  PD_CUDA(cudaSetDevice(c->device));
-  std::vector<int> words(c->control_words, 1);
-  words[0] = words[2] = 0;
-  for (int l = 0; l < c->L; ++l)
-    for (int i = 4; i < 8; ++i) words[4 + 8 * (size_t)l + i] = 0x7fc00000;
-  PD_CUDA(cudaEventRecord(c->ev_begin, c->scr.st));
-  PD_CUDA(cudaMemcpyAsync(c->control, words.data(), words.size() * sizeof(int), cudaMemcpyHostToDevice, c->scr.st));
-  PD_CUDA(cudaStreamSynchronize(c->scr.st));
-  return finish_steps(c, false);
+  return guarded([&]() -> int {
+    if (!c) return fail(PDADMM_EINVAL, "context is null");
+    PD_CUDA(cudaSetDevice(c->device));
+    std::vector<int> words(c->control_words, 1);
+    words[0] = words[2] = 0;
+    for (int l = 0; l < c->L; ++l)
+      for (int i = 4; i < 8; ++i) words[4 + 8 * (size_t)l + i] = 0x7fc00000;
+    PD_CUDA(cudaEventRecord(c->ev_begin, c->scr.st));
+    PD_CUDA(cudaMemcpyAsync(c->control, words.data(), words.size() * sizeof(int), cudaMemcpyHostToDevice, c->scr.st));
+    PD_CUDA(cudaStreamSynchronize(c->scr.st));
+    return finish_steps(c, false);
+  });
 }
 
 // ---- timing ----------------------------------------------------------------------------------------------------
 extern "C" int pdadmm_profile(pdadmm_ctx *c, int enable) {
-  if (!c) return fail(PDADMM_EINVAL, "context is null");
-  PD_CUDA(cudaSetDevice(c->device));
-  PD_TRY(prof_collect(c));
-  for (int k = 0; k < KC_COUNT; ++k) { c->prof_ms[k] = 0; c->prof_n[k] = 0; c->prof_bytes[k] = 0; c->prof_flops[k] = 0; }
-  c->profiling = enable != 0;
-  return PDADMM_OK;
+  return guarded([&]() -> int {
+    if (!c) return fail(PDADMM_EINVAL, "context is null");
+    PD_CUDA(cudaSetDevice(c->device));
+    PD_TRY(prof_collect(c));
+    for (int k = 0; k < KC_COUNT; ++k) { c->prof_ms[k] = 0; c->prof_n[k] = 0; c->prof_bytes[k] = 0; c->prof_flops[k] = 0; }
+    c->profiling = enable != 0;
+    return PDADMM_OK;
+  });
 }
 extern "C" int pdadmm_profile_classes(void) { return KC_COUNT; }
 extern "C" const char *pdadmm_profile_name(int k) { return (k >= 0 && k < KC_COUNT) ? kclass_names[k] : ""; }
 extern "C" int pdadmm_profile_read(pdadmm_ctx *c, int k, double *ms, int64_t *launches, double *bytes, double *flops) {
-  if (!c || k < 0 || k >= KC_COUNT) return fail(PDADMM_EINVAL, "bad argument");
-  PD_TRY(prof_collect(c));
-  if (ms) *ms = c->prof_ms[k];
-  if (launches) *launches = c->prof_n[k];
-  if (bytes) *bytes = c->prof_bytes[k];
-  if (flops) *flops = c->prof_flops[k];
-  return PDADMM_OK;
+  return guarded([&]() -> int {
+    if (!c || k < 0 || k >= KC_COUNT) return fail(PDADMM_EINVAL, "bad argument");
+    PD_TRY(prof_collect(c));
+    if (ms) *ms = c->prof_ms[k];
+    if (launches) *launches = c->prof_n[k];
+    if (bytes) *bytes = c->prof_bytes[k];
+    if (flops) *flops = c->prof_flops[k];
+    return PDADMM_OK;
+  });
 }
 extern "C" int pdadmm_time_augmentation(pdadmm_ctx *c, int reps, double *ms_per_hop, double *bytes_per_hop) {
   if (!c || reps < 1 || reps > 1000 || !ms_per_hop) return fail(PDADMM_EINVAL, "bad argument");

@@ -18,6 +18,7 @@
 
 #include <chrono>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "common.cuh"
@@ -27,7 +28,13 @@ namespace pd {
 struct DeviceBlock { void *p; size_t bytes; };
 
 class DevicePool {
+  static constexpr size_t MAX_STREAMS = 64, MAX_EVENTS = 256;
  public:
+  DevicePool() {                           // giving a stream or an event back never allocates
+    streams_.reserve(MAX_STREAMS);
+    events_[0].reserve(MAX_EVENTS);
+    events_[1].reserve(MAX_EVENTS);
+  }
   // A block of at least `bytes` bytes, at most a quarter more; contents are undefined.  The device must be current.
   cudaError_t take(size_t bytes, DeviceBlock *out) {
     {
@@ -57,8 +64,10 @@ class DevicePool {
   void give(const std::vector<DeviceBlock> &blocks) {
     if (blocks.empty()) return;
     std::vector<DeviceBlock> out;
-    {
+    try {
       std::lock_guard<std::mutex> g(m_);
+      free_.reserve(free_.size() + blocks.size());
+      out.reserve(free_.size() + blocks.size());
       const auto now = std::chrono::steady_clock::now();
       if (asked_ == std::chrono::steady_clock::time_point{} || now - asked_ > std::chrono::milliseconds(500)) {
         size_t free_bytes = 0, total = 0;
@@ -78,6 +87,9 @@ class DevicePool {
         held_ -= free_.front().bytes;
         free_.erase(free_.begin());
       }
+    } catch (const std::bad_alloc &) {       // no room to remember them
+      for (const DeviceBlock &b : blocks) cudaFree(b.p);
+      return;
     }
     for (const DeviceBlock &b : out) cudaFree(b.p);
   }
@@ -101,7 +113,7 @@ class DevicePool {
     if (s == nullptr) return;
     {
       std::lock_guard<std::mutex> g(m_);
-      if (streams_.size() < 64) { streams_.push_back(s); return; }
+      if (streams_.size() < MAX_STREAMS) { streams_.push_back(s); return; }
     }
     cudaStreamDestroy(s);
   }
@@ -117,7 +129,7 @@ class DevicePool {
     if (ev == nullptr) return;
     {
       std::lock_guard<std::mutex> g(m_);
-      if (events_[timing].size() < 256) { events_[timing].push_back(ev); return; }
+      if (events_[timing].size() < MAX_EVENTS) { events_[timing].push_back(ev); return; }
     }
     cudaEventDestroy(ev);
   }

@@ -6,6 +6,8 @@
 
 #include <sys/mman.h>
 
+#include <stdexcept>
+
 using namespace pd;
 static int check(bool ok, const char *what) { printf("%s: %s\n", what, ok ? "yes" : "NO"); return ok ? 0 : 1; }
 
@@ -33,6 +35,26 @@ int main(int argc, char **argv) {
       for (const size_t n : {size_t(1), size_t(100), rows})
         bad += check(copy_rows(0, nullptr, on_device, dev.data(), pitch, width, n, out) == PDADMM_OK, "copied");
     return bad + check(direct_copies >= 6 && launches == 0, "by the driver");
+  }
+  if (what == "no host memory") {
+    int bad = 0;
+    for (int n = 0; n < 40; ++n) {                                   // the n-th allocation and all that follow fail
+      allocations_left = n;
+      const int rc = guarded([&]() -> int { return copy_rows(0, nullptr, host.data(), dev.data(), pitch, width, rows, n % 2 == 0); });
+      allocations_left = -1;
+      bad += rc != PDADMM_OK && rc != PDADMM_ENOMEM;
+      DevicePool pool;
+      std::vector<DeviceBlock> blocks;
+      DeviceBlock b;
+      for (int i = 0; i < 3; ++i) if (pool.take(100, &b) == cudaSuccess) blocks.push_back(b);
+      allocations_left = n % 5;
+      pool.give(blocks);
+      allocations_left = -1;
+      pool.trim();
+    }
+    stage_pool().trim();
+    return check(bad == 0, "an answer or PDADMM_ENOMEM") + check(live_stages == 0, "nothing is lost") +
+           check(guarded([]() -> int { throw std::length_error("x"); }) == PDADMM_ECUDA, "another exception is an error too");
   }
   return 2;
 }

@@ -20,7 +20,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["copies", "launch fails in workers", "launch fails", "device pointer"])
+@pytest.mark.parametrize("scenario", ["copies", "launch fails in workers", "launch fails", "device pointer", "no host memory"])
 def test_host_path(program, scenario):
     p = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stdout + p.stderr
