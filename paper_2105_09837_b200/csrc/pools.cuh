@@ -63,18 +63,12 @@ class DevicePool {
   // No device work may use the blocks any more.
   void give(const std::vector<DeviceBlock> &blocks) {
     if (blocks.empty()) return;
+    ask();
     std::vector<DeviceBlock> out;
     try {
       std::lock_guard<std::mutex> g(m_);
       free_.reserve(free_.size() + blocks.size());
       out.reserve(free_.size() + blocks.size());
-      const auto now = std::chrono::steady_clock::now();
-      if (asked_ == std::chrono::steady_clock::time_point{} || now - asked_ > std::chrono::milliseconds(500)) {
-        size_t free_bytes = 0, total = 0;
-        roomy_ = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= total / 2;
-        total_ = total;
-        asked_ = now;
-      }
       const bool keep = roomy_;
       const size_t total = total_;
       for (const DeviceBlock &b : blocks) {
@@ -135,6 +129,21 @@ class DevicePool {
   }
 
  private:
+  // Whether half of the device is free, asked without the lock: the answer can take milliseconds, and other threads come here
+  // for memory meanwhile.  They go by the answer before (nothing is kept before the first).
+  void ask() {
+    {
+      std::lock_guard<std::mutex> g(m_);
+      const auto now = std::chrono::steady_clock::now();
+      if (asked_ != std::chrono::steady_clock::time_point{} && now - asked_ <= std::chrono::milliseconds(500)) return;
+      asked_ = now;
+    }
+    size_t free_bytes = 0, total = 0;
+    const bool roomy = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= total / 2;
+    std::lock_guard<std::mutex> g(m_);
+    roomy_ = roomy;
+    total_ = total;
+  }
   std::mutex m_;
   std::vector<DeviceBlock> free_;          // oldest first
   size_t held_ = 0, total_ = 0;

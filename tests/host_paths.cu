@@ -6,6 +6,8 @@
 
 #include <sys/mman.h>
 
+#include <atomic>
+#include <chrono>
 #include <stdexcept>
 
 using namespace pd;
@@ -55,6 +57,26 @@ int main(int argc, char **argv) {
     stage_pool().trim();
     return check(bad == 0, "an answer or PDADMM_ENOMEM") + check(live_stages == 0, "nothing is lost") +
            check(guarded([]() -> int { throw std::length_error("x"); }) == PDADMM_ECUDA, "another exception is an error too");
+  }
+  if (what == "asking for free memory") {
+    static DevicePool pool;
+    static std::atomic<bool> took{false}, asked{false};
+    DeviceBlock b;
+    if (pool.take(1000, &b) != cudaSuccess) return 1;
+    while_asking = [] {                                              // waits (two seconds at most) for the other thread's take
+      asked = true;
+      for (int i = 0; i < 2000 && !took; ++i) std::this_thread::sleep_for(std::chrono::milliseconds(1));
+    };
+    std::thread other([] {
+      while (!asked) std::this_thread::yield();
+      DeviceBlock d;
+      if (pool.take(5000, &d) == cudaSuccess) took = true;
+    });
+    const auto t0 = std::chrono::steady_clock::now();
+    pool.give({b});
+    const bool waited = std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(1500);
+    other.join();
+    return check(!waited, "another thread's take does not wait for the question");
   }
   return 2;
 }

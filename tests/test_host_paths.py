@@ -20,7 +20,8 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["copies", "launch fails in workers", "launch fails", "device pointer", "no host memory"])
+@pytest.mark.parametrize("scenario", ["copies", "launch fails in workers", "launch fails", "device pointer", "no host memory",
+                                      "asking for free memory"])
 def test_host_path(program, scenario):
     p = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stdout + p.stderr
