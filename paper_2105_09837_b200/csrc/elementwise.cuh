@@ -364,11 +364,15 @@ check_planes_kernel(const __grid_constant__ Group<PlaneCheck> group) {
 }
 
 // ---- reduction of the split partial tiles of grad_W, scaling by nu, ||grad_W||^2 ------------------
+// `remake`: if the predicted scaling of the planes turned out unusable (the first iterations of a context), the layer's last
+// block makes them again with the exponent of *amax.  It costs one block 30 us for 500 x 500 and 130 us for 1000 x 1000, nothing
+// otherwise; left to the product G p+, every output tile splits G again: 0.85 ms more per layer at 60 000 x 1000, 0.1 ms at
+// 20 000 x 500 (remade_with_sum says when).  Larger matrices have check_planes_kernel.
 struct GradWSum {
   const float *part; int n_split; uint32_t n4;
   float *G;
   uint32_t *amax /* max|G|, may be null */; PlaneOut planes;
-  double *slots; int *done; double *sum /* ||G||^2 */; int n_blocks;
+  double *slots; int *done; double *sum /* ||G||^2 */; int n_blocks, remake;
 };
 __global__ void __launch_bounds__(EW_THREADS)
 reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
@@ -398,10 +402,17 @@ reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
   const double tot = block_sum<EW_THREADS>(ss, red);
   if (threadIdx.x == 0) y.slots[blockIdx.x] = tot;
   if (!last_block(y.done, y.n_blocks, &is_last)) return;
+  const uint32_t top = y.remake ? __ldcg(y.amax) : 0u;           // (on its way while the slots are added)
+  const bool usable = !y.remake || tc_planes_usable(top, *y.planes.exp);
   double v = 0.0;
   for (int i = threadIdx.x; i < y.n_blocks; i += EW_THREADS) v += __ldcg(y.slots + i);
   v = block_sum<EW_THREADS>(v, red);
   if (threadIdx.x == 0) *y.sum = v;
+  if (usable) return;
+  const float again = tc_pow2(tc_scale_exp(top));
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < y.n4; i += EW_THREADS)
+    store_planes4(y.planes, i, __ldcg(reinterpret_cast<const float4 *>(y.G) + i), again);
 }
 
 // ---- what follows theta: W+ and r - (G p+)/theta with its column sums (for the b-update) ----------------------------------

@@ -70,6 +70,7 @@ struct Operand {
   const int *exp = nullptr;
   const uint32_t *check = nullptr;
   float int_mul = 0.f;
+  int uses = 1;                     // output tiles that read an element of it (and would each split it again)
 };
 static Operand int_operand(const __half *plane, int ld, float mul) {
   Operand o{nullptr, ld, nullptr};
@@ -224,6 +225,11 @@ struct pdadmm_ctx {
   cudaGraphExec_t iter_graph = nullptr;   // one captured pdADMM-G iteration (no host round trips in it)
   int64_t iter_graph_launches = 0;
   bool graph_failed = false;
+  // Iterations left in which scalings are still found (see check_planes): two per layer from the start, or from a tensor that was
+  // set; what the first ones change travels one layer further with every second iteration.  They run eagerly if they have
+  // work for check_planes that a replay of a later iteration would leave out (`wide`).
+  int cold = 0;
+  bool wide = false;
   int n_sms = 148;
   bool w_planes_valid = false;
   bool amax_p_valid = false;        // every layer's amax_p covers the stored p
@@ -493,16 +499,19 @@ static void split_rows(pdadmm_ctx *c, cudaStream_t st, const float *x, size_t ro
   Launch l(c, KC_PLANES, st, (lo_too ? 8.0 : 6.0) * rows * cols, 0);
   rows_planes_kernel<<<dim3(ew_grid(n8)), 256, 0, st>>>(x, n8, amax, pl.exp, pl.hi, lo_too ? pl.lo : nullptr);
 }
-// Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel).
-// From 2^20 elements on: below, the launch costs more than it saves.
-constexpr size_t CHECK_PLANES_FROM = size_t(1) << 20;
+// Refused planes of a large matrix are made again by a kernel of their own instead of by the product (check_planes_kernel): always
+// from 2^20 elements on; below, a launch that finds nothing to do costs more than it saves (2000 x 500, 6 layers: 237 us per
+// iteration with it, 229 without), except in a context's first iterations, where maxima that were zero become something and
+// no prediction holds, if many tiles of the product read each element and would split it again (CHECK_PLANES_USES reads;
+// 500 x 2000, 4 layers: 0.86 ms for such an iteration, 0.37 so).
+constexpr size_t CHECK_PLANES_FROM = size_t(1) << 20, CHECK_PLANES_USES = size_t(1) << 21;
 static void check_planes(pdadmm_ctx *c, cudaStream_t st, size_t rows, const std::vector<Operand *> &ops) {
   Group<PlaneCheck> g;
   int n = 0;
   uint32_t n8_max = 0;
   for (Operand *o : ops) {
     const size_t e = rows * o->ld;
-    if (!c->use_tc || o->hi == nullptr || o->check == nullptr || o->x == nullptr || e < CHECK_PLANES_FROM) continue;
+    if (!c->use_tc || o->hi == nullptr || o->check == nullptr || o->x == nullptr || (e < CHECK_PLANES_FROM && !(c->cold > 0 && e * o->uses >= CHECK_PLANES_USES))) continue;
     g.l[n++] = PlaneCheck{o->x, (uint32_t)(e / 8), o->check, o->exp, const_cast<__half *>(o->hi),
                           o->lo == o->hi ? nullptr : const_cast<__half *>(o->lo)};
     n8_max = std::max(n8_max, (uint32_t)(e / 8));
@@ -676,6 +685,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
     Layer &ly = c->layers[l];
     Scratch &s = scratch_of(c, l);
     R.push_back(operand_r(ly));
+    R.back().uses = (int)ceil_div(ly.n_in, TC_BN);
     // The epilogue that writes g writes its planes too (the hi plane alone for the norm-only product), scaled by an exponent
     // predicted from the previous iteration's max|g|: the true one is known only when the product has finished.
     EpiGradT epi{s.s1, ly.ld_in, ly.t, c->nu, c->use_tc ? ly.w_g : nullptr};
@@ -690,6 +700,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
     grad.push_back(p);
     bytes += (c->use_tc ? (norm_only ? 6.0 : 8.0) : 4.0) * N * ly.n_in;
   }
+  for (size_t i = 0; i < batch.size(); ++i) G[i].uses = (int)ceil_div(c->layers[batch[i]].n_out, TC_BN);
   auto check = [&](std::vector<Operand> &ops) {
     std::vector<Operand *> v;
     for (Operand &o : ops) v.push_back(&o);
@@ -819,6 +830,15 @@ static int q_finish(pdadmm_ctx *c, cudaStream_t st, const Batch &batch, bool *hi
   return PDADMM_OK;
 }
 
+// Refused planes of grad_W are made again by the kernel that sums its slices where that is the quicker way: one block takes
+// 0.12 us per 1000 elements, the product G p+ about 2.5 us per round of its tiles and K block; at least twice the time, and more than one round (the test costs
+// the kernel's end half a microsecond, which 2000 x 100 does not get back).
+static bool remade_with_sum(const pdadmm_ctx *c, const Layer &ly) {
+  const size_t e = (size_t)ly.n_out * ly.ld_in;
+  const int64_t rounds = ceil_div(ceil_div(c->N, TC_BM) * ceil_div(ly.n_out, TC_BN), c->n_sms);
+  return c->use_tc && c->reduce == nullptr && e < CHECK_PLANES_FROM && rounds > 1 && (size_t)(rounds * ceil_div(ly.n_in, TC_BK)) * 10000 >= e;
+}
+
 // G = nu r^T p+ (contraction over nodes), theta, W <- W - G/theta, r <- r - (G p+)/theta,
 // b <- b - mean_j r, shift = mean_j r.
 static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
@@ -836,6 +856,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     P.push_back(l == 0 ? operand_X(ly) : c->int_operands ? int_operand(ly.p_plane, ly.ld_in, ly.scale)
                                                           : plane_operand(ly.p, ly.ld_in, s.pl1, ly.amax_p));
     R.push_back(l == 0 ? operand_r(ly) : plane_operand(ly.r, ly.ld_out, s.pl0, ly.amax_r));
+    R.back().uses = (int)ceil_div(ly.n_in, TC_BN);
   }
   if (!c->use_tc) {
     for (int l : batch) {
@@ -884,7 +905,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       // the planes of G are scaled by a prediction, which the product G p+ checks; the parts of a sharded sum come first
       g.l[n++] = GradWSum{s.part, ly.n_split, (uint32_t)n4, ly.gradW, c->use_tc ? ly.w_G : nullptr,
                           c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp), s.slots, ly.done + 1,
-                          &ly.sc->sum_G2, nb};
+                          &ly.sc->sum_G2, nb, remade_with_sum(c, ly)};
       blocks = std::max(blocks, nb);
       bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
     }
@@ -909,10 +930,11 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   for (int l : batch) {
     Layer &ly = c->layers[l];
     G.push_back(c->use_tc ? plane_operand(ly.gradW, ly.ld_in, ly.Gp, ly.w_G) : Operand{ly.gradW, ly.ld_in, nullptr});
+    if (remade_with_sum(c, ly)) G.back().x = nullptr;
   }
   for (size_t i = 0; i < batch.size(); ++i) {
     const Layer &ly = c->layers[batch[i]];
-    if ((size_t)ly.n_out * ly.ld_in < CHECK_PLANES_FROM) continue;
+    if (G[i].x == nullptr || (size_t)ly.n_out * ly.ld_in < CHECK_PLANES_FROM) continue;
     check_planes(c, st, (size_t)ly.n_out, {&G[i]});
   }
   {
@@ -1539,6 +1561,12 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->w_planes_valid = true;
   c->amax_p_valid = true;
   c->x_planes_valid = true;
+  c->cold = 2 * c->L;
+  for (const Layer &ly : c->layers)
+    for (int i = 0; i < 2; ++i) {            // r_l and g_l: of an element, the column tiles of the product that reads it
+      const size_t e = (size_t)N * (i ? ly.ld_in : ly.ld_out), uses = (size_t)ceil_div(i ? ly.n_out : ly.n_in, TC_BN);
+      c->wide |= c->use_tc && e < CHECK_PLANES_FROM && e * uses >= CHECK_PLANES_USES;
+    }
   c->launches = 0;
   c->comm_bytes = 0;
   return PDADMM_OK;
@@ -1700,6 +1728,7 @@ static int ensure_residual(pdadmm_ctx *c) {
     c->t_valid = true;
   }
   if (c->r_valid) return PDADMM_OK;
+  c->cold = 2 * c->L;
   for (int l = 0; l < c->L; ++l) PD_TRY(refresh_residual(c, c->layers[l], c->scr.st));
   c->r_valid = true;
   return PDADMM_OK;
@@ -1724,7 +1753,11 @@ static int run_steps(pdadmm_ctx *c, int n_iters) {
   const bool may_graph = c->levels == 0 && !c->profiling && !c->graph_failed && !(c->flags & PDADMM_FLAG_NO_GRAPH) &&
                          c->reduce == nullptr;
   int k = 0;
-  if (may_graph && c->iter_graph == nullptr && n_iters > 1) {
+  for (; c->wide && c->cold > 0 && k < n_iters; ++k) {
+    PD_TRY(iterate_once(c, &hit_cap));
+    --c->cold;
+  }
+  if (may_graph && c->iter_graph == nullptr && n_iters - k > 1) {
     PD_TRY(iterate_once(c, &hit_cap));
     ++k;
     const int64_t before = c->launches;
@@ -2171,7 +2204,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
         }
         const size_t n4 = (size_t)M * ldc / 4;
         Group<GradWSum> g;
-        g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4)};
+        g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4), 0};
         reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
       }
       double h = 0;
