@@ -319,6 +319,42 @@ def run_workload(name, steps, warmup, flags, device, world, dist, simt, with_cpu
     return rec
 
 
+# --------------------------------------------------------------------------------------- the printed line
+
+def rounded(x, digits=6):
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}")
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    return [rounded(v, digits) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def summary_line(rec, workloads, world, warmup, scaling, config, wall_s):
+    """The headline workload in full except for its kernel classes, of which the time stays; of every workload its own headline."""
+    def without_notes(d):
+        return {k: v for k, v in d.items() if k != "note"} if d else d
+
+    def brief(r):
+        if "error" in r:
+            return {"error": r["error"][:200]}
+        out = {k: r[k] for k in ("value", "steps", "ms_per_step", "gpu_launches", "frac_t_roof")}
+        out["clocks"] = {k: r["clocks"].get(k) for k in ("sm_mhz", "reasons")} if r.get("clocks") else None
+        out["roofline"] = {k: r["roofline"][k] for k in ("kernel", "bound", "frac")}
+        if r.get("e2e"):
+            out["e2e"] = r["e2e"]["value"]
+        if r.get("cpu_baseline"):
+            out["cpu_baseline"] = r["cpu_baseline"]["value"]
+        return out
+    return rounded({
+        "metric": METRIC, "value": rec["value"], "unit": UNIT, "n_gpus": world, "steps": rec["steps"], "warmup": warmup,
+        "ms_per_step": rec["ms_per_step"], "higher_is_better": True, "scaling": scaling, "vs_baseline": None, "dtype": "f32",
+        "data": "synthetic", "config": config, "clocks": rec["clocks"], "e2e": without_notes(rec.get("e2e")),
+        "gpu_launches": rec["gpu_launches"], "roofline": without_notes(rec["roofline"]), "cpu_baseline": rec.get("cpu_baseline"),
+        "t_roof_ms": rec["t_roof_ms"], "frac_t_roof": rec["frac_t_roof"],
+        "kernels_ms_per_iter": {k: v["ms_per_iter"] for k, v in rec["kernels"].items()}, "objective": rec["objective"],
+        "workloads": {k: brief(v) for k, v in sorted(workloads.items())}, "wall_s": wall_s})
+
+
 # --------------------------------------------------------------------------------------- main
 
 ALL = ["c1", "c2", "c3", "c4", "c5"]
@@ -408,15 +444,10 @@ def main():
                 workloads[name] = {"error": f"{type(e).__name__}: {e}"}
 
     if rank == 0:
-        line = {"metric": METRIC, "value": rec["value"], "unit": UNIT, "n_gpus": world, "steps": rec["steps"],
-                "warmup": args.warmup, "ms_per_step": rec["ms_per_step"], "higher_is_better": True,
-                "scaling": "strong" if sharded_run else "weak",
-                "vs_baseline": None, "dtype": "f32", "data": "synthetic", "config": config,
-                "clocks": rec["clocks"], "e2e": rec.get("e2e"), "gpu_launches": rec["gpu_launches"], "roofline": rec["roofline"],
-                "cpu_baseline": rec.get("cpu_baseline"), "t_roof_ms": rec["t_roof_ms"], "frac_t_roof": rec["frac_t_roof"],
-                "kernels": rec["kernels"], "objective": rec["objective"],
-                "workloads": {k: v for k, v in sorted(workloads.items())},
-                "wall_s": time.perf_counter() - t_start}
+        # the whole records (every kernel class of every workload) go to stderr, a line that a reader of the last few thousand
+        # characters still gets whole to stdout
+        print(json.dumps({"workloads": dict(sorted(workloads.items()))}), file=sys.stderr)
+        line = summary_line(rec, workloads, world, args.warmup, "strong" if sharded_run else "weak", config, time.perf_counter() - t_start)
         print(json.dumps(line))
     if dist is not None:
         dist.destroy_process_group()
