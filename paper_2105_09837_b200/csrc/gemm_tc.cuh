@@ -30,6 +30,14 @@
 // three times 2 MFLOP.  So two neighbouring SMs work as a pair on 256 x 128 outputs (tcgen05 cta_group::2): each loads the
 // planes of its own 128 rows of A and of half of the 128 columns of B, 48 KB, and the tensor cores read the other half
 // from the neighbour's shared memory.  No copy is multicast.  Products with few rows run one block per tile.
+// Wide tiles (256 x 256 per pair, choose_wide says when) bring 64 KB per K block for twice the work, two thirds of the traffic:
+// the W-gradient of 20 000 x 500 (9 layers) 410 -> 330 us, of 90 000 x 2000 (8 layers) 9.3 -> 7.6 ms, 1370 TFLOP/s of MMAs at
+// 1.4 GHz under the power limit.  Two accumulators of 256 columns fill tensor memory, so the correction terms share the main
+// term's: they come first, and the first MMA of the main term scales their sum by 2^-11 (relative error 1.5e-7 to 2.2e-7 either
+// way, a hundredth less with the shared one).  A tile's 128 KB of sums per block leave neither registers nor shared memory for
+// epilogue warps: the accumulate warps store it themselves, in bulk copies (with ordinary stores the end of a tile took
+// 10 000 cycles instead of 6500), so the form is built for products that store their sums as they are.  Tried: a finished tile parked
+// in tensor memory and stored between the K blocks of the next one (x W^T of 20 000 x 500, 9 layers: 560 us against 325).
 // Every wait is bounded; a wait that expires raises an error word in global memory and the CTA drains and exits.
 #pragma once
 
@@ -72,8 +80,14 @@ constexpr int TC_ACC_BUFS = 3;                                 // main-term accu
 constexpr int TC_TMEM_COLS = 512;                              // 3 main tiles, 1 correction tile
 constexpr uint32_t TC_COL_CORR = TC_ACC_BUFS * TC_BN;          // first column of the correction tile
 constexpr int TC_TILE_BYTES = 8 * 32 * 64 * 4;                 // finished tile: 8 warps x 32 rows x 64 columns
+// Wide tiles (pairs of SMs, 256 x 256): sixteen accumulate warps, 64 accumulators per thread, that store their piece themselves, in
+// parts of 32 rows x 16 columns through 2 KB of shared memory each; two accumulators of 256 columns in tensor memory.
+constexpr int TC_WIDE = 256, TC_WIDE_WARPS = 16, TC_WIDE_PART = 16;
+constexpr int TC_WIDE_PART_BYTES = 32 * TC_WIDE_PART * 4;
+constexpr int TC_WIDE_REGS_CTRL = 64, TC_WIDE_REGS_ACC = 104;
+static_assert(128 * (TC_WIDE_REGS_CTRL + 4 * TC_WIDE_REGS_ACC) <= TC_THREADS * TC_REGS_LAUNCH, "register shares of the wide form");
 constexpr int TC_SMEM_BYTES = TC_SPACE + 1024 /* alignment slack */ + 512 /* barriers */;
-static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 12 <= 512, "barriers");
+static_assert(8 * (3 * TC_MAX_STAGES + 2 * TC_ACC_BUFS + 3 + 2 * TC_ACC_WARPS) + 24 <= 512, "barriers");
 // How many parts a finished tile is handed over in (none if nothing is stored).  In one part it takes 64 KB; in two, one after
 // the other through 32 KB, it leaves room for one more stage if a stage holds four planes.  Two parts for the contraction
 // over the nodes, which is long and stores little: 100 000 x 500 x 500, 8 layers: 395 us against 444.  For the other products, whose
@@ -112,9 +126,17 @@ struct TcOperand {
 // One launch works on the same product of several layers, whose output tiles form one sequence of work units: a small
 // problem's layers fill the GPU together, and a large one has one partly filled last round instead of one per layer.
 constexpr int TC_MAX_GROUP = 16;
+// Division by a number known on the host: the quotient is the high word of n * inv, inv = ceil(2^32 / d), where that is exact for every
+// n that occurs (n d < 2^32; inv = 0 otherwise).  (Three divisions per tile and role took 650 cycles.)
+struct TcDiv {
+  int d; uint32_t inv;
+  static TcDiv of(int d, int64_t n_max) { return TcDiv{d, n_max * d < (int64_t(1) << 32) && d > 1 ? (uint32_t)(((int64_t(1) << 32) + d - 1) / d) : 0u}; }
+  __device__ __forceinline__ int operator()(int n) const { return d == 1 ? n : inv != 0u ? (int)__umulhi((uint32_t)n, inv) : n / d; }
+};
 template <class Epi>
 struct TcLayer {
   CUtensorMap a, alo, b, blo;      // planes of the operands
+  CUtensorMap c;                   // wide tiles: the output, all slices' rows one after the other
   int M, N, K;            // output rows, output columns, contraction length
   int k_chunk;            // contraction slice (multiple of TC_BK); K rounded up if not split
   int n_split;            // number of contraction slices; slice z writes its own partial output
@@ -134,6 +156,7 @@ struct TcLayer {
   // A slice leaves its accumulators in tail_ws; the warp that finds itself last (tail_count) adds the slices
   // in slice order and runs the epilogue.  tail_split <= 1 switches this off.
   int tail_begin, tail_split;
+  TcDiv tiles_n, tiles_mn;                // column tiles, output tiles
   float *tail_ws;         // [tiles from tail_begin][tail_split][8 or 16 warps][64][32] floats
   int *tail_count;        // [tiles from tail_begin][8 or 16 warps], zero before and after every launch
 };
@@ -170,7 +193,7 @@ struct TcGroup {
 // pdADMM-G-Q that lies on a level set {c s} (the quantised p, or the difference of two of them) is the spacing s times
 // a small integer, and integers up to 2048 are exact in one fp16 plane: its plane holds the integers, there is no lo
 // plane to load and no MMA for it (two MMAs per product instead of three), and mul = s restores the values.
-template <int LAYOUT, class Epi, int ZERO, bool PAIR>
+template <int LAYOUT, class Epi, int ZERO, bool PAIR, bool WIDE>
 __global__ void __maxnreg__(TC_REGS_LAUNCH)
 gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   constexpr bool A_MN = (LAYOUT & TC_A_MN) != 0, B_MN = (LAYOUT & TC_B_MN) != 0, COARSE = epi_coarse<Epi>::value || ZERO == 3;
@@ -180,11 +203,13 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   constexpr bool A_LO = !(ZERO & 1) && !COARSE, B_LO = !(ZERO & 2) && !COARSE;
   constexpr int FLUSH = COARSE ? 8 : TC_FLUSH;        // K blocks per read-out of the main accumulator
   constexpr int A_PLANES = A_LO ? 2 : 1, B_PLANES = B_LO ? 2 : 1;
-  constexpr int CG = PAIR ? 2 : 1, WARPS = CG * TC_ACC_WARPS, TILE_M = PAIR ? 2 * TC_BM : TC_BM;
-  constexpr int B_PLANE_BYTES = PAIR ? TC_BOX_BYTES : TC_PLANE_BYTES, BN = PAIR ? TC_BN / 2 : TC_BN;    // B held by this block
+  static_assert(PAIR || !WIDE, "wide tiles are those of pairs");
+  constexpr int CG = PAIR ? 2 : 1, WARPS = CG * TC_ACC_WARPS, TILE_M = PAIR ? 2 * TC_BM : TC_BM, TILE_N = WIDE ? TC_WIDE : TC_BN;
+  constexpr int BN = TILE_N / CG, B_PLANE_BYTES = BN * TC_BK * 2;    // B held by this block
   constexpr int STAGE_BYTES = A_PLANES * TC_PLANE_BYTES + B_PLANES * B_PLANE_BYTES;
   constexpr bool STORES = epi_stores<Epi>::value;
-  constexpr int PARTS = tc_parts(LAYOUT, STORES), STAGE_SPACE = TC_SPACE - (PARTS > 0 ? TC_TILE_BYTES / PARTS : 0);
+  constexpr int PARTS = tc_parts(LAYOUT, STORES);
+  constexpr int STAGE_SPACE = TC_SPACE - (WIDE ? (STORES ? TC_WIDE_WARPS * TC_WIDE_PART_BYTES : 0) : PARTS > 0 ? TC_TILE_BYTES / PARTS : 0);
   constexpr int STAGES = STAGE_SPACE / STAGE_BYTES < TC_MAX_STAGES ? STAGE_SPACE / STAGE_BYTES : TC_MAX_STAGES;
   constexpr int B_OFF = A_PLANES * TC_PLANE_BYTES;            // stage: A_hi, A_lo, B_hi, B_lo (those that exist)
   extern __shared__ uint8_t smem_raw[];
@@ -192,12 +217,16 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint8_t *tr_base = smem + STAGE_SPACE;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + TC_SPACE);
   uint64_t *full_bar = bars, *empty_bar = bars + STAGES;
-  uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + TC_ACC_BUFS;
-  uint64_t *corr_empty = acc_empty + TC_ACC_BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1, *split_bar = team_bar + 1;
+  constexpr int BUFS = WIDE ? TC_TMEM_COLS / TC_WIDE : TC_ACC_BUFS, READERS = WIDE ? TC_WIDE_WARPS : TC_ACC_WARPS;
+  uint64_t *acc_full = bars + 2 * STAGES, *acc_empty = acc_full + BUFS;
+  uint64_t *corr_empty = acc_empty + BUFS, *drain_bar = corr_empty + 1, *team_bar = drain_bar + 1, *split_bar = team_bar + 1;
   uint64_t *done_full = split_bar + STAGES, *done_empty = done_full + TC_ACC_WARPS;     // one pair per accumulate warp
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
+  // wide: arrivals of accumulate warps at the end of a layer, of all layers; the layers that the block completed; set when every layer
+  // but the last is counted
+  int *layers_left = reinterpret_cast<int *>(tmem_slot + 3);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_rank() : 0u;
@@ -211,18 +240,19 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       ptx::mbar_init(&empty_bar[s], 1);
       ptx::mbar_init(&split_bar[s], CG * TC_SPLIT_WARPS);
     }
-    for (int b = 0; b < TC_ACC_BUFS; ++b) {
+    for (int b = 0; b < BUFS; ++b) {
       ptx::mbar_init(&acc_full[b], 1);
-      ptx::mbar_init(&acc_empty[b], CG * TC_ACC_WARPS);
+      ptx::mbar_init(&acc_empty[b], CG * READERS);
     }
     ptx::mbar_init(corr_empty, CG * TC_ACC_WARPS);
     ptx::mbar_init(drain_bar, 1);
-    ptx::mbar_init(team_bar, TC_ACC_WARPS);
+    ptx::mbar_init(team_bar, READERS);
     for (int w = 0; w < TC_ACC_WARPS; ++w) {
       ptx::mbar_init(&done_full[w], 1);
       ptx::mbar_init(&done_empty[w], 1);
     }
     *abort_flag = 0;
+    layers_left[0] = layers_left[1] = layers_left[2] = 0;
     ptx::fence_barrier_init();
   }
   if (warp == 1) ptx::tmem_alloc<CG>(tmem_slot, TC_TMEM_COLS);
@@ -230,7 +260,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   // them are usable; only of layers this block works on: the step of a finished layer may already have changed the words of
   // the others.
   __shared__ int lay_exp[TC_MAX_GROUP][2];
-  __shared__ double team_scratch[1 + TC_ACC_WARPS];
+  __shared__ double team_scratch[1 + READERS];
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
   if (warp == 2 && lane < grp.n) {
     const TcLayer<Epi> &y = grp.l[lane];
@@ -258,6 +288,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     ptx::prefetch_tmap(&grp.l[g].b);
     if (A_LO) ptx::prefetch_tmap(&grp.l[g].alo);
     if (B_LO) ptx::prefetch_tmap(&grp.l[g].blo);
+    if (WIDE && STORES) ptx::prefetch_tmap(&grp.l[g].c);
   }
   ptx::tc_fence_before_sync();
   if constexpr (PAIR) ptx::cluster_sync();          // the barriers of both blocks are in place
@@ -272,16 +303,15 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     while (unit >= grp.unit_end[t.g]) ++t.g;
     const TcLayer<Epi> &y = grp.l[t.g];
     if (t.g > 0) unit -= grp.unit_end[t.g - 1];
-    const int tiles_n = (y.N + TC_BN - 1) / TC_BN, tiles_m = (y.M + TILE_M - 1) / TILE_M;
     t.out = unit; t.slice = -1;
     if (y.tail_split > 1 && unit >= y.tail_begin) {
       t.out = y.tail_begin + (unit - y.tail_begin) / y.tail_split;
       t.slice = (unit - y.tail_begin) % y.tail_split;
     }
-    t.z = t.out / (tiles_m * tiles_n);
-    const int rem = t.out - t.z * tiles_m * tiles_n;
-    t.m0 = (rem / tiles_n) * TILE_M + (int)rank * TC_BM;       // of this block
-    t.n0 = (rem % tiles_n) * TC_BN;
+    t.z = y.n_split == 1 ? 0 : y.tiles_mn(t.out);
+    const int rem = t.out - t.z * y.tiles_mn.d, row = y.tiles_n(rem);
+    t.m0 = row * TILE_M + (int)rank * TC_BM;       // of this block
+    t.n0 = (rem - row * y.tiles_n.d) * TILE_N;
     t.k_begin = t.z * y.k_chunk;
     const int k_end = min(y.K, t.k_begin + y.k_chunk);
     t.n_kb = (max(k_end - t.k_begin, 0) + TC_BK - 1) / TC_BK;
@@ -292,13 +322,22 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
     }
   };
 
+  auto n_slots = [](const TcLayer<Epi> &y) { return (y.M + TC_BM - 1) / TC_BM * ((y.N + TC_BN - 1) / TC_BN) * TC_ACC_WARPS; };
+  // Adds this block's finished units of a layer to its count; 1 if that completes it.  What the caller waited for -- the sums and
+  // maxima of every accumulate warp -- comes before the count.
+  auto count_units = [&](int g, int visited) {
+    const int units = (grp.unit_end[g] - (g > 0 ? grp.unit_end[g - 1] : 0)) * CG;
+    __threadfence();
+    return atomicAdd(grp.l[g].done, visited) + visited == units ? 1 : 0;
+  };
+
   // Register budgets per warpgroup (every warp of a warpgroup executes the same instruction; the choice is
   // block-uniform, so a block that skips its work leaves the budgets alone).
   const bool skip = PAIR ? ptx::ld_cluster_int(ptx::cluster_addr(const_cast<int *>(skip_flag), 0)) != 0 : *skip_flag != 0;
   if (skip) {
     // nothing: do not queue work behind a block whose bounded wait expired
   } else if (warp < TC_ACC0) {
-    ptx::setmaxnreg_dec<TC_REGS_CTRL>();
+    ptx::setmaxnreg_dec<WIDE ? TC_WIDE_REGS_CTRL : TC_REGS_CTRL>();
     if (warp == 0) {
       // -------------------------------------------------------------- TMA producer (one lane)
       if (lane == 0) {
@@ -355,8 +394,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       // registers.  (With a single lane running this loop, every descriptor word went through a vector register first: 416
       // cycles per K block on top of 72 per MMA.)
       if (rank == 0) {
-        constexpr uint32_t idesc = ptx::idesc_f16(TILE_M, TC_BN, A_MN, B_MN);
-        const uint32_t d_corr = tmem_base + TC_COL_CORR;
+        constexpr uint32_t idesc = ptx::idesc_f16(TILE_M, TILE_N, A_MN, B_MN);
+        const uint32_t d_corr = tmem_base + TC_COL_CORR;        // (not of a wide tile)
         // descriptors with a constant high word; the low word of stage 0 advances by whole stages and K steps (16 values of
         // the contraction index: 32 bytes of every row if K-major, 16 rows if MN-major)
         const uint32_t hi_w = ptx::smem_desc_hi();
@@ -378,16 +417,16 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           for (int kb = 0; kb < n_kb; ++kb) {
             const bool first = kb % FLUSH == 0, last = kb % FLUSH == FLUSH - 1 || kb == n_kb - 1;
             bool good = ptx::mbar_wait(&full_bar[s], sp, abort_flag);
-            if (first && used >= TC_ACC_BUFS) good = good && ptx::mbar_wait(&acc_empty[b], bp, abort_flag);
+            if (first && used >= BUFS) good = good && ptx::mbar_wait(&acc_empty[b], bp, abort_flag);
             ok = __all_sync(0xffffffffu, good);
             if (!ok) break;
             if (PAIR && any_split) ptx::fence_cluster();
             ptx::tc_fence_after_sync();
             const uint32_t la = lo_a0 + (uint32_t)s * (STAGE_BYTES >> 4), lb = lo_b0 + (uint32_t)s * (STAGE_BYTES >> 4);
-            const uint32_t d = tmem_base + (uint32_t)(b * TC_BN);
+            const uint32_t d = tmem_base + (uint32_t)(b * TILE_N);
             auto desc_a = [&](int kk, bool lo) { return ptx::smem_desc(hi_w, la + (lo ? plane_a : 0u) + kk * step_a); };
             auto desc_b = [&](int kk, bool lo) { return ptx::smem_desc(hi_w, lb + (lo ? plane_b : 0u) + kk * step_b); };
-            const bool corr_busy = !COARSE && kb == 0 && ti > 0;
+            const bool corr_busy = !COARSE && !WIDE && kb == 0 && ti > 0;
             if (corr_busy) {
               // The correction tile still holds the previous output tile until the accumulate warps have read it:
               // the main-term MMAs of this block, which do not touch it, go first and keep the tensor pipe busy
@@ -401,7 +440,18 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
               ptx::tc_fence_after_sync();
             }
             if (ptx::elect_one()) {
-              if (corr_busy) {
+              if constexpr (WIDE && !COARSE) {
+                // into one accumulator: the correction terms first, which are small; the first MMA of the main term scales their
+                // sum by 2^-11
+#pragma unroll
+                for (int kk = 0; kk < TC_KSTEPS; ++kk) {
+                  if (A_LO) ptx::mma_f16<CG, ptx::A_ONCE>(d, desc_a(kk, true), desc_b(kk, false), idesc, kk > 0);
+                  if (B_LO) ptx::mma_f16<CG, ptx::A_ONCE>(d, desc_a(kk, false), desc_b(kk, true), idesc, A_LO || kk > 0);
+                }
+                ptx::mma_f16_scaled<CG>(d, desc_a(0, false), desc_b(0, false), idesc);
+#pragma unroll
+                for (int kk = 1; kk < TC_KSTEPS; ++kk) ptx::mma_f16<CG, ptx::A_ONCE>(d, desc_a(kk, false), desc_b(kk, false), idesc, true);
+              } else if (corr_busy) {
 #pragma unroll
                 for (int kk = 0; kk < TC_KSTEPS; ++kk) {
                   // the first correction MMA of a tile overwrites the tile, every later one accumulates
@@ -426,7 +476,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
             }
             if (last) {
               ++used;
-              if (++b == TC_ACC_BUFS) { b = 0; bp ^= 1u; }
+              if (++b == BUFS) { b = 0; bp ^= 1u; }
             }
             if (++s == STAGES) { s = 0; sp ^= 1u; }
           }
@@ -461,17 +511,37 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           if (lo_too) *reinterpret_cast<uint4 *>(dst + boxes * TC_BOX_BYTES + off) = l;
         }
       };
+      // Wide tiles: warp 3 counts the tiles of a layer that the block has no further unit of, once the accumulate warps have arrived,
+      // and notes the layers that this completes; the accumulate warps add those layers' slots at the end.  (With the accumulate
+      // warps counting, and waiting for one another, at every change of layer the tensor cores stood still; with warp 3
+      // adding the slots as well one block became the last of every layer, one after the other.)
+      int left = 0, visited = 0;
+      auto leave = [&](int g) {
+        left += TC_WIDE_WARPS;
+        const long long t0 = clock64();
+        // (a count, not a barrier: the accumulate warps may be several layers ahead)
+        while (*reinterpret_cast<volatile int *>(layers_left) < left) {
+          if (*abort_flag) return false;
+          if (clock64() - t0 > 1000000000ll) { *abort_flag = 1; return false; }
+          __nanosleep(100);
+        }
+        if (lane == 0 && count_units(g, visited)) layers_left[1] |= 1 << g;
+        return true;
+      };
       int s = 0, it = 0;
       uint32_t ph = 1;
-      bool ok = false;
-      for (int g = 0; g < grp.n; ++g) ok |= lay_split[g] != 0;
+      bool ok = true, any_split = false;
+      for (int g = 0; g < grp.n; ++g) any_split |= lay_split[g] != 0;
+      const bool counts = WIDE && Epi::kSumsq && warp == 3 && grp.n > 1;
       Tile u;
-      for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
+      for (int round = 0, unit = unit0; unit < n_units && ok && (counts || any_split); unit = unit_of(++round)) {
+        int g_before = u.g;
         locate(unit, u);
+        if (round == 0) g_before = u.g;
         const TcLayer<Epi> &y = grp.l[u.g];
         const int split = lay_split[u.g];
         const float scale_a = tc_pow2(lay_exp[u.g][0]), scale_b = tc_pow2(lay_exp[u.g][1]);
-        for (int kb = 0; kb < u.n_kb; ++kb, ++it) {
+        for (int kb = 0; any_split && kb < u.n_kb; ++kb, ++it) {
           ok = it < STAGES || ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           uint8_t *st = smem + s * STAGE_BYTES;
@@ -486,8 +556,237 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(&split_bar[s], 0));      // (every stage: the phases stay in step)
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
+        if (ok && counts) {
+          // (the accumulate warps finish the layer before during the first tile of the next one, for which nothing may be left
+          // to do here)
+          if (u.g != g_before) {
+            ok = grp.l[g_before].slots == nullptr || __all_sync(0xffffffffu, leave(g_before));
+            visited = 0;
+          }
+          ++visited;
+        }
+      }
+      if (counts && ok && lane == 0) {
+        __threadfence_block();
+        *reinterpret_cast<volatile int *>(layers_left + 2) = 1;
       }
     }
+  } else if constexpr (WIDE) {
+    // ---------------------------------------------------------------- wide tiles
+    ptx::setmaxnreg_inc<TC_WIDE_REGS_ACC>();
+    // Accumulate warp aw: rows of quarter aw mod 4, columns 64 (aw / 4) .. +63 of every tile of the block.
+    const int aw = warp - TC_ACC0, quarter = warp & 3, col_base = 64 * (aw >> 2), lane_base = quarter * 32;
+    float *buf = reinterpret_cast<float *>(tr_base + (size_t)aw * TC_WIDE_PART_BYTES);
+    bool ok = true;
+    Tile t;
+    int visited = 0;                                   // units of layer t.g that this block has finished
+    // The accumulate warps among themselves, bounded like every other wait.
+    uint32_t team_ph = 0;
+    auto team_sync = [&]() {
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(team_bar);
+      const bool there = ptx::mbar_wait(team_bar, team_ph, abort_flag);
+      team_ph ^= 1u;
+      return __all_sync(0xffffffffu, there) != 0;
+    };
+    // The block has no further unit: add the slots of every layer that it completed, the last one with this.
+    auto leave_last = [&](int g_last) {
+      if (!Epi::kSumsq) return;
+      volatile int *mask_sh = reinterpret_cast<volatile int *>(team_scratch);
+      volatile double *part = team_scratch + 1;
+      if (!team_sync()) return;
+      if (aw == 0 && lane == 0) {
+        int mask = grp.l[g_last].slots != nullptr && count_units(g_last, visited) ? 1 << g_last : 0;
+        if (grp.n > 1) {
+          const long long t0 = clock64();
+          while (*reinterpret_cast<volatile int *>(layers_left + 2) == 0 && !*abort_flag)
+            if (clock64() - t0 > 1000000000ll) *abort_flag = 1;
+          __threadfence();
+          mask |= *reinterpret_cast<volatile int *>(layers_left + 1);
+        }
+        *mask_sh = *abort_flag ? 0 : mask;
+      }
+      if (!team_sync()) return;
+      const int mask = *mask_sh;
+      for (int g = 0; mask >> g; ++g) {
+        if (!(mask >> g & 1)) continue;
+        const TcLayer<Epi> &y = grp.l[g];
+        __threadfence();
+        const int n = n_slots(y);
+        double v = 0.0;
+#pragma unroll 16
+        for (int i = aw * 32 + lane; i < n; i += 32 * TC_WIDE_WARPS) v += __ldcg(y.slots + i);
+        v = warp_sum(v);
+        if (lane == 0) part[aw] = v;
+        if (!team_sync()) return;
+        if (aw == 0 && lane == 0) {
+          double sum = 0.0;
+          for (int w = 0; w < TC_WIDE_WARPS; ++w) sum += part[w];
+          *y.done = 0;
+          finish_step(y.step, sum);
+        }
+        if (!team_sync()) return;
+      }
+    };
+    auto put_sum = [&](const TcLayer<Epi> &y, double v) {
+      v = warp_sum(v);
+      const int tiles_n = (y.N + TC_BN - 1) / TC_BN, tile = t.n0 / TC_BN + (aw >> 3);
+      if (lane == 0 && t.m0 < y.M && tile < tiles_n) y.slots[((size_t)(t.m0 / TC_BM) * tiles_n + tile) * TC_ACC_WARPS + (aw & 7)] = v;
+    };
+    int b = 0;
+    uint32_t ph = 0;                                   // phase of acc_full[b]
+    const uint32_t tm_lane = tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)col_base;
+    for (int round = 0, unit = unit0; unit < n_units && ok; unit = unit_of(++round)) {
+      const int g_before = t.g;
+      locate(unit, t);
+      if (round > 0 && t.g != g_before) {
+        visited = 0;
+        if (Epi::kSumsq && grp.l[g_before].slots != nullptr) {
+          __syncwarp();
+          if (lane == 0) {
+            __threadfence_block();
+            atomicAdd(layers_left, 1);
+          }
+        }
+      }
+      ++visited;
+      const TcLayer<Epi> &y = grp.l[t.g];
+      const int n_grp = (t.n_kb + FLUSH - 1) / FLUSH;    // read-outs of an accumulator for this tile
+      uint64_t acc[32];                                  // columns 2 j, 2 j + 1 in acc[j]
+#pragma unroll
+      for (int j = 0; j < 32; ++j) acc[j] = 0ull;
+      for (int g = 0; g < n_grp; ++g) {
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[b], ph, abort_flag));
+        if (!ok) break;
+        ptx::tc_fence_after_sync();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t v[16];
+          ptx::tmem_ld16(tm_lane + (uint32_t)(b * TC_WIDE + 16 * c), v);
+          ptx::tmem_ld_wait(v);
+          if (c == 3) {
+            // the accumulator is given back (one arrival per warp on block 0's barrier, whose MMA warp waits) as soon as its last
+            // columns are in registers
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_cluster(ptx::cluster_addr(&acc_empty[b], 0));
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[8 * c + j] = ptx::add_f2(acc[8 * c + j], ptx::pack_f2(v[2 * j], v[2 * j + 1]));
+        }
+        if (++b == BUFS) { b = 0; ph ^= 1u; }
+      }
+      if (!ok) break;
+      {
+        // undo the operand scalings (an exact factor, or two where one would leave the range)
+        const int e = lay_exp[t.g][0] + lay_exp[t.g][1], e1 = e >= -120 && e <= 120 ? e : e / 2, e2 = e - e1;
+        const uint32_t u1 = __float_as_uint(tc_pow2(-e1)), u2 = __float_as_uint(tc_pow2(-e2));
+        const uint64_t w1 = ptx::pack_f2(u1, u1), w2 = ptx::pack_f2(u2, u2);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], w1);
+        if (e2 != 0) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], w2);
+        }
+        if constexpr (ZERO != 0) {
+          const uint64_t mul = ptx::pack_f2(__float_as_uint(y.mul), __float_as_uint(y.mul));
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = ptx::mul_f2(acc[j], mul);
+        }
+      }
+      if (STORES && t.slice >= 0) {
+        // contraction slice of a tail tile: park the piece; the last warp to arrive adds the slices, in slice order
+        constexpr int PIECES = CG * TC_WIDE_WARPS;
+        const int t_idx = t.out - y.tail_begin, piece = (int)rank * TC_WIDE_WARPS + aw;
+        float4 *part = reinterpret_cast<float4 *>(y.tail_ws) + ((size_t)t_idx * y.tail_split * PIECES + piece) * 512 + lane;
+        constexpr size_t SLICE = (size_t)PIECES * 512;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          float4 v;
+          ptx::unpack_f2(acc[2 * j], v.x, v.y);
+          ptx::unpack_f2(acc[2 * j + 1], v.z, v.w);
+          part[t.slice * SLICE + j * 32] = v;
+        }
+        __syncwarp();
+        int prev = 0;
+        if (lane == 0) {
+          __threadfence();             // of the whole warp's parked values
+          prev = atomicAdd(y.tail_count + t_idx * PIECES + piece, 1);
+        }
+        prev = __shfl_sync(0xffffffffu, prev, 0);
+        if (prev != y.tail_split - 1) continue;
+        __threadfence();
+        if (lane == 0) y.tail_count[t_idx * PIECES + piece] = 0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = 0ull;
+        for (int sl = 0; sl < y.tail_split; ++sl) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float4 v = __ldcg(part + sl * SLICE + j * 32);
+            acc[2 * j] = ptx::add_f2(acc[2 * j], ptx::pack_f2(__float_as_uint(v.x), __float_as_uint(v.y)));
+            acc[2 * j + 1] = ptx::add_f2(acc[2 * j + 1], ptx::pack_f2(__float_as_uint(v.z), __float_as_uint(v.w)));
+          }
+        }
+      }
+      // Parts of 32 rows x 16 columns, a row per lane, go into the warp's buffer (16-byte groups XOR-ed as the copy's 64-byte swizzle
+      // wants them, which is free of bank conflicts) and out by a bulk copy; rows and columns outside the matrix are clipped.
+      // Columns up to the leading dimension are written: those from N on come out as exact zeros, which keeps the padding of every
+      // matrix zero.  The sum of squares and the largest magnitude (rows and columns outside hold exact zeros) are taken while a
+      // copy reads the buffer: one after the other the end of a tile took 8000 cycles, of which the MMAs run ahead 3000.
+      const int row0 = t.m0 + lane_base;
+      uint64_t s2[4] = {0ull, 0ull, 0ull, 0ull};
+      uint32_t mx = 0u;
+      const bool wants_sum = Epi::kSumsq && y.slots != nullptr;
+      bool wants_max = false;
+      if constexpr (epi_amax<Epi>::value) wants_max = y.epi.amax != nullptr;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        if constexpr (STORES) {
+          const int col = t.n0 + col_base + TC_WIDE_PART * p;
+          ptx::bulk_wait_read();                       // (of the lane that copied) the buffer is free again
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float4 v;
+            ptx::unpack_f2(acc[8 * p + 2 * j], v.x, v.y);
+            ptx::unpack_f2(acc[8 * p + 2 * j + 1], v.z, v.w);
+            reinterpret_cast<float4 *>(buf)[lane * 4 + (j ^ ((lane >> 1) & 3))] = v;
+          }
+          ptx::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0 && row0 < y.M && col < y.epi.ldc) {
+            ptx::tma_store_3d(&y.c, buf, col, row0, t.z);
+            ptx::bulk_commit();
+          }
+        }
+        if (Epi::kSumsq && wants_sum) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) s2[j & 3] = ptx::fma_f2(acc[8 * p + j], acc[8 * p + j], s2[j & 3]);
+        }
+        if constexpr (epi_amax<Epi>::value) {
+          if (wants_max) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              float a0, a1;
+              ptx::unpack_f2(acc[8 * p + j], a0, a1);
+              mx = __vimax3_u32(mx, abs_bits(a0), abs_bits(a1));
+            }
+          }
+        }
+      }
+      if (Epi::kSumsq && wants_sum) {
+        float s4[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ptx::unpack_f2(s2[j], s4[2 * j], s4[2 * j + 1]);
+        put_sum(y, (((double)s4[0] + (double)s4[1]) + ((double)s4[2] + (double)s4[3])) + (((double)s4[4] + (double)s4[5]) + ((double)s4[6] + (double)s4[7])));
+      }
+      if constexpr (epi_amax<Epi>::value) {
+        if (wants_max) commit_amax(mx, y.epi.amax);      // the output is an operand of a later product
+      }
+    }
+    if (STORES) ptx::bulk_wait_all();                 // before shared memory goes, and before the sums are announced
+    __syncwarp();
+    if (ok) leave_last(t.g);
   } else {
     // Accumulate warp aw and epilogue warp aw: rows of quarter aw mod 4, columns col_base .. +63 of every tile of the block.
     const bool accumulates = warp < TC_EPI0;
@@ -528,7 +827,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       if (!team_sync()) return false;
       if (*last != 0) {
         __threadfence();
-        const int n = (y.M + TC_BM - 1) / TC_BM * ((y.N + TC_BN - 1) / TC_BN) * TC_ACC_WARPS;
+        const int n = n_slots(y);
         double v = 0.0;
 #pragma unroll 4
         for (int i = tid; i < n; i += n_threads) v += __ldcg(y.slots + i);

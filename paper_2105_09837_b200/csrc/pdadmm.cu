@@ -118,6 +118,7 @@ struct Layer {
   uint32_t *w_g = nullptr, *w_wg = nullptr, *w_G = nullptr, *w_d = nullptr;
   int *done = nullptr;             // [4] counters of finished blocks (trial, gradient sum, then products), zero between kernels
   int n_split = 1, k_chunk = 0;
+  bool wide_W = false, wide_wg = false, wide_gp = false;      // wide tiles for the W-gradient, W g and G p (choose_wide)
 };
 
 struct Scratch {
@@ -358,6 +359,29 @@ static int get_tmap(pdadmm_ctx *c, const void *base, uint64_t inner, uint64_t ou
   return PDADMM_OK;
 }
 
+// Where the wide tiles of a product store: parts of 32 rows x 16 columns of a matrix [slice][rows][ld] (slices `stride` floats apart),
+// 64-byte swizzle; what lies outside is clipped.
+static int get_out_tmap(pdadmm_ctx *c, const float *base, uint64_t rows, uint64_t ld, uint64_t slices, uint64_t stride, CUtensorMap *out) {
+  auto key = std::make_tuple((const void *)base, ~rows, ld, slices << 40 ^ stride);
+  auto it = c->tmaps.find(key);
+  if (it != c->tmaps.end()) { *out = it->second; return PDADMM_OK; }
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return fail(PDADMM_ECUDA, "cuTensorMapEncodeTiled is not available in this driver");
+  cuuint64_t dims[3] = {ld, rows, slices};
+  cuuint64_t strides[2] = {ld * 4, stride * 4};
+  cuuint32_t box[3] = {(cuuint32_t)TC_WIDE_PART, 32u, 1u};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUtensorMap m;
+  const CUresult r = fn(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(PDADMM_ECUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
+  if (c->tmaps.size() > 4096) c->tmaps.clear();
+  c->tmaps[key] = m;
+  *out = m;
+  return PDADMM_OK;
+}
+
 // One layer's part of a product launch.
 template <class Epi>
 struct Prod {
@@ -370,10 +394,11 @@ struct Prod {
   Step step{};
   int n_split = 1, k_chunk = 0;    // contraction slices, and their length
   size_t stride = 0;               // floats between the partial outputs of two slices
+  bool wide = false;               // may run on wide tiles, and is to (see choose_wide)
 };
-template <int LAYOUT, class Epi, int ZERO, bool PAIR>
+template <int LAYOUT, class Epi, int ZERO, bool PAIR, bool WIDE>
 static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &grp) {
-  auto kern = gemm_tc_kernel<LAYOUT, Epi, ZERO, PAIR>;
+  auto kern = gemm_tc_kernel<LAYOUT, Epi, ZERO, PAIR, WIDE>;
   // the attribute belongs to (kernel, device): one flag per device ordinal for this instantiation
   static bool configured[MAX_DEVICES] = {false};
   const int dev = c->device;
@@ -407,6 +432,7 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &gr
 // 256 rows.  So: where at least three quarters of the pairs get a tile, and padding M to 256 rows instead of 128 adds at most
 // a tenth.  (20 000 x 500 x 500: 43.2 us in pairs, 45.5 us without; x 2000 x 2000: 399 against 457 us; 2000 x 100 x 100, 8
 // pairs: 12.5 against 10.7 us.)
+static bool worth_pairs(int n_sms, int64_t single, int64_t paired) { return paired * 10 <= single * 11 && (paired / 2) * 8 >= 3 * (int64_t)n_sms; }
 template <class Epi>
 static bool use_pairs(const pdadmm_ctx *c, const Prod<Epi> *v, int n) {
   int64_t single = 0, paired = 0;
@@ -415,7 +441,39 @@ static bool use_pairs(const pdadmm_ctx *c, const Prod<Epi> *v, int n) {
     single += ceil_div(v[i].M, TC_BM) * cols;
     paired += 2 * ceil_div(v[i].M, 2 * TC_BM) * cols;
   }
-  return paired * 10 <= single * 11 && (paired / 2) * 8 >= 3 * (int64_t)c->n_sms;
+  return worth_pairs(c->n_sms, single, paired);
+}
+// Whether some products [rows, columns, contraction of a slice, slices], worked on in one launch, run on wide tiles: the shorter
+// estimate of the two.  The persistent grid takes the tiles in rounds; SM cycles per K block and at a tile's end, from traces of
+// 20 000 x 500, 170 000 x 1000 and 90 000 x 2000: a block on its own 1560 and 2800, a pair 1080 and 2800, a pair with a wide
+// tile 1500 and 8800 (its accumulate warps store the tile themselves); with two MMAs per product instead of three (integer
+// operands) 1230, 830, 1130 and 6900 at the end.  So a wide tile, which brings 64 KB per K block where two
+// narrow ones bring 96, wins from some six K blocks on, unless its columns are mostly padding or leave SMs idle.  (170 000 x 1000
+// G p+: 1.04 -> 0.90 ms; 90 000 x 2000: 1.50 -> 1.30 ms; W-gradient of 20 000 x 500, 9 layers: 410 -> 330 us.)
+struct Shape { int64_t M, N, K, n_split; };
+static bool choose_wide(int n_sms, const Shape *v, int n, bool ints, double *cost = nullptr) {
+  double best[2];
+  int64_t single = 0, paired = 0;
+  for (int i = 0; i < n; ++i) {
+    single += ceil_div(v[i].M, TC_BM) * ceil_div(v[i].N, TC_BN) * v[i].n_split;
+    paired += 2 * ceil_div(v[i].M, 2 * TC_BM) * ceil_div(v[i].N, TC_BN) * v[i].n_split;
+  }
+  const bool pairs = worth_pairs(n_sms, single, paired);
+  for (int wide = 0; wide < 2; ++wide) {
+    const int rows = wide || pairs ? 2 * TC_BM : TC_BM, slots = wide || pairs ? n_sms / 2 : n_sms;
+    const double per_block = wide ? (ints ? 1130 : 1500) : pairs ? (ints ? 830 : 1080) : ints ? 1230 : 1560;
+    const double end = wide ? (ints ? 6900 : 8800) : 2800;
+    double work = 0;
+    int64_t units = 0;
+    for (int i = 0; i < n; ++i) {
+      const int64_t u = ceil_div(v[i].M, rows) * ceil_div(v[i].N, wide ? TC_WIDE : TC_BN) * v[i].n_split;
+      units += u;
+      work += (double)u * (per_block * ceil_div(v[i].K, TC_BK) + end);
+    }
+    best[wide] = work / units * ceil_div(units, slots);
+  }
+  if (cost) *cost = std::min(best[0], best[1]);
+  return best[1] < best[0];
 }
 // op(A) is M x K, op(B) is N x K; A_MN: A is stored [K][M], B_MN: B is stored [K][N].  At most TC_MAX_GROUP products.
 template <int LAYOUT, class Epi, int ZERO = 0>
@@ -425,7 +483,11 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
   TcGroup<Epi> grp;
   grp.n = n;
   grp.error = c->d_flag + 1;
-  const bool pair = use_pairs(c, v, n);
+  constexpr bool CAN_WIDE = Epi::kDirect;
+  bool wide = CAN_WIDE;
+  for (int i = 0; i < n; ++i) wide = wide && v[i].wide;
+  const bool pair = wide || use_pairs(c, v, n);
+  const int tile_n = wide ? TC_WIDE : TC_BN;
   int units = 0;
   for (int i = 0; i < n; ++i) {
     const Prod<Epi> &p = v[i];
@@ -437,6 +499,10 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
     PD_TRY(get_tmap(c, p.B.hi, B_MN ? N : K, B_MN ? K : N, (uint64_t)p.B.ld, &y.b));
     if (p.B.lo && p.B.lo != p.B.hi) PD_TRY(get_tmap(c, p.B.lo, B_MN ? N : K, B_MN ? K : N, (uint64_t)p.B.ld, &y.blo));
     else y.blo = y.b;
+    if (wide && epi_stores<Epi>::value)
+      PD_TRY(get_out_tmap(c, p.epi.C, M, (uint64_t)p.epi.ldc, (uint64_t)p.n_split, p.n_split > 1 ? p.stride : M * p.epi.ldc, &y.c));
+    else
+      y.c = y.a;
     y.M = p.M; y.N = p.N; y.K = p.K;
     y.k_chunk = p.n_split > 1 ? p.k_chunk : round_up(p.K, TC_BK);
     y.n_split = p.n_split;
@@ -447,7 +513,9 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
     y.epi = p.epi;
     y.slots = p.slots; y.done = p.done; y.step = p.step;
     y.tail_begin = 0; y.tail_split = 0; y.tail_ws = nullptr; y.tail_count = nullptr;
-    const int n_tiles = (int)(ceil_div(p.M, pair ? 2 * TC_BM : TC_BM) * ceil_div(p.N, TC_BN)) * p.n_split;
+    const int tiles_n = (int)ceil_div(p.N, tile_n), tiles_mn = (int)ceil_div(p.M, pair ? 2 * TC_BM : TC_BM) * tiles_n, n_tiles = tiles_mn * p.n_split;
+    y.tiles_n = TcDiv::of(tiles_n, tiles_mn);
+    y.tiles_mn = TcDiv::of(tiles_mn, n_tiles);
     units += n_tiles;
     // The persistent grid works through the tiles in rounds; a last round that fills only part of the
     // SMs costs as much as a full one, so its tiles are cut along the contraction into as many slices as fit (at least 8 K
@@ -464,8 +532,11 @@ static int launch_tc(pdadmm_ctx *c, cudaStream_t st, const Prod<Epi> *v, int n) 
     }
     grp.unit_end[i] = units;
   }
-  if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true>(c, st, grp);
-  return launch_tc_form<LAYOUT, Epi, ZERO, false>(c, st, grp);
+  if constexpr (CAN_WIDE) {
+    if (wide) return launch_tc_form<LAYOUT, Epi, ZERO, true, true>(c, st, grp);
+  }
+  if (pair) return launch_tc_form<LAYOUT, Epi, ZERO, true, false>(c, st, grp);
+  return launch_tc_form<LAYOUT, Epi, ZERO, false, false>(c, st, grp);
 }
 
 // ---- largest magnitudes of product operands ------------------------------------------------------------------
@@ -716,6 +787,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
       Layer &ly = c->layers[batch[i]];
       Scratch &s = scratch_of(c, batch[i]);
       Prod<decltype(make_epi(0))> p{N, ly.n_out, ly.n_in, G[i], operand_W(ly), make_epi(batch[i]), &s, s.slots + s.n_slots / 2, ly.done + 2};
+      p.wide = ly.wide_wg;
       Step t = make_step(c, ly, STEP_TAU);
       if (c->use_tc) {
         t.w_in = ly.w_g; t.w_out = norm_only ? nullptr : ly.w_wg;
@@ -888,7 +960,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       Layer &ly = c->layers[batch[i]];
       Scratch &s = scratch_of(c, batch[i]);
       Prod<EpiStore> p{ly.n_out, ly.n_in, N, R[i], P[i], EpiStore{s.part, ly.ld_in}, &s};
-      p.n_split = ly.n_split; p.k_chunk = ly.k_chunk; p.stride = (size_t)ly.n_out * ly.ld_in;
+      p.n_split = ly.n_split; p.k_chunk = ly.k_chunk; p.stride = (size_t)ly.n_out * ly.ld_in; p.wide = ly.wide_W;
       v.push_back(p);
     }
     PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, v));
@@ -944,6 +1016,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       Layer &ly = c->layers[l];
       Scratch &s = scratch_of(c, l);
       Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done + 2};
+      p.wide = ly.wide_gp;
       p.step = make_step(c, ly, STEP_THETA);
       if (c->use_tc) { p.step.w_in = ly.w_G; p.step.exp_W = ly.Wp.exp; p.step.exp_r = ly.rp.exp; p.step.exp_g = ly.Gp.exp; }
       v.push_back(p);
@@ -1445,25 +1518,39 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   // fp32 matrices and the two pairs of planes, which are most of it.
   const size_t e_max = (size_t)N * std::max(max_in, max_out);
   const bool small = c->L > 1 && 3 * 16 * e_max <= (size_t(4) << 30);
-  // Node slices of the W-gradient product (slices >= 256 nodes, at most 32).  The persistent grid works through
-  // tiles x slices units in rounds of n_sms, so the count is chosen to fill its last round: the smallest number
-  // of slices within 3 % (relative) of the best fill (fewer slices = fewer partial tiles to write and add up).  Layers that are
-  // worked on together have one common count.
+  // Node slices of the W-gradient product (slices >= 256 nodes, at most 32): the count with the shortest estimated product
+  // (choose_wide) and sum of the slices, which are written and read once more at 3000 bytes per SM cycle (6000 in L2).  Layers that are worked on
+  // together have one common count.
   auto choose_slices = [&](int l0, int l1) {
-    int64_t tiles = 0;
-    for (int l = l0; l < l1; ++l) tiles += ceil_div(c->layers[l].n_in, SG_BN) * ceil_div(c->layers[l].n_out, SG_BM);
     const int max_split = (int)std::max<int64_t>(1, std::min<int64_t>(32, ceil_div(N, 256)));
-    auto slices_for = [&](int want) { return (int)ceil_div(N, round_up((int)ceil_div(N, want), TC_BK)); };
-    auto fill = [&](int want) {
-      const int64_t units = tiles * slices_for(want);
-      return (double)units / (double)(c->n_sms * ceil_div(units, c->n_sms));
-    };
-    double best = 0.0;
-    for (int w = 1; w <= max_split; ++w) best = std::max(best, fill(w));
     int split = 1;
-    while (split < max_split && fill(split) < 0.97 * best) ++split;
+    double best = 0;
+    for (int w = 1; w <= max_split; ++w) {
+      const int64_t chunk = round_up((int)ceil_div(N, w), TC_BK), slices = ceil_div(N, chunk);
+      Shape v[MAX_GROUP];
+      double cost = 0, values = 0;
+      for (int l = l0; l < l1; ++l) {
+        v[l - l0] = Shape{c->layers[l].n_out, c->layers[l].n_in, chunk, slices};
+        values += (double)c->layers[l].n_out * c->layers[l].ld_in;
+      }
+      choose_wide(c->n_sms, v, l1 - l0, c->int_operands, &cost);
+      cost += 8.0 * values * slices / (4.0 * values * slices < 6e7 ? 6000.0 : 3000.0);
+      if (w == 1 || cost < best) { best = cost; split = w; }
+    }
+    Shape vw[MAX_GROUP], vg[MAX_GROUP], vp[MAX_GROUP];
+    int n = 0, n_wg = 0;
+    for (int l = l0; l < l1; ++l, ++n) {
+      const Layer &ly = c->layers[l];
+      const int64_t chunk = round_up((int)ceil_div(N, split), TC_BK);
+      vw[n] = Shape{ly.n_out, ly.n_in, chunk, ceil_div(N, chunk)};
+      vp[n] = Shape{N, ly.n_out, ly.n_in, 1};
+      if (l > 0) vg[n_wg++] = vp[n];
+    }
+    const bool ints = c->int_operands, wide_W = choose_wide(c->n_sms, vw, n, ints), wide_gp = choose_wide(c->n_sms, vp, n, ints);
+    const bool wide_wg = n_wg > 0 && choose_wide(c->n_sms, vg, n_wg, ints);
     for (int l = l0; l < l1; ++l) {
       Layer &ly = c->layers[l];
+      ly.wide_W = wide_W; ly.wide_gp = wide_gp; ly.wide_wg = wide_wg;
       ly.k_chunk = round_up((int)ceil_div(N, split), TC_BK);      // multiple of both kernels' K blocks
       ly.n_split = (int)ceil_div(N, ly.k_chunk);
       max_part = std::max(max_part, (size_t)ly.n_split * ly.n_out * ly.ld_in);
@@ -1486,7 +1573,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   PD_TRY(dev_alloc(c, &s.red, (size_t)max_out + 8));
   if (c->use_tc) {
     if (!small) {                       // (small problems cut no tails)
-      PD_TRY(dev_alloc(c, &s.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+      PD_TRY(dev_alloc(c, &s.tail_ws, (size_t)c->n_sms * TC_BM * TC_WIDE, false));
       s.tail_count = c->control + 4 + 8 * (size_t)c->L;
     }
     PD_TRY(dev_alloc(c, &s.amax_pool, (size_t)AMAX_POOL));
@@ -1519,7 +1606,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &x.red, (size_t)max_out + 8));
     if (c->use_tc) {
       if (!small) {
-        PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+        PD_TRY(dev_alloc(c, &x.tail_ws, (size_t)c->n_sms * TC_BM * TC_WIDE, false));
         x.tail_count = s.tail_count + (size_t)i * c->n_sms * 8;
       }
       x.pl_cap = s.pl_cap;
@@ -2151,7 +2238,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       cudaStream_t st = c->scr.st;
       PD_TRY(dev_alloc(c, &c->d_flag, 4));
       if (c->use_tc) {
-        PD_TRY(dev_alloc(c, &c->scr.tail_ws, (size_t)c->n_sms * TC_BM * TC_BN, false));
+        PD_TRY(dev_alloc(c, &c->scr.tail_ws, (size_t)c->n_sms * TC_BM * TC_WIDE, false));
         PD_TRY(dev_alloc(c, &c->scr.tail_count, (size_t)c->n_sms * 8));
       }
       // operand shapes as stored: rows x cols
@@ -2186,9 +2273,15 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
       step.kind = STEP_SUM; step.sum = res;
       EpiStoreSumsq epi{dC, ldc};
       if (mode == 0) {
-        PD_TRY((gemm_nodes<false, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
+        Prod<EpiStoreSumsq> p{M, N, K, oA, oB, epi, &c->scr, slots, done, step};
+        const Shape shape{M, N, K, 1};
+        p.wide = choose_wide(c->n_sms, &shape, 1, false);
+        PD_TRY((gemm_nodes<false, EpiStoreSumsq>(c, KC_GEMM_WG, st, {p}, 0)));
       } else if (mode == 1) {
-        PD_TRY((gemm_nodes<true, EpiStoreSumsq>(c, KC_GEMM_WG, st, {{M, N, K, oA, oB, epi, &c->scr, slots, done, step}}, 0)));
+        Prod<EpiStoreSumsq> p{M, N, K, oA, oB, epi, &c->scr, slots, done, step};
+        const Shape shape{M, N, K, 1};
+        p.wide = choose_wide(c->n_sms, &shape, 1, false);
+        PD_TRY((gemm_nodes<true, EpiStoreSumsq>(c, KC_GEMM_WG, st, {p}, 0)));
       } else {
         const int split = (int)std::max<int64_t>(1, std::min<int64_t>(8, ceil_div(K, 64)));
         const int k_chunk = round_up((int)ceil_div(K, split), TC_BK);
@@ -2200,6 +2293,8 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
         } else {
           Prod<EpiStore> p{M, N, K, oA, oB, EpiStore{part, ldc}, &c->scr};
           p.n_split = n_split; p.k_chunk = k_chunk; p.stride = (size_t)M * ldc;
+          const Shape shape{M, N, k_chunk, n_split};
+          p.wide = choose_wide(c->n_sms, &shape, 1, false);
           PD_TRY(gemm_over_nodes(c, KC_GEMM_GRADW, st, {p}));
         }
         const size_t n4 = (size_t)M * ldc / 4;

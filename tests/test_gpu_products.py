@@ -10,6 +10,7 @@ import pytest
 from paper_2105_09837_b200 import binding as B
 from paper_2105_09837_b200 import synth
 import oracle.pdadmm_oracle as o
+import error_bounds as E
 import parity_util as U
 from test_gpu_parity import _compare_iteration
 
@@ -85,3 +86,26 @@ def test_host_copies_at_the_edges_of_a_piece(n_nodes, hidden):
     ctx.set_tensor(B.T_Z, 1, x)
     assert np.array_equal(ctx.get_tensor(B.T_Z, 1), x)
     ctx.destroy()
+
+
+# columns at the edges of a wide tile (256) and of its halves, rows at those of a pair's 256 and a block's 128, contractions at those of
+# a K block; large enough that wide tiles are chosen, alone (with the last round cut along the contraction) and over node slices
+@pytest.mark.parametrize("mode,M,N,K", [(0, 18944, 256, 640), (0, 18945, 255, 641), (1, 19000, 257, 1000), (1, 9600, 500, 703),
+                                        (0, 4800, 1025, 1600), (2, 500, 700, 30000), (2, 257, 2049, 16001), (2, 512, 512, 40000)])
+def test_wide_tiles_at_their_edges(mode, M, N, K):
+    """Every element within LAMBDA standard deviations of KAPPA times the root-sum-square of its terms, the product's bound in the
+    iteration tests."""
+    rng = np.random.default_rng(M + N + K)
+    a = rng.standard_normal((K, M) if mode == 2 else (M, K), dtype=np.float32)
+    b = rng.standard_normal((N, K) if mode == 0 else (K, N), dtype=np.float32)
+    c, ss = B.matmul(mode, a, b)
+    at, bt = (a.T if mode == 2 else a).astype(np.float64), (b.T if mode == 0 else b).astype(np.float64)
+    bound = E.LAMBDA * E.kappa(True) * np.sqrt((at ** 2) @ (bt ** 2))
+    assert (np.abs(c - at @ bt) <= bound).all()
+    assert abs(ss - (c.astype(np.float64) ** 2).sum()) <= 1e-6 * ss
+
+
+def test_refused_planes_on_wide_tiles():
+    """The same as above where the product W g runs on wide tiles and splits its refused operands itself (2000 x 500: below 2^20
+    elements)."""
+    test_refused_planes_in_every_form_of_the_product(2000, 500, 10)
