@@ -153,4 +153,17 @@ __device__ __forceinline__ double block_sum(double v, double *smem /* THREADS/32
   return t;
 }
 
+// The same for a block of any whole number of warps.
+__device__ __forceinline__ double block_sum_any(double v, double *smem) {
+  v = warp_sum(v);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, n = (int)blockDim.x >> 5;
+  __syncthreads();
+  if (l == 0) smem[w] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < n; ++i) t += smem[i];
+  return t;
+}
+
 }  // namespace pd

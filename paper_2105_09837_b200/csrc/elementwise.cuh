@@ -133,51 +133,148 @@ __device__ __forceinline__ void store_planes4(const PlaneOut &o, size_t i, float
   reinterpret_cast<uint2 *>(o.lo)[i] = l;
 }
 
+// ---- blocks of rows -------------------------------------------------------------------------------
+// Kernels that sum a matrix's columns beside what they do.  A block works on n_sub rows at a time and goes on to those n_blocks n_sub
+// rows further (all blocks together walk through the matrix: with a run of rows of its own for every block the z-update of
+// 20 000 x 500, 9 layers, took 5 to 8 % longer with 8-bit codes).  A thread owns a group of 4 columns (float4; several groups if the rows are
+// longer than 1024) of one of the rows, so its sums stay in registers; the row subgroups' sums are combined in subgroup
+// order, then written to slots[block][ld].
+struct RowBlocks { int n_rows, ld, n_blocks; double *slots; int cols_per_pass, n_sub; };
+// How a block's threads share rows of ld values: n_sub rows of cols_per_pass groups at a time, as many as leave the fewest lanes of the
+// block's warps idle (rows of 352: 88 groups, 176 of 192 threads; with blocks of 256 the z-update of 7013 x 333 took 121 us, 103 of
+// the previous pass without sums).
+struct RowShare { int cols_per_pass, n_sub, threads; };
+inline RowShare row_share(int ld) {
+  const int groups = ld / 4, passes = (groups + EW_THREADS - 1) / EW_THREADS, cols = (groups + passes - 1) / passes;
+  RowShare best{cols, 1, (cols + 31) / 32 * 32};
+  for (int k = 2; k * cols <= EW_THREADS; ++k) {
+    const int t = (k * cols + 31) / 32 * 32;
+    if ((int64_t)k * cols * best.threads >= (int64_t)best.n_sub * cols * t) best = RowShare{cols, k, t};
+  }
+  return best;
+}
+// at(first float4, stride, count, column group, sums[4]) for every thread's column group; sh: EW_THREADS * 4 doubles.  All threads
+// take part.
+template <class F>
+__device__ __forceinline__ void row_block_sums(const RowBlocks &y, int block, double *sh, F &&at) {
+  const int n_groups = y.ld >> 2, cols_per_pass = y.cols_per_pass, n_sub = y.n_sub;
+  const int sub = threadIdx.x / cols_per_pass, c0 = threadIdx.x % cols_per_pass;
+  const int row0 = block * n_sub + sub, step = y.n_blocks * n_sub, n = row0 < y.n_rows ? (y.n_rows - row0 + step - 1) / step : 0;
+  double *out = y.slots + (size_t)block * y.ld;
+  if (sub < n_sub) {
+    for (int cg = c0; cg < n_groups; cg += cols_per_pass) {
+      double sum[4] = {0, 0, 0, 0};
+      at((uint32_t)row0 * (uint32_t)n_groups + (uint32_t)cg, (uint32_t)step * (uint32_t)n_groups, n, cg, sum);
+      double *dst = (n_sub > 1 ? sh + (size_t)sub * y.ld : out) + 4 * cg;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dst[e] = sum[e];
+    }
+  }
+  if (n_sub > 1) {
+    __syncthreads();
+    for (int c = threadIdx.x; c < y.ld; c += blockDim.x) {
+      double t = 0.0;
+      for (int k = 0; k < n_sub; ++k) t += sh[(size_t)k * y.ld + c];
+      out[c] = t;
+    }
+  }
+}
+__device__ __forceinline__ void add4(double (&s)[4], float4 v) {
+  s[0] += (double)v.x; s[1] += (double)v.y; s[2] += (double)v.z; s[3] += (double)v.w;
+}
+// column sums of a stored matrix (X, the last layer's r; r and p after the start or after the caller has set a tensor)
+struct ColSum { const float *x; RowBlocks rows; double *out; };
+__global__ void __launch_bounds__(EW_THREADS)
+colsum_kernel(const __grid_constant__ Group<ColSum> group) {
+  __shared__ double sh[EW_THREADS * 4];
+  const ColSum &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.rows.n_blocks) return;
+  const float *__restrict__ x = y.x;
+  row_block_sums(y.rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int n, int, double (&sum)[4]) {
+#pragma unroll 4
+    for (; n > 0; --n, i += stride) add4(sum, ld4(x, i));
+  });
+}
+// The slots' totals of TOTAL_COLS columns, the first column at c0: total of column c0 + thread, valid in the block's first TOTAL_COLS
+// threads.  Slot group g = thread / TOTAL_COLS adds the slots g, g + 16, ..., the groups are added in group order.
+constexpr int TOTAL_COLS = 16, TOTAL_GROUPS = EW_THREADS / TOTAL_COLS;
+__device__ __forceinline__ double slot_total(const double *__restrict__ slots, int n_slots, int ld, int c0, double (*sh)[TOTAL_COLS + 1]) {
+  const int g = threadIdx.x / TOTAL_COLS, k0 = threadIdx.x % TOTAL_COLS, c = c0 + k0;
+  double s = 0.0;
+  for (int i0 = g; c < ld && i0 < n_slots; i0 += 16 * TOTAL_GROUPS) {      // sixteen loads on their way, the last ones too
+    double v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = i0 + k * TOTAL_GROUPS < n_slots ? slots[(size_t)(i0 + k * TOTAL_GROUPS) * ld + c] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s += v[k];
+  }
+  sh[g][k0] = s;
+  __syncthreads();
+  double t = 0.0;
+  if (g == 0)
+    for (int k = 0; k < TOTAL_GROUPS; ++k) t += sh[k][k0];
+  return t;
+}
+__global__ void __launch_bounds__(EW_THREADS)
+colsum_total_kernel(const __grid_constant__ Group<ColSum> group) {
+  __shared__ double sh[TOTAL_GROUPS][TOTAL_COLS + 1];
+  const ColSum &y = group.l[blockIdx.y];
+  const int c0 = (int)blockIdx.x * TOTAL_COLS, c = c0 + (int)threadIdx.x;
+  const double t = slot_total(y.rows.slots, y.rows.n_blocks, y.rows.ld, c0, sh);
+  if (threadIdx.x < TOTAL_COLS && c < y.rows.ld) y.out[c] = t;
+}
+
 // ---- p-step of pdADMM-G ----------------------------------------------------------------------------
 // p+ = p - g/tau  (Eq. "update p") and the matching update of the linear residual, r <- r - (W g)/tau, in one launch (the
 // elements of p first, then those of r), with the planes of both for the W-gradient and G p+.  16 bytes per element and
 // matrix: read 8, write 4 and the planes 4.  (Separate passes that split r and p again cost 8 bytes more each, and the
 // products that took them fp32 ran at 0.6 of their speed.)
 struct PStep {
-  float *p; const float *g; uint32_t n4p;
+  float *p; const float *g; RowBlocks p_rows;        // with the column sums of p+ (for the b-update)
   float *r; const float *wg; uint32_t n4r;
   const float *inv_tau;
   PlaneOut pp, rp;
   uint32_t *amax_p, *amax_r;          // receive max|p|, max|r| (see commit_amax); may be null
-  int n_blocks;
+  int n_blocks_r;                     // blocks of r, after those of p
 };
 __global__ void __launch_bounds__(EW_THREADS)
 pstep_kernel(const __grid_constant__ Group<PStep> group) {
+  __shared__ double sh[EW_THREADS * 4];
   const PStep &y = group.l[blockIdx.y];
-  if ((int)blockIdx.x >= y.n_blocks) return;
+  const int block = (int)blockIdx.x - y.p_rows.n_blocks;
+  if (block >= y.n_blocks_r) return;
   const float a = *y.inv_tau;
-  const uint32_t stride = y.n_blocks * EW_THREADS, first = blockIdx.x * EW_THREADS + threadIdx.x;
-  auto pass = [&](float *__restrict__ out, const float *__restrict__ x, uint32_t n4, const PlaneOut &o, uint32_t *amax) {
-    const float scale = o.hi != nullptr ? tc_scale_of(*o.exp) : 1.f;
-    uint32_t m = 0u;
-    // four groups per pass: eight loads in flight per thread
-    for (uint32_t i = first; i < n4; i += 4 * stride) {
-      float4 v[4], w[4];
+  uint32_t m = 0u;
+  // four groups per pass: eight loads in flight per thread
+  auto pass = [&](float *__restrict__ out, const float *__restrict__ x, uint32_t i0, uint32_t step, int n, const PlaneOut &o, float scale, double *sum) {
+    float4 v[4], w[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t q = i + k * stride;
-        if (q < n4) { v[k] = ld4(out, q); w[k] = ld4(x, q); }
-      }
+    for (int k = 0; k < 4; ++k)
+      if (k < n) { v[k] = ld4(out, i0 + k * step); w[k] = ld4(x, i0 + k * step); }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t q = i + k * stride;
-        if (q >= n4) continue;
-        v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
-        v[k].z = fmaf(-a, w[k].z, v[k].z); v[k].w = fmaf(-a, w[k].w, v[k].w);
-        st4(out, q, v[k]);
-        if (o.hi != nullptr) store_planes4(o, q, v[k], scale);
-        m = max(m, abs_bits(v[k]));
-      }
+    for (int k = 0; k < 4; ++k) {
+      if (k >= n) continue;
+      v[k].x = fmaf(-a, w[k].x, v[k].x); v[k].y = fmaf(-a, w[k].y, v[k].y);
+      v[k].z = fmaf(-a, w[k].z, v[k].z); v[k].w = fmaf(-a, w[k].w, v[k].w);
+      st4(out, i0 + k * step, v[k]);
+      if (o.hi != nullptr) store_planes4(o, i0 + k * step, v[k], scale);
+      if (sum != nullptr) { sum[0] += (double)v[k].x; sum[1] += (double)v[k].y; sum[2] += (double)v[k].z; sum[3] += (double)v[k].w; }
+      m = max(m, abs_bits(v[k]));
     }
-    if (amax != nullptr) commit_amax(m, amax);
   };
-  pass(y.p, y.g, y.n4p, y.pp, y.amax_p);
-  pass(y.r, y.wg, y.n4r, y.rp, y.amax_r);
+  if (block < 0) {
+    const float scale = y.pp.hi != nullptr ? tc_scale_of(*y.pp.exp) : 1.f;
+    row_block_sums(y.p_rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int n, int, double (&sum)[4]) {
+      for (; n > 0; n -= 4, i += 4 * stride) pass(y.p, y.g, i, stride, n, y.pp, scale, sum);
+    });
+    if (y.amax_p != nullptr) commit_amax(m, y.amax_p);
+    return;
+  }
+  const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
+  const uint32_t stride = y.n_blocks_r * blockDim.x;
+  for (uint32_t i = block * blockDim.x + threadIdx.x; i < y.n4r; i += 4 * stride)
+    pass(y.r, y.wg, i, stride, (int)((y.n4r - i + stride - 1) / stride), y.rp, scale, nullptr);
+  if (y.amax_r != nullptr) commit_amax(m, y.amax_r);
 }
 
 // ---- quantised trial step ------------------------------------------------------------------------
@@ -191,82 +288,90 @@ struct QuantTrial {
   __half *pn_plane;                        // the new codes, counted from the level zero, as fp16 integers: operand plane of
                                            // p_new = (code - neg_levels) * scale; may be null
   __half *d_plane;                         // new code - old code as fp16 integers (operand plane of d)
-  uint32_t n4;
+  RowBlocks rows;                          // with the column sums of p_new (for the b-update)
   uint32_t *amax_p /* max|p_new|, may be null */, *amax_d /* max|d| */;
-  double *slots; int *done; int n_blocks;
+  double *slots; int *done;
 };
-__global__ void __launch_bounds__(EW_THREADS)
-quant_trial_kernel(const __grid_constant__ Group<QuantTrial> group, int levels, int wide_codes, int neg_levels) {
+// INTS: with integer planes (p+ and d exist as codes and planes of integers alone); WIDE: codes of two bytes.
+template <bool INTS, bool WIDE>
+__global__ void __launch_bounds__(EW_THREADS, INTS ? 5 : 3)
+quant_trial_kernel(const __grid_constant__ Group<QuantTrial> group, int levels, int neg_levels) {
   __shared__ double red[EW_THREADS / 32];
+  __shared__ double sh[EW_THREADS * 4];
   __shared__ int is_last;
   const QuantTrial &y = group.l[blockIdx.y];
-  if ((int)blockIdx.x >= y.n_blocks) return;
-  const float *__restrict__ g = y.g;
-  const void *__restrict__ codes_old = y.codes_old;
-  void *__restrict__ codes = y.codes;
-  float *__restrict__ p_new = y.p_new, *__restrict__ d = y.d;
-  __half *__restrict__ pn_plane = y.pn_plane, *__restrict__ d_plane = y.d_plane;
-  const float scale = y.scale, lo = y.lo;
-  const uint32_t n4 = y.n4;
-  uint32_t *amax_p = y.amax_p, *amax_d = y.amax_d;
-  const float inv_tau = y.sc->inv_tau, neg = (float)neg_levels;
+  if ((int)blockIdx.x >= y.rows.n_blocks) return;
+  const float scale = y.scale, lo = y.lo, inv_tau = y.sc->inv_tau, neg = (float)neg_levels;
   const Quantiser quant = make_quantiser(scale, lo, (float)(levels - 1));
   double ss = 0.0;
   unsigned long long steps2 = 0;                  // with integer planes d = (new code - old code) s: the sum of the squared integers
   uint32_t mp = 0u, md = 0u;
-  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < n4; i += y.n_blocks * EW_THREADS) {
-    const float4 gv = ld4(g, i);
-    unsigned o[4], c[4];
-    if (wide_codes) {
-      const uint2 w = reinterpret_cast<const uint2 *>(codes_old)[i];
-      o[0] = w.x & 0xffffu; o[1] = w.x >> 16; o[2] = w.y & 0xffffu; o[3] = w.y >> 16;
-    } else {
-      const uint32_t w = reinterpret_cast<const uint32_t *>(codes_old)[i];
-      o[0] = w & 0xffu; o[1] = (w >> 8) & 0xffu; o[2] = (w >> 16) & 0xffu; o[3] = w >> 24;
-    }
-    const float gx[4] = {gv.x, gv.y, gv.z, gv.w};
-    float of[4], cf[4], pv[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      of[e] = float_of(o[e]);
-      pv[e] = __fadd_rn(lo, __fmul_rn(of[e], scale));
-      cf[e] = quantise_code(quant, fmaf(-inv_tau, gx[e], pv[e]), c[e]);
-    }
-    if (wide_codes)      // more than 256 levels: 16-bit codes
-      reinterpret_cast<uint2 *>(codes)[i] = make_uint2(c[0] | c[1] << 16, c[2] | c[3] << 16);
-    else
-      reinterpret_cast<uint32_t *>(codes)[i] = c[0] | c[1] << 8 | c[2] << 16 | c[3] << 24;
-    if (pn_plane != nullptr) {
-      // integers up to 2048 are exact in fp16: the planes hold the codes (counted from the level zero) and their change
-      const __half2 a0 = __floats2half2_rn(cf[0] - neg, cf[1] - neg), a1 = __floats2half2_rn(cf[2] - neg, cf[3] - neg);
-      const __half2 e0 = __floats2half2_rn(cf[0] - of[0], cf[1] - of[1]), e1 = __floats2half2_rn(cf[2] - of[2], cf[3] - of[3]);
-      reinterpret_cast<uint2 *>(pn_plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a0), *reinterpret_cast<const uint32_t *>(&a1));
-      reinterpret_cast<uint2 *>(d_plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&e0), *reinterpret_cast<const uint32_t *>(&e1));
-      uint32_t sq = 0;                            // at most 4 * 2047^2
-#pragma unroll
-      for (int e = 0; e < 4; ++e) { const int d = (int)c[e] - (int)o[e]; sq += (uint32_t)(d * d); }
-      steps2 += sq;
-    } else {
-      float nv[4], dv[4];
+  row_block_sums(y.rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int rows, int, double (&sum)[4]) {
+    const float *__restrict__ g = y.g;
+    const void *__restrict__ codes_old = y.codes_old;
+    void *__restrict__ codes = y.codes;
+    __half *__restrict__ pn_plane = y.pn_plane, *__restrict__ d_plane = y.d_plane;
+    unsigned levels_up[4] = {0, 0, 0, 0};         // sums of the codes
+#pragma unroll 2
+    for (int n = rows; n > 0; --n, i += stride) {
+      const float4 gv = ld4(g, i);
+      unsigned o[4], c[4];
+      if (WIDE) {
+        const uint2 w = reinterpret_cast<const uint2 *>(codes_old)[i];
+        o[0] = w.x & 0xffffu; o[1] = w.x >> 16; o[2] = w.y & 0xffffu; o[3] = w.y >> 16;
+      } else {
+        const uint32_t w = reinterpret_cast<const uint32_t *>(codes_old)[i];
+        o[0] = w & 0xffu; o[1] = (w >> 8) & 0xffu; o[2] = (w >> 16) & 0xffu; o[3] = w >> 24;
+      }
+      const float gx[4] = {gv.x, gv.y, gv.z, gv.w};
+      float of[4], cf[4], pv[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        nv[e] = __fadd_rn(lo, __fmul_rn(cf[e], scale));
-        dv[e] = nv[e] - pv[e];
-        ss += (double)dv[e] * dv[e];
-        mp = max(mp, abs_bits(nv[e])); md = max(md, abs_bits(dv[e]));
+        of[e] = float_of(o[e]);
+        pv[e] = __fadd_rn(lo, __fmul_rn(of[e], scale));
+        cf[e] = quantise_code(quant, fmaf(-inv_tau, gx[e], pv[e]), c[e]);
       }
-      if (p_new != nullptr) st4(p_new, i, make_float4(nv[0], nv[1], nv[2], nv[3]));      // with integer planes p+ exists as its codes alone
-      if (d != nullptr) st4(d, i, make_float4(dv[0], dv[1], dv[2], dv[3]));
+      if (WIDE)            // more than 256 levels: 16-bit codes
+        reinterpret_cast<uint2 *>(codes)[i] = make_uint2(c[0] | c[1] << 16, c[2] | c[3] << 16);
+      else
+        reinterpret_cast<uint32_t *>(codes)[i] = c[0] | c[1] << 8 | c[2] << 16 | c[3] << 24;
+      if constexpr (INTS) {
+        // integers up to 2048 are exact in fp16: the planes hold the codes (counted from the level zero) and their change
+        const __half2 a0 = __floats2half2_rn(cf[0] - neg, cf[1] - neg), a1 = __floats2half2_rn(cf[2] - neg, cf[3] - neg);
+        const __half2 e0 = __floats2half2_rn(cf[0] - of[0], cf[1] - of[1]), e1 = __floats2half2_rn(cf[2] - of[2], cf[3] - of[3]);
+        reinterpret_cast<uint2 *>(pn_plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a0), *reinterpret_cast<const uint32_t *>(&a1));
+        reinterpret_cast<uint2 *>(d_plane)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&e0), *reinterpret_cast<const uint32_t *>(&e1));
+        uint32_t sq = 0;                          // at most 4 * 2047^2
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const int d = (int)c[e] - (int)o[e]; sq += (uint32_t)(d * d); levels_up[e] += c[e]; }
+        steps2 += sq;
+      } else {
+        float nv[4], dv[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          nv[e] = __fadd_rn(lo, __fmul_rn(cf[e], scale));
+          dv[e] = nv[e] - pv[e];
+          ss += (double)dv[e] * dv[e];
+          sum[e] += (double)nv[e];
+          mp = max(mp, abs_bits(nv[e])); md = max(md, abs_bits(dv[e]));
+        }
+        st4(y.p_new, i, make_float4(nv[0], nv[1], nv[2], nv[3]));
+        st4(y.d, i, make_float4(dv[0], dv[1], dv[2], dv[3]));
+      }
     }
-  }
-  if (pn_plane != nullptr) ss = (double)scale * (double)scale * (double)steps2;
-  if (amax_p != nullptr) { commit_amax(mp, amax_p); commit_amax(md, amax_d); }
-  const double tot = block_sum<EW_THREADS>(ss, red);
+    if constexpr (INTS) {                         // p_new = (code - neg) s
+#pragma unroll
+      for (int e = 0; e < 4; ++e) sum[e] = (double)scale * ((double)levels_up[e] - (double)rows * neg_levels);
+    }
+  });
+  if (INTS) ss = (double)scale * (double)scale * (double)steps2;
+  if (!INTS && y.amax_p != nullptr) { commit_amax(mp, y.amax_p); commit_amax(md, y.amax_d); }
+  const double tot = block_sum_any(ss, red);
   if (threadIdx.x == 0) y.slots[blockIdx.x] = tot;
-  if (!last_block(y.done, y.n_blocks, &is_last)) return;
+  if (!last_block(y.done, y.rows.n_blocks, &is_last)) return;
   double v = 0.0;
-  for (int i = threadIdx.x; i < y.n_blocks; i += EW_THREADS) v += __ldcg(y.slots + i);
-  v = block_sum<EW_THREADS>(v, red);
+  for (int i = threadIdx.x; i < y.rows.n_blocks; i += blockDim.x) v += __ldcg(y.slots + i);
+  v = block_sum_any(v, red);
   if (threadIdx.x == 0) y.sc->sum_d2 = v;
 }
 
@@ -373,13 +478,29 @@ struct GradWSum {
   float *G;
   uint32_t *amax /* max|G|, may be null */; PlaneOut planes;
   double *slots; int *done; double *sum /* ||G||^2 */; int n_blocks, remake;
+  // Blocks after these: totals of the column sums of p+ (and their change) and of r, TOTAL_COLS columns each, which the W-step takes
+  struct Totals { const double *slots; double *out, *change /* may be null */; int n_slots, ld, n_blocks; } totals[2];
 };
 __global__ void __launch_bounds__(EW_THREADS)
 reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
   __shared__ double red[EW_THREADS / 32];
   __shared__ int is_last;
+  __shared__ double sh[TOTAL_GROUPS][TOTAL_COLS + 1];
   const GradWSum &y = group.l[blockIdx.y];
-  if ((int)blockIdx.x >= y.n_blocks) return;
+  int block = (int)blockIdx.x - y.n_blocks;
+  if (block >= 0) {
+    const int which = block < y.totals[0].n_blocks ? 0 : 1;
+    if (which == 1) block -= y.totals[0].n_blocks;
+    const GradWSum::Totals &t = y.totals[which];
+    if (block >= t.n_blocks) return;
+    const double v = slot_total(t.slots, t.n_slots, t.ld, TOTAL_COLS * block, sh);
+    const int c = TOTAL_COLS * block + (int)threadIdx.x;
+    if (threadIdx.x < TOTAL_COLS && c < t.ld) {
+      if (t.change != nullptr) t.change[c] = v - t.out[c];
+      t.out[c] = v;
+    }
+    return;
+  }
   const float scale = y.planes.hi != nullptr ? tc_scale_of(*y.planes.exp) : 1.f;
   const float *__restrict__ part = y.part;
   const int n_split = y.n_split;
@@ -415,92 +536,77 @@ reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
     store_planes4(y.planes, i, __ldcg(reinterpret_cast<const float4 *>(y.G) + i), again);
 }
 
-// ---- what follows theta: W+ and r - (G p+)/theta with its column sums (for the b-update) ----------------------------------
-// W+ = W - G/theta  (Eq. "update W"), with the planes of W+: the first n_blocks_w blocks of a layer.
-// The other blocks: block b handles rows [b*rows_per_block, ...).  A thread owns one group of 4 columns (float4) and one row
-// subgroup: with ld/4 <= 128 column groups the block's 256 threads cover several rows per pass.  The row
-// subgroups' sums are combined in subgroup order, then written to slots[b][ld].
-constexpr int COLSUM_MAX_SUB = 8;
+// ---- what follows theta: W+ and b+ ----------------------------------------------------------------------------
+// W+ = W - G/theta  (Eq. "update W"), with the planes of W+: a warp per row of W.  b+ = b - mean_j r  (Eq. "update b" with the step
+// 1/(nu N), i.e. the exact minimiser), where r is the linear residual after the p- and the W-step:
+//     sum_j r = sum_j (r as the last z-update left it) + W (sum_j p+ - sum_j p) - (G sum_j p+)/theta,
+// from column sums that the kernels writing r and p kept, in double precision; the warp has the row of W and of G.  shift is the mean,
+// which the z-update subtracts.  The sum of r is that of the stored values, so what the rounding of this iteration's products leaves
+// of the mean is taken out by the next one.  (From sums of z and W+ p+ + b instead it piles up: the products round towards zero,
+// 2e-7 of their size.)  Sums of r - (G p+)/theta itself took a pass of 12 bytes per element of r, 185 us of 2.9 ms at 20 000 x 500,
+// 10 layers, and a launch more; the z-update applies G p+ now.
+// `sums`: a context that owns part of the nodes leaves its part of the sum there instead (finalize_bias_kernel follows).
+// `gp`: where G p+ is not left to the z-update, further blocks do r <- r - (G p+)/theta.
 struct ThetaStep {
-  float *W; const float *G; uint32_t n4w;
+  float *W; const float *G; int n_out, n_in, ld;
   uint32_t *amax_W /* may be null */; PlaneOut Wp;
-  float *r; const float *gp; int n_rows, ld, rows_per_block;
-  double *slots;
+  const double *p_sum, *p_change, *r_sum;
+  float *b, *shift;
+  double *sums /* may be null */;
   const LayerScalars *sc;
-  int n_blocks_w, n_blocks_r;
+  int n_blocks_w;
+  float *r; const float *gp /* may be null */; uint32_t n4r; int n_blocks_r;
 };
 __global__ void __launch_bounds__(EW_THREADS)
-theta_step_kernel(const __grid_constant__ Group<ThetaStep> group) {
-  extern __shared__ double colsum_sh[];                       // [n_sub][ld] when n_sub > 1
+theta_step_kernel(const __grid_constant__ Group<ThetaStep> group, double inv_n) {
   const ThetaStep &y = group.l[blockIdx.y];
   const float a = y.sc->inv_theta;
   if ((int)blockIdx.x < y.n_blocks_w) {
+    const int row = (int)blockIdx.x * (EW_THREADS / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const float scale = y.Wp.hi != nullptr ? tc_scale_of(*y.Wp.exp) : 1.f;
     uint32_t m = 0u;
-    for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4w; i += y.n_blocks_w * EW_THREADS) {
-      float4 v = ld4(y.W, i);
-      const float4 g = ld4(y.G, i);
-      v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
-      st4(y.W, i, v);
-      if (y.Wp.hi != nullptr) store_planes4(y.Wp, i, v, scale);
-      m = max(m, abs_bits(v));
+    double dot = 0.0;
+    if (row < y.n_out) {
+      const float bias = y.b[row];
+      const double rs = y.r_sum[row];
+      const int n4 = y.ld >> 2;
+#pragma unroll 2
+      for (int k = lane; k < n4; k += 32) {
+        const size_t i = (size_t)row * n4 + k;
+        float4 v = ld4(y.W, i);
+        const float4 g = ld4(y.G, i);
+        const double2 p0 = reinterpret_cast<const double2 *>(y.p_sum)[2 * k], p1 = reinterpret_cast<const double2 *>(y.p_sum)[2 * k + 1];
+        const double2 c0 = reinterpret_cast<const double2 *>(y.p_change)[2 * k], c1 = reinterpret_cast<const double2 *>(y.p_change)[2 * k + 1];
+        dot += ((double)v.x * c0.x + (double)v.y * c0.y) + ((double)v.z * c1.x + (double)v.w * c1.y);
+        dot -= (double)a * (((double)g.x * p0.x + (double)g.y * p0.y) + ((double)g.z * p1.x + (double)g.w * p1.y));
+        v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
+        st4(y.W, i, v);
+        if (y.Wp.hi != nullptr) store_planes4(y.Wp, i, v, scale);
+        m = max(m, abs_bits(v));
+      }
+      dot = warp_sum(dot);
+      if (lane == 0) {
+        const double sum = rs + dot;
+        if (y.sums != nullptr) {
+          y.sums[row] = sum;
+        } else {
+          const float mean = (float)(sum * inv_n);
+          y.shift[row] = mean;
+          y.b[row] = bias - mean;
+        }
+      }
     }
     if (y.amax_W != nullptr) commit_amax(m, y.amax_W);        // the next W-step bounds W by it
     return;
   }
   const int block = (int)blockIdx.x - y.n_blocks_w;
   if (block >= y.n_blocks_r) return;
-  const int ld = y.ld, n_groups = ld >> 2;
-  float *__restrict__ r = y.r;
-  const float *__restrict__ gp = y.gp;
-  const int cols_per_pass = min(n_groups, EW_THREADS);
-  const int n_sub = min(EW_THREADS / cols_per_pass, COLSUM_MAX_SUB);
-  const int sub = threadIdx.x / cols_per_pass, c0 = threadIdx.x % cols_per_pass;
-  const int r0 = block * y.rows_per_block, r1 = min(y.n_rows, r0 + y.rows_per_block);
-  double *out = y.slots + (size_t)block * ld;
-  if (sub < n_sub) {
-    for (int cg = c0; cg < n_groups; cg += cols_per_pass) {
-      double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
 #pragma unroll 4
-      for (int j = r0 + sub; j < r1; j += n_sub) {
-        const size_t o = (size_t)j * n_groups + cg;
-        float4 v = ld4(r, o);
-        const float4 g = ld4(gp, o);
-        v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
-        st4(r, o, v);
-        s0 += (double)v.x; s1 += (double)v.y; s2 += (double)v.z; s3 += (double)v.w;
-      }
-      double *dst = (n_sub > 1 ? colsum_sh + (size_t)sub * ld : out) + 4 * cg;
-      dst[0] = s0; dst[1] = s1; dst[2] = s2; dst[3] = s3;
-    }
-  }
-  if (n_sub > 1) {
-    __syncthreads();
-    for (int c = threadIdx.x; c < ld; c += EW_THREADS) {
-      double s = 0.0;
-      for (int k = 0; k < n_sub; ++k) s += colsum_sh[(size_t)k * ld + c];
-      out[c] = s;
-    }
-  }
-}
-
-// out[c] = sum over the blocks' slots of column c (the first half of finalize_bias_kernel, for a context that owns only
-// part of the nodes: the totals are then added over the shards before the mean is taken).  Same thread layout.
-constexpr int BIAS_GROUPS = 8;          // slot groups per block of the two kernels below (blockDim = (32, BIAS_GROUPS))
-__global__ void __launch_bounds__(32 * BIAS_GROUPS)
-colsum_total_kernel(const double *__restrict__ slots, int n_slots, int ld, double *__restrict__ out) {
-  __shared__ double sh[BIAS_GROUPS][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  double s = 0.0;
-  if (c < ld)
-#pragma unroll 8
-    for (int i = threadIdx.y; i < n_slots; i += BIAS_GROUPS) s += slots[(size_t)i * ld + c];
-  sh[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && c < ld) {
-    double t = 0.0;
-    for (int k = 0; k < BIAS_GROUPS; ++k) t += sh[k][threadIdx.x];
-    out[c] = t;
+  for (uint32_t i = block * EW_THREADS + threadIdx.x; i < y.n4r; i += y.n_blocks_r * EW_THREADS) {
+    float4 v = ld4(y.r, i);
+    const float4 g = ld4(y.gp, i);
+    v.x = fmaf(-a, g.x, v.x); v.y = fmaf(-a, g.y, v.y); v.z = fmaf(-a, g.z, v.z); v.w = fmaf(-a, g.w, v.w);
+    st4(y.r, i, v);
   }
 }
 
@@ -520,90 +626,108 @@ sumsq_amax_kernel(const float *__restrict__ G, size_t n4, uint32_t *__restrict__
   if (threadIdx.x == 0) slots[blockIdx.x] = tot;
 }
 
-// b+ = b - mean_j r[j][:]  (Eq. "update b" with the step 1/(nu N), i.e. the exact minimiser);
-// shift[c] = that mean, which the z-update subtracts from r.  blockDim = (32 columns, BIAS_GROUPS slot groups): group g
-// adds the slots g, g + BIAS_GROUPS, ... of its column, the group sums are then added in group order.
-struct BiasStep { const double *slots; int n_slots, ld, width; float *b, *shift; };
-__global__ void __launch_bounds__(32 * BIAS_GROUPS)
-finalize_bias_kernel(const __grid_constant__ Group<BiasStep> group, double inv_n) {
-  __shared__ double sh[BIAS_GROUPS][33];
-  const BiasStep &y = group.l[blockIdx.y];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  if (blockIdx.x * 32 >= (unsigned)y.ld) return;
-  double s = 0.0;
-  if (c < y.ld)
-#pragma unroll 8
-    for (int i = threadIdx.y; i < y.n_slots; i += BIAS_GROUPS) s += y.slots[(size_t)i * y.ld + c];
-  sh[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && c < y.ld) {
-    double t = 0.0;
-    for (int k = 0; k < BIAS_GROUPS; ++k) t += sh[k][threadIdx.x];
-    const float m = c < y.width ? (float)(t * inv_n) : 0.0f;
-    y.shift[c] = m;
-    if (c < y.width) y.b[c] -= m;
-  }
+// The same from sums that were added over the contexts of all nodes.
+__global__ void __launch_bounds__(EW_THREADS)
+finalize_bias_kernel(const double *__restrict__ sums, int width, double inv_n, float *__restrict__ b, float *__restrict__ shift) {
+  const int c = blockIdx.x * EW_THREADS + threadIdx.x;
+  if (c >= width) return;
+  const float m = (float)(sums[c] * inv_n);
+  shift[c] = m;
+  b[c] -= m;
 }
 
 // ---- z-, q-, u-update of a hidden layer, fused ----------------------------------------------------
-// a = W+ p+ + b+ = (r - shift) + z.  z+ by the ReLU closed form of Eq. "update z" (better of the two
+// a = W+ p+ + b+ = (r - (G p+)/theta - shift) + z.  z+ by the ReLU closed form of Eq. "update z" (better of the two
 // half-line minimisers; a tie keeps the non-positive one; slope > 0: leaky ReLU f(x) = slope x for x <= 0, whose
 // minimiser on z <= 0 is (a + slope q + z)/(2 + slope^2)), q+ by Eq. "update q" (q_top >= 0: projected onto
 // the level set of p_{l+1}, the variant at the end of Sec. "Quantization Extension"), residual p_{l+1} - q+,
-// u+ by Eq. "update u", the linear residual of the next iteration r = a - z+, and t_{l+1} = u+ + rho (p_{l+1} - q+),
-// the part of the next p-gradient that does not involve a product.
+// u+ by Eq. "update u", the linear residual of the next iteration r = a - z+, t_{l+1} = u+ + rho (p_{l+1} - q+),
+// the part of the next p-gradient that does not involve a product, and the column sums of that r for the next b-update.
+//
+// q is not kept: the minimiser of the q-subproblem satisfies u+ = nu (q+ - f(z+))  (Lemma "q_opt"), so q = f(z) + u/nu, and
+//     u+ = nu/(rho + nu) (rho (p - f(z+)) + u),   q+ = f(z+) + u+/nu
+// with relative errors of a few roundings of their terms, the cancelling difference p - q+ of u + rho (p - q+) avoided.  `q` is read
+// only in the first iteration after a caller has set z, q or u (which need not satisfy it); its memory holds G p+ meanwhile.
+// 40 bytes per element with that, 56 with q, and r - (G p+)/theta as a pass before: 20 000 x 500, 9 layers 825 us in two
+// kernels.  A q on the level set does not satisfy it: q_out is written and read.
 struct Zqu {
-  float *r, *z, *q, *u; const float *p_next, *shift; float *t_next;
+  float *r, *z; const float *gp /* null: r has it */; const float *q /* null: from z and u */; float *q_out /* null: not kept */;
+  float *u; const float *p_next, *shift; float *t_next;
   const void *codes_next;                 // pdADMM-G-Q: codes of p_next, read instead of it
-  float q_scale, q_lo; uint32_t ld4cols, n4;
+  float q_scale, q_lo; RowBlocks rows;
   uint32_t *amax_r;                       // max|r| (see commit_amax); may be null
   PlaneOut rp;                            // planes of r for the coming p-gradient
-  int n_blocks;
+  const LayerScalars *sc;
 };
 struct ZquParams { float rho, nu, slope, q_top; int wide_codes; float t_lo, t_step; int T, table_even; };
-__global__ void __launch_bounds__(EW_THREADS)
-zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
-  const Zqu &y = group.l[blockIdx.y];
-  if ((int)blockIdx.x >= y.n_blocks) return;
-  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
-  const float *__restrict__ p_next = y.p_next;
-  const void *__restrict__ codes_next = y.codes_next;
-  const float rho = prm.rho, nu = prm.nu, slope = prm.slope, q_top = prm.q_top, q_scale = y.q_scale, q_lo = y.q_lo;
-  const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
-  const Quantiser quant = make_quantiser(q_scale, q_lo, q_top);
-  const float inv_rn = 1.0f / (rho + nu), inv_neg = 1.0f / (2.0f + slope * slope);
-  uint32_t mr = 0u;
-  // the column group of element i is carried along (a division per element costs more than the arithmetic of the update)
-  const uint32_t stride = y.n_blocks * EW_THREADS, stride_col = stride % y.ld4cols;
-  uint32_t col = (blockIdx.x * EW_THREADS + threadIdx.x) % y.ld4cols;
-  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4; i += stride) {
-    const float4 sh = ld4(y.shift, col);
-    col += stride_col;
-    if (col >= y.ld4cols) col -= y.ld4cols;
-    const float4 rv = ld4(r, i), zv = ld4(z, i), qv = ld4(q, i), uv = ld4(u, i);
-    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
-    float4 zn, qn, un, rn, tn;
-#define PD_ZQU(f)                                                                   \
-    {                                                                               \
-      const float a = (rv.f - sh.f) + zv.f;                                         \
-      const float zneg = fminf((fmaf(slope, qv.f, a) + zv.f) * inv_neg, 0.0f);      \
-      const float zpos = fmaxf((a + qv.f + zv.f) * (1.0f / 3.0f), 0.0f);            \
-      const float qneg = qv.f - slope * zneg;                                       \
-      const float fneg = (zneg - a) * (zneg - a) + qneg * qneg + (zneg - zv.f) * (zneg - zv.f); \
-      const float fpos = (zpos - a) * (zpos - a) + (qv.f - zpos) * (qv.f - zpos) + (zpos - zv.f) * (zpos - zv.f); \
-      const float zz = fpos < fneg ? zpos : zneg;                                   \
-      float qq = (rho * pv.f + uv.f + nu * (zz > 0.0f ? zz : slope * zz)) * inv_rn; \
-      if (q_top >= 0.0f) { unsigned code; qq = quantize_one(quant, qq, code); } \
-      const float res = pv.f - qq;                                                  \
-      zn.f = zz; qn.f = qq; un.f = fmaf(rho, res, uv.f); rn.f = a - zz;             \
-      tn.f = fmaf(rho, res, un.f);                                                  \
+// what follows z+ = zz with f = f(z+): q, u and t
+template <bool LEVELS>                      // LEVELS: q may be kept on a level set
+struct QuUpdate {
+  float rho, nu, inv_nu, inv_rn, u_factor, q_top;
+  Quantiser quant;
+  __device__ __forceinline__ QuUpdate(const ZquParams &p, float q_scale, float q_lo)
+      : rho(p.rho), nu(p.nu), inv_nu(1.0f / p.nu), inv_rn(1.0f / (p.rho + p.nu)), u_factor(p.nu / (p.rho + p.nu)), q_top(p.q_top),
+        quant(LEVELS ? make_quantiser(q_scale, q_lo, p.q_top) : Quantiser{}) {}
+  __device__ __forceinline__ void operator()(float f, float p, float u, float &qn, float &un, float &tn) const {
+    if (LEVELS && q_top >= 0.0f) {
+      unsigned code;
+      qn = quantize_one(quant, (rho * p + u + nu * f) * inv_rn, code);
+      un = fmaf(rho, p - qn, u);
+    } else {
+      un = u_factor * fmaf(rho, p - f, u);
+      qn = fmaf(un, inv_nu, f);
     }
-    PD_ZQU(x) PD_ZQU(y) PD_ZQU(z) PD_ZQU(w)
-#undef PD_ZQU
-    st4(z, i, zn); st4(q, i, qn); st4(u, i, un); st4(r, i, rn); st4(t_next, i, tn);
-    if (y.rp.hi != nullptr) store_planes4(y.rp, i, rn, scale);
-    mr = max(mr, abs_bits(rn));
+    tn = fmaf(rho, p - qn, un);
   }
+};
+// GENERAL: q is read, or kept, or G p+ is in r already.  (One kernel for all took 74 registers, three blocks per SM.)
+template <bool CODES, bool GENERAL>
+__global__ void __launch_bounds__(EW_THREADS, GENERAL ? 3 : 4)
+zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
+  __shared__ double sh[EW_THREADS * 4];
+  const Zqu &y = group.l[blockIdx.y];
+  if ((int)blockIdx.x >= y.rows.n_blocks) return;
+  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q_out = y.q_out, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
+  const float *q_in = GENERAL ? y.q : nullptr;     // (may be q_out)
+  const float *__restrict__ gp = y.gp, *__restrict__ p_next = y.p_next;
+  const void *__restrict__ codes_next = y.codes_next;
+  const float slope = prm.slope, q_scale = y.q_scale, q_lo = y.q_lo, theta = !GENERAL || gp != nullptr ? y.sc->inv_theta : 0.f;
+  const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
+  const QuUpdate<GENERAL> update(prm, q_scale, q_lo);
+  const float inv_neg = 1.0f / (2.0f + slope * slope);
+  uint32_t mr = 0u;
+  row_block_sums(y.rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int n, int cg, double (&sum)[4]) {
+    const float4 sh4 = ld4(y.shift, cg);
+    for (; n > 0; --n, i += stride) {
+      float4 rv = ld4(r, i);
+      const float4 zv = ld4(z, i), uv = ld4(u, i);
+      float4 gv = make_float4(0.f, 0.f, 0.f, 0.f), qv = gv;
+      if (!GENERAL || gp != nullptr) gv = ld4(gp, i);
+      if (GENERAL && q_in != nullptr) qv = ld4(q_in, i);
+      const float4 pv = CODES ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
+      float4 zn, qn, un, rn, tn;
+#define PD_ZQU(f)                                                                   \
+      {                                                                             \
+        const float zo = zv.f, qo = GENERAL && q_in != nullptr ? qv.f : fmaf(uv.f, update.inv_nu, zo > 0.0f ? zo : slope * zo); \
+        const float a = (fmaf(-theta, gv.f, rv.f) - sh4.f) + zo;                    \
+        const float zneg = fminf((fmaf(slope, qo, a) + zo) * inv_neg, 0.0f);        \
+        const float zpos = fmaxf((a + qo + zo) * (1.0f / 3.0f), 0.0f);              \
+        const float qneg = qo - slope * zneg;                                       \
+        const float fneg = (zneg - a) * (zneg - a) + qneg * qneg + (zneg - zo) * (zneg - zo); \
+        const float fpos = (zpos - a) * (zpos - a) + (qo - zpos) * (qo - zpos) + (zpos - zo) * (zpos - zo); \
+        const float zz = fpos < fneg ? zpos : zneg;                                 \
+        update(zz > 0.0f ? zz : slope * zz, pv.f, uv.f, qn.f, un.f, tn.f);          \
+        zn.f = zz; rn.f = a - zz;                                                   \
+      }
+      PD_ZQU(x) PD_ZQU(y) PD_ZQU(z) PD_ZQU(w)
+#undef PD_ZQU
+      st4(z, i, zn); st4(u, i, un); st4(r, i, rn); st4(t_next, i, tn);
+      if (GENERAL && q_out != nullptr) st4(q_out, i, qn);
+      if (y.rp.hi != nullptr) store_planes4(y.rp, i, rn, scale);
+      add4(sum, rn);
+      mr = max(mr, abs_bits(rn));
+    }
+  });
   if (y.amax_r != nullptr) commit_amax(mr, y.amax_r);
 }
 
@@ -675,59 +799,83 @@ __device__ __forceinline__ void table_best(const float *__restrict__ f_sh, int T
     if (v < best) { best = v; z_best = z_at(i); f_best = f_sh[i]; }
   }
 }
-__global__ void __launch_bounds__(EW_THREADS)
+template <bool GENERAL>
+__global__ void __launch_bounds__(EW_THREADS, GENERAL ? 3 : 4)
 zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ ZquParams prm) {
+  __shared__ double sh[EW_THREADS * 4];
   const Zqu &y = group.l[blockIdx.y];
-  if ((int)blockIdx.x >= y.n_blocks) return;
-  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q = y.q, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
-  const float *__restrict__ p_next = y.p_next;
+  if ((int)blockIdx.x >= y.rows.n_blocks) return;
+  float *__restrict__ r = y.r, *__restrict__ z = y.z, *__restrict__ q_out = y.q_out, *__restrict__ u = y.u, *__restrict__ t_next = y.t_next;
+  const float *q_in = GENERAL ? y.q : nullptr;
+  const float *__restrict__ gp = y.gp, *__restrict__ p_next = y.p_next;
   const void *__restrict__ codes_next = y.codes_next;
-  const float rho = prm.rho, nu = prm.nu, act = prm.slope, q_top = prm.q_top, q_scale = y.q_scale, q_lo = y.q_lo;
+  const float act = prm.slope, q_scale = y.q_scale, q_lo = y.q_lo, theta = !GENERAL || gp != nullptr ? y.sc->inv_theta : 0.f;
+  const float inv_step = 1.0f / prm.t_step, top = (float)(prm.T - 1);
   const float t_lo = prm.t_lo, t_step = prm.t_step;
   const int T = prm.T;
   const bool even = prm.table_even != 0;
   extern __shared__ float table_sh[];              // f(z_i)
   for (int i = threadIdx.x; i < T; i += blockDim.x) table_sh[i] = act_eval(__fadd_rn(t_lo, __fmul_rn((float)i, t_step)), act);
   __syncthreads();
-  const Quantiser quant = make_quantiser(q_scale, q_lo, q_top);
-  const float inv_rn = 1.0f / (rho + nu);
+  const QuUpdate<GENERAL> update(prm, q_scale, q_lo);
   const float scale = y.rp.hi != nullptr ? tc_scale_of(*y.rp.exp) : 1.f;
   uint32_t mr = 0u;
-  const uint32_t stride = y.n_blocks * EW_THREADS, stride_col = stride % y.ld4cols;
-  uint32_t col = (blockIdx.x * EW_THREADS + threadIdx.x) % y.ld4cols;
-  for (uint32_t i = blockIdx.x * EW_THREADS + threadIdx.x; i < y.n4; i += stride) {
-    const float4 sh = ld4(y.shift, col);
-    col += stride_col;
-    if (col >= y.ld4cols) col -= y.ld4cols;
-    const float4 rv = ld4(r, i), zv = ld4(z, i), qv = ld4(q, i), uv = ld4(u, i);
-    const float4 pv = codes_next != nullptr ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
-    const float a[4] = {(rv.x - sh.x) + zv.x, (rv.y - sh.y) + zv.y, (rv.z - sh.z) + zv.z, (rv.w - sh.w) + zv.w};
-    const float zo[4] = {zv.x, zv.y, zv.z, zv.w}, qo[4] = {qv.x, qv.y, qv.z, qv.w};
-    float zb[4], fb[4];
+  row_block_sums(y.rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int n, int cg, double (&sum)[4]) {
+    const float4 sh4 = ld4(y.shift, cg);
+    for (; n > 0; --n, i += stride) {
+      float4 rv = ld4(r, i);
+      const float4 zv = ld4(z, i), uv = ld4(u, i);
+      if (!GENERAL || gp != nullptr) {
+        const float4 gv = ld4(gp, i);
+        rv.x = fmaf(-theta, gv.x, rv.x); rv.y = fmaf(-theta, gv.y, rv.y); rv.z = fmaf(-theta, gv.z, rv.z); rv.w = fmaf(-theta, gv.w, rv.w);
+      }
+      const float4 pv = codes_next != nullptr ? levels_of4(codes_next, prm.wide_codes, i, q_scale, q_lo) : ld4(p_next, i);
+      const float a[4] = {(rv.x - sh4.x) + zv.x, (rv.y - sh4.y) + zv.y, (rv.z - sh4.z) + zv.z, (rv.w - sh4.w) + zv.w};
+      const float zo[4] = {zv.x, zv.y, zv.z, zv.w}, uo[4] = {uv.x, uv.y, uv.z, uv.w}, pn[4] = {pv.x, pv.y, pv.z, pv.w};
+      float qo[4];
+      if (GENERAL && q_in != nullptr) {
+        const float4 qv = ld4(q_in, i);
+        qo[0] = qv.x; qo[1] = qv.y; qo[2] = qv.z; qo[3] = qv.w;
+      } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) table_best(table_sh, T, t_lo, t_step, even, act, a[e], qo[e], zo[e], zb[e], fb[e]);
-    const float pn[4] = {pv.x, pv.y, pv.z, pv.w}, uo[4] = {uv.x, uv.y, uv.z, uv.w};
-    float zn[4], qn[4], un[4], rn[4], tn[4];
+        for (int e = 0; e < 4; ++e) {
+          // f(z): from the table, as z is one of its candidates (except at the start)
+          const int k = __float2int_rn(fminf(fmaxf((zo[e] - t_lo) * inv_step, 0.0f), top));
+          const float f = __fadd_rn(t_lo, __fmul_rn((float)k, t_step)) == zo[e] ? table_sh[k] : act_eval(zo[e], act);
+          qo[e] = fmaf(uo[e], update.inv_nu, f);
+        }
+      }
+      float zn[4], fn[4], qn[4], un[4], rn[4], tn[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float qq = (rho * pn[e] + uo[e] + nu * fb[e]) * inv_rn;
-      if (q_top >= 0.0f) { unsigned code; qq = quantize_one(quant, qq, code); }
-      const float res = pn[e] - qq;
-      zn[e] = zb[e]; qn[e] = qq; un[e] = fmaf(rho, res, uo[e]); rn[e] = a[e] - zb[e];
-      tn[e] = fmaf(rho, res, un[e]);
+      for (int e = 0; e < 4; ++e) {
+        table_best(table_sh, T, t_lo, t_step, even, act, a[e], qo[e], zo[e], zn[e], fn[e]);
+        update(fn[e], pn[e], uo[e], qn[e], un[e], tn[e]);
+        rn[e] = a[e] - zn[e];
+      }
+      const float4 r4 = make_float4(rn[0], rn[1], rn[2], rn[3]);
+      st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
+      if (GENERAL && q_out != nullptr) st4(q_out, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
+      if (y.rp.hi != nullptr) store_planes4(y.rp, i, r4, scale);
+      st4(r, i, r4); st4(t_next, i, make_float4(tn[0], tn[1], tn[2], tn[3]));
+      add4(sum, r4);
+      mr = max(mr, abs_bits(r4));
     }
-    st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(q, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
-    st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
-    const float4 r4 = make_float4(rn[0], rn[1], rn[2], rn[3]);
-    if (y.rp.hi != nullptr) store_planes4(y.rp, i, r4, scale);
-    st4(r, i, r4); st4(t_next, i, make_float4(tn[0], tn[1], tn[2], tn[3]));
-    mr = max(mr, abs_bits(r4));
-  }
+  });
   if (y.amax_r != nullptr) commit_amax(mr, y.amax_r);
+}
+// q = f(z) + u/nu, for whoever wants the values
+__global__ void __launch_bounds__(EW_THREADS)
+q_of_z_and_u_kernel(const float *__restrict__ z, const float *__restrict__ u, float slope, float nu, float *__restrict__ q, size_t n4) {
+  const float inv_nu = 1.0f / nu;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 zv = ld4(z, i), uv = ld4(u, i);
+    st4(q, i, make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
+                          fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope))));
+  }
 }
 
 // ---- z-update of the last layer -------------------------------------------------------------------
-// a = (r - shift) + z.  Labelled node: z+ = argmin CE(z; y) + (nu/2)||z - a||^2
+// a = (r - (G p+)/theta - shift) + z.  Labelled node: z+ = argmin CE(z; y) + (nu/2)||z - a||^2
 // (Eq. "update zl"), the unique root of softmax(z) - e_y + nu (z - a) = 0, by damped Newton with the
 // Hessian diag(s) + nu I - s s^T inverted through the rank-one update formula; double precision
 // inside, since nu is small and the Hessian is close to singular along (1,..,1).  Unlabelled: z+ = a.
@@ -744,7 +892,8 @@ __global__ void __launch_bounds__(128)
 zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restrict__ shift,
              const int *__restrict__ labels, const uint8_t *__restrict__ mask, int n_rows, int C, int ld,
              double nu, int *__restrict__ not_converged, uint32_t *__restrict__ amax_r /* max|r|, may be null */,
-             int least_squares /* R = 1/2 ||z - e_y||^2: z+ = (e_y + nu a)/(1 + nu) */, PlaneOut rp) {
+             int least_squares /* R = 1/2 ||z - e_y||^2: z+ = (e_y + nu a)/(1 + nu) */, PlaneOut rp,
+             const float *__restrict__ gp /* null: r has it */, const LayerScalars *sc) {
   const int j = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) / G), lane = threadIdx.x % G;
   const bool row = j < n_rows;
   const size_t at = (size_t)(row ? j : n_rows - 1) * ld + 2 * lane;          // ld is a multiple of 32 and C <= 2 G
@@ -763,7 +912,11 @@ zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restri
   double a[2] = {0.0, 0.0}, x[2] = {0.0, 0.0};
 #pragma unroll
   for (int i = 0; i < 2; ++i)
-    if (in[i]) { x[i] = (double)z[at + i]; a[i] = (double)((r[at + i] - shift[c0 + i]) + z[at + i]); }
+    if (in[i]) {
+      const float rv = gp != nullptr ? fmaf(-sc->inv_theta, gp[at + i], r[at + i]) : r[at + i];
+      x[i] = (double)z[at + i];
+      a[i] = (double)((rv - shift[c0 + i]) + z[at + i]);
+    }
   const bool labelled = row && mask[j];
   const int y = labelled ? labels[j] : -1;
   const double e[2] = {c0 == y ? 1.0 : 0.0, c0 + 1 == y ? 1.0 : 0.0};
@@ -841,11 +994,12 @@ zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restri
   if (amax_r != nullptr) commit_amax(mr, amax_r);
 }
 inline void launch_zlast(cudaStream_t st, float *r, float *z, const float *shift, const int *labels, const uint8_t *mask, int n_rows,
-                         int C, int ld, double nu, int *not_converged, uint32_t *amax_r, int least_squares, const PlaneOut &rp) {
+                         int C, int ld, double nu, int *not_converged, uint32_t *amax_r, int least_squares, const PlaneOut &rp,
+                         const float *gp, const LayerScalars *sc) {
   auto go = [&](auto G) {
     constexpr int g = decltype(G)::value;
     zlast_kernel<g><<<(int)ceil_div((int64_t)n_rows * g, 128), 128, 0, st>>>(r, z, shift, labels, mask, n_rows, C, ld, nu, not_converged,
-                                                                            amax_r, least_squares, rp);
+                                                                            amax_r, least_squares, rp, gp, sc);
   };
   if (C <= 8) go(std::integral_constant<int, 4>{});
   else if (C <= 16) go(std::integral_constant<int, 8>{});
@@ -888,16 +1042,16 @@ relu_max_kernel(const float *__restrict__ z, float *__restrict__ q, size_t n4, f
 }
 
 // ---- objective pieces of all layers ---------------------------------------------------------------
-// Blocks (x, y): part x of layer y; sums r^2, (q - f(z))^2, u (p_next - q), (p_next - q)^2 (q == nullptr: only r^2), one
+// Blocks (x, y): part x of layer y; sums r^2, (q - f(z))^2, u (p_next - q), (p_next - q)^2 (u == nullptr: only r^2), one
 // slot of four per block; the block of a layer that finishes last (one counter per layer, back to zero afterwards) adds
 // the layer's slots in block order and writes the four sums to out[4 y ..] -- page-locked host memory, so that the whole
 // read-out is one launch and one wait.  Two launches, a copy and a wait per layer before: 22 launches and 11 waits on
 // ten layers of 2000 x 100 took 307 us, and scalar loads with an fp32 p_next kept the wide layers at 2.3 TB/s.
-// `parts`: OBJ_ALL, or OBJ_RESIDUALS for the last sum alone (reads q and p_next only).
+// `parts`: OBJ_ALL, or OBJ_RESIDUALS for the last sum alone.
 // 16-byte loads, p_next as its codes in pdADMM-G-Q (the same bits).
 constexpr int OBJ_MAX_LAYERS = 40;           // layers per launch: their pointers travel as a kernel argument
 enum : int { OBJ_ALL = 0, OBJ_RESIDUALS = 1 };
-struct ObjLayer { const float *r, *z, *q, *u, *p_next; const void *codes_next; size_t n4; float scale, lo; };
+struct ObjLayer { const float *r, *z, *q /* null: from z and u */, *u /* null: only r^2 */, *p_next; const void *codes_next; size_t n4; float scale, lo; };
 struct ObjLayers { ObjLayer l[OBJ_MAX_LAYERS]; };
 __device__ __forceinline__ void add_sq4(double &s, float4 v) {
   const double a = v.x, b = v.y, c = v.z, d = v.w;
@@ -905,19 +1059,27 @@ __device__ __forceinline__ void add_sq4(double &s, float4 v) {
 }
 template <int PARTS>
 __global__ void __launch_bounds__(EW_THREADS)
-objective_kernel(const __grid_constant__ ObjLayers layers, float slope, int wide_codes, double *slots, int *counters,
+objective_kernel(const __grid_constant__ ObjLayers layers, float slope, float nu, int wide_codes, double *slots, int *counters,
                  double *out) {
   __shared__ double red[EW_THREADS / 32];
   __shared__ int last;
   const ObjLayer &y = layers.l[blockIdx.y];
   double s[4] = {0, 0, 0, 0};
+  const float inv_nu = 1.0f / nu;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < y.n4; i += stride) {
-    if (y.q == nullptr) {
+    if (y.u == nullptr) {
       if (PARTS == OBJ_ALL) add_sq4(s[0], ld4(y.r, i));
       continue;
     }
-    const float4 qv = ld4(y.q, i);
+    float4 qv;
+    if (y.q != nullptr) {
+      qv = ld4(y.q, i);
+    } else {
+      const float4 zv = ld4(y.z, i), uv = ld4(y.u, i);
+      qv = make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
+                       fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope)));
+    }
     const float4 pv = y.codes_next != nullptr ? levels_of4(y.codes_next, wide_codes, i, y.scale, y.lo) : ld4(y.p_next, i);
     if (PARTS == OBJ_ALL) {
       const float4 rv = ld4(y.r, i), zv = ld4(y.z, i), uv = ld4(y.u, i);

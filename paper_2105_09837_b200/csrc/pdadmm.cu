@@ -6,7 +6,7 @@
 // updates in place instead of recomputing the product:
 //     p+ = p - g/tau        =>  r <- r - (W g)/tau            (pdADMM-G-Q: r <- r + W (p+ - p))
 //     W+ = W - G/theta      =>  r <- r - (G p+)/theta
-//     b+ = b - mean_j r     =>  r <- r - mean_j r
+//     b+ = b - mean_j r     =>  r <- r - mean_j r      (mean_j r from column sums of r and p+)
 //     z+                    =>  r <- (r + z) - z+
 // so one iteration of a layer costs four dense products: W^T r (the p-gradient), W g (tau),
 // r^T p+ (the W-gradient, contraction over the nodes) and G p+ (theta).
@@ -41,10 +41,10 @@ enum KClass {
   KC_GEMM_GP,         // G p+, squared norm
   KC_AXPY,            // p -= g/tau, r -= (Wg)/tau
   KC_QUANT,           // quantised trial step
-  KC_COLSUM,          // W -= G/theta; r -= (G p+)/theta with column sums
+  KC_COLSUM,          // W -= G/theta, b (and r -= (G p+)/theta where the z-update does not)
   KC_ZQU,             // fused z, q, u update of a hidden layer
   KC_ZLAST,           // z update of the last layer
-  KC_SMALL,           // bias from the column sums; sums of the CUDA-core products
+  KC_SMALL,           // column sums of r_L; bias of a shard; sums of the CUDA-core products
   KC_AMAX,            // largest magnitude of a product's node-sized operand (for its power-of-two scaling)
   KC_PLANES,          // fp16 planes made or made again by a kernel of their own
   KC_COUNT
@@ -105,6 +105,11 @@ struct Layer {
   int *g_exp = nullptr;     // l >= 2: exponent of the next planes of g_l
   uint32_t *amax_W = nullptr;      // max|W|, bit pattern
   float *shift = nullptr;   // [ld_out] column means removed by the b-update
+  // column sums of p_l (layer 1: X), how the last p-step changed them, and of r_l, which give the b-update; those of r as the z-update's
+  // blocks left them, too
+  double *p_sum = nullptr, *p_change = nullptr, *r_sum = nullptr, *r_slots = nullptr;
+  int p_blocks = 1, r_blocks = 1;            // blocks of the kernels that leave them
+  float *gp = nullptr;      // G p+ on its way to the z-update: the memory of q where that is not kept (c->q_implied), the last layer's own
   uint8_t *codes = nullptr; // [N][ld_in] codes of 1 byte (up to 256 levels) or 2 bytes, quantised mode, l >= 2
   __half *p_plane = nullptr; // [N][ld_in] the codes as fp16 integers: operand plane of p_l = code * scale (see int_operands)
   float scale = 1.0f;       // level spacing s_l of p_l
@@ -133,6 +138,7 @@ struct Scratch {
   float *part = nullptr;    // partial tiles of grad_W
   double *slots = nullptr;  // per-block partial sums
   size_t n_slots = 0;
+  double *p_slots = nullptr;       // column sums of p+ as the p-step's blocks left them
   double *red = nullptr;    // sums on their way through the reduction over shards (widest layer + 8 values)
   float *tail_ws = nullptr; // accumulators of the contraction slices of tail tiles (one tile per SM at most)
   int *tail_count = nullptr;
@@ -195,6 +201,12 @@ struct pdadmm_ctx {
   std::vector<cudaEvent_t> ev_lane; // [n_lanes]: fork / join
   bool r_valid = false;
   bool t_valid = false;             // every layer's t matches the stored u, p, q
+  // q_l = f(z_l) + u_l/nu after every iteration (see zqu_kernel), unless it is kept on a level set: it is not stored then, and its
+  // memory serves G p+.  After the caller has set z, q or u the stored q is read once.
+  bool q_free = false;              // the context may do without it
+  bool q_implied = false;           // z and u give it now
+  bool q_stale = false;             // the stored values are older
+  bool p_sums_valid = false, r_sums_valid = false;          // the column sums of p_l and of r_l are those of the stored values
   // Words that are zero between calls, one block so that one clear covers them: d_flag[0..3] (z_L solver non-convergence, expired
   // wait, non-finite sum, unused), the layers' `done` and w_* words, the tail counts of the lanes that cut tails.
   int *control = nullptr;
@@ -805,25 +817,45 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
   return wg([&](int l) { return EpiStoreSumsq{scratch_of(c, l).s2, c->layers[l].ld_out, c->use_tc ? c->layers[l].w_wg : nullptr}; });
 }
 
+// Blocks of a kernel that sums columns, for each of the layers of its launch; at least four rows for every row subgroup of a block
+// (2000 x 100, 9 layers: p-step 17.0 us with two, 14.9 so).  The z-update gets two full rounds of what the SMs hold at 64
+// registers a thread, four for a layer on its own: 10 000 x 256, 5 layers 122 us, with 3.3 rounds 129; 90 000 x 2000 1.28 ms a layer, with
+// two 1.33.  The p-step and the trial step 16 per SM, the
+// trial of a layer on its own 5 (one round: 170 000 x 1000 1.46 ms, 1.61 with 16).
+static int sum_blocks(const pdadmm_ctx *c, int ld, int layers, bool z) {
+  const RowShare share = row_share(ld);
+  const int per_sm = z ? (layers > 1 ? 2 : 4) * (1024 / share.threads) : c->levels && layers == 1 ? 5 : 16;
+  const int64_t blocks = std::max(1, per_sm * c->n_sms / std::max(layers, 1));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, ceil_div(c->N, 4 * share.n_sub)));
+}
+static RowBlocks row_blocks(const pdadmm_ctx *c, int ld, int blocks, double *slots) {
+  const RowShare s = row_share(ld);
+  return RowBlocks{(int)c->N, ld, blocks, slots, s.cols_per_pass, s.n_sub};
+}
+static RowBlocks p_rows(const pdadmm_ctx *c, const Layer &ly, const Scratch &s) { return row_blocks(c, ly.ld_in, ly.p_blocks, s.p_slots); }
+static RowBlocks r_rows(const pdadmm_ctx *c, const Layer &ly) { return row_blocks(c, ly.ld_out, ly.r_blocks, ly.r_slots); }
+
 // pdADMM-G: p <- p - g/tau, r <- r - (W g)/tau, and the planes of both.
 static void p_step_plain(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   Group<PStep> g;
-  int n = 0, blocks = 0;
+  int n = 0, blocks = 0, threads = 0;
   double bytes = 0;
   for (int l : batch) {
     Layer &ly = c->layers[l];
     Scratch &s = scratch_of(c, l);
-    const size_t n4p = (size_t)c->N * ly.ld_in / 4, n4r = (size_t)c->N * ly.ld_out / 4;
+    const size_t n4r = (size_t)c->N * ly.ld_out / 4;
     // a thread has eight loads in flight if it gets four groups (2000 x 100: 9 layers 18.8 us with a group per thread, 14.7 so;
     // 7013 x 333, 6 layers: 80.9 and 71.5)
-    const int nb = ew_grid((size_t)ceil_div((int64_t)std::max(n4p, n4r), 4));
-    g.l[n++] = PStep{ly.p, s.s1, (uint32_t)n4p, ly.r, s.s2, (uint32_t)n4r, &ly.sc->inv_tau, plane_out(c, s.pl1), plane_out(c, s.pl0),
-                     c->use_tc ? ly.amax_p : nullptr, c->use_tc ? ly.amax_r : nullptr, nb};
-    blocks = std::max(blocks, nb);
+    const int nb = ew_grid((size_t)ceil_div((int64_t)n4r, 4));
+    g.l[n] = PStep{ly.p, s.s1, p_rows(c, ly, s), ly.r, s.s2, (uint32_t)n4r, &ly.sc->inv_tau, plane_out(c, s.pl1),
+                   plane_out(c, s.pl0), c->use_tc ? ly.amax_p : nullptr, c->use_tc ? ly.amax_r : nullptr, nb};
+    blocks = std::max(blocks, g.l[n].p_rows.n_blocks + nb);
+    threads = std::max(threads, row_share(ly.ld_in).threads);
+    ++n;
     bytes += (c->use_tc ? 16.0 : 12.0) * c->N * (ly.n_in + ly.n_out);
   }
   Launch k(c, KC_AXPY, st, bytes, 0);
-  pstep_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g);
+  pstep_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
 }
 
 // pdADMM-G-Q: project p - g/tau on the level set, doubling tau until the stop condition holds.  Each trial ends
@@ -834,22 +866,27 @@ static int q_trial(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const int N = (int)c->N;
   {
     Group<QuantTrial> g;
-    int n = 0, blocks = 0;
+    int n = 0, blocks = 0, threads = 0;
     double bytes = 0;
     for (int l : batch) {
       Layer &ly = c->layers[l];
       Scratch &s = scratch_of(c, l);
-      const size_t n4 = (size_t)N * ly.ld_in / 4;
-      const int nb = ew_grid(n4);
+      const RowBlocks rows = p_rows(c, ly, s);
       // with integer operands p+ and d exist as codes and planes of integers alone
       g.l[n++] = QuantTrial{s.s1, ly.sc, ly.scale, ly.lo, c->int_operands ? nullptr : s.p_new, c->int_operands ? nullptr : s.d, ly.codes,
-                            s.codes_new, s.pn_plane, s.d_plane, (uint32_t)n4, c->use_tc && !c->int_operands ? ly.amax_p : nullptr,
-                            ly.w_d, s.slots, ly.done, nb};
-      blocks = std::max(blocks, nb);
+                            s.codes_new, s.pn_plane, s.d_plane, rows, c->use_tc && !c->int_operands ? ly.amax_p : nullptr,
+                            ly.w_d, s.slots, ly.done};
+      blocks = std::max(blocks, rows.n_blocks);
+      threads = std::max(threads, row_share(ly.ld_in).threads);
       bytes += (c->int_operands ? 8.0 + 2.0 * c->code_bytes : 12.0 + 2.0 * c->code_bytes) * N * ly.n_in;
     }
     Launch k(c, KC_QUANT, st, bytes, 0);
-    quant_trial_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, c->levels, c->code_bytes == 2, c->neg_levels);
+    const dim3 grid((unsigned)blocks, (unsigned)n);
+    const bool wide = c->code_bytes == 2;
+    if (c->int_operands && wide) quant_trial_kernel<true, true><<<grid, threads, 0, st>>>(g, c->levels, c->neg_levels);
+    else if (c->int_operands) quant_trial_kernel<true, false><<<grid, threads, 0, st>>>(g, c->levels, c->neg_levels);
+    else if (wide) quant_trial_kernel<false, true><<<grid, threads, 0, st>>>(g, c->levels, c->neg_levels);
+    else quant_trial_kernel<false, false><<<grid, threads, 0, st>>>(g, c->levels, c->neg_levels);
   }
   // the trial's residual r + W d is written beside r (the two trade places when the trial is taken), with ||W d||^2;
   // max|r| takes the trial's values too, which keeps it an upper bound whether or not the trial is taken
@@ -915,6 +952,7 @@ static bool remade_with_sum(const pdadmm_ctx *c, const Layer &ly) {
 // b <- b - mean_j r, shift = mean_j r.
 static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   const int N = (int)c->N;
+  const bool fused = c->q_implied;                 // the z-update applies G p+
   // p+ (layer 1: X, which never changes; pdADMM-G: planes from the p-step; pdADMM-G-Q: p+ = code * s)
   std::vector<Operand> P, R;
   for (int l : batch) {
@@ -978,7 +1016,10 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       g.l[n++] = GradWSum{s.part, ly.n_split, (uint32_t)n4, ly.gradW, c->use_tc ? ly.w_G : nullptr,
                           c->reduce != nullptr ? PlaneOut{nullptr, nullptr, nullptr} : plane_out(c, ly.Gp), s.slots, ly.done + 1,
                           &ly.sc->sum_G2, nb, remade_with_sum(c, ly)};
-      blocks = std::max(blocks, nb);
+      GradWSum &y = g.l[n - 1];
+      y.totals[0] = GradWSum::Totals{s.p_slots, ly.p_sum, ly.p_change, l > 0 ? p_rows(c, ly, s).n_blocks : 0, ly.ld_in, l > 0 ? (int)ceil_div(ly.ld_in, TOTAL_COLS) : 0};
+      y.totals[1] = GradWSum::Totals{ly.r_slots, ly.r_sum, nullptr, ly.r_blocks, ly.ld_out, (int)ceil_div(ly.ld_out, TOTAL_COLS)};
+      blocks = std::max(blocks, nb + y.totals[0].n_blocks + y.totals[1].n_blocks);
       bytes += (4.0 * (ly.n_split + 1.0) + (c->use_tc ? 4.0 : 0.0)) * ly.n_out * ly.n_in;
     }
     Launch k(c, KC_GRADW_REDUCE, st, bytes, 0);
@@ -1015,7 +1056,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       const int l = batch[i];
       Layer &ly = c->layers[l];
       Scratch &s = scratch_of(c, l);
-      Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done + 2};
+      Prod<EpiStoreSumsq> p{N, ly.n_out, ly.n_in, P[i], G[i], EpiStoreSumsq{fused ? ly.gp : s.s1, ly.ld_out}, &s, s.slots + s.n_slots / 2, ly.done + 2};
       p.wide = ly.wide_gp;
       p.step = make_step(c, ly, STEP_THETA);
       if (c->use_tc) { p.step.w_in = ly.w_G; p.step.exp_W = ly.Wp.exp; p.step.exp_r = ly.rp.exp; p.step.exp_g = ly.Gp.exp; }
@@ -1027,46 +1068,33 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   }
   {
     Group<ThetaStep> g;
-    Group<BiasStep> gb;
-    int n = 0, blocks = 0, ld_max = 0;
-    size_t sh = 0;
-    double bytes = 0, bias_bytes = 0;
+    int n = 0, blocks = 0;
+    double bytes = 0;
     for (int l : batch) {
       Layer &ly = c->layers[l];
       Scratch &s = scratch_of(c, l);
-      const size_t n4w = (size_t)ly.n_out * ly.ld_in / 4;
-      const int nbw = (int)std::min<int64_t>(ceil_div((int64_t)n4w, EW_THREADS), 2 * c->n_sms);
-      // rows in as many blocks as keep the SMs busy, at least 32 of them each (16: an iteration of 2000 x 100 1 % longer, the
-      // bias kernel reads twice as many sums)
-      const int n_blocks = (int)std::min<int64_t>(c->n_sms * 4, ceil_div(N, 32));
-      const int rows_per_block = (int)ceil_div(N, n_blocks), nbr = (int)ceil_div(N, rows_per_block);
-      const int ld4 = ly.ld_out / 4, n_sub = std::min(EW_THREADS / std::min(ld4, EW_THREADS), COLSUM_MAX_SUB);
-      if (n_sub > 1) sh = std::max(sh, (size_t)n_sub * ly.ld_out * sizeof(double));
-      g.l[n] = ThetaStep{ly.W, ly.gradW, (uint32_t)n4w, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp), ly.r, s.s1, N, ly.ld_out,
-                         rows_per_block, s.slots, ly.sc, nbw, nbr};
-      gb.l[n] = BiasStep{s.slots, nbr, ly.ld_out, ly.n_out, ly.b, ly.shift};
-      ++n;
+      const size_t n4r = (size_t)N * ly.ld_out / 4;
+      const int nbw = (int)ceil_div(ly.n_out, EW_THREADS / 32), nbr = fused ? 0 : ew_grid((size_t)ceil_div((int64_t)n4r, 4));
+      g.l[n++] = ThetaStep{ly.W, ly.gradW, ly.n_out, ly.n_in, ly.ld_in, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp),
+                           ly.p_sum, ly.p_change, ly.r_sum, ly.b, ly.shift, c->reduce != nullptr ? s.red : nullptr, ly.sc, nbw,
+                           ly.r, fused ? nullptr : s.s1, (uint32_t)n4r, nbr};
       blocks = std::max(blocks, nbw + nbr);
-      ld_max = std::max(ld_max, ly.ld_out);
-      bytes += 12.0 * N * ly.n_out + (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in;
-      bias_bytes += 8.0 * nbr * ly.ld_out;
+      bytes += (fused ? 0.0 : 12.0) * N * ly.n_out + (c->use_tc ? 16.0 : 12.0) * ly.n_out * ly.n_in;
     }
     {
       Launch k(c, KC_COLSUM, st, bytes, 0);
-      theta_step_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, sh, st>>>(g);
+      theta_step_kernel<<<dim3((unsigned)blocks, (unsigned)n), EW_THREADS, 0, st>>>(g, 1.0 / (double)c->N_total);
     }
     if (c->reduce != nullptr) {
-      // the column sums run over all nodes: this shard's sums, added over the shards, then the mean over |V|
-      for (int i = 0; i < n; ++i) {
-        Scratch &s = scratch_of(c, batch[i]);
-        BiasStep &b = gb.l[i];
-        colsum_total_kernel<<<(int)ceil_div(b.ld, 32), dim3(32, BIAS_GROUPS), 0, st>>>(b.slots, b.n_slots, b.ld, s.red);
-        PD_TRY(shard_sum(c, st, s.red, (size_t)b.ld, 1));
-        b.slots = s.red; b.n_slots = 1;
+      // the sums run over all nodes: this shard's, added over the shards, then the mean over |V|
+      for (int l : batch) {
+        Layer &ly = c->layers[l];
+        Scratch &s = scratch_of(c, l);
+        PD_TRY(shard_sum(c, st, s.red, (size_t)ly.ld_out, 1));
+        Launch k(c, KC_SMALL, st, 8.0 * ly.n_out, 0);
+        finalize_bias_kernel<<<(unsigned)ceil_div(ly.n_out, EW_THREADS), EW_THREADS, 0, st>>>(s.red, ly.n_out, 1.0 / (double)c->N_total, ly.b, ly.shift);
       }
     }
-    Launch k(c, KC_SMALL, st, bias_bytes, 0);
-    finalize_bias_kernel<<<dim3((unsigned)ceil_div(ld_max, 32), (unsigned)n), dim3(32, BIAS_GROUPS), 0, st>>>(gb, 1.0 / (double)c->N_total);
   }
   return PDADMM_OK;
 }
@@ -1074,34 +1102,53 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
 // z, q and u of hidden layers; needs p_{l+1} of this iteration.
 static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
   Group<Zqu> g;
-  int n = 0, blocks = 0;
+  int n = 0, blocks = 0, threads = 0;
   double bytes = 0;
   for (int l : batch) {
     Layer &ly = c->layers[l];
     const Layer &nx = c->layers[l + 1];
-    const size_t n4 = (size_t)c->N * ly.ld_out / 4;
-    const int nb = ew_grid(n4);
-    g.l[n++] = Zqu{ly.r, ly.z, ly.q, ly.u, nx.p, ly.shift, nx.t, c->levels ? nx.codes : nullptr, nx.scale, nx.lo, (uint32_t)ly.ld_out / 4,
-                   (uint32_t)n4, c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), nb};
-    blocks = std::max(blocks, nb);
-    bytes += ((c->levels ? 36.0 + c->code_bytes : 40.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
+    const bool fused = c->q_implied;
+    g.l[n++] = Zqu{ly.r, ly.z, fused ? ly.gp : nullptr, fused ? nullptr : ly.q, c->q_free ? nullptr : ly.q, ly.u, nx.p, ly.shift, nx.t,
+                   c->levels ? nx.codes : nullptr, nx.scale, nx.lo, r_rows(c, ly), c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), ly.sc};
+    blocks = std::max(blocks, ly.r_blocks);
+    threads = std::max(threads, row_share(ly.ld_out).threads);
+    bytes += ((c->levels ? 28.0 + c->code_bytes : 32.0) + 4.0 + (c->q_free ? 0.0 : 4.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
   }
   Launch k(c, KC_ZQU, st, bytes, 0);
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
                       c->table_step, c->table_size, c->table_even ? 1 : 0};
   const dim3 grid((unsigned)blocks, (unsigned)n);
-  if (c->table_size > 0) zqu_table_kernel<<<grid, EW_THREADS, c->table_size * sizeof(float), st>>>(g, prm);
-  else zqu_kernel<<<grid, EW_THREADS, 0, st>>>(g, prm);
+  const bool general = !(c->q_implied && c->q_free);
+  if (c->table_size > 0) {
+    const size_t sh = c->table_size * sizeof(float);
+    if (general) zqu_table_kernel<true><<<grid, threads, sh, st>>>(g, prm);
+    else zqu_table_kernel<false><<<grid, threads, sh, st>>>(g, prm);
+  } else if (c->levels) {
+    if (general) zqu_kernel<true, true><<<grid, threads, 0, st>>>(g, prm);
+    else zqu_kernel<true, false><<<grid, threads, 0, st>>>(g, prm);
+  } else {
+    if (general) zqu_kernel<false, true><<<grid, threads, 0, st>>>(g, prm);
+    else zqu_kernel<false, false><<<grid, threads, 0, st>>>(g, prm);
+  }
+}
+static void r_column_sums(pdadmm_ctx *c, cudaStream_t st, const Layer &ly) {
+  Launch k(c, KC_SMALL, st, 4.0 * c->N * ly.n_out, 0);
+  Group<ColSum> g;
+  g.l[0] = ColSum{ly.r, r_rows(c, ly), nullptr};
+  colsum_kernel<<<ly.r_blocks, row_share(ly.ld_out).threads, 0, st>>>(g);
 }
 static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
   Layer &ly = c->layers[c->L - 1];
   const int N = (int)c->N;
-  Launch k(c, KC_ZLAST, st, (c->use_tc ? 20.0 : 16.0) * N * ly.n_out, 0);
-  launch_zlast(st, ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out, ly.ld_out, (double)c->nu, c->d_flag,
-               c->use_tc ? ly.amax_r : nullptr, c->ls_risk ? 1 : 0, plane_out(c, ly.rp));
+  {
+    Launch k(c, KC_ZLAST, st, (c->use_tc ? 24.0 : 20.0) * N * ly.n_out, 0);
+    launch_zlast(st, ly.r, ly.z, ly.shift, c->labels, c->mask, N, ly.n_out, ly.ld_out, (double)c->nu, c->d_flag,
+                 c->use_tc ? ly.amax_r : nullptr, c->ls_risk ? 1 : 0, plane_out(c, ly.rp), c->q_implied ? ly.gp : nullptr, ly.sc);
+  }
+  r_column_sums(c, st, ly);
 }
 
-static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
+static int iterate_layers(pdadmm_ctx *c, bool *hit_cap) {
   const int S_all = 1 + (int)c->more_lanes.size();
   // Grouped: batches of up to S layers, one launch per kernel and batch, all on the main stream.  Otherwise one layer at a time,
   // layer l on lane l mod S; per-kernel timing wants one kernel at a time, a single lane then.
@@ -1190,6 +1237,14 @@ static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
     PD_CUDA(cudaEventRecord(c->ev_lane[i], lane(c, i).st));
     PD_CUDA(cudaStreamWaitEvent(main, c->ev_lane[i], 0));
   }
+  return PDADMM_OK;
+}
+static void iterated(pdadmm_ctx *c) {
+  if (c->q_free) c->q_implied = c->q_stale = true;
+}
+static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
+  PD_TRY(iterate_layers(c, hit_cap));
+  iterated(c);
   return PDADMM_OK;
 }
 
@@ -1428,6 +1483,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   }
   c->ls_risk = (cfg->flags & PDADMM_FLAG_LEAST_SQUARES) != 0;
   c->rho = cfg->rho; c->nu = cfg->nu; c->flags = cfg->flags;
+  c->q_free = !c->quant_q;
   c->use_tc = (cfg->flags & PDADMM_FLAG_SIMT_GEMM) == 0;
   c->int_operands = c->use_tc && c->levels >= 2 && c->levels <= 2048;
   PD_CUDA(cudaSetDevice(cfg->device));
@@ -1498,10 +1554,14 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     }
     PD_TRY(dev_alloc(c, &ly.b, (size_t)ly.ld_out));
     PD_TRY(dev_alloc(c, &ly.shift, (size_t)ly.ld_out));
+    PD_TRY(dev_alloc(c, &ly.p_sum, (size_t)ly.ld_in));
+    PD_TRY(dev_alloc(c, &ly.p_change, (size_t)ly.ld_in));
+    PD_TRY(dev_alloc(c, &ly.r_sum, (size_t)ly.ld_out));
     PD_TRY(dev_alloc(c, &ly.z, e_out));
     // quantised mode: r_l (l >= 2) trades places with the lane's buffer for the trial's r + W d, so all have one size
     PD_TRY(dev_alloc(c, &ly.r, (c->levels && l > 0) ? (size_t)N * max_out : e_out));
-    if (l + 1 < c->L) { PD_TRY(dev_alloc(c, &ly.q, e_out)); PD_TRY(dev_alloc(c, &ly.u, e_out)); }
+    if (l + 1 < c->L) { PD_TRY(dev_alloc(c, &ly.q, e_out)); PD_TRY(dev_alloc(c, &ly.u, e_out)); ly.gp = ly.q; }
+    else if (c->q_free) PD_TRY(dev_alloc(c, &ly.gp, e_out));
     if (c->levels && l > 0) PD_TRY(dev_alloc(c, &ly.codes, e_in * c->code_bytes));
     if (c->int_operands && l > 0) PD_TRY(dev_alloc(c, &ly.p_plane, e_in));
     if (l > 0) PD_TRY(dev_alloc(c, &ly.t, (size_t)N * ly.ld_in));
@@ -1560,6 +1620,15 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   // for (3000 x 300, 4 layers: 0.94 ms per iteration on one stream, 0.39 on four).
   const bool batched = small && c->use_tc;
   for (int l = 0; l < c->L; l += batched ? MAX_GROUP : 1) choose_slices(l, std::min(c->L, l + (batched ? MAX_GROUP : 1)));
+  // blocks of the kernels that sum columns (the counts of batches, whichever way the layers are queued: every way gives the same bits)
+  const int per_launch = batched ? std::max(1, std::min(c->L - 1, MAX_GROUP)) : 1;       // (no p-step of layer 1, no z_L)
+  size_t max_p_slots = 0;
+  for (Layer &ly : c->layers) {
+    ly.r_blocks = sum_blocks(c, ly.ld_out, per_launch, true);
+    PD_TRY(dev_alloc(c, &ly.r_slots, (size_t)ly.r_blocks * ly.ld_out));
+    ly.p_blocks = sum_blocks(c, ly.ld_in, per_launch, false);
+    max_p_slots = std::max(max_p_slots, (size_t)ly.p_blocks * ly.ld_in);
+  }
   // scratch
   Scratch &s = c->scr;
   const size_t bytes_before_scratch = c->bytes_handed_out;
@@ -1567,6 +1636,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   PD_TRY(dev_alloc(c, &s.s2, (size_t)N * max_out));
   if (c->levels) PD_TRY(alloc_trial_buffers(c, s, (size_t)N * max_in));
   PD_TRY(dev_alloc(c, &s.part, max_part));
+  PD_TRY(dev_alloc(c, &s.p_slots, max_p_slots, false));
   s.n_slots = std::max<size_t>((size_t)c->n_sms * 4 * max_out, 8 * (size_t)ceil_div(N, SG_BM) * ceil_div(std::max(max_in, max_out), SG_BN) + 148 * 8 * 4);
   s.n_slots *= 2;                       // two halves: consecutive reductions of one layer use different halves
   PD_TRY(dev_alloc(c, &s.slots, s.n_slots));
@@ -1600,6 +1670,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
     PD_TRY(dev_alloc(c, &x.s1, e_max));
     PD_TRY(dev_alloc(c, &x.s2, (size_t)N * max_out));
     PD_TRY(dev_alloc(c, &x.part, max_part));
+    PD_TRY(dev_alloc(c, &x.p_slots, max_p_slots, false));
     if (c->levels) PD_TRY(alloc_trial_buffers(c, x, (size_t)N * max_in));
     x.n_slots = s.n_slots;
     PD_TRY(dev_alloc(c, &x.slots, x.n_slots));
@@ -1648,6 +1719,8 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->w_planes_valid = true;
   c->amax_p_valid = true;
   c->x_planes_valid = true;
+  c->q_implied = c->q_free;                 // q = f(z), u = 0
+  c->r_sums_valid = true;                   // (allocated as zero, too)
   c->cold = 2 * c->L;
   for (const Layer &ly : c->layers)
     for (int i = 0; i < 2; ++i) {            // r_l and g_l: of an element, the column tiles of the product that reads it
@@ -1727,6 +1800,8 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
 }
 
 static int refresh_p(pdadmm_ctx *c);
+static int refresh_q(pdadmm_ctx *c);
+static int stored_q(pdadmm_ctx *c);
 
 extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
   return guarded([&]() -> int {
@@ -1734,12 +1809,13 @@ extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
     if (first_layer < 1 || first_layer > c->L) return fail(PDADMM_EINVAL, "first_layer must be in [1, %d]", c->L);
     PD_CUDA(cudaSetDevice(c->device));
     PD_TRY(refresh_p(c));
+    PD_TRY(stored_q(c));
     PD_TRY(feasible_start(c, first_layer - 1));
     PD_CUDA(cudaStreamSynchronize(c->scr.st));
     PD_CUDA(cudaGetLastError());
     // the linear residual of the restarted layers is zero by construction; everything derived from the other tensors
     // (the residual of the kept layers, t, planes, largest magnitudes) is rebuilt by the next call that needs it
-    c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false;
+    c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false; c->r_sums_valid = c->p_sums_valid = false;
     return PDADMM_OK;
   });
 }
@@ -1777,6 +1853,25 @@ static int refresh_p(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
+// q_l as stored values, from z and u where these are newer
+static int refresh_q(pdadmm_ctx *c) {
+  if (!c->q_stale) return PDADMM_OK;
+  for (int l = 0; l + 1 < c->L; ++l) {
+    Layer &ly = c->layers[l];
+    const size_t n4 = (size_t)c->N * ly.ld_out / 4;
+    q_of_z_and_u_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.z, ly.u, c->slope, c->nu, ly.q, n4);
+  }
+  PD_CUDA(cudaGetLastError());
+  c->q_stale = false;
+  return PDADMM_OK;
+}
+// z, q or u is about to be set: q need not follow from the others any more
+static int stored_q(pdadmm_ctx *c) {
+  PD_TRY(refresh_q(c));
+  c->q_implied = false;
+  return PDADMM_OK;
+}
+
 // What products read beside the stored tensors: planes of W, largest magnitudes of p, planes of X.
 static int ensure_operands(pdadmm_ctx *c) {
   if (!c->amax_p_valid || !c->t_valid || !c->r_valid) PD_TRY(refresh_p(c));
@@ -1805,6 +1900,7 @@ static int ensure_operands(pdadmm_ctx *c) {
 static int ensure_residual(pdadmm_ctx *c) {
   PD_TRY(ensure_operands(c));
   if (!c->t_valid) {
+    PD_TRY(refresh_q(c));
     for (int l = 1; l < c->L; ++l) {
       Layer &ly = c->layers[l];
       const Layer &pv = c->layers[l - 1];
@@ -1821,6 +1917,34 @@ static int ensure_residual(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
+// column sums that an iteration finds in place: of r, of p before its p-step
+static int ensure_sums(pdadmm_ctx *c) {
+  cudaStream_t st = c->scr.st;
+  if (!c->r_sums_valid)
+    for (const Layer &ly : c->layers) r_column_sums(c, st, ly);
+  c->r_sums_valid = true;
+  if (c->p_sums_valid) return PDADMM_OK;
+  PD_TRY(refresh_p(c));
+  const int S = std::min(1 + (int)c->more_lanes.size(), MAX_GROUP);        // as many as have slots of their own
+  for (int l0 = 0; l0 < c->L; l0 += S) {
+    Group<ColSum> g;
+    int n = 0, blocks = 0, threads = 0, ld = 0;
+    for (int l = l0; l < std::min(c->L, l0 + S); ++l) {
+      const Layer &ly = c->layers[l];
+      g.l[n] = ColSum{ly.p, p_rows(c, ly, lane(c, n)), ly.p_sum};
+      blocks = std::max(blocks, g.l[n].rows.n_blocks);
+      threads = std::max(threads, row_share(ly.ld_in).threads);
+      ld = std::max(ld, ly.ld_in);
+      ++n;
+    }
+    colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+    colsum_total_kernel<<<dim3((unsigned)ceil_div(ld, TOTAL_COLS), (unsigned)n), EW_THREADS, 0, st>>>(g);
+  }
+  PD_CUDA(cudaGetLastError());
+  c->p_sums_valid = true;
+  return PDADMM_OK;
+}
+
 static int finish_steps(pdadmm_ctx *c, bool hit_cap);
 
 static int run_steps(pdadmm_ctx *c, int n_iters) {
@@ -1831,6 +1955,7 @@ static int run_steps(pdadmm_ctx *c, int n_iters) {
   // the last, and a count that starts from the leftover would take incomplete sums for complete ones.
   PD_CUDA(cudaMemsetAsync(c->control, 0, c->control_words * sizeof(int), c->scr.st));
   PD_TRY(ensure_residual(c));
+  PD_TRY(ensure_sums(c));
   bool hit_cap = false;
   // pdADMM-G has no host decision inside an iteration, so after a first eager iteration the sequence of launches
   // is captured once into a CUDA graph and replayed; pointers and tensor maps never change in that mode.
@@ -1844,6 +1969,8 @@ static int run_steps(pdadmm_ctx *c, int n_iters) {
     PD_TRY(iterate_once(c, &hit_cap));
     --c->cold;
   }
+  // (the stored q is read in the first iteration after it was set: not the iteration that is captured)
+  for (; c->q_free && !c->q_implied && k < n_iters; ++k) PD_TRY(iterate_once(c, &hit_cap));
   if (may_graph && c->iter_graph == nullptr && n_iters - k > 1) {
     PD_TRY(iterate_once(c, &hit_cap));
     ++k;
@@ -1867,6 +1994,7 @@ static int run_steps(pdadmm_ctx *c, int n_iters) {
   for (; k < n_iters; ++k) {
     if (may_graph && c->iter_graph != nullptr) {
       PD_CUDA(cudaGraphLaunch(c->iter_graph, c->scr.st));
+      iterated(c);
       c->launches += c->iter_graph_launches;
     } else {
       PD_TRY(iterate_once(c, &hit_cap));
@@ -1898,7 +2026,7 @@ static int finish_steps(pdadmm_ctx *c, bool hit_cap) {
   if (c->profiling) PD_TRY(prof_collect(c));
   if (c->h_pinned[9] != 0) {
     // nothing derived from the tensors was finished either
-    c->r_valid = c->t_valid = c->w_planes_valid = c->amax_p_valid = false;
+    c->r_valid = c->t_valid = c->w_planes_valid = c->amax_p_valid = c->r_sums_valid = c->p_sums_valid = false;
     return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
   }
   if (c->h_pinned[10] != 0) return fail(PDADMM_ENUMERIC, "a non-finite value reached the gradient norms: the state holds NaN or Inf");
@@ -1922,7 +2050,7 @@ static int read_objective(pdadmm_ctx *c, int parts) {
       const Layer &ly = c->layers[l0 + i];
       const bool hidden = l0 + i + 1 < c->L;
       const Layer *nx = hidden ? &c->layers[l0 + i + 1] : nullptr;
-      o.l[i] = ObjLayer{ly.r, ly.z, hidden ? ly.q : nullptr, ly.u, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
+      o.l[i] = ObjLayer{ly.r, ly.z, hidden && !c->q_stale ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
                         (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f};
       n4_max = std::max(n4_max, o.l[i].n4);
     }
@@ -1932,8 +2060,8 @@ static int read_objective(pdadmm_ctx *c, int parts) {
                                                                                   (size_t)ceil_div(c->n_sms * 8, n))));
     const dim3 grid((unsigned)per_layer, (unsigned)n);
     double *out = c->h_results + 4 * (size_t)l0;
-    if (parts == OBJ_ALL) objective_kernel<OBJ_ALL><<<grid, EW_THREADS, 0, st>>>(o, c->slope, wide, c->scr.slots, c->done, out);
-    else objective_kernel<OBJ_RESIDUALS><<<grid, EW_THREADS, 0, st>>>(o, c->slope, wide, c->scr.slots, c->done, out);
+    if (parts == OBJ_ALL) objective_kernel<OBJ_ALL><<<grid, EW_THREADS, 0, st>>>(o, c->slope, c->nu, wide, c->scr.slots, c->done, out);
+    else objective_kernel<OBJ_RESIDUALS><<<grid, EW_THREADS, 0, st>>>(o, c->slope, c->nu, wide, c->scr.slots, c->done, out);
   }
   if (parts == OBJ_ALL) {
     const Layer &ly = c->layers[c->L - 1];
@@ -2103,6 +2231,7 @@ extern "C" int pdadmm_get_tensor(pdadmm_ctx *c, int kind, int layer, void *host_
       return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                   t.rows * t.width * t.elem, bytes);
     if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
+    if (kind == PDADMM_T_Q) PD_TRY(refresh_q(c));
     return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
   });
 }
@@ -2116,7 +2245,7 @@ static int project_p_on_its_levels(pdadmm_ctx *c, int layer) {
   if (c->int_operands) codes_to_plane_kernel<<<ew_grid(n / 4), EW_THREADS, 0, c->scr.st>>>(y.codes, c->code_bytes == 2, c->neg_levels, n / 4, y.p_plane);
   PD_CUDA(cudaGetLastError());
   PD_CUDA(cudaStreamSynchronize(c->scr.st));
-  c->r_valid = false;
+  c->r_valid = c->r_sums_valid = c->p_sums_valid = false;
   c->amax_p_valid = false;
   c->t_valid = false;
   return PDADMM_OK;
@@ -2144,9 +2273,10 @@ extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void 
     if (bytes != t.rows * t.width * t.elem)
       return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                   t.rows * t.width * t.elem, bytes);
+    if (kind == PDADMM_T_Z || kind == PDADMM_T_Q || kind == PDADMM_T_U) PD_TRY(stored_q(c));
     PD_TRY(copy_rows(c->device, c->scr.st, const_cast<void *>(host_src), t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, false));
     if (kind == PDADMM_T_X || kind == PDADMM_T_P || kind == PDADMM_T_W || kind == PDADMM_T_B || kind == PDADMM_T_Z)
-      c->r_valid = false;
+      c->r_valid = c->r_sums_valid = c->p_sums_valid = false;
     if (kind == PDADMM_T_W) c->w_planes_valid = false;
     if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->amax_p_valid = false;
     if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->x_planes_valid = false;
@@ -2299,7 +2429,7 @@ extern "C" int pdadmm_matmul(int device, int mode, int M, int N, int K, const fl
         }
         const size_t n4 = (size_t)M * ldc / 4;
         Group<GradWSum> g;
-        g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4), 0};
+        g.l[0] = GradWSum{part, n_split, (uint32_t)n4, dC, nullptr, PlaneOut{nullptr, nullptr, nullptr}, slots, done, res, ew_grid(n4), 0, {}};
         reduce_gradW_kernel<<<dim3((unsigned)ew_grid(n4), 1u), EW_THREADS, 0, st>>>(g, 1.0f);
       }
       double h = 0;

@@ -109,3 +109,36 @@ def test_refused_planes_on_wide_tiles():
     """The same as above where the product W g runs on wide tiles and splits its refused operands itself (2000 x 500: below 2^20
     elements)."""
     test_refused_planes_in_every_form_of_the_product(2000, 500, 10)
+
+
+# rows of one group of four columns, of groups that leave lanes of a block idle, of more groups than a block has threads; 8-bit codes
+# (integer operands) and 16-bit codes of more levels than those take
+@pytest.mark.parametrize("hidden,levels", [(4, 0), (33, 0), (349, 0), (1030, 16), (2050, 0), (100, 4096)])
+def test_column_sums_and_unstored_q_at_the_edges_of_a_row(hidden, levels):
+    """q is not stored between iterations (q = f(z) + u/nu): what is read back follows from z and u, and setting it to what was read
+    -- the next iteration then reads the stored q and applies G p+ in a pass of its own -- changes no bit of the iterates.  The
+    iteration in between is the oracle's, with b from the column sums."""
+    inp = synth.make_inputs(synth.small("c2", 261, feat_dim=9, hidden=hidden, n_layers=3, quant_levels=levels))
+    nu = inp.workload.nu
+    got = []
+    for set_again in (False, True):
+        ctx = B.from_inputs(inp)
+        ctx.step(3)
+        for l in (1, 2):
+            z, u, q = (ctx.get_tensor(k, l) for k in (B.T_Z, B.T_U, B.T_Q))
+            f = np.maximum(z, 0)
+            assert (np.abs(q - (f + u / np.float32(nu))) <= 4 * 2.0 ** -23 * (np.abs(f) + np.abs(u / nu))).all()
+            if set_again:
+                ctx.set_tensor(B.T_Q, l, q)
+                ctx.set_tensor(B.T_U, l, u)
+        ctx.step(2)
+        got.append(U.read_state(ctx))
+        ctx.destroy()
+    for k in got[0]:
+        assert all(np.array_equal(a, b) for a, b in zip(got[0][k], got[1][k])), k
+    prm, s, _ = U.oracle_problem(inp)
+    ctx = B.from_inputs(inp)
+    prev = U.round_state(s)
+    U.load_state(ctx, prev, levels > 0)
+    _compare_iteration(ctx, prev, prm, f"h={hidden}/m={levels}")
+    ctx.destroy()
