@@ -1,7 +1,7 @@
 // pdADMM-G / pdADMM-G-Q on one B200: context, host orchestration of one iteration, C ABI.
 //
 // Data layout (device): every N x width matrix is node-major with its leading dimension padded to a
-// multiple of 32 floats (128-byte rows) and zero padding columns.  Per layer l the context keeps p_l, z_l, q_l, u_l,
+// multiple of 16 or 32 floats (row_ld) and zero padding columns.  Per layer l the context keeps p_l, z_l, q_l, u_l,
 // W_l, b_l and the linear residual r_l = W_l p_l + b_l - z_l, which every step of the iteration
 // updates in place instead of recomputing the product:
 //     p+ = p - g/tau        =>  r <- r - (W g)/tau            (pdADMM-G-Q: r <- r + W (p+ - p))
@@ -81,9 +81,6 @@ static Operand plane_operand(const float *x, int ld, const Planes &p, const uint
   return Operand{x, ld, check, p.hi, p.lo, p.exp, check};
 }
 
-// Rows of every node-major matrix start on a 128-byte boundary (leading dimensions are multiples of 32 floats):
-// tile copies and the coalesced stores of the epilogues then move whole 32-byte sectors.
-constexpr int LD_ALIGN = 32;
 // number of lanes for the concurrency across layers (measured on workload c2: 1 lane 241.8, 2 lanes 273.3 iterations/s)
 #ifndef PDADMM_N_LANES
 #define PDADMM_N_LANES 2
@@ -251,6 +248,16 @@ struct pdadmm_ctx {
 };
 
 namespace pd {
+
+// Leading dimension of a matrix of n columns: a multiple of 32 floats (tile copies and the coalesced stores of the epilogues move
+// whole 128-byte lines), or of 16 where that leaves out at least a twenty-fifth of the padded row (whole 32-byte sectors still, of
+// the fp16 planes too): 2000 x 100 in rows of 112 instead of 128 0.1151 -> 0.1139 ms per iteration, 7013 x 333 in 336 instead of 352
+// 0.455 -> 0.441; but 170 000 x 1000 in 1008 instead of 1024 20.7 -> 21.6.  A context that owns part of the nodes keeps
+// whole lines: its gradients go over as rows of them.
+static int row_ld(const pdadmm_ctx *c, int n) {
+  const int a = round_up(n, 32), b = round_up(n, 16);
+  return c->reduce == nullptr && 25 * (a - b) >= a ? b : a;
+}
 
 // ---- allocation bookkeeping -------------------------------------------------------------------------
 // Device memory of a context.  Arrays of up to 64 MB are carved out of chunks (64 MB at first, doubling up to
@@ -1470,7 +1477,7 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   if (sharded) { c->reduce = shard->allreduce; c->reduce_user = shard->user; }
   // the graph stage works on all nodes: c->N is the whole graph until X is built
   c->device = cfg->device; c->N = Ntot; c->L = cfg->n_layers; c->d = cfg->feat_dim; c->n_blocks = cfg->n_hops + 1;
-  c->n0 = c->n_blocks * c->d; c->ld0 = round_up(c->n0, LD_ALIGN); c->C = cfg->n_classes; c->levels = cfg->quant_levels;
+  c->n0 = c->n_blocks * c->d; c->ld0 = row_ld(c, c->n0); c->C = cfg->n_classes; c->levels = cfg->quant_levels;
   c->neg_levels = cfg->quant_neg_levels; c->fixed_step = cfg->quant_step;
   c->code_bytes = cfg->quant_levels > 256 ? 2 : 1;
   c->quant_q = (cfg->flags & PDADMM_FLAG_QUANT_Q) != 0;
@@ -1530,13 +1537,13 @@ static int build(pdadmm_ctx *c, const pdadmm_config *cfg, const pdadmm_shard *sh
   c->layers.resize(c->L);
   int max_in = 0, max_out = 0;
   size_t max_part = 0;
-  for (int l = 1; l < c->L; ++l) max_in = std::max(max_in, round_up(cfg->layer_widths[l - 1], LD_ALIGN));
-  for (int l = 0; l < c->L; ++l) max_out = std::max(max_out, round_up(cfg->layer_widths[l], LD_ALIGN));
+  for (int l = 1; l < c->L; ++l) max_in = std::max(max_in, row_ld(c, cfg->layer_widths[l - 1]));
+  for (int l = 0; l < c->L; ++l) max_out = std::max(max_out, row_ld(c, cfg->layer_widths[l]));
   for (int l = 0; l < c->L; ++l) {
     Layer &ly = c->layers[l];
     ly.n_in = l == 0 ? c->n0 : cfg->layer_widths[l - 1];
     ly.n_out = cfg->layer_widths[l];
-    ly.ld_in = round_up(ly.n_in, LD_ALIGN); ly.ld_out = round_up(ly.n_out, LD_ALIGN);
+    ly.ld_in = row_ld(c, ly.n_in); ly.ld_out = row_ld(c, ly.n_out);
     max_out = std::max(max_out, ly.ld_out);
     const size_t e_out = (size_t)N * ly.ld_out;
     // quantised mode: p_l and its codes trade places with the trial buffers, so all share one size
