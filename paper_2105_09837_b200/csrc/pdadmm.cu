@@ -825,7 +825,7 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
 }
 
 // Blocks of a kernel that sums columns, for each of the layers of its launch; at least four rows for every row subgroup of a block
-// (2000 x 100, 9 layers: p-step 17.0 us with two, 14.9 so).  The z-update gets two full rounds of what the SMs hold at 64
+// (2000 x 100, 9 layers: p-step 17.0 us with two, 14.9 so), fewer where that left SMs without a second block (few layers).  The z-update gets two full rounds of what the SMs hold at 64
 // registers a thread, four for a layer on its own: 10 000 x 256, 5 layers 122 us, with 3.3 rounds 129; 90 000 x 2000 1.28 ms a layer, with
 // two 1.33.  The p-step and the trial step 16 per SM, the
 // trial of a layer on its own 5 (one round: 170 000 x 1000 1.46 ms, 1.61 with 16).
@@ -833,7 +833,9 @@ static int sum_blocks(const pdadmm_ctx *c, int ld, int layers, bool z) {
   const RowShare share = row_share(ld);
   const int per_sm = z ? (layers > 1 ? 2 : 4) * (1024 / share.threads) : c->levels && layers == 1 ? 5 : 16;
   const int64_t blocks = std::max(1, per_sm * c->n_sms / std::max(layers, 1));
-  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, ceil_div(c->N, 4 * share.n_sub)));
+  int rows = 4;
+  while (rows > 1 && layers * ceil_div(c->N, rows * share.n_sub) < 2 * c->n_sms) rows /= 2;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, ceil_div(c->N, rows * share.n_sub)));
 }
 static RowBlocks row_blocks(const pdadmm_ctx *c, int ld, int blocks, double *slots) {
   const RowShare s = row_share(ld);
@@ -1927,8 +1929,17 @@ static int ensure_residual(pdadmm_ctx *c) {
 // column sums that an iteration finds in place: of r, of p before its p-step
 static int ensure_sums(pdadmm_ctx *c) {
   cudaStream_t st = c->scr.st;
-  if (!c->r_sums_valid)
-    for (const Layer &ly : c->layers) r_column_sums(c, st, ly);
+  for (int l0 = 0; !c->r_sums_valid && l0 < c->L; l0 += MAX_GROUP) {
+    Group<ColSum> g;
+    int n = 0, blocks = 0, threads = 0;
+    for (int l = l0; l < std::min(c->L, l0 + MAX_GROUP); ++l) {
+      const Layer &ly = c->layers[l];
+      g.l[n++] = ColSum{ly.r, r_rows(c, ly), nullptr};
+      blocks = std::max(blocks, ly.r_blocks);
+      threads = std::max(threads, row_share(ly.ld_out).threads);
+    }
+    colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+  }
   c->r_sums_valid = true;
   if (c->p_sums_valid) return PDADMM_OK;
   PD_TRY(refresh_p(c));
