@@ -51,6 +51,12 @@ __device__ __forceinline__ bool last_block(int *done, int n_blocks, int *sh) {
 __device__ __forceinline__ float4 ld4(const float *p, size_t i) { return reinterpret_cast<const float4 *>(p)[i]; }
 __device__ __forceinline__ float4 ld4f(const float *p, size_t i) { return reinterpret_cast<const float4 *>(p)[i]; }
 __device__ __forceinline__ void st4(float *p, size_t i, float4 v) { reinterpret_cast<float4 *>(p)[i] = v; }
+// Of group i of a matrix with rows of `groups` groups of four, the columns that are not padding; the group with the others at zero.  For
+// what does not map zero to zero: f = sigmoid.
+__device__ __forceinline__ int columns_inside(size_t i, uint32_t groups, int width) { return width - 4 * (int)(i % groups); }
+__device__ __forceinline__ float4 keep_columns(float4 v, int inside) {
+  return make_float4(inside > 0 ? v.x : 0.f, inside > 1 ? v.y : 0.f, inside > 2 ? v.z : 0.f, inside > 3 ? v.w : 0.f);
+}
 
 // ---- final, fixed-order reduction of per-block slots -------------------------------------------
 // out[j] = sum_i slots[i * stride + j], j < n_out, i < n_slots.  One block of 256 threads: thread t adds the
@@ -654,7 +660,7 @@ struct Zqu {
   float *r, *z; const float *gp /* null: r has it */; const float *q /* null: from z and u */; float *q_out /* null: not kept */;
   float *u; const float *p_next, *shift; float *t_next;
   const void *codes_next;                 // pdADMM-G-Q: codes of p_next, read instead of it
-  float q_scale, q_lo; RowBlocks rows;
+  float q_scale, q_lo; RowBlocks rows; int width;
   uint32_t *amax_r;                       // max|r| (see commit_amax); may be null
   PlaneOut rp;                            // planes of r for the coming p-gradient
   const LayerScalars *sc;
@@ -736,6 +742,8 @@ zqu_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant__ Zqu
 // The table holds T equally spaced candidates z_i = lo + i h with f(z_i); z+ is the candidate with the smallest
 // (z - a)^2 + (q - f(z))^2 + (z - z^k)^2 (the first one if equal), element by element.  q, u, r, t as in zqu_kernel.
 // Dynamic shared memory: T floats, f(z_i).
+// Columns from the layer's width on are left at zero: the best candidate for a = q = z = 0 need not be zero (a table of 300 candidates from
+// -6 to 6 has none there, and f(0) = 1/2 for sigmoid), and t of the padding would enter ||g||^2 and with it tau.
 //
 // The candidate is found without trying them all.  The second derivative of the objective is
 // 4 + 2 f'^2 - 2 f'' (q - f) >= c = 4 - 2 max|f''| (|q| + 1), so for c > 0 (|q| < 1.59 for tanh, < 19.7 for sigmoid) the
@@ -852,6 +860,11 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
         update(fn[e], pn[e], uo[e], qn[e], un[e], tn[e]);
         rn[e] = a[e] - zn[e];
       }
+      if (4 * cg + 4 > y.width) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (4 * cg + e >= y.width) zn[e] = qn[e] = un[e] = rn[e] = tn[e] = 0.f;
+      }
       const float4 r4 = make_float4(rn[0], rn[1], rn[2], rn[3]);
       st4(z, i, make_float4(zn[0], zn[1], zn[2], zn[3])); st4(u, i, make_float4(un[0], un[1], un[2], un[3]));
       if (GENERAL && q_out != nullptr) st4(q_out, i, make_float4(qn[0], qn[1], qn[2], qn[3]));
@@ -865,12 +878,14 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
 }
 // q = f(z) + u/nu, for whoever wants the values
 __global__ void __launch_bounds__(EW_THREADS)
-q_of_z_and_u_kernel(const float *__restrict__ z, const float *__restrict__ u, float slope, float nu, float *__restrict__ q, size_t n4) {
+q_of_z_and_u_kernel(const float *__restrict__ z, const float *__restrict__ u, float slope, float nu, int width, uint32_t groups,
+                    float *__restrict__ q, size_t n4) {
   const float inv_nu = 1.0f / nu;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     const float4 zv = ld4(z, i), uv = ld4(u, i);
-    st4(q, i, make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
-                          fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope))));
+    st4(q, i, keep_columns(make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
+                                       fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope))),
+                           columns_inside(i, groups, width)));
   }
 }
 
@@ -1023,12 +1038,13 @@ gradp_const_kernel(const float *__restrict__ u, const float *__restrict__ p, con
 
 // ---- elementwise helpers of the initial forward pass ---------------------------------------------
 __global__ void __launch_bounds__(EW_THREADS)
-relu_max_kernel(const float *__restrict__ z, float *__restrict__ q, size_t n4, float slope, float *__restrict__ block_max) {
+relu_max_kernel(const float *__restrict__ z, float *__restrict__ q, size_t n4, float slope, int width, uint32_t groups, float *__restrict__ block_max) {
   __shared__ float red[EW_THREADS / 32];
   float m = 0.0f;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float4 v = ld4(z, i);
     v.x = act_eval(v.x, slope); v.y = act_eval(v.y, slope); v.z = act_eval(v.z, slope); v.w = act_eval(v.w, slope);
+    v = keep_columns(v, columns_inside(i, groups, width));
     m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
     st4(q, i, v);
   }
@@ -1051,7 +1067,7 @@ relu_max_kernel(const float *__restrict__ z, float *__restrict__ q, size_t n4, f
 // 16-byte loads, p_next as its codes in pdADMM-G-Q (the same bits).
 constexpr int OBJ_MAX_LAYERS = 40;           // layers per launch: their pointers travel as a kernel argument
 enum : int { OBJ_ALL = 0, OBJ_RESIDUALS = 1 };
-struct ObjLayer { const float *r, *z, *q /* null: from z and u */, *u /* null: only r^2 */, *p_next; const void *codes_next; size_t n4; float scale, lo; };
+struct ObjLayer { const float *r, *z, *q /* null: from z and u */, *u /* null: only r^2 */, *p_next; const void *codes_next; size_t n4; float scale, lo; int width /* 0: padding adds nothing */; uint32_t groups; };
 struct ObjLayers { ObjLayer l[OBJ_MAX_LAYERS]; };
 __device__ __forceinline__ void add_sq4(double &s, float4 v) {
   const double a = v.x, b = v.y, c = v.z, d = v.w;
@@ -1080,16 +1096,22 @@ objective_kernel(const __grid_constant__ ObjLayers layers, float slope, float nu
       qv = make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
                        fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope)));
     }
-    const float4 pv = y.codes_next != nullptr ? levels_of4(y.codes_next, wide_codes, i, y.scale, y.lo) : ld4(y.p_next, i);
+    float4 pv = y.codes_next != nullptr ? levels_of4(y.codes_next, wide_codes, i, y.scale, y.lo) : ld4(y.p_next, i);
+    int inside = 4;
+    if (y.width > 0) {                       // f(0) is not zero: q = f(z) + u/nu of the padding isn't either
+      inside = columns_inside(i, y.groups, y.width);
+      qv = keep_columns(qv, inside);
+      pv = keep_columns(pv, inside);
+    }
     if (PARTS == OBJ_ALL) {
       const float4 rv = ld4(y.r, i), zv = ld4(y.z, i), uv = ld4(y.u, i);
       add_sq4(s[0], rv);
-#define PD_OBJ(f)                                                                  \
+#define PD_OBJ(f, k)                                                               \
       {                                                                            \
-        const double q = qv.f, act = act_eval(zv.f, slope), res = (double)pv.f - q; \
+        const double q = qv.f, act = k < inside ? act_eval(zv.f, slope) : 0.f, res = (double)pv.f - q; \
         s[1] += (q - act) * (q - act); s[2] += (double)uv.f * res; s[3] += res * res; \
       }
-      PD_OBJ(x) PD_OBJ(y) PD_OBJ(z) PD_OBJ(w)
+      PD_OBJ(x, 0) PD_OBJ(y, 1) PD_OBJ(z, 2) PD_OBJ(w, 3)
 #undef PD_OBJ
     } else {
       const double a = (double)pv.x - qv.x, b = (double)pv.y - qv.y, c = (double)pv.z - qv.z, d = (double)pv.w - qv.w;

@@ -1118,7 +1118,7 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     const Layer &nx = c->layers[l + 1];
     const bool fused = c->q_implied;
     g.l[n++] = Zqu{ly.r, ly.z, fused ? ly.gp : nullptr, fused ? nullptr : ly.q, c->q_free ? nullptr : ly.q, ly.u, nx.p, ly.shift, nx.t,
-                   c->levels ? nx.codes : nullptr, nx.scale, nx.lo, r_rows(c, ly), c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), ly.sc};
+                   c->levels ? nx.codes : nullptr, nx.scale, nx.lo, r_rows(c, ly), ly.n_out, c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), ly.sc};
     blocks = std::max(blocks, ly.r_blocks);
     threads = std::max(threads, row_share(ly.ld_out).threads);
     bytes += ((c->levels ? 28.0 + c->code_bytes : 32.0) + 4.0 + (c->q_free ? 0.0 : 4.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
@@ -1436,7 +1436,7 @@ static int feasible_start(pdadmm_ctx *c, int first) {
     const size_t n4 = (size_t)N * ly.ld_out / 4;
     const int grid = ew_grid(n4);
     float *bm = reinterpret_cast<float *>(s.slots);
-    relu_max_kernel<<<grid, EW_THREADS, 0, st>>>(ly.z, ly.q, n4, c->slope, bm);
+    relu_max_kernel<<<grid, EW_THREADS, 0, st>>>(ly.z, ly.q, n4, c->slope, ly.n_out, (uint32_t)ly.ld_out / 4, bm);
     if (c->levels) {
       std::vector<float> hm(grid);
       PD_CUDA(cudaMemcpyAsync(hm.data(), bm, grid * sizeof(float), cudaMemcpyDeviceToHost, st));
@@ -1868,7 +1868,7 @@ static int refresh_q(pdadmm_ctx *c) {
   for (int l = 0; l + 1 < c->L; ++l) {
     Layer &ly = c->layers[l];
     const size_t n4 = (size_t)c->N * ly.ld_out / 4;
-    q_of_z_and_u_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.z, ly.u, c->slope, c->nu, ly.q, n4);
+    q_of_z_and_u_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.z, ly.u, c->slope, c->nu, ly.n_out, (uint32_t)ly.ld_out / 4, ly.q, n4);
   }
   PD_CUDA(cudaGetLastError());
   c->q_stale = false;
@@ -2069,7 +2069,8 @@ static int read_objective(pdadmm_ctx *c, int parts) {
       const bool hidden = l0 + i + 1 < c->L;
       const Layer *nx = hidden ? &c->layers[l0 + i + 1] : nullptr;
       o.l[i] = ObjLayer{ly.r, ly.z, hidden && !c->q_stale ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
-                        (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f};
+                        (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f,
+                         hidden && c->slope == ACT_SIGMOID ? ly.n_out : 0, (uint32_t)ly.ld_out / 4};
       n4_max = std::max(n4_max, o.l[i].n4);
     }
     // all layers side by side: about eight blocks per SM altogether, as many slots as the buffer holds

@@ -7,6 +7,9 @@ import pytest
 
 from paper_2105_09837_b200 import binding as B
 from paper_2105_09837_b200 import synth
+import oracle.pdadmm_oracle as o
+import parity_util as U
+from test_gpu_parity import _compare_iteration
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +88,31 @@ def test_a_table_finer_than_the_numbers_it_holds(act, lo, r, T):
         h = fma(d0, d0, fma(d1, d1, d2 * d2))
         want, best = np.where(h < best, pts[i], want), np.minimum(h, best)
     assert np.array_equal(z, want)
+
+
+# a table without a candidate at zero, and f with f(0) = 1/2; rows of 37 columns lie in rows of 48, of 250 in rows of 256
+@pytest.mark.parametrize("name,code,T,hidden,levels,neg,step", [("tanh", 1, 300, 37, 0, 0, 0.0), ("sigmoid", 2, 300, 250, 0, 0, 0.0),
+                                                                ("sigmoid", 2, 301, 37, 64, 0, 0.0), ("tanh", 1, 300, 37, 33, 16, 0.0625)])
+def test_padding_adds_nothing_to_tau_objective_and_residuals(name, code, T, hidden, levels, neg, step):
+    """After three iterations the device's own state goes through one more on both sides: p, tau and the rest as in every parity test;
+    then objective and residuals of the state that the device holds.  A squared difference p - q carries 2^-23 |q| / |p - q| of itself: 1e-4
+    where p and q agree to three digits."""
+    inp = synth.make_inputs(synth.small("c2", 700, feat_dim=9, hidden=hidden, n_layers=4, quant_levels=levels))
+    table = (T, -6.0, 6.0)
+    prm, prev, _ = U.oracle_problem(inp, neg_levels=neg, step=step, activation=name, table=table)
+    ctx = B.from_inputs(inp, quant_neg_levels=neg, quant_step=step, activation=code, table=table)
+
+    def held():
+        s = prev.copy()
+        for k, v in U.read_state(ctx).items():
+            setattr(s, k, v)
+        if levels:
+            s.scale = [prev.scale[0]] + [float(ctx.get_tensor(B.T_QSCALE, l)[0]) for l in range(2, 5)]
+        return s
+    ctx.step(3)
+    _compare_iteration(ctx, held(), prm, f"{name}/{T}/m={levels}")
+    s = held()
+    want = o.objective(s, prm)
+    assert np.allclose(ctx.objective(), want, rtol=1e-4, atol=1e-6 * abs(want[5]))
+    assert np.allclose(ctx.residuals(), o.residuals_sq(s), rtol=1e-4)
+    ctx.destroy()
