@@ -285,6 +285,12 @@ int pdadmm_matmul_tn_static(int device, int M, int N, int K, const float *dA, in
                             float *dC, void *stream);
 
 /*
+ * pdadmm_product_forms -- how many dense products the calling host thread has launched on the tensor cores so far (not counting
+ * replays of a captured iteration): out = { all, those on 256 x 256 tiles, those that cut the tiles of a partly filled last round }.
+ */
+int pdadmm_product_forms(int64_t out[3]);
+
+/*
  * pdadmm_selftest_bounded_wait -- exercises the error path of PDADMM_ETIMEOUT without any faulty input: one warp
  * waits, with the wait routine of the tensor-core products, on a barrier that nothing arrives at; the wait gives up
  * after about limit_cycles SM cycles (1 .. 1e8), the kernel raises the products' error word and returns by itself.

@@ -30,7 +30,7 @@ OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT, ENUMERIC, ENOTCONV = 0, -1, -2, -3, -4, -5,
 EXPORTS = [
     "pdadmm_init", "pdadmm_init_sharded", "pdadmm_comm_bytes", "pdadmm_start_layers_from", "pdadmm_step", "pdadmm_last_step_ms", "pdadmm_objective", "pdadmm_residuals", "pdadmm_get_tensor",
     "pdadmm_set_tensor", "pdadmm_predict", "pdadmm_quantize", "pdadmm_spmm", "pdadmm_matmul", "pdadmm_matmul_tn_static", "pdadmm_selftest_bounded_wait", "pdadmm_selftest_expired_wait",
-    "pdadmm_profile", "pdadmm_profile_classes",
+    "pdadmm_product_forms", "pdadmm_profile", "pdadmm_profile_classes",
     "pdadmm_profile_name", "pdadmm_profile_read", "pdadmm_launches", "pdadmm_time_augmentation", "pdadmm_destroy", "pdadmm_release_cached_memory", "pdadmm_last_error",
 ]
 
@@ -92,6 +92,7 @@ def lib() -> C.CDLL:
         L.pdadmm_matmul_tn_static.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_int,
                                               C.c_void_p, C.c_void_p]
         L.pdadmm_selftest_expired_wait.argtypes = [C.c_void_p]
+        L.pdadmm_product_forms.argtypes = [C.POINTER(C.c_int64)]
         L.pdadmm_selftest_bounded_wait.argtypes = [C.c_int, C.c_longlong, C.POINTER(C.c_longlong)]
         L.pdadmm_profile.argtypes = [C.c_void_p, C.c_int]
         L.pdadmm_profile_name.argtypes = [C.c_int]
@@ -311,6 +312,13 @@ def spmm(row_ptr, col_idx, val, x, device: int = 0) -> np.ndarray:
                              v.ctypes.data_as(C.c_void_p), a.ctypes.data_as(C.c_void_p), a.shape[1],
                              y.ctypes.data_as(C.c_void_p)))
     return y
+
+
+def product_forms():
+    """``pdadmm_product_forms``: tensor-core products launched by this thread (all, on wide tiles, with cut tail tiles)."""
+    out = (C.c_int64 * 3)()
+    _check(lib().pdadmm_product_forms(out))
+    return tuple(out)
 
 
 def matmul(mode: int, A, B, flags: int = 0, device: int = 0):

@@ -224,9 +224,8 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done_empty + TC_ACC_WARPS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *skip_flag = abort_flag + 1;           // an earlier block gave up: this one does no work
-  // wide: arrivals of accumulate warps at the end of a layer, of all layers; the layers that the block completed; set when every layer
-  // but the last is counted
-  int *layers_left = reinterpret_cast<int *>(tmem_slot + 3);
+  // wide: the layers that the block completed, but for the last one; set when every layer but the last is counted
+  int *layers_done = reinterpret_cast<int *>(tmem_slot + 3);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_rank() : 0u;
@@ -252,7 +251,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       ptx::mbar_init(&done_empty[w], 1);
     }
     *abort_flag = 0;
-    layers_left[0] = layers_left[1] = layers_left[2] = 0;
+    layers_done[0] = layers_done[1] = 0;
     ptx::fence_barrier_init();
   }
   if (warp == 1) ptx::tmem_alloc<CG>(tmem_slot, TC_TMEM_COLS);
@@ -262,12 +261,13 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
   __shared__ int lay_exp[TC_MAX_GROUP][2];
   __shared__ double team_scratch[1 + READERS];
   __shared__ int lay_split[TC_MAX_GROUP];             // bit 0: A has to be split here, bit 1: B has
+  __shared__ int lay_left[TC_MAX_GROUP];              // wide: accumulate warps that have left the layer
   if (warp == 2 && lane < grp.n) {
     const TcLayer<Epi> &y = grp.l[lane];
     const int begin = lane > 0 ? grp.unit_end[lane - 1] : 0, end = grp.unit_end[lane];
     bool has_unit = false;
     for (int k = begin / unit_step; k * unit_step < end && !has_unit; ++k) has_unit = unit_of(k) >= begin && unit_of(k) < end;
-    lay_split[lane] = 0;
+    lay_split[lane] = lay_left[lane] = 0;
     if (has_unit) {
       const int ea = y.oa.exp ? *y.oa.exp : 0, eb = y.ob.exp ? *y.ob.exp : 0;
       const uint32_t ma = y.oa.amax ? *y.oa.amax : 0u, mb = y.ob.amax ? *y.ob.amax : 0u;
@@ -515,17 +515,18 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       // and notes the layers that this completes; the accumulate warps add those layers' slots at the end.  (With the accumulate
       // warps counting, and waiting for one another, at every change of layer the tensor cores stood still; with warp 3
       // adding the slots as well one block became the last of every layer, one after the other.)
-      int left = 0, visited = 0;
+      // A count for each layer, not a barrier: the accumulate warps may be several layers ahead, and ahead of one another (by the two
+      // accumulators, which is two layers where a layer's tile is one read-out), so that in a common count the arrivals of warps that
+      // are ahead would stand for those of one that has not written its sums yet.
+      int visited = 0;
       auto leave = [&](int g) {
-        left += TC_WIDE_WARPS;
         const long long t0 = clock64();
-        // (a count, not a barrier: the accumulate warps may be several layers ahead)
-        while (*reinterpret_cast<volatile int *>(layers_left) < left) {
+        while (*reinterpret_cast<volatile int *>(lay_left + g) < TC_WIDE_WARPS) {
           if (*abort_flag) return false;
           if (clock64() - t0 > 1000000000ll) { *abort_flag = 1; return false; }
           __nanosleep(100);
         }
-        if (lane == 0 && count_units(g, visited)) layers_left[1] |= 1 << g;
+        if (lane == 0 && count_units(g, visited)) layers_done[0] |= 1 << g;
         return true;
       };
       int s = 0, it = 0;
@@ -568,7 +569,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
       }
       if (counts && ok && lane == 0) {
         __threadfence_block();
-        *reinterpret_cast<volatile int *>(layers_left + 2) = 1;
+        *reinterpret_cast<volatile int *>(layers_done + 1) = 1;
       }
     }
   } else if constexpr (WIDE) {
@@ -599,10 +600,10 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
         int mask = grp.l[g_last].slots != nullptr && count_units(g_last, visited) ? 1 << g_last : 0;
         if (grp.n > 1) {
           const long long t0 = clock64();
-          while (*reinterpret_cast<volatile int *>(layers_left + 2) == 0 && !*abort_flag)
+          while (*reinterpret_cast<volatile int *>(layers_done + 1) == 0 && !*abort_flag)
             if (clock64() - t0 > 1000000000ll) *abort_flag = 1;
           __threadfence();
-          mask |= *reinterpret_cast<volatile int *>(layers_left + 1);
+          mask |= *reinterpret_cast<volatile int *>(layers_done);
         }
         *mask_sh = *abort_flag ? 0 : mask;
       }
@@ -645,7 +646,7 @@ gemm_tc_kernel(const __grid_constant__ TcGroup<Epi> grp) {
           __syncwarp();
           if (lane == 0) {
             __threadfence_block();
-            atomicAdd(layers_left, 1);
+            atomicAdd(lay_left + g_before, 1);
           }
         }
       }

@@ -415,6 +415,9 @@ struct Prod {
   size_t stride = 0;               // floats between the partial outputs of two slices
   bool wide = false;               // may run on wide tiles, and is to (see choose_wide)
 };
+// Products that this host thread has launched on the tensor cores: all, on wide tiles, with the last round's tiles cut
+// (pdadmm_product_forms)
+static thread_local int64_t product_forms[3] = {0, 0, 0};
 template <int LAYOUT, class Epi, int ZERO, bool PAIR, bool WIDE>
 static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &grp) {
   auto kern = gemm_tc_kernel<LAYOUT, Epi, ZERO, PAIR, WIDE>;
@@ -445,6 +448,11 @@ static int launch_tc_form(pdadmm_ctx *c, cudaStream_t st, const TcGroup<Epi> &gr
   cfg.attrs = &a;
   cfg.numAttrs = PAIR ? 1 : 0;
   PD_CUDA(cudaLaunchKernelEx(&cfg, kern, grp));
+  bool cut = false;
+  for (int i = 0; i < grp.n; ++i) cut |= grp.l[i].tail_split > 1;
+  product_forms[0] += 1;
+  product_forms[1] += WIDE ? 1 : 0;
+  product_forms[2] += cut ? 1 : 0;
   return PDADMM_OK;
 }
 // Whether products run on pairs of SMs: pairs halve the traffic of B, but a pair's tile has
@@ -1827,6 +1835,12 @@ extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
     c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false; c->r_sums_valid = c->p_sums_valid = false;
     return PDADMM_OK;
   });
+}
+
+extern "C" int pdadmm_product_forms(int64_t out[3]) {
+  if (!out) return fail(PDADMM_EINVAL, "out is null");
+  for (int i = 0; i < 3; ++i) out[i] = product_forms[i];
+  return PDADMM_OK;
 }
 
 extern "C" int pdadmm_release_cached_memory(int device) {

@@ -142,3 +142,34 @@ def test_column_sums_and_unstored_q_at_the_edges_of_a_row(hidden, levels):
     U.load_state(ctx, prev, levels > 0)
     _compare_iteration(ctx, prev, prm, f"h={hidden}/m={levels}")
     ctx.destroy()
+
+
+def test_norms_of_many_wide_layers_of_one_tile_each():
+    """Thirteen layers of 2000 x 512 in one launch: a pair of SMs has one wide tile of each of up to three layers, and a tile of the norm-only product
+    is a single read-out of its accumulator, so warps run ahead of one another by whole layers.  ||W g||^2 of every layer has all of its
+    512 parts: a missing one, or one of an earlier product, moves tau by 2e-3 of itself (g from the oracle's formula in 64 bits on the
+    device's own state: 1e-5 with one fp16 plane, averaged over 10^6 squares).  Every run gives the same bits."""
+    inp = synth.make_inputs(synth.small("c2", 2000, feat_dim=20, hidden=512, n_layers=14, quant_levels=16))
+    prm, s, _ = U.oracle_problem(inp)
+    bits = []
+    for run in range(3):
+        ctx = B.from_inputs(inp)
+        taus = []
+        for it in range(4):
+            if run == 0 and it == 3:
+                for k, v in U.read_state(ctx).items():
+                    setattr(s, k, v)
+            before = B.product_forms()
+            ctx.step(1)
+            # ||W g||^2; the W-gradient and G p+, which take X and integers in launches of their own
+            assert B.product_forms()[1] - before[1] == 5
+            taus.append([float(ctx.get_tensor(B.T_TAU, l)[0]) for l in range(2, 15)])
+        bits.append(taus)
+        if run == 0:
+            for l in range(1, 14):
+                g = o.grad_p_phi(s.p[l], s.W[l], s.b[l], s.z[l], prm.nu, s.q[l - 1], s.u[l - 1], prm.rho)
+                first = prm.rho + prm.nu * np.sum((s.W[l] @ g) ** 2) / np.sum(g ** 2)
+                trials = int(ctx.get_tensor(B.T_TRIALS, l + 1)[0])
+                assert abs(taus[-1][l - 1] / 2.0 ** (trials - 1) - first) <= 2e-4 * first, l
+        ctx.destroy()
+    assert bits[0] == bits[1] == bits[2]
