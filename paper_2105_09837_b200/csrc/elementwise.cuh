@@ -653,7 +653,7 @@ finalize_bias_kernel(const double *__restrict__ sums, int width, double inv_n, f
 // q is not kept: the minimiser of the q-subproblem satisfies u+ = nu (q+ - f(z+))  (Lemma "q_opt"), so q = f(z) + u/nu, and
 //     u+ = nu/(rho + nu) (rho (p - f(z+)) + u),   q+ = f(z+) + u+/nu
 // with relative errors of a few roundings of their terms, the cancelling difference p - q+ of u + rho (p - q+) avoided.  `q` is read
-// only in the first iteration after a caller has set z, q or u (which need not satisfy it); its memory holds G p+ meanwhile.
+// only in the first iteration after a caller has set z, q or u (which need not satisfy it), and written then; its memory holds G p+ otherwise.
 // 40 bytes per element with that, 56 with q, and r - (G p+)/theta as a pass before: 20 000 x 500, 9 layers 825 us in two
 // kernels.  A q on the level set does not satisfy it: q_out is written and read.
 struct Zqu {

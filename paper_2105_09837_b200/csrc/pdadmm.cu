@@ -199,7 +199,8 @@ struct pdadmm_ctx {
   bool r_valid = false;
   bool t_valid = false;             // every layer's t matches the stored u, p, q
   // q_l = f(z_l) + u_l/nu after every iteration (see zqu_kernel), unless it is kept on a level set: it is not stored then, and its
-  // memory serves G p+.  After the caller has set z, q or u the stored q is read once.
+  // memory serves G p+.  After the caller has set z, q or u the stored q is read once (and written, so that it is the layer's q wherever
+  // that iteration ends).
   bool q_free = false;              // the context may do without it
   bool q_implied = false;           // z and u give it now
   bool q_stale = false;             // the stored values are older
@@ -1125,11 +1126,11 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     Layer &ly = c->layers[l];
     const Layer &nx = c->layers[l + 1];
     const bool fused = c->q_implied;
-    g.l[n++] = Zqu{ly.r, ly.z, fused ? ly.gp : nullptr, fused ? nullptr : ly.q, c->q_free ? nullptr : ly.q, ly.u, nx.p, ly.shift, nx.t,
+    g.l[n++] = Zqu{ly.r, ly.z, fused ? ly.gp : nullptr, fused ? nullptr : ly.q, fused ? nullptr : ly.q, ly.u, nx.p, ly.shift, nx.t,
                    c->levels ? nx.codes : nullptr, nx.scale, nx.lo, r_rows(c, ly), ly.n_out, c->use_tc ? ly.amax_r : nullptr, plane_out(c, ly.rp), ly.sc};
     blocks = std::max(blocks, ly.r_blocks);
     threads = std::max(threads, row_share(ly.ld_out).threads);
-    bytes += ((c->levels ? 28.0 + c->code_bytes : 32.0) + 4.0 + (c->q_free ? 0.0 : 4.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
+    bytes += ((c->levels ? 28.0 + c->code_bytes : 32.0) + 4.0 + (fused ? 0.0 : 4.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
   }
   Launch k(c, KC_ZQU, st, bytes, 0);
   const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
@@ -1256,10 +1257,16 @@ static int iterate_layers(pdadmm_ctx *c, bool *hit_cap) {
   }
   return PDADMM_OK;
 }
+// An iteration with q_implied puts G p+ where q is, and may end early (a reduction over shards that fails): z and u give q before and
+// after the z-update of every layer.
+static void will_iterate(pdadmm_ctx *c) {
+  if (c->q_implied) c->q_stale = true;
+}
 static void iterated(pdadmm_ctx *c) {
   if (c->q_free) c->q_implied = c->q_stale = true;
 }
 static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
+  will_iterate(c);
   PD_TRY(iterate_layers(c, hit_cap));
   iterated(c);
   return PDADMM_OK;
@@ -2025,6 +2032,7 @@ static int run_steps(pdadmm_ctx *c, int n_iters) {
   }
   for (; k < n_iters; ++k) {
     if (may_graph && c->iter_graph != nullptr) {
+      will_iterate(c);
       PD_CUDA(cudaGraphLaunch(c->iter_graph, c->scr.st));
       iterated(c);
       c->launches += c->iter_graph_launches;

@@ -154,6 +154,52 @@ def test_shard_arguments_are_checked():
         B.from_inputs(inp, shard=(0, 30, B.ALLREDUCE_FN()))                    # part of the graph, no callback
 
 
+def _failing_reduction():
+    """(callback of a single shard, state): call number state[\"fail_at\"] from now on returns an error, the others are the identity."""
+    state = {"fail_at": 0}
+
+    def cb(user, buf, count, dtype, op, stream):
+        state["fail_at"] -= 1
+        return 1 if state["fail_at"] == 0 else 0
+    return B.ALLREDUCE_FN(cb), state
+
+
+@pytest.mark.parametrize("levels", [0, 16])
+@pytest.mark.parametrize("flags", [0, B.FLAG_ONE_LANE | B.FLAG_NO_GRAPH])
+@pytest.mark.parametrize("read_first", [False, True])
+def test_a_failed_reduction_leaves_q(levels, flags, read_first):
+    """A step that ends at its k-th reduction: q is what z and u give (it is not stored between iterations, and its memory serves
+    another matrix within one), read back, in the objective's terms and in the next iteration after u has been set.  In the first
+    iteration of a context, and after q has been read, that memory held q."""
+    inp = synth.make_inputs(synth.small("c2", 300, feat_dim=12, hidden=40, n_layers=4, quant_levels=levels))
+    nu = np.float32(inp.workload.nu)
+    for k in range(1, 30):
+        cb, state = _failing_reduction()
+        ctx = B.from_inputs(inp, flags=flags, shard=(0, 300, cb))
+        if read_first:
+            ctx.step(2)
+            for l in range(1, 4):
+                ctx.get_tensor(B.T_Q, l)
+        state["fail_at"] = k
+        try:
+            ctx.step(1)
+            assert k > 8                                  # W-gradient and its sums of four layers at least
+            ctx.destroy()
+            break
+        except B.PdadmmError as e:
+            assert "reduction callback" in str(e)
+        want = np.zeros(3)
+        for l in range(1, 4):
+            z, u, q, p = (ctx.get_tensor(kind, l + (kind == B.T_P)) for kind in (B.T_Z, B.T_U, B.T_Q, B.T_P))
+            f = np.maximum(z, 0)
+            assert (np.abs(q - (f + u / nu)) <= 4 * 2.0 ** -23 * (np.abs(f) + np.abs(u / nu))).all(), (k, l)
+            want[l - 1] = ((p.astype(np.float64) - q) ** 2).sum()
+            ctx.set_tensor(B.T_U, l, u)
+            assert np.array_equal(ctx.get_tensor(B.T_Q, l), q)
+        assert np.allclose(ctx.residuals(), want, rtol=1e-6)
+        ctx.destroy()
+
+
 def test_nccl_callback_with_one_rank_equals_the_unsharded_context():
     """The callback that bench.py uses on several GPUs (torch.distributed all_reduce on the library's stream, on a
     tensor that wraps the library's buffer), here in a process group of one NCCL rank: every sum over shards is the
