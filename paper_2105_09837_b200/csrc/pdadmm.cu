@@ -204,6 +204,7 @@ struct pdadmm_ctx {
   bool q_free = false;              // the context may do without it
   bool q_implied = false;           // z and u give it now
   bool q_stale = false;             // the stored values are older
+  bool in_iteration = false;        // an iteration was begun and has not been queued to its end
   bool p_sums_valid = false, r_sums_valid = false;          // the column sums of p_l and of r_l are those of the stored values
   // Words that are zero between calls, one block so that one clear covers them: d_flag[0..3] (z_L solver non-convergence, expired
   // wait, non-finite sum, unused), the layers' `done` and w_* words, the tail counts of the lanes that cut tails.
@@ -1261,9 +1262,15 @@ static int iterate_layers(pdadmm_ctx *c, bool *hit_cap) {
 // after the z-update of every layer.
 static void will_iterate(pdadmm_ctx *c) {
   if (c->q_implied) c->q_stale = true;
+  c->in_iteration = true;
 }
 static void iterated(pdadmm_ctx *c) {
   if (c->q_free) c->q_implied = c->q_stale = true;
+  c->in_iteration = false;
+}
+// What is derived from the tensors (the residual, t, planes and magnitudes, column sums) is formed again by the next call that needs it.
+static void forget_derived(pdadmm_ctx *c) {
+  c->r_valid = c->t_valid = c->w_planes_valid = c->amax_p_valid = c->r_sums_valid = c->p_sums_valid = false;
 }
 static int iterate_once(pdadmm_ctx *c, bool *hit_cap) {
   will_iterate(c);
@@ -1839,7 +1846,7 @@ extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
     PD_CUDA(cudaGetLastError());
     // the linear residual of the restarted layers is zero by construction; everything derived from the other tensors
     // (the residual of the kept layers, t, planes, largest magnitudes) is rebuilt by the next call that needs it
-    c->r_valid = false; c->t_valid = false; c->w_planes_valid = false; c->amax_p_valid = false; c->r_sums_valid = c->p_sums_valid = false;
+    forget_derived(c);
     return PDADMM_OK;
   });
 }
@@ -2049,6 +2056,9 @@ extern "C" int pdadmm_step(pdadmm_ctx *c, int n_iters) {
   // an iteration that was abandoned half way may have work on lanes that the main stream has not joined
   if (rc == PDADMM_ENOMEM || rc == PDADMM_ECUDA)
     for (auto &x : c->more_lanes) cudaStreamSynchronize(x->own);
+  // and W and b are ahead of the residual, which the z-update brings after them
+  if (c->in_iteration) forget_derived(c);
+  c->in_iteration = false;
   return rc;
 }
 
@@ -2066,7 +2076,7 @@ static int finish_steps(pdadmm_ctx *c, bool hit_cap) {
   if (c->profiling) PD_TRY(prof_collect(c));
   if (c->h_pinned[9] != 0) {
     // nothing derived from the tensors was finished either
-    c->r_valid = c->t_valid = c->w_planes_valid = c->amax_p_valid = c->r_sums_valid = c->p_sums_valid = false;
+    forget_derived(c);
     return fail(PDADMM_ETIMEOUT, "a bounded wait inside a tensor-core product expired");
   }
   if (c->h_pinned[10] != 0) return fail(PDADMM_ENUMERIC, "a non-finite value reached the gradient norms: the state holds NaN or Inf");

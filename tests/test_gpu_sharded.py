@@ -13,6 +13,7 @@ import oracle.pdadmm_oracle as o
 from paper_2105_09837_b200 import binding as B
 from paper_2105_09837_b200 import sharded, synth
 import parity_util as U
+from test_gpu_parity import _compare_iteration
 
 pytestmark = pytest.mark.gpu
 
@@ -197,6 +198,33 @@ def test_a_failed_reduction_leaves_q(levels, flags, read_first):
             ctx.set_tensor(B.T_U, l, u)
             assert np.array_equal(ctx.get_tensor(B.T_Q, l), q)
         assert np.allclose(ctx.residuals(), want, rtol=1e-6)
+        ctx.destroy()
+
+
+@pytest.mark.parametrize("levels", [0, 16])
+def test_the_step_after_a_failed_one_is_an_iteration_of_what_it_left(levels):
+    """A step that ends at its k-th reduction leaves W and b of some layers ahead of the others; what the next one makes of those
+    tensors is the oracle's iteration of them, with the residual, t, planes and column sums that belong to them."""
+    inp = synth.make_inputs(synth.small("c2", 300, feat_dim=12, hidden=40, n_layers=3, quant_levels=levels))
+    prm, first, _ = U.oracle_problem(inp)
+    for k in range(1, 30):
+        cb, state = _failing_reduction()
+        ctx = B.from_inputs(inp, shard=(0, 300, cb))
+        ctx.step(2)
+        state["fail_at"] = k
+        try:
+            ctx.step(1)
+            ctx.destroy()
+            assert k > 8
+            break
+        except B.PdadmmError as e:
+            assert "reduction callback" in str(e)
+        prev = first.copy()
+        for name, v in U.read_state(ctx).items():
+            setattr(prev, name, v)
+        if levels:
+            prev.scale = [prev.scale[0]] + [float(ctx.get_tensor(B.T_QSCALE, l)[0]) for l in (2, 3)]
+        _compare_iteration(ctx, prev, prm, f"k={k}")
         ctx.destroy()
 
 
