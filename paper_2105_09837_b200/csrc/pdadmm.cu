@@ -1134,7 +1134,7 @@ static void zqu_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
     bytes += ((c->levels ? 28.0 + c->code_bytes : 32.0) + 4.0 + (fused ? 0.0 : 4.0) + (c->use_tc && ly.rp.hi ? 4.0 : 0.0)) * c->N * ly.n_out;
   }
   Launch k(c, KC_ZQU, st, bytes, 0);
-  const ZquParams prm{c->rho, c->nu, c->slope, c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
+  const ZquParams prm{c->rho, c->nu, c->slope, two_term(1.0, 2.0 + (double)c->slope * c->slope), c->quant_q ? (float)(c->levels - 1) : -1.0f, c->code_bytes == 2, c->table_lo,
                       c->table_step, c->table_size, c->table_even ? 1 : 0};
   const dim3 grid((unsigned)blocks, (unsigned)n);
   const bool general = !(c->q_implied && c->q_free);
