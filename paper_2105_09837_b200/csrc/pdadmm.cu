@@ -1966,6 +1966,7 @@ static int ensure_sums(pdadmm_ctx *c) {
       blocks = std::max(blocks, ly.r_blocks);
       threads = std::max(threads, row_share(ly.ld_out).threads);
     }
+    Launch k(c, KC_SMALL, st, 0, 0);
     colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
   }
   c->r_sums_valid = true;
@@ -1983,7 +1984,11 @@ static int ensure_sums(pdadmm_ctx *c) {
       ld = std::max(ld, ly.ld_in);
       ++n;
     }
-    colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+    {
+      Launch k(c, KC_SMALL, st, 0, 0);
+      colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+    }
+    Launch k(c, KC_SMALL, st, 0, 0);
     colsum_total_kernel<<<dim3((unsigned)ceil_div(ld, TOTAL_COLS), (unsigned)n), EW_THREADS, 0, st>>>(g);
   }
   PD_CUDA(cudaGetLastError());
@@ -2327,7 +2332,8 @@ extern "C" int pdadmm_set_tensor(pdadmm_ctx *c, int kind, int layer, const void 
     if (kind == PDADMM_T_Z || kind == PDADMM_T_Q || kind == PDADMM_T_U) PD_TRY(stored_q(c));
     PD_TRY(copy_rows(c->device, c->scr.st, const_cast<void *>(host_src), t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, false));
     if (kind == PDADMM_T_X || kind == PDADMM_T_P || kind == PDADMM_T_W || kind == PDADMM_T_B || kind == PDADMM_T_Z)
-      c->r_valid = c->r_sums_valid = c->p_sums_valid = false;
+      c->r_valid = c->r_sums_valid = false;
+    if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->p_sums_valid = false;
     if (kind == PDADMM_T_W) c->w_planes_valid = false;
     if (kind == PDADMM_T_X || kind == PDADMM_T_P) c->amax_p_valid = false;
     if (kind == PDADMM_T_X || (kind == PDADMM_T_P && layer == 1)) c->x_planes_valid = false;

@@ -173,3 +173,31 @@ def test_norms_of_many_wide_layers_of_one_tile_each():
                 assert abs(taus[-1][l - 1] / 2.0 ** (trials - 1) - first) <= 2e-4 * first, l
         ctx.destroy()
     assert bits[0] == bits[1] == bits[2]
+
+
+@pytest.mark.parametrize("levels", [0, 256, 4096])
+def test_column_sums_of_p_outlast_other_tensors(levels):
+    """Setting W, b or z leaves p as it is: the next step sums r again and not X and every p.  (Beside the sums of an iteration, those of
+    r_L: one launch for r, two for p.)  It is still the oracle's iteration."""
+    inp = synth.make_inputs(synth.small("c2", 261, feat_dim=9, hidden=33, n_layers=4, quant_levels=levels))
+    prm, s, _ = U.oracle_problem(inp)
+    ctx = B.from_inputs(inp)
+    ctx.step(3)
+    ctx.profile(True)
+
+    def summing(kind):
+        if kind is not None:
+            ctx.set_tensor(kind, 2, ctx.get_tensor(kind, 2) * np.float32(1 if kind == B.T_P else 0.75))
+        before = ctx.profile_read()["finalize"]["launches"]
+        ctx.step(1)
+        return ctx.profile_read()["finalize"]["launches"] - before
+    own = summing(None)
+    assert [summing(k) - own for k in (B.T_W, B.T_B, B.T_Z, B.T_P)] == [1, 1, 1, 3]
+    ctx.profile(False)
+    ctx.set_tensor(B.T_W, 3, ctx.get_tensor(B.T_W, 3) * np.float32(1.25))
+    for k, v in U.read_state(ctx).items():
+        setattr(s, k, v)
+    if levels:
+        s.scale = [s.scale[0]] + [float(ctx.get_tensor(B.T_QSCALE, l)[0]) for l in (2, 3, 4)]
+    _compare_iteration(ctx, s, prm, f"m={levels}")
+    ctx.destroy()
