@@ -93,6 +93,7 @@ struct Layer {
   float *b = nullptr;       // [ld_out]
   float *z = nullptr, *r = nullptr;          // [N][ld_out]
   float *q = nullptr, *u = nullptr;          // [N][ld_out], hidden layers only
+  bool q_stale = false;     // the stored q is older than z and u, which give it (c->q_implied)
   float *t = nullptr;       // [N][ld_in], l >= 2: u_{l-1} + rho (p_l - q_{l-1}), the product-free part of grad_p phi
   float *gradW = nullptr;   // [n_out][ld_in]
   // Tensor-core path: planes of W, of grad_W and of r (written by the z-step for the next p-gradient;
@@ -203,7 +204,6 @@ struct pdadmm_ctx {
   // that iteration ends).
   bool q_free = false;              // the context may do without it
   bool q_implied = false;           // z and u give it now
-  bool q_stale = false;             // the stored values are older
   bool in_iteration = false;        // an iteration was begun and has not been queued to its end
   bool p_sums_valid = false, r_sums_valid = false;          // the column sums of p_l and of r_l are those of the stored values
   // Words that are zero between calls, one block so that one clear covers them: d_flag[0..3] (z_L solver non-convergence, expired
@@ -1258,14 +1258,17 @@ static int iterate_layers(pdadmm_ctx *c, bool *hit_cap) {
   }
   return PDADMM_OK;
 }
+static void mark_q_stale(pdadmm_ctx *c) {
+  for (int l = 0; l + 1 < c->L; ++l) c->layers[l].q_stale = true;
+}
 // An iteration with q_implied puts G p+ where q is, and may end early (a reduction over shards that fails): z and u give q before and
 // after the z-update of every layer.
 static void will_iterate(pdadmm_ctx *c) {
-  if (c->q_implied) c->q_stale = true;
+  if (c->q_implied) mark_q_stale(c);
   c->in_iteration = true;
 }
 static void iterated(pdadmm_ctx *c) {
-  if (c->q_free) c->q_implied = c->q_stale = true;
+  if (c->q_free) { c->q_implied = true; mark_q_stale(c); }
   c->in_iteration = false;
 }
 // What is derived from the tensors (the residual, t, planes and magnitudes, column sums) is formed again by the next call that needs it.
@@ -1831,7 +1834,6 @@ extern "C" int pdadmm_init_sharded(const pdadmm_config *cfg, const pdadmm_shard 
 }
 
 static int refresh_p(pdadmm_ctx *c);
-static int refresh_q(pdadmm_ctx *c);
 static int stored_q(pdadmm_ctx *c);
 
 extern "C" int pdadmm_start_layers_from(pdadmm_ctx *c, int first_layer) {
@@ -1890,21 +1892,22 @@ static int refresh_p(pdadmm_ctx *c) {
   return PDADMM_OK;
 }
 
-// q_l as stored values, from z and u where these are newer
-static int refresh_q(pdadmm_ctx *c) {
-  if (!c->q_stale) return PDADMM_OK;
-  for (int l = 0; l + 1 < c->L; ++l) {
+// q of hidden layers first..last (0-based) as stored values, from z and u where these are newer
+static int refresh_q(pdadmm_ctx *c, int first, int last) {
+  for (int l = first; l <= last; ++l) {
     Layer &ly = c->layers[l];
+    if (!ly.q_stale) continue;
+    Launch k(c, KC_AXPY, c->scr.st, 12.0 * c->N * ly.n_out, 0);
     const size_t n4 = (size_t)c->N * ly.ld_out / 4;
     q_of_z_and_u_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.z, ly.u, c->slope, c->nu, ly.n_out, (uint32_t)ly.ld_out / 4, ly.q, n4);
+    ly.q_stale = false;
   }
   PD_CUDA(cudaGetLastError());
-  c->q_stale = false;
   return PDADMM_OK;
 }
 // z, q or u is about to be set: q need not follow from the others any more
 static int stored_q(pdadmm_ctx *c) {
-  PD_TRY(refresh_q(c));
+  PD_TRY(refresh_q(c, 0, c->L - 2));
   c->q_implied = false;
   return PDADMM_OK;
 }
@@ -1937,7 +1940,7 @@ static int ensure_operands(pdadmm_ctx *c) {
 static int ensure_residual(pdadmm_ctx *c) {
   PD_TRY(ensure_operands(c));
   if (!c->t_valid) {
-    PD_TRY(refresh_q(c));
+    PD_TRY(refresh_q(c, 0, c->L - 2));
     for (int l = 1; l < c->L; ++l) {
       Layer &ly = c->layers[l];
       const Layer &pv = c->layers[l - 1];
@@ -2105,7 +2108,7 @@ static int read_objective(pdadmm_ctx *c, int parts) {
       const Layer &ly = c->layers[l0 + i];
       const bool hidden = l0 + i + 1 < c->L;
       const Layer *nx = hidden ? &c->layers[l0 + i + 1] : nullptr;
-      o.l[i] = ObjLayer{ly.r, ly.z, hidden && !c->q_stale ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
+      o.l[i] = ObjLayer{ly.r, ly.z, hidden && !ly.q_stale ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
                         (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f,
                          hidden && c->slope == ACT_SIGMOID ? ly.n_out : 0, (uint32_t)ly.ld_out / 4};
       n4_max = std::max(n4_max, o.l[i].n4);
@@ -2287,7 +2290,7 @@ extern "C" int pdadmm_get_tensor(pdadmm_ctx *c, int kind, int layer, void *host_
       return fail(PDADMM_EINVAL, "tensor kind %d layer %d has %zu bytes, caller passed %zu", kind, layer,
                   t.rows * t.width * t.elem, bytes);
     if (kind == PDADMM_T_P) PD_TRY(refresh_p(c));
-    if (kind == PDADMM_T_Q) PD_TRY(refresh_q(c));
+    if (kind == PDADMM_T_Q) PD_TRY(refresh_q(c, layer - 1, layer - 1));
     return copy_rows(c->device, c->scr.st, host_dst, t.ptr, t.ld * t.elem, t.width * t.elem, t.rows, true);
   });
 }

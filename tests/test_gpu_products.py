@@ -201,3 +201,21 @@ def test_column_sums_of_p_outlast_other_tensors(levels):
         s.scale = [s.scale[0]] + [float(ctx.get_tensor(B.T_QSCALE, l)[0]) for l in (2, 3, 4)]
     _compare_iteration(ctx, s, prm, f"m={levels}")
     ctx.destroy()
+
+
+def test_reading_q_of_one_layer_forms_that_layer_s():
+    inp = synth.make_inputs(synth.small("c2", 261, feat_dim=9, hidden=33, n_layers=5, quant_levels=0))
+    nu = np.float32(inp.workload.nu)
+    ctx = B.from_inputs(inp)
+    ctx.step(2)
+    before = ctx.launches()
+    q = {l: ctx.get_tensor(B.T_Q, l) for l in (3, 3, 1)}
+    assert ctx.launches() - before == 2
+    ctx.set_tensor(B.T_U, 2, ctx.get_tensor(B.T_U, 2))         # q may be set apart from z and u now: every layer's is stored
+    assert ctx.launches() - before == 4
+    for l in range(1, 5):
+        z, u, got = (ctx.get_tensor(k, l) for k in (B.T_Z, B.T_U, B.T_Q))
+        f = np.maximum(z, 0)
+        assert (np.abs(got - (f + u / nu)) <= 4 * 2.0 ** -23 * (np.abs(f) + np.abs(u / nu))).all()
+        assert l not in q or np.array_equal(q[l], got)
+    ctx.destroy()
