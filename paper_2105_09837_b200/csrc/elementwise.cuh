@@ -1076,14 +1076,19 @@ relu_max_kernel(const float *__restrict__ z, float *__restrict__ q, size_t n4, f
 // 16-byte loads, p_next as its codes in pdADMM-G-Q (the same bits).
 constexpr int OBJ_MAX_LAYERS = 40;           // layers per launch: their pointers travel as a kernel argument
 enum : int { OBJ_ALL = 0, OBJ_RESIDUALS = 1 };
-struct ObjLayer { const float *r, *z, *q /* null: from z and u */, *u /* null: only r^2 */, *p_next; const void *codes_next; size_t n4; float scale, lo; int width /* 0: padding adds nothing */; uint32_t groups; };
+constexpr int obj_blocks_per_sm(int parts, bool smooth) { return parts == OBJ_ALL || smooth ? 4 : 6; }      // resident ones, which is what a launch has
+struct ObjLayer { const float *r, *z, *q, *u /* null: only r^2 */, *p_next; const void *codes_next; size_t n4; float scale, lo; int width /* 0: padding adds nothing */; uint32_t groups /* of 4 columns in a row */; };
 struct ObjLayers { ObjLayer l[OBJ_MAX_LAYERS]; };
 __device__ __forceinline__ void add_sq4(double &s, float4 v) {
   const double a = v.x, b = v.y, c = v.z, d = v.w;
   s += (a * a + b * b) + (c * c + d * d);
 }
-template <int PARTS>
-__global__ void __launch_bounds__(EW_THREADS)
+// IMPLIED: q from z and u (every layer's, see zqu_kernel).  SMOOTH: f = tanh or sigmoid, whose evaluation would otherwise stand between the
+// loads.  A thread has the loads of two groups on their way, and the blocks are one round of what the SMs hold.  Bound by memory: 16 bytes per
+// element, the residuals alone 12 (q is not stored: 8 with it).  60 000 x 1000, 4 layers: objective 460 us, residuals 350; with f in its
+// general form between the loads of one group 705 and 363, with a stored q and 20 bytes 552 and 246.
+template <int PARTS, bool IMPLIED, bool SMOOTH>
+__global__ void __launch_bounds__(EW_THREADS, obj_blocks_per_sm(PARTS, SMOOTH))
 objective_kernel(const __grid_constant__ ObjLayers layers, float slope, float nu, int wide_codes, double *slots, int *counters,
                  double *out) {
   __shared__ double red[EW_THREADS / 32];
@@ -1092,39 +1097,49 @@ objective_kernel(const __grid_constant__ ObjLayers layers, float slope, float nu
   double s[4] = {0, 0, 0, 0};
   const float inv_nu = 1.0f / nu;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < y.n4; i += stride) {
+  auto f = [&](float x) { return SMOOTH ? act_eval(x, slope) : x > 0.0f ? x : slope * x; };
+  constexpr int U = 2;
+  for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < y.n4; i0 += U * stride) {
     if (y.u == nullptr) {
-      if (PARTS == OBJ_ALL) add_sq4(s[0], ld4(y.r, i));
+      if (PARTS == OBJ_ALL)
+        for (size_t i = i0; i < y.n4 && i < i0 + U * stride; i += stride) add_sq4(s[0], ld4(y.r, i));
       continue;
     }
-    float4 qv;
-    if (y.q != nullptr) {
-      qv = ld4(y.q, i);
-    } else {
-      const float4 zv = ld4(y.z, i), uv = ld4(y.u, i);
-      qv = make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
-                       fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope)));
+    float4 rv[U], zv[U], uv[U], qv[U], pv[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const size_t i = i0 + k * stride;
+      if (i >= y.n4) continue;
+      if (PARTS == OBJ_ALL) rv[k] = ld4(y.r, i);
+      if (PARTS == OBJ_ALL || IMPLIED) { zv[k] = ld4(y.z, i); uv[k] = ld4(y.u, i); }
+      if (!IMPLIED) qv[k] = ld4(y.q, i);
+      pv[k] = y.codes_next != nullptr ? levels_of4(y.codes_next, wide_codes, i, y.scale, y.lo) : ld4(y.p_next, i);
     }
-    float4 pv = y.codes_next != nullptr ? levels_of4(y.codes_next, wide_codes, i, y.scale, y.lo) : ld4(y.p_next, i);
-    int inside = 4;
-    if (y.width > 0) {                       // f(0) is not zero: q = f(z) + u/nu of the padding isn't either
-      inside = columns_inside(i, y.groups, y.width);
-      qv = keep_columns(qv, inside);
-      pv = keep_columns(pv, inside);
-    }
-    if (PARTS == OBJ_ALL) {
-      const float4 rv = ld4(y.r, i), zv = ld4(y.z, i), uv = ld4(y.u, i);
-      add_sq4(s[0], rv);
-#define PD_OBJ(f, k)                                                               \
-      {                                                                            \
-        const double q = qv.f, act = k < inside ? act_eval(zv.f, slope) : 0.f, res = (double)pv.f - q; \
-        s[1] += (q - act) * (q - act); s[2] += (double)uv.f * res; s[3] += res * res; \
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const size_t i = i0 + k * stride;
+      if (i >= y.n4) continue;
+      float4 fv = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (PARTS == OBJ_ALL || IMPLIED) fv = make_float4(f(zv[k].x), f(zv[k].y), f(zv[k].z), f(zv[k].w));
+      if (IMPLIED) qv[k] = make_float4(fmaf(uv[k].x, inv_nu, fv.x), fmaf(uv[k].y, inv_nu, fv.y), fmaf(uv[k].z, inv_nu, fv.z), fmaf(uv[k].w, inv_nu, fv.w));
+      if (SMOOTH && y.width > 0) {           // f(0) is not zero: q = f(z) + u/nu of the padding isn't either
+        const int inside = columns_inside(i, y.groups, y.width);
+        fv = keep_columns(fv, inside);
+        qv[k] = keep_columns(qv[k], inside);
+        pv[k] = keep_columns(pv[k], inside);
       }
-      PD_OBJ(x, 0) PD_OBJ(y, 1) PD_OBJ(z, 2) PD_OBJ(w, 3)
+#define PD_OBJ(e)                                                                       \
+      {                                                                                 \
+        const double q = qv[k].e, res = (double)pv[k].e - q;                            \
+        if (PARTS == OBJ_ALL) {                                                         \
+          const double d = q - (double)fv.e;                                            \
+          s[1] += d * d; s[2] += (double)uv[k].e * res;                                 \
+        }                                                                               \
+        s[3] += res * res;                                                              \
+      }
+      if (PARTS == OBJ_ALL) add_sq4(s[0], rv[k]);
+      PD_OBJ(x) PD_OBJ(y) PD_OBJ(z) PD_OBJ(w)
 #undef PD_OBJ
-    } else {
-      const double a = (double)pv.x - qv.x, b = (double)pv.y - qv.y, c = (double)pv.z - qv.z, d = (double)pv.w - qv.w;
-      s[3] += (a * a + b * b) + (c * c + d * d);
     }
   }
   double *mine = slots + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4;

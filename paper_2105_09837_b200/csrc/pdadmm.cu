@@ -2108,19 +2108,31 @@ static int read_objective(pdadmm_ctx *c, int parts) {
       const Layer &ly = c->layers[l0 + i];
       const bool hidden = l0 + i + 1 < c->L;
       const Layer *nx = hidden ? &c->layers[l0 + i + 1] : nullptr;
-      o.l[i] = ObjLayer{ly.r, ly.z, hidden && !ly.q_stale ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
+      o.l[i] = ObjLayer{ly.r, ly.z, hidden ? ly.q : nullptr, hidden ? ly.u : nullptr, hidden ? nx->p : nullptr, hidden && c->levels ? nx->codes : nullptr,
                         (size_t)c->N * ly.ld_out / 4, hidden ? nx->scale : 0.f, hidden ? nx->lo : 0.f,
                          hidden && c->slope == ACT_SIGMOID ? ly.n_out : 0, (uint32_t)ly.ld_out / 4};
       n4_max = std::max(n4_max, o.l[i].n4);
     }
-    // all layers side by side: about eight blocks per SM altogether, as many slots as the buffer holds
+    // all layers side by side: the hidden ones, which are nearly all of the work, have one round of blocks, as many slots as the buffer holds
+    const int n_hidden = std::max(1, l0 + n == c->L ? n - 1 : n);
     const size_t fit = std::min<size_t>(OBJ_MAX_BLOCKS, c->scr.n_slots / (4 * (size_t)n));
     const int per_layer = (int)std::max<size_t>(1, std::min(fit, std::min<size_t>((n4_max + EW_THREADS - 1) / EW_THREADS,
-                                                                                  (size_t)ceil_div(c->n_sms * 8, n))));
+                                                                                  (size_t)(obj_blocks_per_sm(parts, c->table_size > 0) * c->n_sms / n_hidden))));
     const dim3 grid((unsigned)per_layer, (unsigned)n);
     double *out = c->h_results + 4 * (size_t)l0;
-    if (parts == OBJ_ALL) objective_kernel<OBJ_ALL><<<grid, EW_THREADS, 0, st>>>(o, c->slope, c->nu, wide, c->scr.slots, c->done, out);
-    else objective_kernel<OBJ_RESIDUALS><<<grid, EW_THREADS, 0, st>>>(o, c->slope, c->nu, wide, c->scr.slots, c->done, out);
+    auto launch = [&](auto parts_, auto implied, auto smooth) {
+      objective_kernel<decltype(parts_)::value, decltype(implied)::value, decltype(smooth)::value>
+          <<<grid, EW_THREADS, 0, st>>>(o, c->slope, c->nu, wide, c->scr.slots, c->done, out);
+    };
+    auto with = [&](auto parts_) {
+      using T = std::true_type;
+      using F = std::false_type;
+      const bool smooth = c->table_size > 0;
+      if (c->q_implied) { if (smooth) launch(parts_, T{}, T{}); else launch(parts_, T{}, F{}); }
+      else { if (smooth) launch(parts_, F{}, T{}); else launch(parts_, F{}, F{}); }
+    };
+    if (parts == OBJ_ALL) with(std::integral_constant<int, OBJ_ALL>{});
+    else with(std::integral_constant<int, OBJ_RESIDUALS>{});
   }
   if (parts == OBJ_ALL) {
     const Layer &ly = c->layers[c->L - 1];
