@@ -886,15 +886,16 @@ zqu_table_kernel(const __grid_constant__ Group<Zqu> group, const __grid_constant
   if (y.amax_r != nullptr) commit_amax(mr, y.amax_r);
 }
 // q = f(z) + u/nu, for whoever wants the values
+struct QOfZU { const float *z, *u; float *q; int width; uint32_t groups /* of 4 columns in a row */; size_t n4; };
 __global__ void __launch_bounds__(EW_THREADS)
-q_of_z_and_u_kernel(const float *__restrict__ z, const float *__restrict__ u, float slope, float nu, int width, uint32_t groups,
-                    float *__restrict__ q, size_t n4) {
+q_of_z_and_u_kernel(const __grid_constant__ Group<QOfZU> group, float slope, float nu) {
+  const QOfZU &y = group.l[blockIdx.y];
   const float inv_nu = 1.0f / nu;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 zv = ld4(z, i), uv = ld4(u, i);
-    st4(q, i, keep_columns(make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
-                                       fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope))),
-                           columns_inside(i, groups, width)));
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < y.n4; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 zv = ld4(y.z, i), uv = ld4(y.u, i);
+    st4(y.q, i, keep_columns(make_float4(fmaf(uv.x, inv_nu, act_eval(zv.x, slope)), fmaf(uv.y, inv_nu, act_eval(zv.y, slope)),
+                                         fmaf(uv.z, inv_nu, act_eval(zv.z, slope)), fmaf(uv.w, inv_nu, act_eval(zv.w, slope))),
+                             columns_inside(i, y.groups, y.width)));
   }
 }
 

@@ -1894,13 +1894,22 @@ static int refresh_p(pdadmm_ctx *c) {
 
 // q of hidden layers first..last (0-based) as stored values, from z and u where these are newer
 static int refresh_q(pdadmm_ctx *c, int first, int last) {
-  for (int l = first; l <= last; ++l) {
-    Layer &ly = c->layers[l];
-    if (!ly.q_stale) continue;
-    Launch k(c, KC_AXPY, c->scr.st, 12.0 * c->N * ly.n_out, 0);
-    const size_t n4 = (size_t)c->N * ly.ld_out / 4;
-    q_of_z_and_u_kernel<<<ew_grid(n4), EW_THREADS, 0, c->scr.st>>>(ly.z, ly.u, c->slope, c->nu, ly.n_out, (uint32_t)ly.ld_out / 4, ly.q, n4);
-    ly.q_stale = false;
+  for (int l = first; l <= last;) {
+    Group<QOfZU> g;
+    int n = 0;
+    size_t n4_max = 0;
+    double bytes = 0;
+    for (; l <= last && n < MAX_GROUP; ++l) {
+      Layer &ly = c->layers[l];
+      if (!ly.q_stale) continue;
+      g.l[n++] = QOfZU{ly.z, ly.u, ly.q, ly.n_out, (uint32_t)ly.ld_out / 4, (size_t)c->N * ly.ld_out / 4};
+      n4_max = std::max(n4_max, g.l[n - 1].n4);
+      bytes += 12.0 * c->N * ly.n_out;
+      ly.q_stale = false;
+    }
+    if (n == 0) break;
+    Launch k(c, KC_AXPY, c->scr.st, bytes, 0);
+    q_of_z_and_u_kernel<<<dim3((unsigned)ew_grid(n4_max), (unsigned)n), EW_THREADS, 0, c->scr.st>>>(g, c->slope, c->nu);
   }
   PD_CUDA(cudaGetLastError());
   return PDADMM_OK;
