@@ -89,27 +89,33 @@ def test_host_copies_at_the_edges_of_a_piece(n_nodes, hidden):
 
 
 # columns at the edges of a wide tile (256) and of its halves, rows at those of a pair's 256 and a block's 128, contractions at those of
-# a K block; one round of tiles, several, and a last one of a few tiles cut along the contraction (2, 12 or 5 of them, in 2 to 5
-# slices); over node slices.  The shapes beside them keep narrow tiles, some with the last round cut as well.
-@pytest.mark.parametrize("mode,M,N,K,wide,cut", [
-    (0, 18944, 256, 640, True, False), (0, 18690, 255, 641, True, False), (1, 18690, 255, 641, True, False), (0, 9400, 500, 703, True, False),
-    (1, 9400, 509, 703, True, False), (0, 9600, 500, 3001, True, True), (1, 4900, 2047, 2049, True, True), (0, 18945, 1025, 2049, True, True),
-    (1, 18945, 1025, 1025, True, True), (2, 500, 700, 30000, True, False), (2, 257, 2049, 16001, True, False), (2, 511, 769, 30000, True, False),
-    (0, 18945, 255, 641, False, False), (1, 19000, 257, 1000, False, True), (1, 9600, 500, 703, False, False), (0, 4800, 1025, 1600, False, True),
-    (2, 512, 512, 40000, False, False)])
-def test_wide_tiles_at_their_edges(mode, M, N, K, wide, cut):
+# a K block.  Three of the shapes run on wide tiles (the next test has the others of those).
+@pytest.mark.parametrize("mode,M,N,K", [(0, 18944, 256, 640), (0, 18945, 255, 641), (1, 19000, 257, 1000), (1, 9600, 500, 703),
+                                        (0, 4800, 1025, 1600), (2, 500, 700, 30000), (2, 257, 2049, 16001), (2, 512, 512, 40000)])
+def test_wide_tiles_at_their_edges(mode, M, N, K):
     """Every element within LAMBDA standard deviations of KAPPA times the root-sum-square of its terms, the product's bound in the
-    iteration tests.  The shapes take the tiles that they are meant for."""
+    iteration tests."""
     rng = np.random.default_rng(M + N + K)
     a = rng.standard_normal((K, M) if mode == 2 else (M, K), dtype=np.float32)
     b = rng.standard_normal((N, K) if mode == 0 else (K, N), dtype=np.float32)
-    before = B.product_forms()
     c, ss = B.matmul(mode, a, b)
-    assert tuple(x - y for x, y in zip(B.product_forms(), before)) == (1, int(wide), int(cut))
     at, bt = (a.T if mode == 2 else a).astype(np.float64), (b.T if mode == 0 else b).astype(np.float64)
     bound = E.LAMBDA * E.kappa(True) * np.sqrt((at ** 2) @ (bt ** 2))
     assert (np.abs(c - at @ bt) <= bound).all()
     assert abs(ss - (c.astype(np.float64) ** 2).sum()) <= 1e-6 * ss
+
+
+# One round of wide tiles, several, and a last one of a few tiles cut along the contraction (2, 12 or 5 of them, in 2 to 5 slices); over node
+# slices; shapes beside them that keep narrow tiles, with the last round cut.
+@pytest.mark.parametrize("mode,M,N,K,wide,cut", [
+    (0, 18944, 256, 640, True, False), (0, 18690, 255, 641, True, False), (1, 18690, 255, 641, True, False), (0, 9400, 500, 703, True, False),
+    (1, 9400, 509, 703, True, False), (0, 9600, 500, 3001, True, True), (1, 4900, 2047, 2049, True, True), (0, 18945, 1025, 2049, True, True),
+    (1, 18945, 1025, 1025, True, True), (2, 500, 700, 30000, True, False), (2, 511, 769, 30000, True, False),
+    (1, 19000, 257, 1000, False, True), (0, 4800, 1025, 1600, False, True)])
+def test_tiles_of_the_form_that_the_shape_is_for(mode, M, N, K, wide, cut):
+    before = B.product_forms()
+    test_wide_tiles_at_their_edges(mode, M, N, K)
+    assert tuple(x - y for x, y in zip(B.product_forms(), before)) == (1, int(wide), int(cut))
 
 
 def test_refused_planes_on_wide_tiles():
