@@ -554,7 +554,7 @@ reduce_gradW_kernel(const __grid_constant__ Group<GradWSum> group, float nu) {
 // `sums`: a context that owns part of the nodes leaves its part of the sum there instead (finalize_bias_kernel follows).
 // `gp`: where G p+ is not left to the z-update, further blocks do r <- r - (G p+)/theta.
 struct ThetaStep {
-  float *W; const float *G; int n_out, n_in, ld;
+  float *W; const float *G; int n_out, ld;
   uint32_t *amax_W /* may be null */; PlaneOut Wp;
   const double *p_sum, *p_change, *r_sum;
   float *b, *shift;
@@ -921,7 +921,7 @@ zlast_kernel(float *__restrict__ r, float *__restrict__ z, const float *__restri
              const float *__restrict__ gp /* null: r has it */, const LayerScalars *sc) {
   const int j = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) / G), lane = threadIdx.x % G;
   const bool row = j < n_rows;
-  const size_t at = (size_t)(row ? j : n_rows - 1) * ld + 2 * lane;          // ld is a multiple of 32 and C <= 2 G
+  const size_t at = (size_t)(row ? j : n_rows - 1) * ld + 2 * lane;          // (may lie beyond the row: every access is guarded by in[])
   const int c0 = 2 * lane;
   const bool in[2] = {c0 < C, c0 + 1 < C};
   auto sum = [&](double v) {

@@ -157,8 +157,10 @@ struct TcLayer {
   // in slice order and runs the epilogue.  tail_split <= 1 switches this off.
   int tail_begin, tail_split;
   TcDiv tiles_n, tiles_mn;                // column tiles, output tiles
-  float *tail_ws;         // [tiles from tail_begin][tail_split][8 or 16 warps][64][32] floats
-  int *tail_count;        // [tiles from tail_begin][8 or 16 warps], zero before and after every launch
+  // Pieces of 32 rows x 64 columns, one per accumulate warp: 8 of a block's tile, 16 of a pair's, 32 of a pair's wide one.  A round has n_sms
+  // units of blocks or n_sms / 2 of pairs and a cut takes at least two of them, so n_sms * 8 counts are enough (n_sms / 4 wide tiles).
+  float *tail_ws;         // [tiles from tail_begin][tail_split][pieces][64][32] floats
+  int *tail_count;        // [tiles from tail_begin][pieces], zero before and after every launch
 };
 template <class Epi>
 struct TcGroup {

@@ -476,9 +476,12 @@ static bool use_pairs(const pdadmm_ctx *c, const Prod<Epi> *v, int n) {
 // estimate of the two.  The persistent grid takes the tiles in rounds; SM cycles per K block and at a tile's end, from traces of
 // 20 000 x 500, 170 000 x 1000 and 90 000 x 2000: a block on its own 1560 and 2800, a pair 1080 and 2800, a pair with a wide
 // tile 1500 and 8800 (its accumulate warps store the tile themselves); with two MMAs per product instead of three (integer
-// operands) 1230, 830, 1130 and 6900 at the end.  So a wide tile, which brings 64 KB per K block where two
-// narrow ones bring 96, wins from some six K blocks on, unless its columns are mostly padding or leave SMs idle.  (170 000 x 1000
-// G p+: 1.04 -> 0.90 ms; 90 000 x 2000: 1.50 -> 1.30 ms; W-gradient of 20 000 x 500, 9 layers: 410 -> 330 us.)
+// operands) 1230, 830, 1130 and 6900 at the end.  A wide tile brings 64 KB per K block where two narrow ones bring 96.  By the
+// estimate it wins from some six K blocks on, unless its columns are mostly padding or leave SMs idle; measured it wins from 16 on
+// (170 000 x 1000 G p+: 1.04 -> 0.90 ms; 90 000 x 2000: 1.50 -> 1.30 ms; W-gradient of 20 000 x 500, 9 layers: 410 -> 330 us) and
+// makes no difference at 8 (20 000 x 500, W g and G p+: 272 and 300 TFLOP/s either way), where the estimate says 7 %.  The norm-only product,
+// which stores nothing, is estimated as one that stores.  The estimate has no cut of the last round's tiles along the contraction in it
+// (launch_tc, single products), so where a form's last round is sparse it counts that round as a full one.
 struct Shape { int64_t M, N, K, n_split; };
 static bool choose_wide(int n_sms, const Shape *v, int n, bool ints, double *cost = nullptr) {
   double best[2];
@@ -835,10 +838,10 @@ static int p_gradient_and_tau(pdadmm_ctx *c, cudaStream_t st, const Batch &batch
 }
 
 // Blocks of a kernel that sums columns, for each of the layers of its launch; at least four rows for every row subgroup of a block
-// (2000 x 100, 9 layers: p-step 17.0 us with two, 14.9 so), fewer where that left SMs without a second block (few layers).  The z-update gets two full rounds of what the SMs hold at 64
-// registers a thread, four for a layer on its own: 10 000 x 256, 5 layers 122 us, with 3.3 rounds 129; 90 000 x 2000 1.28 ms a layer, with
-// two 1.33.  The p-step and the trial step 16 per SM, the
-// trial of a layer on its own 5 (one round: 170 000 x 1000 1.46 ms, 1.61 with 16).
+// (2000 x 100, 9 layers: p-step 17.0 us with two, 14.9 so), fewer where that left SMs without a second block (few layers).
+// The z-update gets two full rounds of what the SMs hold at 64 registers a thread, four for a layer on its own: 10 000 x 256, 5 layers 122 us,
+// with 3.3 rounds 129; 90 000 x 2000 1.28 ms a layer, with two 1.33.  The p-step and the trial step get 16 per SM, the trial of a layer on its
+// own 5 (one round: 170 000 x 1000 1.46 ms, 1.61 with 16).
 static int sum_blocks(const pdadmm_ctx *c, int ld, int layers, bool z) {
   const RowShare share = row_share(ld);
   const int per_sm = z ? (layers > 1 ? 2 : 4) * (1024 / share.threads) : c->levels && layers == 1 ? 5 : 16;
@@ -1094,7 +1097,7 @@ static int w_and_b_step(pdadmm_ctx *c, cudaStream_t st, const Batch &batch) {
       Scratch &s = scratch_of(c, l);
       const size_t n4r = (size_t)N * ly.ld_out / 4;
       const int nbw = (int)ceil_div(ly.n_out, EW_THREADS / 32), nbr = fused ? 0 : ew_grid((size_t)ceil_div((int64_t)n4r, 4));
-      g.l[n++] = ThetaStep{ly.W, ly.gradW, ly.n_out, ly.n_in, ly.ld_in, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp),
+      g.l[n++] = ThetaStep{ly.W, ly.gradW, ly.n_out, ly.ld_in, c->use_tc ? ly.amax_W : nullptr, plane_out(c, ly.Wp),
                            ly.p_sum, ly.p_change, ly.r_sum, ly.b, ly.shift, c->reduce != nullptr ? s.red : nullptr, ly.sc, nbw,
                            ly.r, fused ? nullptr : s.s1, (uint32_t)n4r, nbr};
       blocks = std::max(blocks, nbw + nbr);
