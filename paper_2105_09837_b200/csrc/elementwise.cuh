@@ -189,14 +189,35 @@ __device__ __forceinline__ void add4(double (&s)[4], float4 v) {
   s[0] += (double)v.x; s[1] += (double)v.y; s[2] += (double)v.z; s[3] += (double)v.w;
 }
 // column sums of a stored matrix (X, the last layer's r; r and p after the start or after the caller has set a tensor)
-struct ColSum { const float *x; RowBlocks rows; double *out; };
+struct ColSum { const float *x; RowBlocks rows; double *out; const void *codes /* may be null: read instead of x */; float scale; };
+// CODES: of a p that the products read as integers, (code - neg_levels) scale, as quant_trial_kernel sums the next p (the fp32 values are
+// rounded from it: the difference of two sums would not be zero where p does not change).
+template <bool CODES>
 __global__ void __launch_bounds__(EW_THREADS)
-colsum_kernel(const __grid_constant__ Group<ColSum> group) {
+colsum_kernel(const __grid_constant__ Group<ColSum> group, int wide_codes, int neg_levels) {
   __shared__ double sh[EW_THREADS * 4];
   const ColSum &y = group.l[blockIdx.y];
   if ((int)blockIdx.x >= y.rows.n_blocks) return;
   const float *__restrict__ x = y.x;
+  const void *__restrict__ codes = y.codes;
   row_block_sums(y.rows, (int)blockIdx.x, sh, [&](uint32_t i, uint32_t stride, int n, int, double (&sum)[4]) {
+    if (CODES && codes != nullptr) {
+      const int rows = n;
+      unsigned up[4] = {0, 0, 0, 0};
+#pragma unroll 4
+      for (; n > 0; --n, i += stride) {
+        if (wide_codes) {
+          const uint2 w = reinterpret_cast<const uint2 *>(codes)[i];
+          up[0] += w.x & 0xffffu; up[1] += w.x >> 16; up[2] += w.y & 0xffffu; up[3] += w.y >> 16;
+        } else {
+          const uint32_t w = reinterpret_cast<const uint32_t *>(codes)[i];
+          up[0] += w & 0xffu; up[1] += (w >> 8) & 0xffu; up[2] += (w >> 16) & 0xffu; up[3] += w >> 24;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) sum[e] = (double)y.scale * ((double)up[e] - (double)rows * neg_levels);
+      return;
+    }
 #pragma unroll 4
     for (; n > 0; --n, i += stride) add4(sum, ld4(x, i));
   });

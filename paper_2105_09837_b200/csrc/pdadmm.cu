@@ -1157,7 +1157,7 @@ static void r_column_sums(pdadmm_ctx *c, cudaStream_t st, const Layer &ly) {
   Launch k(c, KC_SMALL, st, 4.0 * c->N * ly.n_out, 0);
   Group<ColSum> g;
   g.l[0] = ColSum{ly.r, r_rows(c, ly), nullptr};
-  colsum_kernel<<<ly.r_blocks, row_share(ly.ld_out).threads, 0, st>>>(g);
+  colsum_kernel<false><<<ly.r_blocks, row_share(ly.ld_out).threads, 0, st>>>(g, 0, 0);
 }
 static void zlast_step(pdadmm_ctx *c, cudaStream_t st) {
   Layer &ly = c->layers[c->L - 1];
@@ -1982,18 +1982,18 @@ static int ensure_sums(pdadmm_ctx *c) {
       threads = std::max(threads, row_share(ly.ld_out).threads);
     }
     Launch k(c, KC_SMALL, st, 0, 0);
-    colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+    colsum_kernel<false><<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g, 0, 0);
   }
   c->r_sums_valid = true;
   if (c->p_sums_valid) return PDADMM_OK;
-  PD_TRY(refresh_p(c));
+  if (!c->int_operands) PD_TRY(refresh_p(c));
   const int S = std::min(1 + (int)c->more_lanes.size(), MAX_GROUP);        // as many as have slots of their own
   for (int l0 = 0; l0 < c->L; l0 += S) {
     Group<ColSum> g;
     int n = 0, blocks = 0, threads = 0, ld = 0;
     for (int l = l0; l < std::min(c->L, l0 + S); ++l) {
       const Layer &ly = c->layers[l];
-      g.l[n] = ColSum{ly.p, p_rows(c, ly, lane(c, n)), ly.p_sum};
+      g.l[n] = ColSum{ly.p, p_rows(c, ly, lane(c, n)), ly.p_sum, c->int_operands && l > 0 ? ly.codes : nullptr, ly.scale};
       blocks = std::max(blocks, g.l[n].rows.n_blocks);
       threads = std::max(threads, row_share(ly.ld_in).threads);
       ld = std::max(ld, ly.ld_in);
@@ -2001,7 +2001,9 @@ static int ensure_sums(pdadmm_ctx *c) {
     }
     {
       Launch k(c, KC_SMALL, st, 0, 0);
-      colsum_kernel<<<dim3((unsigned)blocks, (unsigned)n), threads, 0, st>>>(g);
+      const dim3 grid((unsigned)blocks, (unsigned)n);
+      if (c->int_operands) colsum_kernel<true><<<grid, threads, 0, st>>>(g, c->code_bytes == 2, c->neg_levels);
+      else colsum_kernel<false><<<grid, threads, 0, st>>>(g, 0, 0);
     }
     Launch k(c, KC_SMALL, st, 0, 0);
     colsum_total_kernel<<<dim3((unsigned)ceil_div(ld, TOTAL_COLS), (unsigned)n), EW_THREADS, 0, st>>>(g);

@@ -232,3 +232,17 @@ def test_reading_q_of_one_layer_forms_that_layer_s():
         assert (np.abs(got - (f + u / nu)) <= 4 * 2.0 ** -23 * (np.abs(f) + np.abs(u / nu))).all()
         assert l not in q or np.array_equal(q[l], got)
     ctx.destroy()
+
+
+@pytest.mark.parametrize("levels,neg,step", [(0, 0, 0.0), (16, 0, 0.0), (256, 0, 0.0), (300, 0, 0.0), (22, 1, 1.0), (4096, 0, 0.0)])
+def test_first_iteration_leaves_b_at_zero(levels, neg, step):
+    """From the feasible start p stays as it is and every r is zero, so the mean that b takes is zero: the sums of p before the p-step and after it
+    are the same bits."""
+    inp = synth.make_inputs(synth.small("c2", 1033, feat_dim=9, hidden=33, n_layers=4, quant_levels=levels))
+    ctx = B.from_inputs(inp, quant_neg_levels=neg, quant_step=step)
+    p = [ctx.get_tensor(B.T_P, l) for l in range(1, 5)]
+    ctx.step(1)
+    for l in range(1, 5):
+        assert np.array_equal(p[l - 1], ctx.get_tensor(B.T_P, l)), l
+        assert not ctx.get_tensor(B.T_B, l).any(), l
+    ctx.destroy()
